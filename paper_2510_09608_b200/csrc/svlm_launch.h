@@ -22,6 +22,19 @@ cudaError_t svlm_allow_smem(size_t bytes) {
     return e;
 }
 
+// Streaming multiprocessors of the current device (looked up once per device).
+inline int svlm_sm_count() {
+    static std::atomic<int> known[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+    int n = known[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 148;
+        known[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
 // metadata (svlm_meta.cu)
 void svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n, cudaStream_t st);
 void svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st);
@@ -73,5 +86,10 @@ cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int i
 
 // tcgen05/TMEM/TMA chunk prefill, n_q >= 2 (svlm_prefill_sm100.cu)
 bool svlm_prefill_supported(int n_pages, int group);
+// scratch: svlm_prefill_scratch_bytes of the first cache, its first svlm_prefill_counter_bytes zero before the first
+// launch (the kernel leaves them zero); launches that share it must not overlap.  pages: how many pages each cache is
+// expected to hold (only the balance of the work depends on it).
+size_t svlm_prefill_scratch_bytes(int n_pages, int head_dim);
+constexpr size_t svlm_prefill_counter_bytes = 4096;
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
-                                int n_q, int q_heads, void* out, cudaStream_t st);
+                                int n_q, int q_heads, void* out, const int* pages, void* scratch, cudaStream_t st);

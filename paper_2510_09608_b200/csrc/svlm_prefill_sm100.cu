@@ -1,33 +1,44 @@
 // Chunk-prefill attention for sm_100a: the new chunk's queries (n_q >= 2 rows) attend over the
 // retained cache plus, causally, the chunk itself (paper Section 2.1: the retained KV is reused, only
 // the new second of tokens is computed).  This is the one dense contraction of the path, so it runs
-// on the 5th-generation tensor cores:
-//   * the G query heads that share a KV head are packed along M (row = (token, head-in-group));
-//   * a CTA owns 256 such rows as two 128-row tiles A and B.  Both tiles use every K/V page the CTA
-//     streams, which halves the bytes per flop that have to come out of L2 (with 128 rows per CTA
-//     the K/V stream alone took as long as the whole kernel should);
-//   * the K/V pages of one (tile pair, KV head) are split between the two CTAs of a thread-block
-//     cluster; at the end each CTA hands the un-normalised result of one tile to the other through
-//     distributed shared memory and merges and writes the tile it keeps;
-//   * K and V pages (128 slots) arrive by TMA (128-byte swizzle) into one 5-stage ring, K(j) V(j)
-//     K(j+1) ..., in the order the tensor pipe consumes them;
-//   * one thread issues tcgen05.mma: S_A, S_B = Q K^T into two 128-column TMEM buffers, O_A, O_B += P V
-//     into two TMEM accumulators, in the order PV_A(j) S_A(j+1) PV_B(j) S_B(j+1), so the tensor
-//     pipe works for one tile while the other tile's softmax warpgroup exponentiates;
-//   * two softmax warpgroups (one thread per row) read S with tcgen05.ld in 32-column chunks (a first
-//     pass for the row maximum, a second for the exponentials, the next chunk always in flight),
-//     write P as bf16 back into the TMEM columns of S, where it is the A operand of P V (no
-//     shared-memory round trip); the running maximum moves lazily (O is rescaled only when the
-//     maximum grows by more than 2^8);
-//   * rotation factors of the queries come from a table; causal and partial-page masking only
-//     touches the few pages that hold new-chunk tokens or a ring's ragged end; pages that no row
-//     of the CTA may see are skipped.
-// Every mbarrier wait is bounded: on expiry the CTA records SVLM_ERR_TIMEOUT in the cache's status
-// word, drains its outstanding copies, frees its TMEM and returns (both CTAs of a cluster still meet
-// at the hardware cluster barriers, which every thread reaches on every path).
+// on the 5th-generation tensor cores.
+//
+// Work split.  A unit is 256 packed rows (row = (token, head in the GQA group)) of one KV head of one problem
+// (cache, layer): two 128-row tiles A and B that share every K/V page (with 128 rows per CTA the K/V stream out of L2
+// alone took as long as the whole kernel should).  One CTA per SM walks a list of work computed by every CTA for
+// itself from the device-side page counts: first whole units, round by round over the grid (neighbouring CTAs then
+// stream the same pages at the same time), then its share of the last one to two rounds' units, dealt out evenly in
+// pages, so that no SM idles in a last wave (120 of 148 SMs had work for one stream's chunk before, 960 CTAs were 6.5
+// waves for eight streams).  A unit that is cut between CTAs is merged by the last of them to finish it: the others
+// leave their un-normalised (O, m, l) in the cache's scratch, arrival counters say who is last, nobody waits.
+//
+// Roles (384 threads, registers moved from warpgroup 2 to the softmax with setmaxnreg):
+//   warps 0-3, 4-7   softmax of tile A, B, one thread per row; also that tile's query rotation and output
+//   warp 8           TMA: K and V pages (128 slots, 128-byte swizzle) into one 4-stage ring, K(0) V(0) K(1) ...; it
+//                    runs ahead into the next unit while the current one ends
+//   warps 9, 10      issue tcgen05.mma for tile A, B: S = Q K^T into 128 TMEM columns, O += P V with P read from
+//                    TMEM (P is written over the first 64 columns of S: no shared-memory round trip)
+//   warp 11          the work list
+// What bounds the page loop is each tile's serial chain S -> softmax -> P V -> next S beside the tensor time of both
+// tiles (2048 cycles per page pair).  Measured on it (cycles per page pair, head_dim 128):
+//   3750 -> 3490  two issuers with the turn handed on through a named barrier: a wait on an mbarrier costs ~300 cycles
+//                 even when it is already complete (the shared-memory pipe is saturated by the operand reads), and the
+//                 tensor queue is only ~2 MMAs deep, so a single issuer idled the pipe for four such waits per pair;
+//                 now each issuer's waits run while the other one's MMAs execute
+//   3490 -> 2700  P handed over through named barriers instead of mbarriers (450 -> 50 cycles), in two halves, so that
+//                 the first half's P V runs under the second half's exponentials
+//   softmax of a page 2200 -> 1500 cycles: the whole row in registers (one pass over TMEM), packed fp32 pairs, a
+//                 quarter of the exponentials as a polynomial on the FMA pipe (MUFU alone would need 1024 cycles)
+// Per-page bookkeeping that cost a masked page 2 us (descriptor loads, two barriers and a bisection through shared
+// memory) is now a few shuffles on values that arrive while the thread waits for S.
+// Every mbarrier wait is bounded: on expiry the CTA records SVLM_ERR_TIMEOUT in the caches' status words, keeps up its
+// named-barrier arrivals (their number depends on the work list only), drains its copies, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
+
 #include "svlm_dev.h"
 #include "svlm_launch.h"
 #include "svlm_ptx.cuh"
@@ -39,542 +50,960 @@ namespace {
 using namespace svlm_ptx;
 using namespace svlm_tc;
 
-#ifndef PF_ISSUERS
-#define PF_ISSUERS 1                  // threads that issue tcgen05.mma (two interleaving streams measured slower)
-#endif
-constexpr int PF_THREADS = 288 + 32 * PF_ISSUERS;   // warps 0-3: softmax of tile A, 4-7: tile B; warp 8: TMA; warp 9 (, 10): MMA issue
-constexpr int PF_RING = 5;            // K/V page stages
+constexpr int PF_THREADS = 384;
+constexpr int PF_RING = 4;            // K/V page stages (3: 18 % slower, the next K arrives late; 5: no faster)
 constexpr int PF_MAX_TILES = 512;
-constexpr int PF_ROWS = 256;          // rows per CTA
+constexpr int PF_ROWS = 256;          // rows per unit
+constexpr int PF_MAX_CTAS = 160;
+constexpr int PF_MIN_PAGES = 6;       // pages a CTA should have at least when units are cut
+constexpr size_t PF_HEAD_BYTES = svlm_prefill_counter_bytes;   // counters in front of the scratch's slots
+constexpr int PF_PIECE = 10;          // what beginning another unit costs, in pages (one stream: 3 and 6: 78 us, 10: 76, 16: 78)
+constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
+constexpr int PF_CS_BYTES = 16384;    // rotation factors of one tile's tokens (5 or more heads per KV head, all at head_dim 64 with 2 or more)
+// Registers per thread after the split; 216 * 256 + 72 * 128 = 168 * 384, what the block is launched with (checked at launch).
+constexpr int PF_REGS_LAUNCH = 168;
 
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
+// The work split, made on the host: it needs the numbers of rows, and of the pages only an estimate (a unit's pages are
+// cut at fractions), so the kernel starts on its first unit without waiting for anything on the device.
+constexpr int PF_FRAC = 128;          // a unit's pages are cut at multiples of 1/128
+struct PfPlan {
+    int units;                        // all units of the launch
+    int off[SVLM_MAX_BATCH + 1];      // first unit of every cache: (layer, KV head, row tile), row tile fastest
+    int rounds;                       // whole units per CTA first: CTA i takes units i, grid + i, ...
+    int tail;                         // the units from here on are dealt out by x
+    unsigned short x[PF_MAX_CTAS + 1];// where each CTA's share of them begins, in 1/128 units
+    unsigned g_magic;                 // for dividing by the heads per KV head (pf_div)
+    unsigned* counters;               // [2 * PF_MAX_CTAS][2] arrivals per (tail unit, tile), zero between launches
+    unsigned char* slots;             // [2 * grid] partial results
+};
+static_assert(2 * PF_MAX_CTAS * 2 * sizeof(unsigned) <= PF_HEAD_BYTES, "counters");
+
+template <int D>
+__host__ __device__ constexpr size_t pf_slot_bytes() { return (size_t)PF_ROWS * D * 4 + PF_ROWS * 8; }
+
+// ---- packed fp32 pairs ---------------------------------------------------------------------------------------
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 pk64(float a, float b) { u64 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ void un64(u64 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) { u64 r; asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ u64 add2(u64 a, u64 b) { u64 r; asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) { u64 r; asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ float max3(float a, float b, float c) { float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r; }
+__device__ __forceinline__ float ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+
+// 2^x of a pair on the FMA pipe: x = n + f with n the nearest integer (added and taken off again with 1.5 * 2^23),
+// 2^f by the degree-5 minimax polynomial on [-1/2, 1/2] (Remez exchange on the relative error; 2.1e-7 with fp32
+// Horner steps, the size of ex2.approx's own error), n added to the exponent field.  x is held above -126.
+__device__ __forceinline__ u64 exp2_poly2(u64 x) {
+    float a, b;
+    un64(x, a, b);
+    x = pk64(fmaxf(a, -126.f), fmaxf(b, -126.f));
+    constexpr float MAGIC = 12582912.f;
+    const u64 t = add2(x, pk64(MAGIC, MAGIC));
+    const u64 n = add2(t, pk64(-MAGIC, -MAGIC));
+    const u64 f = fma2(n, pk64(-1.f, -1.f), x);
+    u64 p = pk64(0.0013276472454890609f, 0.0013276472454890609f);
+    p = fma2(p, f, pk64(0.009675540961325169f, 0.009675540961325169f));
+    p = fma2(p, f, pk64(0.05550713092088699f, 0.05550713092088699f));
+    p = fma2(p, f, pk64(0.24022120237350464f, 0.24022120237350464f));
+    p = fma2(p, f, pk64(0.6931469440460205f, 0.6931469440460205f));
+    p = fma2(p, f, pk64(1.0000001192092896f, 1.0000001192092896f));
+    float ta, tb, pa, pb;
+    un64(t, ta, tb);
+    un64(p, pa, pb);
+    pa = __int_as_float(__float_as_int(pa) + (__float_as_int(ta) << 23));
+    pb = __int_as_float(__float_as_int(pb) + (__float_as_int(tb) << 23));
+    return pk64(pa, pb);
+}
+
+// ---- named barriers (the hardware's, not shared memory): ids ----------------------------------------------------
+constexpr int BAR_WG = 1;      // + tile: the softmax warpgroup alone (128)
+constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM and it is this tile's turn (128 softmax + 32 other issuer + 32 issuer)
+constexpr int BAR_P2 = 5;      // + tile: second half of P (128 + 32)
+constexpr int BAR_TURN_B = 7;  // first S of tile B in a unit (32 + 32)
+constexpr int BAR_TURN_A = 8;  // first S of tile A in a unit after the first
+constexpr int BAR_Q = 9;       // + tile: the tile's query rows are in shared memory, its accumulator is free (128 + 32)
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// Rescale the row's accumulator when its reference maximum moves (rare).  Eight columns at a time: with the row of
+// scores live there are few registers left.
+__device__ __forceinline__ void rescale_o(unsigned tO, int D, float corr) {
+#pragma unroll 1
+    for (int q = 0; q < D; q += 8) {
+        float o[8];
+        tmem_ld8(tO + q, o);
+        tmem_wait_ld();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o[k] *= corr;
+        tmem_st8(tO + q, o);
+    }
 }
 
 // One page of one row: S (128 fp32 columns at tS, this thread's TMEM lane) -> P (bf16 pairs in the first 64
-// columns of the same buffer), with the lazily moving reference maximum.  Two passes over S in halves of
-// 64 columns (two 32-column loads in flight at a time): row maximum, then exponentials.  P chunk ch
-// (16 columns) lands where S columns [16 ch, 16 ch + 16) were; those have been read by then and the
-// loads still in flight lie beyond them.  On MASKED pages the row sees the columns [vlo, vlo + vlen): stream
-// ordinals grow with the offset inside a page, so the valid and causally visible columns of a row are one interval.
+// columns of the same buffer), with a lazily moving reference maximum (O is rescaled only when the maximum grows by
+// more than 2^8).  The whole row is loaded once; the first half's maximum is taken while the second half is on its
+// way.  P goes out in chunks of 32 keys; once the exponentials of the third chunk are done, the first two chunks are
+// certainly stored and are handed to the issuer (BAR_P1).  On MASKED pages the row sees the columns [vlo, vlo + vlen).
+constexpr int PF_POLY = 2;             // of every 8 pairs, those whose exponential goes to the FMA pipe (0: +5 %, 1: +2 %, 3: +9 % time)
 template <bool MASKED>
-__device__ __noinline__ void softmax_page(unsigned tS, unsigned tO, int D, unsigned vlo, unsigned vlen,
-                                             float c, float m_ref, bool have_o, float& rowsum, float& corr, float& m_new) {
+__device__ __forceinline__ void softmax_page(int g, unsigned tS, unsigned tO, int D, unsigned vlo, unsigned vlen, float c,
+                                             float m_ref, bool have_o, float& rowsum, float& corr, float& m_new) {
     auto visible = [&](int k) { return (unsigned)k - vlo < vlen; };
-    float ca[32], cb[32];
-    // ---- pass 1: row maximum
-    float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    float s[128];
+    tmem_ld32(tS, s);
+    tmem_ld32(tS + 32, s + 32);
+    tmem_wait_ld();
+    tmem_ld32(tS + 64, s + 64);
+    tmem_ld32(tS + 96, s + 96);
+    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-    for (int hf = 0; hf < 2; ++hf) {
-        tmem_ld32(tS + hf * 64, ca);
-        tmem_ld32(tS + hf * 64 + 32, cb);
-        tmem_wait_ld();
+    for (int h = 0; h < 2; ++h) {
+        if (MASKED) {
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            const float a = MASKED ? (visible(hf * 64 + k) ? ca[k] : -INFINITY) : ca[k];
-            const float bq = MASKED ? (visible(hf * 64 + 32 + k) ? cb[k] : -INFINITY) : cb[k];
-            mx4[k & 3] = fmaxf(mx4[k & 3], fmaxf(a, bq));
+            for (int k = 64 * h; k < 64 * h + 64; ++k) s[k] = visible(k) ? s[k] : -INFINITY;
+        }
+#pragma unroll
+        for (int k = 64 * h; k < 64 * h + 64; k += 2) mx[(k >> 1) & 3] = max3(mx[(k >> 1) & 3], s[k], s[k + 1]);
+        if (h == 0) tmem_wait_ld();
+    }
+    const float mx_row = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]) * c;
+    const bool grow = mx_row > m_ref + 8.f;
+    m_new = grow ? mx_row : m_ref;
+    const float m_use = m_new == -INFINITY ? 0.f : m_new;
+    corr = 1.f;
+    if (__any_sync(0xffffffffu, grow)) {
+        corr = grow ? exp2f(m_ref - m_use) : 1.f;   // m_ref = -inf gives 0
+        if (have_o) rescale_o(tO, D, corr);         // S of this page was issued after P V of the previous one: O is quiescent
+    }
+    const u64 c2 = pk64(c, c), nm2 = pk64(-m_use, -m_use);
+    u64 sum[2] = {0ull, 0ull};
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) {
+        unsigned pk[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int k = ch * 32 + 2 * i;
+            const u64 t = fma2(pk64(s[k], s[k + 1]), c2, nm2);
+            float e0, e1;
+            u64 e;
+            if ((i & 7) < PF_POLY) {
+                e = exp2_poly2(t);
+                un64(e, e0, e1);
+                if (MASKED) {
+                    e0 = s[k] == -INFINITY ? 0.f : e0;
+                    e1 = s[k + 1] == -INFINITY ? 0.f : e1;
+                    e = pk64(e0, e1);
+                }
+            } else {
+                un64(t, e0, e1);
+                e0 = ex2(e0);
+                e1 = ex2(e1);
+                e = pk64(e0, e1);
+            }
+            sum[i & 1] = add2(sum[i & 1], e);
+            pk[i] = pack2(e0, e1);
+        }
+        if (ch == 2) {
+            tmem_wait_st();
+            tc_fence_before();
+            bar_arrive(BAR_P1 + g, 192);
+        }
+        tmem_st16(tS + ch * 16, pk);
+    }
+    float a0, a1, b0, b1;
+    un64(sum[0], a0, a1);
+    un64(sum[1], b0, b1);
+    rowsum = (a0 + a1) + (b0 + b1);
+}
+
+// n / G with magic = ceil(2^32 / G), which is exact for n < 2^32 / G; magic = 0: the launch has other numbers.
+__device__ __forceinline__ int pf_div(int n, unsigned magic, int G) { return magic ? (int)__umulhi((unsigned)n, magic) : (G == 1 ? n : n / G); }
+// a / b for small numbers without the long division (a once-executed division costs hundreds of cycles of instruction fetch)
+__device__ __forceinline__ int pf_small_div(int a, int b) {
+    return a < (1 << 18) ? (int)(((float)a + 0.5f) * __frcp_rn((float)b)) : a / b;
+}
+
+// A piece of the work list.
+struct PfSeg {
+    int unit;                // unit of the launch
+    int a, e;                // its pages [a, e) in 1/128 of all the unit's pages
+    int tail;                // index among the tail's units, -1: a whole unit of the first rounds
+};
+
+// A CTA's walk over its work list.
+struct PfWalk {
+    int round, pos, end;
+    __device__ __forceinline__ void begin(const PfPlan& plan) {
+        round = 0;
+        pos = plan.x[blockIdx.x];
+        end = plan.x[blockIdx.x + 1];
+    }
+    __device__ __forceinline__ bool more(const PfPlan& plan) const { return round < plan.rounds || pos < end; }
+    __device__ __forceinline__ PfSeg next(const PfPlan& plan) {
+        PfSeg s;
+        if (round < plan.rounds) {
+            s.unit = round * gridDim.x + blockIdx.x;
+            s.a = 0; s.e = PF_FRAC; s.tail = -1;
+            ++round;
+        } else {
+            s.tail = pos / PF_FRAC;
+            s.unit = plan.tail + s.tail;
+            s.a = pos % PF_FRAC;
+            pos = min(end, (s.tail + 1) * PF_FRAC);
+            s.e = pos - s.tail * PF_FRAC;
+        }
+        return s;
+    }
+};
+
+__device__ __forceinline__ int pf_rows_of(const SvlmAttendBatch& b, int ci, int n_q_arg) { return b.q_varlen ? b.q_cnt[ci] : n_q_arg; }
+
+// Where a segment's rows lie, from the launch's arguments alone (warp-uniform).
+struct PfRows {
+    int ci, hk, n_q, m0, m_total;
+    size_t q_row0, p_row0;   // first row in Q and out, in q_pos
+    size_t head_row0;        // the head's first slot row in the K/V slabs
+};
+__device__ __forceinline__ PfRows pf_rows(const SvlmAttendBatch& b, const PfPlan& plan, int unit, int n_q_arg, int G, int layer0, int n_layers) {
+    PfRows r;
+    r.ci = 0;
+    while (r.ci + 1 < b.n_caches && unit >= plan.off[r.ci + 1]) ++r.ci;
+    r.n_q = pf_rows_of(b, r.ci, n_q_arg);
+    r.m_total = r.n_q * G;
+    const int R = (r.m_total + PF_ROWS - 1) / PF_ROWS, local = unit - plan.off[r.ci], t = pf_small_div(local, R);
+    r.m0 = (local - t * R) * PF_ROWS;
+    const int li = pf_small_div(t, b.kv_heads);
+    r.hk = t - li * b.kv_heads;
+    r.head_row0 = ((size_t)(layer0 + li) * b.kv_heads + r.hk) * b.n_slots;
+    r.q_row0 = b.q_varlen ? (size_t)b.q_off[r.ci] : (size_t)(r.ci * n_layers + li) * n_q_arg;
+    r.p_row0 = b.q_varlen ? (size_t)b.q_off[r.ci] : (size_t)r.ci * n_q_arg;
+    return r;
+}
+
+// What the cache's metadata adds: the segment's pages.
+struct PfWork {
+    const SvlmAttendView* vw;
+    int n_tiles, p0, n_proc;       // entries of the page list; of the pages that some row of the unit may see, [p0, p0 + n_proc)
+    long long gid_hi, gid_q0;      // ordinals of the unit's last row's token and of the first query token
+    long long shift;
+    unsigned wait_limit;
+};
+// In two steps, so that a caller can have more in flight: the loads (the first pages' ordinals without waiting for their
+// count, so that everything takes one round trip), then what they say.
+struct PfAsk {
+    long long first[4], n_total, shift;
+    int n_tiles;
+    unsigned wait_limit;
+};
+__device__ __forceinline__ PfAsk pf_ask(const SvlmAttendBatch& b, const PfRows& r) {
+    PfAsk q;
+    const SvlmAttendView& vw = b.view[r.ci];
+    const int lane = threadIdx.x & 31, n_pages = b.n_slots / SVLM_PAGE;
+    q.n_tiles = __ldcg(&vw.ctrl->n_tiles);
+    q.n_total = __ldcg(&vw.ctrl->n_total);
+    q.shift = __ldcg(&vw.ctrl->shift_total);
+    q.wait_limit = __ldcg(&vw.ctrl->wait_limit);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q.first[k] = __ldcg(&vw.tiles[min(lane + 32 * k, n_pages - 1)].min_gid);
+    return q;
+}
+__device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfSeg& s, const PfRows& r, unsigned g_magic, int G, const PfAsk& q) {
+    PfWork w;
+    w.vw = &b.view[r.ci];
+    w.n_tiles = q.n_tiles;
+    w.gid_q0 = q.n_total - r.n_q;
+    w.shift = q.shift;
+    w.wait_limit = q.wait_limit;
+    w.gid_hi = w.gid_q0 + min(r.n_q - 1, pf_div(r.m0 + PF_ROWS - 1, g_magic, G));
+    const int lane = threadIdx.x & 31;
+    int n_act = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) n_act += lane + 32 * k < w.n_tiles && q.first[k] <= w.gid_hi;
+    for (int j = lane + 128; j < w.n_tiles; j += 32) n_act += __ldcg(&w.vw->tiles[j].min_gid) <= w.gid_hi;
+    n_act = __reduce_add_sync(0xffffffffu, n_act);
+    w.p0 = s.a * n_act / PF_FRAC;
+    w.n_proc = s.e * n_act / PF_FRAC - w.p0;
+    return w;
+}
+
+// The softmax warpgroups keep what they know about their segment in shared memory: the page loop needs nearly all of
+// their registers for the row of scores.
+struct PfGroup {
+    PfSeg seg;
+    PfRows rows;
+    PfWork w;
+    PfWalk walk;
+    int more;                // segments follow
+    int merge_later;         // a cut unit whose pieces this CTA has to put together at the end (-1: none)
+};
+
+struct PfShared {            // control part of shared memory, behind the tiles
+    unsigned long long full[PF_RING], empty[PF_RING];
+    unsigned long long s_full[2], all_done[2];
+    unsigned tmem_base;
+    int abort_flag;
+    int last[2];                           // per tile: this CTA's piece of the unit was the last to be done
+    PfGroup group[2];
+};
+static_assert(sizeof(PfShared) <= 3072, "control block must fit behind the tiles");
+
+// A warp's walk over the pages of a segment, 32 tiles of the cache's page list at a time, one per lane.
+struct PfPages {
+    int base, seen;
+    unsigned left, info;     // pages of the window still to come; per lane: page | lo << 14 | (hi - 1) << 21 | masked << 28 | causal << 29
+    __device__ __forceinline__ void begin() { base = 0; seen = 0; left = 0; info = 0; }
+    // r_lo: rows from this token on are served; a page all of them see in full needs no mask
+    __device__ __forceinline__ unsigned next(const PfWork& w, int r_lo) {
+        const int lane = threadIdx.x & 31;
+        while (left == 0 && base < w.n_tiles) {
+            const int j = base + lane;
+            bool vis = false;
+            if (j < w.n_tiles) {
+                const SvlmTile* tp = w.vw->tiles + j;
+                const int4 a = __ldcg(reinterpret_cast<const int4*>(tp));
+                const longlong2 g = __ldcg(reinterpret_cast<const longlong2*>(&tp->min_gid));
+                vis = g.x <= w.gid_hi;
+                const unsigned causal = g.y > w.gid_q0 + r_lo, ragged = a.y > 0 || a.z < SVLM_PAGE;
+                info = (unsigned)a.x | ((unsigned)a.y << 14) | ((unsigned)(a.z - 1) << 21) | ((causal | ragged) << 28) | (causal << 29);
+            }
+            const unsigned all = __ballot_sync(0xffffffffu, vis);
+            const int rank = seen + __popc(all & ((1u << lane) - 1));
+            left = __ballot_sync(0xffffffffu, vis && rank >= w.p0 && rank < w.p0 + w.n_proc);
+            seen += __popc(all);
+            base += 32;
+        }
+        const int at = left ? __ffs(left) - 1 : 0;
+        left &= left - 1;
+        return __shfl_sync(0xffffffffu, info, at);
+    }
+};
+// Rotates one 128-row tile of queries at q_pos - shift_total, rounds to bf16 and stores it K-major swizzled.  Called by
+// the 128 threads of the tile's softmax warpgroup.  A work item is (row, 8 pairs): a 16-byte chunk of the row's low half
+// with its partner of the high half; a thread keeps its chunk and takes every 128 / CH-th row.  The raw rows go to their
+// places in shared memory asynchronously and are rotated there; meanwhile the factors of the tile's tokens (a token's G
+// rows share them) are looked up, in batches without branches (look-ups that branched on the size of the position went
+// out one by one).  This code runs once per unit, at the pace of the instruction fetch (4-8 cycles per instruction), so
+// its loops are short: 15000 cycles when everything was unrolled.
+template <int D>
+struct PfTileRotation {
+    static constexpr int HALF = D / 2, CH = D / 16, STEP = 128 / CH;      // chunks per half row; rows between a thread's items
+    static constexpr int TPT = 128 / HALF;                                // tokens per pass of the 128 threads over the factors
+    static constexpr int UN = 5;                                          // factors in flight per thread
+
+    // element e of a row lives in block e/64, 16-byte chunk (e%64)/8, XOR-swizzled by row&7
+    __device__ __forceinline__ static int at(int row, int e) { return (e / 64) * (128 * 128) + row * 128 + ((((e % 64) / 8) ^ (row & 7)) << 4); }
+
+    __device__ __forceinline__ static void load(const PfRows& w, int g, int m, int G, unsigned g_magic, int q_heads, const uint16_t* __restrict__ Q, unsigned char* sQ) {
+        const int c8 = m % CH;
+        const uint16_t* base = Q + (w.q_row0 * q_heads + w.hk * G) * D + c8 * 8;
+        const unsigned dst = smem_u32(sQ);
+#pragma unroll 2
+        for (int u = 0; u < CH; ++u) {
+            const int row = m / CH + u * STEP, mg = w.m0 + g * 128 + row;
+            const bool live = mg < w.m_total;
+            // row (token r, head h) lies at r * q_heads + h = r * (q_heads - G) + mg
+            const uint16_t* src = live ? base + (size_t)(unsigned)(pf_div(mg, g_magic, G) * (q_heads - G) + mg) * D : base;
+            const int n = live ? 16 : 0;                              // the rest is filled with zeros
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + at(row, c8 * 8)), "l"(src), "r"(n) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + at(row, HALF + c8 * 8)), "l"(src + HALF), "r"(n) : "memory");
         }
     }
-    tmem_ld32(tS, ca);            // first half again, for pass 2
-    tmem_ld32(tS + 32, cb);
-    const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * c;
-    // lazy running maximum: only move the reference when it would be exceeded by 2^8
-    const bool grow = mx > m_ref + 8.f;
-    m_new = grow ? mx : m_ref;
-    const float m_use = m_new == -INFINITY ? 0.f : m_new;
-    corr = grow ? exp2f(m_ref - m_use) : 1.f;   // m_ref = -inf gives 0
-    tmem_wait_ld();
-    if (have_o && __any_sync(0xffffffffu, grow)) {
-        // S of this page was issued after P V of the previous one: O is quiescent
+    __device__ __forceinline__ static int axis_of(const SvlmAttendBatch& b, int pair) {
+        return b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
+    }
+    // (cos, sin)(c * theta) for |c| < 2^16: two table entries, loaded without a branch (see svlm_rope.cuh)
+    struct Near { float2 a, b; bool neg; };
+    __device__ __forceinline__ static Near near_load(const float2* __restrict__ tab, int pair, int c) {
+        const unsigned u = (unsigned)abs(c) & 0xffffu;
+        return Near{__ldg(tab + (u & 255u) * HALF + pair), __ldg(tab + (256 + (u >> 8)) * HALF + pair), c < 0};
+    }
+    __device__ __forceinline__ static float2 near_value(const Near& n) {
+        float2 r = svlm_cmul(n.a, n.b);
+        if (n.neg) r.y = -r.y;
+        return r;
+    }
+    __device__ __forceinline__ static bool is_near(long long c) { return c > -65536 && c < 65536; }
+
+    // the tile's tokens and whether their factors fit the area
+    __device__ __forceinline__ static bool staged(const PfRows& w, int g, unsigned g_magic, int G, int& t_lo, int& n_tok) {
+        const int mt = w.m0 + g * 128;
+        t_lo = min(w.n_q - 1, pf_div(mt, g_magic, G));
+        n_tok = min(w.n_q - 1, pf_div(mt + 127, g_magic, G)) - t_lo + 1;
+        return n_tok * (HALF * 8) <= PF_CS_BYTES;
+    }
+    // factors: per token HALF cosines, then HALF sines.  Eight consecutive lanes read eight values each at a time; the
+    // 16-byte chunks are swizzled so that their halves fall into different banks
+    __device__ __forceinline__ static int cs_at(int pair) { return (((pair >> 2) ^ ((pair >> 5) & 1)) << 2) | (pair & 3); }
+    int c[UN];               // positions of the thread's first UN factors
+    __device__ __forceinline__ void load_pos(const SvlmAttendBatch& b, const PfRows& w, const int* __restrict__ q_pos, int m, int t_lo, int n_tok, int tk0) {
+        const int pw = b.rope_mode == 0 ? 1 : 3;
+        const int* qp = q_pos + (w.p_row0 + t_lo) * pw + axis_of(b, m % HALF);
+#pragma unroll
+        for (int u = 0; u < UN; ++u) c[u] = __ldg(qp + (size_t)min(tk0 + u * TPT, n_tok - 1) * pw);
+    }
+    __device__ __forceinline__ void stage(const SvlmAttendBatch& b, const PfRows& w, long long shift, const int* __restrict__ q_pos, int m, int t_lo, int n_tok, float* s_cs) {
+        const int pair = m % HALF;
+        const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
+        float* dst = s_cs + cs_at(pair);
+        bool far = false;
+#pragma unroll 1
+        for (int tk0 = m / HALF; tk0 < n_tok; tk0 += TPT * UN) {
+            Near v[UN];
+            if (tk0 >= TPT) load_pos(b, w, q_pos, m, t_lo, n_tok, tk0);      // (the first batch is here already)
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                const long long cl = (long long)c[u] - shift;
+                far |= !is_near(cl);
+                v[u] = near_load(tab, pair, (int)cl);
+            }
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                const int tk = tk0 + u * TPT;
+                const float2 f = near_value(v[u]);
+                if (tk < n_tok) {
+                    dst[(size_t)tk * 2 * HALF] = f.x;
+                    dst[(size_t)tk * 2 * HALF + HALF] = f.y;
+                }
+            }
+        }
+        if (far) {                                     // native positions of a long stream
+            const int pw = b.rope_mode == 0 ? 1 : 3;
+            const int* qp = q_pos + (w.p_row0 + t_lo) * pw + axis_of(b, pair);
+#pragma unroll 1
+            for (int tk = m / HALF; tk < n_tok; tk += TPT) {
+                const float2 f = svlm_rope_cs(tab, HALF, pair, (long long)__ldg(qp + (size_t)tk * pw) - shift, b.theta[pair]);
+                dst[(size_t)tk * 2 * HALF] = f.x;
+                dst[(size_t)tk * 2 * HALF + HALF] = f.y;
+            }
+        }
+    }
+
+    __device__ __forceinline__ static void rotate(const SvlmAttendBatch& b, const PfRows& w, long long shift, const int* __restrict__ q_pos, int g, int m,
+                                                  unsigned g_magic, int G, int t_lo, bool from_stage, const float* s_cs, unsigned char* sQ) {
+        const int c8 = m % CH;
+#pragma unroll 2
+        for (int u = 0; u < CH; ++u) {
+            const int row = m / CH + u * STEP;
+            const int tk = min(pf_div(w.m0 + g * 128 + row, g_magic, G), w.n_q - 1);
+            uint4* plo = reinterpret_cast<uint4*>(sQ + at(row, c8 * 8));
+            uint4* phi = reinterpret_cast<uint4*>(sQ + at(row, HALF + c8 * 8));
+            const uint4 lo4 = *plo, hi4 = *phi;
+            u64 cs[4], sn[4];                          // cosines and sines of the chunk's pairs, two and two
+            if (from_stage) {
+                const float* base = s_cs + (size_t)(tk - t_lo) * 2 * HALF;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(base + cs_at(c8 * 8 + 4 * j));
+                    const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(base + HALF + cs_at(c8 * 8 + 4 * j));
+                    cs[2 * j] = x.x; cs[2 * j + 1] = x.y;
+                    sn[2 * j] = y.x; sn[2 * j + 1] = y.y;
+                }
+            } else {                                   // few heads per KV head: too many tokens for the area
+                const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
+                const int pw = b.rope_mode == 0 ? 1 : 3;
+                const int* qp = q_pos + (w.p_row0 + tk) * pw;
+                const long long p[3] = {__ldg(qp) - shift, __ldg(qp + pw / 2) - shift, __ldg(qp + pw - 1) - shift};
+                Near v[8];
+                bool far = false;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int a = axis_of(b, c8 * 8 + i);
+                    const long long c = a == 0 ? p[0] : (a == 1 ? p[1] : p[2]);
+                    far |= !is_near(c);
+                    v[i] = near_load(tab, c8 * 8 + i, (int)c);
+                }
+                float2 f[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) f[i] = near_value(v[i]);
+                if (far) {
+#pragma unroll 1
+                    for (int i = 0; i < 8; ++i) {
+                        const int a = axis_of(b, c8 * 8 + i);
+                        const float2 x = svlm_rope_cs(tab, HALF, c8 * 8 + i, a == 0 ? p[0] : (a == 1 ? p[1] : p[2]), b.theta[c8 * 8 + i]);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) if (q == i) f[q] = x;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { cs[j] = pk64(f[2 * j].x, f[2 * j + 1].x); sn[j] = pk64(f[2 * j].y, f[2 * j + 1].y); }
+            }
+            const unsigned* lw = reinterpret_cast<const unsigned*>(&lo4);
+            const unsigned* hw = reinterpret_cast<const unsigned*>(&hi4);
+            unsigned lo_o[4], hi_o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const u64 xl = pk64(__uint_as_float(lw[j] << 16), __uint_as_float(lw[j] & 0xffff0000u));
+                const u64 xh = pk64(__uint_as_float(hw[j] << 16), __uint_as_float(hw[j] & 0xffff0000u));
+                float a, c;
+                un64(fma2(xl, cs[j], mul2(xh, sn[j] ^ 0x8000000080000000ull)), a, c);
+                lo_o[j] = pack2(a, c);
+                un64(fma2(xh, cs[j], mul2(xl, sn[j])), a, c);
+                hi_o[j] = pack2(a, c);
+            }
+            *plo = make_uint4(lo_o[0], lo_o[1], lo_o[2], lo_o[3]);
+            *phi = make_uint4(hi_o[0], hi_o[1], hi_o[2], hi_o[3]);
+        }
+    }
+};
+
+// End of the columns a row may see on a page with causal limits: stream ordinals grow with the offset, so it is the
+// number of offsets whose ordinal (relative to the first query token) does not exceed the row's, found by bisection
+// with shuffles over the page's 128 ordinals, four per lane (v; offsets below the valid range count as visible).
+__device__ __forceinline__ int causal_end(const int (&v)[4], int r) {
+    int L = 0;                                 // lanes all of whose four offsets are visible
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const int x = __shfl_sync(0xffffffffu, v[3], L + s - 1);
+        if (x <= r) L += s;
+    }
+    {
+        const int x = __shfl_sync(0xffffffffu, v[3], L);
+        if (x <= r) L += 1;                    // (L was at most 31)
+    }
+    int n = 4 * L;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int x = __shfl_sync(0xffffffffu, v[k], L & 31);
+        if (L < 32 && x <= r) ++n;
+    }
+    return n;
+}
+
+__device__ __forceinline__ void store_row32(uint16_t* dst, const float* o) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        *reinterpret_cast<uint4*>(dst + 8 * k) = make_uint4(pack2(o[8 * k], o[8 * k + 1]), pack2(o[8 * k + 2], o[8 * k + 3]),
+                                                            pack2(o[8 * k + 4], o[8 * k + 5]), pack2(o[8 * k + 6], o[8 * k + 7]));
+}
+
+__device__ __forceinline__ uint16_t* out_row(uint16_t* out, const PfRows& w, int mg, unsigned g_magic, int G, int q_heads, int D) {
+    const int r = pf_div(mg, g_magic, G);      // row (token r, head h) lies at r * q_heads + h = r * (q_heads - G) + mg
+    return out + (w.q_row0 * q_heads + w.hk * G + (size_t)(unsigned)(r * (q_heads - G) + mg)) * D;
+}
+
+// The scratch of a cut unit: CTA k's piece lies in k's first slot if it is k's first piece of the tail, else in the second.
+template <int D>
+struct PfSlot {
+    unsigned char* base;
+    __device__ __forceinline__ PfSlot(const PfPlan& plan, int tail, int k)
+        : base(plan.slots + (size_t)(2 * k + (plan.x[k] >= tail * PF_FRAC ? 0 : 1)) * pf_slot_bytes<D>()) {}
+    __device__ __forceinline__ float4* o(int g, int m) const { return reinterpret_cast<float4*>(base) + (size_t)g * 128 * (D / 4) + m; }   // + 128 per 4 columns
+    __device__ __forceinline__ float2* ml(int g, int m) const { return reinterpret_cast<float2*>(base + (size_t)PF_ROWS * D * 4) + g * 128 + m; }
+};
+
+// This CTA's piece of a cut unit into its slot (un-normalised, fp32), then counted.  True in the CTA whose piece was the
+// last one (for all 128 threads of the warpgroup).
+template <int D>
+__device__ __forceinline__ bool publish_piece(PfShared& sh, const PfPlan& plan, int tail, int pieces, int g, int m, unsigned tO, float m_row, float l, bool have_o) {
+    const PfSlot<D> slot(plan, tail, blockIdx.x);
+    float4* po = slot.o(g, m);
+    if (have_o)
 #pragma unroll 1
         for (int q4 = 0; q4 < D / 32; ++q4) {
             float o[32];
             tmem_ld32(tO + q4 * 32, o);
             tmem_wait_ld();
 #pragma unroll
-            for (int k = 0; k < 32; ++k) o[k] *= corr;
-            tmem_st32(tO + q4 * 32, o);
+            for (int i = 0; i < 8; ++i) __stcg(po + (q4 * 8 + i) * 128, make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]));
         }
+    __stcg(slot.ml(g, m), make_float2(have_o ? m_row : -INFINITY, l));
+    __threadfence();
+    bar_sync(BAR_WG + g, 128);
+    if (m == 0) {
+        unsigned prev;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(prev) : "l"(plan.counters + tail * 2 + g) : "memory");
+        sh.last[g] = prev == (unsigned)pieces - 1;
     }
-    // ---- pass 2: exponentials in stages (all scale-subtracts, all ex2, then sums and packing), so
-    //      that the special-function pipe always has independent work queued
-    float rs4[4] = {0.f, 0.f, 0.f, 0.f};
-    auto exp_chunk = [&](float* x, int ch) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) x[k] = fmaf(x[k], c, -m_use);
-#pragma unroll
-        for (int k = 0; k < 32; ++k) x[k] = ex2(x[k]);
-        if (MASKED) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) x[k] = visible(ch * 32 + k) ? x[k] : 0.f;
-        }
-        unsigned pk[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            rs4[k & 3] += x[2 * k] + x[2 * k + 1];
-            pk[k] = pack2(x[2 * k], x[2 * k + 1]);
-        }
-        tmem_st16(tS + ch * 16, pk);
-    };
-    exp_chunk(ca, 0);
-    exp_chunk(cb, 1);
-    tmem_ld32(tS + 64, ca);       // columns 64..127 are untouched by P (columns 0..63)
-    tmem_ld32(tS + 96, cb);
-    tmem_wait_ld();
-    exp_chunk(ca, 2);
-    exp_chunk(cb, 3);
-    rowsum = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
+    bar_sync(BAR_WG + g, 128);
+    return sh.last[g] != 0;
 }
 
-struct PfShared {            // control part of shared memory (tiles follow, 1024-byte aligned)
-    unsigned long long full[PF_RING], empty[PF_RING];
-    unsigned long long s_full[2], p_full[2], all_done;
-    unsigned tmem_base;
-    int abort_flag;
-    unsigned short tile[PF_MAX_TILES];     // page | mask << 14 | skip << 15
-    unsigned short minrow[2][SVLM_PAGE];   // per softmax group: first query token that may see the column
-};
-static_assert(sizeof(PfShared) <= 2040, "control block must leave room for the tiles");
+// CTAs that hold pieces of a tail unit: [first, last], those with an empty share left out.  near: one of them.
+__device__ __forceinline__ int count_pieces(const PfPlan& plan, int tail, int near, int& first, int& last) {
+    const int u0 = tail * PF_FRAC;
+    for (first = near; plan.x[first] > u0; --first) {}
+    for (last = near; plan.x[last + 1] < u0 + PF_FRAC; ++last) {}
+    int n = 0;
+    for (int k = first; k <= last; ++k) n += plan.x[k] < plan.x[k + 1];
+    return n;
+}
+
+// The output of a cut unit's tile from the slots of its pieces, by the CTA that came last; that CTA's own piece may
+// still be in TMEM (own).  In the order of the pieces, whoever comes last: the same bits every time.
+template <int D>
+__device__ __forceinline__ void merge_pieces(const PfPlan& plan, int tail, const PfRows& w, int g, int m, int G, int q_heads, bool own,
+                                             unsigned tO, float m_row, float l, bool have_o, uint16_t* __restrict__ out) {
+    __threadfence();
+    if (m == 0) plan.counters[tail * 2 + g] = 0;      // ready for the next launch
+    int first, last;
+    count_pieces(plan, tail, blockIdx.x, first, last);      // (this CTA holds a piece)
+    const int me = own ? (int)blockIdx.x : -1;
+    const float m_own = have_o ? m_row : -INFINITY;
+    float M = -INFINITY, L = 0.f;
+#pragma unroll 1
+    for (int k0 = first; k0 <= last; k0 += 4) {              // four pieces' (m, l) in flight
+        float2 ml[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = min(k0 + i, last);
+            ml[i] = k == me ? make_float2(m_own, l) : __ldcg(PfSlot<D>(plan, tail, k).ml(g, m));
+            if (k0 + i > last || plan.x[k] >= plan.x[k + 1]) ml[i].x = -INFINITY;
+        }
+        const float Mn = fmaxf(fmaxf(M, fmaxf(ml[0].x, ml[1].x)), fmaxf(ml[2].x, ml[3].x));
+        if (Mn > -INFINITY) {
+            L *= exp2f(M - Mn);                              // M = -inf gives 0
+#pragma unroll
+            for (int i = 0; i < 4; ++i) if (ml[i].x > -INFINITY) L += ml[i].y * exp2f(ml[i].x - Mn);
+            M = Mn;
+        }
+    }
+    const float inv = L > 0.f ? 1.f / L : 0.f;
+    const int mg = w.m0 + g * 128 + m;
+    uint16_t* dst = out_row(out, w, min(mg, w.m_total - 1), plan.g_magic, G, q_heads, D);
+    // 64 columns at a time: 16 loads in flight per thread and piece (with 8 this step took 16 us, one latency after another)
+#pragma unroll 1
+    for (int h = 0; h < D / 64; ++h) {
+        float acc[64];
+#pragma unroll
+        for (int i = 0; i < 64; ++i) acc[i] = 0.f;
+#pragma unroll 1
+        for (int k = first; k <= last; ++k) {
+            if (plan.x[k] >= plan.x[k + 1]) continue;
+            float o[64], mk = m_own;
+            if (k == me) {
+                if (have_o) {
+                    tmem_ld32(tO + h * 64, o);
+                    tmem_ld32(tO + h * 64 + 32, o + 32);
+                    tmem_wait_ld();
+                }
+            } else {
+                const PfSlot<D> slot(plan, tail, k);
+                mk = __ldcg(slot.ml(g, m)).x;
+                const float4* po = slot.o(g, m) + h * 16 * 128;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {        // (of a piece without pages: left over from earlier, not used)
+                    const float4 v = __ldcg(po + i * 128);
+                    o[4 * i] = v.x; o[4 * i + 1] = v.y; o[4 * i + 2] = v.z; o[4 * i + 3] = v.w;
+                }
+            }
+            if (mk > -INFINITY) {
+                const float f = exp2f(mk - M) * inv;
+#pragma unroll
+                for (int i = 0; i < 64; ++i) acc[i] += o[i] * f;
+            }
+        }
+        if (mg < w.m_total) {
+            store_row32(dst + h * 64, acc);
+            store_row32(dst + h * 64 + 32, acc + 32);
+        }
+    }
+}
 
 template <int D>
 __global__ void __launch_bounds__(PF_THREADS, 1)
-prefill_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t* __restrict__ Q,
-               const int* __restrict__ q_pos, int n_q_arg, int q_heads, uint16_t* __restrict__ out) {
+prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant__ PfPlan plan, int layer0, int n_layers,
+               const uint16_t* __restrict__ Q, const int* __restrict__ q_pos, int n_q_arg, int q_heads, uint16_t* __restrict__ out) {
     constexpr int KB = D / 64;                 // 64-element (128-byte) blocks along d
     constexpr int TILE_BYTES = 128 * D * 2;    // one K or V page of one head, or one 128-row Q tile
-    constexpr int HALF = D / 2;
-    extern __shared__ unsigned char smem_raw[];
-    PfShared& sh = *reinterpret_cast<PfShared*>(smem_raw);
-    unsigned char* tiles_base = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + sizeof(PfShared) + 1023) & ~(uintptr_t)1023);
-    unsigned char* sQ = tiles_base;                           // [2 tiles][KB][128 rows][128 B]
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* sQ = smem_raw;                             // [2 tiles][KB][128 rows][128 B]
     unsigned char* ring = sQ + 2 * TILE_BYTES;                // [stage][KB][128 keys][128 B]
+    unsigned char* s_cs = ring + PF_RING * TILE_BYTES;        // [2 tiles] rotation factors
+    PfShared& sh = *reinterpret_cast<PfShared*>(s_cs + 2 * PF_CS_BYTES);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int G = q_heads / b.kv_heads;
-    const int hk = blockIdx.y;
-    const int prob = blockIdx.z;
-    const int ci = prob / n_layers, li = prob % n_layers;
-    const int layer = layer0 + li;
-    const SvlmAttendView& vw = b.view[ci];
-    // rows of this problem: n_q_arg per problem, or (caches with chunks of different lengths) the cache's own count
-    const int n_q = b.q_varlen ? b.q_cnt[ci] : n_q_arg;
-    const size_t q_row0 = b.q_varlen ? (size_t)b.q_off[ci] : (size_t)prob * n_q_arg;   // first row in Q and out
-    const size_t p_row0 = b.q_varlen ? (size_t)b.q_off[ci] : (size_t)ci * n_q_arg;     // first row in q_pos
-    if ((int)(blockIdx.x >> 1) * PF_ROWS >= n_q * G) return;   // a shorter chunk: both CTAs of the pair leave at once
-    const int m_total = n_q * G;
-    const unsigned rank = cluster_rank();      // which half of the pages this CTA takes
-    const int m0 = (blockIdx.x >> 1) * PF_ROWS;
-    const int r_lo = m0 / G, r_hi = min(n_q - 1, (m0 + PF_ROWS - 1) / G);
-
-    // The CTA's query rows and positions are read a few microseconds from now, in four dependent rounds of loads:
-    // ask for their lines now, so that those rounds find them in L2 (one token's G heads are G * D * 2 contiguous bytes).
-    {
-        const int line_per_tok = (G * D * 2 + 127) / 128;
-        for (int i = threadIdx.x; i < (r_hi - r_lo + 1) * line_per_tok; i += PF_THREADS) {
-            const int tk = i / line_per_tok, ln = i % line_per_tok;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(Q + ((q_row0 + r_lo + tk) * q_heads + hk * G) * D) + ln * 128));
-        }
-        if (threadIdx.x < 32)
-            for (int i = threadIdx.x * 32; i < (r_hi - r_lo + 1) * (b.rope_mode == 0 ? 1 : 3); i += 32 * 32)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(q_pos + (p_row0 + r_lo) * (b.rope_mode == 0 ? 1 : 3) + i));
+    volatile int* abort_flag = &sh.abort_flag;
+    if (smem_u32(smem_raw) & 1023) {           // swizzled tiles need a 1024-byte aligned base; same in every CTA
+        if (threadIdx.x == 0) atomicCAS(const_cast<int*>(&b.view[0].ctrl->status), 0, -4);   // SVLM_ERR_CUDA
+        return;
     }
-    const int n_tiles = min(vw.ctrl->n_tiles, PF_MAX_TILES);
-    const long long gid_q0 = vw.ctrl->n_total - n_q;
-    const long long shift = vw.ctrl->shift_total;
-    const unsigned wait_limit = vw.ctrl->wait_limit;
 
-    // ---- set-up: barriers, TMEM, page list ------------------------------------------------------
+    // ---- set-up: barriers, TMEM ------------------------------------------------------
     if (threadIdx.x == 0) {
-        for (int s = 0; s < PF_RING; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], PF_ISSUERS); }   // every issuer releases a page
-        for (int s = 0; s < 2; ++s) { mbar_init(&sh.s_full[s], 1); mbar_init(&sh.p_full[s], 128); }
-        mbar_init(&sh.all_done, PF_ISSUERS);
+        for (int s = 0; s < PF_RING; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 2); }   // both issuers release a page
+        for (int s = 0; s < 2; ++s) { mbar_init(&sh.s_full[s], 1); mbar_init(&sh.all_done[s], 1); }
         sh.abort_flag = 0;
         mbar_init_fence();
-    }
-    for (int i = threadIdx.x; i < n_tiles; i += PF_THREADS) {
-        const SvlmTile tl = vw.tiles[i];
-        const int skip = tl.min_gid > gid_q0 + r_hi;
-        const int mask = tl.lo > 0 || tl.hi < SVLM_PAGE || tl.max_gid > gid_q0 + r_lo;
-        sh.tile[i] = (unsigned short)(tl.page | (mask << 14) | (skip << 15));
     }
     if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-
-    __syncthreads();   // barriers and page list are ready: the producer may start
-
-    const size_t head_row0 = ((size_t)layer * b.kv_heads + hk) * b.n_slots;
-    // this CTA's share of the processed pages: [p0, p1) of the non-skipped ones
-    int n_all = 0;
-    for (int j = 0; j < n_tiles; ++j) n_all += !(sh.tile[j] >> 15);
-    const int half = (n_all + 1) / 2;
-    const int p0 = rank == 0 ? 0 : half, p1 = rank == 0 ? half : n_all;
-    const int n_proc = p1 - p0;
-    volatile int* abort_flag = &sh.abort_flag;
-
-    // K/V producer state (warp 8, lane 0); the first PF_RING - 2 loads go out before the query prologue,
-    // the last two stages are borrowed by the prologue for the rotation factors
-    int pr_j = 0, pr_pi = 0, pr_n = 0;
-    bool pr_ok = true;
-    auto produce = [&](int limit) {   // issue loads until `limit` ring items have been issued in total
-        const void* tmK = vw.tmaps;
-        const void* tmV = reinterpret_cast<const unsigned char*>(vw.tmaps) + 128;
-        while (pr_ok && pr_n < limit && pr_j < n_tiles) {
-            const unsigned t = sh.tile[pr_j];
-            if (t >> 15) { ++pr_j; continue; }
-            if (pr_pi < p0 || pr_pi >= p1) { ++pr_pi; ++pr_j; continue; }
-            const int y = (int)(head_row0 + (size_t)(t & 0x3FFF) * SVLM_PAGE);
-            const int kv = pr_n & 1;      // even items are K pages, odd items V pages of the same page
-            const int st = pr_n % PF_RING;
-            pr_ok = mbar_wait(&sh.empty[st], ((pr_n / PF_RING) & 1) ^ 1, abort_flag, wait_limit);   // first pass: already free
-            if (!pr_ok) break;
-            mbar_expect_tx(&sh.full[st], TILE_BYTES);
-#pragma unroll
-            for (int kb = 0; kb < KB; ++kb)
-                tma_load_2d(ring + st * TILE_BYTES + kb * (128 * 128), kv ? tmV : tmK, kb * 64, y, &sh.full[st]);
-            ++pr_n;
-            if (kv) { ++pr_pi; ++pr_j; }
-        }
-    };
-    if (warp == 8 && lane == 0) produce(PF_RING - 2);
-
-    // ---- query tiles: rotate at q_pos - shift_total, round to bf16, store K-major swizzled -------
-    // (1) rotation factors of the CTA's tokens, all threads: [token][pair] (cos, sin) in the last two ring
-    //     stages (the rows of a token's G heads share them); with few heads per KV head there are too many
-    //     tokens for that space and every thread looks its own factors up instead
-    float2* s_cs = reinterpret_cast<float2*>(ring + (PF_RING - 2) * TILE_BYTES);
-    const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
-    const int n_tok = r_hi - r_lo + 1;
-    const bool cs_shared = (size_t)n_tok * HALF * sizeof(float2) <= (size_t)2 * TILE_BYTES;
-    if (cs_shared) {
-        constexpr int UN = 8;   // entries per thread in flight: positions first, then the table look-ups
-        const int n_ent = n_tok * HALF;
-        const int pw = b.rope_mode == 0 ? 1 : 3;
-        for (int base = 0; base < n_ent; base += PF_THREADS * UN) {
-            long long cpos[UN];
-#pragma unroll
-            for (int u = 0; u < UN; ++u) {
-                const int i = base + u * PF_THREADS + threadIdx.x;
-                if (i < n_ent) {
-                    const int tk = i / HALF, pair = i % HALF;
-                    const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
-                    cpos[u] = (long long)__ldg(q_pos + (p_row0 + r_lo + tk) * pw + axis) - shift;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < UN; ++u) {
-                const int i = base + u * PF_THREADS + threadIdx.x;
-                if (i < n_ent) {
-                    // a token's factors are read back 64 bytes per thread at a 64-byte lane stride: the 16-byte
-                    // chunks are XOR-swizzled so that eight such lanes hit eight different bank groups
-                    const int tk = i / HALF, pair = i % HALF;
-                    s_cs[tk * HALF + ((((pair >> 1) ^ (pair >> 4)) << 1) | (pair & 1))] =
-                        svlm_rope_cs(tab, HALF, pair, cpos[u], b.theta[pair]);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    // (2) rotation of the 256 rows, coalesced: a work item is (row, chunk c of 8 pairs) = the 16-byte chunk c of the
-    //     row's low half with its partner chunk of the high half; consecutive threads take consecutive chunks of a
-    //     row, so global loads and factor look-ups of a warp touch few lines and several items are in flight.
-    if (warp < 8) {
-        constexpr int CH = HALF / 8;               // chunks per half row
-        constexpr int ITEMS = PF_ROWS * CH, PER = ITEMS / 256, UN = 4;
-        static_assert(PER % UN == 0, "items per thread");
-#pragma unroll 1
-        for (int it0 = 0; it0 < PER; it0 += UN) {
-            uint4 lo4[UN], hi4[UN];
-            int row[UN], c8v[UN], tok[UN];
-#pragma unroll
-            for (int u = 0; u < UN; ++u) {         // all loads of the batch first
-                const int item = (it0 + u) * 256 + threadIdx.x;
-                row[u] = item / CH; c8v[u] = item % CH;
-                const int mg = m0 + row[u];
-                const bool live = mg < m_total;
-                const int r = live ? mg / G : r_lo, h = live ? mg % G : 0;
-                tok[u] = r;
-                const uint4* src = reinterpret_cast<const uint4*>(Q + ((q_row0 + r) * q_heads + hk * G + h) * D);
-                lo4[u] = live ? __ldg(src + c8v[u]) : make_uint4(0, 0, 0, 0);
-                hi4[u] = live ? __ldg(src + CH + c8v[u]) : make_uint4(0, 0, 0, 0);
-            }
-#pragma unroll
-            for (int u = 0; u < UN; ++u) {
-                const int c8 = c8v[u], g = row[u] >> 7, m = row[u] & 127;
-                const float2* cs_row = s_cs + (size_t)(tok[u] - r_lo) * HALF;
-                const int* qp = q_pos + (p_row0 + tok[u]) * (b.rope_mode == 0 ? 1 : 3);
-                const unsigned* lw = reinterpret_cast<const unsigned*>(&lo4[u]);
-                const unsigned* hw = reinterpret_cast<const unsigned*>(&hi4[u]);
-                float2 cs8[8];
-                if (cs_shared) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float4 v = *reinterpret_cast<const float4*>(cs_row + (((4 * c8 + j) ^ (c8 >> 1)) << 1));
-                        cs8[2 * j] = make_float2(v.x, v.y);
-                        cs8[2 * j + 1] = make_float2(v.z, v.w);
-                    }
-                } else {
-#pragma unroll 1
-                    for (int i = 0; i < 8; ++i) {      // direct look-ups (too many tokens for the shared table)
-                        const int pair = c8 * 8 + i;
-                        const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
-                        const float2 v = svlm_rope_cs(tab, HALF, pair, (long long)qp[b.rope_mode == 0 ? 0 : axis] - shift, b.theta[pair]);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) if (q == i) cs8[q] = v;
-                    }
-                }
-                unsigned lo_o[4], hi_o[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float xl[2] = {__uint_as_float(lw[j] << 16), __uint_as_float(lw[j] & 0xffff0000u)};
-                    float xh[2] = {__uint_as_float(hw[j] << 16), __uint_as_float(hw[j] & 0xffff0000u)};
-                    float ol[2], oh[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float2 cs = cs8[2 * j + e];
-                        ol[e] = xl[e] * cs.x - xh[e] * cs.y;
-                        oh[e] = xh[e] * cs.x + xl[e] * cs.y;
-                    }
-                    lo_o[j] = pack2(ol[0], ol[1]);
-                    hi_o[j] = pack2(oh[0], oh[1]);
-                }
-                // element e of the row lives in block e/64, 16-byte chunk (e%64)/8, XOR-swizzled by row&7
-                unsigned char* sQg = sQ + g * TILE_BYTES;
-                const int e_lo = c8 * 8, e_hi = HALF + c8 * 8;
-                unsigned char* dl = sQg + (e_lo / 64) * (128 * 128) + m * 128 + ((((e_lo % 64) / 8) ^ (m & 7)) << 4);
-                unsigned char* dh = sQg + (e_hi / 64) * (128 * 128) + m * 128 + ((((e_hi % 64) / 8) ^ (m & 7)) << 4);
-                *reinterpret_cast<uint4*>(dl) = make_uint4(lo_o[0], lo_o[1], lo_o[2], lo_o[3]);
-                *reinterpret_cast<uint4*>(dh) = make_uint4(hi_o[0], hi_o[1], hi_o[2], hi_o[3]);
-            }
-        }
-    }
-    fence_proxy_async();   // the query tiles feed the tensor core, the borrowed ring stages get TMA writes next
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const unsigned tmem = sh.tmem_base;
-    // tile g: S (then P as bf16 pairs in its first 64 columns) at columns 128 g, O at 256 + 128 g
 
-    if (warp == 8) {
-        // ================= TMA producer: K(0) V(0) K(1) V(1) ... through one ring =================
-        if (lane == 0) produce(0x7fffffff);
-        __syncwarp();
-    } else if (warp >= 9) {
-        // ================= MMA issuers: warp 9 for tile A, warp 10 for tile B =================
-        // Per tile the order is S(0) | PV(j) S(j+1) | ...: the tensor pipe executes one thread's instructions in
-        // order, so S(j+1) overwrites the columns of P(j) only after PV(j) has read them.  Two issuing threads keep
-        // the pipe fed while one of them sits in a wait.
-        // The whole warp runs the loop (waits, descriptor arithmetic: warp-uniform values the compiler can keep in
-        // uniform registers); one elected lane executes the tcgen05 instructions.
-        if (warp - 9 < PF_ISSUERS) {
-            const int g0 = warp - 9;
+    if (warp >= 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        PfWalk walk;
+        walk.begin(plan);
+        bool ok = true;
+        if (warp == 8) {
+            // ================= TMA producer: K(0) V(0) K(1) V(1) ... through one ring, unit after unit =================
+            unsigned item = 0;
+            while (walk.more(plan)) {
+                const PfSeg seg = walk.next(plan);
+                const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
+                const PfWork w = pf_work(b, seg, rows, plan.g_magic, G, pf_ask(b, rows));
+                const void* tmK = w.vw->tmaps;
+                const void* tmV = reinterpret_cast<const unsigned char*>(w.vw->tmaps) + 128;
+                PfPages pages;
+                pages.begin();
+                for (int j = 0; j < w.n_proc && ok; ++j) {
+                    const int y = (int)(rows.head_row0 + (size_t)(pages.next(w, 0) & 0x3FFF) * SVLM_PAGE);
+                    if (lane == 0) {
+#pragma unroll
+                        for (int kv = 0; kv < 2; ++kv) {
+                            const unsigned st = (item + kv) % PF_RING;
+                            if (ok) ok = mbar_wait(&sh.empty[st], (((item + kv) / PF_RING) & 1) ^ 1, abort_flag, w.wait_limit);   // first pass: already free
+                            if (!ok) break;
+                            mbar_expect_tx(&sh.full[st], TILE_BYTES);
+#pragma unroll
+                            for (int kb = 0; kb < KB; ++kb)
+                                tma_load_2d(ring + st * TILE_BYTES + kb * (128 * 128), kv ? tmV : tmK, kb * 64, y, &sh.full[st]);
+                        }
+                    }
+                    ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                    item += 2;
+                }
+                if (!ok) break;
+            }
+        } else if (warp < 11) {
+            // ================= MMA issuer of tile g =================
+            // Per tile the order is S(0) | PV(j) S(j+1) | ...: the tensor pipe executes one thread's instructions in
+            // order, so S(j+1) overwrites the columns of P(j) only after PV(j) has read them.  The whole warp runs the
+            // loop (waits, descriptor arithmetic: warp-uniform values the compiler can keep in uniform registers); one
+            // elected lane executes the tcgen05 instructions.  The number of named-barrier operations depends on the
+            // work list only, never on whether a wait has run out.
+            const int g = warp - 9;
             const unsigned tmem = __shfl_sync(0xffffffffu, sh.tmem_base, 0);
             const bool leader = elect_one();
             constexpr unsigned IDESC_S = make_idesc(128, 128, 0);
             constexpr unsigned IDESC_O = make_idesc(128, D, 1);
             // descriptors: the 14-bit start-address field counts 16-byte units, so moving inside a tile is an
             // addition to the low word (all tile addresses stay below the field's range: shared memory is 228 KB)
-            const unsigned long long dq = smem_desc(smem_u32(sQ), 16, 1024);                    // Q, K: K-major
+            const unsigned long long dq = smem_desc(smem_u32(sQ + g * TILE_BYTES), 16, 1024);   // Q, K: K-major
             const unsigned long long dk = smem_desc(smem_u32(ring), 16, 1024);
             const unsigned long long dv = smem_desc(smem_u32(ring), 128 * 128, 1024);           // V: MN-major
-            // every wait gives the same answer in all lanes, so the warp stays converged
-            auto wait_bar = [&](void* bar, unsigned parity) {   // one lane polls, all lanes get the answer
+            unsigned wait_limit = 0;
+            auto wait_item = [&](unsigned n) {                      // one lane polls, all lanes get the answer
                 int r = 1;
-                if (lane == 0) r = mbar_wait(bar, parity, abort_flag, wait_limit);
+                if (lane == 0) r = mbar_wait(&sh.full[n % PF_RING], (n / PF_RING) & 1, abort_flag, wait_limit);
                 return __shfl_sync(0xffffffffu, r, 0) != 0;
             };
-            auto wait_item = [&](int n) { return wait_bar(&sh.full[n % PF_RING], (n / PF_RING) & 1); };
-            auto issue_S = [&](int g, int j, bool release) {      // S_g = Q_g K(j)^T; K(j) is ring item 2j
-                const int st = (2 * j) % PF_RING;
-                const unsigned long long a0 = dq + (unsigned)(g * TILE_BYTES >> 4), b0 = dk + (unsigned)(st * TILE_BYTES >> 4);
+            auto issue_S = [&](unsigned n) {                        // S = Q K^T, K is ring item n
+                const unsigned st = n % PF_RING;
+                const unsigned long long b0 = dk + (unsigned)(st * TILE_BYTES >> 4);
                 if (leader) {
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks) {
                         const unsigned off = ((ks / 4) * (128 * 128) + (ks % 4) * 32) >> 4;
-                        tc_mma_ss(tmem + g * 128, a0 + off, b0 + off, IDESC_S, ks > 0);
+                        tc_mma_ss(tmem + g * 128, dq + off, b0 + off, IDESC_S, ks > 0);
                     }
                     tc_commit(&sh.s_full[g]);
-                    if (release) tc_commit(&sh.empty[st]);
+                    tc_commit(&sh.empty[st]);
                 }
                 __syncwarp();
             };
-            auto issue_PV = [&](int g, int j, bool release) {     // O_g += P_g V(j); V(j) is ring item 2j+1
-                const int st = (2 * j + 1) % PF_RING;
+            auto issue_PV = [&](unsigned n, int half, bool accumulate) {   // O += P V for 64 keys, V is ring item n
+                const unsigned st = n % PF_RING;
                 const unsigned long long b0 = dv + (unsigned)(st * TILE_BYTES >> 4);
                 if (leader) {
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)      // 128 keys, 16 per MMA: A = 8 TMEM columns of bf16 pairs
-                        tc_mma_ts(tmem + 256 + g * 128, tmem + g * 128 + ks * 8, b0 + (unsigned)(ks * 2048 >> 4), IDESC_O,
-                                  (j > 0) || (ks > 0));
-                    if (release) tc_commit(&sh.empty[st]);
+                    for (int k = 0; k < 4; ++k) {                   // 16 keys per MMA: A = 8 TMEM columns of bf16 pairs
+                        const int ks = half * 4 + k;
+                        tc_mma_ts(tmem + 256 + g * 128, tmem + g * 128 + ks * 8, b0 + (unsigned)(ks * 2048 >> 4), IDESC_O, accumulate || k > 0);
+                    }
+                    if (half) tc_commit(&sh.empty[st]);
                 }
                 __syncwarp();
             };
-            // with one issuer the thread serves both tiles in turn and releases a page after tile B's use of it
-            constexpr int NG = 3 - PF_ISSUERS;      // tiles per issuer: 1 or 2
-            bool ok = true;
-            if (n_proc > 0) {
-                ok = wait_item(0);
-                if (ok) {
-                    tc_fence_after();
-#pragma unroll
-                    for (int i = 0; i < NG; ++i) issue_S(g0 + i, 0, i == NG - 1);
-                }
-            }
-            for (int j = 0; j < n_proc && ok; ++j) {
-                ok = wait_item(2 * j + 1);                                                   // V(j)
-                if (ok && j + 1 < n_proc) ok = wait_item(2 * j + 2);                         // K(j+1)
-#pragma unroll
-                for (int i = 0; i < NG && ok; ++i) {
-                    ok = wait_bar(&sh.p_full[g0 + i], j & 1);                                 // P(j)
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_PV(g0 + i, j, i == NG - 1);
-                    if (j + 1 < n_proc) issue_S(g0 + i, j + 1, i == NG - 1);
-                }
-            }
-            if (ok && leader) {
-                if (n_proc > 0) tc_commit(&sh.all_done);
-                else mbar_arrive(&sh.all_done);   // nothing was issued: nothing to track
-            }
-        }
-        __syncwarp();
-    } else {
-        // ================= softmax groups: one thread per row of tile g =================
-        const int g = warp >> 2;
-        const int m = threadIdx.x & 127;
-        const int mg = m0 + g * 128 + m;
-        const int r = min(mg / G, n_q - 1);
-        const unsigned lane_base = (unsigned)((warp & 3) * 32) << 16;
-        const unsigned tS = tmem + g * 128 + lane_base, tO = tmem + 256 + g * 128 + lane_base;
-        const float c = 1.4426950408889634f * rsqrtf((float)D);
-        const unsigned short* mrow = sh.minrow[g];
-        float m_ref = -INFINITY, l = 0.f;
-        int pi = 0, it = 0;
-        bool ok = true;
-        for (int j = 0; j < n_tiles && ok; ++j) {
-            const unsigned t = sh.tile[j];
-            if (t >> 15) continue;
-            if (pi < p0 || pi >= p1) { ++pi; continue; }
-            ++pi;
-            const bool masked = (t >> 14) & 1;
-            unsigned vlo = 0, vlen = SVLM_PAGE;
-            if (masked) {
-                // Column m's stream ordinal relative to the first query token (clamped), shared through
-                // shared memory; it grows with the column, so the columns this row may see, valid ones with
-                // ordinal <= the row's, form the interval [lo, bound) found by bisection.
-                const SvlmTile tl = vw.tiles[j];
-                unsigned short mr = 0xFFFF;
-                if (m >= tl.lo && m < tl.hi) {
-                    const long long rel = vw.slot_gid[tl.page * SVLM_PAGE + m] - gid_q0;
-                    mr = rel <= 0 ? 0 : (rel > 0xFFF0ll ? 0xFFF0 : (unsigned short)rel);
-                }
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + g));   // the previous masked page's readers are done
-                sh.minrow[g][m] = mr;
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + g));
-                int a = tl.lo, e = tl.hi;
-                while (a < e) {
-                    const int mid = (a + e) >> 1;
-                    if ((unsigned)mrow[mid] <= (unsigned)r) a = mid + 1; else e = mid;
-                }
-                vlo = tl.lo;
-                vlen = a - tl.lo;
-            }
-            ok = mbar_wait(&sh.s_full[g], it & 1, abort_flag, wait_limit);
-            if (!ok) break;
-            tc_fence_after();
-            float rowsum, corr, m_new;
-            if (masked) softmax_page<true>(tS, tO, D, vlo, vlen, c, m_ref, it > 0, rowsum, corr, m_new);
-            else softmax_page<false>(tS, tO, D, vlo, vlen, c, m_ref, it > 0, rowsum, corr, m_new);
-            tmem_wait_st();
-            l = l * corr + rowsum;
-            m_ref = m_new;
-            tc_fence_before();
-            mbar_arrive(&sh.p_full[g]);
-            ++it;
-        }
-        if (ok) ok = mbar_wait(&sh.all_done, 0, abort_flag, wait_limit);
-        tc_fence_after();
-
-        // ---- hand-over between the two CTAs of the cluster, then the output ------------------------
-        // CTA k of the pair finishes tile k.  Both warpgroups work on both steps, each on one half of the head
-        // dimension (a warp reaches its TMEM lane quadrant in either tile): first tile 1-k's (O, m, l) goes to
-        // the partner, then tile k's accumulator is merged with what the partner sent and written out.  The
-        // exchange area is the K/V ring, idle once a CTA's MMAs have completed (cluster barrier #1 says so for
-        // both); a row's (m, l) reaches the other warpgroup through the same area.
-        float* xo = reinterpret_cast<float*>(ring);                      // [D/4 chunks][128 rows] float4
-        float* xml = xo + (size_t)128 * D;                               // [128 rows][2]: the partner's (m, l)
-        float2* lml = reinterpret_cast<float2*>(xml + 2 * 128);          // [2 tiles][128 rows]: this CTA's (m, l)
-        const bool mine = n_proc > 0;                                    // this CTA processed pages
-        lml[g * 128 + m] = make_float2(ok && mine ? m_ref : -INFINITY, ok && mine ? l : 0.f);
-        cluster_sync_all();   // #1: neither CTA needs its ring any more; (m, l) of every row is visible
-        const int gk = (int)rank, gs = gk ^ 1;                           // tile kept, tile sent
-        constexpr int QH = D / 64;                                       // 32-column chunks of O per half
-        {
-            const unsigned tOs = tmem + 256 + gs * 128 + lane_base;
-            const unsigned dst_o = map_to_rank(xo, rank ^ 1), dst_ml = map_to_rank(xml, rank ^ 1);
-#pragma unroll 1
-            for (int q4 = g * QH; q4 < (g + 1) * QH; ++q4) {
-                float o[32];
-                if (mine) { tmem_ld32(tOs + q4 * 32, o); tmem_wait_ld(); }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float4 v = mine ? make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3])
-                                          : make_float4(0.f, 0.f, 0.f, 0.f);
-                    st_cluster_v4(dst_o + (unsigned)(((q4 * 8 + i) * 128 + m) * 16), v);
-                }
-            }
-            if (g == 0) st_cluster_v2(dst_ml + (unsigned)(m * 8), lml[gs * 128 + m]);
-        }
-        cluster_sync_all();   // #2: the partner's rows have arrived
-        if (ok) {
-            const unsigned tOk = tmem + 256 + gk * 128 + lane_base;
-            const int mgk = m0 + gk * 128 + m;
-            const int rk = min(mgk / G, n_q - 1);
-            const float mb = xml[m * 2], lb = xml[m * 2 + 1];
-            const float2 own = lml[gk * 128 + m];
-            const float ma = own.x, la = own.y;
-            const float M = fmaxf(ma, mb);
-            const float fa = ma == -INFINITY ? 0.f : exp2f(ma - M), fb = mb == -INFINITY ? 0.f : exp2f(mb - M);
-            const float L = la * fa + lb * fb;
-            const float inv = L > 0.f ? 1.f / L : 0.f;
-            const float ga = fa * inv, gb = fb * inv;
-            const bool live = mgk < m_total;
-            uint16_t* dst = out + ((q_row0 + rk) * q_heads + hk * G + (mgk % G)) * D;
-#pragma unroll 1
-            for (int q4 = g * QH; q4 < (g + 1) * QH; ++q4) {
-                float o[32];
-                if (mine) { tmem_ld32(tOk + q4 * 32, o); tmem_wait_ld(); }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float4 pb = *reinterpret_cast<const float4*>(xo + (size_t)((q4 * 8 + i) * 128 + m) * 4);
-                    o[4 * i] = (ma > -INFINITY ? o[4 * i] * ga : 0.f) + (mb > -INFINITY ? pb.x * gb : 0.f);
-                    o[4 * i + 1] = (ma > -INFINITY ? o[4 * i + 1] * ga : 0.f) + (mb > -INFINITY ? pb.y * gb : 0.f);
-                    o[4 * i + 2] = (ma > -INFINITY ? o[4 * i + 2] * ga : 0.f) + (mb > -INFINITY ? pb.z * gb : 0.f);
-                    o[4 * i + 3] = (ma > -INFINITY ? o[4 * i + 3] * ga : 0.f) + (mb > -INFINITY ? pb.w * gb : 0.f);
-                }
-                if (live) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        uint4 v;
-                        v.x = pack2(o[8 * k], o[8 * k + 1]);
-                        v.y = pack2(o[8 * k + 2], o[8 * k + 3]);
-                        v.z = pack2(o[8 * k + 4], o[8 * k + 5]);
-                        v.w = pack2(o[8 * k + 6], o[8 * k + 7]);
-                        *reinterpret_cast<uint4*>(dst + q4 * 32 + 8 * k) = v;
+            unsigned item = 0;
+            bool first_unit = true;
+            while (walk.more(plan)) {
+                const PfSeg seg = walk.next(plan);
+                const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
+                const PfWork w = pf_work(b, seg, rows, plan.g_magic, G, pf_ask(b, rows));
+                const bool more = walk.more(plan);
+                wait_limit = w.wait_limit;
+                const int n = w.n_proc;
+                if (ok && n > 0) ok = wait_item(item);
+                bar_sync(BAR_Q + g, 160);
+                if (g == 0) { if (!first_unit) bar_sync(BAR_TURN_A, 64); }
+                else bar_sync(BAR_TURN_B, 64);
+                if (ok && n > 0) { tc_fence_after(); issue_S(item); }
+                if (g == 0) bar_arrive(BAR_TURN_B, 64);
+                else if (n > 0) bar_arrive(BAR_P1, 192);
+                else if (more) bar_arrive(BAR_TURN_A, 64);
+                for (int j = 0; j < n; ++j) {
+                    if (ok) ok = wait_item(item + 2 * j + 1);                           // V(j)
+                    if (ok && j + 1 < n) ok = wait_item(item + 2 * j + 2);              // K(j+1)
+                    bar_sync(BAR_P1 + g, 192);
+                    if (ok) { tc_fence_after(); issue_PV(item + 2 * j + 1, 0, j > 0); }
+                    bar_sync(BAR_P2 + g, 160);
+                    if (ok) {
+                        tc_fence_after();
+                        issue_PV(item + 2 * j + 1, 1, true);
+                        if (j + 1 < n) issue_S(item + 2 * j + 2);
                     }
+                    if (g == 0) bar_arrive(BAR_P1 + 1, 192);
+                    else if (j + 1 < n) bar_arrive(BAR_P1, 192);
+                    else if (more) bar_arrive(BAR_TURN_A, 64);
                 }
+                if (leader && ok) {
+                    if (n > 0) tc_commit(&sh.all_done[g]);
+                    else mbar_arrive(&sh.all_done[g]);              // nothing was issued: nothing to track
+                }
+                __syncwarp();
+                item += 2 * n;
+                first_unit = false;
             }
         }
-    }
-    if (warp >= 8) {          // the producer and issuer warps take part in the two cluster barriers as well
-        cluster_sync_all();
-        cluster_sync_all();
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        // ================= softmax warpgroups: one thread per row of tile g =================
+        const int g = warp >> 2, m = threadIdx.x & 127;
+        const unsigned tS = sh.tmem_base + g * 128 + ((unsigned)((warp & 3) * 32) << 16), tO = tS + 256;
+        constexpr float c = D == 128 ? 0.12751743082459868f : 0.18033688011112042f;      // log2(e) / sqrt(D)
+        unsigned phases = 0;                  // parities of the barriers this group waits on: bit 0 S, bit 1 end of a unit
+        bool ok = true;
+        PfGroup& gr = sh.group[g];
+        unsigned char* sQg = sQ + g * TILE_BYTES;
+        float* cs_g = reinterpret_cast<float*>(s_cs + g * PF_CS_BYTES);
+        float m_ref = -INFINITY, l = 0.f;
+        if (m == 0) { gr.walk.begin(plan); gr.merge_later = -1; gr.more = gr.walk.more(plan); gr.seg.a = 0; gr.seg.e = PF_FRAC; }
+        bar_sync(BAR_WG + g, 128);
+        while (gr.more) {
+            bar_sync(BAR_WG + g, 128);        // everybody is through with the previous segment's fields
+            {
+                PfWalk walk = gr.walk;
+                const PfSeg seg = walk.next(plan);
+                const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
+                // in the order in which the answers are needed: the memory system takes them one after another
+                PfTileRotation<D> rot;
+                int t_lo, n_tok;
+                const bool staged = PfTileRotation<D>::staged(rows, g, plan.g_magic, G, t_lo, n_tok);
+                const PfAsk ask = pf_ask(b, rows);
+                if (staged) rot.load_pos(b, rows, q_pos, m, t_lo, n_tok, m / PfTileRotation<D>::HALF);
+                PfTileRotation<D>::load(rows, g, m, G, plan.g_magic, q_heads, Q, sQg);
+                const PfWork nw = pf_work(b, seg, rows, plan.g_magic, G, ask);
+                if (m == 0) { gr.seg = seg; gr.rows = rows; gr.w = nw; gr.more = walk.more(plan); }
+                if (staged) rot.stage(b, rows, nw.shift, q_pos, m, t_lo, n_tok, cs_g);
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                bar_sync(BAR_WG + g, 128);
+                if (m == 0) gr.walk = walk;
+                PfTileRotation<D>::rotate(b, rows, nw.shift, q_pos, g, m, plan.g_magic, G, t_lo, staged, cs_g, sQg);
+            }
+            fence_proxy_async();              // the tile feeds the tensor core
+            tc_fence_before();                // (the previous unit's accumulator has been read)
+            const PfWork& w = gr.w;
+            const int n_proc = w.n_proc;
+            // (arrive: the issuer takes it from here.  A thread that would not be held up by the tensor pipe afterwards
+            // has to sync instead, or it could arrive again before the issuer has seen the first time.)
+            if (ok && n_proc > 0) bar_arrive(BAR_Q + g, 160);
+            else bar_sync(BAR_Q + g, 160);
+            const int mt = gr.rows.m0 + g * 128;
+            const int r = min(pf_div(mt + m, plan.g_magic, G), gr.rows.n_q - 1), r_lo = min(pf_div(mt, plan.g_magic, G), gr.rows.n_q - 1);
+            m_ref = -INFINITY;
+            l = 0.f;
+            PfPages pages;
+            pages.begin();
+            for (int j = 0; j < n_proc; ++j) {
+                const unsigned pi = pages.next(w, r_lo);
+                const bool masked = (pi >> 28) & 1;
+                unsigned vlo = 0, vlen = SVLM_PAGE;
+                if (masked) {
+                    const int lo = (pi >> 14) & 127, hi = ((pi >> 21) & 127) + 1;
+                    int end = hi;
+                    if ((pi >> 29) & 1) {     // the new chunk's tokens: causal
+                        const long long* gp = w.vw->slot_gid + (size_t)(pi & 0x3FFF) * SVLM_PAGE + 4 * lane;
+                        const longlong2 ga = __ldg(reinterpret_cast<const longlong2*>(gp)), gb = __ldg(reinterpret_cast<const longlong2*>(gp) + 1);
+                        const long long gv[4] = {ga.x, ga.y, gb.x, gb.y};
+                        int v[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const long long rel = gv[k] - w.gid_q0;
+                            const int o = 4 * lane + k;
+                            v[k] = o < lo ? -1 : (o >= hi ? 0x7fffffff : (rel < 0 ? -1 : (int)min(rel, 0x7ffffffell)));
+                        }
+                        end = causal_end(v, r);
+                    }
+                    vlo = lo;
+                    vlen = max(end, lo) - lo;
+                }
+                if (ok) ok = mbar_wait(&sh.s_full[g], phases & 1, abort_flag, w.wait_limit);
+                phases ^= 1;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) {                    // keep the issuer's barriers supplied, in step with it
+                    bar_sync(BAR_P1 + g, 192);
+                    bar_sync(BAR_P2 + g, 160);
+                    continue;
+                }
+                tc_fence_after();
+                float rowsum, corr, m_new;
+                if (masked) softmax_page<true>(g, tS, tO, D, vlo, vlen, c, m_ref, j > 0, rowsum, corr, m_new);
+                else softmax_page<false>(g, tS, tO, D, vlo, vlen, c, m_ref, j > 0, rowsum, corr, m_new);
+                tmem_wait_st();
+                tc_fence_before();
+                bar_arrive(BAR_P2 + g, 160);
+                l = l * corr + rowsum;
+                m_ref = m_new;
+            }
+            if (ok) ok = mbar_wait(&sh.all_done[g], phases >> 1, abort_flag, w.wait_limit);
+            phases ^= 2;
+            ok = __all_sync(0xffffffffu, ok);
+            tc_fence_after();
+            const bool have_o = ok && n_proc > 0;
+            if (gr.seg.e - gr.seg.a == PF_FRAC) {                      // all of the unit's pages
+                const float inv = l > 0.f ? 1.f / l : 0.f;
+                const int mg = mt + m;
+                uint16_t* dst = out_row(out, gr.rows, min(mg, gr.rows.m_total - 1), plan.g_magic, G, q_heads, D);
+#pragma unroll 1
+                for (int q4 = 0; q4 < D / 32; ++q4) {
+                    float o[32];
+                    if (have_o) {
+                        tmem_ld32(tO + q4 * 32, o);
+                        tmem_wait_ld();
+                    }
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = have_o ? o[i] * inv : 0.f;
+                    if (mg < gr.rows.m_total) store_row32(dst + q4 * 32, o);
+                }
+            } else if (gr.more) {
+                int first, last;
+                const int pieces = count_pieces(plan, gr.seg.tail, blockIdx.x, first, last);
+                if (publish_piece<D>(sh, plan, gr.seg.tail, pieces, g, m, tO, m_ref, l, have_o) && m == 0) gr.merge_later = gr.seg.tail;
+            }
+        }
+        // What is left of cut units (outside the loop over segments: its code would cost the page loop registers).  The
+        // last segment's piece stays in TMEM when the others are already there, which is the usual case.
+        int mine_tail = -1;
+        bool own = false;
+        const bool have_o = ok && gr.w.n_proc > 0;
+        if (gr.seg.e - gr.seg.a < PF_FRAC) {
+            const int tail = gr.seg.tail;
+            int first, last;
+            const int pieces = count_pieces(plan, tail, blockIdx.x, first, last);
+            bar_sync(BAR_WG + g, 128);
+            if (m == 0) {
+                unsigned n;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(plan.counters + tail * 2 + g) : "memory");
+                sh.last[g] = n == (unsigned)pieces - 1;
+            }
+            bar_sync(BAR_WG + g, 128);
+            own = sh.last[g] != 0;                                     // (then nobody else is left to arrive)
+            bar_sync(BAR_WG + g, 128);
+            if (own || publish_piece<D>(sh, plan, tail, pieces, g, m, tO, m_ref, l, have_o)) mine_tail = tail;
+        }
+        bar_sync(BAR_WG + g, 128);
+        for (int pass = 0; pass < 2; ++pass) {
+            const int tail = pass == 0 ? mine_tail : gr.merge_later;
+            if (tail < 0) continue;
+            const PfRows rows = pf_rows(b, plan, plan.tail + tail, n_q_arg, G, layer0, n_layers);
+            merge_pieces<D>(plan, tail, rows, g, m, G, q_heads, pass == 0 && own, tO, m_ref, l, have_o, out);
+        }
     }
 
     // ---- teardown ------------------------------------------------------------------------------
@@ -587,38 +1016,111 @@ prefill_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t* __re
             for (int s = 0; s < PF_RING; ++s)
                 for (unsigned p = 0; p < 2; ++p)
                     for (unsigned w = 0; w < (1u << 16) && !mbar_test(&sh.full[s], p); ++w) __nanosleep(32);
-            atomicCAS(const_cast<int*>(&vw.ctrl->status), 0, -5);   // SVLM_ERR_TIMEOUT
+            for (int i = 0; i < b.n_caches; ++i) atomicCAS(const_cast<int*>(&b.view[i].ctrl->status), 0, -5);   // SVLM_ERR_TIMEOUT
         }
         __syncthreads();
     }
     if (warp == 8) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sh.tmem_base), "r"(512));
     }
 }
 
 template <int D>
-constexpr size_t prefill_smem() { return sizeof(PfShared) + 1024 + (size_t)(2 + PF_RING) * 128 * D * 2; }
+constexpr size_t prefill_smem() { return (size_t)(2 + PF_RING) * 128 * D * 2 + 2 * PF_CS_BYTES + sizeof(PfShared); }
+
+// The work split of one launch (see the top of the file): whole units in rounds over the grid while at least two rounds
+// are left, the rest cut so that every CTA has the same number of expected pages.  pages: an estimate of every cache's
+// page count; a wrong one costs balance only.
+void make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, int G, const int* pages, int max_ctas, int& grid) {
+    plan.units = 0;
+    long long all = 0;                                     // pages of the whole launch
+    const int per_unit = n_layers * b.kv_heads;
+    auto rows_of = [&](int i) { return b.q_varlen ? b.q_cnt[i] : n_q; };
+    auto tiles_of = [&](int i) { return (rows_of(i) * G + PF_ROWS - 1) / PF_ROWS; };
+    // expected pages of row tile rt of cache i: the chunk's own pages behind its last row are invisible
+    auto cost = [&](int i, int rt) { return std::max(1, pages[i] - std::max(0, rows_of(i) - 1 - (rt * PF_ROWS + PF_ROWS - 1) / G) / SVLM_PAGE); };
+    for (int i = 0; i < b.n_caches; ++i) {
+        plan.off[i] = plan.units;
+        const int R = tiles_of(i);
+        plan.units += per_unit * R;
+        for (int rt = 0; rt < R; ++rt) all += (long long)per_unit * cost(i, rt);
+    }
+    plan.off[b.n_caches] = plan.units;
+    const int U = plan.units;
+    const bool cut = plan.slots != nullptr;
+    grid = (int)std::min<long long>(max_ctas, cut ? std::max<long long>(U, all / PF_MIN_PAGES) : U);
+    plan.rounds = std::max(0, U / grid - 1);
+    plan.tail = plan.rounds * grid;
+    const int nt = U - plan.tail;
+    if (!cut || grid == U || (grid < U && nt == grid && plan.rounds == 0)) {      // whole units only
+        for (int i = 0; i <= grid; ++i) plan.x[i] = (unsigned short)((long long)i * nt / grid * PF_FRAC);
+        return;
+    }
+    // walk the units in order, first to add up what the whole rounds give each CTA, then to cut the tail
+    int ci = 0, rt = 0, R = tiles_of(0), left = R * per_unit;    // position of unit u
+    auto step = [&] {
+        if (++rt == R) rt = 0;
+        if (--left == 0 && ci + 1 < b.n_caches) { ++ci; R = tiles_of(ci); left = R * per_unit; rt = 0; }
+    };
+    int load[PF_MAX_CTAS] = {};
+    for (int u = 0, at = 0; u < plan.tail; ++u) {
+        load[at] += cost(ci, rt);
+        if (++at == grid) at = 0;
+        step();
+    }
+    int tail_cost[2 * PF_MAX_CTAS];
+    for (int t = 0; t < nt; ++t) { tail_cost[t] = cost(ci, rt); step(); }
+    // The level at which every CTA ends, counting what beginning another unit costs: from below, raised by what a deal at
+    // that level leaves over.
+    double level = (double)all / grid;
+    for (int pass = 0; pass < 10; ++pass) {
+        int t = 0;
+        double rem = tail_cost[0];
+        for (int i = 0; i < grid; ++i) {
+            plan.x[i] = (unsigned short)(t < nt ? t * PF_FRAC + (int)((tail_cost[t] - rem) / tail_cost[t] * PF_FRAC + 0.5) : nt * PF_FRAC);
+            double room = level - load[i];
+            for (bool first = true; room > 0 && t < nt; first = false) {
+                if (!first && (room -= PF_PIECE) < PF_SNAP) break;
+                double take = std::min(room, rem);
+                if (rem - take < PF_SNAP) take = rem;                // no slivers
+                room -= take;
+                rem -= take;
+                if (rem <= 0 && ++t < nt) rem = tail_cost[t];
+            }
+        }
+        if (t >= nt) break;
+        double over = rem;
+        for (int k = t + 1; k < nt; ++k) over += tail_cost[k];
+        level += over / grid + 0.1;
+    }
+    plan.x[grid] = (unsigned short)(nt * PF_FRAC);                   // the last CTA takes what is left
+}
 
 template <int D>
 cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uint16_t* Q, const int* q_pos, int n_q,
-                   int q_heads, uint16_t* out, cudaStream_t st) {
+                   int q_heads, uint16_t* out, const int* pages, void* scratch, cudaStream_t st) {
     cudaError_t e = svlm_allow_smem<prefill_kernel<D>>(prefill_smem<D>());
     if (e != cudaSuccess) return e;
+    // the register split inside the kernel adds up only if the block is launched with exactly this many
+    static const bool regs_ok = [] {
+        cudaFuncAttributes a;
+        return cudaFuncGetAttributes(&a, prefill_kernel<D>) == cudaSuccess && a.numRegs == PF_REGS_LAUNCH;
+    }();
+    if (!regs_ok) return cudaErrorLaunchOutOfResources;
+    PfPlan plan;
+    plan.counters = static_cast<unsigned*>(scratch);
+    plan.slots = svlm_prefill_scratch_bytes(b.n_slots / SVLM_PAGE, D) > PF_HEAD_BYTES ? static_cast<unsigned char*>(scratch) + PF_HEAD_BYTES : nullptr;
     const int G = q_heads / b.kv_heads;
+    plan.g_magic = G > 1 && (unsigned long long)n_q * G * G < 0x100000000ull - 256ull * G ? (unsigned)((0x100000000ull + G - 1) / G) : 0u;   // (tiles reach past the last row)
+    int grid;
+    make_plan(plan, b, n_layers, n_q, G, pages, std::min(svlm_sm_count(), PF_MAX_CTAS), grid);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * ((n_q * G + PF_ROWS - 1) / PF_ROWS), b.kv_heads, b.n_caches * n_layers);
+    cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(PF_THREADS);
     cfg.dynamicSmemBytes = prefill_smem<D>();
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;     // the two CTAs that share the pages of one row tile
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, prefill_kernel<D>, b, layer0, n_layers, Q, q_pos, n_q, q_heads, out);
+    e = cudaLaunchKernelEx(&cfg, prefill_kernel<D>, b, plan, layer0, n_layers, Q, q_pos, n_q, q_heads, out);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -626,11 +1128,17 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
 
 bool svlm_prefill_supported(int n_pages, int group) { return n_pages <= PF_MAX_TILES && group >= 1; }
 
+// Arrival counters, and the slots for pieces of units where a cache is long enough for cutting to pay.
+size_t svlm_prefill_scratch_bytes(int n_pages, int head_dim) {
+    if (n_pages < 3 * PF_MIN_PAGES) return PF_HEAD_BYTES;
+    return PF_HEAD_BYTES + (size_t)2 * std::min(svlm_sm_count(), PF_MAX_CTAS) * (head_dim == 128 ? pf_slot_bytes<128>() : pf_slot_bytes<64>());
+}
+
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
-                                int n_q, int q_heads, void* out, cudaStream_t st) {
+                                int n_q, int q_heads, void* out, const int* pages, void* scratch, cudaStream_t st) {
     const cudaError_t e = b.head_dim == 128
-        ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, st)
-        : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, st);
+        ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, scratch, st)
+        : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, scratch, st);
     svlm_count_launch();
     return e;
 }

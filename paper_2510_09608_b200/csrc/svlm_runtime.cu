@@ -195,6 +195,17 @@ int make_list(svlm_cache* const* caches, int n_caches, SvlmCacheList& list) {
     return SVLM_OK;
 }
 
+// The host's idea of what a cache stores (it does not know the tokens' types, nor what a replayed graph has appended).
+void note_append(svlm_cache* c, int n) {
+    c->appended += n;
+    c->pending_n = n;
+    c->stored_est = std::min<long long>(c->stored_est + n, c->dev.capacity);
+}
+void note_evict(svlm_cache* c) {
+    c->stored_est = std::min<long long>(c->stored_est, (long long)c->dev.n_sink + c->dev.vision_window + c->dev.text_window);
+}
+int expected_pages(const svlm_cache* c) { return std::max(1, (int)std::min<long long>(c->stored_est / SVLM_PAGE + 1, c->dev.n_pages)); }
+
 int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void* Q, const int32_t* q_pos, int n_q,
                   int q_heads, void* out, const void* Knew = nullptr, const void* Vnew = nullptr) {
     svlm_cache* c0 = caches[0];
@@ -246,7 +257,9 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     }
     if (Knew) return SVLM_ERR_ARG;   // the fused step exists for the split-KV kernel only
     if (n_q >= 2 && svlm_prefill_supported(c0->dev.n_pages, group)) {
-        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, c0->stream));
+        int pages[SVLM_MAX_BATCH];
+        for (int i = 0; i < n_caches; ++i) pages[i] = expected_pages(caches[i]);
+        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, pages, c0->prefill_scratch, c0->stream));
         return SVLM_OK;
     }
     svlm_launch_attend_simple(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, c0->stream);
@@ -308,6 +321,8 @@ int svlm_cache_create(svlm_cache** out, int layers, int kv_heads, int head_dim, 
         // the per-layer kernel's tagged records: zero-filled here, afterwards written by that kernel alone
         A(dev_alloc(c, &c->decode_tagged, svlm_decode_tagged_bytes(kv_heads, head_dim, svlm_decode_splits(d.n_pages, kv_heads, 1))));
     }
+    A(dev_alloc(c, &c->prefill_scratch, svlm_prefill_scratch_bytes(d.n_pages, head_dim), false));
+    if (rc == SVLM_OK && cudaMemset(c->prefill_scratch, 0, svlm_prefill_counter_bytes) != cudaSuccess) rc = SVLM_ERR_CUDA;
     A(dev_alloc(c, &d.K, slab));
     A(dev_alloc(c, &d.V, slab));
     {
@@ -404,8 +419,7 @@ int svlm_cache_append(svlm_cache* c, int layer, const void* K, const void* V, co
         if (n > c->dev.capacity) return SVLM_ERR_CAPACITY;
         c->configured_locked = true;
         svlm_launch_append_meta(c->dev, token_type, pos, n, c->stream);
-        c->appended += n;
-        c->pending_n = n;
+        note_append(c, n);
     } else if (n != c->pending_n) {
         return SVLM_ERR_ORDER;
     }
@@ -432,8 +446,7 @@ int svlm_qkv_append(svlm_cache* c, int layer, const void* X, const void* W, int 
         if (n > c->dev.capacity) return SVLM_ERR_CAPACITY;
         c->configured_locked = true;
         svlm_launch_append_meta(c->dev, token_type, pos, n, c->stream);
-        c->appended += n;
-        c->pending_n = n;
+        note_append(c, n);
     } else if (n != c->pending_n) {
         return SVLM_ERR_ORDER;
     }
@@ -466,6 +479,7 @@ int svlm_cache_evict(svlm_cache* c) {
     if (!c) return SVLM_ERR_ARG;
     DeviceGuard guard(c->device);
     c->last_decode_layer = -1;
+    note_evict(c);
     svlm_launch_evict_meta(c->dev, c->stream);
     if (c->dev.contiguous) svlm_launch_evict_rotate(c->dev, c->stream);
     SVLM_CUDA(cudaGetLastError());
@@ -481,6 +495,7 @@ int svlm_cache_evict_batched(svlm_cache* const* caches, int n_caches) {
     bool rotate = false;
     for (int i = 0; i < n_caches; ++i) {
         caches[i]->last_decode_layer = -1;
+        note_evict(caches[i]);
         rotate = rotate || caches[i]->dev.contiguous;   // a cache with native positions never sets evict_moved
     }
     svlm_launch_evict_meta_batch(list, c0->stream);
@@ -506,8 +521,7 @@ int svlm_decode_step(svlm_cache* c, int layer, const void* K, const void* V, con
         c->configured_locked = true;
         c->last_decode_layer = -1;
         svlm_launch_append_meta(c->dev, token_type, pos, 1, c->stream);
-        c->appended += 1;
-        c->pending_n = 1;
+        note_append(c, 1);
     } else if (c->pending_n != 1) {
         return SVLM_ERR_ORDER;
     }
@@ -531,8 +545,7 @@ int svlm_decode_step_batched(svlm_cache* const* caches, int n_caches, int layer,
             svlm_cache* c = caches[i];
             c->configured_locked = true;
             c->last_decode_layer = -1;
-            c->appended += 1;
-            c->pending_n = 1;
+            note_append(c, 1);
         }
         svlm_launch_append_meta_batch(list, token_type, pos, 1, c0->stream);
     } else {
@@ -568,7 +581,9 @@ int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int laye
     }
     if (off > 0x7fffffffll) return SVLM_ERR_ARG;
     DeviceGuard guard(c0->device);
-    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, Q, q_pos, n_max, q_heads, out, c0->stream));
+    int pages[SVLM_MAX_BATCH];
+    for (int i = 0; i < n_caches; ++i) pages[i] = expected_pages(caches[i]);
+    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, Q, q_pos, n_max, q_heads, out, pages, c0->prefill_scratch, c0->stream));
     return SVLM_OK;
 }
 
