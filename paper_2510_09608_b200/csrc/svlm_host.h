@@ -17,7 +17,8 @@ struct svlm_cache {
     bool configured_locked = false;
     unsigned wait_limit_host = 0;  // source buffer of svlm_debug_set_wait_limit's copy
     unsigned char* decode_tagged = nullptr;   // per-layer decode kernel: epochs and tagged records (device memory)
-    unsigned char* prefill_scratch = nullptr; // chunk prefill: arrival counters, partial results of cut units (device memory)
+    unsigned char* prefill_counters = nullptr;  // chunk prefill: arrival counters and
+    unsigned char* prefill_slots = nullptr;     //   partial results of cut units (null: the cache is too short to cut; device memory)
     // What the latest enqueued operation was, for the decode step's early loads: a decode of one layer
     // may start reading its pages while the previous kernel still runs only if that kernel was a decode
     // of another layer of this cache (which writes neither the metadata nor this layer's pages).
@@ -25,6 +26,9 @@ struct svlm_cache {
     int calls_since_decode = 0;   // library calls on this cache's stream since that decode that left the record alone (projections)
     int last_decode_batch = 0;    // how many caches that launch served, and the first of them
     const svlm_cache* last_decode_first = nullptr;
+    // A chunk-prefill launch of this cache is enqueued behind its latest metadata kernel (it starts when that has
+    // finished): whatever comes behind it may read the metadata without waiting for its own predecessor.
+    bool meta_settled = false;
     SvlmCacheDev* dev_copy = nullptr;   // `dev` in device memory, for the batched kernels
     // staging for the *_host entry points
     void* stage = nullptr;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include "svlm_dev.h"
 #include "svlm_launch.h"
+#include "svlm_ptx.cuh"
 #include "svlm_rope.cuh"
 
 namespace {
@@ -28,33 +29,37 @@ __device__ __forceinline__ void rotate8(Bf16x8& lo, Bf16x8& hi, const float* cs,
     }
 }
 
-// One thread per (token, group of 8 pairs); it serves the kv heads of its share of the layers
-// (grid.y splits the layers when layer < 0), so the rotation factors are looked up once (table, see
-// svlm_rope.cuh).  The source rows do not depend on the metadata, so the loads of the first rows are
-// issued before the chain slot -> position -> factors is walked.
+// One thread per (token, group of 8 pairs) and per share of the [layer][kv_head] rows (blockIdx.y), so the rotation
+// factors are looked up once per share (table, see svlm_rope.cuh).  What bounds it is latency: source rows, and the chain
+// new slot -> position -> factors, which depend on nothing of each other.  early != 0: the caller vouches that no kernel
+// that may still be running writes this cache's metadata; the chain is then walked before the wait for the predecessor
+// (programmatic dependent launch), which leaves one round trip to memory after it.  Per layer of a 524-token chunk
+// between two chunk-prefill launches: 14 us in the stream with 17 blocks, a longer chain and a full launch gap.
 template <int UNROLL>
 __global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int layer, const uint16_t* __restrict__ K,
-                                                       const uint16_t* __restrict__ V, int n, int layers_per_block) {
+                                                       const uint16_t* __restrict__ V, int n, int rows_per_block, int early) {
+    if (!early) svlm_ptx::pdl_wait();
+    svlm_ptx::pdl_launch_dependents();    // (after the wait: a successor's early reads must find all earlier work done)
     const int half = cd.head_dim / 2;
-    const int groups = half / 8;          // threads per token
+    const int gshift = cd.head_dim == 128 ? 3 : 2;      // log2 of the groups (threads) per token
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = t / groups, g = t % groups;
-    if (i >= n) return;
+    const int i = t >> gshift, g = t & ((1 << gshift) - 1);
+    const bool live = i < n;
     const int d = cd.head_dim;
-    const int l0 = layer < 0 ? blockIdx.y * layers_per_block : layer;
-    const int l1 = layer < 0 ? min(cd.layers, l0 + layers_per_block) : layer + 1;
-    const int row0 = l0 * cd.kv_heads, row1 = l1 * cd.kv_heads;      // rows of [layer][kv_head]
+    const int n_rows = layer < 0 ? cd.layers * cd.kv_heads : cd.kv_heads;      // rows of [layer][kv_head] in this call
+    const int row0 = blockIdx.y * rows_per_block, row1 = min(n_rows, row0 + rows_per_block);
+    const int first_row = layer < 0 ? 0 : layer * cd.kv_heads;                 // of the cache
     // source of row r: [layer (only when all layers are given)][token][kv_head]
     auto src_of = [&](int r) {
-        const int l = r / cd.kv_heads, h = r % cd.kv_heads;
-        return (((size_t)(layer < 0 ? l : 0) * n + i) * cd.kv_heads + h) * d + g * 8;
+        const int l = r / cd.kv_heads, h = r - l * cd.kv_heads;
+        return (((size_t)l * n + i) * cd.kv_heads + h) * d + g * 8;
     };
     Bf16x8 lo[UNROLL], hi[UNROLL];
     uint4 vlo[UNROLL], vhi[UNROLL];
     auto load_rows = [&](int r) {
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u)
-            if (r + u < row1) {
+            if (live && r + u < row1) {
                 const size_t src = src_of(r + u);
                 lo[u] = *reinterpret_cast<const Bf16x8*>(K + src);
                 hi[u] = *reinterpret_cast<const Bf16x8*>(K + src + half);
@@ -62,29 +67,51 @@ __global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int laye
                 vhi[u] = *reinterpret_cast<const uint4*>(V + src + half);
             }
     };
-    load_rows(row0);
-    if (cd.ctrl->append_n != n) return;   // the metadata append was dropped (capacity) or does not match
-    const int slot = cd.new_slot[i];
-    // A layer's keys may arrive after an eviction has already shifted these tokens (layers are
-    // computed one after another): rotate at the slot's CURRENT position, and skip a token that
-    // the eviction has dropped in the meantime.
-    if (cd.slot_gid[slot] != cd.ctrl->n_total - n + i) return;
+    if (!early) load_rows(row0);
+    const int append_n = __ldcg(&cd.ctrl->append_n);
+    const long long n_total = __ldcg(&cd.ctrl->n_total);
+    int slot = live ? __ldcg(cd.new_slot + i) : -1;      // (of an append that was dropped: left over, not used)
     float cs[8], sn[8];
+    if (slot >= 0) {
+        // A layer's keys may arrive after an eviction has already shifted these tokens (layers are
+        // computed one after another): rotate at the slot's CURRENT position, and skip a token that
+        // the eviction has dropped in the meantime.
+        const long long gid = __ldcg(cd.slot_gid + slot);
+        int c[3];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int pair = g * 8 + j;
-        const int axis = cd.rope_mode == 0 ? 0 : (pair < cd.sec_t ? 0 : (pair < cd.sec_th ? 1 : 2));
-        const float2 f = svlm_rope_cs(reinterpret_cast<const float2*>(cd.rope_tab), half, pair,
-                                      cd.slot_c[axis * cd.n_slots + slot], cd.theta[pair]);
-        cs[j] = f.x;
-        sn[j] = f.y;
+        for (int k = 0; k < 3; ++k) c[k] = __ldcg(cd.slot_c + (size_t)k * cd.n_slots + slot);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int pair = g * 8 + j;
+            const int axis = cd.rope_mode == 0 ? 0 : (pair < cd.sec_t ? 0 : (pair < cd.sec_th ? 1 : 2));
+            const float2 f = svlm_rope_cs_batched(reinterpret_cast<const float2*>(cd.rope_tab), half, pair, axis == 0 ? c[0] : (axis == 1 ? c[1] : c[2]));
+            cs[j] = f.x;
+            sn[j] = f.y;
+        }
+        const int lim = 1 << 16;
+        if (c[0] <= -lim || c[0] >= lim || c[1] <= -lim || c[1] >= lim || c[2] <= -lim || c[2] >= lim) {   // native positions of a long stream
+#pragma unroll 1
+            for (int j = 0; j < 8; ++j) {
+                const int pair = g * 8 + j;
+                const int axis = cd.rope_mode == 0 ? 0 : (pair < cd.sec_t ? 0 : (pair < cd.sec_th ? 1 : 2));
+                const float2 f = svlm_rope_cs(reinterpret_cast<const float2*>(cd.rope_tab), half, pair, axis == 0 ? c[0] : (axis == 1 ? c[1] : c[2]), cd.theta[pair]);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) if (q == j) { cs[q] = f.x; sn[q] = f.y; }
+            }
+        }
+        if (gid != n_total - n + i) slot = -1;
     }
+    if (early) {
+        svlm_ptx::pdl_wait();
+        load_rows(row0);
+    }
+    if (append_n != n || slot < 0) return;   // the metadata append was dropped (capacity) or does not match
     for (int r = row0; r < row1; r += UNROLL) {
         if (r != row0) load_rows(r);
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u)
             if (r + u < row1) {
-                const size_t dst = ((size_t)(r + u) * cd.n_slots + slot) * d + g * 8;
+                const size_t dst = ((size_t)(first_row + r + u) * cd.n_slots + slot) * d + g * 8;
                 rotate8(lo[u], hi[u], cs, sn);
                 *reinterpret_cast<Bf16x8*>(cd.K + dst) = lo[u];
                 *reinterpret_cast<Bf16x8*>(cd.K + dst + half) = hi[u];
@@ -161,13 +188,28 @@ int rotate_layers_per_block(int layers, int kv_heads) {
 
 }  // namespace
 
-void svlm_launch_kv_write(const SvlmCacheDev& cd, int layer, const void* K, const void* V, int n, cudaStream_t st) {
-    const int groups = cd.head_dim / 16;
-    const int threads = n * groups;
-    const int lpb = rotate_layers_per_block(cd.layers, cd.kv_heads);
-    dim3 grid((threads + 255) / 256, layer < 0 ? (cd.layers + lpb - 1) / lpb : 1);
-    kv_write_kernel<4><<<grid, 256, 0, st>>>(cd, layer, (const uint16_t*)K, (const uint16_t*)V, n, lpb);
+cudaError_t svlm_launch_kv_write(const SvlmCacheDev& cd, int layer, const void* K, const void* V, int n, int early, cudaStream_t st) {
+    const int threads = n * (cd.head_dim / 16);
+    const int x = (threads + 255) / 256;
+    const int rows = layer < 0 ? cd.layers * cd.kv_heads : cd.kv_heads;
+    // one row per thread while that leaves the grid at a few blocks per SM, then up to eight
+    int per = 1;
+    while (per < 8 && (long long)x * ((rows + per - 1) / per) > 8 * svlm_sm_count()) per *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(x, (rows + per - 1) / per);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const uint16_t* k = static_cast<const uint16_t*>(K);
+    const uint16_t* v = static_cast<const uint16_t*>(V);
+    const cudaError_t e = per < 4 ? cudaLaunchKernelEx(&cfg, kv_write_kernel<1>, cd, layer, k, v, n, per, early)
+                                  : cudaLaunchKernelEx(&cfg, kv_write_kernel<4>, cd, layer, k, v, n, per, early);
     svlm_count_launch();
+    return e;
 }
 
 void svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st) {

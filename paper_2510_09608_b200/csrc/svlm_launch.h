@@ -45,7 +45,8 @@ void svlm_launch_evict_meta_batch(const SvlmCacheList& list, cudaStream_t st);
 
 // key/value movement (svlm_kv.cu)
 // layer < 0: K,V are [layers][n][kv_heads][d]; otherwise [n][kv_heads][d] for that layer.
-void svlm_launch_kv_write(const SvlmCacheDev& cd, int layer, const void* K, const void* V, int n, cudaStream_t st);
+// early != 0: the caller vouches that no kernel still running when this one may start writes the cache's metadata.
+cudaError_t svlm_launch_kv_write(const SvlmCacheDev& cd, int layer, const void* K, const void* V, int n, int early, cudaStream_t st);
 void svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st);
 // every cache of the list has the geometry of geom
 void svlm_launch_evict_rotate_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
@@ -86,10 +87,11 @@ cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int i
 
 // tcgen05/TMEM/TMA chunk prefill, n_q >= 2 (svlm_prefill_sm100.cu)
 bool svlm_prefill_supported(int n_pages, int group);
-// scratch: svlm_prefill_scratch_bytes of the first cache, its first svlm_prefill_counter_bytes zero before the first
-// launch (the kernel leaves them zero); launches that share it must not overlap.  pages: how many pages each cache is
-// expected to hold (only the balance of the work depends on it).
-size_t svlm_prefill_scratch_bytes(int n_pages, int head_dim);
+// counters: svlm_prefill_counter_bytes of the first cache, zero before the first launch (the kernel leaves them zero);
+// slots: its svlm_prefill_slot_bytes (0: null).  Launches that share them must not overlap.  pages: how many pages each
+// cache is expected to hold (only the balance of the work depends on it).
+size_t svlm_prefill_slot_bytes(int n_pages, int head_dim);
 constexpr size_t svlm_prefill_counter_bytes = 4096;
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
-                                int n_q, int q_heads, void* out, const int* pages, void* scratch, cudaStream_t st);
+                                int n_q, int q_heads, void* out, const int* pages, void* counters, void* slots,
+                                cudaStream_t st);

@@ -56,7 +56,6 @@ constexpr int PF_MAX_TILES = 512;
 constexpr int PF_ROWS = 256;          // rows per unit
 constexpr int PF_MAX_CTAS = 160;
 constexpr int PF_MIN_PAGES = 6;       // pages a CTA should have at least when units are cut
-constexpr size_t PF_HEAD_BYTES = svlm_prefill_counter_bytes;   // counters in front of the scratch's slots
 constexpr int PF_PIECE = 10;          // what beginning another unit costs, in pages (one stream: 3 and 6: 78 us, 10: 76, 16: 78)
 constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
 constexpr int PF_CS_BYTES = 16384;    // rotation factors of one tile's tokens (5 or more heads per KV head, all at head_dim 64 with 2 or more)
@@ -76,7 +75,7 @@ struct PfPlan {
     unsigned* counters;               // [2 * PF_MAX_CTAS][2] arrivals per (tail unit, tile), zero between launches
     unsigned char* slots;             // [2 * grid] partial results
 };
-static_assert(2 * PF_MAX_CTAS * 2 * sizeof(unsigned) <= PF_HEAD_BYTES, "counters");
+static_assert(2 * PF_MAX_CTAS * 2 * sizeof(unsigned) <= svlm_prefill_counter_bytes, "counters");
 
 template <int D>
 __host__ __device__ constexpr size_t pf_slot_bytes() { return (size_t)PF_ROWS * D * 4 + PF_ROWS * 8; }
@@ -731,6 +730,10 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
+    // Set up while the predecessor ends (programmatic dependent launch); everything read from here on may be its work.
+    // The wait comes before the trigger: a successor that starts early then finds all earlier work done.
+    pdl_wait();
+    pdl_launch_dependents();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1099,7 +1102,7 @@ void make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, in
 
 template <int D>
 cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uint16_t* Q, const int* q_pos, int n_q,
-                   int q_heads, uint16_t* out, const int* pages, void* scratch, cudaStream_t st) {
+                   int q_heads, uint16_t* out, const int* pages, void* counters, void* slots, cudaStream_t st) {
     cudaError_t e = svlm_allow_smem<prefill_kernel<D>>(prefill_smem<D>());
     if (e != cudaSuccess) return e;
     // the register split inside the kernel adds up only if the block is launched with exactly this many
@@ -1109,8 +1112,8 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
     }();
     if (!regs_ok) return cudaErrorLaunchOutOfResources;
     PfPlan plan;
-    plan.counters = static_cast<unsigned*>(scratch);
-    plan.slots = svlm_prefill_scratch_bytes(b.n_slots / SVLM_PAGE, D) > PF_HEAD_BYTES ? static_cast<unsigned char*>(scratch) + PF_HEAD_BYTES : nullptr;
+    plan.counters = static_cast<unsigned*>(counters);
+    plan.slots = static_cast<unsigned char*>(slots);
     const int G = q_heads / b.kv_heads;
     plan.g_magic = G > 1 && (unsigned long long)n_q * G * G < 0x100000000ull - 256ull * G ? (unsigned)((0x100000000ull + G - 1) / G) : 0u;   // (tiles reach past the last row)
     int grid;
@@ -1120,6 +1123,11 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
     cfg.blockDim = dim3(PF_THREADS);
     cfg.dynamicSmemBytes = prefill_smem<D>();
     cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, prefill_kernel<D>, b, plan, layer0, n_layers, Q, q_pos, n_q, q_heads, out);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1128,17 +1136,17 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
 
 bool svlm_prefill_supported(int n_pages, int group) { return n_pages <= PF_MAX_TILES && group >= 1; }
 
-// Arrival counters, and the slots for pieces of units where a cache is long enough for cutting to pay.
-size_t svlm_prefill_scratch_bytes(int n_pages, int head_dim) {
-    if (n_pages < 3 * PF_MIN_PAGES) return PF_HEAD_BYTES;
-    return PF_HEAD_BYTES + (size_t)2 * std::min(svlm_sm_count(), PF_MAX_CTAS) * (head_dim == 128 ? pf_slot_bytes<128>() : pf_slot_bytes<64>());
+// The slots for pieces of units, where a cache is long enough for cutting to pay.
+size_t svlm_prefill_slot_bytes(int n_pages, int head_dim) {
+    if (n_pages < 3 * PF_MIN_PAGES) return 0;
+    return (size_t)2 * std::min(svlm_sm_count(), PF_MAX_CTAS) * (head_dim == 128 ? pf_slot_bytes<128>() : pf_slot_bytes<64>());
 }
 
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
-                                int n_q, int q_heads, void* out, const int* pages, void* scratch, cudaStream_t st) {
+                                int n_q, int q_heads, void* out, const int* pages, void* counters, void* slots, cudaStream_t st) {
     const cudaError_t e = b.head_dim == 128
-        ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, scratch, st)
-        : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, scratch, st);
+        ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, counters, slots, st)
+        : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, counters, slots, st);
     svlm_count_launch();
     return e;
 }

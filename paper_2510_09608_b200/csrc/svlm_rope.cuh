@@ -40,3 +40,12 @@ __device__ __forceinline__ float2 svlm_rope_cs(const float2* __restrict__ tab, i
     if (c < 0) r.y = -r.y;
     return r;
 }
+
+// The same for |c| < 2^16 (anything else: garbage, but no access out of the table), without a branch, so that a caller's
+// look-ups of several pairs are all in flight together.
+__device__ __forceinline__ float2 svlm_rope_cs_batched(const float2* __restrict__ tab, int half, int pair, int c) {
+    const unsigned u = (unsigned)abs(c) & 0xffffu;
+    float2 r = svlm_cmul(__ldg(tab + (size_t)(u & 255u) * half + pair), __ldg(tab + (size_t)(256 + (u >> 8)) * half + pair));
+    if (c < 0) r.y = -r.y;
+    return r;
+}

@@ -41,15 +41,28 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
-template <typename T>
-int dev_alloc(svlm_cache* c, T** p, size_t count, bool zero = true) {
-    void* q = nullptr;
-    if (cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T)) != cudaSuccess) return SVLM_ERR_NOMEM;
-    c->allocs.push_back(q);
-    if (zero && cudaMemset(q, 0, std::max<size_t>(count, 1) * sizeof(T)) != cudaSuccess) return SVLM_ERR_CUDA;
-    *p = static_cast<T*>(q);
-    return SVLM_OK;
-}
+// A cache's device memory is one allocation: its parts are laid out first, those that start at zero in front.  (Some
+// twenty allocations, each with its own clearing and freeing, were most of the time a cache took to create.)
+struct Arena {
+    struct Part { void** at; size_t bytes; bool zero; };
+    std::vector<Part> parts;
+    template <typename T>
+    void add(T** p, size_t count, bool zero = true) {
+        parts.push_back({reinterpret_cast<void**>(p), (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256, zero});
+    }
+    int allocate(svlm_cache* c) {
+        size_t total = 0, zeros = 0;
+        for (const Part& p : parts) { total += p.bytes; zeros += p.zero ? p.bytes : 0; }
+        void* base = nullptr;
+        if (cudaMalloc(&base, total) != cudaSuccess) { cudaGetLastError(); return SVLM_ERR_NOMEM; }
+        c->allocs.push_back(base);
+        char* at = static_cast<char*>(base);
+        for (int pass = 0; pass < 2; ++pass)
+            for (const Part& p : parts)
+                if (p.zero == (pass == 0)) { *p.at = at; at += p.bytes; }
+        return cudaMemset(base, 0, zeros) == cudaSuccess ? SVLM_OK : SVLM_ERR_CUDA;
+    }
+};
 
 void fill_theta(SvlmCacheDev& d, double base) {
     for (int i = 0; i < d.head_dim / 2; ++i) d.theta[i] = std::pow(base, -2.0 * i / d.head_dim);
@@ -92,18 +105,26 @@ void fill_view(const svlm_cache* c, SvlmAttendView& v) {
     v.slot_c = c->dev.slot_c;
 }
 
-// Rotation table: (cos, sin)(k * 256^level * theta_i) in fp32 from fp64 (see svlm_rope.cuh).
+// Rotation table: (cos, sin)(k * 256^level * theta_i) in fp32 from fp64 (see svlm_rope.cuh).  k = 16 a + b: the 16
+// multiples of either kind are evaluated, their 256 sums follow by the angle-addition identity in fp64 (error ~3e-16).
 int upload_rope_table(svlm_cache* c) {
     const SvlmCacheDev& d = c->dev;
     const int half = d.head_dim / 2;
     std::vector<float> tab((size_t)3 * 256 * half * 2);
     for (int level = 0; level < 3; ++level)
-        for (int k = 0; k < 256; ++k)
-            for (int i = 0; i < half; ++i) {
-                const double ang = (double)k * std::pow(256.0, level) * d.theta[i];
-                tab[(((size_t)level * 256 + k) * half + i) * 2] = (float)std::cos(ang);
-                tab[(((size_t)level * 256 + k) * half + i) * 2 + 1] = (float)std::sin(ang);
+        for (int i = 0; i < half; ++i) {
+            const double step = std::pow(256.0, level) * d.theta[i];
+            double hi_c[16], hi_s[16], lo_c[16], lo_s[16];
+            for (int k = 0; k < 16; ++k) {
+                hi_c[k] = std::cos(16.0 * k * step); hi_s[k] = std::sin(16.0 * k * step);
+                lo_c[k] = std::cos(k * step); lo_s[k] = std::sin(k * step);
             }
+            for (int k = 0; k < 256; ++k) {
+                float* f = &tab[(((size_t)level * 256 + k) * half + i) * 2];
+                f[0] = (float)(hi_c[k >> 4] * lo_c[k & 15] - hi_s[k >> 4] * lo_s[k & 15]);
+                f[1] = (float)(hi_s[k >> 4] * lo_c[k & 15] + hi_c[k >> 4] * lo_s[k & 15]);
+            }
+        }
     if (cudaMemcpy(d.rope_tab, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
         return SVLM_ERR_CUDA;
     return SVLM_OK;
@@ -197,11 +218,13 @@ int make_list(svlm_cache* const* caches, int n_caches, SvlmCacheList& list) {
 
 // The host's idea of what a cache stores (it does not know the tokens' types, nor what a replayed graph has appended).
 void note_append(svlm_cache* c, int n) {
+    c->meta_settled = false;
     c->appended += n;
     c->pending_n = n;
     c->stored_est = std::min<long long>(c->stored_est + n, c->dev.capacity);
 }
 void note_evict(svlm_cache* c) {
+    c->meta_settled = false;
     c->stored_est = std::min<long long>(c->stored_est, (long long)c->dev.n_sink + c->dev.vision_window + c->dev.text_window);
 }
 int expected_pages(const svlm_cache* c) { return std::max(1, (int)std::min<long long>(c->stored_est / SVLM_PAGE + 1, c->dev.n_pages)); }
@@ -258,8 +281,8 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     if (Knew) return SVLM_ERR_ARG;   // the fused step exists for the split-KV kernel only
     if (n_q >= 2 && svlm_prefill_supported(c0->dev.n_pages, group)) {
         int pages[SVLM_MAX_BATCH];
-        for (int i = 0; i < n_caches; ++i) pages[i] = expected_pages(caches[i]);
-        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, pages, c0->prefill_scratch, c0->stream));
+        for (int i = 0; i < n_caches; ++i) { pages[i] = expected_pages(caches[i]); caches[i]->meta_settled = true; }
+        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, pages, c0->prefill_counters, c0->prefill_slots, c0->stream));
         return SVLM_OK;
     }
     svlm_launch_attend_simple(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, c0->stream);
@@ -297,41 +320,39 @@ int svlm_cache_create(svlm_cache** out, int layers, int kv_heads, int head_dim, 
 
     int rc = SVLM_OK;
     const size_t slab = (size_t)layers * kv_heads * d.n_slots * head_dim;
-    auto A = [&](int r) { if (rc == SVLM_OK) rc = r; };
-    A(dev_alloc(c, &d.ctrl, 1));
-    A(dev_alloc(c, &d.free_stack, d.n_pages));
-    A(dev_alloc(c, &d.page_table[0], d.pt_size));
-    A(dev_alloc(c, &d.page_table[1], d.pt_size));
-    A(dev_alloc(c, &d.slot_gid, d.n_slots));
-    A(dev_alloc(c, &d.slot_c, 3 * (size_t)d.n_slots));
-    A(dev_alloc(c, &d.slot_a, d.n_slots));
-    A(dev_alloc(c, &d.slot_delta, d.n_slots));
-    A(dev_alloc(c, &d.slot_type, d.n_slots));
-    A(dev_alloc(c, &d.tiles, d.n_pages));
-    A(dev_alloc(c, &d.new_slot, capacity));
-    A(dev_alloc(c, &d.new_c, 3 * (size_t)capacity));
+    Arena mem;
+    mem.add(&d.ctrl, 1);
+    mem.add(&d.free_stack, d.n_pages);
+    mem.add(&d.page_table[0], d.pt_size);
+    mem.add(&d.page_table[1], d.pt_size);
+    mem.add(&d.slot_gid, d.n_slots);
+    mem.add(&d.slot_c, 3 * (size_t)d.n_slots);
+    mem.add(&d.slot_a, d.n_slots);
+    mem.add(&d.slot_delta, d.n_slots);
+    mem.add(&d.slot_type, d.n_slots);
+    mem.add(&d.tiles, d.n_pages);
+    mem.add(&d.new_slot, capacity);
+    mem.add(&d.new_c, 3 * (size_t)capacity);
     for (int t = 0; t < 2; ++t) {
-        A(dev_alloc(c, &d.ev_gid[t], capacity));
-        A(dev_alloc(c, &d.ev_pref[t], (size_t)capacity + 1));
+        mem.add(&d.ev_gid[t], capacity);
+        mem.add(&d.ev_pref[t], (size_t)capacity + 1);
     }
     {   // split-KV scratch: the larger of a one-layer launch and an all-layers launch
         const size_t one = svlm_decode_ws_floats(layers, kv_heads, head_dim, svlm_decode_splits(d.n_pages, kv_heads, 1));
         const size_t all = svlm_decode_ws_floats(layers, kv_heads, head_dim, svlm_decode_splits(d.n_pages, kv_heads, layers));
-        A(dev_alloc(c, &d.ws, std::max(one, all)));
+        mem.add(&d.ws, std::max(one, all));
         // the per-layer kernel's tagged records: zero-filled here, afterwards written by that kernel alone
-        A(dev_alloc(c, &c->decode_tagged, svlm_decode_tagged_bytes(kv_heads, head_dim, svlm_decode_splits(d.n_pages, kv_heads, 1))));
+        mem.add(&c->decode_tagged, svlm_decode_tagged_bytes(kv_heads, head_dim, svlm_decode_splits(d.n_pages, kv_heads, 1)));
     }
-    A(dev_alloc(c, &c->prefill_scratch, svlm_prefill_scratch_bytes(d.n_pages, head_dim), false));
-    if (rc == SVLM_OK && cudaMemset(c->prefill_scratch, 0, svlm_prefill_counter_bytes) != cudaSuccess) rc = SVLM_ERR_CUDA;
-    A(dev_alloc(c, &d.K, slab));
-    A(dev_alloc(c, &d.V, slab));
-    {
-        unsigned char* tm = nullptr;
-        A(dev_alloc(c, &tm, 512));
-        d.tmaps = tm;
-    }
-    A(dev_alloc(c, &d.rope_tab, (size_t)3 * 256 * (head_dim / 2) * 2, false));
-    A(dev_alloc(c, &c->dev_copy, 1));
+    mem.add(&c->prefill_counters, svlm_prefill_counter_bytes);
+    const size_t slot_bytes = svlm_prefill_slot_bytes(d.n_pages, head_dim);
+    if (slot_bytes) mem.add(&c->prefill_slots, slot_bytes, false);
+    mem.add(&d.K, slab);
+    mem.add(&d.V, slab);
+    mem.add(reinterpret_cast<unsigned char**>(&d.tmaps), 512);
+    mem.add(&d.rope_tab, (size_t)3 * 256 * (head_dim / 2) * 2, false);
+    mem.add(&c->dev_copy, 1);
+    rc = mem.allocate(c);
     if (rc == SVLM_OK) rc = make_tensor_maps(c);
     if (rc == SVLM_OK) rc = upload_rope_table(c);
     if (rc == SVLM_OK) rc = sync_dev_copy(c);
@@ -406,6 +427,7 @@ int svlm_cache_set_policy(svlm_cache* c, int sink_any_type, int contiguous) {
 int svlm_cache_set_stream(svlm_cache* c, void* cuda_stream) {
     if (!c) return SVLM_ERR_ARG;
     c->stream = static_cast<cudaStream_t>(cuda_stream);
+    c->meta_settled = false;
     return SVLM_OK;
 }
 
@@ -423,8 +445,8 @@ int svlm_cache_append(svlm_cache* c, int layer, const void* K, const void* V, co
     } else if (n != c->pending_n) {
         return SVLM_ERR_ORDER;
     }
-    svlm_launch_kv_write(c->dev, layer, K, V, n, c->stream);
-    SVLM_CUDA(cudaGetLastError());
+    // a later layer's write behind an attention call of this cache: that call ran after the latest metadata kernel
+    SVLM_CUDA(svlm_launch_kv_write(c->dev, layer, K, V, n, layer > 0 && c->meta_settled, c->stream));
     return SVLM_OK;
 }
 
@@ -582,8 +604,8 @@ int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int laye
     if (off > 0x7fffffffll) return SVLM_ERR_ARG;
     DeviceGuard guard(c0->device);
     int pages[SVLM_MAX_BATCH];
-    for (int i = 0; i < n_caches; ++i) pages[i] = expected_pages(caches[i]);
-    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, Q, q_pos, n_max, q_heads, out, pages, c0->prefill_scratch, c0->stream));
+    for (int i = 0; i < n_caches; ++i) { pages[i] = expected_pages(caches[i]); caches[i]->meta_settled = true; }
+    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, Q, q_pos, n_max, q_heads, out, pages, c0->prefill_counters, c0->prefill_slots, c0->stream));
     return SVLM_OK;
 }
 
