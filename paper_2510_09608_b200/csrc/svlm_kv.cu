@@ -168,6 +168,8 @@ __device__ __forceinline__ void evict_rotate_body(const SvlmCacheDev& cd, int la
 
 template <int UNROLL>
 __global__ void __launch_bounds__(256) evict_rotate_kernel(SvlmCacheDev cd, int layers_per_block) {
+    svlm_ptx::pdl_wait();
+    svlm_ptx::pdl_launch_dependents();
     evict_rotate_body<UNROLL>(cd, layers_per_block);
 }
 
@@ -176,6 +178,8 @@ template <int UNROLL>
 __global__ void __launch_bounds__(256) evict_rotate_batch_kernel(SvlmCacheList list, int layers_per_block) {
     __shared__ SvlmCacheDev s_cd;
     svlm_load_desc(&s_cd, list.cd[blockIdx.z]);
+    svlm_ptx::pdl_wait();
+    svlm_ptx::pdl_launch_dependents();
     evict_rotate_body<UNROLL>(s_cd, layers_per_block);
 }
 
@@ -195,21 +199,11 @@ cudaError_t svlm_launch_kv_write(const SvlmCacheDev& cd, int layer, const void* 
     // one row per thread while that leaves the grid at a few blocks per SM, then up to eight
     int per = 1;
     while (per < 8 && (long long)x * ((rows + per - 1) / per) > 8 * svlm_sm_count()) per *= 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(x, (rows + per - 1) / per);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const dim3 grid(x, (rows + per - 1) / per);
     const uint16_t* k = static_cast<const uint16_t*>(K);
     const uint16_t* v = static_cast<const uint16_t*>(V);
-    const cudaError_t e = per < 4 ? cudaLaunchKernelEx(&cfg, kv_write_kernel<1>, cd, layer, k, v, n, per, early)
-                                  : cudaLaunchKernelEx(&cfg, kv_write_kernel<4>, cd, layer, k, v, n, per, early);
-    svlm_count_launch();
-    return e;
+    return per < 4 ? svlm_launch_chained(kv_write_kernel<1>, grid, dim3(256), 0, 1, st, cd, layer, k, v, n, per, early)
+                   : svlm_launch_chained(kv_write_kernel<4>, grid, dim3(256), 0, 1, st, cd, layer, k, v, n, per, early);
 }
 
 void svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st) {
@@ -217,14 +211,12 @@ void svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st) {
     const int threads = cd.n_slots * groups;
     const int lpb = rotate_layers_per_block(cd.layers, cd.kv_heads);
     dim3 grid((threads + 255) / 256, (cd.layers + lpb - 1) / lpb);
-    evict_rotate_kernel<4><<<grid, 256, 0, st>>>(cd, lpb);
-    svlm_count_launch();
+    svlm_launch_chained(evict_rotate_kernel<4>, grid, dim3(256), 0, 1, st, cd, lpb);
 }
 
 void svlm_launch_evict_rotate_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st) {
     const int threads = geom.n_slots * (geom.head_dim / 16);
     const int lpb = rotate_layers_per_block(geom.layers, geom.kv_heads);
     dim3 grid((threads + 255) / 256, (geom.layers + lpb - 1) / lpb, list.n);
-    evict_rotate_batch_kernel<4><<<grid, 256, 0, st>>>(list, lpb);
-    svlm_count_launch();
+    svlm_launch_chained(evict_rotate_batch_kernel<4>, grid, dim3(256), 0, 1, st, list, lpb);
 }

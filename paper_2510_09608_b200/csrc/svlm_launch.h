@@ -22,6 +22,28 @@ cudaError_t svlm_allow_smem(size_t bytes) {
     return e;
 }
 
+// Launches a kernel that may become resident while its predecessor in the stream ends (programmatic dependent launch: the
+// kernel itself waits, griddepcontrol), as clusters of `cluster` CTAs, and counts it.
+template <typename... P, typename... A>
+cudaError_t svlm_launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    svlm_count_launch();
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Streaming multiprocessors of the current device (looked up once per device).
 inline int svlm_sm_count() {
     static std::atomic<int> known[64];

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include "svlm_dev.h"
 #include "svlm_launch.h"
+#include "svlm_ptx.cuh"
 
 namespace {
 
@@ -571,65 +572,59 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
     }
 }
 
+// All of these kernels are launched programmatically (svlm_launch_chained): they start while their predecessor ends, wait
+// for it first and only then let their own successor start, so that whoever starts early behind them finds everything
+// enqueued before them done.  Batched forms: block i serves cache i, whose descriptor it first copies from device memory
+// into shared memory.  types is [n_caches][n], pos [n_caches][n] (1D) or [n_caches][n][3].
 __global__ void __launch_bounds__(META_THREADS) append_meta_kernel(SvlmCacheDev cd, const unsigned char* types,
                                                                    const int* pos, int n) {
+    svlm_ptx::pdl_wait();
+    // One token: a decode step follows, one CTA per SM with a second slot free on each for the next layer's.  Started
+    // beside this kernel it finds one SM half taken, puts two CTAs on another, and every later layer-step of the chain
+    // inherits the unevenness (6.57 -> 7.27 us each); so there the successor starts when this CTA is gone.
+    if (n > 1) svlm_ptx::pdl_launch_dependents();
     append_meta_body(cd, types, pos, n);
 }
 
-__global__ void __launch_bounds__(META_THREADS) evict_meta_kernel(SvlmCacheDev cd) { evict_meta_body(cd); }
+__global__ void __launch_bounds__(META_THREADS) evict_meta_kernel(SvlmCacheDev cd) {
+    svlm_ptx::pdl_wait();
+    svlm_ptx::pdl_launch_dependents();
+    evict_meta_body(cd);
+}
 
-// Batched forms: block i serves cache i, whose descriptor it first copies from device memory into
-// shared memory.  types is [n_caches][n], pos [n_caches][n] (1D) or [n_caches][n][3].
 __global__ void __launch_bounds__(META_THREADS) append_meta_batch_kernel(SvlmCacheList list, const unsigned char* types,
                                                                          const int* pos, int n) {
     __shared__ SvlmCacheDev s_cd;
-    svlm_load_desc(&s_cd, list.cd[blockIdx.x]);
+    svlm_load_desc(&s_cd, list.cd[blockIdx.x]);      // (frozen by the first append: no kernel writes it)
+    svlm_ptx::pdl_wait();
+    if (n > 1) svlm_ptx::pdl_launch_dependents();
     append_meta_body(s_cd, types + (size_t)blockIdx.x * n, pos + (size_t)blockIdx.x * n * (s_cd.rope_mode == 0 ? 1 : 3), n);
 }
 
 __global__ void __launch_bounds__(META_THREADS) evict_meta_batch_kernel(SvlmCacheList list) {
     __shared__ SvlmCacheDev s_cd;
     svlm_load_desc(&s_cd, list.cd[blockIdx.x / EV_CLUSTER]);
+    svlm_ptx::pdl_wait();
+    svlm_ptx::pdl_launch_dependents();
     evict_meta_body(s_cd);
-}
-
-// Launch `clusters` clusters of EV_CLUSTER CTAs.
-template <typename... Args>
-void launch_evict_meta(void (*kernel)(Args...), int clusters, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(EV_CLUSTER * clusters);
-    cfg.blockDim = dim3(META_THREADS);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = EV_CLUSTER;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 }  // namespace
 
 void svlm_launch_append_meta_batch(const SvlmCacheList& list, const unsigned char* types, const int* pos, int n,
                                    cudaStream_t st) {
-    append_meta_batch_kernel<<<list.n, META_THREADS, 0, st>>>(list, types, pos, n);
-    svlm_count_launch();
+    svlm_launch_chained(append_meta_batch_kernel, dim3(list.n), dim3(META_THREADS), 0, 1, st, list, types, pos, n);
 }
 
 void svlm_launch_evict_meta_batch(const SvlmCacheList& list, cudaStream_t st) {
-    launch_evict_meta(evict_meta_batch_kernel, list.n, st, list);
-    svlm_count_launch();
+    svlm_launch_chained(evict_meta_batch_kernel, dim3(EV_CLUSTER * list.n), dim3(META_THREADS), 0, EV_CLUSTER, st, list);
 }
 
 void svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n,
                              cudaStream_t st) {
-    append_meta_kernel<<<1, META_THREADS, 0, st>>>(cd, types, pos, n);
-    svlm_count_launch();
+    svlm_launch_chained(append_meta_kernel, dim3(1), dim3(META_THREADS), 0, 1, st, cd, types, pos, n);
 }
 
 void svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st) {
-    launch_evict_meta(evict_meta_kernel, 1, st, cd);
-    svlm_count_launch();
+    svlm_launch_chained(evict_meta_kernel, dim3(EV_CLUSTER), dim3(META_THREADS), 0, EV_CLUSTER, st, cd);
 }

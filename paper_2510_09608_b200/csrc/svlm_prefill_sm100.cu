@@ -1118,18 +1118,8 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
     plan.g_magic = G > 1 && (unsigned long long)n_q * G * G < 0x100000000ull - 256ull * G ? (unsigned)((0x100000000ull + G - 1) / G) : 0u;   // (tiles reach past the last row)
     int grid;
     make_plan(plan, b, n_layers, n_q, G, pages, std::min(svlm_sm_count(), PF_MAX_CTAS), grid);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(PF_THREADS);
-    cfg.dynamicSmemBytes = prefill_smem<D>();
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, prefill_kernel<D>, b, plan, layer0, n_layers, Q, q_pos, n_q, q_heads, out);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return svlm_launch_chained(prefill_kernel<D>, dim3((unsigned)grid), dim3(PF_THREADS), prefill_smem<D>(), 1, st, b, plan, layer0, n_layers, Q, q_pos,
+                               n_q, q_heads, out);
 }
 
 }  // namespace
@@ -1144,9 +1134,7 @@ size_t svlm_prefill_slot_bytes(int n_pages, int head_dim) {
 
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
                                 int n_q, int q_heads, void* out, const int* pages, void* counters, void* slots, cudaStream_t st) {
-    const cudaError_t e = b.head_dim == 128
+    return b.head_dim == 128
         ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, counters, slots, st)
         : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, counters, slots, st);
-    svlm_count_launch();
-    return e;
 }
