@@ -30,6 +30,9 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
+
 #include "svlm_dev.h"
 #include "svlm_launch.h"
 #include "svlm_ptx.cuh"
@@ -167,7 +170,7 @@ __device__ __forceinline__ void ld_tagged2(const void* p, unsigned long long& a,
 // TAGGED: the record goes out in the per-layer kernel's tagged format (ll_rec_bytes).
 template <int D, bool TAGGED, typename Stamp>
 __device__ __forceinline__ void cta_merge_and_record(const float (&o)[D / 16][4], const float (&m)[2], const float (&l)[2],
-                                                     float* buf, unsigned char* part, unsigned tag, Stamp stamp) {
+                                                     float* buf, unsigned char* part, Stamp stamp, const int* tag_at = nullptr) {
     constexpr int MROW = D + MERGE_PAD, DBLK = D / 16;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     float* s_o = buf;                                     // [warp][8 heads][MROW]
@@ -210,6 +213,7 @@ __device__ __forceinline__ void cta_merge_and_record(const float (&o)[D / 16][4]
         pk.x = pack_bf16(acc[0], acc[1]); pk.y = pack_bf16(acc[2], acc[3]);
         pk.z = pack_bf16(acc[4], acc[5]); pk.w = pack_bf16(acc[6], acc[7]);
         if constexpr (TAGGED) {
+            const unsigned tag = (unsigned)*tag_at;
             st_tagged2(part + (size_t)(h * D + d0) * 4, pk.x, pk.y, tag);
             st_tagged2(part + (size_t)(h * D + d0) * 4 + 16, pk.z, pk.w, tag);
         } else {
@@ -224,7 +228,7 @@ __device__ __forceinline__ void cta_merge_and_record(const float (&o)[D / 16][4]
 #pragma unroll
             for (int w = 0; w < DEC_CWARPS; ++w) L += s_l[w * 8 + h] * exp2f(s_m[w * 8 + h] - M);
         if constexpr (TAGGED) {
-            st_tagged2(part + 8 * D * 4 + h * 16, __float_as_uint(M), __float_as_uint(L), tag);
+            st_tagged2(part + 8 * D * 4 + h * 16, __float_as_uint(M), __float_as_uint(L), (unsigned)*tag_at);
         } else {
             float* ml = reinterpret_cast<float*>(part + 8 * D * 2);
             ml[h] = M;
@@ -351,17 +355,17 @@ __device__ __forceinline__ void arrive_and_combine(int* s_last, unsigned* counte
 // wait is for stragglers only.
 //
 // The loads are coalesced: eight lanes of a warp cover the (up to) eight groups of the CTA's share, which lie side
-// by side in a record, the four lane groups of the 7 warps take 28 records at a time, two rounds in flight (one
+// by side in a record, the four lane groups of the six warps take 24 records at a time, two rounds in flight (one
 // record per lane with the lanes a record apart was 2 us slower: 32 cache lines per load instruction).  The four
-// record lanes meet through shuffles, the warps through `buf` (7 x 8 x 12 floats), and four threads per group
+// record lanes meet through shuffles, the warps through `buf` (6 x 8 x 12 floats), and four threads per group
 // write the result.  Split 0, which by then has seen every split's record and therefore knows that every CTA of
 // the KV head has read the epoch, moves the epoch on for the next launch.  Called by all DEC_THREADS threads of the
 // first `shares` splits after a __syncthreads() that follows their last use of `buf`.
 // stamp: trace hook (stations 12, 15).
-constexpr int DEC_WARPS = DEC_THREADS / 32;
+constexpr int LAY_THREADS = DEC_CWARPS * 32;         // the per-layer kernel: consumer warps only (168 registers with two CTAs per SM)
 
 __host__ __device__ inline int combine_shares(int groups, int splits) {
-    const int want = (groups + DEC_WARPS - 1) / DEC_WARPS;
+    const int want = (groups + 6) / 7;                       // at most eight groups a share, seven measured best
     return want < splits ? want : splits;
 }
 
@@ -386,18 +390,18 @@ __device__ __forceinline__ void combine_tagged(int share, int shares, int splits
         float M = -INFINITY, L = 0.f;
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-        for (int r0 = warp * 4 + rl; r0 < splits; r0 += 2 * DEC_WARPS * 4) {
+        for (int r0 = warp * 4 + rl; r0 < splits; r0 += 2 * DEC_CWARPS * 4) {
             unsigned long long w[2][6];                      // per record: o words 0..3, (m, tag), (l, tag)
             bool want[2];
 #pragma unroll
-            for (int k = 0; k < 2; ++k) want[k] = valid && r0 + k * DEC_WARPS * 4 < splits;
+            for (int k = 0; k < 2; ++k) want[k] = valid && r0 + k * DEC_CWARPS * 4 < splits;
             for (unsigned polls = 0;; ++polls) {
                 if (__builtin_expect(polls >= wait_limit, 0)) { timed_out = true; break; }
                 bool ok = true;
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     if (!want[k]) continue;
-                    const size_t off = (size_t)(r0 + k * DEC_WARPS * 4) * REC;
+                    const size_t off = (size_t)(r0 + k * DEC_CWARPS * 4) * REC;
                     ld_tagged2(ov + off, w[k][0], w[k][1]);
                     ld_tagged2(ov + off + 16, w[k][2], w[k][3]);
                     ld_tagged2(ml + off, w[k][4], w[k][5]);
@@ -462,11 +466,11 @@ __device__ __forceinline__ void combine_tagged(int share, int shares, int splits
             const float* sl = buf + (size_t)fg * 12;
             float Ma = -INFINITY;
 #pragma unroll
-            for (int wp = 0; wp < DEC_WARPS; ++wp) Ma = fmaxf(Ma, sl[wp * 96]);
+            for (int wp = 0; wp < DEC_CWARPS; ++wp) Ma = fmaxf(Ma, sl[wp * 96]);
             float La = 0.f, a0 = 0.f, a1 = 0.f;
             if (Ma > -INFINITY)
 #pragma unroll
-                for (int wp = 0; wp < DEC_WARPS; ++wp) {
+                for (int wp = 0; wp < DEC_CWARPS; ++wp) {
                     const float wt = exp2f(sl[wp * 96] - Ma);
                     const float2 a = *reinterpret_cast<const float2*>(sl + wp * 96 + 2 + 2 * e2);
                     La += sl[wp * 96 + 1] * wt;
@@ -800,7 +804,7 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
             l[1] += __shfl_xor_sync(0xffffffffu, l[1], sft);
         }
         // the ring is free once all consumer warps are here (the merge waits for that)
-        cta_merge_and_record<D, false>(o, m, l, reinterpret_cast<float*>(ring), part, 0u, [](int) {});
+        cta_merge_and_record<D, false>(o, m, l, reinterpret_cast<float*>(ring), part, [](int) {});
     }
 
     // ---- last CTA of this (cache, layer, kv head) combines the splits -----------------------------
@@ -833,6 +837,8 @@ struct LayShared {
     int tag;                           // this launch's tag of the records' words
     int wait_limit;                    // times a combining thread may read a word again
     int pad[2];
+    uint16_t q[8 * (128 + QROW_PAD)];  // rotated query rows
+    uint16_t fresh[2 * 128];           // fused step: the new token's rotated key [D], then its value [D]
     unsigned tile_pk[DEC_MAX_TILES];   // page | lo << 16 | hi << 24
 };
 
@@ -843,30 +849,26 @@ __device__ __forceinline__ int lay_off(int key, int chunk) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(DEC_THREADS, 2)
+__global__ void __launch_bounds__(LAY_THREADS, 2)
 decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q, const int* __restrict__ q_pos, int q_heads,
                     uint16_t* __restrict__ out, int splits, const uint16_t* __restrict__ Knew,
                     const uint16_t* __restrict__ Vnew, int early_loads, unsigned char* __restrict__ records TRACE_PARAM) {
     if (threadIdx.x == 0) STAMP(0);                  // kernel entry
     constexpr int CH = D / 8;                        // 16-byte chunks per row
     constexpr int ITEM_BYTES = UNIT * D * 2;         // K or V of one unit
-    constexpr int KSTEPS = D / 16;
+    constexpr int KSTEPS = D / 16, HKS = KSTEPS / 2; // k-steps of 16 dims; of half the head
     constexpr int DBLK = D / 16;
     constexpr int HALF = D / 2;
-    constexpr int RING_BYTES = DEC_CWARPS * LAY_SLOTS * ITEM_BYTES;
     extern __shared__ unsigned char smem_raw[];
     LayShared& sh = *reinterpret_cast<LayShared*>(smem_raw);
     unsigned char* ring = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + sizeof(LayShared) + 127) & ~(uintptr_t)127);
-    uint16_t* s_q = reinterpret_cast<uint16_t*>(ring + RING_BYTES);   // [8][D] bf16
-    uint16_t* s_new = s_q + 8 * (D + QROW_PAD);       // fused step: the new token's rotated key [D], then its value [D]
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int split = blockIdx.x, hk = blockIdx.y;
     const SvlmAttendView& vw = b.view[0];
     const int G = q_heads / b.kv_heads;
-    const bool consumer = warp < DEC_CWARPS;
 
     // The metadata was written by an earlier kernel in the stream.  When the launcher vouches that
     // the kernel directly before this one did not write it (early_loads), it is read at once;
@@ -876,11 +878,11 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     if (!early_loads) pdl_wait();
     pdl_launch_dependents();
     const int n_tiles = min(__ldcg(&vw.ctrl->n_tiles), DEC_MAX_TILES);
-    for (int i = threadIdx.x; i < n_tiles; i += DEC_THREADS) {
+    for (int i = threadIdx.x; i < n_tiles; i += LAY_THREADS) {
         const int4 tl = __ldcg(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
         sh.tile_pk[i] = (unsigned)tl.x | ((unsigned)tl.y << 16) | ((unsigned)tl.z << 24);
     }
-    if (early_loads && warp == DEC_CWARPS && lane < 3) {
+    if (early_loads && warp == DEC_CWARPS - 1 && lane < 3) {
         // Bring the call's own small inputs towards L2 while the previous kernel still runs (a hint:
         // they are read for real only after the grid-dependency wait).
         const size_t qoff = (size_t)hk * G * D, koff = (size_t)hk * D;
@@ -894,7 +896,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     const long long shift = __ldcg(&vw.ctrl->shift_total);
     // the new token of a fused step: where it lives and whether it is still stored there
     int new_slot = -1;
-    if (Knew && consumer) {
+    if (Knew) {
         const int s = __ldcg(vw.new_slot);
         if (__ldcg(&vw.ctrl->append_n) == 1 && __ldcg(vw.slot_gid + s) == __ldcg(&vw.ctrl->n_total) - 1) new_slot = s;
     }
@@ -912,212 +914,242 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     unsigned char* ws_parts = records + ll_head_bytes(b.kv_heads) + (size_t)hk * splits * REC;   // this KV head's records
     unsigned char* part = ws_parts + (size_t)split * REC;                                       // 16-byte aligned
 
-    if (consumer) {
-        const uint16_t* Kh = vw.K + head_row0 * D;
-        const uint16_t* Vh = vw.V + head_row0 * D;
-        unsigned char* my = ring + warp * (LAY_SLOTS * ITEM_BYTES);   // this warp's four slots
-        // This warp's units of round r are e = warp, warp + 6, warp + 12 of the round.  For unit j: the first
-        // slot of the cache it covers (-1: no such unit, or no valid slot in it), the page's valid offsets.
-        struct Units { int row[UPW], k0[UPW], lo[UPW], hi[UPW]; };
-        auto get_units = [&](int r, Units& u) {
+    const uint16_t* Kh = vw.K + head_row0 * D;
+    const uint16_t* Vh = vw.V + head_row0 * D;
+    unsigned char* my = ring + warp * (LAY_SLOTS * ITEM_BYTES);   // this warp's four slots
+    // This warp's units of round r: those of e = warp, warp + 6, warp + 12 that hold valid keys, the present ones first.
+    // For unit j: the first slot of the cache it covers, its first and past-the-last valid key.
+    struct Units { int n, row[UPW], lohi[UPW]; };    // n: how many; lohi: 8 bits each
+    auto get_units = [&](int r, Units& u) {
+        u.n = 0;
 #pragma unroll
-            for (int j = 0; j < UPW; ++j) {
-                const int e = r * GROUP + warp + DEC_CWARPS * j;
-                u.row[j] = -1; u.k0[j] = u.lo[j] = u.hi[j] = 0;
-                if (e >= n_units) continue;
-                const unsigned pk = sh.tile_pk[(u0 + e) >> 3];
-                const int page = pk & 0xFFFF;
-                u.lo[j] = (pk >> 16) & 0xFF; u.hi[j] = pk >> 24;
-                u.k0[j] = ((u0 + e) & 7) * UNIT;
-                if (u.k0[j] < u.hi[j] && u.k0[j] + UNIT > u.lo[j]) u.row[j] = page * SVLM_PAGE + u.k0[j];
-            }
-        };
-        // all 32 lanes copy one unit (16 rows of D elements, contiguous in the cache) into a slot
-        auto load_unit = [&](const uint16_t* base, int row, unsigned char* dst) {
-            const uint16_t* src = base + (size_t)row * D;
+        for (int j = 0; j < UPW; ++j) { u.row[j] = 0; u.lohi[j] = 0; }
 #pragma unroll
-            for (int i = lane; i < UNIT * CH; i += 32) cp_async16(dst + lay_off(i / CH, i % CH), src + (size_t)i * 8);
-        };
-        // front of a round: the key units (copy group 1) and the first value unit (copy group 2)
-        auto issue_front = [&](const Units& u) {
+        for (int j = 0; j < UPW; ++j) {
+            const int e = r * GROUP + warp + DEC_CWARPS * j;
+            if (e >= n_units) continue;
+            const unsigned pk = sh.tile_pk[(u0 + e) >> 3];
+            const int k0 = ((u0 + e) & 7) * UNIT;
+            const int lo = max((int)((pk >> 16) & 0xFF) - k0, 0), hi = min((int)(pk >> 24) - k0, UNIT);
+            if (lo >= hi) continue;
 #pragma unroll
-            for (int j = 0; j < UPW; ++j)
-                if (u.row[j] >= 0) load_unit(Kh, u.row[j], my + j * ITEM_BYTES);
-            cp_async_commit();
-            if (u.row[0] >= 0) load_unit(Vh, u.row[0], my + UPW * ITEM_BYTES);
-            cp_async_commit();
-        };
-        Units u;
-        // the value units that have to wait for a key slot go towards L2 meanwhile
-        auto value_to_l2 = [&](int row) {
-            for (int o = lane * 128; o < ITEM_BYTES; o += 32 * 128)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(Vh + (size_t)row * D) + o));
-        };
-        if (n_rounds > 0) {
-            get_units(0, u);
-            if (early_loads == 2) {
-                // Reading ahead of a previous decode step there is time, and that kernel's short dependent loads
-                // (query, partial results) queue behind whatever the whole grid has in flight: the warp asks
-                // for one unit's worth at a time (keys of unit j with the values of unit j, copied or
-                // prefetched) and lets it land before the next, a third of the burst's depth.
-#pragma unroll
-                for (int j = 0; j < UPW; ++j) {
-                    if (u.row[j] >= 0) {
-                        load_unit(Kh, u.row[j], my + j * ITEM_BYTES);
-                        if (j == 0) load_unit(Vh, u.row[0], my + UPW * ITEM_BYTES);
-                        else value_to_l2(u.row[j]);
-                    }
-                    cp_async_commit();
-                    if (j + 1 < UPW) cp_async_wait<0>();
-                }
-                cp_async_commit();   // (empty: the round's "all but the latest group" then covers the last keys)
-            } else {
-                issue_front(u);
-#pragma unroll
-                for (int j = 1; j < UPW; ++j)
-                    if (u.row[j] >= 0) value_to_l2(u.row[j]);
-            }
+            for (int q = 0; q < UPW; ++q)
+                if (q == u.n) { u.row[q] = (int)(pk & 0xFFFF) * SVLM_PAGE + k0; u.lohi[q] = lo | (hi << 8); }
+            ++u.n;
         }
-        if (threadIdx.x == 0) STAMP(2);              // the first round's copies are issued
+    };
+    // all 32 lanes copy one unit (16 rows of D elements, contiguous in the cache) into a slot
+    auto load_unit = [&](const uint16_t* base, int row, unsigned char* dst) {
+        const uint16_t* src = base + (size_t)row * D;
+#pragma unroll
+        for (int i = lane; i < UNIT * CH; i += 32) cp_async16(dst + lay_off(i / CH, i % CH), src + (size_t)i * 8);
+    };
+    // the value units that have to wait for a key slot go towards L2 meanwhile
+    auto value_to_l2 = [&](int row) {
+        for (int o = lane * 128; o < ITEM_BYTES; o += 32 * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(Vh + (size_t)row * D) + o));
+    };
+    // where the value units go: unit 0 has its own slot, units 1 and 2 take over the slots of key units 0 and 1
+    unsigned char* const sv[UPW] = {my + UPW * ITEM_BYTES, my, my + ITEM_BYTES};
+    const int lm_i = lane >> 3, lm_r = lane & 7;     // ldmatrix: which 8x8 matrix this lane addresses, and its row
+    constexpr int RPW = 2;                           // units whose fragments wait in registers (a third would spill)
+    unsigned kf[RPW][KSTEPS][4];                     // the round's first key fragments, later value fragments
+    auto key_fragment = [&](int j, int ks, unsigned (&a)[4]) {
+        ldmatrix_x4(a[0], a[1], a[2], a[3], my + j * ITEM_BYTES + lay_off((lm_i & 1) * 8 + lm_r, ks * 2 + (lm_i >> 1)));
+    };
+    auto value_fragment = [&](int j, int db, unsigned (&a)[4]) {
+        ldmatrix_x4_trans(a[0], a[1], a[2], a[3], sv[j] + lay_off((lm_i >> 1) * 8 + lm_r, db * 2 + (lm_i & 1)));
+    };
+    Units u;
+    // Front of a round: the three key units and the first value unit are copied, the keys go on into fragment
+    // registers, the other two value units follow into the key slots.  PACED: reading ahead of a previous decode step
+    // there is time, and that kernel's short dependent loads (query, partial results) queue behind whatever the whole
+    // grid has in flight: the warp asks for one unit's worth at a time (keys of unit j with the values of unit j, copied
+    // or prefetched) and lets it land before the next, a third of the burst's depth.
+    auto front = [&](bool paced) {
+#pragma unroll
+        for (int j = 0; j < UPW; ++j) {
+            if (j < u.n) {
+                load_unit(Kh, u.row[j], my + j * ITEM_BYTES);
+                if (j == 0) load_unit(Vh, u.row[0], sv[0]);
+                else value_to_l2(u.row[j]);
+            }
+            cp_async_commit();
+            if (paced) cp_async_wait<0>();
+        }
+        cp_async_wait<0>();
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < RPW; ++j) {
+            if (j >= u.n) continue;                  // warp-uniform
+#pragma unroll
+            for (int ks = 0; ks < KSTEPS; ++ks) key_fragment(j, ks, kf[j][ks]);
+        }
+        __syncwarp();                                // every lane has these fragments: the slots of key units 0 and 1 are free
+#pragma unroll
+        for (int j = 1; j < UPW; ++j)
+            if (j < u.n) load_unit(Vh, u.row[j], sv[j]);
+        cp_async_commit();
+    };
+    if (n_rounds > 0) {
+        get_units(0, u);
+        front(early_loads == 2);
+    }
+    if (threadIdx.x == 0) STAMP(2);                  // the first round's keys are in registers
 
-        const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
-        // ---- query rows: rotate at q_pos - shift_total, round to bf16, park in shared memory ----
-        {
-            const int pair = threadIdx.x & (HALF - 1);
+    // ---- query rows: rotate at q_pos - shift_total, round to bf16, park in shared memory -----------------------
+    // A thread takes two neighbouring pairs (i, i + D/2) of a head.  In a fused step the query is the appended token, its
+    // position is already in the metadata, so the factors do not have to wait for the previous kernel; otherwise the
+    // position comes with the call.  (Every warp loading the query straight into its fragments: 0.2 us later.)
+    unsigned qf[KSTEPS][2];
+    const int new_row16 = new_slot & ~15;            // first slot of the unit that holds the new token (fused step)
+    {
+        constexpr int LPH = HALF / 2;                // threads per head
+        constexpr int HSTEP = LAY_THREADS / LPH, HN = (8 + HSTEP - 1) / HSTEP;   // heads in one pass; passes
+        const int p2 = threadIdx.x % LPH;
+        if (new_slot < 0 && early_loads) pdl_wait();
+        float2 f[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int pair = 2 * p2 + e;
             const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
-            // fused step: the query is the appended token, its position is already in the metadata, so the
-            // rotation factors do not have to wait for the previous kernel; otherwise the position comes with the call
-            long long cpos = 0;
-            if (new_slot >= 0) {
-                cpos = __ldcg(vw.slot_c + (size_t)axis * b.n_slots + new_slot);
-            } else {
-                if (early_loads) pdl_wait();
-                cpos = (long long)q_pos[b.rope_mode == 0 ? 0 : axis] - shift;
-            }
-            const float2 cs = svlm_rope_cs(tab, HALF, pair, cpos, b.theta[pair]);
-            if (new_slot >= 0 && early_loads) pdl_wait();
-            if (threadIdx.x == 0) STAMP(3);          // the previous kernel has completed
-            unsigned ep = 0;                         // the KV head's epoch (same round trip as the query)
-            if (threadIdx.x == 0) ep = __ldcg(epoch);
-            constexpr int HSTEP = (DEC_CWARPS * 32) / HALF, HN = (8 + HSTEP - 1) / HSTEP;   // heads per thread
-            uint16_t qx[HN], qy[HN];
-            // fused step: the new token's key and value rows come in with the query (same round trip); the key is
-            // rotated with the query's factors (same token, same position) and both wait in shared memory for the
-            // warp whose unit holds the token's slot
-            const bool prep_new = new_slot >= 0 && threadIdx.x < HALF;
-            uint16_t kx = 0, ky = 0, vx = 0, vy = 0;
-            if (prep_new) {
-                const size_t noff = (size_t)hk * D;
-                kx = Knew[noff + pair]; ky = Knew[noff + pair + HALF];
-                vx = Vnew[noff + pair]; vy = Vnew[noff + pair + HALF];
-            }
-#pragma unroll
-            for (int k = 0; k < HN; ++k) {      // all loads first: one round trip
-                const int h = threadIdx.x / HALF + k * HSTEP;
-                const size_t off = (size_t)(hk * G + (h < G ? h : 0)) * D;   // n_q = 1
-                qx[k] = Q[off + pair];
-                qy[k] = Q[off + pair + HALF];
-            }
-#pragma unroll
-            for (int k = 0; k < HN; ++k) {
-                const int h = threadIdx.x / HALF + k * HSTEP;
-                if (h >= 8) continue;
-                const float x = h < G ? __bfloat162float(__ushort_as_bfloat16(qx[k])) : 0.f;
-                const float y = h < G ? __bfloat162float(__ushort_as_bfloat16(qy[k])) : 0.f;
-                s_q[h * (D + QROW_PAD) + pair] = __bfloat16_as_ushort(__float2bfloat16_rn(x * cs.x - y * cs.y));
-                s_q[h * (D + QROW_PAD) + pair + HALF] = __bfloat16_as_ushort(__float2bfloat16_rn(y * cs.x + x * cs.y));
-            }
-            if (prep_new) {
-                const float x = __bfloat162float(__ushort_as_bfloat16(kx)), y = __bfloat162float(__ushort_as_bfloat16(ky));
-                s_new[pair] = __bfloat16_as_ushort(__float2bfloat16_rn(x * cs.x - y * cs.y));
-                s_new[pair + HALF] = __bfloat16_as_ushort(__float2bfloat16_rn(y * cs.x + x * cs.y));
-                s_new[D + pair] = vx;
-                s_new[D + pair + HALF] = vy;
-            }
-            if (threadIdx.x == 0) sh.tag = (int)(ep + 1);
+            const long long c = new_slot >= 0 ? (long long)__ldcg(vw.slot_c + (size_t)axis * b.n_slots + new_slot)
+                                              : (long long)q_pos[b.rope_mode == 0 ? 0 : axis] - shift;
+            const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
+            f[e] = svlm_rope_cs_batched(tab, HALF, pair, (int)c);
+            if (__builtin_expect(c <= -65536 || c >= 65536, 0)) f[e] = svlm_rope_cs(tab, HALF, pair, c, b.theta[pair]);
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(DEC_CWARPS * 32));   // consumer warps only
-        if (threadIdx.x == 0) STAMP(4);              // rotated query in shared memory
-        unsigned qf[KSTEPS][2];   // B fragments of Q^T: (d = ks*16 + 2t.., head g)
+        if (new_slot >= 0 && early_loads) pdl_wait();
+        if (threadIdx.x == 0) STAMP(3);              // the previous kernel has completed
+        unsigned ep = 0;                             // the KV head's epoch (same round trip as the query)
+        if (threadIdx.x == 0) ep = __ldcg(epoch);
+        auto rotate2 = [&](unsigned& lo, unsigned& hi) {
+            const float x0 = __uint_as_float(lo << 16), x1 = __uint_as_float(lo & 0xffff0000u);
+            const float y0 = __uint_as_float(hi << 16), y1 = __uint_as_float(hi & 0xffff0000u);
+            lo = pack_bf16(x0 * f[0].x - y0 * f[0].y, x1 * f[1].x - y1 * f[1].y);
+            hi = pack_bf16(y0 * f[0].x + x0 * f[0].y, y1 * f[1].x + x1 * f[1].y);
+        };
+        unsigned lo[HN], hi[HN];
 #pragma unroll
-        for (int ks = 0; ks < KSTEPS; ++ks) {
-            qf[ks][0] = *reinterpret_cast<const unsigned*>(s_q + g * (D + QROW_PAD) + ks * 16 + 2 * t);
-            qf[ks][1] = *reinterpret_cast<const unsigned*>(s_q + g * (D + QROW_PAD) + ks * 16 + 2 * t + 8);
+        for (int k = 0; k < HN; ++k) {               // all loads first: one round trip
+            const int h = threadIdx.x / LPH + k * HSTEP;
+            const uint16_t* row = Q + (size_t)(hk * G + (h < G ? h : 0)) * D + 2 * p2;   // n_q = 1
+            lo[k] = *reinterpret_cast<const unsigned*>(row);
+            hi[k] = *reinterpret_cast<const unsigned*>(row + HALF);
         }
-
-        const float scale = 1.4426950408889634f * rsqrtf((float)D);
-        float o[DBLK][4];
+        // fused step: the new token's key and value rows come in with the query; the key is rotated with the query's
+        // factors (same token, same position) and both wait in shared memory for the warp whose unit holds the token's slot
+        const bool prep_new = new_slot >= 0 && threadIdx.x < LPH;
+        unsigned klo = 0, khi = 0, vlo = 0, vhi = 0;
+        if (prep_new) {
+            const size_t off = (size_t)hk * D + 2 * p2;
+            klo = *reinterpret_cast<const unsigned*>(Knew + off); khi = *reinterpret_cast<const unsigned*>(Knew + off + HALF);
+            vlo = *reinterpret_cast<const unsigned*>(Vnew + off); vhi = *reinterpret_cast<const unsigned*>(Vnew + off + HALF);
+        }
 #pragma unroll
-        for (int i = 0; i < DBLK; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-        float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};   // heads 2t, 2t+1 (l: this thread's share)
-        const int lm_i = lane >> 3, lm_r = lane & 7;   // ldmatrix: which 8x8 matrix this lane addresses, and its row
-        const int new_row16 = new_slot & ~15;          // first slot of the unit that holds the new token (fused step)
+        for (int k = 0; k < HN; ++k) {
+            const int h = threadIdx.x / LPH + k * HSTEP;
+            if (h >= 8) continue;
+            rotate2(lo[k], hi[k]);
+            *reinterpret_cast<unsigned*>(sh.q + h * (D + QROW_PAD) + 2 * p2) = h < G ? lo[k] : 0u;
+            *reinterpret_cast<unsigned*>(sh.q + h * (D + QROW_PAD) + HALF + 2 * p2) = h < G ? hi[k] : 0u;
+        }
+        if (prep_new) {
+            rotate2(klo, khi);
+            *reinterpret_cast<unsigned*>(sh.fresh + 2 * p2) = klo;
+            *reinterpret_cast<unsigned*>(sh.fresh + HALF + 2 * p2) = khi;
+            *reinterpret_cast<unsigned*>(sh.fresh + D + 2 * p2) = vlo;
+            *reinterpret_cast<unsigned*>(sh.fresh + D + HALF + 2 * p2) = vhi;
+        }
+        if (threadIdx.x == 0) sh.tag = (int)(ep + 1);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int ks = 0; ks < KSTEPS; ++ks) {            // B fragments of Q^T: (d = ks*16 + 2t.., head g)
+        qf[ks][0] = *reinterpret_cast<const unsigned*>(sh.q + g * (D + QROW_PAD) + ks * 16 + 2 * t);
+        qf[ks][1] = *reinterpret_cast<const unsigned*>(sh.q + g * (D + QROW_PAD) + ks * 16 + 2 * t + 8);
+    }
+    if (threadIdx.x == 0) STAMP(4);                  // rotated query in shared memory
 
-        for (int r = 0; r < n_rounds; ++r) {
-            if (__builtin_expect(r > 0, 0)) {          // (larger caches only) the previous round is consumed: load the next
-                __syncwarp();
-                get_units(r, u);
-                issue_front(u);
-            }
-            cp_async_wait<1>();                        // the key units have landed (the value unit may be in flight)
+    const float scale = 1.4426950408889634f * rsqrtf((float)D);
+    float o[DBLK][4];
+#pragma unroll
+    for (int i = 0; i < DBLK; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};   // heads 2t, 2t+1 (l: this thread's share)
+
+    for (int r = 0; r < n_rounds; ++r) {
+        if (__builtin_expect(r > 0, 0)) {              // (larger caches only) the previous round is consumed: load the next
             __syncwarp();
-            if (threadIdx.x == 32 && r == 0) STAMP(5);   // warp 1 has its keys
-            // where the value units go: unit 0 has its own slot, units 1 and 2 take over the slots of key units 0 and 1
-            unsigned char* const sv[UPW] = {my + UPW * ITEM_BYTES, my, my + ITEM_BYTES};
-            int newj = -1;                             // the unit of this warp that holds the new token, if any
+            get_units(r, u);
+            front(false);
+        }
+        if (threadIdx.x == 32 && r == 0) STAMP(5);     // warp 1 has its keys and the query
+        int newj = -1;                                 // the unit of this warp that holds the new token, if any
 #pragma unroll
-            for (int j = 0; j < UPW; ++j)
-                if (new_slot >= 0 && u.row[j] == new_row16) newj = j;
-            if (__builtin_expect(newj >= 0, 0)) {
-                // fused append, key half: the rotated key goes into its shared-memory row and into the cache
-                uint16_t* kdst = const_cast<uint16_t*>(Kh) + (size_t)new_slot * D;
-                unsigned char* skw = my + newj * ITEM_BYTES;
-#pragma unroll 1
-                for (int e2 = lane; e2 < D; e2 += 32) {
-                    const uint16_t kvl = s_new[e2];
-                    kdst[e2] = kvl;
-                    *reinterpret_cast<uint16_t*>(skw + lay_off(new_slot & 15, e2 >> 3) + (e2 & 7) * 2) = kvl;
+        for (int j = 0; j < UPW; ++j)
+            if (new_slot >= 0 && j < u.n && u.row[j] == new_row16) newj = j;
+        if (__builtin_expect(newj >= 0, 0)) {
+            // fused append, key half: the rotated key goes into its row of the fragments and into the cache
+            const int r16 = new_slot & 15;
+            const uint16_t* fresh = sh.fresh;
+            if (lane < CH)
+                *reinterpret_cast<uint4*>(const_cast<uint16_t*>(Kh) + (size_t)new_slot * D + lane * 8) = *reinterpret_cast<const uint4*>(fresh + lane * 8);
+            if (newj == RPW) {
+                if (lane < CH) *reinterpret_cast<uint4*>(my + RPW * ITEM_BYTES + lay_off(r16, lane)) = *reinterpret_cast<const uint4*>(fresh + lane * 8);
+                __syncwarp();
+            } else if (g == (r16 & 7)) {
+#pragma unroll
+                for (int j = 0; j < RPW; ++j)
+                    if (j == newj)
+#pragma unroll
+                        for (int ks = 0; ks < KSTEPS; ++ks) {
+                            const unsigned x = *reinterpret_cast<const unsigned*>(fresh + ks * 16 + 2 * t), y = *reinterpret_cast<const unsigned*>(fresh + ks * 16 + 2 * t + 8);
+                            if (r16 < 8) { kf[j][ks][0] = x; kf[j][ks][2] = y; }
+                            else { kf[j][ks][1] = x; kf[j][ks][3] = y; }
+                        }
+            }
+        }
+        // The rest of the round, compiled for each number of units: with conditions around the single MMAs it was
+        // slower than one straight run even for the CTAs that have all three.
+        auto attend = [&](auto NU_) {
+            constexpr int NU = decltype(NU_)::value;
+            // ---- S^T[16 NU keys x 8 heads] = K Q^T: independent accumulation chains ----
+            float s[NU][4];
+#pragma unroll
+            for (int j = 0; j < NU; ++j) s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < KSTEPS; ++ks) {
+                unsigned a2[4];
+                if (NU > RPW) key_fragment(RPW, ks, a2);
+#pragma unroll
+                for (int j = 0; j < NU; ++j) {
+                    unsigned(&a)[4] = j < RPW ? kf[j < RPW ? j : 0][ks] : a2;
+                    mma_bf16(s[j], a[0], a[1], a[2], a[3], qf[ks][0], qf[ks][1]);
+                }
+            }
+            // ---- value fragments take the key fragments' registers while the softmax runs ----
+            cp_async_wait<0>();
+            __syncwarp();
+            if (__builtin_expect(newj >= 0, 0)) {          // fused append, value half
+                uint16_t* vdst = const_cast<uint16_t*>(Vh) + (size_t)new_slot * D;
+                unsigned char* slot = newj == 0 ? sv[0] : (newj == 1 ? sv[1] : sv[2]);
+                if (lane < CH) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(sh.fresh + D + lane * 8);
+                    *reinterpret_cast<uint4*>(vdst + lane * 8) = v;
+                    *reinterpret_cast<uint4*>(slot + lay_off(new_slot & 15, lane)) = v;
                 }
                 __syncwarp();
             }
-            // ---- S^T[48 keys x 8 heads] = K Q^T: three independent accumulation chains ----
-            float s[UPW][4];
 #pragma unroll
-            for (int j = 0; j < UPW; ++j) s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
-            // (fragment loads in batches ahead of the MMAs that use them)
-#pragma unroll
-            for (int ks = 0; ks < KSTEPS; ks += 2) {
-                unsigned a[UPW][2][4];
-#pragma unroll
-                for (int j = 0; j < UPW; ++j)
-#pragma unroll
-                    for (int kk = 0; kk < 2; ++kk) {
-                        if (u.row[j] < 0) continue;    // warp-uniform
-                        const int key = (lm_i & 1) * 8 + lm_r;
-                        const int chunk = (ks + kk) * 2 + (lm_i >> 1);
-                        ldmatrix_x4(a[j][kk][0], a[j][kk][1], a[j][kk][2], a[j][kk][3], my + j * ITEM_BYTES + lay_off(key, chunk));
-                    }
-#pragma unroll
-                for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-                    for (int j = 0; j < UPW; ++j) {
-                        if (u.row[j] < 0) continue;
-                        mma_bf16(s[j], a[j][kk][0], a[j][kk][1], a[j][kk][2], a[j][kk][3], qf[ks + kk][0], qf[ks + kk][1]);
-                    }
-            }
-            __syncwarp();                              // every lane has its key fragments: the key slots are free
-#pragma unroll
-            for (int j = 1; j < UPW; ++j)
-                if (u.row[j] >= 0) load_unit(Vh, u.row[j], sv[j]);
-            cp_async_commit();                         // copy group 3 (possibly empty)
-            // scale, mask slots outside [lo, hi), column (head) maxima over the warp's keys
+            for (int db = 0; db < DBLK; ++db) value_fragment(0, db, kf[0][db]);
+            // scale, mask keys outside the unit's valid range, column (head) maxima over the warp's keys
             float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-            for (int j = 0; j < UPW; ++j)
+            for (int j = 0; j < NU; ++j)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int key = u.k0[j] + g + (e >> 1) * 8;
-                    const bool in = u.row[j] >= 0 && key >= u.lo[j] && key < u.hi[j];
+                    const int key = g + (e >> 1) * 8;
+                    const bool in = key >= (u.lohi[j] & 0xFF) && key < (u.lohi[j] >> 8);
                     s[j][e] = in ? s[j][e] * scale : -INFINITY;
                     mx[e & 1] = fmaxf(mx[e & 1], s[j][e]);
                 }
@@ -1126,6 +1158,9 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
                 mx[0] = fmaxf(mx[0], __shfl_xor_sync(0xffffffffu, mx[0], sft));
                 mx[1] = fmaxf(mx[1], __shfl_xor_sync(0xffffffffu, mx[1], sft));
             }
+            if (NU > 1)
+#pragma unroll
+                for (int db = 0; db < DBLK; ++db) value_fragment(1, db, kf[1][db]);
             float corr[2], mu[2];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -1135,9 +1170,9 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
                 m[c] = mn;
                 l[c] *= corr[c];
             }
-            unsigned pb[UPW][2];   // P^T as B fragments, per unit: [k halves]
+            unsigned pb[NU][2];   // P^T as B fragments, per unit: [k halves]
 #pragma unroll
-            for (int j = 0; j < UPW; ++j) {
+            for (int j = 0; j < NU; ++j) {
                 float p[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -1155,52 +1190,38 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
                     o[db][1] *= corr[1]; o[db][3] *= corr[1];
                 }
             }
-            // ---- O^T[D x 8 heads] += V^T P^T, unit by unit as the values arrive ----
+            // ---- O^T[D x 8 heads] += V^T P^T ----
 #pragma unroll
-            for (int j = 0; j < UPW; ++j) {
-                if (j == 0) cp_async_wait<1>();        // the first value unit (copied before the scores)
-                if (j == 1) cp_async_wait<0>();        // the two that followed the scores
-                if (j < 2) __syncwarp();
-                if (u.row[j] < 0) continue;
-                if (__builtin_expect(newj == j, 0)) {  // fused append, value half
-                    uint16_t* vdst = const_cast<uint16_t*>(Vh) + (size_t)new_slot * D;
-#pragma unroll 1
-                    for (int e2 = lane; e2 < D; e2 += 32) {
-                        const uint16_t vvl = s_new[D + e2];
-                        vdst[e2] = vvl;
-                        *reinterpret_cast<uint16_t*>(sv[j] + lay_off(new_slot & 15, e2 >> 3) + (e2 & 7) * 2) = vvl;
-                    }
-                    __syncwarp();
-                }
-#pragma unroll
-                for (int db = 0; db < DBLK; db += 4) {
-                    unsigned a[4][4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int key = (lm_i >> 1) * 8 + lm_r;
-                        const int chunk = (db + q) * 2 + (lm_i & 1);
-                        ldmatrix_x4_trans(a[q][0], a[q][1], a[q][2], a[q][3], sv[j] + lay_off(key, chunk));
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) mma_bf16(o[db + q], a[q][0], a[q][1], a[q][2], a[q][3], pb[j][0], pb[j][1]);
-                }
+            for (int db = 0; db < DBLK; ++db) {
+                mma_bf16(o[db], kf[0][db][0], kf[0][db][1], kf[0][db][2], kf[0][db][3], pb[0][0], pb[0][1]);
+                if (NU > RPW) value_fragment(RPW, db, kf[0][db]);      // (unit 0's registers are free)
             }
-        }
-        if (threadIdx.x == 32) STAMP(6);             // warp 1 through with its units
-        // l: sum the shares of the 8 lane groups that hold the same heads
 #pragma unroll
-        for (int sft = 4; sft < 32; sft <<= 1) {
-            l[0] += __shfl_xor_sync(0xffffffffu, l[0], sft);
-            l[1] += __shfl_xor_sync(0xffffffffu, l[1], sft);
-        }
-        // the slots are free once all consumer warps are here (the merge waits for that)
-#ifdef SVLM_DECODE_TRACE
-        auto stamp7 = [&](int i) { STAMP(i); };
-#else
-        auto stamp7 = [](int) {};
-#endif
-        cta_merge_and_record<D, true>(o, m, l, reinterpret_cast<float*>(ring), part, (unsigned)sh.tag, stamp7);
+            for (int j = 1; j < NU; ++j)
+#pragma unroll
+                for (int db = 0; db < DBLK; ++db) {
+                    unsigned(&a)[4] = kf[j < RPW ? j : 0][db];
+                    mma_bf16(o[db], a[0], a[1], a[2], a[3], pb[j][0], pb[j][1]);
+                }
+        };
+        if (u.n == 3) attend(std::integral_constant<int, 3>{});
+        else if (u.n == 2) attend(std::integral_constant<int, 2>{});
+        else if (u.n == 1) attend(std::integral_constant<int, 1>{});
     }
+    if (threadIdx.x == 32) STAMP(6);             // warp 1 through with its units
+    // l: sum the shares of the 8 lane groups that hold the same heads
+#pragma unroll
+    for (int sft = 4; sft < 32; sft <<= 1) {
+        l[0] += __shfl_xor_sync(0xffffffffu, l[0], sft);
+        l[1] += __shfl_xor_sync(0xffffffffu, l[1], sft);
+    }
+    // the slots are free once all warps are here (the merge waits for that)
+#ifdef SVLM_DECODE_TRACE
+    auto stamp7 = [&](int i) { STAMP(i); };
+#else
+    auto stamp7 = [](int) {};
+#endif
+    cta_merge_and_record<D, true>(o, m, l, reinterpret_cast<float*>(ring), part, stamp7, &sh.tag);
 
     // ---- the first splits of this KV head combine all the splits' records -----------------------------
     __syncthreads();                                  // the merge slabs in `ring` are read
@@ -1225,7 +1246,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
 
 template <int D>
 constexpr size_t decode_layer_smem() {
-    return sizeof(LayShared) + 128 + (size_t)DEC_CWARPS * LAY_SLOTS * UNIT * D * 2 + 8 * (D + QROW_PAD) * 2 + 2 * D * 2;
+    return sizeof(LayShared) + 128 + (size_t)DEC_CWARPS * LAY_SLOTS * UNIT * D * 2;
 }
 static_assert(merge_bytes<128>() <= (size_t)DEC_CWARPS * LAY_SLOTS * UNIT * 128 * 2 && merge_bytes<64>() <= (size_t)DEC_CWARPS * LAY_SLOTS * UNIT * 64 * 2,
               "the merge slabs live in the warps' slots");
@@ -1261,7 +1282,7 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
     const int problems = b.n_caches * n_layers;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(splits, b.kv_heads, problems);
-    cfg.blockDim = dim3(DEC_THREADS);
+    cfg.blockDim = dim3(problems == 1 && tagged ? LAY_THREADS : DEC_THREADS);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
