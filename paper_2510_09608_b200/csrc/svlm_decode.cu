@@ -945,9 +945,9 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
         for (int i = lane; i < UNIT * CH; i += 32) cp_async16(dst + lay_off(i / CH, i % CH), src + (size_t)i * 8);
     };
     // the value units that have to wait for a key slot go towards L2 meanwhile
-    auto value_to_l2 = [&](int row) {
+    auto rows_to_l2 = [&](const uint16_t* base, int row) {
         for (int o = lane * 128; o < ITEM_BYTES; o += 32 * 128)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(Vh + (size_t)row * D) + o));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(base + (size_t)row * D) + o));
     };
     // where the value units go: unit 0 has its own slot, units 1 and 2 take over the slots of key units 0 and 1
     unsigned char* const sv[UPW] = {my + UPW * ITEM_BYTES, my, my + ITEM_BYTES};
@@ -972,7 +972,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
             if (j < u.n) {
                 load_unit(Kh, u.row[j], my + j * ITEM_BYTES);
                 if (j == 0) load_unit(Vh, u.row[0], sv[0]);
-                else value_to_l2(u.row[j]);
+                else rows_to_l2(Vh, u.row[j]);
             }
             cp_async_commit();
             if (paced) cp_async_wait<0>();
@@ -994,6 +994,17 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     if (n_rounds > 0) {
         get_units(0, u);
         front(early_loads == 2);
+        // The units of a second round (many KV heads, large windows) come out of L2 then: ask for them now, while the
+        // predecessor still runs and HBM would idle (8 KV heads of 9216 keys: 11.1 -> 10.1 us; asking for four rounds
+        // at once is slower again).
+        if (early_loads)
+            for (int r = 1; r < min(n_rounds, 2); ++r) {
+                Units v;
+                get_units(r, v);
+#pragma unroll
+                for (int j = 0; j < UPW; ++j)
+                    if (j < v.n) { rows_to_l2(Kh, v.row[j]); rows_to_l2(Vh, v.row[j]); }
+            }
     }
     if (threadIdx.x == 0) STAMP(2);                  // the first round's keys are in registers
 
@@ -1263,6 +1274,11 @@ size_t svlm_decode_ws_floats(int layers, int kv_heads, int head_dim, int splits)
 size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits) {
     return ll_head_bytes(kv_heads) + (size_t)kv_heads * splits * (head_dim == 128 ? ll_rec_bytes<128>() : ll_rec_bytes<64>());
 }
+
+// The per-layer kernel holds one round of a CTA's keys and values on chip before the query comes and the next in L2; with a
+// third round it is only a slower streaming kernel (16 query / 8 KV heads, 17,408 keys, 4 rounds: 19.4 us, streaming
+// 17.9; two rounds: 9.3 against 11.5).
+bool svlm_decode_streams(int pages, int splits) { return (8 * pages + splits - 1) / splits > 2 * GROUP; }
 
 bool svlm_decode_supported(int n_pages) { return n_pages <= DEC_MAX_TILES; }
 

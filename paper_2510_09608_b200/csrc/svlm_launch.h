@@ -95,6 +95,8 @@ bool svlm_decode_supported(int n_pages);
 cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
                                int q_heads, void* out, int splits, const void* Knew, const void* Vnew, int early_loads,
                                void* tagged, cudaStream_t st);
+// One problem with so many pages per CTA that the streaming kernel is the better one (either gives the same result).
+bool svlm_decode_streams(int pages, int splits);
 size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits);
 
 // Q/K/V projection with the append as its epilogue, head_dim 128 (svlm_qkv_sm100.cu).  tmX, tmW: host copies of

@@ -275,7 +275,8 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     if (n_q == 1 && group <= 8 && svlm_decode_supported(c0->dev.n_pages)) {
         // split-KV decode; every cache's scratch was sized for this launch shape at creation
         const int splits = svlm_decode_splits(c0->dev.n_pages, c0->dev.kv_heads, n_caches * n_layers);
-        SVLM_CUDA(svlm_launch_decode(b, layer0, n_layers, Q, q_pos, q_heads, out, splits, Knew, Vnew, early, c0->decode_tagged, c0->stream));
+        void* tagged = svlm_decode_streams(expected_pages(c0), splits) ? nullptr : c0->decode_tagged;
+        SVLM_CUDA(svlm_launch_decode(b, layer0, n_layers, Q, q_pos, q_heads, out, splits, Knew, Vnew, early, tagged, c0->stream));
         return SVLM_OK;
     }
     if (Knew) return SVLM_ERR_ARG;   // the fused step exists for the split-KV kernel only
