@@ -1,10 +1,11 @@
 // Projections of a few tokens at a time (decode): Y = X W^T for n <= 16 rows of X.  With so few rows the
-// work is reading W once, so this is a bandwidth kernel, not a tensor-core one: a warp owns output rows
-// (one row of W each, 16-byte loads, several in flight per lane), multiplies them with all n token vectors
-// held in shared memory, accumulates in fp32 and reduces with shuffles (up to 4 tokens; more take the
-// tensor-core form further down).  It serves svlm_out_proj for small n, on both sides of the decode step: [q | k | v] = W_qkv x before svlm_decode_step, W_o a after it.
+// work is reading W once, so these are bandwidth kernels; the arithmetic rides on mma.sync, with the tokens as (mostly
+// empty) M rows, because it takes a fifth of the instructions of unpacking and multiplying on the FMA pipe.  They serve
+// svlm_out_proj for small n, on both sides of the decode step: [q | k | v] = W_qkv x before svlm_decode_step, W_o a after it.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "svlm_dev.h"
 #include "svlm_launch.h"
@@ -12,89 +13,191 @@
 
 namespace {
 
-constexpr int GV_THREADS = 256;
-// 16-byte chunks of a W row in flight per lane: the fewer token vectors share the registers, the more loads
-template <int NX> __host__ __device__ constexpr int gv_unroll() { return NX == 1 ? 16 : (NX <= 4 ? 8 : 4); }
+__device__ __forceinline__ void mma_bf16_16816(float* c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
 
-template <int NX>
-__global__ void __launch_bounds__(GV_THREADS) gemv_kernel(const uint16_t* __restrict__ X, const uint16_t* __restrict__ W,
-                                                         uint16_t* __restrict__ Y, int n, int in_dim, int out_dim) {
-    constexpr int GV_UNROLL = gv_unroll<NX>();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint4* sx = reinterpret_cast<uint4*>(smem_raw);            // [NX][in_dim / 8] chunks of 8 bf16; rows >= n are zero
-    const int chunks = in_dim / 8;
-    const int lane = threadIdx.x & 31;
-    const int warp = blockIdx.x * (GV_THREADS / 32) + (threadIdx.x >> 5), n_warps = gridDim.x * (GV_THREADS / 32);
-    uint4 w[GV_UNROLL];
-    auto load_w = [&](int row, int c0) {
-        const uint4* wrow = reinterpret_cast<const uint4*>(W + (size_t)row * in_dim);
-#pragma unroll
-        for (int u = 0; u < GV_UNROLL; ++u) {
-            const int c = c0 + 32 * u;
-            w[u] = c < chunks ? __ldg(wrow + c) : make_uint4(0, 0, 0, 0);
-        }
-    };
-    // The weights do not depend on anything earlier in the stream: the kernel is launched while its predecessor
-    // may still run and fetches the first row of every warp at once; the token vectors wait for the predecessor.
-    svlm_ptx::pdl_launch_dependents();
-    if (warp < out_dim) load_w(warp, lane);
-    svlm_ptx::pdl_wait();
-    for (int i = threadIdx.x; i < NX * chunks; i += GV_THREADS) {
-        const int t = i / chunks;
-        sx[i] = t < n ? *reinterpret_cast<const uint4*>(X + (size_t)t * in_dim + (size_t)(i % chunks) * 8) : make_uint4(0, 0, 0, 0);
+// Up to 4 tokens.  Block i owns a run of output rows and walks it in stages of eight rows x KS elements of K; a stage
+// belongs to one warp, which computes the eight rows' partial dot products with mma.sync (a lane's 16 bytes of a W row are
+// the B fragments of two MMAs: a dot product does not care in which order k is summed).  A warp's stages come in turn
+// through a shared-memory slot (cp.async.bulk) and through registers, so there are no hand-offs between warps.  Partial
+// sums wait in shared memory and are added in the order of K at the end: the same bits every time.
+// The weights depend on nothing earlier in the stream: while the predecessor still runs (programmatic dependent launch)
+// the block fills slots and registers (135 KB) and asks for the rest of its rows into L2; behind the wait only the token
+// vectors come from the predecessor.  Sized to fit beside a decode step's CTA: a decoder's chain of projections and decode
+// steps otherwise leaves HBM idle while a decode step combines its partial results.  Chain of 3584 -> 4608, decode step,
+// 3584 -> 3584 (77.6 MB): 28.9 us per layer with two blocks per SM that fetched one row per warp ahead, 24.5 with slots
+// only (each refill is a round trip to L2 of over 1 us), 23.3 with both.
+constexpr int GV_THREADS = 256;
+constexpr int GT_WARPS = 8;
+constexpr int GT_SLOTS = GT_WARPS;      // one per warp
+constexpr int GT_KS = 512;              // most elements of K in a stage
+constexpr int GT_KB = GT_KS / 32;       // k-blocks of 32
+constexpr int GT_ROW = GT_KS * 2 + 64;  // bytes between a stage's rows: two rows' 64-byte pieces fill the 32 banks
+constexpr int GT_MAX_STAGES = 64;       // stages of one block (partial sums in shared memory); more rows take more blocks
+constexpr int GT_PAD = 32;              // elements between the token rows, for the same reason
+constexpr int GT_MAX_X = 100 * 1024;    // bytes of the token rows
+
+struct __align__(16) GtShared {
+    float part[GT_MAX_STAGES][4][8];    // [stage][token][row]
+    unsigned long long full[GT_SLOTS];
+    int abort_flag;
+};
+static_assert(sizeof(GtShared) % 16 == 0 && (GT_SLOTS * 8 * GT_ROW) % 128 == 0 && GT_ROW % 16 == 0 && GT_PAD % 8 == 0, "16-byte accesses");
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, void* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(svlm_ptx::smem_u32(dst)), "l"(src), "r"(bytes), "r"(svlm_ptx::smem_u32(bar)) : "memory");
+}
+
+// parts: stages per group of eight rows; ks: elements of K per stage (a multiple of 64; the last part may be shorter)
+__global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16_t* __restrict__ X, const uint16_t* __restrict__ W,
+                                                                 uint16_t* __restrict__ Y, int n, int in_dim, int out_dim, int parts,
+                                                                 int ks, SvlmCtrl* ctrl) {
+    using namespace svlm_ptx;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char* ring = smem_raw;                                         // [slot][8 rows][GT_ROW]
+    GtShared& sh = *reinterpret_cast<GtShared*>(ring + GT_SLOTS * 8 * GT_ROW);
+    uint16_t* sx = reinterpret_cast<uint16_t*>(&sh + 1);                    // [n][in_dim + GT_PAD]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, kq = lane & 3;
+    const int r0 = (int)((long long)out_dim * blockIdx.x / gridDim.x), r1 = (int)((long long)out_dim * (blockIdx.x + 1) / gridDim.x);
+    const int n_stages = (r1 - r0 + 7) / 8 * parts;
+    volatile int* abort_flag = &sh.abort_flag;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < GT_SLOTS; ++i) mbar_init(&sh.full[i], 1);
+        sh.abort_flag = 0;
+        mbar_init_fence();
     }
     __syncthreads();
-    for (int row = warp; row < out_dim; row += n_warps) {
-        float acc[NX];
+    pdl_launch_dependents();
+    // stage s: rows from r0 + (s / parts) * 8, elements from (s % parts) * ks.  A warp's stages are warp, warp + GT_WARPS, ...:
+    // those at even places come through its slot, those at odd places through registers.
+    auto fetch = [&](int s) {
+        if (s >= n_stages) return;
+        const int row = r0 + s / parts * 8, k0 = s % parts * ks, rows = min(8, r1 - row), len = min(ks, in_dim - k0) * 2;
+        void* bar = &sh.full[warp];
+        if (lane == 0) mbar_expect_tx(bar, rows * len);
+        __syncwarp();
+        if (lane < rows) bulk_load(ring + (warp * 8 + lane) * GT_ROW, W + (size_t)(row + lane) * in_dim + k0, len, bar);
+    };
+    uint4 wr[GT_KB];
+    auto load_regs = [&](int s) {
+        if (s >= n_stages) return;
+        const int row = min(r0 + s / parts * 8 + g, r1 - 1), k0 = s % parts * ks, kbs = min(ks, in_dim - k0) / 32;
+        const uint4* p = reinterpret_cast<const uint4*>(W + (size_t)row * in_dim + k0) + kq;
 #pragma unroll
-        for (int t = 0; t < NX; ++t) acc[t] = 0.f;
-        for (int c0 = lane; c0 < chunks; c0 += 32 * GV_UNROLL) {
-            if (row != warp || c0 != lane) load_w(row, c0);      // the first batch is already here
+        for (int kb = 0; kb < GT_KB; ++kb) wr[kb] = kb < kbs ? __ldg(p + 4 * kb) : make_uint4(0, 0, 0, 0);
+    };
+    fetch(warp);
+    load_regs(warp + GT_WARPS);
+    {   // whole groups behind those: rows lie one after another
+        const int row = min(r0 + 2 * GT_WARPS / parts * 8, r1);
+        const char* p = reinterpret_cast<const char*>(W + (size_t)row * in_dim);
+        const size_t bytes = (size_t)(r1 - row) * in_dim * 2;               // a multiple of 128
+        for (size_t o = (size_t)threadIdx.x * 2048; o < bytes; o += GT_WARPS * 32 * 2048)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p + o), "r"((unsigned)min((size_t)2048, bytes - o)) : "memory");
+    }
+    const unsigned wait_limit = __ldcg(&ctrl->wait_limit);                  // written at creation only, never by a kernel
+    pdl_wait();
+    const int row16 = in_dim / 8;                                           // 16-byte chunks of a token row
+    for (int i = threadIdx.x; i < n * row16; i += GT_WARPS * 32)
+        *reinterpret_cast<uint4*>(sx + (size_t)(i / row16) * GT_PAD + (size_t)i * 8) = __ldcg(reinterpret_cast<const uint4*>(X) + i);
+    __syncthreads();
+    const bool live = g < n;
+    const uint16_t* xrow = sx + (size_t)min(g, n - 1) * (in_dim + GT_PAD) + kq * 8;
+    auto put = [&](int s, const float (&c)[4][4]) {
+        if (live)
+            *reinterpret_cast<float2*>(&sh.part[s][g][2 * kq]) = make_float2((c[0][0] + c[1][0]) + (c[2][0] + c[3][0]), (c[0][1] + c[1][1]) + (c[2][1] + c[3][1]));
+    };
+    unsigned phase = 0;
+    for (int s = warp; s < n_stages; s += 2 * GT_WARPS) {
+        const int s1 = s + GT_WARPS;
+        if (s1 < n_stages) {
+            const int k0 = s1 % parts * ks, last = min(ks, in_dim - k0) / 32 - 1;
+            const uint16_t* xs = xrow + k0;
+            float c[4][4] = {};                                             // four independent chains
 #pragma unroll
-            for (int u = 0; u < GV_UNROLL; ++u) {
-                const int c = c0 + 32 * u;
-                if (c >= chunks) continue;
-                const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&w[u]);
-                float2 wf[4];
+            for (int kb = 0; kb < GT_KB; ++kb) {
+                uint4 a = *reinterpret_cast<const uint4*>(xs + min(kb, last) * 32);
+                if (!live || kb > last) a = make_uint4(0, 0, 0, 0);
+                mma_bf16_16816(c[2 * (kb & 1)], a.x, 0u, a.y, 0u, wr[kb].x, wr[kb].y);
+                mma_bf16_16816(c[2 * (kb & 1) + 1], a.z, 0u, a.w, 0u, wr[kb].z, wr[kb].w);
+            }
+            load_regs(s1 + 2 * GT_WARPS);
+            put(s1, c);
+        }
+        const bool ok = mbar_wait(&sh.full[warp], phase, abort_flag, wait_limit);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        phase ^= 1;
+        const int k0 = s % parts * ks, kbs = min(ks, in_dim - k0) / 32;     // an even number
+        const unsigned char* wrow = ring + (warp * 8 + g) * GT_ROW + kq * 16;
+        const uint16_t* xs = xrow + k0;
+        float c[4][4] = {};
+#pragma unroll 2
+        for (int kb = 0; kb < kbs; kb += 2) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) wf[q] = __bfloat1622float2(wp[q]);
-#pragma unroll
-                for (int t = 0; t < NX; ++t) {
-                    const uint4 xv = sx[t * chunks + c];
-                    const __nv_bfloat162* xp = reinterpret_cast<const __nv_bfloat162*>(&xv);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float2 xf = __bfloat1622float2(xp[q]);
-                        acc[t] = fmaf(wf[q].x, xf.x, acc[t]);
-                        acc[t] = fmaf(wf[q].y, xf.y, acc[t]);
-                    }
-                }
+            for (int u = 0; u < 2; ++u) {
+                const uint4 w = *reinterpret_cast<const uint4*>(wrow + (kb + u) * 64);
+                uint4 a = *reinterpret_cast<const uint4*>(xs + (kb + u) * 32);
+                if (!live) a = make_uint4(0, 0, 0, 0);
+                mma_bf16_16816(c[2 * u], a.x, 0u, a.y, 0u, w.x, w.y);
+                mma_bf16_16816(c[2 * u + 1], a.z, 0u, a.w, 0u, w.z, w.w);
             }
         }
-#pragma unroll
-        for (int t = 0; t < NX; ++t) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
+        __syncwarp();
+        fence_proxy_async();                                                // the slot's reads before the copy that refills it
+        fetch(s + 2 * GT_WARPS);
+        put(s, c);
+    }
+    __syncthreads();
+    if (sh.abort_flag) {
+        // Somebody gave up.  Copies already issued still land in this block's shared memory: give every barrier a
+        // bounded chance to complete before the memory is released.
+        if (threadIdx.x == 0) {
+            for (int i = 0; i < GT_SLOTS; ++i)
+                for (unsigned p = 0; p < 2; ++p)
+                    for (unsigned w = 0; w < (1u << 12) && !mbar_test(&sh.full[i], p); ++w) __nanosleep(32);
+            atomicCAS(&ctrl->status, 0, -5);   // SVLM_ERR_TIMEOUT
         }
-        if (lane == 0) {
-#pragma unroll
-            for (int t = 0; t < NX; ++t)
-                if (t < n) Y[(size_t)t * out_dim + row] = __bfloat16_as_ushort(__float2bfloat16_rn(acc[t]));
-        }
+        __syncthreads();
+        return;
+    }
+    for (int i = threadIdx.x; i < (r1 - r0) * n; i += GT_WARPS * 32) {
+        const int t = i / (r1 - r0), r = i - t * (r1 - r0);
+        float sum = 0.f;
+        for (int p = 0; p < parts; ++p) sum += sh.part[(r >> 3) * parts + p][t][r & 7];
+        Y[(size_t)t * out_dim + r0 + r] = __bfloat16_as_ushort(__float2bfloat16_rn(sum));
     }
 }
 
-// 5 to 16 tokens: the tokens are the M = 16 rows of mma.sync.m16n8k16, eight rows of W the N.  A block owns
+cudaError_t launch_few(const uint16_t* X, const uint16_t* W, uint16_t* Y, int n, int in_dim, int out_dim, SvlmCtrl* ctrl, cudaStream_t st) {
+    const size_t fixed = (size_t)GT_SLOTS * 8 * GT_ROW + sizeof(GtShared);
+    // (the limit of the longest token rows this kernel takes, so that a later call finds it raised)
+    const cudaError_t e = svlm_allow_smem<gemv_few_kernel>(fixed + GT_MAX_X);
+    if (e != cudaSuccess) return e;
+    const int parts = (in_dim + GT_KS - 1) / GT_KS;
+    const int ks = ((in_dim + parts - 1) / parts + 63) / 64 * 64;
+    const int most_rows = GT_MAX_STAGES / parts * 8;
+    const int blocks = std::max(std::min((out_dim + 7) / 8, svlm_sm_count()), (out_dim + most_rows - 1) / most_rows);
+    return svlm_launch_chained(gemv_few_kernel, dim3(blocks), dim3(GT_WARPS * 32), fixed + (size_t)n * (in_dim + GT_PAD) * 2, 1, st, X, W, Y, n,
+                               in_dim, out_dim, parts, ks, ctrl);
+}
+
+// What the kernel above takes: the token rows fit beside the ring, a group's stages fit the partial sums, and the last
+// stage of a group is not empty (in_dim is a multiple of 64).
+bool few_supported(int n, int in_dim) {
+    const int parts = (in_dim + GT_KS - 1) / GT_KS;
+    const int ks = ((in_dim + parts - 1) / parts + 63) / 64 * 64;
+    return n <= 4 && in_dim % 64 == 0 && parts <= GT_MAX_STAGES && (parts - 1) * ks < in_dim && (size_t)n * (in_dim + GT_PAD) * 2 <= GT_MAX_X;
+}
+
+// More tokens, up to 16 (or longer rows than the kernel above takes): the tokens are the M = 16 rows of mma.sync.m16n8k16, eight rows of W the N.  A block owns
 // eight output rows; its eight warps split K (k-blocks of 32, strided), every lane loading 16 bytes of one W
 // row and of two token rows per k-block straight into the fragment registers (the dot product does not care
 // in which order k is summed, so the eight consecutive elements a lane loads serve two MMAs), several k-blocks
 // in flight; the warps' partial tiles meet in shared memory.
 constexpr int GM_KB_IN_FLIGHT = 7;
-
-__device__ __forceinline__ void mma_bf16_16816(float* c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
 __global__ void __launch_bounds__(GV_THREADS) gemv_mma_kernel(const uint16_t* __restrict__ X, const uint16_t* __restrict__ W,
                                                              uint16_t* __restrict__ Y, int n, int in_dim, int out_dim) {
@@ -117,9 +220,12 @@ __global__ void __launch_bounds__(GV_THREADS) gemv_mma_kernel(const uint16_t* __
             w[u] = kb < n_kb ? __ldg(wp + 4 * kb) : make_uint4(0, 0, 0, 0);
         }
     };
-    // as in the FMA form: the first batch of weights is fetched before the wait for the predecessor
+    // as above: the first batch of weights is fetched before the wait for the predecessor, the rest asked into L2
+    // (5 tokens, 33 MB: 8.75 -> 7.7 us)
     svlm_ptx::pdl_launch_dependents();
     load_w(warp);
+    for (int kb = warp + (GV_THREADS / 32) * GM_KB_IN_FLIGHT; kb < n_kb; kb += GV_THREADS / 32)
+        if ((kb & 1) == 0 && kq == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(wp + 4 * kb));
     svlm_ptx::pdl_wait();
     for (int kb0 = warp; kb0 < n_kb; kb0 += (GV_THREADS / 32) * GM_KB_IN_FLIGHT) {
         uint4 a[GM_KB_IN_FLIGHT], bq[GM_KB_IN_FLIGHT];
@@ -151,52 +257,14 @@ __global__ void __launch_bounds__(GV_THREADS) gemv_mma_kernel(const uint16_t* __
     }
 }
 
-template <int NX>
-cudaError_t launch(const uint16_t* X, const uint16_t* W, uint16_t* Y, int n, int in_dim, int out_dim, cudaStream_t st) {
-    const size_t smem = (size_t)NX * in_dim * 2;
-    cudaError_t e = svlm_allow_smem<gemv_kernel<NX>>(smem);
-    if (e != cudaSuccess) return e;
-    const int rows_per_block = GV_THREADS / 32;
-    int blocks = (out_dim + rows_per_block - 1) / rows_per_block;
-    if (blocks > 2 * 148) blocks = 2 * 148;         // two resident blocks per SM, each warp walks a few rows
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(GV_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // weights are fetched under the predecessor's tail
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, gemv_kernel<NX>, X, W, Y, n, in_dim, out_dim);
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 }  // namespace
 
 bool svlm_gemv_supported(int n, int in_dim) { return n >= 1 && n <= 16 && in_dim % 32 == 0 && (size_t)4 * in_dim * 2 <= 200 * 1024; }
 
-cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, cudaStream_t st) {
+cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, SvlmCtrl* ctrl, cudaStream_t st) {
     const uint16_t* x = static_cast<const uint16_t*>(X);
     const uint16_t* w = static_cast<const uint16_t*>(W);
     uint16_t* y = static_cast<uint16_t*>(Y);
-    cudaError_t e;
-    if (n == 1) e = launch<1>(x, w, y, n, in_dim, out_dim, st);
-    else if (n <= 4) e = launch<4>(x, w, y, n, in_dim, out_dim, st);
-    else {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((out_dim + 7) / 8);
-        cfg.blockDim = dim3(GV_THREADS);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, gemv_mma_kernel, x, w, y, n, in_dim, out_dim);
-        if (e == cudaSuccess) e = cudaGetLastError();
-    }
-    svlm_count_launch();
-    return e;
+    if (few_supported(n, in_dim)) return launch_few(x, w, y, n, in_dim, out_dim, ctrl, st);
+    return svlm_launch_chained(gemv_mma_kernel, dim3((out_dim + 7) / 8), dim3(GV_THREADS), 0, 1, st, x, w, y, n, in_dim, out_dim);
 }

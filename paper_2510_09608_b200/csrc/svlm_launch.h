@@ -107,7 +107,8 @@ cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmC
 
 // Y = X W^T for a few rows of X (decode-time projections), a bandwidth kernel (svlm_gemv.cu)
 bool svlm_gemv_supported(int n, int in_dim);
-cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, cudaStream_t st);
+// ctrl: where a wait that runs out is recorded, and the poll limit
+cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, SvlmCtrl* ctrl, cudaStream_t st);
 
 // tcgen05/TMEM/TMA chunk prefill, n_q >= 2 (svlm_prefill_sm100.cu)
 bool svlm_prefill_supported(int n_pages, int group);
