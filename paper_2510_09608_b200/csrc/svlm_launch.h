@@ -100,10 +100,12 @@ bool svlm_decode_streams(int pages, int splits);
 size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits);
 
 // Q/K/V projection with the append as its epilogue, head_dim 128 (svlm_qkv_sm100.cu).  tmX, tmW: host copies of
-// the CUtensorMap of X [n][hidden] (64 x 128 box) and W [(q_heads + 2 kv_heads) * 128][hidden] (64 x 256 box), 128-byte swizzle.
+// the CUtensorMap of X [n][hidden] (64 x width / 2 box) and W [(q_heads + 2 kv_heads) * 128][hidden] (64 x 128 box), 128-byte
+// swizzle; width: svlm_proj_tile for the number of 128-row blocks of W.
 // with_append = false: the plain projection Y = X W^T with q_heads blocks of 128 output columns, all written to Q_out.
+int svlm_proj_tile(int n, int hidden, int blocks128);
 cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmCacheDev& cd, int layer, int n, int hidden,
-                                   int q_heads, bool with_append, void* Q_out, cudaStream_t st);
+                                   int q_heads, bool with_append, int width, void* Q_out, cudaStream_t st);
 
 // Y = X W^T for a few rows of X (decode-time projections), a bandwidth kernel (svlm_gemv.cu)
 bool svlm_gemv_supported(int n, int in_dim);

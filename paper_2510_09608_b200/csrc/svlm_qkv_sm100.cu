@@ -3,18 +3,31 @@
 // go to the caller's Q buffer, the key columns are rotated at each token's contiguous position
 // (paper Section 2.1, "Contiguous RoPE") and written, with the value columns, straight into the
 // token's cache slot: K and V never make a round trip through global memory between the GEMM and
-// the cache.
+// the cache.  The plain projection after the attention is the same kernel.
 //
-// A dense contraction, so it runs on the tensor cores: one CTA per 128 x 256 output tile (128 tokens x
-// two heads: head_dim is 128, so the rotation partners j and j + 64 of a key sit in the same tile; with
-// 128 x 128 tiles the operand stream out of L2, 64 flop per byte, bounded the kernel at ~700 TFLOP/s),
-// X and W tiles by TMA (128-byte swizzle) through a 4-stage ring, one thread issuing
-// tcgen05.mma (M128 N256 K16) into a 256-column TMEM accumulator, four epilogue warps reading the
-// accumulator with tcgen05.ld, one row per thread, one head after the other.  Every mbarrier wait is bounded; on expiry the CTA
-// records SVLM_ERR_TIMEOUT, drains its copies, frees its TMEM and returns.
+// A dense contraction, so it runs on the tensor cores.  Two CTAs work as a pair (cta_group::2) on a tile of 256 output
+// features x N tokens, each bringing in its own 128 rows of W and half of the tokens' rows.  The features are the M side:
+// with tokens there, a chunk of 524 would fill 3 tiles of 256 (a third of it padding); as the N side they are cut in equal
+// tiles of any multiple of 32, and the launch picks the width that fills the SM pairs best (svlm_proj_tile).
+// What bounded the kernel was the pace of its single threads, not memory or math: 690 cycles per k-block in the issuing
+// thread (stage numbers by division, descriptors moved into uniform registers one by one), whatever the tile, so that 32
+// to 1024 tokens all took 25-29 us at hidden 3584.  With counted stages, the whole warp in the issuer's loop and two
+// producers a k-block takes the 2 N cycles of its math, from N = 160 on; below that the issuer's 320.
+// Hidden 3584, 4608 features, us: 32 tokens 25.4 -> 12.5, 531 tokens 27.6 -> 17.1, 1024 tokens 29.2 -> 25.3, 4096 tokens
+// 107 -> 99 (1364 TFLOP/s; the clock then drops with the power limit).
+//   warps 0, 10  TMA (128-byte swizzle) into a ring of up to eight stages, in turns; both CTAs' bytes are counted on the
+//                leader's barrier
+//   warp 1       of the leading CTA: one thread issues tcgen05.mma M256 N K16 into N TMEM columns of both CTAs
+//   warps 2-9    epilogue: a CTA's 128 accumulator rows are one head; they are transposed through shared memory (the ring,
+//                idle by then), so that a token's row leaves in one coalesced 256-byte store and a key's rotation
+//                partners j, j + 64 meet in one lane
+// Every mbarrier wait is bounded; on expiry the CTA records SVLM_ERR_TIMEOUT, drains its copies, meets its partner at the
+// cluster barrier, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "svlm_dev.h"
 #include "svlm_launch.h"
@@ -27,193 +40,212 @@ namespace {
 using namespace svlm_ptx;
 using namespace svlm_tc;
 
-constexpr int QK_STAGES = 4;
+constexpr int QK_MAX_STAGES = 8;
+constexpr int QK_RING = 6 * 32768;              // bytes: six stages of the widest tile
 constexpr int QK_BK = 64;                       // k-block: 64 bf16 = one 128-byte swizzle row
-constexpr int QK_TILE = 128 * QK_BK * 2;        // bytes of the X tile (128 rows); the W tile (256 rows) is twice that
-constexpr int QK_STAGE = 3 * QK_TILE;
-constexpr int QK_THREADS = 192;                 // warp 0: TMA, warp 1: MMA issue + TMEM, warps 2-5: epilogue
-
-// Out of line: the rare fp64 path of the look-up would otherwise be copied into every unrolled pair.
-__device__ __noinline__ float2 rope_cs_call(const float2* tab, int pair, long long c, double theta) {
-    return svlm_rope_cs(tab, 64, pair, c, theta);
-}
-
-// The table look-up without the fp64 path: |c| < 2^24 (see svlm_rope.cuh).
-__device__ __forceinline__ float2 rope_cs_fast(const float2* __restrict__ tab, int pair, int c) {
-    const unsigned u = (unsigned)(c < 0 ? -c : c);
-    float2 r = __ldg(tab + (size_t)(u & 255u) * 64 + pair);
-    if (u >> 8) {
-        r = svlm_cmul(r, __ldg(tab + (size_t)(256 + ((u >> 8) & 255u)) * 64 + pair));
-        if (u >> 16) r = svlm_cmul(r, __ldg(tab + (size_t)(512 + (u >> 16)) * 64 + pair));
-    }
-    if (c < 0) r.y = -r.y;
-    return r;
-}
+constexpr int QK_W_TILE = 128 * QK_BK * 2;      // bytes of this CTA's rows of W in a stage
+constexpr int QK_EPI_WARPS = 8;
+constexpr int QK_THREADS = 96 + 32 * QK_EPI_WARPS;   // two producers, the issuer, the epilogue
+constexpr int QK_EPI_ROW = 128 + 4;             // floats between the transposed rows (16-byte aligned, conflict-free)
+static_assert(256 * QK_EPI_ROW * 4 <= QK_RING, "the transposed tile lives in the ring");
 
 struct QkShared {
-    unsigned long long full[QK_STAGES], empty[QK_STAGES], acc_full;
+    unsigned long long full[QK_MAX_STAGES], empty[QK_MAX_STAGES], acc_full;
     unsigned tmem_base;
     int abort_flag;
 };
 
+// ---- the paired forms (cta_group::2) ---------------------------------------------------------------------------
+// A tile into this CTA's shared memory; the bytes are counted on `bar`, an address of the pair's leading CTA.
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, int x, int y, unsigned bar) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+// D (both CTAs' tensor memory) (+)= A B, operands in both CTAs' shared memory at the same addresses
+__device__ __forceinline__ void tc_mma_ss_pair(unsigned d_tmem, unsigned long long a_desc, unsigned long long b_desc, unsigned idesc,
+                                               unsigned accumulate) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
+                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// Arrives on this barrier of both CTAs when the MMAs issued so far have completed.
+__device__ __forceinline__ void tc_commit_pair(void* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
+}
+
 // kv_heads_used = cd.kv_heads for the projection with append; 0 turns the kernel into the plain projection
 // Y = X W^T (the output projection after attention): every 128-column block is then a "query head" and goes to Q_out.
+// Grid: (2 * pairs of heads, token tiles of `width`), clusters of two.
 __global__ void __launch_bounds__(QK_THREADS, 1)
-qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, SvlmCacheDev cd,
-                  int layer, int n, int hidden, int q_heads, int kv_heads_used, uint16_t* __restrict__ Q_out) {
+qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ SvlmCacheDev cd,
+                  int layer, int n, int hidden, int q_heads, int kv_heads_used, int width, uint16_t* __restrict__ Q_out) {
     constexpr int D = 128, HALF = 64;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* ring = smem_raw;                                      // [stage][X tile | W tile]
-    QkShared& sh = *reinterpret_cast<QkShared*>(ring + QK_STAGES * QK_STAGE);
+    unsigned char* ring = smem_raw;                                      // [stage][W tile | half of the X tile]
+    QkShared& sh = *reinterpret_cast<QkShared*>(ring + QK_RING);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int head0 = 2 * blockIdx.x;            // the tile's two heads, in the order query heads, key heads, value heads
+    const unsigned rank = cluster_rank();
+    const int head = blockIdx.x;                 // this CTA's head, in the order query heads, key heads, value heads
     const int n_heads = q_heads + 2 * kv_heads_used;
-    const int m0 = blockIdx.y * 128;             // first token of the tile
+    const int i0 = blockIdx.y * width;           // first token of the tile
     const int n_kb = hidden / QK_BK;
+    const int stage_bytes = QK_W_TILE + width / 2 * 128;
+    const int n_stages = min(QK_MAX_STAGES, QK_RING / stage_bytes);
     volatile int* abort_flag = &sh.abort_flag;
-    const unsigned wait_limit = cd.ctrl->wait_limit;   // written at creation only, never by a kernel
+    const unsigned wait_limit = __ldcg(&cd.ctrl->wait_limit);   // written at creation only, never by a kernel
 
     if (smem_u32(smem_raw) & 1023) {             // swizzled tiles need a 1024-byte aligned base; same in every CTA
         if (threadIdx.x == 0) atomicCAS(&cd.ctrl->status, 0, -4);   // SVLM_ERR_CUDA
         return;
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < QK_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
+        for (int s = 0; s < QK_MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
         mbar_init(&sh.acc_full, 1);
         sh.abort_flag = 0;
         mbar_init_fence();
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "r"(256));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "r"(256));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
     }
+    // Set up while the predecessor ends (programmatic dependent launch); the wait comes before the trigger.
+    pdl_wait();
+    pdl_launch_dependents();
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();                          // both CTAs' barriers are initialised
     tc_fence_after();
     const unsigned tmem = sh.tmem_base;
 
-    if (warp == 0) {
-        // ================= TMA producer =================
+    if (warp == 0 || warp == 2 + QK_EPI_WARPS) {
+        // ================= TMA producers, a k-block each in turn =================
+        // (this loop and the issuer's are paced by their own instructions, one dependent after the other: stage numbers
+        // and phases are counted, not divided out, and addresses advance with them)
         if (lane == 0) {
-            for (int kb = 0; kb < n_kb; ++kb) {
-                const int st = kb % QK_STAGES;
-                if (!mbar_wait(&sh.empty[st], ((kb / QK_STAGES) & 1) ^ 1, abort_flag, wait_limit)) break;   // first pass: already free
-                unsigned char* dst = ring + st * QK_STAGE;
-                mbar_expect_tx(&sh.full[st], QK_STAGE);
-                tma_load_2d(dst, &tmX, kb * QK_BK, m0, &sh.full[st]);                 // rows past the end read as zeros
-                tma_load_2d(dst + QK_TILE, &tmW, kb * QK_BK, head0 * D, &sh.full[st]);
+            const int first = warp ? 1 : 0, y = i0 + (int)rank * (width / 2);
+            unsigned bar = map_to_rank(&sh.full[first], 0);
+            int st = first;
+            unsigned phase = 1;                                  // first pass: already free
+            unsigned char* dst = ring + first * stage_bytes;
+            for (int kb = first, x = first * QK_BK; kb < n_kb; kb += 2, x += 2 * QK_BK) {
+                if (!mbar_wait(&sh.empty[st], phase, abort_flag, wait_limit)) break;
+                if (rank == 0) mbar_expect_tx(&sh.full[st], 2 * stage_bytes);
+                tma_load_2d_pair(dst, &tmW, x, head * D, bar);   // rows past the end read as zeros
+                tma_load_2d_pair(dst + QK_W_TILE, &tmX, x, y, bar);
+                dst += 2 * stage_bytes;
+                bar += 16;
+                if ((st += 2) >= n_stages) { st -= n_stages; phase ^= 1; dst -= n_stages * stage_bytes; bar -= 8 * n_stages; }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ================= MMA issuer =================
-        if (lane == 0) {
-            constexpr unsigned IDESC = make_idesc(128, 256, 0);
+        // ================= MMA issuer (leading CTA) =================
+        // The whole warp runs the loop, so that descriptors live in uniform registers; one elected lane executes the
+        // tcgen05 instructions.
+        if (rank == 0) {
+            const bool leader = elect_one();
+            const unsigned idesc = make_idesc(256, 0, 0) | ((unsigned)(width >> 3) << 17);
+            const unsigned td = __shfl_sync(0xffffffffu, tmem, 0);
+            unsigned long long da = smem_desc(smem_u32(ring), 16, 1024), db = smem_desc(smem_u32(ring + QK_W_TILE), 16, 1024);
+            const unsigned step = (unsigned)stage_bytes >> 4;
+            int st = 0;
+            unsigned phase = 0;
             bool ok = true;
-            for (int kb = 0; kb < n_kb && ok; ++kb) {
-                const int st = kb % QK_STAGES;
-                ok = mbar_wait(&sh.full[st], (kb / QK_STAGES) & 1, abort_flag, wait_limit);
-                if (!ok) break;
+            for (int kb = 0; kb < n_kb; ++kb) {
+                ok = mbar_wait(&sh.full[st], phase, abort_flag, wait_limit);
+                if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
                 tc_fence_after();
-                const unsigned long long da = smem_desc(smem_u32(ring + st * QK_STAGE), 16, 1024);
-                const unsigned long long db = smem_desc(smem_u32(ring + st * QK_STAGE + QK_TILE), 16, 1024);
+                if (leader) {
 #pragma unroll
-                for (int ks = 0; ks < QK_BK / 16; ++ks)
-                    tc_mma_ss(tmem, da + (unsigned)(ks * 32 >> 4), db + (unsigned)(ks * 32 >> 4), IDESC, (kb | ks) != 0);
-                tc_commit(&sh.empty[st]);
+                    for (int ks = 0; ks < QK_BK / 16; ++ks)
+                        tc_mma_ss_pair(td, da + (unsigned)(ks * 32 >> 4), db + (unsigned)(ks * 32 >> 4), idesc, (kb | ks) != 0);
+                    tc_commit_pair(&sh.empty[st]);
+                }
+                __syncwarp();
+                da += step;
+                db += step;
+                if (++st == n_stages) { st = 0; phase ^= 1; da -= (unsigned long long)step * n_stages; db -= (unsigned long long)step * n_stages; }
             }
-            if (ok) tc_commit(&sh.acc_full);
+            if (ok && leader) tc_commit_pair(&sh.acc_full);
         }
         __syncwarp();
     } else {
-        // ================= epilogue: one thread per token of the tile =================
-        const int quad = warp & 3;                               // the TMEM lane quadrant this warp may read
-        const int row = quad * 32 + lane;
-        const int i = m0 + row;
-        // where the token lives (key and value heads): the append's slot, if the append stood
-        int slot = -1;
-        if (head0 + 1 >= q_heads && i < n && cd.ctrl->append_n == n) {
-            const int s = cd.new_slot[i];
-            if (cd.slot_gid[s] == cd.ctrl->n_total - n + i) slot = s;
-        }
-        // A tile with key heads: the token's 64 rotation factors are looked up into registers now, while the
-        // tensor pipe is still busy with the tile (64 dependent-latency look-ups after it took longer than the GEMM).
-        const float2* tab = reinterpret_cast<const float2*>(cd.rope_tab);
-        float2 cs[HALF];
-        bool have_cs = false;
-        int cpos[3] = {0, 0, 0};
-        if (slot >= 0 && head0 < q_heads + kv_heads_used) {
-            cpos[0] = cd.slot_c[slot]; cpos[1] = cd.slot_c[cd.n_slots + slot]; cpos[2] = cd.slot_c[2 * cd.n_slots + slot];
-            const int lim = 1 << 24;
-            have_cs = cpos[0] > -lim && cpos[0] < lim && cpos[1] > -lim && cpos[1] < lim && cpos[2] > -lim && cpos[2] < lim;
-            if (have_cs) {
-#pragma unroll
-                for (int pair = 0; pair < HALF; ++pair) {
-                    const int axis = cd.rope_mode == 0 ? 0 : (pair < cd.sec_t ? 0 : (pair < cd.sec_th ? 1 : 2));
-                    cs[pair] = rope_cs_fast(tab, pair, axis == 0 ? cpos[0] : (axis == 1 ? cpos[1] : cpos[2]));
+        // ================= epilogue: this CTA's head, `width` tokens =================
+        const int ew = warp - 2, quad = warp & 3;                // quad: the TMEM lane quadrant this warp may read
+        const int kv = head - q_heads;                           // < 0: query head; < kv_heads: key head; else value head
+        const bool key = kv >= 0 && kv < kv_heads_used;
+        // where this warp's tokens (ew, ew + 8, ...; one per lane) live, and their positions, if the append stood
+        int slot = -1, c0 = 0, c1 = 0, c2 = 0;
+        if (kv >= 0 && head < n_heads) {
+            const int t = ew + QK_EPI_WARPS * lane, i = i0 + t;
+            if (t < width && i < n && __ldcg(&cd.ctrl->append_n) == n) {
+                const int s = __ldcg(cd.new_slot + i);
+                if (__ldcg(cd.slot_gid + s) == __ldcg(&cd.ctrl->n_total) - n + i) slot = s;
+                if (key) {
+                    c0 = __ldcg(cd.slot_c + s);
+                    c1 = __ldcg(cd.slot_c + cd.n_slots + s);
+                    c2 = __ldcg(cd.slot_c + 2 * (size_t)cd.n_slots + s);
                 }
             }
         }
-        const bool ok = mbar_wait(&sh.acc_full, 0, abort_flag, wait_limit);
+        bool ok = mbar_wait(&sh.acc_full, 0, abort_flag, wait_limit);
+        ok = __all_sync(0xffffffffu, ok);
         tc_fence_after();
-#pragma unroll 1
-        for (int hh = 0; hh < 2 && ok; ++hh) {
-            const int head = head0 + hh;
-            if (head >= n_heads) break;                          // odd head count: the last tile is half empty
-            const unsigned tacc = tmem + ((unsigned)(quad * 32) << 16) + hh * D;
-            const int kv = head - q_heads;                       // < 0: query head; < kv_heads: key head; else value head
-            if (kv >= 0 && kv < cd.kv_heads) {
-                // key: pairs (j, j + 64), rotated at the slot's current position, 32 pairs at a time
-                uint16_t* dst = cd.K + (((size_t)layer * cd.kv_heads + kv) * cd.n_slots + (slot >= 0 ? slot : 0)) * D;
+        if (ok) {
+            float* tr = reinterpret_cast<float*>(ring) + quad * 32 + lane;
+            const unsigned tacc = tmem + ((unsigned)(quad * 32) << 16);
+            for (int c32 = ew >> 2; c32 < width / 32; c32 += 2) {
+                float v[32];
+                tmem_ld32(tacc + c32 * 32, v);
+                tmem_wait_ld();
 #pragma unroll
-                for (int c32 = 0; c32 < 2; ++c32) {
-                    float lo[32], hi[32];
-                    tmem_ld32(tacc + c32 * 32, lo);
-                    tmem_ld32(tacc + HALF + c32 * 32, hi);
-                    tmem_wait_ld();
-                    if (slot >= 0) {
-#pragma unroll
-                        for (int k = 0; k < 32; ++k) {
-                            const int pair = c32 * 32 + k;
-                            float2 f;
-                            if (have_cs) {
-                                f = cs[pair];
-                            } else {   // a position beyond the table's range (native positions of a very long stream)
-                                const int axis = cd.rope_mode == 0 ? 0 : (pair < cd.sec_t ? 0 : (pair < cd.sec_th ? 1 : 2));
-                                f = rope_cs_call(tab, pair, axis == 0 ? cpos[0] : (axis == 1 ? cpos[1] : cpos[2]), cd.theta[pair]);
-                            }
-                            const float x = lo[k], y = hi[k];
-                            lo[k] = x * f.x - y * f.y;
-                            hi[k] = y * f.x + x * f.y;
-                        }
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            *reinterpret_cast<uint4*>(dst + c32 * 32 + 8 * k) =
-                                make_uint4(pack2(lo[8 * k], lo[8 * k + 1]), pack2(lo[8 * k + 2], lo[8 * k + 3]),
-                                           pack2(lo[8 * k + 4], lo[8 * k + 5]), pack2(lo[8 * k + 6], lo[8 * k + 7]));
-                            *reinterpret_cast<uint4*>(dst + HALF + c32 * 32 + 8 * k) =
-                                make_uint4(pack2(hi[8 * k], hi[8 * k + 1]), pack2(hi[8 * k + 2], hi[8 * k + 3]),
-                                           pack2(hi[8 * k + 4], hi[8 * k + 5]), pack2(hi[8 * k + 6], hi[8 * k + 7]));
-                        }
+                for (int k = 0; k < 32; ++k) tr[(c32 * 32 + k) * QK_EPI_ROW] = v[k];
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * QK_EPI_WARPS) : "memory");
+        if (ok && head < n_heads) {
+            const int here = min(width, n - i0);                 // tokens of the tile
+            if (key) {
+                const float2* tab = reinterpret_cast<const float2*>(cd.rope_tab);
+                const int a0 = cd.rope_mode == 0 ? 0 : (2 * lane < cd.sec_t ? 0 : (2 * lane < cd.sec_th ? 1 : 2));
+                const int a1 = cd.rope_mode == 0 ? 0 : (2 * lane + 1 < cd.sec_t ? 0 : (2 * lane + 1 < cd.sec_th ? 1 : 2));
+#pragma unroll 4
+                for (int j = 0; j < 32; ++j) {
+                    const int t = ew + QK_EPI_WARPS * j;
+                    if (t >= here) break;
+                    const float* row = reinterpret_cast<const float*>(ring) + t * QK_EPI_ROW;
+                    const int s = __shfl_sync(0xffffffffu, slot, j);
+                    // pairs (2 lane, 2 lane + 1) with their partners 64 further on, rotated at the slot's current position
+                    const int p0 = __shfl_sync(0xffffffffu, c0, j), p1 = __shfl_sync(0xffffffffu, c1, j), p2 = __shfl_sync(0xffffffffu, c2, j);
+                    if (s < 0) continue;
+                    const int x0 = a0 == 0 ? p0 : (a0 == 1 ? p1 : p2), x1 = a1 == 0 ? p0 : (a1 == 1 ? p1 : p2);
+                    float2 f0 = svlm_rope_cs_batched(tab, HALF, 2 * lane, x0), f1 = svlm_rope_cs_batched(tab, HALF, 2 * lane + 1, x1);
+                    const int lim = 1 << 16;
+                    if (p0 <= -lim || p0 >= lim || p1 <= -lim || p1 >= lim || p2 <= -lim || p2 >= lim) {   // native positions of a long stream
+                        f0 = svlm_rope_cs(tab, HALF, 2 * lane, x0, cd.theta[2 * lane]);
+                        f1 = svlm_rope_cs(tab, HALF, 2 * lane + 1, x1, cd.theta[2 * lane + 1]);
                     }
+                    const float2 x = *reinterpret_cast<const float2*>(row + 2 * lane), y = *reinterpret_cast<const float2*>(row + HALF + 2 * lane);
+                    uint16_t* dst = cd.K + (((size_t)layer * cd.kv_heads + kv) * cd.n_slots + s) * D + 2 * lane;
+                    *reinterpret_cast<unsigned*>(dst) = pack2(x.x * f0.x - y.x * f0.y, x.y * f1.x - y.y * f1.y);
+                    *reinterpret_cast<unsigned*>(dst + HALF) = pack2(y.x * f0.x + x.x * f0.y, y.y * f1.x + x.y * f1.y);
                 }
             } else {
-                // query head -> the caller's buffer; value head -> the cache slot: a plain bf16 copy of the row
-                uint16_t* dst = nullptr;
-                if (kv < 0) { if (i < n) dst = Q_out + ((size_t)i * q_heads + head) * D; }
-                else if (slot >= 0) dst = cd.V + (((size_t)layer * cd.kv_heads + (kv - cd.kv_heads)) * cd.n_slots + slot) * D;
-#pragma unroll 1
-                for (int c32 = 0; c32 < 4; ++c32) {
-                    float v[32];
-                    tmem_ld32(tacc + c32 * 32, v);
-                    tmem_wait_ld();
-                    if (dst) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            *reinterpret_cast<uint4*>(dst + c32 * 32 + 8 * k) =
-                                make_uint4(pack2(v[8 * k], v[8 * k + 1]), pack2(v[8 * k + 2], v[8 * k + 3]),
-                                           pack2(v[8 * k + 4], v[8 * k + 5]), pack2(v[8 * k + 6], v[8 * k + 7]));
-                    }
+                // query head -> the caller's buffer; value head -> the cache slot: a plain bf16 copy of the row, two rows
+                // at a time (half a warp each)
+                const int sub = lane >> 4, e = (lane & 15) * 8;
+                uint16_t* q_base = Q_out + ((size_t)i0 * q_heads + head) * D + e;
+                uint16_t* v_base = cd.V + ((size_t)layer * cd.kv_heads + (kv - kv_heads_used)) * cd.n_slots * D + e;
+#pragma unroll 4
+                for (int j = 0; j < 32; j += 2) {
+                    const int t = ew + QK_EPI_WARPS * (j + sub);
+                    if (ew + QK_EPI_WARPS * j >= here) break;
+                    const int s = __shfl_sync(0xffffffffu, slot, j + sub);
+                    if (t >= here || (kv >= 0 && s < 0)) continue;
+                    const float* row = reinterpret_cast<const float*>(ring) + t * QK_EPI_ROW + e;
+                    const float4 x = *reinterpret_cast<const float4*>(row), y = *reinterpret_cast<const float4*>(row + 4);
+                    uint16_t* dst = kv < 0 ? q_base + (size_t)t * q_heads * D : v_base + (size_t)s * D;
+                    *reinterpret_cast<uint4*>(dst) = make_uint4(pack2(x.x, x.y), pack2(x.z, x.w), pack2(y.x, y.y), pack2(y.z, y.w));
                 }
             }
         }
@@ -222,33 +254,45 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     // ---- teardown ------------------------------------------------------------------------------
     tc_fence_before();
     __syncthreads();
-    if (sh.abort_flag) {
-        if (threadIdx.x == 0) {   // copies already issued still land here: give every stage a bounded chance to complete
-            for (int s = 0; s < QK_STAGES; ++s)
-                for (unsigned p = 0; p < 2; ++p)
-                    for (unsigned w = 0; w < (1u << 16) && !mbar_test(&sh.full[s], p); ++w) __nanosleep(32);
-            atomicCAS(&cd.ctrl->status, 0, -5);   // SVLM_ERR_TIMEOUT
-        }
-        __syncthreads();
+    if (sh.abort_flag && threadIdx.x == 0) {   // copies already issued still land here: give every stage a bounded chance to complete
+        for (int s = 0; s < QK_MAX_STAGES; ++s)
+            for (unsigned p = 0; p < 2; ++p)
+                for (unsigned w = 0; w < (1u << 16) && !mbar_test(&sh.full[s], p); ++w) __nanosleep(32);
+        atomicCAS(&cd.ctrl->status, 0, -5);   // SVLM_ERR_TIMEOUT
     }
+    __syncthreads();
+    cluster_sync_all();                          // neither CTA's memory is read or signalled by the other's work any more
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
     }
 }
 
-constexpr size_t qkv_smem() { return (size_t)QK_STAGES * QK_STAGE + sizeof(QkShared); }
+constexpr size_t qkv_smem() { return (size_t)QK_RING + sizeof(QkShared); }
 
 }  // namespace
 
+// Tokens per tile: the width at which the rounds of SM pairs, each as long as its math (2 N cycles per k-block, or the 320
+// that the issuer needs) and 14,000 cycles for filling the pipe and the epilogue, end first.
+int svlm_proj_tile(int n, int hidden, int blocks128) {
+    const int pairs_sm = std::max(1, svlm_sm_count() / 2), tiles_m = (blocks128 + 1) / 2;
+    int best = 256;
+    long long best_cost = -1;
+    for (int w = 32; w <= 256; w += 32) {
+        const long long tiles = (long long)tiles_m * ((n + w - 1) / w);
+        const long long rounds = (tiles + pairs_sm - 1) / pairs_sm;
+        const long long cost = rounds * ((long long)std::max(2 * w, 320) * (hidden / QK_BK) + 14000);
+        if (best_cost < 0 || cost <= best_cost) { best_cost = cost; best = w; }
+    }
+    return best;
+}
+
 cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmCacheDev& cd, int layer, int n, int hidden,
-                                   int q_heads, bool with_append, void* Q_out, cudaStream_t st) {
+                                   int q_heads, bool with_append, int width, void* Q_out, cudaStream_t st) {
     cudaError_t e = svlm_allow_smem<qkv_append_kernel>(qkv_smem());
     if (e != cudaSuccess) return e;
     const int kv = with_append ? cd.kv_heads : 0;
-    const dim3 grid((q_heads + 2 * kv + 1) / 2, (n + 127) / 128);
-    qkv_append_kernel<<<grid, QK_THREADS, qkv_smem(), st>>>(*static_cast<const CUtensorMap*>(tmX), *static_cast<const CUtensorMap*>(tmW),
-                                                             cd, layer, n, hidden, q_heads, kv, static_cast<uint16_t*>(Q_out));
-    svlm_count_launch();
-    return cudaGetLastError();
+    const dim3 grid((q_heads + 2 * kv + 1) / 2 * 2, (n + width - 1) / width);
+    return svlm_launch_chained(qkv_append_kernel, grid, dim3(QK_THREADS), qkv_smem(), 2, st, *static_cast<const CUtensorMap*>(tmX),
+                               *static_cast<const CUtensorMap*>(tmW), cd, layer, n, hidden, q_heads, kv, width, static_cast<uint16_t*>(Q_out));
 }

@@ -459,8 +459,9 @@ int svlm_qkv_append(svlm_cache* c, int layer, const void* X, const void* W, int 
     static const EncodeTiledFn encode = tensor_map_encoder();
     if (!encode) return SVLM_ERR_CUDA;
     alignas(64) CUtensorMap tmX, tmW;
-    if (!encode_matrix_map(encode, &tmX, X, n, hidden, 128) ||
-        !encode_matrix_map(encode, &tmW, W, (long long)(q_heads + 2 * c->dev.kv_heads) * 128, hidden, 256))
+    const int width = svlm_proj_tile(n, hidden, q_heads + 2 * c->dev.kv_heads);
+    if (!encode_matrix_map(encode, &tmX, X, n, hidden, width / 2) ||
+        !encode_matrix_map(encode, &tmW, W, (long long)(q_heads + 2 * c->dev.kv_heads) * 128, hidden, 128))
         return SVLM_ERR_CUDA;
     c->last_decode_layer = -1;
     if (layer == 0) {
@@ -472,7 +473,7 @@ int svlm_qkv_append(svlm_cache* c, int layer, const void* X, const void* W, int 
     } else if (n != c->pending_n) {
         return SVLM_ERR_ORDER;
     }
-    SVLM_CUDA(svlm_launch_qkv_append(&tmX, &tmW, c->dev, layer, n, hidden, q_heads, true, Q_out, c->stream));
+    SVLM_CUDA(svlm_launch_qkv_append(&tmX, &tmW, c->dev, layer, n, hidden, q_heads, true, width, Q_out, c->stream));
     return SVLM_OK;
 }
 
@@ -491,9 +492,10 @@ int svlm_out_proj(svlm_cache* c, const void* A, const void* Wo, int in_dim, int 
     static const EncodeTiledFn encode = tensor_map_encoder();
     if (!encode) return SVLM_ERR_CUDA;
     alignas(64) CUtensorMap tmA, tmW;
-    if (!encode_matrix_map(encode, &tmA, A, n, in_dim, 128) || !encode_matrix_map(encode, &tmW, Wo, out_dim, in_dim, 256))
+    const int width = svlm_proj_tile(n, in_dim, out_dim / 128);
+    if (!encode_matrix_map(encode, &tmA, A, n, in_dim, width / 2) || !encode_matrix_map(encode, &tmW, Wo, out_dim, in_dim, 128))
         return SVLM_ERR_CUDA;
-    SVLM_CUDA(svlm_launch_qkv_append(&tmA, &tmW, c->dev, 0, n, in_dim, out_dim / 128, false, Y, c->stream));
+    SVLM_CUDA(svlm_launch_qkv_append(&tmA, &tmW, c->dev, 0, n, in_dim, out_dim / 128, false, width, Y, c->stream));
     return SVLM_OK;
 }
 
