@@ -31,6 +31,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "svlm_dev.h"
@@ -852,7 +853,7 @@ template <int D>
 __global__ void __launch_bounds__(LAY_THREADS, 2)
 decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q, const int* __restrict__ q_pos, int q_heads,
                     uint16_t* __restrict__ out, int splits, const uint16_t* __restrict__ Knew,
-                    const uint16_t* __restrict__ Vnew, int early_loads, unsigned char* __restrict__ records TRACE_PARAM) {
+                    const uint16_t* __restrict__ Vnew, int early_loads TRACE_PARAM) {
     if (threadIdx.x == 0) STAMP(0);                  // kernel entry
     constexpr int CH = D / 8;                        // 16-byte chunks per row
     constexpr int ITEM_BYTES = UNIT * D * 2;         // K or V of one unit
@@ -867,8 +868,11 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int split = blockIdx.x, hk = blockIdx.y;
-    const SvlmAttendView& vw = b.view[0];
+    const int ci = blockIdx.z;                       // cache (one layer of each)
+    const SvlmAttendView& vw = b.view[ci];
+    unsigned char* const records = vw.tagged;
     const int G = q_heads / b.kv_heads;
+    const size_t q_head0 = (size_t)ci * q_heads + hk * G, kv_head = (size_t)ci * b.kv_heads + hk;   // rows of Q and out, of Knew and Vnew
 
     // The metadata was written by an earlier kernel in the stream.  When the launcher vouches that
     // the kernel directly before this one did not write it (early_loads), it is read at once;
@@ -885,7 +889,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     if (early_loads && warp == DEC_CWARPS - 1 && lane < 3) {
         // Bring the call's own small inputs towards L2 while the previous kernel still runs (a hint:
         // they are read for real only after the grid-dependency wait).
-        const size_t qoff = (size_t)hk * G * D, koff = (size_t)hk * D;
+        const size_t qoff = q_head0 * D, koff = kv_head * D;
         const void* p = lane == 0 ? (const void*)(Q + qoff) : lane == 1 ? (const void*)(Knew ? Knew + koff : Q + qoff)
                                                                         : (const void*)(Vnew ? Vnew + koff : Q + qoff);
         const int bytes = lane == 0 ? G * D * 2 : D * 2;
@@ -1025,7 +1029,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
             const int pair = 2 * p2 + e;
             const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
             const long long c = new_slot >= 0 ? (long long)__ldcg(vw.slot_c + (size_t)axis * b.n_slots + new_slot)
-                                              : (long long)q_pos[b.rope_mode == 0 ? 0 : axis] - shift;
+                                              : (long long)q_pos[b.rope_mode == 0 ? ci : 3 * ci + axis] - shift;
             const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
             f[e] = svlm_rope_cs_batched(tab, HALF, pair, (int)c);
             if (__builtin_expect(c <= -65536 || c >= 65536, 0)) f[e] = svlm_rope_cs(tab, HALF, pair, c, b.theta[pair]);
@@ -1044,7 +1048,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
 #pragma unroll
         for (int k = 0; k < HN; ++k) {               // all loads first: one round trip
             const int h = threadIdx.x / LPH + k * HSTEP;
-            const uint16_t* row = Q + (size_t)(hk * G + (h < G ? h : 0)) * D + 2 * p2;   // n_q = 1
+            const uint16_t* row = Q + (q_head0 + (h < G ? h : 0)) * D + 2 * p2;   // n_q = 1
             lo[k] = *reinterpret_cast<const unsigned*>(row);
             hi[k] = *reinterpret_cast<const unsigned*>(row + HALF);
         }
@@ -1053,7 +1057,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
         const bool prep_new = new_slot >= 0 && threadIdx.x < LPH;
         unsigned klo = 0, khi = 0, vlo = 0, vhi = 0;
         if (prep_new) {
-            const size_t off = (size_t)hk * D + 2 * p2;
+            const size_t off = kv_head * D + 2 * p2;
             klo = *reinterpret_cast<const unsigned*>(Knew + off); khi = *reinterpret_cast<const unsigned*>(Knew + off + HALF);
             vlo = *reinterpret_cast<const unsigned*>(Vnew + off); vhi = *reinterpret_cast<const unsigned*>(Vnew + off + HALF);
         }
@@ -1248,7 +1252,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     auto stamp = [](int) {};
 #endif
     combine_tagged<D>(split, shares, splits, ws_parts, (unsigned)sh.tag, epoch, reinterpret_cast<float*>(ring), G,
-                      out + (size_t)hk * G * D, (unsigned)sh.wait_limit, const_cast<int*>(&vw.ctrl->status), stamp);
+                      out + q_head0 * D, (unsigned)sh.wait_limit, const_cast<int*>(&vw.ctrl->status), stamp);
 #ifdef SVLM_DECODE_TRACE
     __syncthreads();
     if (threadIdx.x == 0) { STAMP(11); STAMP(13); }   // output written; leaving
@@ -1277,8 +1281,15 @@ size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits) {
 
 // The per-layer kernel holds one round of a CTA's keys and values on chip before the query comes and the next in L2; with a
 // third round it is only a slower streaming kernel (16 query / 8 KV heads, 17,408 keys, 4 rounds: 19.4 us, streaming
-// 17.9; two rounds: 9.3 against 11.5).
-bool svlm_decode_streams(int pages, int splits) { return (8 * pages + splits - 1) / splits > 2 * GROUP; }
+// 17.9; two rounds: 9.3 against 11.5; two streams of 9,216 keys: 10.9 against 13.0, of 3,072: 7.7 against 11.3).  Its CTAs
+// wait for one another's partial results, so several caches take it only while all CTAs fit the SMs, one each, and while
+// a KV head has enough of them to share the combine (8 caches of 4 heads, 4 CTAs a head: 13.5 against 11.5).
+int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches) {
+    const int splits = std::min(148 / (kv_heads * n_caches), 4 * n_pages);
+    if (n_caches > 1 && splits < 12) return 0;
+    const int s = std::max(splits, 1);
+    return (8 * pages + s - 1) / s > 2 * GROUP ? 0 : s;
+}
 
 bool svlm_decode_supported(int n_pages) { return n_pages <= DEC_MAX_TILES; }
 
@@ -1294,11 +1305,11 @@ int svlm_decode_splits(int n_pages, int kv_heads, int problems) {
 
 cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
                                int q_heads, void* out, int splits, const void* Knew, const void* Vnew, int early_loads,
-                               void* tagged, cudaStream_t st) {
+                               bool tagged, cudaStream_t st) {
     const int problems = b.n_caches * n_layers;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(splits, b.kv_heads, problems);
-    cfg.blockDim = dim3(problems == 1 && tagged ? LAY_THREADS : DEC_THREADS);
+    cfg.blockDim = dim3(tagged ? LAY_THREADS : DEC_THREADS);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1310,7 +1321,7 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
     const uint16_t* Kn = (const uint16_t*)Knew;
     const uint16_t* Vn = (const uint16_t*)Vnew;
     cudaError_t e;
-    if (problems == 1 && tagged) {
+    if (tagged) {
 #ifdef SVLM_DECODE_TRACE
         int trace_idx = -1;
         if (g_decode_trace_next >= 0 && g_decode_trace_next < SVLM_TR_LAUNCHES && splits * b.kv_heads <= SVLM_TR_CTAS)
@@ -1321,13 +1332,13 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
             if (e != cudaSuccess) return e;
             cfg.dynamicSmemBytes = decode_layer_smem<128>();
             e = cudaLaunchKernelEx(&cfg, decode_layer_kernel<128>, b, layer0, Qp, q_pos, q_heads, Op, splits, Kn, Vn,
-                                   early_loads, (unsigned char*)tagged TRACE_ARG);
+                                   early_loads TRACE_ARG);
         } else {
             e = svlm_allow_smem<decode_layer_kernel<64>>(decode_layer_smem<64>());
             if (e != cudaSuccess) return e;
             cfg.dynamicSmemBytes = decode_layer_smem<64>();
             e = cudaLaunchKernelEx(&cfg, decode_layer_kernel<64>, b, layer0, Qp, q_pos, q_heads, Op, splits, Kn, Vn,
-                                   early_loads, (unsigned char*)tagged TRACE_ARG);
+                                   early_loads TRACE_ARG);
         }
     } else if (b.head_dim == 128) {
         e = svlm_allow_smem<decode_stream_kernel<128>>(decode_stream_smem<128>());

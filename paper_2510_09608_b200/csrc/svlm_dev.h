@@ -97,6 +97,7 @@ struct SvlmAttendView {      // what attention needs from one cache
     const void* tmaps;       // four 128-byte TMA descriptors in device memory (see SvlmCacheDev)
     const int* new_slot;     // slots of the latest append
     const int* slot_c;       // [3][n_slots] current positions
+    unsigned char* tagged;   // per-layer decode kernel: epochs and tagged records
 };
 
 struct SvlmAttendBatch {     // kernel parameter: up to 32 caches share one launch

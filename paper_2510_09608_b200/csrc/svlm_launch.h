@@ -89,14 +89,15 @@ bool svlm_decode_supported(int n_pages);
 // layers attended here, so the kernel may read them before the previous kernel has finished.
 // early_loads == 2: moreover that previous kernel was itself a decode step of this cache (the per-layer kernel then
 // paces its read-ahead, one unit's worth per warp at a time).
-// tagged: the cache's area of svlm_decode_tagged_bytes(kv_heads, head_dim, splits) bytes for a launch of one cache
-// and one layer (the per-layer kernel, whose splits hand their partial results over in tagged words); null, or
-// several problems in the launch: the streaming kernel with its arrival counters in the view's scratch.
+// tagged: the per-layer kernel (one layer of one or a few caches; its splits hand their partial results over in tagged
+// words in the views' areas of svlm_decode_tagged_bytes, sized for one cache's splits); otherwise the streaming kernel
+// with its arrival counters in the views' scratch.
 cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
                                int q_heads, void* out, int splits, const void* Knew, const void* Vnew, int early_loads,
-                               void* tagged, cudaStream_t st);
-// One problem with so many pages per CTA that the streaming kernel is the better one (either gives the same result).
-bool svlm_decode_streams(int pages, int splits);
+                               bool tagged, cudaStream_t st);
+// Splits of the per-layer kernel for one layer of n_caches caches with `pages` pages or fewer, 0 where the streaming kernel
+// is the better one (either gives the same result).
+int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches);
 size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits);
 
 // Q/K/V projection with the append as its epilogue, head_dim 128 (svlm_qkv_sm100.cu).  tmX, tmW: host copies of

@@ -103,6 +103,7 @@ void fill_view(const svlm_cache* c, SvlmAttendView& v) {
     v.tmaps = c->dev.tmaps;
     v.new_slot = c->dev.new_slot;
     v.slot_c = c->dev.slot_c;
+    v.tagged = c->decode_tagged;
 }
 
 // Rotation table: (cos, sin)(k * 256^level * theta_i) in fp32 from fp64 (see svlm_rope.cuh).  k = 16 a + b: the 16
@@ -274,8 +275,11 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     }
     if (n_q == 1 && group <= 8 && svlm_decode_supported(c0->dev.n_pages)) {
         // split-KV decode; every cache's scratch was sized for this launch shape at creation
-        const int splits = svlm_decode_splits(c0->dev.n_pages, c0->dev.kv_heads, n_caches * n_layers);
-        void* tagged = svlm_decode_streams(expected_pages(c0), splits) ? nullptr : c0->decode_tagged;
+        int pages = 1;
+        for (int i = 0; i < n_caches; ++i) pages = std::max(pages, expected_pages(caches[i]));
+        int splits = layer >= 0 ? svlm_decode_layer_splits(c0->dev.n_pages, pages, c0->dev.kv_heads, n_caches) : 0;
+        const bool tagged = splits > 0;
+        if (!tagged) splits = svlm_decode_splits(c0->dev.n_pages, c0->dev.kv_heads, n_caches * n_layers);
         SVLM_CUDA(svlm_launch_decode(b, layer0, n_layers, Q, q_pos, q_heads, out, splits, Knew, Vnew, early, tagged, c0->stream));
         return SVLM_OK;
     }
