@@ -60,10 +60,10 @@ inline int svlm_sm_count() {
 // metadata (svlm_meta.cu)
 void svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n, cudaStream_t st);
 void svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st);
-// batched forms, one block per cache: types [n_caches][n], pos [n_caches][n](x3)
-void svlm_launch_append_meta_batch(const SvlmCacheList& list, const unsigned char* types, const int* pos, int n,
+// batched forms, one block per cache: types [n_caches][n], pos [n_caches][n](x3); every cache has the geometry of geom
+void svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, const unsigned char* types, const int* pos, int n,
                                    cudaStream_t st);
-void svlm_launch_evict_meta_batch(const SvlmCacheList& list, cudaStream_t st);
+void svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
 
 // key/value movement (svlm_kv.cu)
 // layer < 0: K,V are [layers][n][kv_heads][d]; otherwise [n][kv_heads][d] for that layer.

@@ -526,7 +526,7 @@ int svlm_cache_evict_batched(svlm_cache* const* caches, int n_caches) {
         note_evict(caches[i]);
         rotate = rotate || caches[i]->dev.contiguous;   // a cache with native positions never sets evict_moved
     }
-    svlm_launch_evict_meta_batch(list, c0->stream);
+    svlm_launch_evict_meta_batch(list, c0->dev, c0->stream);
     if (rotate) svlm_launch_evict_rotate_batch(list, c0->dev, c0->stream);
     SVLM_CUDA(cudaGetLastError());
     return SVLM_OK;
@@ -575,7 +575,7 @@ int svlm_decode_step_batched(svlm_cache* const* caches, int n_caches, int layer,
             c->last_decode_layer = -1;
             note_append(c, 1);
         }
-        svlm_launch_append_meta_batch(list, token_type, pos, 1, c0->stream);
+        svlm_launch_append_meta_batch(list, c0->dev, token_type, pos, 1, c0->stream);
     } else {
         for (int i = 0; i < n_caches; ++i)
             if (caches[i]->pending_n != 1) return SVLM_ERR_ORDER;
