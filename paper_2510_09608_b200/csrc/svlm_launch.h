@@ -116,10 +116,14 @@ cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int i
 // tcgen05/TMEM/TMA chunk prefill, n_q >= 2 (svlm_prefill_sm100.cu)
 bool svlm_prefill_supported(int n_pages, int group);
 // counters: svlm_prefill_counter_bytes of the first cache, zero before the first launch (the kernel leaves them zero);
-// slots: its svlm_prefill_slot_bytes (0: null).  Launches that share them must not overlap.  pages: how many pages each
-// cache is expected to hold (only the balance of the work depends on it).
+// slots: its svlm_prefill_slot_bytes (0: null).  Launches that share them must not overlap.  held: what each cache is
+// expected to hold (only the balance of the work depends on it).
+struct SvlmPrefillLoad {
+    int pages;      // stored pages
+    int windows;    // most tokens the windows keep, i.e. most of a chunk that can be stored
+};
 size_t svlm_prefill_slot_bytes(int n_pages, int head_dim);
 constexpr size_t svlm_prefill_counter_bytes = 4096;
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
-                                int n_q, int q_heads, void* out, const int* pages, void* counters, void* slots,
+                                int n_q, int q_heads, void* out, const SvlmPrefillLoad* held, void* counters, void* slots,
                                 cudaStream_t st);

@@ -38,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "svlm_dev.h"
 #include "svlm_launch.h"
@@ -56,7 +57,7 @@ constexpr int PF_MAX_TILES = 512;
 constexpr int PF_ROWS = 256;          // rows per unit
 constexpr int PF_MAX_CTAS = 160;
 constexpr int PF_MIN_PAGES = 6;       // pages a CTA should have at least when units are cut
-constexpr int PF_PIECE = 10;          // what beginning another unit costs, in pages (one stream: 3 and 6: 78 us, 10: 76, 16: 78)
+constexpr int PF_PIECE = 10;          // what beginning a unit costs, in pages (one stream: 3 and 6: 78 us, 10: 76, 16: 78)
 constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
 constexpr int PF_CS_BYTES = 16384;    // rotation factors of one tile's tokens (5 or more heads per KV head, all at head_dim 64 with 2 or more)
 // Registers per thread after the split; 216 * 256 + 72 * 128 = 168 * 384, what the block is launched with (checked at launch).
@@ -1033,16 +1034,20 @@ template <int D>
 constexpr size_t prefill_smem() { return (size_t)(2 + PF_RING) * 128 * D * 2 + 2 * PF_CS_BYTES + sizeof(PfShared); }
 
 // The work split of one launch (see the top of the file): whole units in rounds over the grid while at least two rounds
-// are left, the rest cut so that every CTA has the same number of expected pages.  pages: an estimate of every cache's
-// page count; a wrong one costs balance only.
-void make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, int G, const int* pages, int max_ctas, int& grid) {
+// are left, the rest cut so that every CTA ends at the same level.  Beginning a unit, or another piece of one, costs as
+// much as PF_PIECE pages.  The numbers of pages are estimates; a wrong one costs balance only.
+void make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, int G, const SvlmPrefillLoad* held, int max_ctas, int& grid) {
     plan.units = 0;
     long long all = 0;                                     // pages of the whole launch
     const int per_unit = n_layers * b.kv_heads;
     auto rows_of = [&](int i) { return b.q_varlen ? b.q_cnt[i] : n_q; };
     auto tiles_of = [&](int i) { return (rows_of(i) * G + PF_ROWS - 1) / PF_ROWS; };
-    // expected pages of row tile rt of cache i: the chunk's own pages behind its last row are invisible
-    auto cost = [&](int i, int rt) { return std::max(1, pages[i] - std::max(0, rows_of(i) - 1 - (rt * PF_ROWS + PF_ROWS - 1) / G) / SVLM_PAGE); };
+    // expected pages of row tile rt of cache i: what is stored of the chunk behind its last row is invisible (of a chunk
+    // longer than the windows little is stored)
+    auto cost = [&](int i, int rt) {
+        const int later = std::max(0, rows_of(i) - 1 - (rt * PF_ROWS + PF_ROWS - 1) / G);
+        return std::max(1, held[i].pages - std::min(later, held[i].windows) / SVLM_PAGE);
+    };
     for (int i = 0; i < b.n_caches; ++i) {
         plan.off[i] = plan.units;
         const int R = tiles_of(i);
@@ -1056,53 +1061,70 @@ void make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, in
     plan.rounds = std::max(0, U / grid - 1);
     plan.tail = plan.rounds * grid;
     const int nt = U - plan.tail;
-    if (!cut || grid == U || (grid < U && nt == grid && plan.rounds == 0)) {      // whole units only
+    if (!cut || grid == U) {                               // whole units only
         for (int i = 0; i <= grid; ++i) plan.x[i] = (unsigned short)((long long)i * nt / grid * PF_FRAC);
         return;
     }
-    // walk the units in order, first to add up what the whole rounds give each CTA, then to cut the tail
+    // walk the units in order: what the whole rounds give each CTA, then the tail's costs
     int ci = 0, rt = 0, R = tiles_of(0), left = R * per_unit;    // position of unit u
     auto step = [&] {
         if (++rt == R) rt = 0;
         if (--left == 0 && ci + 1 < b.n_caches) { ++ci; R = tiles_of(ci); left = R * per_unit; rt = 0; }
     };
-    int load[PF_MAX_CTAS] = {};
+    int load[PF_MAX_CTAS] = {}, tail_cost[2 * PF_MAX_CTAS], most = 0, dearest = 1;
     for (int u = 0, at = 0; u < plan.tail; ++u) {
-        load[at] += cost(ci, rt);
+        load[at] += cost(ci, rt) + PF_PIECE;
+        most = std::max(most, load[at]);
         if (++at == grid) at = 0;
         step();
     }
-    int tail_cost[2 * PF_MAX_CTAS];
-    for (int t = 0; t < nt; ++t) { tail_cost[t] = cost(ci, rt); step(); }
-    // The level at which every CTA ends, counting what beginning another unit costs: from below, raised by what a deal at
-    // that level leaves over.
-    double level = (double)all / grid;
-    for (int pass = 0; pass < 10; ++pass) {
+    for (int t = 0; t < nt; ++t) { tail_cost[t] = cost(ci, rt); dearest = std::max(dearest, tail_cost[t]); step(); }
+    // deals the tail out at a level; true when everything has found its place
+    auto deal = [&](double level) {
         int t = 0;
         double rem = tail_cost[0];
         for (int i = 0; i < grid; ++i) {
             plan.x[i] = (unsigned short)(t < nt ? t * PF_FRAC + (int)((tail_cost[t] - rem) / tail_cost[t] * PF_FRAC + 0.5) : nt * PF_FRAC);
             double room = level - load[i];
-            for (bool first = true; room > 0 && t < nt; first = false) {
-                if (!first && (room -= PF_PIECE) < PF_SNAP) break;
+            while (t < nt && (room -= PF_PIECE) >= std::min((double)PF_SNAP, rem)) {
                 double take = std::min(room, rem);
                 if (rem - take < PF_SNAP) take = rem;                // no slivers
                 room -= take;
                 rem -= take;
-                if (rem <= 0 && ++t < nt) rem = tail_cost[t];
+                if (rem > 0) break;
+                if (++t < nt) rem = tail_cost[t];
             }
         }
-        if (t >= nt) break;
-        double over = rem;
-        for (int k = t + 1; k < nt; ++k) over += tail_cost[k];
-        level += over / grid + 0.1;
+        return t >= nt;
+    };
+    // the lowest level that does, by bisection between the average and whole units for everybody
+    double lo = ((double)all + (double)PF_PIECE * U) / grid, hi = most + (double)((nt + grid - 1) / grid) * (dearest + PF_PIECE) + PF_SNAP;
+    for (int it = 0; it < 8 && hi - lo > 0.5; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        (deal(mid) ? hi : lo) = mid;
     }
-    plan.x[grid] = (unsigned short)(nt * PF_FRAC);                   // the last CTA takes what is left
+    deal(hi);
+    plan.x[grid] = (unsigned short)(nt * PF_FRAC);
 }
+
+// What a plan is made from; the layers of a chunk come one after another with the same numbers, so a thread keeps its
+// latest plan (making one takes microseconds).
+struct PfPlanKey {
+    int n_caches, kv_heads, n_layers, n_q, G, max_ctas, varlen;
+    int rows[SVLM_MAX_BATCH];
+    SvlmPrefillLoad held[SVLM_MAX_BATCH];
+    const void* counters;
+    const void* slots;
+};
+struct PfPlanMemo {
+    PfPlanKey key;
+    PfPlan plan;
+    int grid = 0;
+};
 
 template <int D>
 cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uint16_t* Q, const int* q_pos, int n_q,
-                   int q_heads, uint16_t* out, const int* pages, void* counters, void* slots, cudaStream_t st) {
+                   int q_heads, uint16_t* out, const SvlmPrefillLoad* held, void* counters, void* slots, cudaStream_t st) {
     cudaError_t e = svlm_allow_smem<prefill_kernel<D>>(prefill_smem<D>());
     if (e != cudaSuccess) return e;
     // the register split inside the kernel adds up only if the block is launched with exactly this many
@@ -1111,13 +1133,26 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
         return cudaFuncGetAttributes(&a, prefill_kernel<D>) == cudaSuccess && a.numRegs == PF_REGS_LAUNCH;
     }();
     if (!regs_ok) return cudaErrorLaunchOutOfResources;
-    PfPlan plan;
-    plan.counters = static_cast<unsigned*>(counters);
-    plan.slots = static_cast<unsigned char*>(slots);
     const int G = q_heads / b.kv_heads;
-    plan.g_magic = G > 1 && (unsigned long long)n_q * G * G < 0x100000000ull - 256ull * G ? (unsigned)((0x100000000ull + G - 1) / G) : 0u;   // (tiles reach past the last row)
-    int grid;
-    make_plan(plan, b, n_layers, n_q, G, pages, std::min(svlm_sm_count(), PF_MAX_CTAS), grid);
+    thread_local PfPlanMemo memo;
+    PfPlanKey key;
+    std::memset(&key, 0, sizeof key);
+    key.n_caches = b.n_caches; key.kv_heads = b.kv_heads; key.n_layers = n_layers; key.n_q = n_q; key.G = G;
+    key.max_ctas = std::min(svlm_sm_count(), PF_MAX_CTAS);
+    key.varlen = b.q_varlen;
+    for (int i = 0; i < b.n_caches; ++i) { key.rows[i] = b.q_varlen ? b.q_cnt[i] : n_q; key.held[i] = held[i]; }
+    key.counters = counters;
+    key.slots = slots;
+    if (memo.grid == 0 || std::memcmp(&memo.key, &key, sizeof key) != 0) {
+        PfPlan& plan = memo.plan;
+        plan.counters = static_cast<unsigned*>(counters);
+        plan.slots = static_cast<unsigned char*>(slots);
+        plan.g_magic = G > 1 && (unsigned long long)n_q * G * G < 0x100000000ull - 256ull * G ? (unsigned)((0x100000000ull + G - 1) / G) : 0u;   // (tiles reach past the last row)
+        make_plan(plan, b, n_layers, n_q, G, held, key.max_ctas, memo.grid);
+        memo.key = key;
+    }
+    const PfPlan& plan = memo.plan;
+    const int grid = memo.grid;
     return svlm_launch_chained(prefill_kernel<D>, dim3((unsigned)grid), dim3(PF_THREADS), prefill_smem<D>(), 1, st, b, plan, layer0, n_layers, Q, q_pos,
                                n_q, q_heads, out);
 }
@@ -1133,8 +1168,8 @@ size_t svlm_prefill_slot_bytes(int n_pages, int head_dim) {
 }
 
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
-                                int n_q, int q_heads, void* out, const int* pages, void* counters, void* slots, cudaStream_t st) {
+                                int n_q, int q_heads, void* out, const SvlmPrefillLoad* held, void* counters, void* slots, cudaStream_t st) {
     return b.head_dim == 128
-        ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, counters, slots, st)
-        : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, pages, counters, slots, st);
+        ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, held, counters, slots, st)
+        : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, held, counters, slots, st);
 }

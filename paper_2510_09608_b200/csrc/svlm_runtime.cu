@@ -230,6 +230,12 @@ void note_evict(svlm_cache* c) {
 }
 int expected_pages(const svlm_cache* c) { return std::max(1, (int)std::min<long long>(c->stored_est / SVLM_PAGE + 1, c->dev.n_pages)); }
 
+// Before an eviction all of a chunk is stored, afterwards no more than the windows hold.
+SvlmPrefillLoad expected_load(const svlm_cache* c) {
+    const long long keep = (long long)c->dev.vision_window + c->dev.text_window;
+    return {expected_pages(c), (int)std::min<long long>(c->stored_est > c->dev.n_sink + keep ? c->stored_est : keep, 1 << 30)};
+}
+
 int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void* Q, const int32_t* q_pos, int n_q,
                   int q_heads, void* out, const void* Knew = nullptr, const void* Vnew = nullptr) {
     svlm_cache* c0 = caches[0];
@@ -285,9 +291,9 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     }
     if (Knew) return SVLM_ERR_ARG;   // the fused step exists for the split-KV kernel only
     if (n_q >= 2 && svlm_prefill_supported(c0->dev.n_pages, group)) {
-        int pages[SVLM_MAX_BATCH];
-        for (int i = 0; i < n_caches; ++i) { pages[i] = expected_pages(caches[i]); caches[i]->meta_settled = true; }
-        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, pages, c0->prefill_counters, c0->prefill_slots, c0->stream));
+        SvlmPrefillLoad held[SVLM_MAX_BATCH];
+        for (int i = 0; i < n_caches; ++i) { held[i] = expected_load(caches[i]); caches[i]->meta_settled = true; }
+        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, held, c0->prefill_counters, c0->prefill_slots, c0->stream));
         return SVLM_OK;
     }
     svlm_launch_attend_simple(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, c0->stream);
@@ -609,9 +615,9 @@ int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int laye
     }
     if (off > 0x7fffffffll) return SVLM_ERR_ARG;
     DeviceGuard guard(c0->device);
-    int pages[SVLM_MAX_BATCH];
-    for (int i = 0; i < n_caches; ++i) { pages[i] = expected_pages(caches[i]); caches[i]->meta_settled = true; }
-    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, Q, q_pos, n_max, q_heads, out, pages, c0->prefill_counters, c0->prefill_slots, c0->stream));
+    SvlmPrefillLoad held[SVLM_MAX_BATCH];
+    for (int i = 0; i < n_caches; ++i) { held[i] = expected_load(caches[i]); caches[i]->meta_settled = true; }
+    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, Q, q_pos, n_max, q_heads, out, held, c0->prefill_counters, c0->prefill_slots, c0->stream));
     return SVLM_OK;
 }
 
