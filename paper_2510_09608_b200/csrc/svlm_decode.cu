@@ -964,6 +964,14 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     auto value_fragment = [&](int j, int db, unsigned (&a)[4]) {
         ldmatrix_x4_trans(a[0], a[1], a[2], a[3], sv[j] + lay_off((lm_i >> 1) * 8 + lm_r, db * 2 + (lm_i & 1)));
     };
+    // all rows of a round go towards L2
+    auto round_to_l2 = [&](int r) {
+        Units v;
+        get_units(r, v);
+#pragma unroll
+        for (int j = 0; j < UPW; ++j)
+            if (j < v.n) { rows_to_l2(Kh, v.row[j]); rows_to_l2(Vh, v.row[j]); }
+    };
     Units u;
     // Front of a round: the three key units and the first value unit are copied, the keys go on into fragment
     // registers, the other two value units follow into the key slots.  PACED: reading ahead of a previous decode step
@@ -1001,14 +1009,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
         // The units of a second round (many KV heads, large windows) come out of L2 then: ask for them now, while the
         // predecessor still runs and HBM would idle (8 KV heads of 9216 keys: 11.1 -> 10.1 us; asking for four rounds
         // at once is slower again).
-        if (early_loads)
-            for (int r = 1; r < min(n_rounds, 2); ++r) {
-                Units v;
-                get_units(r, v);
-#pragma unroll
-                for (int j = 0; j < UPW; ++j)
-                    if (j < v.n) { rows_to_l2(Kh, v.row[j]); rows_to_l2(Vh, v.row[j]); }
-            }
+        if (early_loads && n_rounds > 1) round_to_l2(1);
     }
     if (threadIdx.x == 0) STAMP(2);                  // the first round's keys are in registers
 
@@ -1280,15 +1281,19 @@ size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits) {
 }
 
 // The per-layer kernel holds one round of a CTA's keys and values on chip before the query comes and the next in L2; with a
-// third round it is only a slower streaming kernel (16 query / 8 KV heads, 17,408 keys, 4 rounds: 19.4 us, streaming
-// 17.9; two rounds: 9.3 against 11.5; two streams of 9,216 keys: 10.9 against 13.0, of 3,072: 7.7 against 11.3).  Its CTAs
-// wait for one another's partial results, so several caches take it only while all CTAs fit the SMs, one each, and while
-// a KV head has enough of them to share the combine (8 caches of 4 heads, 4 CTAs a head: 13.5 against 11.5).
-int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches) {
-    const int splits = std::min(148 / (kv_heads * n_caches), 4 * n_pages);
-    if (n_caches > 1 && splits < 12) return 0;
-    const int s = std::max(splits, 1);
-    return (8 * pages + s - 1) / s > 2 * GROUP ? 0 : s;
+// third round it is only a slower streaming kernel where a KV head has few CTAs (head size 128, us per layer-step: 8 heads
+// of 16,900 keys 22.9 against 20.5, with two rounds 10.1 against 11.8; 4 heads of 24,300 keys, whose 37 CTAs the streaming
+// kernel's last CTA combines alone, 17.1 against 18.2; head size 64, half the bytes, is better here at any length).
+// Two streams of 9,216 keys: 10.9 against 13.0, of 3,072: 7.7 against 11.3.  Its CTAs wait for one another's partial
+// results, so several caches take it only while all CTAs fit the SMs, one each, and while a KV head has enough of them to
+// share the combine (8 caches of 4 heads, 4 CTAs a head: 13.5 against 11.5; 3 caches, 12 CTAs a head: 8.9 against 10.3 with
+// one round, 13.7 against 12.7 with two).
+int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches, int head_dim) {
+    const int splits = std::max(1, std::min(148 / (kv_heads * n_caches), 4 * n_pages));
+    const int rounds = ((8 * pages + splits - 1) / splits + GROUP - 1) / GROUP;
+    if (n_caches == 1) return rounds > 2 && head_dim == 128 && splits < 24 ? 0 : splits;
+    if (splits < 12 || kv_heads * n_caches * splits > 148) return 0;
+    return rounds > (splits >= 16 ? 2 : 1) ? 0 : splits;
 }
 
 bool svlm_decode_supported(int n_pages) { return n_pages <= DEC_MAX_TILES; }

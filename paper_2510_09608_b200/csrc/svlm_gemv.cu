@@ -261,10 +261,11 @@ __global__ void __launch_bounds__(GV_THREADS) gemv_mma_kernel(const uint16_t* __
 
 bool svlm_gemv_supported(int n, int in_dim) { return n >= 1 && n <= 16 && in_dim % 32 == 0 && (size_t)4 * in_dim * 2 <= 200 * 1024; }
 
-cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, SvlmCtrl* ctrl, cudaStream_t st) {
+cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, bool from_l2, SvlmCtrl* ctrl, cudaStream_t st) {
     const uint16_t* x = static_cast<const uint16_t*>(X);
     const uint16_t* w = static_cast<const uint16_t*>(W);
     uint16_t* y = static_cast<uint16_t*>(Y);
-    if (few_supported(n, in_dim)) return launch_few(x, w, y, n, in_dim, out_dim, ctrl, st);
+    // weights that stay in L2 from token to token: fetching ahead buys nothing, and more, smaller blocks are 2 us faster
+    if (!from_l2 && few_supported(n, in_dim)) return launch_few(x, w, y, n, in_dim, out_dim, ctrl, st);
     return svlm_launch_chained(gemv_mma_kernel, dim3((out_dim + 7) / 8), dim3(GV_THREADS), 0, 1, st, x, w, y, n, in_dim, out_dim);
 }

@@ -97,7 +97,7 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
                                bool tagged, cudaStream_t st);
 // Splits of the per-layer kernel for one layer of n_caches caches with `pages` pages or fewer, 0 where the streaming kernel
 // is the better one (either gives the same result).
-int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches);
+int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches, int head_dim);
 size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits);
 
 // Q/K/V projection with the append as its epilogue, head_dim 128 (svlm_qkv_sm100.cu).  tmX, tmW: host copies of
@@ -110,8 +110,8 @@ cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmC
 
 // Y = X W^T for a few rows of X (decode-time projections), a bandwidth kernel (svlm_gemv.cu)
 bool svlm_gemv_supported(int n, int in_dim);
-// ctrl: where a wait that runs out is recorded, and the poll limit
-cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, SvlmCtrl* ctrl, cudaStream_t st);
+// from_l2: W is likely to be in L2 already.  ctrl: where a wait that runs out is recorded, and the poll limit
+cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int in_dim, int out_dim, bool from_l2, SvlmCtrl* ctrl, cudaStream_t st);
 
 // tcgen05/TMEM/TMA chunk prefill, n_q >= 2 (svlm_prefill_sm100.cu)
 bool svlm_prefill_supported(int n_pages, int group);

@@ -283,7 +283,7 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
         // split-KV decode; every cache's scratch was sized for this launch shape at creation
         int pages = 1;
         for (int i = 0; i < n_caches; ++i) pages = std::max(pages, expected_pages(caches[i]));
-        int splits = layer >= 0 ? svlm_decode_layer_splits(c0->dev.n_pages, pages, c0->dev.kv_heads, n_caches) : 0;
+        int splits = n_layers == 1 ? svlm_decode_layer_splits(c0->dev.n_pages, pages, c0->dev.kv_heads, n_caches, c0->dev.head_dim) : 0;
         const bool tagged = splits > 0;
         if (!tagged) splits = svlm_decode_splits(c0->dev.n_pages, c0->dev.kv_heads, n_caches * n_layers);
         SVLM_CUDA(svlm_launch_decode(b, layer0, n_layers, Q, q_pos, q_heads, out, splits, Knew, Vnew, early, tagged, c0->stream));
@@ -496,7 +496,9 @@ int svlm_out_proj(svlm_cache* c, const void* A, const void* Wo, int in_dim, int 
     // between: the decode then has less time before its inputs are ready and does not pace its read-ahead.
     ++c->calls_since_decode;
     if (svlm_gemv_supported(n, in_dim)) {      // a few tokens (decode): reading Wo once is all the work
-        SVLM_CUDA(svlm_launch_gemv(A, Wo, Y, n, in_dim, out_dim, c->dev.ctrl, c->stream));
+        // all layers' projections on both sides of the decode step, taken to be of this one's size, against the 126 MB of L2
+        const bool from_l2 = (size_t)c->dev.layers * 2 * in_dim * out_dim * 2 < (size_t)96 << 20;
+        SVLM_CUDA(svlm_launch_gemv(A, Wo, Y, n, in_dim, out_dim, from_l2, c->dev.ctrl, c->stream));
         return SVLM_OK;
     }
     static const EncodeTiledFn encode = tensor_map_encoder();
