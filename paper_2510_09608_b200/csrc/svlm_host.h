@@ -37,5 +37,6 @@ struct svlm_cache {
     size_t hstage_bytes = 0;
     // copy streams and per-layer events of the pipelined host-buffer chunk prefill (created on first use)
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
+    cudaEvent_t ev_start = nullptr;
     std::vector<cudaEvent_t> ev_in, ev_done;
 };

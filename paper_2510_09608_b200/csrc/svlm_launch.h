@@ -24,8 +24,11 @@ cudaError_t svlm_allow_smem(size_t bytes) {
 
 // Launches a kernel that may become resident while its predecessor in the stream ends (programmatic dependent launch: the
 // kernel itself waits, griddepcontrol), as clusters of `cluster` CTAs, and counts it.
-template <typename... P, typename... A>
-cudaError_t svlm_launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st, A... args) {
+template <typename T>
+struct svlm_same { typedef T type; };
+template <typename... P>
+cudaError_t svlm_launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st,
+                                const typename svlm_same<P>::type&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -41,7 +44,8 @@ cudaError_t svlm_launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, siz
     cfg.attrs = attr;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     svlm_count_launch();
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    void* at[] = {const_cast<void*>(static_cast<const void*>(&args))...};      // (kilobytes of parameters: no copies on the way)
+    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), at);
 }
 
 // Streaming multiprocessors of the current device (looked up once per device).

@@ -400,6 +400,7 @@ void svlm_cache_destroy(svlm_cache* c) {
     if (c->hstage) cudaFreeHost(c->hstage);
     if (c->copy_in) { cudaStreamSynchronize(c->copy_in); cudaStreamDestroy(c->copy_in); }
     if (c->copy_out) { cudaStreamSynchronize(c->copy_out); cudaStreamDestroy(c->copy_out); }
+    if (c->ev_start) cudaEventDestroy(c->ev_start);
     for (cudaEvent_t e : c->ev_in) cudaEventDestroy(e);
     for (cudaEvent_t e : c->ev_done) cudaEventDestroy(e);
     delete c;
@@ -669,6 +670,7 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
         if (!c->copy_in) {
             SVLM_CUDA(cudaStreamCreateWithFlags(&c->copy_in, cudaStreamNonBlocking));
             SVLM_CUDA(cudaStreamCreateWithFlags(&c->copy_out, cudaStreamNonBlocking));
+            SVLM_CUDA(cudaEventCreateWithFlags(&c->ev_start, cudaEventDisableTiming));
         }
         while ((int)c->ev_in.size() < nl) {
             cudaEvent_t a = nullptr, b = nullptr;
@@ -680,10 +682,15 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
         const size_t layer_bytes = (size_t)n_q * q_heads * c->dev.head_dim * 2;
         const size_t pos_n = (size_t)n_q * (c->dev.rope_mode == SVLM_ROPE_1D ? 1 : 3) * sizeof(int32_t);
         // The staging buffer, and by contract the caller's, may still be in use by earlier work on the cache's stream.
-        // Waited for here and not with an event on the copy stream: copies queued behind an event that is still
-        // pending run one direction after the other (28 layers of 524 queries behind an append and an eviction:
-        // 4.85 ms, this way 3.29 of which 0.7 are that work; the call ends with a synchronisation anyway).
-        SVLM_CUDA(cudaStreamSynchronize(c->stream));
+        // Large transfers wait for it here: copies queued behind an event that is still pending run one direction after
+        // the other (28 layers of 524 queries behind an append and an eviction: 4.85 ms, this way 3.29 of which 0.7 are
+        // that work).  Small ones are paced by their enqueueing, which an event lets overlap with that work.
+        if (nl * layer_bytes >= ((size_t)16 << 20)) {
+            SVLM_CUDA(cudaStreamSynchronize(c->stream));
+        } else {
+            SVLM_CUDA(cudaEventRecord(c->ev_start, c->stream));
+            SVLM_CUDA(cudaStreamWaitEvent(c->copy_in, c->ev_start, 0));
+        }
         SVLM_CUDA(cudaMemcpyAsync(s + 2 * q_bytes, q_pos_host, pos_n, cudaMemcpyHostToDevice, c->stream));
         for (int l = 0; l < nl; ++l) {
             SVLM_CUDA(cudaMemcpyAsync(s + l * layer_bytes, static_cast<const char*>(Q_host) + l * layer_bytes, layer_bytes,
