@@ -1,0 +1,150 @@
+"""The kernels' dispatch at the sizes where it can go wrong: edges of tiles, remainders, the smallest and largest of a
+range, and the branches between kernels, each against the fp64 checker."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _wl(config, **kw):
+    from paper_2510_09608_b200 import streamgen as sg
+    return dataclasses.replace(sg.workloads()[config], **kw)
+
+
+# --- chunk prefill: units cut between thread blocks (caches of 18 pages and more), one head per KV head (no shared
+# --- rotation factors), ragged row tiles, a chunk longer than the windows keep, positions beyond 2^16
+@pytest.mark.parametrize("d,hq,hk,frames,vw,base,contiguous", [
+    (128, 28, 4, 1, 2304, 0, True), (128, 4, 4, 3, 1984, 0, True), (64, 7, 1, 3, 2304, 0, True), (64, 16, 8, 1, 2000, 0, True),
+    (128, 28, 4, 9, 192, 0, True), (64, 12, 2, 7, 64, 0, True), (128, 6, 2, 2, 512, 70000, False)])
+def test_chunk_prefill_work_split(d, hq, hk, frames, vw, base, contiguous):
+    from harness import SideBySide, assert_close
+    wl = _wl(2, layers=1, q_heads=hq, kv_heads=hk, head_dim=d, sections=(d // 8, d // 16 * 3, d // 16 * 3), n_sink=40, vision_window=vw, text_window=70,
+             frames=frames, grid_h=8, grid_w=9, text_max=21)
+    s = SideBySide(wl, contiguous=contiguous)
+    s.stream.base = base
+    for _ in range(2 + (vw + 70) // (72 * frames)):
+        s.append_chunk()
+        s.evict()
+    s.append_chunk()
+    s.evict()
+    s.check_metadata()
+    n = len(s.last[0])
+    rows = sorted({0, 1, n // 2, n - 2, n - 1, *range(0, n, 37)})
+    assert_close(s.attend(0, rows=rows))
+
+
+# --- append metadata: one token, up to 1024 (one per thread), more; sinks of either rule that end inside a chunk; evictions
+# --- of more tokens than fit the lists in shared memory
+@pytest.mark.parametrize("sink_any", [False, True])
+@pytest.mark.parametrize("sizes", [(1, 31, 32, 33, 96, 97, 128), (1023, 1024, 1025, 2), (1500, 900, 1, 1700, 40)])
+def test_append_sizes_and_large_evictions(sizes, sink_any):
+    from harness import SideBySide
+    wl = _wl(2, layers=1, q_heads=2, kv_heads=1, head_dim=64, rope_mode=0, sections=(32, 0, 0), n_sink=60, vision_window=150, text_window=130)
+    s = SideBySide(wl, capacity=6000, sink_any=sink_any)
+    rng = np.random.default_rng(sum(sizes))
+    gid = pos = 0
+    for rep in range(2):
+        for i, n in enumerate(sizes):
+            types = rng.integers(0, 2, n).astype(np.uint8)
+            s._append(np.arange(gid, gid + n), types, (pos + np.arange(n)).astype(np.int32))
+            gid, pos = gid + n, pos + n
+            s.check_metadata()
+            if i % 3 == 2 or i == len(sizes) - 1:
+                s.evict()
+                s.check_metadata()
+    s.check_kv(0)
+
+
+# --- decode: one to three units per warp, a second round, the step to the streaming kernel; one, two and three caches
+@pytest.mark.parametrize("d,hq,hk,vw,streams", [
+    (128, 28, 4, 100, 1), (64, 5, 1, 40, 1), (128, 8, 8, 4700, 1), (128, 8, 8, 6300, 1), (64, 16, 8, 6300, 1),
+    (128, 14, 2, 300, 2), (128, 28, 4, 6200, 2), (64, 4, 1, 700, 3), (128, 28, 4, 3000, 3)])
+def test_decode_kernel_choice(d, hq, hk, vw, streams):
+    from harness import SideBySide, assert_close, bits_to_dev, dev_to_f64
+    from paper_2510_09608_b200 import binding
+    wl = _wl(2, layers=1, q_heads=hq, kv_heads=hk, head_dim=d, sections=(d // 8, d // 16 * 3, d // 16 * 3), n_sink=20, vision_window=vw, text_window=30,
+             frames=4, grid_h=12, grid_w=13, text_max=9)
+    sides = [SideBySide(wl, stream=i) for i in range(streams)]
+    for i, s in enumerate(sides):
+        for _ in range(1 + vw // 624 + i % 2):
+            s.append_chunk()
+            s.evict()
+    for step in range(2):
+        toks = [s.stream.next_decode_token() for s in sides]
+        K, V, Q = (np.stack([getattr(s.stream, w)(0, t[0])[0] for s, t in zip(sides, toks)]) for w in "kvq")
+        ty = torch.from_numpy(np.concatenate([t[1] for t in toks])).cuda()
+        ps = torch.from_numpy(np.ascontiguousarray(np.stack([t[2][0] for t in toks]))).cuda()
+        out = dev_to_f64(binding.decode_step_batched([s.cache for s in sides], 0, bits_to_dev(K), bits_to_dev(V), ty, ps, bits_to_dev(Q)))
+        for i, (s, t) in enumerate(zip(sides, toks)):
+            assert s.cache.status() == binding.OK
+            s.ref.append(None, None, t[1], t[2])
+            s._give_values_to_ref(0)
+            assert_close(s._stats(out[i][None], s.ref.attend(0, Q[i][None], t[2])))
+    for s in sides:
+        s.check_metadata()
+        s.check_kv(0)
+
+
+# --- projections: a few tokens with weights beyond L2 (512 layers' worth of this size) and within, stages that do not fill,
+# --- more rows than one wave of blocks takes; token tiles around multiples of 32, odd numbers of 128-row blocks
+@pytest.mark.parametrize("layers,n,in_dim,out_dim", [
+    (512, 1, 576, 128), (512, 4, 1088, 384), (512, 2, 3584, 640), (512, 3, 4160, 8448), (512, 1, 128, 1152), (1, 1, 4160, 640),
+    (512, 4, 25600, 128),
+    (1, 17, 64, 128), (1, 31, 128, 384), (1, 33, 448, 640), (1, 160, 64, 256), (1, 161, 192, 896), (1, 257, 3584, 256), (1, 1400, 128, 1152)])
+def test_projection_shapes(layers, n, in_dim, out_dim):
+    from harness import bits_to_dev, dev_to_f64
+    from oracle import qkv
+    from paper_2510_09608_b200 import binding
+    rng = np.random.default_rng(n + in_dim)
+    A = qkv.to_bf16_bits(rng.standard_normal((n, in_dim)))
+    W = qkv.to_bf16_bits(rng.standard_normal((out_dim, in_dim)) / np.sqrt(in_dim))
+    c = binding.Cache(layers, 1, 64, 4, 64, 16, 128)
+    a, w = bits_to_dev(A), bits_to_dev(W)
+    want = qkv.out_project(A, W)
+    for _ in range(2):                               # the second call starts while the first one ends
+        Y = c.out_proj(a, w)
+    assert np.all(np.abs(dev_to_f64(Y) - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * np.sqrt(in_dim))
+    assert c.status() == binding.OK
+
+
+def test_host_prefill_of_large_transfers():
+    """All layers of a chunk whose queries are more than the size from which the host waits before it enqueues the copies."""
+    from harness import bits_to_dev
+    from paper_2510_09608_b200 import binding, streamgen as sg
+    wl = _wl(2, layers=4, n_sink=16, vision_window=900, text_window=32, frames=3, grid_h=14, grid_w=14)
+    stream = sg.Stream(wl, 0)
+    c = binding.Cache(wl.layers, wl.kv_heads, wl.head_dim, wl.n_sink, wl.vision_window, wl.text_window, wl.capacity)
+    c.set_rope(wl.rope_mode, wl.rope_base, wl.sections)
+    for _ in range(2):
+        gids, types, pos = stream.next_chunk()
+        K, V, Q = (np.stack([getattr(stream, w)(l, gids) for l in range(wl.layers)]) for w in "kvq")
+        ps = torch.from_numpy(np.ascontiguousarray(pos))
+        c.append(-1, bits_to_dev(K), bits_to_dev(V), torch.from_numpy(types).cuda(), ps.cuda())
+        c.evict()
+        assert Q.nbytes >= 16 << 20
+        got = torch.empty(Q.shape, dtype=torch.int16).pin_memory()
+        c.attend_host(-1, torch.from_numpy(Q.view(np.int16)).pin_memory(), ps.pin_memory(), got)
+        want = torch.stack([c.attend(l, bits_to_dev(Q[l]), ps.cuda()) for l in range(wl.layers)])
+        assert torch.equal(got, want.view(torch.int16).cpu())
+        assert c.status() == binding.OK
+
+
+def test_few_token_projection_gives_up_and_recovers():
+    """Every wait of the projection for a few tokens made to run out: the status appears, the kernel returns, and with the
+    limit restored it computes."""
+    from harness import bits_to_dev, dev_to_f64
+    from oracle import qkv
+    from paper_2510_09608_b200 import binding
+    rng = np.random.default_rng(5)
+    A, W = qkv.to_bf16_bits(rng.standard_normal((2, 1088))), qkv.to_bf16_bits(rng.standard_normal((384, 1088)) / 33)
+    c = binding.Cache(512, 1, 64, 4, 64, 16, 128)
+    a, w = bits_to_dev(A), bits_to_dev(W)
+    c.debug_set_wait_limit(0)
+    c.out_proj(a, w)
+    assert c.status() == binding.ERR_TIMEOUT
+    c.debug_set_wait_limit(1 << 20)
+    want = qkv.out_project(A, W)
+    assert np.all(np.abs(dev_to_f64(c.out_proj(a, w)) - want) <= 2.0 ** -8 * np.abs(want) + 1e-3)
