@@ -27,8 +27,7 @@
 //                 now each issuer's waits run while the other one's MMAs execute
 //   3490 -> 2700  P handed over through named barriers instead of mbarriers (450 -> 50 cycles), in two halves, so that
 //                 the first half's P V runs under the second half's exponentials
-//   softmax of a page 2200 -> 1500 cycles: the whole row in registers (one pass over TMEM), packed fp32 pairs, a
-//                 quarter of the exponentials as a polynomial on the FMA pipe (MUFU alone would need 1024 cycles)
+//   softmax of a page 2200 -> 1500 cycles: the whole row in registers (one pass over TMEM), packed fp32 pairs
 // Per-page bookkeeping that cost a masked page 2 us (descriptor loads, two barriers and a bisection through shared
 // memory) is now a few shuffles on values that arrive while the thread waits for S.
 // Every mbarrier wait is bounded: on expiry the CTA records SVLM_ERR_TIMEOUT in the caches' status words, keeps up its
@@ -91,31 +90,6 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b) { u64 r; asm("mul.rn.ftz.f32x2
 __device__ __forceinline__ float max3(float a, float b, float c) { float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r; }
 __device__ __forceinline__ float ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
-// 2^x of a pair on the FMA pipe: x = n + f with n the nearest integer (added and taken off again with 1.5 * 2^23),
-// 2^f by the degree-5 minimax polynomial on [-1/2, 1/2] (Remez exchange on the relative error; 2.1e-7 with fp32
-// Horner steps, the size of ex2.approx's own error), n added to the exponent field.  x is held above -126.
-__device__ __forceinline__ u64 exp2_poly2(u64 x) {
-    float a, b;
-    un64(x, a, b);
-    x = pk64(fmaxf(a, -126.f), fmaxf(b, -126.f));
-    constexpr float MAGIC = 12582912.f;
-    const u64 t = add2(x, pk64(MAGIC, MAGIC));
-    const u64 n = add2(t, pk64(-MAGIC, -MAGIC));
-    const u64 f = fma2(n, pk64(-1.f, -1.f), x);
-    u64 p = pk64(0.0013276472454890609f, 0.0013276472454890609f);
-    p = fma2(p, f, pk64(0.009675540961325169f, 0.009675540961325169f));
-    p = fma2(p, f, pk64(0.05550713092088699f, 0.05550713092088699f));
-    p = fma2(p, f, pk64(0.24022120237350464f, 0.24022120237350464f));
-    p = fma2(p, f, pk64(0.6931469440460205f, 0.6931469440460205f));
-    p = fma2(p, f, pk64(1.0000001192092896f, 1.0000001192092896f));
-    float ta, tb, pa, pb;
-    un64(t, ta, tb);
-    un64(p, pa, pb);
-    pa = __int_as_float(__float_as_int(pa) + (__float_as_int(ta) << 23));
-    pb = __int_as_float(__float_as_int(pb) + (__float_as_int(tb) << 23));
-    return pk64(pa, pb);
-}
-
 // ---- named barriers (the hardware's, not shared memory): ids ----------------------------------------------------
 constexpr int BAR_WG = 1;      // + tile: the softmax warpgroup alone (128)
 constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM and it is this tile's turn (128 softmax + 32 other issuer + 32 issuer)
@@ -145,7 +119,9 @@ __device__ __forceinline__ void rescale_o(unsigned tO, int D, float corr) {
 // more than 2^8).  The whole row is loaded once; the first half's maximum is taken while the second half is on its
 // way.  P goes out in chunks of 32 keys; once the exponentials of the third chunk are done, the first two chunks are
 // certainly stored and are handed to the issuer (BAR_P1).  On MASKED pages the row sees the columns [vlo, vlo + vlen).
-constexpr int PF_POLY = 2;             // of every 8 pairs, those whose exponential goes to the FMA pipe (0: +5 %, 1: +2 %, 3: +9 % time)
+// All exponentials on the special-function unit, although it then has as many cycles of work as the tensor pipe: a polynomial
+// on the FMA pipe for a quarter of them made a cold launch 5 % faster, but a chunk of many layers runs at the power limit,
+// where its instructions cost clock (28 layers 2580 -> 2535 us, four layers of a long chunk 1740 -> 1718, one layer 105.0).
 template <bool MASKED>
 __device__ __forceinline__ void softmax_page(int g, unsigned tS, unsigned tO, int D, unsigned vlo, unsigned vlen, float c,
                                              float m_ref, bool have_o, float& rowsum, float& corr, float& m_new) {
@@ -186,22 +162,10 @@ __device__ __forceinline__ void softmax_page(int g, unsigned tS, unsigned tO, in
             const int k = ch * 32 + 2 * i;
             const u64 t = fma2(pk64(s[k], s[k + 1]), c2, nm2);
             float e0, e1;
-            u64 e;
-            if ((i & 7) < PF_POLY) {
-                e = exp2_poly2(t);
-                un64(e, e0, e1);
-                if (MASKED) {
-                    e0 = s[k] == -INFINITY ? 0.f : e0;
-                    e1 = s[k + 1] == -INFINITY ? 0.f : e1;
-                    e = pk64(e0, e1);
-                }
-            } else {
-                un64(t, e0, e1);
-                e0 = ex2(e0);
-                e1 = ex2(e1);
-                e = pk64(e0, e1);
-            }
-            sum[i & 1] = add2(sum[i & 1], e);
+            un64(t, e0, e1);
+            e0 = ex2(e0);
+            e1 = ex2(e1);
+            sum[i & 1] = add2(sum[i & 1], pk64(e0, e1));
             pk[i] = pack2(e0, e1);
         }
         if (ch == 2) {
