@@ -126,8 +126,16 @@ struct SvlmPrefillLoad {
     int pages;      // stored pages
     int windows;    // most tokens the windows keep, i.e. most of a chunk that can be stored
 };
+// few rows over few pages: a kernel of their own (svlm_prefill_small.cu)
+struct SvlmPrefillSmall {
+    int tiles;      // of 16 rows per CTA; 0: the tensor-core kernel's business
+    int parts;      // CTAs (a cluster) that divide the keys
+};
+SvlmPrefillSmall svlm_prefill_small_plan(const SvlmAttendBatch& b, int call_layers, int n_q, int q_heads, const SvlmPrefillLoad* held);
+cudaError_t svlm_launch_prefill_small(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
+                                      int n_q, int q_heads, SvlmPrefillSmall how, void* out, cudaStream_t st);
 size_t svlm_prefill_slot_bytes(int n_pages, int head_dim);
 constexpr size_t svlm_prefill_counter_bytes = 4096;
-cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
+cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, int call_layers, const void* Q, const int* q_pos,
                                 int n_q, int q_heads, void* out, const SvlmPrefillLoad* held, void* counters, void* slots,
                                 cudaStream_t st);

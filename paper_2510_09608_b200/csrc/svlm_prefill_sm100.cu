@@ -1,7 +1,7 @@
 // Chunk-prefill attention for sm_100a: the new chunk's queries (n_q >= 2 rows) attend over the
 // retained cache plus, causally, the chunk itself (paper Section 2.1: the retained KV is reused, only
 // the new second of tokens is computed).  This is the one dense contraction of the path, so it runs
-// on the 5th-generation tensor cores.
+// on the 5th-generation tensor cores (chunks of few rows over short windows: svlm_prefill_small.cu).
 //
 // Work split.  A unit is 256 packed rows (row = (token, head in the GQA group)) of one KV head of one problem
 // (cache, layer): two 128-row tiles A and B that share every K/V page (with 128 rows per CTA the K/V stream out of L2
@@ -1131,8 +1131,10 @@ size_t svlm_prefill_slot_bytes(int n_pages, int head_dim) {
     return (size_t)2 * std::min(svlm_sm_count(), PF_MAX_CTAS) * (head_dim == 128 ? pf_slot_bytes<128>() : pf_slot_bytes<64>());
 }
 
-cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
+cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, int call_layers, const void* Q, const int* q_pos,
                                 int n_q, int q_heads, void* out, const SvlmPrefillLoad* held, void* counters, void* slots, cudaStream_t st) {
+    const SvlmPrefillSmall small = svlm_prefill_small_plan(b, call_layers, n_q, q_heads, held);
+    if (small.tiles > 0) return svlm_launch_prefill_small(b, layer0, n_layers, Q, q_pos, n_q, q_heads, small, out, st);
     return b.head_dim == 128
         ? launch<128>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, held, counters, slots, st)
         : launch<64>(b, layer0, n_layers, (const uint16_t*)Q, q_pos, n_q, q_heads, (uint16_t*)out, held, counters, slots, st);

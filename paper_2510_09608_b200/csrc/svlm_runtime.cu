@@ -236,8 +236,9 @@ SvlmPrefillLoad expected_load(const svlm_cache* c) {
     return {expected_pages(c), (int)std::min<long long>(c->stored_est > c->dev.n_sink + keep ? c->stored_est : keep, 1 << 30)};
 }
 
+// call_layers: of a call that is launched layer by layer, all its layers (it takes the kernel that one launch of them would).
 int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void* Q, const int32_t* q_pos, int n_q,
-                  int q_heads, void* out, const void* Knew = nullptr, const void* Vnew = nullptr) {
+                  int q_heads, void* out, const void* Knew = nullptr, const void* Vnew = nullptr, int call_layers = 0) {
     svlm_cache* c0 = caches[0];
     if (!Q || !q_pos || !out || n_q < 1 || q_heads < 1) return SVLM_ERR_ARG;
     if (q_heads % c0->dev.kv_heads) return SVLM_ERR_ARG;
@@ -293,7 +294,8 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     if (n_q >= 2 && svlm_prefill_supported(c0->dev.n_pages, group)) {
         SvlmPrefillLoad held[SVLM_MAX_BATCH];
         for (int i = 0; i < n_caches; ++i) { held[i] = expected_load(caches[i]); caches[i]->meta_settled = true; }
-        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, held, c0->prefill_counters, c0->prefill_slots, c0->stream));
+        SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, std::max(n_layers, call_layers), Q, q_pos, n_q, q_heads, out, held, c0->prefill_counters,
+                                      c0->prefill_slots, c0->stream));
         return SVLM_OK;
     }
     svlm_launch_attend_simple(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, c0->stream);
@@ -620,7 +622,7 @@ int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int laye
     DeviceGuard guard(c0->device);
     SvlmPrefillLoad held[SVLM_MAX_BATCH];
     for (int i = 0; i < n_caches; ++i) { held[i] = expected_load(caches[i]); caches[i]->meta_settled = true; }
-    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, Q, q_pos, n_max, q_heads, out, held, c0->prefill_counters, c0->prefill_slots, c0->stream));
+    SVLM_CUDA(svlm_launch_prefill(b, layer, 1, 1, Q, q_pos, n_max, q_heads, out, held, c0->prefill_counters, c0->prefill_slots, c0->stream));
     return SVLM_OK;
 }
 
@@ -665,6 +667,7 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
     if (rc != SVLM_OK) return rc;
     char* s = static_cast<char*>(c->stage);
     if (layer < 0 && nl > 1 && n_q >= 2) {
+        svlm_cache* one[1] = {c};
         // All layers of a chunk: the layers' queries go up, are attended and their outputs come down as a
         // pipeline over three streams, so that the copies of one layer hide behind the attention of another.
         if (!c->copy_in) {
@@ -699,8 +702,8 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
         }
         for (int l = 0; l < nl; ++l) {
             SVLM_CUDA(cudaStreamWaitEvent(c->stream, c->ev_in[l], 0));
-            rc = svlm_attend(c, l, s + l * layer_bytes, reinterpret_cast<const int32_t*>(s + 2 * q_bytes), n_q, q_heads,
-                             s + q_bytes + l * layer_bytes);
+            rc = attend_common(one, 1, l, s + l * layer_bytes, reinterpret_cast<const int32_t*>(s + 2 * q_bytes), n_q, q_heads,
+                               s + q_bytes + l * layer_bytes, nullptr, nullptr, nl);
             if (rc != SVLM_OK) break;
             SVLM_CUDA(cudaEventRecord(c->ev_done[l], c->stream));
             SVLM_CUDA(cudaStreamWaitEvent(c->copy_out, c->ev_done[l], 0));

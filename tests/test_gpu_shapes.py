@@ -36,6 +36,50 @@ def test_chunk_prefill_work_split(d, hq, hk, frames, vw, base, contiguous):
     assert_close(s.attend(0, rows=rows))
 
 
+# --- chunks of few rows: rows at the edges of a 16-row tile, one to eight thread blocks over the keys, two tiles per block,
+# --- partly filled pages, positions beyond 2^16
+@pytest.mark.parametrize("d,hq,hk,frames,gh,gw,vw,base,contiguous", [
+    (64, 4, 1, 1, 2, 2, 64, 0, True), (128, 4, 4, 1, 1, 15, 70, 0, True), (128, 4, 4, 1, 1, 17, 330, 0, True), (64, 1, 1, 1, 1, 2, 30, 0, True),
+    (64, 4, 1, 1, 6, 6, 2300, 0, True), (128, 8, 4, 1, 6, 6, 2300, 0, True), (64, 16, 8, 1, 6, 6, 2300, 0, True), (128, 28, 4, 1, 5, 6, 2000, 0, True),
+    (64, 16, 8, 2, 8, 10, 500, 0, True), (128, 28, 4, 2, 8, 8, 300, 0, True), (128, 9, 1, 1, 3, 5, 200, 70000, False), (64, 3, 1, 1, 5, 5, 20, 0, True)])
+def test_chunk_prefill_of_few_rows(d, hq, hk, frames, gh, gw, vw, base, contiguous):
+    from harness import SideBySide, assert_close
+    wl = _wl(2, layers=1, q_heads=hq, kv_heads=hk, head_dim=d, sections=(d // 8, d // 16 * 3, d // 16 * 3), n_sink=5, vision_window=vw, text_window=37,
+             frames=frames, grid_h=gh, grid_w=gw, text_max=2)
+    s = SideBySide(wl, contiguous=contiguous)
+    s.stream.base = base
+    for _ in range(2 + vw // (frames * gh * gw)):
+        s.append_chunk()
+        s.evict()
+    for _ in range(2):
+        s.append_chunk()
+        s.evict()
+        assert_close(s.attend(0))
+
+
+# --- the tensor-core prefill kernel's waits made to run out (the few rows of other give-up tests are the small kernel's)
+@pytest.mark.parametrize("d,hq,hk", [(128, 28, 4), (64, 12, 2)])
+def test_large_chunk_prefill_gives_up_and_recovers(d, hq, hk):
+    from harness import SideBySide, assert_close, bits_to_dev, dev_to_f64
+    from paper_2510_09608_b200 import binding
+    wl = _wl(2, layers=1, q_heads=hq, kv_heads=hk, head_dim=d, sections=(d // 8, d // 16 * 3, d // 16 * 3), n_sink=40, vision_window=2304, text_window=70,
+             frames=9, grid_h=8, grid_w=9, text_max=21)
+    s = SideBySide(wl)
+    for _ in range(5):
+        s.append_chunk()
+        s.evict()
+    gids, _, pos = s.last
+    Q, qp = bits_to_dev(s.stream.q(0, gids)), torch.from_numpy(np.ascontiguousarray(pos)).cuda()
+    s.cache.debug_set_wait_limit(0)
+    s.cache.attend(0, Q, qp)
+    assert s.cache.status() == binding.ERR_TIMEOUT
+    s.cache.debug_set_wait_limit(1 << 20)
+    out = dev_to_f64(s.cache.attend(0, Q, qp))
+    s._give_values_to_ref(0)
+    rows = list(range(0, len(gids), 29))
+    assert_close(s._stats(out[rows], s.ref.attend(0, s.stream.q(0, gids), pos, rows=rows)))
+
+
 # --- append metadata: one token, up to 1024 (one per thread), more; sinks of either rule that end inside a chunk; evictions
 # --- of more tokens than fit the lists in shared memory
 @pytest.mark.parametrize("sink_any", [False, True])
