@@ -55,7 +55,11 @@ constexpr int PF_RING = 4;            // K/V page stages (3: 18 % slower, the ne
 constexpr int PF_MAX_TILES = 512;
 constexpr int PF_ROWS = 256;          // rows per unit
 constexpr int PF_MAX_CTAS = 160;
-constexpr int PF_MIN_PAGES = 6;       // pages a CTA should have at least when units are cut
+// When units are cut: pages a CTA should have at least, and pieces per unit beyond which merging them costs what the shorter
+// pieces save.  133 to 261 tokens over 1200 keys, 28/4 heads: 6 pages 31-33 us, 4 28.6-30; 69 tokens over 9200 keys: 18 pieces
+// 56.6 us, 12 48.9, 8 44.8.
+constexpr int PF_MIN_PAGES = 4;
+constexpr int PF_MAX_PIECES = 9;
 constexpr int PF_PIECE = 10;          // what beginning a unit costs, in pages (one stream: 3 and 6: 78 us, 10: 76, 16: 78)
 constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
 constexpr int PF_CS_BYTES = 16384;    // rotation factors of one tile's tokens (5 or more heads per KV head, all at head_dim 64 with 2 or more)
@@ -1021,7 +1025,7 @@ void make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, in
     plan.off[b.n_caches] = plan.units;
     const int U = plan.units;
     const bool cut = plan.slots != nullptr;
-    grid = (int)std::min<long long>(max_ctas, cut ? std::max<long long>(U, all / PF_MIN_PAGES) : U);
+    grid = (int)std::min<long long>(max_ctas, cut ? std::max<long long>(U, std::min<long long>(all / PF_MIN_PAGES, (long long)PF_MAX_PIECES * U)) : U);
     plan.rounds = std::max(0, U / grid - 1);
     plan.tail = plan.rounds * grid;
     const int nt = U - plan.tail;
