@@ -2,29 +2,27 @@
 // paper Section 3.3: per-token latency over a fixed-length context is the figure of merit), optionally
 // fused with the append of that token's own key and value (one "decode step" of a layer).
 //
-// The step reads every stored key and value exactly once, so it is bound by HBM bandwidth.  Two kernels
-// share the work split (grid = (splits, kv_heads, problems), about one CTA per SM; the G <= 8 query heads of
-// a KV head ride in the N dimension of m16n8k16 MMAs, S^T = K Q^T and O^T += V^T P^T, so K and V are read
-// once per group; rotation factors from a table; the new token of a fused step is patched into its
-// shared-memory rows and written to the cache by the warp that owns its keys) and the combine (the six
-// consumer warps merge through a bank-conflict-free buffer, a CTA's partial (o bf16, m, l) goes to scratch,
-// the last CTA of a (cache, layer, KV head) to arrive merges all partials: arrival counter, nobody waits):
+// The step reads every stored key and value exactly once, so it is bound by HBM bandwidth.  Two kernels share the work
+// split (grid = (splits, kv_heads, problems); the G <= 8 query heads of a KV head ride in the N dimension of m16n8k16 MMAs,
+// S^T = K Q^T and O^T += V^T P^T, so K and V are read once per group; rotation factors from a table; the new token of a
+// fused step is patched into the rows of the warp that owns its place, which also writes it to the cache), and a CTA's six
+// consumer warps merge through a bank-conflict-free buffer into the CTA's partial result (o bf16, m, l):
 //
-//   decode_stream_kernel   several problems per launch (batched streams, all layers of a token): a CTA walks
-//       many 32-key sub-tiles; one producer thread streams them with TMA (128-byte swizzle) through a six-stage
-//       ring, one stage per consumer warp, full/empty mbarriers with bounded waits.  Throughput kernel.
+//   decode_stream_kernel   many problems per launch (batches of streams, all layers of a token), or more keys than the other
+//       kernel holds: a CTA walks many 32-key sub-tiles; one producer thread streams them with TMA (128-byte swizzle)
+//       through a six-stage ring, one stage per consumer warp, full/empty mbarriers with bounded waits; the last CTA of a
+//       (cache, layer, KV head) to arrive merges all partials (arrival counter, nobody waits).  Throughput kernel.
 //
-//   decode_layer_kernel    one problem per launch (one layer of one stream: the layer-sequential decoder).
+//   decode_layer_kernel    one layer of one stream or of a few (the layer-sequential decoder), about one CTA per SM.
 //       At 19 MB per layer the data time is under 3 us and the launch is chained behind the previous layer's
-//       (programmatic dependent launch): the next layer's kernel is resident while this one finishes, and
-//       what a layer-step costs is the chain AFTER the query is known.  The kernel is arranged around that
-//       chain.  A CTA's keys (about 270) are dealt out to the six consumer warps in 16-key units, three per
-//       warp, and every warp loads its own units with cp.async into four private 4 KB slots: before the
-//       dependency wait its three key units and its first value unit; the other two value units go into
-//       the key slots as soon as the scores are computed and arrive (from L2, where a prefetch has put them)
-//       while the softmax runs.  No producer thread, no barrier hand-offs, nothing to wait on but the
-//       warp's own copies.  One pass: scores of 48 keys per warp in three independent MMA chains, one
-//       softmax, P V unit by unit.
+//       (programmatic dependent launch): the next layer's kernel is resident while this one finishes, and what a layer-step
+//       costs is the chain AFTER the query is known.  The kernel is arranged around that chain.  A CTA's keys (about 270)
+//       are dealt out to its six warps in 16-key units, three per warp; before the dependency wait every warp copies its
+//       units with cp.async into private 4 KB slots, moves the keys of two of them on into fragment registers and lets the
+//       values take over their slots, so that behind the wait nothing is left to fetch but the query.  No producer thread,
+//       no barrier hand-offs.  The code behind the wait is compiled per number of units and has no loop over them.  The
+//       partials meet as tagged words polled by the first CTAs of a KV head, each combining a share.  9.3 us per layer-step
+//       in the first version, 6.5 with the values fetched behind the scores, 6.0 now.
 // Everything that depends on earlier kernels (query, new key/value, scratch) is read after the grid-dependency
 // wait; the cache pages are not (the caller's contract, see the launcher).
 #include <cuda.h>
@@ -839,7 +837,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     if (threadIdx.x == 0) STAMP(0);                  // kernel entry
     constexpr int CH = D / 8;                        // 16-byte chunks per row
     constexpr int ITEM_BYTES = UNIT * D * 2;         // K or V of one unit
-    constexpr int KSTEPS = D / 16, HKS = KSTEPS / 2; // k-steps of 16 dims; of half the head
+    constexpr int KSTEPS = D / 16;                  // k-steps of 16 dims
     constexpr int DBLK = D / 16;
     constexpr int HALF = D / 2;
     extern __shared__ unsigned char smem_raw[];
