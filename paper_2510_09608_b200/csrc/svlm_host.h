@@ -33,8 +33,9 @@ struct svlm_cache {
     // staging for the *_host entry points
     void* stage = nullptr;
     size_t stage_bytes = 0;
-    void* hstage = nullptr;       // page-locked host buffer: small inputs of a host-buffer call are gathered here for one copy
-    size_t hstage_bytes = 0;
+    void* hstage = nullptr;       // page-locked host buffer: small inputs of a host-buffer call are gathered here for one transfer,
+    size_t hstage_bytes = 0;      // small outputs arrive here; in front of them (HSTAGE_DATA bytes) the ticket of the latest call
+    unsigned ticket = 0;          // that has completed on the device
     // copy streams and per-layer events of the pipelined host-buffer chunk prefill (created on first use)
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
     cudaEvent_t ev_start = nullptr;

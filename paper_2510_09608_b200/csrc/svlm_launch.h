@@ -69,6 +69,10 @@ void svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmCacheDev
                                    cudaStream_t st);
 void svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
 
+// small transfers from and to page-locked host memory (svlm_host_io.cu); 16-byte aligned, sizes rounded up to 16
+cudaError_t svlm_launch_host_in(void* dst, const void* src, size_t bytes, cudaStream_t st);
+cudaError_t svlm_launch_host_out(void* dst, const void* src, size_t bytes, unsigned* done, unsigned ticket, cudaStream_t st);
+
 // key/value movement (svlm_kv.cu)
 // layer < 0: K,V are [layers][n][kv_heads][d]; otherwise [n][kv_heads][d] for that layer.
 // early != 0: the caller vouches that no kernel still running when this one may start writes the cache's metadata.

@@ -81,7 +81,9 @@ int ensure_stage(svlm_cache* c, size_t bytes) {
 
 // The page-locked gathering buffer.  A host-buffer call that uses it ends with a synchronisation of the cache's
 // stream, so the buffer is free again when the next call starts.
+constexpr size_t HSTAGE_DATA = 256;
 int ensure_hstage(svlm_cache* c, size_t bytes) {
+    bytes += HSTAGE_DATA;
     if (bytes <= c->hstage_bytes) return SVLM_OK;
     SVLM_CUDA(cudaStreamSynchronize(c->stream));
     if (c->hstage) cudaFreeHost(c->hstage);
@@ -89,7 +91,23 @@ int ensure_hstage(svlm_cache* c, size_t bytes) {
     c->hstage_bytes = 0;
     bytes = std::max<size_t>(bytes, 64 << 10);
     if (cudaHostAlloc(&c->hstage, bytes, cudaHostAllocDefault) != cudaSuccess) return SVLM_ERR_NOMEM;
+    std::memset(c->hstage, 0, HSTAGE_DATA);
     c->hstage_bytes = bytes;
+    return SVLM_OK;
+}
+
+// Brings `bytes` from the device to `dst` (in c's page-locked buffer) behind everything enqueued so far and returns when they are
+// there.  The host watches for the call's ticket in memory; now and then it asks the stream, in case that has failed.
+int fetch_and_wait(svlm_cache* c, void* dst, const void* src, size_t bytes) {
+    unsigned* done = static_cast<unsigned*>(c->hstage);
+    const unsigned ticket = ++c->ticket;
+    SVLM_CUDA(svlm_launch_host_out(dst, src, bytes, done, ticket, c->stream));
+    for (unsigned polls = 1; __atomic_load_n(done, __ATOMIC_ACQUIRE) != ticket; ++polls) {
+        if (polls % 4096) continue;
+        const cudaError_t e = cudaStreamQuery(c->stream);
+        if (e == cudaSuccess) break;                       // complete: so is the transfer
+        if (e != cudaErrorNotReady) return SVLM_ERR_CUDA;
+    }
     return SVLM_OK;
 }
 
@@ -758,12 +776,11 @@ int svlm_decode_step_host(svlm_cache* c, int layer, const void* K_host, const vo
         void* dP = dQ ? mapped_alias(pos_host) : nullptr;
         void* dO = dP ? mapped_alias(out_host) : nullptr;
         void* dT = dO ? mapped_alias(token_type_host) : nullptr;
-        if (dT && !(((uintptr_t)dK | (uintptr_t)dV | (uintptr_t)dQ | (uintptr_t)dO) & 15) && !((uintptr_t)dP & 3)) {
+        if (dT && ensure_hstage(c, 0) == SVLM_OK && !(((uintptr_t)dK | (uintptr_t)dV | (uintptr_t)dQ | (uintptr_t)dO) & 15) && !((uintptr_t)dP & 3)) {
             const int rc = svlm_decode_step(c, layer, dK, dV, static_cast<const uint8_t*>(dT), static_cast<const int32_t*>(dP), dQ,
                                             q_heads, dO);
             if (rc != SVLM_OK) return rc;
-            SVLM_CUDA(cudaStreamSynchronize(c->stream));
-            return SVLM_OK;
+            return fetch_and_wait(c, nullptr, nullptr, 0);
         }
     }
     const int nl = layer < 0 ? c->dev.layers : 1;
@@ -774,17 +791,22 @@ int svlm_decode_step_host(svlm_cache* c, int layer, const void* K_host, const vo
     int rc = ensure_stage(c, oO + up(q_bytes));
     if (rc != SVLM_OK) return rc;
     char* s = static_cast<char*>(c->stage);
+    // A small step's inputs are gathered in page-locked memory and go up in one transfer instead of five; up to 64 KB by a kernel,
+    // and the output comes back the same way: one layer of 28/4 heads by itself 34.9 us with copies and a stream
+    // synchronisation, 31.3 so.
+    const bool small = oO + q_bytes <= (64 << 10);
     if (oO <= (256 << 10)) {
-        // the step's inputs are small: gathered in page-locked memory they go up in one copy instead of five
-        rc = ensure_hstage(c, oO);
+        rc = ensure_hstage(c, oO + up(q_bytes));
         if (rc != SVLM_OK) return rc;
-        char* h = static_cast<char*>(c->hstage);
+        char* h = static_cast<char*>(c->hstage) + HSTAGE_DATA;
         std::memcpy(h + oK, K_host, kv_bytes);
         std::memcpy(h + oV, V_host, kv_bytes);
         std::memcpy(h + oQ, Q_host, q_bytes);
         std::memcpy(h + oP, pos_host, pos_bytes);
         if (layer <= 0) h[oT] = static_cast<char>(*token_type_host);
-        SVLM_CUDA(cudaMemcpyAsync(s, h, oT + 16, cudaMemcpyHostToDevice, c->stream));
+        if (small) SVLM_CUDA(svlm_launch_host_in(s, h, oT + 16, c->stream));
+        else SVLM_CUDA(cudaMemcpyAsync(s, h, oT + 16, cudaMemcpyHostToDevice, c->stream));
+        ++c->calls_since_decode;                           // (nothing runs that a read-ahead would hold up)
     } else {
         SVLM_CUDA(cudaMemcpyAsync(s + oK, K_host, kv_bytes, cudaMemcpyHostToDevice, c->stream));
         SVLM_CUDA(cudaMemcpyAsync(s + oV, V_host, kv_bytes, cudaMemcpyHostToDevice, c->stream));
@@ -794,7 +816,16 @@ int svlm_decode_step_host(svlm_cache* c, int layer, const void* K_host, const vo
     }
     rc = svlm_decode_step(c, layer, s + oK, s + oV, reinterpret_cast<const uint8_t*>(s + oT), reinterpret_cast<const int32_t*>(s + oP),
                           s + oQ, q_heads, s + oO);
-    if (rc != SVLM_OK) return rc;
+    if (rc != SVLM_OK) {
+        SVLM_CUDA(cudaStreamSynchronize(c->stream));       // (the inputs are still being read)
+        return rc;
+    }
+    if (small) {
+        char* h = static_cast<char*>(c->hstage) + HSTAGE_DATA + oO;
+        rc = fetch_and_wait(c, h, s + oO, q_bytes);
+        if (rc == SVLM_OK) std::memcpy(out_host, h, q_bytes);
+        return rc;
+    }
     SVLM_CUDA(cudaMemcpyAsync(out_host, s + oO, q_bytes, cudaMemcpyDeviceToHost, c->stream));
     SVLM_CUDA(cudaStreamSynchronize(c->stream));
     return SVLM_OK;
