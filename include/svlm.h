@@ -20,7 +20,11 @@
  *     svlm_cache_query, svlm_cache_status and the *_host variants' final copy where stated;
  *   - conditions only the device can see (a type mix that overflows the capacity) set a sticky
  *     status word that svlm_cache_status returns; the offending append is dropped as a whole;
- *   - bf16 means the 16-bit brain-float bit pattern; Q/K are passed UN-rotated.
+ *   - bf16 means the 16-bit brain-float bit pattern; Q/K are passed UN-rotated;
+ *   - alignment of device pointers: int32 arrays 4 bytes.  Chunks (svlm_cache_append, svlm_attend* with more than one query
+ *     row, svlm_attend_batched_varlen): K, V, Q and out 16 bytes.  One query token (svlm_decode_step*, svlm_attend* with
+ *     n_q == 1, svlm_attend_decode_noalloc): Q, K and V anywhere an array of bf16 may begin (2 bytes), out 4 bytes.  The
+ *     projections: 16 bytes.  Anything else is SVLM_ERR_ARG.  The *_host variants' buffers may lie anywhere.
  */
 #ifndef SVLM_H
 #define SVLM_H

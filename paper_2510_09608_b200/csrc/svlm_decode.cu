@@ -320,7 +320,13 @@ __device__ __forceinline__ void arrive_and_combine(int* s_last, unsigned* counte
         uint4 pk;
         pk.x = pack_bf16(acc[0] * inv, acc[1] * inv); pk.y = pack_bf16(acc[2] * inv, acc[3] * inv);
         pk.z = pack_bf16(acc[4] * inv, acc[5] * inv); pk.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-        *reinterpret_cast<uint4*>(out_row0 + (size_t)h * D + d0) = pk;
+        uint16_t* dst = out_row0 + (size_t)h * D + d0;
+        if (!(reinterpret_cast<uintptr_t>(dst) & 15)) {
+            *reinterpret_cast<uint4*>(dst) = pk;
+        } else {                                        // (the caller's buffer need only be 4-byte aligned)
+            unsigned* words = reinterpret_cast<unsigned*>(dst);
+            words[0] = pk.x; words[1] = pk.y; words[2] = pk.z; words[3] = pk.w;
+        }
     }
 }
 
@@ -829,7 +835,8 @@ __device__ __forceinline__ int lay_off(int key, int chunk) {
     return (chunk >> 3) * (UNIT * 128) + key * 128 + (((chunk & 7) ^ (key & 7)) << 4);
 }
 
-template <int D>
+// ANYWHERE: Q, Knew or Vnew does not begin at a word (a choice inside the kernel cost 4 % of a layer-step).
+template <int D, bool ANYWHERE>
 __global__ void __launch_bounds__(LAY_THREADS, 2)
 decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q, const int* __restrict__ q_pos, int q_heads,
                     uint16_t* __restrict__ out, int splits, const uint16_t* __restrict__ Knew,
@@ -1025,13 +1032,16 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
             lo = pack_bf16(x0 * f[0].x - y0 * f[0].y, x1 * f[1].x - y1 * f[1].y);
             hi = pack_bf16(y0 * f[0].x + x0 * f[0].y, y1 * f[1].x + x1 * f[1].y);
         };
+        auto two = [](const uint16_t* p) {           // two neighbouring elements
+            return ANYWHERE ? (unsigned)p[0] | (unsigned)p[1] << 16 : *reinterpret_cast<const unsigned*>(p);
+        };
         unsigned lo[HN], hi[HN];
 #pragma unroll
         for (int k = 0; k < HN; ++k) {               // all loads first: one round trip
             const int h = threadIdx.x / LPH + k * HSTEP;
             const uint16_t* row = Q + (q_head0 + (h < G ? h : 0)) * D + 2 * p2;   // n_q = 1
-            lo[k] = *reinterpret_cast<const unsigned*>(row);
-            hi[k] = *reinterpret_cast<const unsigned*>(row + HALF);
+            lo[k] = two(row);
+            hi[k] = two(row + HALF);
         }
         // fused step: the new token's key and value rows come in with the query; the key is rotated with the query's
         // factors (same token, same position) and both wait in shared memory for the warp whose unit holds the token's slot
@@ -1039,8 +1049,8 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
         unsigned klo = 0, khi = 0, vlo = 0, vhi = 0;
         if (prep_new) {
             const size_t off = kv_head * D + 2 * p2;
-            klo = *reinterpret_cast<const unsigned*>(Knew + off); khi = *reinterpret_cast<const unsigned*>(Knew + off + HALF);
-            vlo = *reinterpret_cast<const unsigned*>(Vnew + off); vhi = *reinterpret_cast<const unsigned*>(Vnew + off + HALF);
+            klo = two(Knew + off); khi = two(Knew + off + HALF);
+            vlo = two(Vnew + off); vhi = two(Vnew + off + HALF);
         }
 #pragma unroll
         for (int k = 0; k < HN; ++k) {
@@ -1312,19 +1322,20 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
         if (g_decode_trace_next >= 0 && g_decode_trace_next < SVLM_TR_LAUNCHES && splits * b.kv_heads <= SVLM_TR_CTAS)
             trace_idx = g_decode_trace_next++;
 #endif
-        if (b.head_dim == 128) {
-            e = svlm_allow_smem<decode_layer_kernel<128>>(decode_layer_smem<128>());
-            if (e != cudaSuccess) return e;
-            cfg.dynamicSmemBytes = decode_layer_smem<128>();
-            e = cudaLaunchKernelEx(&cfg, decode_layer_kernel<128>, b, layer0, Qp, q_pos, q_heads, Op, splits, Kn, Vn,
-                                   early_loads TRACE_ARG);
-        } else {
-            e = svlm_allow_smem<decode_layer_kernel<64>>(decode_layer_smem<64>());
-            if (e != cudaSuccess) return e;
-            cfg.dynamicSmemBytes = decode_layer_smem<64>();
-            e = cudaLaunchKernelEx(&cfg, decode_layer_kernel<64>, b, layer0, Qp, q_pos, q_heads, Op, splits, Kn, Vn,
-                                   early_loads TRACE_ARG);
-        }
+        auto go = [&](auto kernel, size_t smem, cudaError_t allowed) {
+            if (allowed != cudaSuccess) return allowed;
+            cfg.dynamicSmemBytes = smem;
+            return cudaLaunchKernelEx(&cfg, kernel, b, layer0, Qp, q_pos, q_heads, Op, splits, Kn, Vn, early_loads TRACE_ARG);
+        };
+        constexpr size_t smem128 = decode_layer_smem<128>(), smem64 = decode_layer_smem<64>();
+        const bool words = (((uintptr_t)Q | (uintptr_t)Knew | (uintptr_t)Vnew) & 3) == 0;
+        if (b.head_dim == 128)
+            e = words ? go(decode_layer_kernel<128, false>, smem128, svlm_allow_smem<decode_layer_kernel<128, false>>(smem128))
+                      : go(decode_layer_kernel<128, true>, smem128, svlm_allow_smem<decode_layer_kernel<128, true>>(smem128));
+        else
+            e = words ? go(decode_layer_kernel<64, false>, smem64, svlm_allow_smem<decode_layer_kernel<64, false>>(smem64))
+                      : go(decode_layer_kernel<64, true>, smem64, svlm_allow_smem<decode_layer_kernel<64, true>>(smem64));
+        if (e != cudaSuccess) return e;
     } else if (b.head_dim == 128) {
         e = svlm_allow_smem<decode_stream_kernel<128>>(decode_stream_smem<128>());
         if (e != cudaSuccess) return e;

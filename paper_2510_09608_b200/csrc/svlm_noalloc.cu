@@ -55,6 +55,7 @@ int scratch_for_device(int device, float** out) {
 extern "C" int svlm_attend_decode_noalloc(svlm_cache* c, int layer, const void* Q, const int32_t* q_pos, int q_heads,
                                           void* out) {
     if (!c || !Q || !q_pos || !out || q_heads < 1) return SVLM_ERR_ARG;
+    if (((uintptr_t)Q & 1) || (((uintptr_t)out | (uintptr_t)q_pos) & 3)) return SVLM_ERR_ARG;
     const SvlmCacheDev& d = c->dev;
     if (layer < 0 || layer >= d.layers || q_heads % d.kv_heads) return SVLM_ERR_ARG;
     const int group = q_heads / d.kv_heads;

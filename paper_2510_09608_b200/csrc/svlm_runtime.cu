@@ -235,6 +235,15 @@ int make_list(svlm_cache* const* caches, int n_caches, SvlmCacheList& list) {
     return SVLM_OK;
 }
 
+// Every given pointer is a multiple of `bytes`.
+template <typename... P>
+bool aligned(size_t bytes, const P*... p) { return (((uintptr_t)p | ...) & (bytes - 1)) == 0; }
+
+// One query token's attention reads and writes arrays of bf16: Q (and K, V of a fused step) may begin anywhere, out at 4 bytes.
+bool decode_aligned(const void* Q, const void* K, const void* V, const void* out, const void* pos) {
+    return aligned(2, Q, K, V) && aligned(4, out, pos);
+}
+
 // The host's idea of what a cache stores (it does not know the tokens' types, nor what a replayed graph has appended).
 void note_append(svlm_cache* c, int n) {
     c->meta_settled = false;
@@ -261,6 +270,11 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     if (!Q || !q_pos || !out || n_q < 1 || q_heads < 1) return SVLM_ERR_ARG;
     if (q_heads % c0->dev.kv_heads) return SVLM_ERR_ARG;
     if (layer < -1 || layer >= c0->dev.layers) return SVLM_ERR_ARG;
+    const int group = q_heads / c0->dev.kv_heads;
+    const bool split_kv = n_q == 1 && group <= 8 && svlm_decode_supported(c0->dev.n_pages);
+    const bool chunk = n_q >= 2 && svlm_prefill_supported(c0->dev.n_pages, group);
+    if (split_kv && !decode_aligned(Q, Knew, Vnew, out, q_pos)) return SVLM_ERR_ARG;
+    if (chunk && !(aligned(16, Q, out) && aligned(4, q_pos))) return SVLM_ERR_ARG;      // (the general kernel reads and writes element by element)
     SvlmAttendBatch b;
     b.n_caches = n_caches;
     fill_batch_geometry(c0, b);
@@ -274,7 +288,6 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     DeviceGuard guard(c0->device);
     const int layer0 = layer < 0 ? 0 : layer;
     const int n_layers = layer < 0 ? c0->dev.layers : 1;
-    const int group = q_heads / c0->dev.kv_heads;
     int early = 0;
     if (n_q == 1 && layer >= 0) {
         // early loads: the kernel directly before this one on the stream was a decode of another layer that
@@ -298,7 +311,7 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     } else {
         for (int i = 0; i < n_caches; ++i) caches[i]->last_decode_layer = -1;
     }
-    if (n_q == 1 && group <= 8 && svlm_decode_supported(c0->dev.n_pages)) {
+    if (split_kv) {
         // split-KV decode; every cache's scratch was sized for this launch shape at creation
         int pages = 1;
         for (int i = 0; i < n_caches; ++i) pages = std::max(pages, expected_pages(caches[i]));
@@ -309,7 +322,7 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
         return SVLM_OK;
     }
     if (Knew) return SVLM_ERR_ARG;   // the fused step exists for the split-KV kernel only
-    if (n_q >= 2 && svlm_prefill_supported(c0->dev.n_pages, group)) {
+    if (chunk) {
         SvlmPrefillLoad held[SVLM_MAX_BATCH];
         for (int i = 0; i < n_caches; ++i) { held[i] = expected_load(caches[i]); caches[i]->meta_settled = true; }
         SVLM_CUDA(svlm_launch_prefill(b, layer0, n_layers, std::max(n_layers, call_layers), Q, q_pos, n_q, q_heads, out, held, c0->prefill_counters,
@@ -464,7 +477,7 @@ int svlm_cache_set_stream(svlm_cache* c, void* cuda_stream) {
 
 int svlm_cache_append(svlm_cache* c, int layer, const void* K, const void* V, const uint8_t* token_type,
                       const int32_t* pos, int n) {
-    if (!c || !K || !V || n < 1 || layer < -1 || layer >= c->dev.layers) return SVLM_ERR_ARG;
+    if (!c || !K || !V || n < 1 || layer < -1 || layer >= c->dev.layers || !aligned(16, K, V)) return SVLM_ERR_ARG;
     DeviceGuard guard(c->device);
     c->last_decode_layer = -1;
     if (layer <= 0) {
@@ -572,6 +585,7 @@ int svlm_decode_step(svlm_cache* c, int layer, const void* K, const void* V, con
     if (!c || !K || !V || !pos || !Q || !out || layer < -1 || layer >= c->dev.layers || q_heads < 1) return SVLM_ERR_ARG;
     if (q_heads % c->dev.kv_heads || q_heads / c->dev.kv_heads > 8) return SVLM_ERR_ARG;
     if (!svlm_decode_supported(c->dev.n_pages)) return SVLM_ERR_ARG;   // more pages than the fused kernel's page list holds
+    if (!decode_aligned(Q, K, V, out, pos)) return SVLM_ERR_ARG;
     DeviceGuard guard(c->device);
     if (layer <= 0) {
         if (!token_type) return SVLM_ERR_ARG;
@@ -594,7 +608,7 @@ int svlm_decode_step_batched(svlm_cache* const* caches, int n_caches, int layer,
     svlm_cache* c0 = caches[0];
     if (!K || !V || !pos || !Q || !out || layer < 0 || layer >= c0->dev.layers || q_heads < 1) return SVLM_ERR_ARG;
     if (q_heads % c0->dev.kv_heads || q_heads / c0->dev.kv_heads > 8) return SVLM_ERR_ARG;
-    if (!svlm_decode_supported(c0->dev.n_pages)) return SVLM_ERR_ARG;
+    if (!svlm_decode_supported(c0->dev.n_pages) || !decode_aligned(Q, K, V, out, pos)) return SVLM_ERR_ARG;
     DeviceGuard guard(c0->device);
     if (layer == 0) {
         if (!token_type) return SVLM_ERR_ARG;
@@ -620,6 +634,7 @@ int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int laye
     svlm_cache* c0 = caches[0];
     if (!Q || !q_pos || !n_q || !out || q_heads < 1 || layer < 0 || layer >= c0->dev.layers) return SVLM_ERR_ARG;
     if (q_heads % c0->dev.kv_heads || !svlm_prefill_supported(c0->dev.n_pages, q_heads / c0->dev.kv_heads)) return SVLM_ERR_ARG;
+    if (!aligned(16, Q, out) || !aligned(4, q_pos)) return SVLM_ERR_ARG;
     SvlmAttendBatch b;
     b.n_caches = n_caches;
     fill_batch_geometry(c0, b);

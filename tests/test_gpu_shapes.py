@@ -219,3 +219,39 @@ def test_few_token_projection_gives_up_and_recovers():
     c.debug_set_wait_limit(1 << 20)
     want = qkv.out_project(A, W)
     assert np.all(np.abs(dev_to_f64(c.out_proj(a, w)) - want) <= 2.0 ** -8 * np.abs(want) + 1e-3)
+
+
+# --- one token's rows at any element of an array and its output at any word: per-layer kernel (one cache, two), streaming
+# --- kernel (three rounds of keys, many caches); the same bits as from aligned buffers
+@pytest.mark.parametrize("d,hq,hk,kept,streams", [(128, 28, 4, 300, 1), (64, 5, 1, 90, 1), (128, 8, 8, 11000, 1), (128, 14, 2, 300, 2), (64, 16, 8, 200, 4)])
+def test_decode_inputs_at_any_element(d, hq, hk, kept, streams):
+    from paper_2510_09608_b200 import binding
+
+    def shifted(t, by):
+        flat = torch.zeros(t.numel() + 8, dtype=t.dtype, device="cuda")
+        flat[by:by + t.numel()] = t.flatten()
+        return flat[by:by + t.numel()].view(t.shape)
+
+    def run(by):
+        gen = torch.Generator(device="cuda").manual_seed(kept)
+        normal = lambda *shape: torch.randn(*shape, generator=gen, device="cuda", dtype=torch.bfloat16)      # noqa: E731
+        caches = [binding.Cache(1, hk, d, 4, kept, 60, kept + 200) for _ in range(streams)]
+        for c in caches:
+            c.append(-1, normal(1, kept, hk, d), normal(1, kept, hk, d), torch.ones(kept, dtype=torch.uint8, device="cuda"),
+                     torch.arange(kept, dtype=torch.int32, device="cuda"))
+        outs = []
+        for t in range(3):
+            k, v, q = (shifted(normal(streams, h, d), b) for h, b in ((hk, by), (hk, 3 * by), (hq, by)))
+            ty = torch.zeros(streams, dtype=torch.uint8, device="cuda")
+            ps = torch.full((streams,), kept + t, dtype=torch.int32, device="cuda")
+            out = shifted(torch.zeros_like(q), 2 * by)
+            if streams == 1:
+                caches[0].decode_step(0, k, v, ty, ps, q, out)
+            else:
+                binding.decode_step_batched(caches, 0, k, v, ty, ps, q, out)
+            outs.append(out.clone())
+        assert all(c.status() == binding.OK for c in caches)
+        return torch.stack(outs).view(torch.int16)
+
+    want = run(0)
+    assert torch.equal(run(1), want) and want.any()

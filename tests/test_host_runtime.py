@@ -1,0 +1,85 @@
+"""The library's host side (argument checks, routes, failing calls) on a stand-in for the CUDA runtime: no GPU, nothing runs."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+# What every test program starts with: the library over the stand-in, a one-stream cache, and short calls.  Pointers are
+# made-up numbers: the host side never follows them.
+PRELUDE = """
+import ctypes as C, sys
+fake = C.CDLL(sys.argv[1], mode=C.RTLD_GLOBAL)
+lib = C.CDLL(sys.argv[2])
+fake.fake_log.restype = C.c_char_p
+fake.fake_alloc_limit.argtypes = [C.c_size_t]
+OK, ARG, CAPACITY, ORDER, CUDA = 0, -1, -2, -3, -4
+P = 1 << 20
+vp = C.c_void_p
+
+def new(layers=1, hk=4, d=128, sink=4, vw=1000, tw=100, capacity=1500):
+    h = vp()
+    assert lib.svlm_cache_create(C.byref(h), layers, hk, d, sink, vw, tw, capacity) == OK
+    return h
+
+def append(c, n, layer=0, K=P, V=P):
+    return lib.svlm_cache_append(c, layer, vp(K), vp(V), vp(P), vp(P), n)
+
+def attend(c, n, hq=28, layer=0, Q=P, out=P, pos=P):
+    return lib.svlm_attend(c, layer, vp(Q), vp(pos), n, hq, vp(out))
+
+def step(c, hq=28, layer=0, K=P, V=P, Q=P, out=P):
+    return lib.svlm_decode_step(c, layer, vp(K), vp(V), vp(P), vp(P), vp(Q), hq, vp(out))
+
+def arr(caches):
+    return (vp * len(caches))(*caches)
+
+def ran():
+    return fake.fake_log().decode().splitlines()
+"""
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    from paper_2510_09608_b200 import build
+    fake = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.check_call(["g++", "-shared", "-fPIC", "-O1", "-I/usr/local/cuda/include", "-o", fake, os.path.join(ROOT, "tests", "fake_cudart.cpp")])
+    lib = build.build()
+
+    def run(body):
+        res = subprocess.run([sys.executable, "-c", PRELUDE + body, fake, lib], capture_output=True, text=True, timeout=120)
+        assert res.returncode == 0, res.stdout + res.stderr
+        return res.stdout
+    return run
+
+
+def test_alignment_of_device_pointers(host):
+    """One token's rows may begin at any element and its output at any word; chunks want 16 bytes; what is refused launches nothing."""
+    host("""
+c = new()
+assert append(c, 40) == OK
+ran()
+for kw in (dict(K=P + 8), dict(V=P + 2)):
+    assert append(c, 40, **kw) == ARG
+for kw in (dict(Q=P + 2), dict(out=P + 8), dict(pos=P + 2)):
+    assert attend(c, 40, **kw) == ARG
+for kw in (dict(Q=P + 1), dict(out=P + 2), dict(K=P + 3), dict(V=P + 1)):
+    assert step(c, **kw) == ARG
+assert attend(c, 1, out=P + 2) == ARG and attend(c, 1, Q=P + 1) == ARG
+two = arr([c, new()])
+assert append(two[1], 40) == OK
+ran()
+call = lambda Q, out: lib.svlm_decode_step_batched(two, 2, 0, vp(P), vp(P), vp(P), vp(P), vp(Q), 28, vp(out))
+assert call(P + 1, P) == ARG and call(P, P + 2) == ARG
+n = (C.c_int32 * 2)(3, 4)
+assert lib.svlm_attend_batched_varlen(two, 2, 0, vp(P + 2), vp(P), n, 28, vp(P)) == ARG
+assert lib.svlm_attend_decode_noalloc(c, 0, vp(P), vp(P), 28, vp(P + 2)) == ARG
+assert ran() == []
+assert step(c, K=P + 2, V=P + 6, Q=P + 2, out=P + 4) == OK and attend(c, 1, Q=P + 2, out=P + 4) == OK
+assert call(P + 2, P + 4) == OK
+assert lib.svlm_attend_decode_noalloc(c, 0, vp(P + 2), vp(P), 28, vp(P + 4)) == OK
+wide = new(hk=1, capacity=70000)                    # more pages than the fast kernels' lists: the general kernel, element by element
+assert append(wide, 40) == OK and attend(wide, 40, hq=4, Q=P + 2, out=P + 2) == OK and attend(wide, 1, hq=9, Q=P + 2, out=P + 2) == OK
+""")
