@@ -1335,7 +1335,6 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
         else
             e = words ? go(decode_layer_kernel<64, false>, smem64, svlm_allow_smem<decode_layer_kernel<64, false>>(smem64))
                       : go(decode_layer_kernel<64, true>, smem64, svlm_allow_smem<decode_layer_kernel<64, true>>(smem64));
-        if (e != cudaSuccess) return e;
     } else if (b.head_dim == 128) {
         e = svlm_allow_smem<decode_stream_kernel<128>>(decode_stream_smem<128>());
         if (e != cudaSuccess) return e;
@@ -1350,5 +1349,6 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
                                early_loads);
     }
     svlm_count_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
+    const cudaError_t last = cudaGetLastError();
+    return e != cudaSuccess ? e : last;
 }

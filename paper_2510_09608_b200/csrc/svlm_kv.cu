@@ -206,17 +206,17 @@ cudaError_t svlm_launch_kv_write(const SvlmCacheDev& cd, int layer, const void* 
                    : svlm_launch_chained(kv_write_kernel<4>, grid, dim3(256), 0, 1, st, cd, layer, k, v, n, per, early);
 }
 
-void svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st) {
+cudaError_t svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st) {
     const int groups = cd.head_dim / 16;
     const int threads = cd.n_slots * groups;
     const int lpb = rotate_layers_per_block(cd.layers, cd.kv_heads);
     dim3 grid((threads + 255) / 256, (cd.layers + lpb - 1) / lpb);
-    svlm_launch_chained(evict_rotate_kernel<4>, grid, dim3(256), 0, 1, st, cd, lpb);
+    return svlm_launch_chained(evict_rotate_kernel<4>, grid, dim3(256), 0, 1, st, cd, lpb);
 }
 
-void svlm_launch_evict_rotate_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st) {
+cudaError_t svlm_launch_evict_rotate_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st) {
     const int threads = geom.n_slots * (geom.head_dim / 16);
     const int lpb = rotate_layers_per_block(geom.layers, geom.kv_heads);
     dim3 grid((threads + 255) / 256, (geom.layers + lpb - 1) / lpb, list.n);
-    svlm_launch_chained(evict_rotate_batch_kernel<4>, grid, dim3(256), 0, 1, st, list, lpb);
+    return svlm_launch_chained(evict_rotate_batch_kernel<4>, grid, dim3(256), 0, 1, st, list, lpb);
 }

@@ -45,7 +45,9 @@ cudaError_t svlm_launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, siz
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     svlm_count_launch();
     void* at[] = {const_cast<void*>(static_cast<const void*>(&args))...};      // (kilobytes of parameters: no copies on the way)
-    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), at);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), at);
+    if (e != cudaSuccess) cudaGetLastError();      // reported here, not to whoever asks the runtime next
+    return e;
 }
 
 // Streaming multiprocessors of the current device (looked up once per device).
@@ -61,13 +63,14 @@ inline int svlm_sm_count() {
     return n;
 }
 
-// metadata (svlm_meta.cu)
-void svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n, cudaStream_t st);
-void svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st);
+// metadata (svlm_meta.cu).  Where one of these fails, whatever was to follow it must not be launched: it would take the
+// metadata of the operation before for its own.
+cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n, cudaStream_t st);
+cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st);
 // batched forms, one block per cache: types [n_caches][n], pos [n_caches][n](x3); every cache has the geometry of geom
-void svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, const unsigned char* types, const int* pos, int n,
+cudaError_t svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, const unsigned char* types, const int* pos, int n,
                                    cudaStream_t st);
-void svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
+cudaError_t svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
 
 // small transfers from and to page-locked host memory (svlm_host_io.cu); 16-byte aligned, sizes rounded up to 16
 cudaError_t svlm_launch_host_in(void* dst, const void* src, size_t bytes, cudaStream_t st);
@@ -77,9 +80,9 @@ cudaError_t svlm_launch_host_out(void* dst, const void* src, size_t bytes, unsig
 // layer < 0: K,V are [layers][n][kv_heads][d]; otherwise [n][kv_heads][d] for that layer.
 // early != 0: the caller vouches that no kernel still running when this one may start writes the cache's metadata.
 cudaError_t svlm_launch_kv_write(const SvlmCacheDev& cd, int layer, const void* K, const void* V, int n, int early, cudaStream_t st);
-void svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st);
+cudaError_t svlm_launch_evict_rotate(const SvlmCacheDev& cd, cudaStream_t st);
 // every cache of the list has the geometry of geom
-void svlm_launch_evict_rotate_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
+cudaError_t svlm_launch_evict_rotate_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
 
 // attention (svlm_attend_simple.cu)
 // Q, out: [n_caches][n_layers][n_q][q_heads][d]; q_pos: [n_caches][n_q](x3)

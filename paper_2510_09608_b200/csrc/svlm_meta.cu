@@ -829,27 +829,27 @@ int append_threads(int form, int n) {
 
 }  // namespace
 
-void svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, const unsigned char* types, const int* pos, int n,
+cudaError_t svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, const unsigned char* types, const int* pos, int n,
                                    cudaStream_t st) {
     const int form = append_form_of(n, geom.n_pages);
     auto* kernel = form == APPEND_ONE ? append_meta_batch_kernel<APPEND_ONE> : form == APPEND_FEW ? append_meta_batch_kernel<APPEND_FEW> : append_meta_batch_kernel<APPEND_ANY>;
-    svlm_launch_chained(kernel, dim3(list.n), dim3(append_threads(form, n)), 0, 1, st, list, types, pos, n);
+    return svlm_launch_chained(kernel, dim3(list.n), dim3(append_threads(form, n)), 0, 1, st, list, types, pos, n);
 }
 
-void svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st) {
+cudaError_t svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st) {
     int c = evict_cluster(geom.n_slots);            // (the caches share the number of pages, not the exact capacity)
     while (c > 1 && c * list.n > 96) c /= 2;        // 16 clusters of 8 do not find room at once (a CTA fills an SM)
-    svlm_launch_chained(evict_meta_batch_kernel, dim3(c * list.n), dim3(META_THREADS), 0, c, st, list);
+    return svlm_launch_chained(evict_meta_batch_kernel, dim3(c * list.n), dim3(META_THREADS), 0, c, st, list);
 }
 
-void svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n,
+cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n,
                              cudaStream_t st) {
     const int form = append_form_of(n, cd.n_pages);
     auto* kernel = form == APPEND_ONE ? append_meta_kernel<APPEND_ONE> : form == APPEND_FEW ? append_meta_kernel<APPEND_FEW> : append_meta_kernel<APPEND_ANY>;
-    svlm_launch_chained(kernel, dim3(1), dim3(append_threads(form, n)), 0, 1, st, cd, types, pos, n);
+    return svlm_launch_chained(kernel, dim3(1), dim3(append_threads(form, n)), 0, 1, st, cd, types, pos, n);
 }
 
-void svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st) {
+cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st) {
     const int c = evict_cluster(cd.capacity);
-    svlm_launch_chained(evict_meta_kernel, dim3(c), dim3(META_THREADS), 0, c, st, cd);
+    return svlm_launch_chained(evict_meta_kernel, dim3(c), dim3(META_THREADS), 0, c, st, cd);
 }

@@ -484,7 +484,7 @@ int svlm_cache_append(svlm_cache* c, int layer, const void* K, const void* V, co
         if (!token_type || !pos) return SVLM_ERR_ARG;
         if (n > c->dev.capacity) return SVLM_ERR_CAPACITY;
         c->configured_locked = true;
-        svlm_launch_append_meta(c->dev, token_type, pos, n, c->stream);
+        SVLM_CUDA(svlm_launch_append_meta(c->dev, token_type, pos, n, c->stream));
         note_append(c, n);
     } else if (n != c->pending_n) {
         return SVLM_ERR_ORDER;
@@ -512,7 +512,7 @@ int svlm_qkv_append(svlm_cache* c, int layer, const void* X, const void* W, int 
         if (!token_type || !pos) return SVLM_ERR_ARG;
         if (n > c->dev.capacity) return SVLM_ERR_CAPACITY;
         c->configured_locked = true;
-        svlm_launch_append_meta(c->dev, token_type, pos, n, c->stream);
+        SVLM_CUDA(svlm_launch_append_meta(c->dev, token_type, pos, n, c->stream));
         note_append(c, n);
     } else if (n != c->pending_n) {
         return SVLM_ERR_ORDER;
@@ -549,10 +549,9 @@ int svlm_cache_evict(svlm_cache* c) {
     if (!c) return SVLM_ERR_ARG;
     DeviceGuard guard(c->device);
     c->last_decode_layer = -1;
+    SVLM_CUDA(svlm_launch_evict_meta(c->dev, c->stream));
     note_evict(c);
-    svlm_launch_evict_meta(c->dev, c->stream);
-    if (c->dev.contiguous) svlm_launch_evict_rotate(c->dev, c->stream);
-    SVLM_CUDA(cudaGetLastError());
+    if (c->dev.contiguous) SVLM_CUDA(svlm_launch_evict_rotate(c->dev, c->stream));
     return SVLM_OK;
 }
 
@@ -565,12 +564,11 @@ int svlm_cache_evict_batched(svlm_cache* const* caches, int n_caches) {
     bool rotate = false;
     for (int i = 0; i < n_caches; ++i) {
         caches[i]->last_decode_layer = -1;
-        note_evict(caches[i]);
         rotate = rotate || caches[i]->dev.contiguous;   // a cache with native positions never sets evict_moved
     }
-    svlm_launch_evict_meta_batch(list, c0->dev, c0->stream);
-    if (rotate) svlm_launch_evict_rotate_batch(list, c0->dev, c0->stream);
-    SVLM_CUDA(cudaGetLastError());
+    SVLM_CUDA(svlm_launch_evict_meta_batch(list, c0->dev, c0->stream));
+    for (int i = 0; i < n_caches; ++i) note_evict(caches[i]);
+    if (rotate) SVLM_CUDA(svlm_launch_evict_rotate_batch(list, c0->dev, c0->stream));
     return SVLM_OK;
 }
 
@@ -591,7 +589,7 @@ int svlm_decode_step(svlm_cache* c, int layer, const void* K, const void* V, con
         if (!token_type) return SVLM_ERR_ARG;
         c->configured_locked = true;
         c->last_decode_layer = -1;
-        svlm_launch_append_meta(c->dev, token_type, pos, 1, c->stream);
+        SVLM_CUDA(svlm_launch_append_meta(c->dev, token_type, pos, 1, c->stream));
         note_append(c, 1);
     } else if (c->pending_n != 1) {
         return SVLM_ERR_ORDER;
@@ -616,9 +614,9 @@ int svlm_decode_step_batched(svlm_cache* const* caches, int n_caches, int layer,
             svlm_cache* c = caches[i];
             c->configured_locked = true;
             c->last_decode_layer = -1;
-            note_append(c, 1);
         }
-        svlm_launch_append_meta_batch(list, c0->dev, token_type, pos, 1, c0->stream);
+        SVLM_CUDA(svlm_launch_append_meta_batch(list, c0->dev, token_type, pos, 1, c0->stream));
+        for (int i = 0; i < n_caches; ++i) note_append(caches[i], 1);
     } else {
         for (int i = 0; i < n_caches; ++i)
             if (caches[i]->pending_n != 1) return SVLM_ERR_ORDER;

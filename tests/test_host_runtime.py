@@ -83,3 +83,25 @@ assert lib.svlm_attend_decode_noalloc(c, 0, vp(P + 2), vp(P), 28, vp(P + 4)) == 
 wide = new(hk=1, capacity=70000)                    # more pages than the fast kernels' lists: the general kernel, element by element
 assert append(wide, 40) == OK and attend(wide, 40, hq=4, Q=P + 2, out=P + 2) == OK and attend(wide, 1, hq=9, Q=P + 2, out=P + 2) == OK
 """)
+
+
+def test_a_failed_metadata_launch_ends_the_call(host):
+    """Nothing that relies on the metadata is launched behind it, the host's counts stay, and the error is the call's alone."""
+    host("""
+c, d = new(layers=2), new(layers=2)
+both = arr([c, d])
+qkv = lambda: lib.svlm_qkv_append(c, 0, vp(P), vp(P), 128, 28, vp(P), vp(P), 40, vp(P))
+steps = lambda: lib.svlm_decode_step_batched(both, 2, 0, vp(P), vp(P), vp(P), vp(P), vp(P), 28, vp(P))
+for x in (c, d):
+    assert append(x, 40) == OK
+ran()
+fake.fake_fail(b"append_meta")
+for call in (lambda: append(c, 40), lambda: append(c, 40, layer=-1), qkv, lambda: step(c), steps):
+    assert call() == CUDA and ran() == [] and fake.cudaGetLastError() == 0
+    assert attend(c, 41) == ORDER and append(c, 40, layer=1) == OK       # the host still reckons with the first 40 tokens
+    ran()
+fake.fake_fail(b"evict_meta")
+assert lib.svlm_cache_evict(c) == CUDA and lib.svlm_cache_evict_batched(both, 2) == CUDA and ran() == [] and fake.cudaGetLastError() == 0
+fake.fake_fail(b"")
+assert append(c, 40) == OK and steps() == OK and lib.svlm_cache_evict(c) == OK
+""")
