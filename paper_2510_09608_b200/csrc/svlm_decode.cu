@@ -493,9 +493,9 @@ __device__ __forceinline__ int sw_off(int key, int chunk) {
 
 template <int D>
 __global__ void __launch_bounds__(DEC_THREADS, 2)
-decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t* __restrict__ Q,
-              const int* __restrict__ q_pos, int q_heads, uint16_t* __restrict__ out, int splits,
-              const uint16_t* __restrict__ Knew, const uint16_t* __restrict__ Vnew, int early_loads) {
+decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t* Q,
+              const int* q_pos, int q_heads, uint16_t* __restrict__ out, int splits,
+              const uint16_t* Knew, const uint16_t* Vnew, int early_loads) {
     constexpr int KB = D / 64;                       // 64-dim panels per row
     constexpr int PANEL_BYTES = SUB * 128;
     constexpr int STAGE_BYTES = 2 * KB * PANEL_BYTES;   // K panels then V panels
@@ -531,10 +531,10 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
     // kernel (whatever that kernel's own trigger), not merely behind one that has been launched.
     if (!early_loads) pdl_wait();
     pdl_launch_dependents();
-    const int n_tiles = min(__ldcg(&vw.ctrl->n_tiles), DEC_MAX_TILES);
-    const unsigned wait_limit = __ldcg(&vw.ctrl->wait_limit);
+    const int n_tiles = min(ld_l2(&vw.ctrl->n_tiles), DEC_MAX_TILES);
+    const unsigned wait_limit = ld_l2(&vw.ctrl->wait_limit);
     for (int i = threadIdx.x; i < n_tiles; i += DEC_THREADS) {
-        const int4 tl = __ldcg(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
+        const int4 tl = ld_l2(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
         sh.tile_pk[i] = (unsigned)tl.x | ((unsigned)tl.y << 16) | ((unsigned)tl.z << 24);
     }
     if (early_loads && threadIdx.x < 3) {
@@ -547,12 +547,12 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
         for (int o = 0; o < bytes; o += 128)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p) + o));
     }
-    const long long shift = __ldcg(&vw.ctrl->shift_total);
+    const long long shift = ld_l2(&vw.ctrl->shift_total);
     // the new token of a fused step: where it lives and whether it is still stored there
     int new_slot = -1;
     if (Knew && warp < DEC_CWARPS) {
-        const int s = __ldcg(vw.new_slot);
-        if (__ldcg(&vw.ctrl->append_n) == 1 && __ldcg(vw.slot_gid + s) == __ldcg(&vw.ctrl->n_total) - 1) new_slot = s;
+        const int s = ld_l2(vw.new_slot);
+        if (ld_l2(&vw.ctrl->append_n) == 1 && ld_l2(vw.slot_gid + s) == ld_l2(&vw.ctrl->n_total) - 1) new_slot = s;
     }
     __syncthreads();
 
@@ -621,12 +621,12 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
             if (new_slot >= 0) {
                 // fused step: the query is the appended token, its position is already in the metadata,
                 // so the rotation factors do not have to wait for the previous kernel
-                cs = svlm_rope_cs(tab, HALF, pair, __ldcg(vw.slot_c + (size_t)axis * b.n_slots + new_slot), b.theta[pair]);
+                cs = svlm_rope_cs(tab, HALF, pair, ld_l2(vw.slot_c + (size_t)axis * b.n_slots + new_slot), b.theta[pair]);
                 if (early_loads) pdl_wait();
             } else {
                 if (early_loads) pdl_wait();
                 const int* qp = q_pos + (size_t)ci * (b.rope_mode == 0 ? 1 : 3);
-                cs = svlm_rope_cs(tab, HALF, pair, (long long)qp[b.rope_mode == 0 ? 0 : axis] - shift, b.theta[pair]);
+                cs = svlm_rope_cs(tab, HALF, pair, (long long)ld_in(qp + (b.rope_mode == 0 ? 0 : axis)) - shift, b.theta[pair]);
             }
             constexpr int HSTEP = (DEC_CWARPS * 32) / HALF, HN = (8 + HSTEP - 1) / HSTEP;   // heads per thread
             uint16_t qx[HN], qy[HN];
@@ -637,15 +637,15 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
             uint16_t kx = 0, ky = 0, vx = 0, vy = 0;
             if (prep_new) {
                 const size_t noff = ((size_t)prob * b.kv_heads + hk) * D;
-                kx = Knew[noff + pair]; ky = Knew[noff + pair + HALF];
-                vx = Vnew[noff + pair]; vy = Vnew[noff + pair + HALF];
+                kx = ld_in(Knew + noff + pair); ky = ld_in(Knew + noff + pair + HALF);
+                vx = ld_in(Vnew + noff + pair); vy = ld_in(Vnew + noff + pair + HALF);
             }
 #pragma unroll
             for (int k = 0; k < HN; ++k) {      // all loads first: one round trip
                 const int h = threadIdx.x / HALF + k * HSTEP;
                 const size_t off = (((size_t)prob) * q_heads + hk * G + (h < G ? h : 0)) * D;   // n_q = 1
-                qx[k] = Q[off + pair];
-                qy[k] = Q[off + pair + HALF];
+                qx[k] = ld_in(Q + off + pair);
+                qy[k] = ld_in(Q + off + pair + HALF);
             }
 #pragma unroll
             for (int k = 0; k < HN; ++k) {
@@ -838,9 +838,9 @@ __device__ __forceinline__ int lay_off(int key, int chunk) {
 // ANYWHERE: Q, Knew or Vnew does not begin at a word (a choice inside the kernel cost 4 % of a layer-step).
 template <int D, bool ANYWHERE>
 __global__ void __launch_bounds__(LAY_THREADS, 2)
-decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q, const int* __restrict__ q_pos, int q_heads,
-                    uint16_t* __restrict__ out, int splits, const uint16_t* __restrict__ Knew,
-                    const uint16_t* __restrict__ Vnew, int early_loads TRACE_PARAM) {
+decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* q_pos, int q_heads,
+                    uint16_t* __restrict__ out, int splits, const uint16_t* Knew,
+                    const uint16_t* Vnew, int early_loads TRACE_PARAM) {
     if (threadIdx.x == 0) STAMP(0);                  // kernel entry
     constexpr int CH = D / 8;                        // 16-byte chunks per row
     constexpr int ITEM_BYTES = UNIT * D * 2;         // K or V of one unit
@@ -868,9 +868,9 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
     // kernel (whatever that kernel's own trigger), not merely behind one that has been launched.
     if (!early_loads) pdl_wait();
     pdl_launch_dependents();
-    const int n_tiles = min(__ldcg(&vw.ctrl->n_tiles), DEC_MAX_TILES);
+    const int n_tiles = min(ld_l2(&vw.ctrl->n_tiles), DEC_MAX_TILES);
     for (int i = threadIdx.x; i < n_tiles; i += LAY_THREADS) {
-        const int4 tl = __ldcg(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
+        const int4 tl = ld_l2(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
         sh.tile_pk[i] = (unsigned)tl.x | ((unsigned)tl.y << 16) | ((unsigned)tl.z << 24);
     }
     if (early_loads && warp == DEC_CWARPS - 1 && lane < 3) {
@@ -883,13 +883,13 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
         for (int o = 0; o < bytes; o += 128)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p) + o));
     }
-    if (threadIdx.x == 0) sh.wait_limit = (int)min(__ldcg(&vw.ctrl->wait_limit), 0x7fffffffu);
-    const long long shift = __ldcg(&vw.ctrl->shift_total);
+    if (threadIdx.x == 0) sh.wait_limit = (int)min(ld_l2(&vw.ctrl->wait_limit), 0x7fffffffu);
+    const long long shift = ld_l2(&vw.ctrl->shift_total);
     // the new token of a fused step: where it lives and whether it is still stored there
     int new_slot = -1;
     if (Knew) {
-        const int s = __ldcg(vw.new_slot);
-        if (__ldcg(&vw.ctrl->append_n) == 1 && __ldcg(vw.slot_gid + s) == __ldcg(&vw.ctrl->n_total) - 1) new_slot = s;
+        const int s = ld_l2(vw.new_slot);
+        if (ld_l2(&vw.ctrl->append_n) == 1 && ld_l2(vw.slot_gid + s) == ld_l2(&vw.ctrl->n_total) - 1) new_slot = s;
     }
     __syncthreads();
     if (threadIdx.x == 0) STAMP(1);                  // page list in shared memory
@@ -1016,8 +1016,8 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
         for (int e = 0; e < 2; ++e) {
             const int pair = 2 * p2 + e;
             const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
-            const long long c = new_slot >= 0 ? (long long)__ldcg(vw.slot_c + (size_t)axis * b.n_slots + new_slot)
-                                              : (long long)q_pos[b.rope_mode == 0 ? ci : 3 * ci + axis] - shift;
+            const long long c = new_slot >= 0 ? (long long)ld_l2(vw.slot_c + (size_t)axis * b.n_slots + new_slot)
+                                              : (long long)ld_in(q_pos + (b.rope_mode == 0 ? ci : 3 * ci + axis)) - shift;
             const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
             f[e] = svlm_rope_cs_batched(tab, HALF, pair, (int)c);
             if (__builtin_expect(c <= -65536 || c >= 65536, 0)) f[e] = svlm_rope_cs(tab, HALF, pair, c, b.theta[pair]);
@@ -1025,7 +1025,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
         if (new_slot >= 0 && early_loads) pdl_wait();
         if (threadIdx.x == 0) STAMP(3);              // the previous kernel has completed
         unsigned ep = 0;                             // the KV head's epoch (same round trip as the query)
-        if (threadIdx.x == 0) ep = __ldcg(epoch);
+        if (threadIdx.x == 0) ep = ld_l2(epoch);
         auto rotate2 = [&](unsigned& lo, unsigned& hi) {
             const float x0 = __uint_as_float(lo << 16), x1 = __uint_as_float(lo & 0xffff0000u);
             const float y0 = __uint_as_float(hi << 16), y1 = __uint_as_float(hi & 0xffff0000u);
@@ -1033,7 +1033,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* __restrict__ Q
             hi = pack_bf16(y0 * f[0].x + x0 * f[0].y, y1 * f[1].x + x1 * f[1].y);
         };
         auto two = [](const uint16_t* p) {           // two neighbouring elements
-            return ANYWHERE ? (unsigned)p[0] | (unsigned)p[1] << 16 : *reinterpret_cast<const unsigned*>(p);
+            return ANYWHERE ? (unsigned)ld_in(p) | (unsigned)ld_in(p + 1) << 16 : ld_in(reinterpret_cast<const unsigned*>(p));
         };
         unsigned lo[HN], hi[HN];
 #pragma unroll

@@ -52,7 +52,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
 }
 
 // parts: stages per group of eight rows; ks: elements of K per stage (a multiple of 64; the last part may be shorter)
-__global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16_t* __restrict__ X, const uint16_t* __restrict__ W,
+__global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16_t* X, const uint16_t* __restrict__ W,
                                                                  uint16_t* __restrict__ Y, int n, int in_dim, int out_dim, int parts,
                                                                  int ks, SvlmCtrl* ctrl) {
     using namespace svlm_ptx;
@@ -98,11 +98,11 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         for (size_t o = (size_t)threadIdx.x * 2048; o < bytes; o += GT_WARPS * 32 * 2048)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p + o), "r"((unsigned)min((size_t)2048, bytes - o)) : "memory");
     }
-    const unsigned wait_limit = __ldcg(&ctrl->wait_limit);                  // written at creation only, never by a kernel
+    const unsigned wait_limit = ld_l2(&ctrl->wait_limit);                  // written at creation only, never by a kernel
     pdl_wait();
     const int row16 = in_dim / 8;                                           // 16-byte chunks of a token row
     for (int i = threadIdx.x; i < n * row16; i += GT_WARPS * 32)
-        *reinterpret_cast<uint4*>(sx + (size_t)(i / row16) * GT_PAD + (size_t)i * 8) = __ldcg(reinterpret_cast<const uint4*>(X) + i);
+        *reinterpret_cast<uint4*>(sx + (size_t)(i / row16) * GT_PAD + (size_t)i * 8) = ld_l2(reinterpret_cast<const uint4*>(X) + i);
     __syncthreads();
     const bool live = g < n;
     const uint16_t* xrow = sx + (size_t)min(g, n - 1) * (in_dim + GT_PAD) + kq * 8;
@@ -199,7 +199,7 @@ bool few_supported(int n, int in_dim) {
 // in flight; the warps' partial tiles meet in shared memory.
 constexpr int GM_KB_IN_FLIGHT = 7;
 
-__global__ void __launch_bounds__(GV_THREADS) gemv_mma_kernel(const uint16_t* __restrict__ X, const uint16_t* __restrict__ W,
+__global__ void __launch_bounds__(GV_THREADS, 4) gemv_mma_kernel(const uint16_t* X, const uint16_t* __restrict__ W,
                                                              uint16_t* __restrict__ Y, int n, int in_dim, int out_dim) {
     __shared__ float part[GV_THREADS / 32][16][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(GV_THREADS) gemv_mma_kernel(const uint16_t* __
         for (int u = 0; u < GM_KB_IN_FLIGHT; ++u) {
             const int kb = kb0 + u * (GV_THREADS / 32);
             const bool live = kb < n_kb;
-            a[u] = live && lo_live ? __ldg(xlo + 4 * kb) : make_uint4(0, 0, 0, 0);
-            bq[u] = live && hi_live ? __ldg(xhi + 4 * kb) : make_uint4(0, 0, 0, 0);
+            a[u] = live && lo_live ? svlm_ptx::ld_in(xlo + 4 * kb) : make_uint4(0, 0, 0, 0);
+            bq[u] = live && hi_live ? svlm_ptx::ld_in(xhi + 4 * kb) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
         for (int u = 0; u < GM_KB_IN_FLIGHT; ++u) {

@@ -13,7 +13,7 @@ namespace {
 constexpr int IO_THREADS = 256;
 
 // host -> device, 16 bytes per thread; .cv: what the host wrote since the last time must be seen
-__global__ void __launch_bounds__(IO_THREADS) host_in_kernel(uint4* __restrict__ dst, const uint4* __restrict__ src, int n16) {
+__global__ void __launch_bounds__(IO_THREADS) host_in_kernel(uint4* __restrict__ dst, const uint4* src, int n16) {
     svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();
     const int i = blockIdx.x * IO_THREADS + threadIdx.x;
@@ -22,11 +22,11 @@ __global__ void __launch_bounds__(IO_THREADS) host_in_kernel(uint4* __restrict__
 
 // device -> host, then the ticket that the host is waiting for (also without anything to copy: everything before this
 // kernel in the stream is complete then)
-__global__ void __launch_bounds__(IO_THREADS) host_out_kernel(uint4* __restrict__ dst, const uint4* __restrict__ src, int n16, volatile unsigned* done,
+__global__ void __launch_bounds__(IO_THREADS) host_out_kernel(uint4* __restrict__ dst, const uint4* src, int n16, volatile unsigned* done,
                                                              unsigned ticket) {
     svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();
-    for (int i = threadIdx.x; i < n16; i += IO_THREADS) dst[i] = __ldcg(src + i);
+    for (int i = threadIdx.x; i < n16; i += IO_THREADS) dst[i] = svlm_ptx::ld_l2(src + i);
     __threadfence_system();
     __syncthreads();
     if (threadIdx.x == 0) *done = ticket;

@@ -12,6 +12,7 @@
 namespace {
 
 struct __align__(16) Bf16x8 { __nv_bfloat162 v[4]; };
+__device__ __forceinline__ Bf16x8 bf16x8(const uint4& x) { return reinterpret_cast<const Bf16x8&>(x); }
 
 // Rotate 8 consecutive pairs (lo[j], hi[j]) by (cs[j], sn[j]) in fp32, round to bf16.
 __device__ __forceinline__ void rotate8(Bf16x8& lo, Bf16x8& hi, const float* cs, const float* sn) {
@@ -36,8 +37,8 @@ __device__ __forceinline__ void rotate8(Bf16x8& lo, Bf16x8& hi, const float* cs,
 // (programmatic dependent launch), which leaves one round trip to memory after it.  Per layer of a 524-token chunk
 // between two chunk-prefill launches: 14 us in the stream with 17 blocks, a longer chain and a full launch gap.
 template <int UNROLL>
-__global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int layer, const uint16_t* __restrict__ K,
-                                                       const uint16_t* __restrict__ V, int n, int rows_per_block, int early) {
+__global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int layer, const uint16_t* K,
+                                                       const uint16_t* V, int n, int rows_per_block, int early) {
     if (!early) svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();    // (after the wait: a successor's early reads must find all earlier work done)
     const int half = cd.head_dim / 2;
@@ -61,25 +62,25 @@ __global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int laye
         for (int u = 0; u < UNROLL; ++u)
             if (live && r + u < row1) {
                 const size_t src = src_of(r + u);
-                lo[u] = *reinterpret_cast<const Bf16x8*>(K + src);
-                hi[u] = *reinterpret_cast<const Bf16x8*>(K + src + half);
-                vlo[u] = *reinterpret_cast<const uint4*>(V + src);
-                vhi[u] = *reinterpret_cast<const uint4*>(V + src + half);
+                lo[u] = bf16x8(svlm_ptx::ld_in(reinterpret_cast<const uint4*>(K + src)));
+                hi[u] = bf16x8(svlm_ptx::ld_in(reinterpret_cast<const uint4*>(K + src + half)));
+                vlo[u] = svlm_ptx::ld_in(reinterpret_cast<const uint4*>(V + src));
+                vhi[u] = svlm_ptx::ld_in(reinterpret_cast<const uint4*>(V + src + half));
             }
     };
     if (!early) load_rows(row0);
-    const int append_n = __ldcg(&cd.ctrl->append_n);
-    const long long n_total = __ldcg(&cd.ctrl->n_total);
-    int slot = live ? __ldcg(cd.new_slot + i) : -1;      // (of an append that was dropped: left over, not used)
+    const int append_n = svlm_ptx::ld_l2(&cd.ctrl->append_n);
+    const long long n_total = svlm_ptx::ld_l2(&cd.ctrl->n_total);
+    int slot = live ? svlm_ptx::ld_l2(cd.new_slot + i) : -1;      // (of an append that was dropped: left over, not used)
     float cs[8], sn[8];
     if (slot >= 0) {
         // A layer's keys may arrive after an eviction has already shifted these tokens (layers are
         // computed one after another): rotate at the slot's CURRENT position, and skip a token that
         // the eviction has dropped in the meantime.
-        const long long gid = __ldcg(cd.slot_gid + slot);
+        const long long gid = svlm_ptx::ld_l2(cd.slot_gid + slot);
         int c[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) c[k] = __ldcg(cd.slot_c + (size_t)k * cd.n_slots + slot);
+        for (int k = 0; k < 3; ++k) c[k] = svlm_ptx::ld_l2(cd.slot_c + (size_t)k * cd.n_slots + slot);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int pair = g * 8 + j;

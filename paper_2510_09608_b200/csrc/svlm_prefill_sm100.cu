@@ -268,12 +268,12 @@ __device__ __forceinline__ PfAsk pf_ask(const SvlmAttendBatch& b, const PfRows& 
     PfAsk q;
     const SvlmAttendView& vw = b.view[r.ci];
     const int lane = threadIdx.x & 31, n_pages = b.n_slots / SVLM_PAGE;
-    q.n_tiles = __ldcg(&vw.ctrl->n_tiles);
-    q.n_total = __ldcg(&vw.ctrl->n_total);
-    q.shift = __ldcg(&vw.ctrl->shift_total);
-    q.wait_limit = __ldcg(&vw.ctrl->wait_limit);
+    q.n_tiles = ld_l2(&vw.ctrl->n_tiles);
+    q.n_total = ld_l2(&vw.ctrl->n_total);
+    q.shift = ld_l2(&vw.ctrl->shift_total);
+    q.wait_limit = ld_l2(&vw.ctrl->wait_limit);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) q.first[k] = __ldcg(&vw.tiles[min(lane + 32 * k, n_pages - 1)].min_gid);
+    for (int k = 0; k < 4; ++k) q.first[k] = ld_l2(&vw.tiles[min(lane + 32 * k, n_pages - 1)].min_gid);
     return q;
 }
 __device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfSeg& s, const PfRows& r, unsigned g_magic, int G, const PfAsk& q) {
@@ -288,7 +288,7 @@ __device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfSeg&
     int n_act = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) n_act += lane + 32 * k < w.n_tiles && q.first[k] <= w.gid_hi;
-    for (int j = lane + 128; j < w.n_tiles; j += 32) n_act += __ldcg(&w.vw->tiles[j].min_gid) <= w.gid_hi;
+    for (int j = lane + 128; j < w.n_tiles; j += 32) n_act += ld_l2(&w.vw->tiles[j].min_gid) <= w.gid_hi;
     n_act = __reduce_add_sync(0xffffffffu, n_act);
     w.p0 = s.a * n_act / PF_FRAC;
     w.n_proc = s.e * n_act / PF_FRAC - w.p0;
@@ -329,8 +329,8 @@ struct PfPages {
             bool vis = false;
             if (j < w.n_tiles) {
                 const SvlmTile* tp = w.vw->tiles + j;
-                const int4 a = __ldcg(reinterpret_cast<const int4*>(tp));
-                const longlong2 g = __ldcg(reinterpret_cast<const longlong2*>(&tp->min_gid));
+                const int4 a = ld_l2(reinterpret_cast<const int4*>(tp));
+                const longlong2 g = ld_l2(reinterpret_cast<const longlong2*>(&tp->min_gid));
                 vis = g.x <= w.gid_hi;
                 const unsigned causal = g.y > w.gid_q0 + r_lo, ragged = a.y > 0 || a.z < SVLM_PAGE;
                 info = (unsigned)a.x | ((unsigned)a.y << 14) | ((unsigned)(a.z - 1) << 21) | ((causal | ragged) << 28) | (causal << 29);
@@ -362,7 +362,7 @@ struct PfTileRotation {
     // element e of a row lives in block e/64, 16-byte chunk (e%64)/8, XOR-swizzled by row&7
     __device__ __forceinline__ static int at(int row, int e) { return (e / 64) * (128 * 128) + row * 128 + ((((e % 64) / 8) ^ (row & 7)) << 4); }
 
-    __device__ __forceinline__ static void load(const PfRows& w, int g, int m, int G, unsigned g_magic, int q_heads, const uint16_t* __restrict__ Q, unsigned char* sQ) {
+    __device__ __forceinline__ static void load(const PfRows& w, int g, int m, int G, unsigned g_magic, int q_heads, const uint16_t* Q, unsigned char* sQ) {
         const int c8 = m % CH;
         const uint16_t* base = Q + (w.q_row0 * q_heads + w.hk * G) * D + c8 * 8;
         const unsigned dst = smem_u32(sQ);
@@ -404,13 +404,13 @@ struct PfTileRotation {
     // 16-byte chunks are swizzled so that their halves fall into different banks
     __device__ __forceinline__ static int cs_at(int pair) { return (((pair >> 2) ^ ((pair >> 5) & 1)) << 2) | (pair & 3); }
     int c[UN];               // positions of the thread's first UN factors
-    __device__ __forceinline__ void load_pos(const SvlmAttendBatch& b, const PfRows& w, const int* __restrict__ q_pos, int m, int t_lo, int n_tok, int tk0) {
+    __device__ __forceinline__ void load_pos(const SvlmAttendBatch& b, const PfRows& w, const int* q_pos, int m, int t_lo, int n_tok, int tk0) {
         const int pw = b.rope_mode == 0 ? 1 : 3;
         const int* qp = q_pos + (w.p_row0 + t_lo) * pw + axis_of(b, m % HALF);
 #pragma unroll
-        for (int u = 0; u < UN; ++u) c[u] = __ldg(qp + (size_t)min(tk0 + u * TPT, n_tok - 1) * pw);
+        for (int u = 0; u < UN; ++u) c[u] = ld_in(qp + (size_t)min(tk0 + u * TPT, n_tok - 1) * pw);
     }
-    __device__ __forceinline__ void stage(const SvlmAttendBatch& b, const PfRows& w, long long shift, const int* __restrict__ q_pos, int m, int t_lo, int n_tok, float* s_cs) {
+    __device__ __forceinline__ void stage(const SvlmAttendBatch& b, const PfRows& w, long long shift, const int* q_pos, int m, int t_lo, int n_tok, float* s_cs) {
         const int pair = m % HALF;
         const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
         float* dst = s_cs + cs_at(pair);
@@ -440,14 +440,14 @@ struct PfTileRotation {
             const int* qp = q_pos + (w.p_row0 + t_lo) * pw + axis_of(b, pair);
 #pragma unroll 1
             for (int tk = m / HALF; tk < n_tok; tk += TPT) {
-                const float2 f = svlm_rope_cs(tab, HALF, pair, (long long)__ldg(qp + (size_t)tk * pw) - shift, b.theta[pair]);
+                const float2 f = svlm_rope_cs(tab, HALF, pair, (long long)ld_in(qp + (size_t)tk * pw) - shift, b.theta[pair]);
                 dst[(size_t)tk * 2 * HALF] = f.x;
                 dst[(size_t)tk * 2 * HALF + HALF] = f.y;
             }
         }
     }
 
-    __device__ __forceinline__ static void rotate(const SvlmAttendBatch& b, const PfRows& w, long long shift, const int* __restrict__ q_pos, int g, int m,
+    __device__ __forceinline__ static void rotate(const SvlmAttendBatch& b, const PfRows& w, long long shift, const int* q_pos, int g, int m,
                                                   unsigned g_magic, int G, int t_lo, bool from_stage, const float* s_cs, unsigned char* sQ) {
         const int c8 = m % CH;
 #pragma unroll 2
@@ -471,7 +471,7 @@ struct PfTileRotation {
                 const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
                 const int pw = b.rope_mode == 0 ? 1 : 3;
                 const int* qp = q_pos + (w.p_row0 + tk) * pw;
-                const long long p[3] = {__ldg(qp) - shift, __ldg(qp + pw / 2) - shift, __ldg(qp + pw - 1) - shift};
+                const long long p[3] = {ld_in(qp) - shift, ld_in(qp + pw / 2) - shift, ld_in(qp + pw - 1) - shift};
                 Near v[8];
                 bool far = false;
 #pragma unroll
@@ -615,7 +615,7 @@ __device__ __forceinline__ void merge_pieces(const PfPlan& plan, int tail, const
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int k = min(k0 + i, last);
-            ml[i] = k == me ? make_float2(m_own, l) : __ldcg(PfSlot<D>(plan, tail, k).ml(g, m));
+            ml[i] = k == me ? make_float2(m_own, l) : ld_l2(PfSlot<D>(plan, tail, k).ml(g, m));
             if (k0 + i > last || plan.x[k] >= plan.x[k + 1]) ml[i].x = -INFINITY;
         }
         const float Mn = fmaxf(fmaxf(M, fmaxf(ml[0].x, ml[1].x)), fmaxf(ml[2].x, ml[3].x));
@@ -647,11 +647,11 @@ __device__ __forceinline__ void merge_pieces(const PfPlan& plan, int tail, const
                 }
             } else {
                 const PfSlot<D> slot(plan, tail, k);
-                mk = __ldcg(slot.ml(g, m)).x;
+                mk = ld_l2(slot.ml(g, m)).x;
                 const float4* po = slot.o(g, m) + h * 16 * 128;
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {        // (of a piece without pages: left over from earlier, not used)
-                    const float4 v = __ldcg(po + i * 128);
+                    const float4 v = ld_l2(po + i * 128);
                     o[4 * i] = v.x; o[4 * i + 1] = v.y; o[4 * i + 2] = v.z; o[4 * i + 3] = v.w;
                 }
             }
@@ -671,7 +671,7 @@ __device__ __forceinline__ void merge_pieces(const PfPlan& plan, int tail, const
 template <int D>
 __global__ void __launch_bounds__(PF_THREADS, 1)
 prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant__ PfPlan plan, int layer0, int n_layers,
-               const uint16_t* __restrict__ Q, const int* __restrict__ q_pos, int n_q_arg, int q_heads, uint16_t* __restrict__ out) {
+               const uint16_t* Q, const int* q_pos, int n_q_arg, int q_heads, uint16_t* __restrict__ out) {
     constexpr int KB = D / 64;                 // 64-element (128-byte) blocks along d
     constexpr int TILE_BYTES = 128 * D * 2;    // one K or V page of one head, or one 128-row Q tile
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -891,7 +891,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     int end = hi;
                     if ((pi >> 29) & 1) {     // the new chunk's tokens: causal
                         const long long* gp = w.vw->slot_gid + (size_t)(pi & 0x3FFF) * SVLM_PAGE + 4 * lane;
-                        const longlong2 ga = __ldg(reinterpret_cast<const longlong2*>(gp)), gb = __ldg(reinterpret_cast<const longlong2*>(gp) + 1);
+                        const longlong2 ga = ld_in(reinterpret_cast<const longlong2*>(gp)), gb = ld_in(reinterpret_cast<const longlong2*>(gp) + 1);
                         const long long gv[4] = {ga.x, ga.y, gb.x, gb.y};
                         int v[4];
 #pragma unroll

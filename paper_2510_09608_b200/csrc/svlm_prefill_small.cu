@@ -55,8 +55,8 @@ __device__ __forceinline__ int sm_off(int key, int chunk) { return (chunk >> 3) 
 
 template <int D, int MT>
 __global__ void __launch_bounds__(32 * sm_warps<D>, 1)
-prefill_small_kernel(const __grid_constant__ SvlmAttendBatch b, int layer0, int n_layers, const uint16_t* __restrict__ Q,
-                     const int* __restrict__ q_pos, int n_q_arg, int q_heads, int parts, uint16_t* __restrict__ out) {
+prefill_small_kernel(const __grid_constant__ SvlmAttendBatch b, int layer0, int n_layers, const uint16_t* Q,
+                     const int* q_pos, int n_q_arg, int q_heads, int parts, uint16_t* __restrict__ out) {
     constexpr int ROWS = SM_TILE * MT;
     constexpr int W = sm_warps<D>, HALF = D / 2, KB = D / 64, STAGE = sm_stage_bytes<D>, V_AT = STAGE / 2;
     constexpr float c = D == 128 ? 0.12751743082459868f : 0.18033688011112042f;      // log2(e) / sqrt(D)
@@ -84,13 +84,13 @@ prefill_small_kernel(const __grid_constant__ SvlmAttendBatch b, int layer0, int 
 
     // ---- everything the prologue needs, in one round trip ----
     const int n_pages = b.n_slots / SVLM_PAGE;
-    const int n_tiles = min(__ldcg(&vw.ctrl->n_tiles), SM_MAX_TILES);
-    const long long gid_q0 = __ldcg(&vw.ctrl->n_total) - n_q, shift = __ldcg(&vw.ctrl->shift_total);
-    const unsigned wait_limit = __ldcg(&vw.ctrl->wait_limit);
+    const int n_tiles = min(ld_l2(&vw.ctrl->n_tiles), SM_MAX_TILES);
+    const long long gid_q0 = ld_l2(&vw.ctrl->n_total) - n_q, shift = ld_l2(&vw.ctrl->shift_total);
+    const unsigned wait_limit = ld_l2(&vw.ctrl->wait_limit);
     const int r_lo = m0 / G, r_hi = min(n_q - 1, (m0 + ROWS - 1) / G);
     for (int i = tid; i < n_pages && (i < (int)blockDim.x || i < n_tiles); i += blockDim.x) {     // (the first ones without waiting for their count)
-        const int4 a = __ldcg(reinterpret_cast<const int4*>(vw.tiles + i));
-        const longlong2 g = __ldcg(reinterpret_cast<const longlong2*>(&vw.tiles[i].min_gid));
+        const int4 a = ld_l2(reinterpret_cast<const int4*>(vw.tiles + i));
+        const longlong2 g = ld_l2(reinterpret_cast<const longlong2*>(&vw.tiles[i].min_gid));
         const unsigned causal = g.y > gid_q0 + r_lo, unseen = g.x > gid_q0 + r_hi;
         sh.tile[i] = (unsigned)a.x | ((unsigned)a.y << 14) | ((unsigned)(a.z - 1) << 21) | (causal << 28) | (unseen << 29);
     }
@@ -103,11 +103,11 @@ prefill_small_kernel(const __grid_constant__ SvlmAttendBatch b, int layer0, int 
     for (int u = 0; u < ITEMS; ++u) {
         const int it = min(tid + u * 32 * W, ROWS * CH - 1), mg = min(m0 + it / CH, m_total - 1), r = mg / G;
         const uint16_t* src = Q + ((q_row0 + r) * q_heads + hk * G + (mg - r * G)) * D + (it % CH) * 8;
-        lo4[u] = __ldg(reinterpret_cast<const uint4*>(src));
-        hi4[u] = __ldg(reinterpret_cast<const uint4*>(src + HALF));
+        lo4[u] = ld_in(reinterpret_cast<const uint4*>(src));
+        hi4[u] = ld_in(reinterpret_cast<const uint4*>(src + HALF));
         const int pw = b.rope_mode == 0 ? 1 : 3;
         const int* qp = q_pos + ((b.q_varlen ? (size_t)b.q_off[ci] : (size_t)ci * n_q) + r) * pw;
-        p[u][0] = __ldg(qp); p[u][1] = __ldg(qp + pw / 2); p[u][2] = __ldg(qp + pw - 1);
+        p[u][0] = ld_in(qp); p[u][1] = ld_in(qp + pw / 2); p[u][2] = ld_in(qp + pw - 1);
     }
     __syncthreads();
 
@@ -228,7 +228,7 @@ prefill_small_kernel(const __grid_constant__ SvlmAttendBatch b, int layer0, int 
         if (causal) {
             const long long* gp = vw.slot_gid + (size_t)(ti & 0x3FFF) * SVLM_PAGE + k0 + 2 * t;
 #pragma unroll
-            for (int nb = 0; nb < 4; ++nb) gid[nb] = __ldcg(reinterpret_cast<const longlong2*>(gp + nb * 8));
+            for (int nb = 0; nb < 4; ++nb) gid[nb] = ld_l2(reinterpret_cast<const longlong2*>(gp + nb * 8));
         }
         const int st = done % SM_STAGES;
         ok = mbar_wait(&full[st], (done / SM_STAGES) & 1, abort_flag, wait_limit);

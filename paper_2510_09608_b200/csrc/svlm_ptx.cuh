@@ -71,6 +71,32 @@ __device__ __forceinline__ void mma_bf16(float* c, unsigned a0, unsigned a1, uns
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// Loads of what an earlier kernel of the stream writes.  With programmatic dependent launch that kernel may still be running
+// when this one starts, so such data must not take the read-only path (ld.global.nc, which __ldg and const __restrict__
+// parameters allow: it is for data that nobody writes while the kernel runs, and the compiler may move such a load above
+// the wait).  These are volatile and stay behind pdl_wait().  ld_l2 reads past L1.
+#define SVLM_LOAD1(T, type, reg)                                                                                                  \
+    __device__ __forceinline__ T ld_in(const T* p) { T v; asm volatile("ld.global." type " %0, [%1];" : reg(v) : "l"(p) : "memory"); return v; }    \
+    __device__ __forceinline__ T ld_l2(const T* p) { T v; asm volatile("ld.global.cg." type " %0, [%1];" : reg(v) : "l"(p) : "memory"); return v; }
+#define SVLM_LOAD2(T, type, reg)                                                                                                  \
+    __device__ __forceinline__ T ld_in(const T* p) { T v; asm volatile("ld.global.v2." type " {%0, %1}, [%2];" : reg(v.x), reg(v.y) : "l"(p) : "memory"); return v; }    \
+    __device__ __forceinline__ T ld_l2(const T* p) { T v; asm volatile("ld.global.cg.v2." type " {%0, %1}, [%2];" : reg(v.x), reg(v.y) : "l"(p) : "memory"); return v; }
+#define SVLM_LOAD4(T, type, reg)                                                                                                  \
+    __device__ __forceinline__ T ld_in(const T* p) { T v; asm volatile("ld.global.v4." type " {%0, %1, %2, %3}, [%4];" : reg(v.x), reg(v.y), reg(v.z), reg(v.w) : "l"(p) : "memory"); return v; }    \
+    __device__ __forceinline__ T ld_l2(const T* p) { T v; asm volatile("ld.global.cg.v4." type " {%0, %1, %2, %3}, [%4];" : reg(v.x), reg(v.y), reg(v.z), reg(v.w) : "l"(p) : "memory"); return v; }
+SVLM_LOAD1(uint16_t, "u16", "=h")
+SVLM_LOAD1(int, "s32", "=r")
+SVLM_LOAD1(unsigned, "u32", "=r")
+SVLM_LOAD1(long long, "s64", "=l")
+SVLM_LOAD2(longlong2, "s64", "=l")
+SVLM_LOAD2(float2, "f32", "=f")
+SVLM_LOAD4(float4, "f32", "=f")
+SVLM_LOAD4(int4, "s32", "=r")
+SVLM_LOAD4(uint4, "u32", "=r")
+#undef SVLM_LOAD1
+#undef SVLM_LOAD2
+#undef SVLM_LOAD4
+
 // Programmatic dependent launch: let the next kernel in the stream start; wait for the previous one.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

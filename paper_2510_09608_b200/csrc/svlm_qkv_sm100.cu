@@ -94,7 +94,7 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     const int stage_bytes = QK_W_TILE + width / 2 * 128;
     const int n_stages = min(QK_MAX_STAGES, QK_RING / stage_bytes);
     volatile int* abort_flag = &sh.abort_flag;
-    const unsigned wait_limit = __ldcg(&cd.ctrl->wait_limit);   // written at creation only, never by a kernel
+    const unsigned wait_limit = ld_l2(&cd.ctrl->wait_limit);   // written at creation only, never by a kernel
 
     if (smem_u32(smem_raw) & 1023) {             // swizzled tiles need a 1024-byte aligned base; same in every CTA
         if (threadIdx.x == 0) atomicCAS(&cd.ctrl->status, 0, -4);   // SVLM_ERR_CUDA
@@ -179,13 +179,13 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         int slot = -1, c0 = 0, c1 = 0, c2 = 0;
         if (kv >= 0 && head < n_heads) {
             const int t = ew + QK_EPI_WARPS * lane, i = i0 + t;
-            if (t < width && i < n && __ldcg(&cd.ctrl->append_n) == n) {
-                const int s = __ldcg(cd.new_slot + i);
-                if (__ldcg(cd.slot_gid + s) == __ldcg(&cd.ctrl->n_total) - n + i) slot = s;
+            if (t < width && i < n && ld_l2(&cd.ctrl->append_n) == n) {
+                const int s = ld_l2(cd.new_slot + i);
+                if (ld_l2(cd.slot_gid + s) == ld_l2(&cd.ctrl->n_total) - n + i) slot = s;
                 if (key) {
-                    c0 = __ldcg(cd.slot_c + s);
-                    c1 = __ldcg(cd.slot_c + cd.n_slots + s);
-                    c2 = __ldcg(cd.slot_c + 2 * (size_t)cd.n_slots + s);
+                    c0 = ld_l2(cd.slot_c + s);
+                    c1 = ld_l2(cd.slot_c + cd.n_slots + s);
+                    c2 = ld_l2(cd.slot_c + 2 * (size_t)cd.n_slots + s);
                 }
             }
         }
