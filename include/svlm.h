@@ -154,6 +154,9 @@ int svlm_cache_evict(svlm_cache* c);
  * zeros.  n_q == 1 takes the split-KV decode path, n_q >= 2 the chunk-prefill path; shapes neither of
  * them is built for (more than 8 query heads per KV head at n_q == 1; a cache of more than 512 pages of 128
  * slots, i.e. a capacity beyond roughly 65,000 tokens) take a slower general kernel with the same result.
+ * Which of several kernels serves a shape follows from the sizes and from about how many tokens the cache holds as far as
+ * the host can tell (it does not see the tokens' types; a call that is captured into a CUDA graph is reckoned with full
+ * windows, since the graph runs later): the results agree to within the rounding of bf16, the bits may differ.
  * Errors: SVLM_ERR_ARG (q_heads not a multiple of kv_heads, n_q < 1, null pointers),
  * SVLM_ERR_ORDER (n_q exceeds the tokens appended so far).
  */

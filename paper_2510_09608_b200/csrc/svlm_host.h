@@ -12,7 +12,7 @@ struct svlm_cache {
     int device = 0;
     std::vector<void*> allocs;
     long long appended = 0;       // tokens accepted by the host checks so far
-    long long stored_est = 0;     // about how many tokens are stored (what the device keeps exactly); for balancing work only
+    long long stored_est = 0;     // about how many tokens are stored (what the device keeps exactly): chooses kernels, balances work
     int pending_n = 0;            // n of the latest metadata append (layers 1.. must match)
     bool configured_locked = false;
     unsigned wait_limit_host = 0;  // source buffer of svlm_debug_set_wait_limit's copy

@@ -128,7 +128,7 @@ cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int i
 bool svlm_prefill_supported(int n_pages, int group);
 // counters: svlm_prefill_counter_bytes of the first cache, zero before the first launch (the kernel leaves them zero);
 // slots: its svlm_prefill_slot_bytes (0: null).  Launches that share them must not overlap.  held: what each cache is
-// expected to hold (only the balance of the work depends on it).
+// expected to hold (the kernel and the balance of the work depend on it, the result only in the order of its sums).
 struct SvlmPrefillLoad {
     int pages;      // stored pages
     int windows;    // most tokens the windows keep, i.e. most of a chunk that can be stored

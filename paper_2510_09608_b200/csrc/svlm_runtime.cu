@@ -244,11 +244,25 @@ bool decode_aligned(const void* Q, const void* K, const void* V, const void* out
     return aligned(2, Q, K, V) && aligned(4, out, pos);
 }
 
-// The host's idea of what a cache stores (it does not know the tokens' types, nor what a replayed graph has appended).
+// The host's idea of what a cache stores: the choice between kernels and the balance of their work rest on it, never the
+// result.  It does not know the tokens' types, so a cache that has seen one type only is reckoned as long as both windows.
+long long full_windows(const svlm_cache* c) {
+    return std::min<long long>((long long)c->dev.n_sink + c->dev.vision_window + c->dev.text_window, c->dev.capacity);
+}
+// A captured call runs later and again, with more stored than now, and its appends are not seen here when they run: from the
+// first one on the cache is reckoned full.  (Captured on a nearly empty cache and replayed over 9216 keys, 28/4 heads, 133
+// tokens kept the few-rows kernel: 97 us, this way 48; 266 tokens 124 and 55.)
+void note_capture(svlm_cache* c) {
+    if (c->stored_est >= full_windows(c)) return;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+    else if (st != cudaStreamCaptureStatusNone) c->stored_est = full_windows(c);
+}
 void note_append(svlm_cache* c, int n) {
     c->meta_settled = false;
     c->appended += n;
     c->pending_n = n;
+    note_capture(c);
     c->stored_est = std::min<long long>(c->stored_est + n, c->dev.capacity);
 }
 void note_evict(svlm_cache* c) {
@@ -279,10 +293,11 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     b.n_caches = n_caches;
     fill_batch_geometry(c0, b);
     for (int i = 0; i < n_caches; ++i) {
-        const svlm_cache* c = caches[i];
+        svlm_cache* c = caches[i];
         if (!c) return SVLM_ERR_ARG;
         if (!same_geometry(c, c0)) return SVLM_ERR_ARG;
         if (n_q > c->appended) return SVLM_ERR_ORDER;
+        note_capture(c);
         fill_view(c, b.view[i]);
     }
     DeviceGuard guard(c0->device);
@@ -646,6 +661,7 @@ int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int laye
         b.q_cnt[i] = n_q[i];
         off += n_q[i];
         n_max = std::max(n_max, n_q[i]);
+        note_capture(caches[i]);
         fill_view(caches[i], b.view[i]);
         caches[i]->last_decode_layer = -1;
     }

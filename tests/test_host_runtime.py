@@ -105,3 +105,34 @@ assert lib.svlm_cache_evict(c) == CUDA and lib.svlm_cache_evict_batched(both, 2)
 fake.fake_fail(b"")
 assert append(c, 40) == OK and steps() == OK and lib.svlm_cache_evict(c) == OK
 """)
+
+
+def test_a_captured_call_is_reckoned_with_full_windows(host):
+    """A graph captured while the windows fill is replayed when they are full: the kernels are chosen for that, and so they are
+    for plain calls of the same cache afterwards, whose appends the host may not have seen."""
+    host("""
+def kernels(call):
+    ran()
+    assert call() == OK
+    return [l.split()[0] for l in ran()]
+small = lambda names: any("prefill_small" in n for n in names)
+layer = lambda names: any("decode_layer" in n for n in names)
+big = dict(hk=8, vw=12000, tw=500, capacity=13000)
+for calls in (lambda c: attend(c, 133, hq=32), lambda c: lib.svlm_attend_batched_varlen(arr([c]), 1, 0, vp(P), vp(P), (C.c_int32 * 1)(133), 32, vp(P))):
+    c = new(**big)
+    assert append(c, 133) == OK and small(kernels(lambda: calls(c)))
+    fake.fake_capturing(1)
+    assert not small(kernels(lambda: calls(c)))
+    fake.fake_capturing(0)
+    assert not small(kernels(lambda: calls(c)))
+    full = new(**big)                                    # what an ordinary stream takes when its windows are full
+    for _ in range(120):
+        assert append(full, 133) == OK and lib.svlm_cache_evict(full) == OK
+    assert not small(kernels(lambda: calls(full)))
+c = new(**big)
+assert append(c, 133) == OK and layer(kernels(lambda: step(c, hq=32)))
+fake.fake_capturing(1)
+assert append(c, 133) == OK                              # captured: the host does not see when it runs
+fake.fake_capturing(0)
+assert not layer(kernels(lambda: step(c, hq=32))) and not layer(kernels(lambda: step(full, hq=32)))
+""")
