@@ -1271,17 +1271,23 @@ size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits) {
 }
 
 // The per-layer kernel holds one round of a CTA's keys and values on chip before the query comes and the next in L2; with a
-// third round it is only a slower streaming kernel where a KV head has few CTAs (head size 128, us per layer-step: 8 heads
-// of 16,900 keys 22.9 against 20.5, with two rounds 10.1 against 11.8; 4 heads of 24,300 keys, whose 37 CTAs the streaming
-// kernel's last CTA combines alone, 17.1 against 18.2; head size 64, half the bytes, is better here at any length).
+// third round it is only a slower streaming kernel where a KV head has few CTAs and the keys come from HBM (8 heads of 128, us
+// per layer-step, streaming against per-layer: 6 layers of 10,500 keys 14.2 against 15.0, of 17,000 18.9 against 20.8; with
+// two rounds 11.8 against 10.1).  It stays the better one where the cache's keys and values remain in L2 from token to token,
+// most of its 126 MB (one layer of 13,000 keys 18.2 against 15.6, of 17,000 20.7 against 17.8; two of 10,500, 86 MB, 14.7
+// against 14.2, of 13,000, 107 MB, 16.8 against 17.2), with more CTAs (4 heads of 24,300 keys, whose 37 CTAs the streaming
+// kernel's last CTA combines alone, 18.2 against 17.1) and for head size 64, half the bytes.
 // Two streams of 9,216 keys: 10.9 against 13.0, of 3,072: 7.7 against 11.3.  Its CTAs wait for one another's partial
 // results, so several caches take it only while all CTAs fit the SMs, one each, and while a KV head has enough of them to
 // share the combine (8 caches of 4 heads, 4 CTAs a head: 13.5 against 11.5; 3 caches, 12 CTAs a head: 8.9 against 10.3 with
 // one round, 13.7 against 12.7 with two).
-int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches, int head_dim) {
+int svlm_decode_layer_splits(int n_pages, int pages, int layers, int kv_heads, int n_caches, int head_dim) {
     const int splits = std::max(1, std::min(148 / (kv_heads * n_caches), 4 * n_pages));
     const int rounds = ((8 * pages + splits - 1) / splits + GROUP - 1) / GROUP;
-    if (n_caches == 1) return rounds > 2 && head_dim == 128 && splits < 24 ? 0 : splits;
+    if (n_caches == 1) {
+        const bool from_l2 = (size_t)layers * kv_heads * pages * SVLM_PAGE * head_dim * 4 < (size_t)96 << 20;
+        return rounds > 2 && head_dim == 128 && splits < 24 && !from_l2 ? 0 : splits;
+    }
     if (splits < 12 || kv_heads * n_caches * splits > 148) return 0;
     return rounds > (splits >= 16 ? 2 : 1) ? 0 : splits;
 }

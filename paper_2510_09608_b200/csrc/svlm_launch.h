@@ -108,7 +108,7 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
                                bool tagged, cudaStream_t st);
 // Splits of the per-layer kernel for one layer of n_caches caches with `pages` pages or fewer, 0 where the streaming kernel
 // is the better one (either gives the same result).
-int svlm_decode_layer_splits(int n_pages, int pages, int kv_heads, int n_caches, int head_dim);
+int svlm_decode_layer_splits(int n_pages, int pages, int layers, int kv_heads, int n_caches, int head_dim);
 size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits);
 
 // Q/K/V projection with the append as its epilogue, head_dim 128 (svlm_qkv_sm100.cu).  tmX, tmW: host copies of

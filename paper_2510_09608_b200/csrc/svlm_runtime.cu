@@ -330,7 +330,7 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
         // split-KV decode; every cache's scratch was sized for this launch shape at creation
         int pages = 1;
         for (int i = 0; i < n_caches; ++i) pages = std::max(pages, expected_pages(caches[i]));
-        int splits = n_layers == 1 ? svlm_decode_layer_splits(c0->dev.n_pages, pages, c0->dev.kv_heads, n_caches, c0->dev.head_dim) : 0;
+        int splits = n_layers == 1 ? svlm_decode_layer_splits(c0->dev.n_pages, pages, c0->dev.layers, c0->dev.kv_heads, n_caches, c0->dev.head_dim) : 0;
         const bool tagged = splits > 0;
         if (!tagged) splits = svlm_decode_splits(c0->dev.n_pages, c0->dev.kv_heads, n_caches * n_layers);
         SVLM_CUDA(svlm_launch_decode(b, layer0, n_layers, Q, q_pos, q_heads, out, splits, Knew, Vnew, early, tagged, c0->stream));

@@ -117,7 +117,7 @@ def kernels(call):
     return [l.split()[0] for l in ran()]
 small = lambda names: any("prefill_small" in n for n in names)
 layer = lambda names: any("decode_layer" in n for n in names)
-big = dict(hk=8, vw=12000, tw=500, capacity=13000)
+big = dict(layers=6, hk=8, vw=12000, tw=500, capacity=13000)
 for calls in (lambda c: attend(c, 133, hq=32), lambda c: lib.svlm_attend_batched_varlen(arr([c]), 1, 0, vp(P), vp(P), (C.c_int32 * 1)(133), 32, vp(P))):
     c = new(**big)
     assert append(c, 133) == OK and small(kernels(lambda: calls(c)))
@@ -135,4 +135,17 @@ fake.fake_capturing(1)
 assert append(c, 133) == OK                              # captured: the host does not see when it runs
 fake.fake_capturing(0)
 assert not layer(kernels(lambda: step(c, hq=32))) and not layer(kernels(lambda: step(full, hq=32)))
+""")
+
+
+@pytest.mark.parametrize("layers,kv_heads,d,keys,kernel", [
+    (1, 8, 128, 10000, "layer"), (1, 8, 128, 23000, "layer"), (1, 8, 128, 26000, "stream"), (2, 8, 128, 10500, "layer"), (2, 8, 128, 13000, "stream"),
+    (6, 8, 128, 5000, "layer"), (6, 8, 128, 10500, "stream"), (28, 4, 128, 20000, "layer"), (28, 8, 64, 20000, "layer")])
+def test_decode_kernel_of_one_stream(host, layers, kv_heads, d, keys, kernel):
+    """Few thread blocks per KV head and more than two rounds of keys: the streaming kernel, unless the keys stay in L2."""
+    host(f"""
+c = new(layers={layers}, hk={kv_heads}, d={d}, vw={keys}, tw=100, capacity={keys} + 300)
+assert append(c, {keys}) == OK
+ran()
+assert step(c, hq={kv_heads}) == OK and "decode_{kernel}" in "".join(ran())
 """)
