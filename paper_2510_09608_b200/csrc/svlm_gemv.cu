@@ -265,7 +265,12 @@ cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int i
     const uint16_t* x = static_cast<const uint16_t*>(X);
     const uint16_t* w = static_cast<const uint16_t*>(W);
     uint16_t* y = static_cast<uint16_t*>(Y);
-    // weights that stay in L2 from token to token: fetching ahead buys nothing, and more, smaller blocks are 2 us faster
-    if (!from_l2 && few_supported(n, in_dim)) return launch_few(x, w, y, n, in_dim, out_dim, ctrl, st);
+    // Weights that stay in L2 from token to token: fetching ahead buys nothing, and more, smaller blocks are faster while a warp
+    // of theirs has all its weights in flight at once (rows of up to 1792), or in two batches and there are two blocks per SM:
+    // us, one or four tokens, this kernel against the other: 1024 x 1536 2.5 / 2.5-2.9, 2560 x 4096 4.9 / 5.4, 3584 x 2560
+    // 5.1 / 5.6, 3584 x 4608 5.6 / 6.6-7.4.  Not with fewer rows of W (3584 x 2048 4.8 / 4.3, x 512 3.9 / 3.2), longer ones
+    // (4096 x 1536 5.6 / 4.2, 8192 x 1024 8.0 / 4.8) or such as lie a multiple of 4 KB apart (2048 x 6144 7.0 / 5.4).
+    const bool in_batches = in_dim <= 1792 || (in_dim <= 3584 && in_dim % 2048 && out_dim / 8 >= 2 * svlm_sm_count());
+    if (few_supported(n, in_dim) && !(from_l2 && in_batches)) return launch_few(x, w, y, n, in_dim, out_dim, ctrl, st);
     return svlm_launch_chained(gemv_mma_kernel, dim3((out_dim + 7) / 8), dim3(GV_THREADS), 0, 1, st, x, w, y, n, in_dim, out_dim);
 }

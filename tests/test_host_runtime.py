@@ -149,3 +149,14 @@ assert append(c, {keys}) == OK
 ran()
 assert step(c, hq={kv_heads}) == OK and "decode_{kernel}" in "".join(ran())
 """)
+
+
+@pytest.mark.parametrize("layers,in_dim,out_dim,n,kernel", [
+    (1, 64, 128, 1, "mma"), (1, 1792, 512, 4, "mma"), (1, 1856, 512, 1, "few"), (1, 3584, 2304, 4, "few"), (1, 3584, 2432, 4, "mma"), (1, 2048, 6144, 1, "few"),
+    (1, 3648, 4608, 1, "few"), (1, 3584, 4608, 5, "mma"), (28, 3584, 4608, 1, "few"), (1, 25600, 128, 4, "mma")])
+def test_projection_kernel_of_a_few_tokens(host, layers, in_dim, out_dim, n, kernel):
+    host(f"""
+c = new(layers={layers}, capacity=1500 if {layers} == 1 else 200)
+assert lib.svlm_out_proj(c, vp(P), vp(P), {in_dim}, {out_dim}, {n}, vp(P)) == OK
+assert "gemv_{kernel}" in "".join(ran())
+""")
