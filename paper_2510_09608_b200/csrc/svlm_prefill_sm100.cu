@@ -37,10 +37,10 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cstring>
 
 #include "svlm_dev.h"
 #include "svlm_launch.h"
+#include "svlm_prefill_plan.h"
 #include "svlm_ptx.cuh"
 #include "svlm_rope.cuh"
 #include "svlm_tc.cuh"
@@ -53,33 +53,9 @@ using namespace svlm_tc;
 constexpr int PF_THREADS = 384;
 constexpr int PF_RING = 4;            // K/V page stages (3: 18 % slower, the next K arrives late; 5: no faster)
 constexpr int PF_MAX_TILES = 512;
-constexpr int PF_ROWS = 256;          // rows per unit
-constexpr int PF_MAX_CTAS = 160;
-// When units are cut: pages a CTA should have at least, and pieces per unit beyond which merging them costs what the shorter
-// pieces save.  133 to 261 tokens over 1200 keys, 28/4 heads: 6 pages 31-33 us, 4 28.6-30; 69 tokens over 9200 keys: 18 pieces
-// 56.6 us, 12 48.9, 8 44.8.
-constexpr int PF_MIN_PAGES = 4;
-constexpr int PF_MAX_PIECES = 9;
-constexpr int PF_PIECE = 10;          // what beginning a unit costs, in pages (one stream: 3 and 6: 78 us, 10: 76, 16: 78)
-constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
 constexpr int PF_CS_BYTES = 16384;    // rotation factors of one tile's tokens (5 or more heads per KV head, all at head_dim 64 with 2 or more)
 // Registers per thread after the split; 216 * 256 + 72 * 128 = 168 * 384, what the block is launched with (checked at launch).
 constexpr int PF_REGS_LAUNCH = 168;
-
-// The work split, made on the host: it needs the numbers of rows, and of the pages only an estimate (a unit's pages are
-// cut at fractions), so the kernel starts on its first unit without waiting for anything on the device.
-constexpr int PF_FRAC = 128;          // a unit's pages are cut at multiples of 1/128
-struct PfPlan {
-    int units;                        // all units of the launch
-    int off[SVLM_MAX_BATCH + 1];      // first unit of every cache: (layer, KV head, row tile), row tile fastest
-    int rounds;                       // whole units per CTA first: CTA i takes units i, grid + i, ...
-    int tail;                         // the units from here on are dealt out by x
-    unsigned short x[PF_MAX_CTAS + 1];// where each CTA's share of them begins, in 1/128 units
-    unsigned g_magic;                 // for dividing by the heads per KV head (pf_div)
-    unsigned* counters;               // [2 * PF_MAX_CTAS][2] arrivals per (tail unit, tile), zero between launches
-    unsigned char* slots;             // [2 * grid] partial results
-};
-static_assert(2 * PF_MAX_CTAS * 2 * sizeof(unsigned) <= svlm_prefill_counter_bytes, "counters");
 
 template <int D>
 __host__ __device__ constexpr size_t pf_slot_bytes() { return (size_t)PF_ROWS * D * 4 + PF_ROWS * 8; }
@@ -1001,95 +977,6 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
 template <int D>
 constexpr size_t prefill_smem() { return (size_t)(2 + PF_RING) * 128 * D * 2 + 2 * PF_CS_BYTES + sizeof(PfShared); }
 
-// The work split of one launch (see the top of the file): whole units in rounds over the grid while at least two rounds
-// are left, the rest cut so that every CTA ends at the same level.  Beginning a unit, or another piece of one, costs as
-// much as PF_PIECE pages.  The numbers of pages are estimates; a wrong one costs balance only.
-void make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, int G, const SvlmPrefillLoad* held, int max_ctas, int& grid) {
-    plan.units = 0;
-    long long all = 0;                                     // pages of the whole launch
-    const int per_unit = n_layers * b.kv_heads;
-    auto rows_of = [&](int i) { return b.q_varlen ? b.q_cnt[i] : n_q; };
-    auto tiles_of = [&](int i) { return (rows_of(i) * G + PF_ROWS - 1) / PF_ROWS; };
-    // expected pages of row tile rt of cache i: what is stored of the chunk behind its last row is invisible (of a chunk
-    // longer than the windows little is stored)
-    auto cost = [&](int i, int rt) {
-        const int later = std::max(0, rows_of(i) - 1 - (rt * PF_ROWS + PF_ROWS - 1) / G);
-        return std::max(1, held[i].pages - std::min(later, held[i].windows) / SVLM_PAGE);
-    };
-    for (int i = 0; i < b.n_caches; ++i) {
-        plan.off[i] = plan.units;
-        const int R = tiles_of(i);
-        plan.units += per_unit * R;
-        for (int rt = 0; rt < R; ++rt) all += (long long)per_unit * cost(i, rt);
-    }
-    plan.off[b.n_caches] = plan.units;
-    const int U = plan.units;
-    const bool cut = plan.slots != nullptr;
-    grid = (int)std::min<long long>(max_ctas, cut ? std::max<long long>(U, std::min<long long>(all / PF_MIN_PAGES, (long long)PF_MAX_PIECES * U)) : U);
-    plan.rounds = std::max(0, U / grid - 1);
-    plan.tail = plan.rounds * grid;
-    const int nt = U - plan.tail;
-    if (!cut || grid == U) {                               // whole units only
-        for (int i = 0; i <= grid; ++i) plan.x[i] = (unsigned short)((long long)i * nt / grid * PF_FRAC);
-        return;
-    }
-    // walk the units in order: what the whole rounds give each CTA, then the tail's costs
-    int ci = 0, rt = 0, R = tiles_of(0), left = R * per_unit;    // position of unit u
-    auto step = [&] {
-        if (++rt == R) rt = 0;
-        if (--left == 0 && ci + 1 < b.n_caches) { ++ci; R = tiles_of(ci); left = R * per_unit; rt = 0; }
-    };
-    int load[PF_MAX_CTAS] = {}, tail_cost[2 * PF_MAX_CTAS], most = 0, dearest = 1;
-    for (int u = 0, at = 0; u < plan.tail; ++u) {
-        load[at] += cost(ci, rt) + PF_PIECE;
-        most = std::max(most, load[at]);
-        if (++at == grid) at = 0;
-        step();
-    }
-    for (int t = 0; t < nt; ++t) { tail_cost[t] = cost(ci, rt); dearest = std::max(dearest, tail_cost[t]); step(); }
-    // deals the tail out at a level; true when everything has found its place
-    auto deal = [&](double level) {
-        int t = 0;
-        double rem = tail_cost[0];
-        for (int i = 0; i < grid; ++i) {
-            plan.x[i] = (unsigned short)(t < nt ? t * PF_FRAC + (int)((tail_cost[t] - rem) / tail_cost[t] * PF_FRAC + 0.5) : nt * PF_FRAC);
-            double room = level - load[i];
-            while (t < nt && (room -= PF_PIECE) >= std::min((double)PF_SNAP, rem)) {
-                double take = std::min(room, rem);
-                if (rem - take < PF_SNAP) take = rem;                // no slivers
-                room -= take;
-                rem -= take;
-                if (rem > 0) break;
-                if (++t < nt) rem = tail_cost[t];
-            }
-        }
-        return t >= nt;
-    };
-    // the lowest level that does, by bisection between the average and whole units for everybody
-    double lo = ((double)all + (double)PF_PIECE * U) / grid, hi = most + (double)((nt + grid - 1) / grid) * (dearest + PF_PIECE) + PF_SNAP;
-    for (int it = 0; it < 8 && hi - lo > 0.5; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        (deal(mid) ? hi : lo) = mid;
-    }
-    deal(hi);
-    plan.x[grid] = (unsigned short)(nt * PF_FRAC);
-}
-
-// What a plan is made from; the layers of a chunk come one after another with the same numbers, so a thread keeps its
-// latest plan (making one takes microseconds).
-struct PfPlanKey {
-    int n_caches, kv_heads, n_layers, n_q, G, max_ctas, varlen;
-    int rows[SVLM_MAX_BATCH];
-    SvlmPrefillLoad held[SVLM_MAX_BATCH];
-    const void* counters;
-    const void* slots;
-};
-struct PfPlanMemo {
-    PfPlanKey key;
-    PfPlan plan;
-    int grid = 0;
-};
-
 template <int D>
 cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uint16_t* Q, const int* q_pos, int n_q,
                    int q_heads, uint16_t* out, const SvlmPrefillLoad* held, void* counters, void* slots, cudaStream_t st) {
@@ -1102,25 +989,11 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
     }();
     if (!regs_ok) return cudaErrorLaunchOutOfResources;
     const int G = q_heads / b.kv_heads;
-    thread_local PfPlanMemo memo;
-    PfPlanKey key;
-    std::memset(&key, 0, sizeof key);
-    key.n_caches = b.n_caches; key.kv_heads = b.kv_heads; key.n_layers = n_layers; key.n_q = n_q; key.G = G;
-    key.max_ctas = std::min(svlm_sm_count(), PF_MAX_CTAS);
-    key.varlen = b.q_varlen;
-    for (int i = 0; i < b.n_caches; ++i) { key.rows[i] = b.q_varlen ? b.q_cnt[i] : n_q; key.held[i] = held[i]; }
-    key.counters = counters;
-    key.slots = slots;
-    if (memo.grid == 0 || std::memcmp(&memo.key, &key, sizeof key) != 0) {
-        PfPlan& plan = memo.plan;
-        plan.counters = static_cast<unsigned*>(counters);
-        plan.slots = static_cast<unsigned char*>(slots);
-        plan.g_magic = G > 1 && (unsigned long long)n_q * G * G < 0x100000000ull - 256ull * G ? (unsigned)((0x100000000ull + G - 1) / G) : 0u;   // (tiles reach past the last row)
-        make_plan(plan, b, n_layers, n_q, G, held, key.max_ctas, memo.grid);
-        memo.key = key;
-    }
-    const PfPlan& plan = memo.plan;
-    const int grid = memo.grid;
+    const PfPlanned& planned = pf_plan(b, n_layers, n_q, G, held, std::min(svlm_sm_count(), PF_MAX_CTAS), slots != nullptr);
+    const int grid = planned.grid;
+    PfPlan plan = planned.plan;
+    plan.counters = static_cast<unsigned*>(counters);
+    plan.slots = static_cast<unsigned char*>(slots);
     return svlm_launch_chained(prefill_kernel<D>, dim3((unsigned)grid), dim3(PF_THREADS), prefill_smem<D>(), 1, st, b, plan, layer0, n_layers, Q, q_pos,
                                n_q, q_heads, out);
 }

@@ -160,3 +160,55 @@ c = new(layers={layers}, capacity=1500 if {layers} == 1 else 200)
 assert lib.svlm_out_proj(c, vp(P), vp(P), {in_dim}, {out_dim}, {n}, vp(P)) == OK
 assert "gemv_{kernel}" in "".join(ran())
 """)
+
+
+PLAN_PROGRAM = r"""
+#include <cassert>
+#include <cstdio>
+#include "svlm_prefill_plan.h"
+
+static SvlmAttendBatch batch(int kv_heads) { SvlmAttendBatch b{}; b.n_caches = 1; b.kv_heads = kv_heads; return b; }
+
+int main() {
+    PfPlanMemo& memo = pf_plan_memo();
+    SvlmAttendBatch b = batch(4);
+    SvlmPrefillLoad held[SVLM_MAX_BATCH] = {{76, 8704}};
+    // streams served in turn, layer after layer: a split per size, not per call
+    for (int layer = 0; layer < 28; ++layer)
+        for (int stream = 0; stream < 8; ++stream) pf_plan(b, 1, 512 + stream, 7, held, 148, true);
+    assert(memo.made == 8);
+    for (int layer = 0; layer < 28; ++layer) pf_plan(b, 1, 524, 7, held, 148, true);      // more streams than entries: still right
+    for (int n = 2; n < 400; n += 13) pf_plan(b, 1, n, 7, held, 148, true);
+    // every page fraction of every unit is dealt out once, in order
+    long long checked = 0;
+    for (int kv_heads : {1, 4, 8})
+        for (int G : {1, 4, 7})
+            for (int n : {2, 37, 256, 531, 4133})
+                for (int pages : {1, 12, 76, 512})
+                    for (int layers : {1, 28})
+                        for (int cut : {0, 1}) {
+                            b = batch(kv_heads);
+                            held[0] = {pages, pages * 128};
+                            const PfPlanned& p = pf_plan(b, layers, n, G, held, 148, cut != 0);
+                            const int nt = p.plan.units - p.plan.tail;
+                            assert(p.grid >= 1 && p.grid <= 148 && p.plan.rounds * p.grid == p.plan.tail && nt >= 0 && nt < 2 * PF_MAX_CTAS);
+                            assert(p.plan.units == layers * kv_heads * ((n * G + PF_ROWS - 1) / PF_ROWS));
+                            assert(p.plan.x[0] == 0 && p.plan.x[p.grid] == nt * PF_FRAC);
+                            for (int i = 0; i < p.grid; ++i) {
+                                assert(p.plan.x[i] <= p.plan.x[i + 1]);
+                                if (!cut) assert(p.plan.x[i] % PF_FRAC == 0);
+                            }
+                            ++checked;
+                        }
+    std::printf("%lld\n", checked);
+}
+"""
+
+
+def test_chunk_prefill_work_split(tmp_path):
+    """The host's work split: remembered by sizes alone, and complete."""
+    src, exe = tmp_path / "plan.cpp", tmp_path / "plan"
+    src.write_text(PLAN_PROGRAM)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I/usr/local/cuda/include", "-I" + os.path.join(ROOT, "paper_2510_09608_b200", "csrc"),
+                           "-o", str(exe), str(src)])
+    assert subprocess.check_output([str(exe)], text=True).strip() == str(3 * 3 * 5 * 4 * 2 * 2)
