@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import os
+import re
 import subprocess
 import sys
 
@@ -25,6 +26,17 @@ def _headers():
     return hs
 
 
+def check_register_split(src: str, log: str):
+    """The chunk prefill hands registers from one warpgroup to the others (setmaxnreg), which adds up only for the number its
+    block is launched with: PF_REGS_LAUNCH in the source, against what ptxas says it uses."""
+    want = re.search(r"constexpr int PF_REGS_LAUNCH = (\d+);", open(src).read())
+    if not want:
+        return
+    used = re.findall(r"Compiling entry function '\w*?prefill_kernel\w*'.*?Used (\d+) registers", log, flags=re.S)
+    if not used or set(used) != {want.group(1)}:
+        raise RuntimeError(f"{src}: prefill_kernel uses {used} registers, its register split is made for {want.group(1)}")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     newest_header = max(os.path.getmtime(h) for h in _headers())
@@ -42,6 +54,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 sys.stderr.write(res.stdout + res.stderr)
             if res.returncode:
                 raise RuntimeError("nvcc failed on " + src)
+            try:
+                check_register_split(src, res.stdout + res.stderr)
+            except RuntimeError:
+                os.remove(obj)                          # (or the next build would take it as up to date)
+                raise
             relink = True
     if relink or any(os.path.getmtime(o) > os.path.getmtime(LIB) for o in objs):
         subprocess.check_call(["nvcc", "-shared", "-o", LIB, *objs, "-lcudart"])

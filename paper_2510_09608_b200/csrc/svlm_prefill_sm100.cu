@@ -982,7 +982,7 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
                    int q_heads, uint16_t* out, const SvlmPrefillLoad* held, void* counters, void* slots, cudaStream_t st) {
     cudaError_t e = svlm_allow_smem<prefill_kernel<D>>(prefill_smem<D>());
     if (e != cudaSuccess) return e;
-    // the register split inside the kernel adds up only if the block is launched with exactly this many
+    // the register split inside the kernel adds up only if the block is launched with exactly this many (the build sees to it)
     static const bool regs_ok = [] {
         cudaFuncAttributes a;
         return cudaFuncGetAttributes(&a, prefill_kernel<D>) == cudaSuccess && a.numRegs == PF_REGS_LAUNCH;

@@ -31,3 +31,18 @@ def test_binding_constants_match_the_header():
     assert m and binding.NOALLOC_SCRATCH_BYTES == int(m.group(1)) << int(m.group(2))
     for name, value in re.findall(r"SVLM_(ERR_[A-Z_]+|OK)\s*=\s*(-?\d+)", header):
         assert getattr(binding, name) == int(value), name
+
+
+def test_build_refuses_a_register_split_that_does_not_add_up(tmp_path):
+    import pytest
+
+    from paper_2510_09608_b200 import build
+    src = tmp_path / "k.cu"
+    src.write_text("constexpr int PF_REGS_LAUNCH = 168;\n")
+    log = "".join(f"ptxas info : Compiling entry function '_Z14prefill_kernelILi{d}EEv' for 'sm_100a'\nptxas info : Used {{}} registers\n" for d in (64, 128))
+    build.check_register_split(str(src), log.format(168, 168))
+    for bad in (log.format(168, 166), ""):
+        with pytest.raises(RuntimeError):
+            build.check_register_split(str(src), bad)
+    src.write_text("// another file")
+    build.check_register_split(str(src), "")
