@@ -56,8 +56,11 @@ enum svlm_status {
  * 512 tokens/s is 8192).  capacity is the largest number of tokens that is ever stored at once,
  * i.e. retained tokens plus everything appended before the next svlm_cache_evict.
  * head_dim is 64 or 128.  Allocates device memory for `layers` K and V slabs
- * ([layers][kv_heads][pages*128][head_dim] bf16, pages*128 >= capacity), per-token metadata and
- * split-KV scratch; the current CUDA device at the time of the call owns the cache.
+ * ([layers][kv_heads][pages*128][head_dim] bf16, pages*128 >= capacity), per-token metadata,
+ * split-KV scratch and, for 12 pages or more, scratch in which the chunk prefill divides its work over all SMs: two
+ * slots per SM, 39 MB at head_dim 128 and 20 MB at 64 whatever the number of layers (a batched call uses the first cache's).
+ * Where that last part does not fit in memory the cache does without: the same results, one stream's chunks slower.
+ * The current CUDA device at the time of the call owns the cache.
  * Defaults: 1D RoPE with base 10000, sinks are text tokens, contiguous positions, legacy stream 0.
  */
 int svlm_cache_create(svlm_cache** out, int layers, int kv_heads, int head_dim, int n_sink, int vision_window,

@@ -404,14 +404,18 @@ int svlm_cache_create(svlm_cache** out, int layers, int kv_heads, int head_dim, 
         mem.add(&c->decode_tagged, svlm_decode_tagged_bytes(kv_heads, head_dim, svlm_decode_splits(d.n_pages, kv_heads, 1)));
     }
     mem.add(&c->prefill_counters, svlm_prefill_counter_bytes);
-    const size_t slot_bytes = svlm_prefill_slot_bytes(d.n_pages, head_dim);
-    if (slot_bytes) mem.add(&c->prefill_slots, slot_bytes, false);
     mem.add(&d.K, slab);
     mem.add(&d.V, slab);
     mem.add(reinterpret_cast<unsigned char**>(&d.tmaps), 512);
     mem.add(&d.rope_tab, (size_t)3 * 256 * (head_dim / 2) * 2, false);
     mem.add(&c->dev_copy, 1);
+    const size_t slot_bytes = svlm_prefill_slot_bytes(d.n_pages, head_dim);
+    if (slot_bytes) mem.add(&c->prefill_slots, slot_bytes, false);
     rc = mem.allocate(c);
+    if (rc == SVLM_ERR_NOMEM && slot_bytes) {      // without the scratch for cut units the chunk prefill serves whole ones
+        mem.parts.pop_back();
+        rc = mem.allocate(c);
+    }
     if (rc == SVLM_OK) rc = make_tensor_maps(c);
     if (rc == SVLM_OK) rc = upload_rope_table(c);
     if (rc == SVLM_OK) rc = sync_dev_copy(c);

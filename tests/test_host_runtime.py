@@ -212,3 +212,24 @@ def test_chunk_prefill_work_split(tmp_path):
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-I/usr/local/cuda/include", "-I" + os.path.join(ROOT, "paper_2510_09608_b200", "csrc"),
                            "-o", str(exe), str(src)])
     assert subprocess.check_output([str(exe)], text=True).strip() == str(3 * 3 * 5 * 4 * 2 * 2)
+
+
+def test_a_cache_that_fits_without_the_scratch_for_cut_units(host):
+    """Memory for the cache but not for the slots of cut units: it is created, and its chunks take whole units."""
+    host("""
+def blocks(c):
+    assert append(c, 300) == OK
+    for _ in range(4):
+        assert append(c, 250) == OK
+    ran()
+    assert attend(c, 250) == OK
+    name, grid, _ = ran()[-1].split()
+    assert "prefill_kernel" in name
+    return int(grid.split(",")[0])
+size = dict(hk=4, vw=2000, tw=100, capacity=2400)
+assert blocks(new(**size)) > 60                     # 28 units of 256 rows, cut in pieces
+fake.fake_alloc_limit(20 << 20)
+assert blocks(new(**size)) == 28
+fake.fake_alloc_limit(1 << 20)
+assert lib.svlm_cache_create(C.byref(vp()), 1, 4, 128, 4, 2000, 100, 2400) == -6 and fake.cudaGetLastError() == 0
+""")
