@@ -255,3 +255,33 @@ def test_decode_inputs_at_any_element(d, hq, hk, kept, streams):
 
     want = run(0)
     assert torch.equal(run(1), want) and want.any()
+
+
+def test_decode_alternating_single_and_batched():
+    """The same caches decode by themselves, in pairs and all together in turn: the per-layer kernel writes its tagged records
+    with 37 splits, then 18, the streaming kernel its own scratch with 9, and none may take another's leftovers for its own."""
+    from harness import SideBySide, assert_close, bits_to_dev, dev_to_f64
+    from paper_2510_09608_b200 import binding
+    wl = _wl(2, layers=1, n_sink=20, vision_window=1500, text_window=30, frames=4, grid_h=8, grid_w=8, text_max=9)
+    sides = [SideBySide(wl, stream=i) for i in range(4)]
+    for s in sides:
+        for _ in range(7):
+            s.append_chunk()
+            s.evict()
+    for group in (1, 2, 4, 2, 1, 1, 4, 1, 2):
+        for at in range(0, 4, group):
+            part = sides[at:at + group]
+            toks = [s.stream.next_decode_token() for s in part]
+            K, V, Q = (np.stack([getattr(s.stream, w)(0, t[0])[0] for s, t in zip(part, toks)]) for w in "kvq")
+            ty = torch.from_numpy(np.concatenate([t[1] for t in toks])).cuda()
+            ps = torch.from_numpy(np.ascontiguousarray(np.stack([t[2][0] for t in toks]))).cuda()
+            if group == 1:
+                out = part[0].cache.decode_step(0, bits_to_dev(K), bits_to_dev(V), ty, ps, bits_to_dev(Q))
+            else:
+                out = binding.decode_step_batched([s.cache for s in part], 0, bits_to_dev(K), bits_to_dev(V), ty, ps, bits_to_dev(Q))
+            out = dev_to_f64(out)
+            for i, (s, t) in enumerate(zip(part, toks)):
+                assert s.cache.status() == binding.OK
+                s.ref.append(None, None, t[1], t[2])
+                s._give_values_to_ref(0)
+                assert_close(s._stats(out[i][None], s.ref.attend(0, Q[i][None], t[2])))

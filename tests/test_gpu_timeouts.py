@@ -42,7 +42,7 @@ def test_chunk_prefill_gives_up_and_recovers(d128):
     Q = bits_to_dev(s.stream.q(0, gids))
     qp = torch.from_numpy(np.ascontiguousarray(pos)).cuda()
     s.cache.debug_set_wait_limit(0)
-    s.cache.attend(0, Q, qp)                              # tcgen05 kernel: every CTA gives up, frees TMEM, meets its partner
+    s.cache.attend(0, Q, qp)                              # few rows: prefill_small_kernel (the tcgen05 kernel's own: test_gpu_shapes.py)
     assert s.cache.status() == binding.ERR_TIMEOUT
     s.cache.debug_set_wait_limit(1 << 20)
     from harness import dev_to_f64                        # (the harness's own attend insists on an OK status: compare by hand)
@@ -57,12 +57,12 @@ def test_chunk_prefill_gives_up_and_recovers(d128):
 
 
 def test_batched_decode_gives_up_counter_returns_to_zero():
-    """The streaming split-KV kernel (several caches per launch): CTAs that give up still count themselves as
+    """The streaming split-KV kernel (four caches of 4 KV heads: too few splits each for the per-layer kernel): CTAs that give up still count themselves as
     arrived, so the arrival counters are back at zero and the next launch combines correctly."""
     from harness import assert_close, bits_to_dev, dev_to_f64
     from paper_2510_09608_b200 import binding
     wl = _small(True)
-    sides = [_filled(wl, stream_id=i) for i in range(2)]
+    sides = [_filled(wl, stream_id=i) for i in range(4)]
     for s in sides:
         s.append_decode_token()
     caches = [s.cache for s in sides]

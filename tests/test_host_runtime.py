@@ -233,3 +233,24 @@ assert blocks(new(**size)) == 28
 fake.fake_alloc_limit(1 << 20)
 assert lib.svlm_cache_create(C.byref(vp()), 1, 4, 128, 4, 2000, 100, 2400) == -6 and fake.cudaGetLastError() == 0
 """)
+
+
+def test_shapes_of_other_tests_take_the_kernels_they_name(host):
+    """The give-up tests (8 pages, 28/4 heads of 128; four caches) and the smoke test's two chunk shapes."""
+    host("""
+mk = lambda: new(sink=16, vw=192, tw=40, capacity=400)
+caches = [mk() for _ in range(4)]
+for c in caches:
+    assert append(c, 248) == OK
+ran()
+assert attend(caches[0], 70) == OK and "prefill_small" in ran()[-1]
+assert attend(caches[0], 1) == OK and "decode_layer" in ran()[-1]
+both = lambda n: lib.svlm_attend_batched(arr(caches[:n]), n, 0, vp(P), vp(P), 1, 28, vp(P))
+assert both(2) == OK and "decode_layer" in ran()[-1]
+assert both(4) == OK and "decode_stream" in ran()[-1]
+for vw, tw, n, kernel in ((512, 64, 130, "prefill_small"), (1536, 128, 520, "14prefill_kernel")):
+    c = new(layers=2, sink=32, vw=vw, tw=tw, capacity=vw + tw + n + 40)
+    assert append(c, n) == OK and append(c, vw + tw + 32 - n) == OK and append(c, n) == OK and lib.svlm_cache_evict(c) == OK
+    ran()
+    assert attend(c, n) == OK and kernel in ran()[-1], kernel
+""")
