@@ -1282,13 +1282,13 @@ size_t svlm_decode_tagged_bytes(int kv_heads, int head_dim, int splits) {
 // share the combine (8 caches of 4 heads, 4 CTAs a head: 13.5 against 11.5; 3 caches, 12 CTAs a head: 8.9 against 10.3 with
 // one round, 13.7 against 12.7 with two).
 int svlm_decode_layer_splits(int n_pages, int pages, int layers, int kv_heads, int n_caches, int head_dim) {
-    const int splits = std::max(1, std::min(148 / (kv_heads * n_caches), 4 * n_pages));
+    const int splits = std::max(1, std::min(svlm_sm_count() / (kv_heads * n_caches), 4 * n_pages));
     const int rounds = ((8 * pages + splits - 1) / splits + GROUP - 1) / GROUP;
     if (n_caches == 1) {
         const bool from_l2 = (size_t)layers * kv_heads * pages * SVLM_PAGE * head_dim * 4 < (size_t)96 << 20;
         return rounds > 2 && head_dim == 128 && splits < 24 && !from_l2 ? 0 : splits;
     }
-    if (splits < 12 || kv_heads * n_caches * splits > 148) return 0;
+    if (splits < 12 || kv_heads * n_caches * splits > svlm_sm_count()) return 0;
     return rounds > (splits >= 16 ? 2 : 1) ? 0 : splits;
 }
 
@@ -1299,7 +1299,7 @@ int svlm_decode_splits(int n_pages, int kv_heads, int problems) {
     // partial once and more splits than needed to fill the machine only lengthen the tail.  Several
     // problems in one launch: up to two resident CTAs per SM (measured on 16 streams x 4 KV heads:
     // 256 CTAs 64 us, 128 CTAs 70 us, 384 CTAs, which no longer fit at once, 74 us).
-    int splits = (problems > 1 ? 296 : 148) / (kv_heads * problems);
+    int splits = (problems > 1 ? 2 : 1) * svlm_sm_count() / (kv_heads * problems);
     splits = splits < 1 ? 1 : splits;
     return splits > 4 * n_pages ? 4 * n_pages : splits;
 }

@@ -60,7 +60,6 @@ struct SvlmCacheDev {        // passed by value to kernels
     unsigned char* slot_type;// [n_slots]
     SvlmTile* tiles;         // [n_pages]
     int* new_slot;           // [capacity] slots of the latest append
-    int* new_c;              // [capacity][3] positions of the latest append
     long long* ev_gid[2];    // [capacity] evict scratch: ordinals of evicted ring tokens
     long long* ev_pref[2];   // [capacity+1] exclusive prefix of their cursor advances
     uint16_t* K;             // [layers][kv_heads][n_slots][head_dim] bf16, rotated at slot_c

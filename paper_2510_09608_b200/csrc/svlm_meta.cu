@@ -265,11 +265,7 @@ __device__ __forceinline__ void append_one_body(const SvlmCacheDev& cd, const un
         cd.slot_a[slot] = (int)max(0ll, top - cursor0);
         cd.slot_delta[slot] = 0;
         cd.new_slot[0] = slot;
-        for (int k = 0; k < 3; ++k) {
-            const int c = (int)(p[k] - shift);
-            cd.slot_c[k * cd.n_slots + slot] = c;
-            cd.new_c[k] = c;
-        }
+        for (int k = 0; k < 3; ++k) cd.slot_c[k * cd.n_slots + slot] = (int)(p[k] - shift);
         ctrl->n_total = n_total0 + 1;
         ctrl->n_type[ty] = ord + 1;
         ctrl->cursor = max(cursor0, top);
@@ -394,11 +390,7 @@ __device__ __forceinline__ void append_few_body(const SvlmCacheDev& cd, const un
         cd.slot_a[slot] = (int)max(0ll, top - cur_before);
         cd.slot_delta[slot] = 0;
         cd.new_slot[tid] = slot;
-        for (int k = 0; k < 3; ++k) {
-            const int c = (int)(p[k] - shift);
-            cd.slot_c[k * cd.n_slots + slot] = c;
-            cd.new_c[3 * tid + k] = c;
-        }
+        for (int k = 0; k < 3; ++k) cd.slot_c[k * cd.n_slots + slot] = (int)(p[k] - shift);
     }
     // the list of active pages: which page and which offsets are known already, the ordinals behind the barrier
     const TileList tl(sink_fill1, ring_lo0, ring_n1);
@@ -531,11 +523,7 @@ __device__ __forceinline__ void append_meta_body(const SvlmCacheDev& cd, const u
         cd.slot_a[slot] = (int)a;
         cd.slot_delta[slot] = 0;
         cd.new_slot[i] = slot;
-        for (int k = 0; k < 3; ++k) {
-            const int c = (int)(p[k] - shift);
-            cd.slot_c[k * cd.n_slots + slot] = c;
-            cd.new_c[3 * i + k] = c;
-        }
+        for (int k = 0; k < 3; ++k) cd.slot_c[k * cd.n_slots + slot] = (int)(p[k] - shift);
     }
     __syncthreads();
     const int sink_fill1 = sink_fill0 + sink_new[0] + sink_new[1];

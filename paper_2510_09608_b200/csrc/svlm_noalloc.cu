@@ -63,19 +63,16 @@ extern "C" int svlm_attend_decode_noalloc(svlm_cache* c, int layer, const void* 
     if (c->appended < 1) return SVLM_ERR_ORDER;
     if (!svlm_decode_supported(d.n_pages)) return SVLM_ERR_TOO_LARGE;   // more pages than the kernel's page list holds
 
+    int prev = -1;
+    if (cudaGetDevice(&prev) != cudaSuccess) return SVLM_ERR_CUDA;
+    if (prev != c->device && cudaSetDevice(c->device) != cudaSuccess) return SVLM_ERR_CUDA;
     const int splits = svlm_decode_splits(d.n_pages, d.kv_heads, 1);
     // counters for every (layer, kv head) of the cache, then one layer's partials
     auto up4 = [](size_t x) { return (x + 3) & ~(size_t)3; };
     const size_t need = (up4((size_t)d.layers * d.kv_heads) - up4((size_t)d.kv_heads) +
                          svlm_decode_ws_floats(1, d.kv_heads, d.head_dim, splits)) * sizeof(float);
-    if (need > kScratchBytes) return SVLM_ERR_TOO_LARGE;
-
-    int prev = -1;
-    if (cudaGetDevice(&prev) != cudaSuccess) return SVLM_ERR_CUDA;
-    if (prev != c->device && cudaSetDevice(c->device) != cudaSuccess) return SVLM_ERR_CUDA;
-    int rc = SVLM_OK;
     float* scratch = nullptr;
-    rc = scratch_for_device(c->device, &scratch);
+    int rc = need > kScratchBytes ? SVLM_ERR_TOO_LARGE : scratch_for_device(c->device, &scratch);
     // What this call enqueues is not "a decode step of another layer" in the sense the regular entry points use to
     // let their next launch read early: forget the record.
     c->last_decode_layer = -1;

@@ -6,9 +6,6 @@
 
 namespace svlm_ptx {
 
-constexpr unsigned WAIT_LIMIT = 1u << 20;   // default number of polls before a wait gives up (seconds at worst);
-                                            // the limit in force is a field of the cache's control block
-
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(void* bar, unsigned count) {

@@ -391,7 +391,6 @@ int svlm_cache_create(svlm_cache** out, int layers, int kv_heads, int head_dim, 
     mem.add(&d.slot_type, d.n_slots);
     mem.add(&d.tiles, d.n_pages);
     mem.add(&d.new_slot, capacity);
-    mem.add(&d.new_c, 3 * (size_t)capacity);
     for (int t = 0; t < 2; ++t) {
         mem.add(&d.ev_gid[t], capacity);
         mem.add(&d.ev_pref[t], (size_t)capacity + 1);
