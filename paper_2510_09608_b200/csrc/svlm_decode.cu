@@ -74,8 +74,7 @@ namespace {
 using namespace svlm_ptx;
 
 constexpr int DEC_CWARPS = 6;                       // consumer warps
-constexpr int DEC_THREADS = (DEC_CWARPS + 1) * 32;  // + one more warp: the producer of the streaming kernel; in
-                                                    //   the per-layer kernel it only helps with the final merge
+constexpr int DEC_THREADS = (DEC_CWARPS + 1) * 32;  // the streaming kernel: + its producer warp
 // Streaming kernel: one ring stage per consumer warp, so that a warp meets every phase of its stage's
 // barriers in turn.  (With a stage shared between warps a waiter would skip phases, and a parity wait
 // cannot tell the phase it wants from the one two earlier.)
@@ -346,7 +345,7 @@ __device__ __forceinline__ void arrive_and_combine(int* s_last, unsigned* counte
 // record per lane with the lanes a record apart was 2 us slower: 32 cache lines per load instruction).  The four
 // record lanes meet through shuffles, the warps through `buf` (6 x 8 x 12 floats), and four threads per group
 // write the result.  Split 0, which by then has seen every split's record and therefore knows that every CTA of
-// the KV head has read the epoch, moves the epoch on for the next launch.  Called by all DEC_THREADS threads of the
+// the KV head has read the epoch, moves the epoch on for the next launch.  Called by all LAY_THREADS threads of the
 // first `shares` splits after a __syncthreads() that follows their last use of `buf`.
 // stamp: trace hook (stations 12, 15).
 constexpr int LAY_THREADS = DEC_CWARPS * 32;         // the per-layer kernel: consumer warps only (168 registers with two CTAs per SM)

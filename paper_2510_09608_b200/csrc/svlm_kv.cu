@@ -35,7 +35,7 @@ __device__ __forceinline__ void rotate8(Bf16x8& lo, Bf16x8& hi, const float* cs,
 // new slot -> position -> factors, which depend on nothing of each other.  early != 0: the caller vouches that no kernel
 // that may still be running writes this cache's metadata; the chain is then walked before the wait for the predecessor
 // (programmatic dependent launch), which leaves one round trip to memory after it.  Per layer of a 524-token chunk
-// between two chunk-prefill launches: 14 us in the stream with 17 blocks, a longer chain and a full launch gap.
+// between two chunk-prefill launches: 8.3 us in the stream with 17 blocks, a longer chain and a full launch gap, 4.3 now.
 template <int UNROLL>
 __global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int layer, const uint16_t* K,
                                                        const uint16_t* V, int n, int rows_per_block, int early) {

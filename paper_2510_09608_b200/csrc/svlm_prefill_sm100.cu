@@ -5,10 +5,10 @@
 //
 // Work split.  A unit is 256 packed rows (row = (token, head in the GQA group)) of one KV head of one problem
 // (cache, layer): two 128-row tiles A and B that share every K/V page (with 128 rows per CTA the K/V stream out of L2
-// alone took as long as the whole kernel should).  One CTA per SM walks a list of work computed by every CTA for
-// itself from the device-side page counts: first whole units, round by round over the grid (neighbouring CTAs then
-// stream the same pages at the same time), then its share of the last one to two rounds' units, dealt out evenly in
-// pages, so that no SM idles in a last wave (120 of 148 SMs had work for one stream's chunk before, 960 CTAs were 6.5
+// alone took as long as the whole kernel should).  One CTA per SM walks its part of a list of work that the host has
+// made from the numbers of rows and an estimate of the pages (svlm_prefill_plan.h): first whole units, round by round over
+// the grid (neighbouring CTAs then stream the same pages at the same time), then its share of the last one to two rounds'
+// units, dealt out evenly in pages, so that no SM idles in a last wave (120 of 148 SMs had work for one stream's chunk before, 960 CTAs were 6.5
 // waves for eight streams).  A unit that is cut between CTAs is merged by the last of them to finish it: the others
 // leave their un-normalised (O, m, l) in the cache's scratch, arrival counters say who is last, nobody waits.
 //
@@ -18,9 +18,9 @@
 //                    runs ahead into the next unit while the current one ends
 //   warps 9, 10      issue tcgen05.mma for tile A, B: S = Q K^T into 128 TMEM columns, O += P V with P read from
 //                    TMEM (P is written over the first 64 columns of S: no shared-memory round trip)
-//   warp 11          the work list
+//   warp 11          nothing (setmaxnreg works on whole warpgroups)
 // What bounds the page loop is each tile's serial chain S -> softmax -> P V -> next S beside the tensor time of both
-// tiles (2048 cycles per page pair).  Measured on it (cycles per page pair, head_dim 128):
+// tiles (2048 cycles per page pair).  Measured on it (cycles per page pair, head_dim 128, clock read in an instrumented copy):
 //   3750 -> 3490  two issuers with the turn handed on through a named barrier: a wait on an mbarrier costs ~300 cycles
 //                 even when it is already complete (the shared-memory pipe is saturated by the operand reads), and the
 //                 tensor queue is only ~2 MMAs deep, so a single issuer idled the pipe for four such waits per pair;

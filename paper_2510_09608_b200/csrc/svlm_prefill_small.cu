@@ -1,8 +1,9 @@
 // Chunk-prefill attention for chunks of few rows (svlm_prefill_sm100.cu serves the rest): the smallest streams, and short
 // chunks over short windows.  There the tensor-core kernel's time is not work but its fixed chain: tensor memory,
 // register hand-over, 128-row prologue, one 128-key page after another through a single CTA, all of it code that runs once.
-// Here a CTA takes 16 packed rows (row = (token, head in the GQA group)) of a KV head, its warps share the keys in
-// sub-tiles of 32 (mma.sync, the rows being the M side), and meet once at the end; nothing is shared between CTAs.
+// Here a CTA takes 16 or 32 packed rows (row = (token, head in the GQA group)) of a KV head, its warps share the keys in
+// sub-tiles of 32 (mma.sync, the rows being the M side), and meet once at the end; with long windows the keys are divided
+// over a cluster of up to eight CTAs, which then merge through distributed shared memory.
 // A warp fetches its own sub-tiles by TMA into two private stages; the first two are under way while the queries are
 // rotated.  Every mbarrier wait is bounded; on expiry the CTA records SVLM_ERR_TIMEOUT, drains its copies and returns.
 #include <cuda.h>
@@ -442,9 +443,10 @@ cudaError_t launch(const SvlmAttendBatch& b, int layer0, int n_layers, const uin
 // takes a fixed part and a part per 1000 keys, both listed below; a launch takes that for every round of CTAs, and there
 // are as many at once as clusters of that size find room for (4: 112 fit, 136 do not; 8: 80 fit, 128 do not).  Two tiles
 // per CTA cost more than one, but less than a second round.  The tensor-core kernel takes what is estimated at the end,
-// more with many rows, and that again for every 148 units of 256 rows; so the few rows are here, up to long windows, and more rows with short ones.  4 heads of 64, 37
-// tokens, 240 keys: 17.3 -> 4.8; 28/4 heads of 128, 37 tokens: 20 -> 7 at 180 keys, 48 -> 37 at 9100; 133 tokens: 19 -> 11
-// and (by the other kernel) 48.
+// more with many rows, and that again for every 148 units of 256 rows; so the few rows are here, up to long windows, and more rows with short ones.  The
+// tensor-core kernel -> this one: 4 heads of 64, 37 tokens, 240 keys: 17.3 -> 4.8; 28/4 heads of 128: 37 tokens, 180 keys
+// 20 -> 7; 133 tokens, 700 keys 25 -> 16; 37 tokens, 9100 keys 48 -> 37.  133 tokens over 9100 keys stay with the
+// tensor-core kernel (48 against 97 here).
 SvlmPrefillSmall svlm_prefill_small_plan(const SvlmAttendBatch& b, int call_layers, int n_q, int q_heads, const SvlmPrefillLoad* held) {
     struct Shape { int tiles, parts, at_once; float fixed[2], per_key[2]; };       // [head size 128, 64]
     static constexpr Shape shapes[] = {{1, 1, 148, {6.0f, 4.4f}, {6.1f, 3.6f}}, {1, 2, 144, {7.0f, 5.8f}, {3.3f, 1.95f}},

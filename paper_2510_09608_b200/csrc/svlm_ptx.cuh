@@ -72,25 +72,38 @@ __device__ __forceinline__ void mma_bf16(float* c, unsigned a0, unsigned a1, uns
 // when this one starts, so such data must not take the read-only path (ld.global.nc, which __ldg and const __restrict__
 // parameters allow: it is for data that nobody writes while the kernel runs, and the compiler may move such a load above
 // the wait).  These are volatile and stay behind pdl_wait().  ld_l2 reads past L1.
-#define SVLM_LOAD1(T, type, reg)                                                                                                  \
-    __device__ __forceinline__ T ld_in(const T* p) { T v; asm volatile("ld.global." type " %0, [%1];" : reg(v) : "l"(p) : "memory"); return v; }    \
-    __device__ __forceinline__ T ld_l2(const T* p) { T v; asm volatile("ld.global.cg." type " %0, [%1];" : reg(v) : "l"(p) : "memory"); return v; }
-#define SVLM_LOAD2(T, type, reg)                                                                                                  \
-    __device__ __forceinline__ T ld_in(const T* p) { T v; asm volatile("ld.global.v2." type " {%0, %1}, [%2];" : reg(v.x), reg(v.y) : "l"(p) : "memory"); return v; }    \
-    __device__ __forceinline__ T ld_l2(const T* p) { T v; asm volatile("ld.global.cg.v2." type " {%0, %1}, [%2];" : reg(v.x), reg(v.y) : "l"(p) : "memory"); return v; }
-#define SVLM_LOAD4(T, type, reg)                                                                                                  \
-    __device__ __forceinline__ T ld_in(const T* p) { T v; asm volatile("ld.global.v4." type " {%0, %1, %2, %3}, [%4];" : reg(v.x), reg(v.y), reg(v.z), reg(v.w) : "l"(p) : "memory"); return v; }    \
-    __device__ __forceinline__ T ld_l2(const T* p) { T v; asm volatile("ld.global.cg.v4." type " {%0, %1, %2, %3}, [%4];" : reg(v.x), reg(v.y), reg(v.z), reg(v.w) : "l"(p) : "memory"); return v; }
-SVLM_LOAD1(uint16_t, "u16", "=h")
-SVLM_LOAD1(int, "s32", "=r")
-SVLM_LOAD1(unsigned, "u32", "=r")
-SVLM_LOAD1(long long, "s64", "=l")
-SVLM_LOAD2(longlong2, "s64", "=l")
-SVLM_LOAD2(float2, "f32", "=f")
-SVLM_LOAD4(float4, "f32", "=f")
-SVLM_LOAD4(int4, "s32", "=r")
-SVLM_LOAD4(uint4, "u32", "=r")
-#undef SVLM_LOAD1
+#define SVLM_LOAD(name, T, instr, reg)                                       \
+    __device__ __forceinline__ T name(const T* p) {                         \
+        T v;                                                                \
+        asm volatile(instr " %0, [%1];" : reg(v) : "l"(p) : "memory");      \
+        return v;                                                           \
+    }
+#define SVLM_LOAD2(name, T, instr, reg)                                                             \
+    __device__ __forceinline__ T name(const T* p) {                                                 \
+        T v;                                                                                        \
+        asm volatile(instr " {%0, %1}, [%2];" : reg(v.x), reg(v.y) : "l"(p) : "memory");            \
+        return v;                                                                                   \
+    }
+#define SVLM_LOAD4(name, T, instr, reg)                                                                                             \
+    __device__ __forceinline__ T name(const T* p) {                                                                                 \
+        T v;                                                                                                                        \
+        asm volatile(instr " {%0, %1, %2, %3}, [%4];" : reg(v.x), reg(v.y), reg(v.z), reg(v.w) : "l"(p) : "memory");                \
+        return v;                                                                                                                   \
+    }
+SVLM_LOAD(ld_in, uint16_t, "ld.global.u16", "=h")
+SVLM_LOAD(ld_in, int, "ld.global.s32", "=r")
+SVLM_LOAD(ld_in, unsigned, "ld.global.u32", "=r")
+SVLM_LOAD2(ld_in, longlong2, "ld.global.v2.s64", "=l")
+SVLM_LOAD4(ld_in, uint4, "ld.global.v4.u32", "=r")
+SVLM_LOAD(ld_l2, int, "ld.global.cg.s32", "=r")
+SVLM_LOAD(ld_l2, unsigned, "ld.global.cg.u32", "=r")
+SVLM_LOAD(ld_l2, long long, "ld.global.cg.s64", "=l")
+SVLM_LOAD2(ld_l2, longlong2, "ld.global.cg.v2.s64", "=l")
+SVLM_LOAD2(ld_l2, float2, "ld.global.cg.v2.f32", "=f")
+SVLM_LOAD4(ld_l2, float4, "ld.global.cg.v4.f32", "=f")
+SVLM_LOAD4(ld_l2, int4, "ld.global.cg.v4.s32", "=r")
+SVLM_LOAD4(ld_l2, uint4, "ld.global.cg.v4.u32", "=r")
+#undef SVLM_LOAD
 #undef SVLM_LOAD2
 #undef SVLM_LOAD4
 
