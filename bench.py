@@ -832,8 +832,7 @@ def bench_qkv(args, wl, base, peaks, rank, world, local):
         cache.close()
         ms = statistics.median(times)
         flops = 2.0 * n * hidden * n_out
-        rows.append(dict(n=n, ms_per_layer=ms, tflops=flops / (ms * 1e-3) / 1e12, frac=flops / (ms * 1e-3) / 1e12 / peaks["bf16_burst"],
-                         ctas=(n + 127) // 128 * ((wl.q_heads + 2 * wl.kv_heads + 1) // 2)))
+        rows.append(dict(n=n, ms_per_layer=ms, tflops=flops / (ms * 1e-3) / 1e12, frac=flops / (ms * 1e-3) / 1e12 / peaks["bf16_burst"]))
     # decode-time projections (a few tokens): the bandwidth kernel behind svlm_out_proj, weights of the layers in turn
     cache = binding.Cache(1, wl.kv_heads, wl.head_dim, 0, 0, 0, 128)
     small = []
