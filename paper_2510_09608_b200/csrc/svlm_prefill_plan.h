@@ -13,7 +13,7 @@ constexpr int PF_MAX_CTAS = 160;
 // 56.6 us, 12 48.9, 8 44.8.
 constexpr int PF_MIN_PAGES = 4;
 constexpr int PF_MAX_PIECES = 9;
-constexpr int PF_PIECE = 10;          // what beginning a unit is reckoned as, in pages: fitted, not measured (one stream: 3 and 6: 78 us, 10: 76, 16: 78)
+constexpr int PF_PIECE = 8;           // what beginning a unit is reckoned as, in pages (one stream, 28 layers: 10: 2.52 ms, 8: 2.43, 5: 2.43; four layers of a long chunk 1.71, 1.72 with 5)
 constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
 
 // The work split, made on the host: it needs the numbers of rows, and of the pages only an estimate (a unit's pages are

@@ -271,6 +271,33 @@ __device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfSeg&
     return w;
 }
 
+// How a cut unit of the tail is divided, from the launch's arguments alone: its pieces lie with the CTAs [first, last], those
+// with an empty share left out; the CTAs that end in it (all of them but one that has other segments to come) share the merge,
+// in blocks of 16 columns, the first `sharers` of them.
+struct PfCut {
+    int first, last, pieces, sharers;
+    int me;                  // this CTA's share, -1: none
+};
+template <int D>
+__device__ __forceinline__ PfCut pf_cut(const PfPlan& plan, int tail) {
+    const int u0 = tail * PF_FRAC, u1 = u0 + PF_FRAC, cta = blockIdx.x;
+    PfCut c;
+    for (c.first = cta; plan.x[c.first] > u0; --c.first) {}
+    for (c.last = cta; plan.x[c.last + 1] < u1; ++c.last) {}
+    int ends = 0;
+    c.pieces = 0;
+    c.me = -1;
+    for (int k = c.first; k <= c.last; ++k) {
+        if (plan.x[k] == plan.x[k + 1]) continue;
+        ++c.pieces;
+        if (plan.x[k + 1] > u1) continue;
+        if (k == cta) c.me = ends;
+        ++ends;
+    }
+    c.sharers = min(ends, D / 16);
+    if (c.me >= c.sharers) c.me = -1;
+    return c;
+}
 // The softmax warpgroups keep what they know about their segment in shared memory: the page loop needs nearly all of
 // their registers for the row of scores.
 struct PfGroup {
@@ -279,7 +306,7 @@ struct PfGroup {
     PfWork w;
     PfWalk walk;
     int more;                // segments follow
-    int merge_later;         // a cut unit whose pieces this CTA has to put together at the end (-1: none)
+    unsigned merge_later;    // shares of the first segment's unit that this CTA has to merge at the end
 };
 
 struct PfShared {            // control part of shared memory, behind the tiles
@@ -287,7 +314,9 @@ struct PfShared {            // control part of shared memory, behind the tiles
     unsigned long long s_full[2], all_done[2];
     unsigned tmem_base;
     int abort_flag;
-    int last[2];                           // per tile: this CTA's piece of the unit was the last to be done
+    unsigned take[2];                      // per tile: shares of a cut unit that this CTA has to merge
+    int leave[2];                          // its own share is left to whoever comes last
+    PfCut cut[2];                          // of the CTA's last segment, of its first one
     PfGroup group[2];
 };
 static_assert(sizeof(PfShared) <= 3072, "control block must fit behind the tiles");
@@ -514,9 +543,9 @@ __device__ __forceinline__ int causal_end(const int (&v)[4], int r) {
     return n;
 }
 
-__device__ __forceinline__ void store_row32(uint16_t* dst, const float* o) {
+__device__ __forceinline__ void store_row16(uint16_t* dst, const float* o) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 2; ++k)
         *reinterpret_cast<uint4*>(dst + 8 * k) = make_uint4(pack2(o[8 * k], o[8 * k + 1]), pack2(o[8 * k + 2], o[8 * k + 3]),
                                                             pack2(o[8 * k + 4], o[8 * k + 5]), pack2(o[8 * k + 6], o[8 * k + 7]));
 }
@@ -536,110 +565,161 @@ struct PfSlot {
     __device__ __forceinline__ float2* ml(int g, int m) const { return reinterpret_cast<float2*>(base + (size_t)PF_ROWS * D * 4) + g * 128 + m; }
 };
 
-// This CTA's piece of a cut unit into its slot (un-normalised, fp32), then counted.  True in the CTA whose piece was the
-// last one (for all 128 threads of the warpgroup).
 template <int D>
-__device__ __forceinline__ bool publish_piece(PfShared& sh, const PfPlan& plan, int tail, int pieces, int g, int m, unsigned tO, float m_row, float l, bool have_o) {
-    const PfSlot<D> slot(plan, tail, blockIdx.x);
-    float4* po = slot.o(g, m);
-    if (have_o)
+__device__ __forceinline__ int share_begin(const PfCut& c, int s) { return pf_small_div(s * (D / 16), c.sharers); }   // in blocks of 16 columns
+
+// Columns of this CTA's piece of a cut unit into its slot (un-normalised, fp32): the blocks of 16 in [q0, q1), or all others.
+template <int D>
+__device__ __forceinline__ void publish_columns(const PfPlan& plan, int tail, int g, int m, unsigned tO, bool have_o, int q0, int q1, bool others) {
+    if (!have_o) return;
+    float4* po = PfSlot<D>(plan, tail, blockIdx.x).o(g, m);
 #pragma unroll 1
-        for (int q4 = 0; q4 < D / 32; ++q4) {
-            float o[32];
-            tmem_ld32(tO + q4 * 32, o);
-            tmem_wait_ld();
+    for (int q = 0; q < D / 16; ++q) {
+        if ((q >= q0 && q < q1) == others) continue;
+        float o[16];
+        tmem_ld16_wait(tO + q * 16, o);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) __stcg(po + (q4 * 8 + i) * 128, make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]));
-        }
+        for (int i = 0; i < 4; ++i) __stcg(po + (q * 4 + i) * 128, make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]));
+    }
+}
+
+// The meeting of a unit's pieces, per tile: a word that counts arrivals (bits 0-7) and sharers that are through with it
+// (8-15) and names the shares whose owners did not wait (16-23).  A sharer has put down what the others need of its piece,
+// counts itself in and waits for the rest, which the work split lets end at the same time: `polls` times at most.  If they
+// are not there by then (their thread blocks may not even be running: another launch may hold the SMs) it puts down its own
+// columns too, names its share and leaves; whoever comes last merges those shares.  So nothing depends on a wait, and
+// whoever brings the word to its end clears it for the next launch.  Returns the shares this CTA has to merge.
+constexpr int PF_MEET_POLLS = 14;         // polls: the control block's limit >> this (64 by default, some 40 us)
+template <int D>
+__device__ __forceinline__ unsigned meet_pieces(PfShared& sh, const PfPlan& plan, int tail, const PfCut& cut, int g, int m, unsigned tO, float m_row, float l,
+                                                bool have_o, unsigned polls) {
+    unsigned* word = plan.counters + tail * 2 + g;
+    const int q0 = cut.me < 0 ? 0 : share_begin<D>(cut, cut.me), q1 = cut.me < 0 ? 0 : share_begin<D>(cut, cut.me + 1);
+    auto add = [&](unsigned v) {                          // returns the new value; the end of the meeting clears the word
+        unsigned prev;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(prev) : "l"(word), "r"(v) : "memory");
+        prev += v;
+        if ((prev & 0xffff) == (unsigned)(cut.pieces | cut.sharers << 8)) *word = 0;
+        return prev;
+    };
+    const PfSlot<D> slot(plan, tail, blockIdx.x);
     __stcg(slot.ml(g, m), make_float2(have_o ? m_row : -INFINITY, l));
-    __threadfence();
+    publish_columns<D>(plan, tail, g, m, tO, have_o, q0, q1, true);
     bar_sync(BAR_WG + g, 128);
     if (m == 0) {
-        unsigned prev;
-        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(prev) : "l"(plan.counters + tail * 2 + g) : "memory");
-        sh.last[g] = prev == (unsigned)pieces - 1;
+        __threadfence();
+        const unsigned seen = add(1);
+        bool all = (seen & 255) == (unsigned)cut.pieces;
+        unsigned take = all ? seen >> 16 : 0;
+        if (cut.me >= 0) {
+            for (unsigned p = 0; !all && p < polls; ++p) {
+                unsigned now;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(word) : "memory");
+                all = (now & 255) == (unsigned)cut.pieces;
+            }
+            if (all) { take |= 1u << cut.me; add(1u << 8); }
+        }
+        sh.take[g] = take;
+        sh.leave[g] = cut.me >= 0 && !all;
     }
     bar_sync(BAR_WG + g, 128);
-    return sh.last[g] != 0;
-}
-
-// CTAs that hold pieces of a tail unit: [first, last], those with an empty share left out.  near: one of them.
-__device__ __forceinline__ int count_pieces(const PfPlan& plan, int tail, int near, int& first, int& last) {
-    const int u0 = tail * PF_FRAC;
-    for (first = near; plan.x[first] > u0; --first) {}
-    for (last = near; plan.x[last + 1] < u0 + PF_FRAC; ++last) {}
-    int n = 0;
-    for (int k = first; k <= last; ++k) n += plan.x[k] < plan.x[k + 1];
-    return n;
-}
-
-// The output of a cut unit's tile from the slots of its pieces, by the CTA that came last; that CTA's own piece may
-// still be in TMEM (own).  In the order of the pieces, whoever comes last: the same bits every time.
-template <int D>
-__device__ __forceinline__ void merge_pieces(const PfPlan& plan, int tail, const PfRows& w, int g, int m, int G, int q_heads, bool own,
-                                             unsigned tO, float m_row, float l, bool have_o, uint16_t* __restrict__ out) {
-    __threadfence();
-    if (m == 0) plan.counters[tail * 2 + g] = 0;      // ready for the next launch
-    int first, last;
-    count_pieces(plan, tail, blockIdx.x, first, last);      // (this CTA holds a piece)
-    const int me = own ? (int)blockIdx.x : -1;
-    const float m_own = have_o ? m_row : -INFINITY;
-    float M = -INFINITY, L = 0.f;
-#pragma unroll 1
-    for (int k0 = first; k0 <= last; k0 += 4) {              // four pieces' (m, l) in flight
-        float2 ml[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = min(k0 + i, last);
-            ml[i] = k == me ? make_float2(m_own, l) : ld_l2(PfSlot<D>(plan, tail, k).ml(g, m));
-            if (k0 + i > last || plan.x[k] >= plan.x[k + 1]) ml[i].x = -INFINITY;
+    if (sh.leave[g]) {
+        publish_columns<D>(plan, tail, g, m, tO, have_o, q0, q1, false);
+        bar_sync(BAR_WG + g, 128);
+        if (m == 0) {
+            __threadfence();
+            const unsigned seen = add((1u << 8) + (0x10000u << cut.me));
+            sh.take[g] = (seen & 255) == (unsigned)cut.pieces ? 1u << cut.me : 0;      // (the last one came in between: it did not see the name)
         }
-        const float Mn = fmaxf(fmaxf(M, fmaxf(ml[0].x, ml[1].x)), fmaxf(ml[2].x, ml[3].x));
-        if (Mn > -INFINITY) {
-            L *= exp2f(M - Mn);                              // M = -inf gives 0
-#pragma unroll
-            for (int i = 0; i < 4; ++i) if (ml[i].x > -INFINITY) L += ml[i].y * exp2f(ml[i].x - Mn);
-            M = Mn;
-        }
+        bar_sync(BAR_WG + g, 128);
     }
-    const float inv = L > 0.f ? 1.f / L : 0.f;
+    return sh.take[g];
+}
+
+// Some shares of a cut unit's output from its pieces: those of a share's owner come last, from TMEM if the owner is this CTA
+// (own: its last segment), all others from the slots in their order.  So the same bits come out every time, whoever does it.
+// 64 columns of two other pieces are asked for at once, together with the pieces' (m, l): mostly that is all there is (one
+// round trip to L2, where two pieces' 32 columns at a time, after the (m, l), took four).
+template <int D>
+__device__ __forceinline__ void merge_shares(const PfPlan& plan, int tail, const PfCut& cut, unsigned take, const PfRows& w, int g, int m, int G, int q_heads,
+                                             bool own, unsigned tO, float m_row, float l, bool have_o, uint16_t* __restrict__ out) {
+    const int last = cut.last;
+    int owner = blockIdx.x, left;
+    auto after = [&](int k) {                                // the next piece that is not the owner's, last + 1: none
+        for (++k; k <= last && (k == owner || plan.x[k] >= plan.x[k + 1]); ++k) {}
+        return k;
+    };
+    auto load = [&](int k, int q, int nb, float (&o)[64]) {  // nb blocks of 16 columns (of a piece without pages: left over from earlier, not used)
+        const float4* po = PfSlot<D>(plan, tail, k).o(g, m) + q * 4 * 128;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (j < 4 * nb) {
+                const float4 v = ld_l2(po + j * 128);
+                o[4 * j] = v.x; o[4 * j + 1] = v.y; o[4 * j + 2] = v.z; o[4 * j + 3] = v.w;
+            }
+    };
+    auto ml_of = [&](int k) { return k > last ? make_float2(-INFINITY, 0.f) : ld_l2(PfSlot<D>(plan, tail, k).ml(g, m)); };
     const int mg = w.m0 + g * 128 + m;
     uint16_t* dst = out_row(out, w, min(mg, w.m_total - 1), plan.g_magic, G, q_heads, D);
-    // 64 columns at a time: 16 loads in flight per thread and piece (with 8 this step took 16 us, one latency after another)
 #pragma unroll 1
-    for (int h = 0; h < D / 64; ++h) {
-        float acc[64];
-#pragma unroll
-        for (int i = 0; i < 64; ++i) acc[i] = 0.f;
+    for (; take; take &= take - 1) {
+        const int s = __ffs(take) - 1, q1 = share_begin<D>(cut, s + 1);
+        const bool mine = own && s == cut.me;
+        owner = blockIdx.x;
+        if (!mine)                                           // the s-th of the unit's pieces: those of the CTAs that end in it come first
+            for (owner = cut.first - 1, left = s; left >= 0; --left)
+                for (++owner; plan.x[owner] >= plan.x[owner + 1]; ++owner) {}
+        const int k1 = after(cut.first - 1), k2 = after(k1);
+        const float2 mla = mine ? make_float2(have_o ? m_row : -INFINITY, l) : ml_of(owner), ml1 = ml_of(k1), ml2 = ml_of(k2);
+        float M = -INFINITY, inv = 0.f;
 #pragma unroll 1
-        for (int k = first; k <= last; ++k) {
-            if (plan.x[k] >= plan.x[k + 1]) continue;
-            float o[64], mk = m_own;
-            if (k == me) {
-                if (have_o) {
-                    tmem_ld32(tO + h * 64, o);
-                    tmem_ld32(tO + h * 64 + 32, o + 32);
-                    tmem_wait_ld();
+        for (int q = share_begin<D>(cut, s); q < q1; q += 4) {
+            const int nb = min(4, q1 - q);
+            float o1[64], o2[64];
+            load(k1, q, nb, o1);                             // (a cut unit has two pieces at least)
+            if (k2 <= last) load(k2, q, nb, o2);
+            if (inv == 0.f) {                                // first time: the row's maximum and sum over all pieces
+                M = max3(mla.x, ml1.x, ml2.x);
+                float L = 0.f;
+                auto add = [&](const float2& ml) { if (ml.x > -INFINITY) L += ml.y * exp2f(ml.x - M); };
+                add(mla); add(ml1); add(ml2);
+                for (int k = after(k2); k <= last; k = after(k)) {
+                    const float2 ml = ml_of(k);
+                    const float Mn = fmaxf(M, ml.x);
+                    if (Mn > M) { L *= exp2f(M - Mn); M = Mn; }      // M = -inf gives 0
+                    add(ml);
                 }
-            } else {
-                const PfSlot<D> slot(plan, tail, k);
-                mk = ld_l2(slot.ml(g, m)).x;
-                const float4* po = slot.o(g, m) + h * 16 * 128;
+                inv = L > 0.f ? 1.f / L : 1.f;               // nothing visible: all weights below are 0
+            }
+            auto weight = [&](float mk) { return mk > -INFINITY ? exp2f(mk - M) * inv : 0.f; };
+            const float fa = weight(mla.x), f1 = weight(ml1.x), f2 = weight(ml2.x);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {        // (of a piece without pages: left over from earlier, not used)
-                    const float4 v = ld_l2(po + i * 128);
-                    o[4 * i] = v.x; o[4 * i + 1] = v.y; o[4 * i + 2] = v.z; o[4 * i + 3] = v.w;
+            for (int c = 0; c < 64; ++c) {
+                float x = 0.f;
+                if (f1 > 0.f) x += o1[c] * f1;
+                if (f2 > 0.f) x += o2[c] * f2;
+                o1[c] = x;
+            }
+#pragma unroll 1
+            for (int k = after(k2); k <= last; k = after(k)) {
+                const float f = weight(ml_of(k).x);
+                load(k, q, nb, o2);
+#pragma unroll
+                for (int c = 0; c < 64; ++c) if (f > 0.f) o1[c] += o2[c] * f;
+            }
+            if (!mine) load(owner, q, nb, o2);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < nb) {
+                    float* a = o2 + 16 * i;
+                    if (mine && have_o) {
+                        __syncwarp();
+                        tmem_ld16_wait(tO + (q + i) * 16, a);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) if (fa > 0.f) o1[16 * i + c] += a[c] * fa;
+                    if (mg < w.m_total) store_row16(dst + (q + i) * 16, o1 + 16 * i);
                 }
-            }
-            if (mk > -INFINITY) {
-                const float f = exp2f(mk - M) * inv;
-#pragma unroll
-                for (int i = 0; i < 64; ++i) acc[i] += o[i] * f;
-            }
-        }
-        if (mg < w.m_total) {
-            store_row32(dst + h * 64, acc);
-            store_row32(dst + h * 64 + 32, acc + 32);
         }
     }
 }
@@ -674,6 +754,10 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
     if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (threadIdx.x == 32 || threadIdx.x == 64) {      // cut units: the last segment's, and the first one's where that is the end of one
+        const int x0 = plan.x[blockIdx.x], x1 = plan.x[blockIdx.x + 1], which = threadIdx.x / 32 - 1;
+        if (x0 < x1) sh.cut[which] = pf_cut<D>(plan, (which ? x0 : x1 - 1) / PF_FRAC);
     }
     // Set up while the predecessor ends (programmatic dependent launch); everything read from here on may be its work.
     // The wait comes before the trigger: a successor that starts early then finds all earlier work done.
@@ -821,7 +905,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         unsigned char* sQg = sQ + g * TILE_BYTES;
         float* cs_g = reinterpret_cast<float*>(s_cs + g * PF_CS_BYTES);
         float m_ref = -INFINITY, l = 0.f;
-        if (m == 0) { gr.walk.begin(plan); gr.merge_later = -1; gr.more = gr.walk.more(plan); gr.seg.a = 0; gr.seg.e = PF_FRAC; }
+        if (m == 0) { gr.walk.begin(plan); gr.merge_later = 0; gr.more = gr.walk.more(plan); gr.seg.a = 0; gr.seg.e = PF_FRAC; }
         bar_sync(BAR_WG + g, 128);
         while (gr.more) {
             bar_sync(BAR_WG + g, 128);        // everybody is through with the previous segment's fields
@@ -917,40 +1001,26 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     }
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] = have_o ? o[i] * inv : 0.f;
-                    if (mg < gr.rows.m_total) store_row32(dst + q4 * 32, o);
+                    if (mg < gr.rows.m_total) { store_row16(dst + q4 * 32, o); store_row16(dst + q4 * 32 + 16, o + 16); }
                 }
-            } else if (gr.more) {
-                int first, last;
-                const int pieces = count_pieces(plan, gr.seg.tail, blockIdx.x, first, last);
-                if (publish_piece<D>(sh, plan, gr.seg.tail, pieces, g, m, tO, m_ref, l, have_o) && m == 0) gr.merge_later = gr.seg.tail;
+            } else if (gr.more) {                                      // the end of a unit that others have begun
+                const unsigned take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[1], g, m, tO, m_ref, l, have_o, 0);
+                if (m == 0) gr.merge_later = take;
             }
         }
-        // What is left of cut units (outside the loop over segments: its code would cost the page loop registers).  The
-        // last segment's piece stays in TMEM when the others are already there, which is the usual case.
-        int mine_tail = -1;
-        bool own = false;
+        // What is left of cut units (outside the loop over segments: its code would cost the page loop registers).
         const bool have_o = ok && gr.w.n_proc > 0;
-        if (gr.seg.e - gr.seg.a < PF_FRAC) {
-            const int tail = gr.seg.tail;
-            int first, last;
-            const int pieces = count_pieces(plan, tail, blockIdx.x, first, last);
-            bar_sync(BAR_WG + g, 128);
-            if (m == 0) {
-                unsigned n;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(plan.counters + tail * 2 + g) : "memory");
-                sh.last[g] = n == (unsigned)pieces - 1;
-            }
-            bar_sync(BAR_WG + g, 128);
-            own = sh.last[g] != 0;                                     // (then nobody else is left to arrive)
-            bar_sync(BAR_WG + g, 128);
-            if (own || publish_piece<D>(sh, plan, tail, pieces, g, m, tO, m_ref, l, have_o)) mine_tail = tail;
-        }
+        unsigned take = 0;
+        if (gr.seg.e - gr.seg.a < PF_FRAC)
+            take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[0], g, m, tO, m_ref, l, have_o, gr.w.wait_limit >> PF_MEET_POLLS);
         bar_sync(BAR_WG + g, 128);
+#pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
-            const int tail = pass == 0 ? mine_tail : gr.merge_later;
-            if (tail < 0) continue;
+            const unsigned shares = pass == 0 ? take : gr.merge_later;
+            if (!shares) continue;
+            const int tail = (pass == 0 ? plan.x[blockIdx.x + 1] - 1 : (int)plan.x[blockIdx.x]) / PF_FRAC;
             const PfRows rows = pf_rows(b, plan, plan.tail + tail, n_q_arg, G, layer0, n_layers);
-            merge_pieces<D>(plan, tail, rows, g, m, G, q_heads, pass == 0 && own, tO, m_ref, l, have_o, out);
+            merge_shares<D>(plan, tail, sh.cut[pass], shares, rows, g, m, G, q_heads, pass == 0, tO, m_ref, l, have_o, out);
         }
     }
 

@@ -80,6 +80,34 @@ def test_large_chunk_prefill_gives_up_and_recovers(d, hq, hk):
     assert_close(s._stats(out[rows], s.ref.attend(0, s.stream.q(0, gids), pos, rows=rows)))
 
 
+# --- pieces of a cut unit that do not wait for one another: the poll limit leaves the other waits alone and the meeting none,
+# --- so that whoever comes last puts the others' shares together; the same bits as when each merges its own
+@pytest.mark.parametrize("d,hq,hk,frames,vw", [(128, 28, 4, 7, 2304), (128, 28, 4, 1, 6000), (64, 12, 2, 7, 2304), (64, 16, 8, 1, 9000)])
+def test_cut_units_without_waiting(d, hq, hk, frames, vw):
+    from harness import SideBySide, bits_to_dev
+    from paper_2510_09608_b200 import binding
+    wl = _wl(2, layers=1, q_heads=hq, kv_heads=hk, head_dim=d, sections=(d // 8, d // 16 * 3, d // 16 * 3), n_sink=40, vision_window=vw, text_window=70,
+             frames=frames, grid_h=8, grid_w=9, text_max=21)
+    s = SideBySide(wl)
+    for _ in range(2 + (vw + 70) // (72 * frames)):
+        s.append_chunk()
+        s.evict()
+    gids, _, pos = s.last
+    Q, qp = bits_to_dev(s.stream.q(0, gids)), torch.from_numpy(np.ascontiguousarray(pos)).cuda()
+    s._give_values_to_ref(0)
+    rows = list(range(0, len(gids), 31))
+    want = s.ref.attend(0, s.stream.q(0, gids), pos, rows=rows)
+    out = s.cache.attend(0, Q, qp).clone()
+    s.cache.debug_set_wait_limit((1 << 14) - 1)
+    for _ in range(3):                                     # (the counters come back to zero)
+        again = s.cache.attend(0, Q, qp)
+        assert torch.equal(out, again)
+    s.cache.debug_set_wait_limit(1 << 20)
+    assert torch.equal(out, s.cache.attend(0, Q, qp)) and s.cache.status() == binding.OK
+    from harness import assert_close, dev_to_f64
+    assert_close(s._stats(dev_to_f64(out)[rows], want))
+
+
 # --- append metadata: one token, up to 1024 (one per thread), more; sinks of either rule that end inside a chunk; evictions
 # --- of more tokens than fit the lists in shared memory
 @pytest.mark.parametrize("sink_any", [False, True])
