@@ -306,6 +306,10 @@ struct PfGroup {
     PfWork w;
     PfWalk walk;
     int more;                // segments follow
+    int known;               // the cache that the next three belong to (-1: none): a launch does not change its metadata
+    int n_tiles;
+    long long n_total, shift;
+    long long first[128];    // smallest ordinals of the first pages of its list
     unsigned merge_later;    // shares of the first segment's unit that this CTA has to merge at the end
 };
 
@@ -543,11 +547,19 @@ __device__ __forceinline__ int causal_end(const int (&v)[4], int r) {
     return n;
 }
 
-__device__ __forceinline__ void store_row16(uint16_t* dst, const float* o) {
+// 16 elements of an output row; wide: the launch's output begins at a multiple of 32 bytes.  A warp's store touches 32 rows, and
+// what it costs is the rows, not the bytes: two 16-byte stores take twice as long as one of 32.
+__device__ __forceinline__ void store_row16(uint16_t* dst, const float* o, bool wide) {
+    unsigned v[8];
 #pragma unroll
-    for (int k = 0; k < 2; ++k)
-        *reinterpret_cast<uint4*>(dst + 8 * k) = make_uint4(pack2(o[8 * k], o[8 * k + 1]), pack2(o[8 * k + 2], o[8 * k + 3]),
-                                                            pack2(o[8 * k + 4], o[8 * k + 5]), pack2(o[8 * k + 6], o[8 * k + 7]));
+    for (int k = 0; k < 8; ++k) v[k] = pack2(o[2 * k], o[2 * k + 1]);
+    if (wide) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                     ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+    } else {
+        reinterpret_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
 }
 
 __device__ __forceinline__ uint16_t* out_row(uint16_t* out, const PfRows& w, int mg, unsigned g_magic, int G, int q_heads, int D) {
@@ -661,6 +673,7 @@ __device__ __forceinline__ void merge_shares(const PfPlan& plan, int tail, const
     auto ml_of = [&](int k) { return k > last ? make_float2(-INFINITY, 0.f) : ld_l2(PfSlot<D>(plan, tail, k).ml(g, m)); };
     const int mg = w.m0 + g * 128 + m;
     uint16_t* dst = out_row(out, w, min(mg, w.m_total - 1), plan.g_magic, G, q_heads, D);
+    const bool wide = !(reinterpret_cast<uintptr_t>(out) & 31);
 #pragma unroll 1
     for (; take; take &= take - 1) {
         const int s = __ffs(take) - 1, q1 = share_begin<D>(cut, s + 1);
@@ -718,7 +731,7 @@ __device__ __forceinline__ void merge_shares(const PfPlan& plan, int tail, const
                     }
 #pragma unroll
                     for (int c = 0; c < 16; ++c) if (fa > 0.f) o1[16 * i + c] += a[c] * fa;
-                    if (mg < w.m_total) store_row16(dst + (q + i) * 16, o1 + 16 * i);
+                    if (mg < w.m_total) store_row16(dst + (q + i) * 16, o1 + 16 * i, wide);
                 }
         }
     }
@@ -905,7 +918,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         unsigned char* sQg = sQ + g * TILE_BYTES;
         float* cs_g = reinterpret_cast<float*>(s_cs + g * PF_CS_BYTES);
         float m_ref = -INFINITY, l = 0.f;
-        if (m == 0) { gr.walk.begin(plan); gr.merge_later = 0; gr.more = gr.walk.more(plan); gr.seg.a = 0; gr.seg.e = PF_FRAC; }
+        if (m == 0) { gr.walk.begin(plan); gr.merge_later = 0; gr.known = -1; gr.more = gr.walk.more(plan); gr.seg.a = 0; gr.seg.e = PF_FRAC; }
         bar_sync(BAR_WG + g, 128);
         while (gr.more) {
             bar_sync(BAR_WG + g, 128);        // everybody is through with the previous segment's fields
@@ -917,7 +930,15 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 PfTileRotation<D> rot;
                 int t_lo, n_tok;
                 const bool staged = PfTileRotation<D>::staged(rows, g, plan.g_magic, G, t_lo, n_tok);
-                const PfAsk ask = pf_ask(b, rows);
+                const bool fresh = rows.ci != gr.known;
+                PfAsk ask;
+                if (fresh) {
+                    ask = pf_ask(b, rows);
+                } else {
+                    ask.n_tiles = gr.n_tiles; ask.n_total = gr.n_total; ask.shift = gr.shift; ask.wait_limit = gr.w.wait_limit;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) ask.first[k] = gr.first[lane + 32 * k];
+                }
                 if (staged) rot.load_pos(b, rows, q_pos, m, t_lo, n_tok, m / PfTileRotation<D>::HALF);
                 PfTileRotation<D>::load(rows, g, m, G, plan.g_magic, q_heads, Q, sQg);
                 const PfWork nw = pf_work(b, seg, rows, plan.g_magic, G, ask);
@@ -926,6 +947,11 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 bar_sync(BAR_WG + g, 128);
                 if (m == 0) gr.walk = walk;
+                if (fresh && m < 32) {
+                    if (m == 0) { gr.known = rows.ci; gr.n_tiles = ask.n_tiles; gr.n_total = ask.n_total; gr.shift = ask.shift; }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) gr.first[m + 32 * k] = ask.first[k];
+                }
                 PfTileRotation<D>::rotate(b, rows, nw.shift, q_pos, g, m, plan.g_magic, G, t_lo, staged, cs_g, sQg);
             }
             fence_proxy_async();              // the tile feeds the tensor core
@@ -992,6 +1018,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 const float inv = l > 0.f ? 1.f / l : 0.f;
                 const int mg = mt + m;
                 uint16_t* dst = out_row(out, gr.rows, min(mg, gr.rows.m_total - 1), plan.g_magic, G, q_heads, D);
+                const bool wide = !(reinterpret_cast<uintptr_t>(out) & 31);
 #pragma unroll 1
                 for (int q4 = 0; q4 < D / 32; ++q4) {
                     float o[32];
@@ -1001,7 +1028,10 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     }
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] = have_o ? o[i] * inv : 0.f;
-                    if (mg < gr.rows.m_total) { store_row16(dst + q4 * 32, o); store_row16(dst + q4 * 32 + 16, o + 16); }
+                    if (mg < gr.rows.m_total) {
+                        store_row16(dst + q4 * 32, o, wide);
+                        store_row16(dst + q4 * 32 + 16, o + 16, wide);
+                    }
                 }
             } else if (gr.more) {                                      // the end of a unit that others have begun
                 const unsigned take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[1], g, m, tO, m_ref, l, have_o, 0);
