@@ -8,27 +8,9 @@
 #include "svlm_launch.h"
 #include "svlm_ptx.cuh"
 #include "svlm_rope.cuh"
+#include "svlm_rotate.cuh"
 
 namespace {
-
-struct __align__(16) Bf16x8 { __nv_bfloat162 v[4]; };
-__device__ __forceinline__ Bf16x8 bf16x8(const uint4& x) { return reinterpret_cast<const Bf16x8&>(x); }
-
-// Rotate 8 consecutive pairs (lo[j], hi[j]) by (cs[j], sn[j]) in fp32, round to bf16.
-__device__ __forceinline__ void rotate8(Bf16x8& lo, Bf16x8& hi, const float* cs, const float* sn) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float2 a = __bfloat1622float2(lo.v[j]);
-        const float2 b = __bfloat1622float2(hi.v[j]);
-        float2 ra, rb;
-        ra.x = a.x * cs[2 * j] - b.x * sn[2 * j];
-        rb.x = b.x * cs[2 * j] + a.x * sn[2 * j];
-        ra.y = a.y * cs[2 * j + 1] - b.y * sn[2 * j + 1];
-        rb.y = b.y * cs[2 * j + 1] + a.y * sn[2 * j + 1];
-        lo.v[j] = __float22bfloat162_rn(ra);
-        hi.v[j] = __float22bfloat162_rn(rb);
-    }
-}
 
 // One thread per (token, group of 8 pairs) and per share of the [layer][kv_head] rows (blockIdx.y), so the rotation
 // factors are looked up once per share (table, see svlm_rope.cuh).  What bounds it is latency: source rows, and the chain
@@ -81,25 +63,7 @@ __global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int laye
         int c[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) c[k] = svlm_ptx::ld_l2(cd.slot_c + (size_t)k * cd.n_slots + slot);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int pair = g * 8 + j;
-            const int axis = cd.rope_mode == 0 ? 0 : (pair < cd.sec_t ? 0 : (pair < cd.sec_th ? 1 : 2));
-            const float2 f = svlm_rope_cs_batched(reinterpret_cast<const float2*>(cd.rope_tab), half, pair, axis == 0 ? c[0] : (axis == 1 ? c[1] : c[2]));
-            cs[j] = f.x;
-            sn[j] = f.y;
-        }
-        const int lim = 1 << 16;
-        if (c[0] <= -lim || c[0] >= lim || c[1] <= -lim || c[1] >= lim || c[2] <= -lim || c[2] >= lim) {   // native positions of a long stream
-#pragma unroll 1
-            for (int j = 0; j < 8; ++j) {
-                const int pair = g * 8 + j;
-                const int axis = cd.rope_mode == 0 ? 0 : (pair < cd.sec_t ? 0 : (pair < cd.sec_th ? 1 : 2));
-                const float2 f = svlm_rope_cs(reinterpret_cast<const float2*>(cd.rope_tab), half, pair, axis == 0 ? c[0] : (axis == 1 ? c[1] : c[2]), cd.theta[pair]);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) if (q == j) { cs[q] = f.x; sn[q] = f.y; }
-            }
-        }
+        first_rotation(cd, g, c, cs, sn);
         if (gid != n_total - n + i) slot = -1;
     }
     if (early) {

@@ -66,11 +66,16 @@ inline int svlm_sm_count() {
 // metadata (svlm_meta.cu).  Where one of these fails, whatever was to follow it must not be launched: it would take the
 // metadata of the operation before for its own.
 cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n, cudaStream_t st);
-cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st);
+// rotate: the launch re-rotates the moved keys too (svlm_evict_in_one; otherwise svlm_launch_evict_rotate has to follow)
+bool svlm_evict_in_one(const SvlmCacheDev& cd);
+cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, bool rotate, cudaStream_t st);
+// an append's metadata and its keys and values (svlm_launch_kv_write's) in one launch, where svlm_append_in_one says so
+bool svlm_append_in_one(const SvlmCacheDev& cd, int layer, int n);
+cudaError_t svlm_launch_append_in_one(const SvlmCacheDev& cd, int layer, const void* K, const void* V, const unsigned char* types, const int* pos, int n, cudaStream_t st);
 // batched forms, one block per cache: types [n_caches][n], pos [n_caches][n](x3); every cache has the geometry of geom
 cudaError_t svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, const unsigned char* types, const int* pos, int n,
                                    cudaStream_t st);
-cudaError_t svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st);
+cudaError_t svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, bool rotate, cudaStream_t st);
 
 // small transfers from and to page-locked host memory (svlm_host_io.cu); 16-byte aligned, sizes rounded up to 16
 cudaError_t svlm_launch_host_in(void* dst, const void* src, size_t bytes, cudaStream_t st);

@@ -2,9 +2,13 @@
 // of eviction (paper Section 2.1, "Streaming-aware KV Cache" and "Contiguous RoPE").  Integer work
 // only; one CTA each (a few thousand records), results must be bit-exact.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+
 #include "svlm_dev.h"
 #include "svlm_launch.h"
 #include "svlm_ptx.cuh"
+#include "svlm_rotate.cuh"
 
 namespace {
 
@@ -284,8 +288,10 @@ __device__ __forceinline__ void append_one_body(const SvlmCacheDev& cd, const un
 // Append of up to blockDim tokens, one per thread (a chunk): the general kernel's bookkeeping in three dependent round
 // trips (control block with types and positions; page table or free stack; ordinals for the page list) and two block
 // barriers.  Every warp adds up all warps' totals for itself, and every thread knows which page of the free stack its
-// ring page becomes, so that nothing waits for one thread's page allocation.
-__device__ __forceinline__ void append_few_body(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n) {
+// ring page becomes, so that nothing waits for one thread's page allocation.  placed(slot, c) is called for the thread's token
+// with its slot and position.  False if the append was dropped (the same in every thread).
+template <typename Placed>
+__device__ __forceinline__ bool append_few_body(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n, Placed placed) {
     __shared__ int s_text[META_WARPS], s_sink[META_WARPS];       // per warp: text tokens; text tokens among the any-type sinks
     __shared__ long long s_top[META_WARPS];                      // per warp: largest native index + 1
     SvlmCtrl* ctrl = cd.ctrl;
@@ -364,7 +370,7 @@ __device__ __forceinline__ void append_few_body(const SvlmCacheDev& cd, const un
             ctrl->append_n = 0;
             if (ctrl->status == 0) ctrl->status = -2;   // SVLM_ERR_CAPACITY
         }
-        return;
+        return false;
     }
     // ring page k of type t: an open one from the page table, a new one from the free stack (text ring's first)
     auto page_of = [&](int t, long long k) {
@@ -390,7 +396,9 @@ __device__ __forceinline__ void append_few_body(const SvlmCacheDev& cd, const un
         cd.slot_a[slot] = (int)max(0ll, top - cur_before);
         cd.slot_delta[slot] = 0;
         cd.new_slot[tid] = slot;
-        for (int k = 0; k < 3; ++k) cd.slot_c[k * cd.n_slots + slot] = (int)(p[k] - shift);
+        const int c[3] = {(int)(p[0] - shift), (int)(p[1] - shift), (int)(p[2] - shift)};
+        for (int k = 0; k < 3; ++k) cd.slot_c[k * cd.n_slots + slot] = c[k];
+        placed(slot, c);
     }
     // the list of active pages: which page and which offsets are known already, the ordinals behind the barrier
     const TileList tl(sink_fill1, ring_lo0, ring_n1);
@@ -418,6 +426,7 @@ __device__ __forceinline__ void append_few_body(const SvlmCacheDev& cd, const un
         ctrl->n_stored = n_stored0 + n;
         ctrl->append_n = n;
     }
+    return true;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -589,12 +598,17 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // are dealt out among the CTAs, the last CTA writes the page list, and CTA 0 alone changes what the others read (behind
 // the cluster barrier) and keeps the books.  The chain had ten round trips, one stage after another: 11.9 us at config 3,
 // 7 now (append and eviction of a chunk in a row: 22.6 -> 17.4 us).
+//
+// ROTATE: a single CTA serves the cache (a retained token per thread at most) and re-rotates the moved keys as well, where
+// that is so little that a launch of its own costs more (svlm_evict_in_one).
+template <bool ROTATE>
 __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
     const int crank = (int)cluster_ctarank(), n_ctas = (int)cluster_nctarank();
     __shared__ long long wbuf64[2][META_WARPS];
     __shared__ long long s_gid[EV_SMEM];       // ordinals of the evicted tokens: text ring, then vision ring
     __shared__ long long s_pref[EV_SMEM + 2];  // exclusive prefix sums of their advances (n+1 entries per ring)
     __shared__ int s_moved;
+    __shared__ int2 moved_slots[ROTATE ? META_THREADS : 1]; // slot and shift of the retained tokens (slot -1: none, or not moved)
     SvlmCtrl* ctrl = cd.ctrl;
     const int tid = threadIdx.x;
     if (tid == 0) s_moved = 0;
@@ -690,6 +704,7 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
     cluster_arrive();    // this CTA has read the control block and the evicted slots' metadata
 
     int moved = 0;
+    if (ROTATE) moved_slots[tid] = make_int2(-1, 0);
     for (long long base = base0; base < n_kept; base += (long long)n_ctas * EV_PER_CTA) {
         if (base != base0) { kept_slots(base); kept_data(); }
         int E[KEPT_BATCH];
@@ -707,6 +722,7 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
             cd.slot_delta[k_slot[u]] = E[u];
             if (E[u]) {
                 moved = 1;
+                if (ROTATE && u == 0) moved_slots[tid] = make_int2(k_slot[u], E[u]);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) cd.slot_c[k * cd.n_slots + k_slot[u]] = k_c[u][k] - E[u];
             }
@@ -759,6 +775,26 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
         if (n_ctas == 1) ctrl->evict_moved = s_moved;
         else if (s_moved) atomicOr(&ctrl->evict_moved, 1);
     }
+    if (ROTATE && s_moved) {                       // (moved_slots was complete at the barrier above)
+        const int half = cd.head_dim / 2, gshift = cd.head_dim == 128 ? 3 : 2, rows = cd.layers * cd.kv_heads;
+        const size_t stride = (size_t)cd.n_slots * cd.head_dim;
+        for (int i = tid; i < (int)n_kept << gshift; i += META_THREADS) {
+            const int2 mv = moved_slots[i >> gshift];
+            if (mv.x < 0) continue;
+            const int g = i & ((1 << gshift) - 1);
+            uint16_t* at = cd.K + (size_t)mv.x * cd.head_dim + g * 8;
+            const int c[3] = {-mv.y, -mv.y, -mv.y};      // all three indices of a token shift by the same amount
+            float cs[8], sn[8];
+            first_rotation(cd, g, c, cs, sn);
+#pragma unroll 2
+            for (int r = 0; r < rows; ++r, at += stride) {
+                Bf16x8 lo = *reinterpret_cast<const Bf16x8*>(at), hi = *reinterpret_cast<const Bf16x8*>(at + half);
+                rotate8(lo, hi, cs, sn);
+                *reinterpret_cast<Bf16x8*>(at) = lo;
+                *reinterpret_cast<Bf16x8*>(at + half) = hi;
+            }
+        }
+    }
 }
 
 // All of these kernels are launched programmatically (svlm_launch_chained): they start while their predecessor ends, wait
@@ -775,7 +811,7 @@ __device__ __forceinline__ void append_form(const SvlmCacheDev& cd, const unsign
     svlm_ptx::pdl_wait();
     if (FORM != APPEND_ONE) svlm_ptx::pdl_launch_dependents();
     if (FORM == APPEND_ONE) append_one_body(cd, types, pos);
-    else if (FORM == APPEND_FEW) append_few_body(cd, types, pos, n);
+    else if (FORM == APPEND_FEW) append_few_body(cd, types, pos, n, [](int, const int (&)[3]) {});
     else append_meta_body(cd, types, pos, n);
 }
 
@@ -793,18 +829,65 @@ __global__ void __launch_bounds__(FORM == APPEND_ONE ? ONE_THREADS : META_THREAD
     append_form<FORM>(s_cd, types + (size_t)blockIdx.x * n, pos + (size_t)blockIdx.x * n * (s_cd.rope_mode == 0 ? 1 : 3), n);
 }
 
+// Append of a few tokens with the write of their keys and values in one launch: the block that places the tokens also rotates
+// and stores their rows, a thread per (token, 8 pairs) and row of [layer][kv head].  The first rows are asked for before
+// the metadata, which they have nothing to do with.
+__global__ void __launch_bounds__(META_THREADS) append_meta_write_kernel(SvlmCacheDev cd, const unsigned char* types, const int* pos, int n, const uint16_t* K,
+                                                                         const uint16_t* V, int layers) {
+    __shared__ int s_slot[META_THREADS], s_c[META_THREADS][3];
+    svlm_ptx::pdl_wait();
+    svlm_ptx::pdl_launch_dependents();
+    const int half = cd.head_dim / 2, gshift = cd.head_dim == 128 ? 3 : 2, d = cd.head_dim, rows = layers * cd.kv_heads;
+    const int items = (n * rows) << gshift;           // (small: APPEND_WRITE_ELEMENTS)
+    Bf16x8 lo, hi;
+    uint4 vlo, vhi;
+    auto row_of = [&](int i) { return (i >> gshift) % rows; };                   // the same token's rows lie together in a layer
+    auto token_of = [&](int i) { return (i >> gshift) / rows; };
+    auto load = [&](int i) {
+        const int r = row_of(i), l = r / cd.kv_heads, h = r - l * cd.kv_heads;
+        const size_t src = (((size_t)l * n + token_of(i)) * cd.kv_heads + h) * d + (i & ((1 << gshift) - 1)) * 8;
+        lo = bf16x8(svlm_ptx::ld_in(reinterpret_cast<const uint4*>(K + src)));
+        hi = bf16x8(svlm_ptx::ld_in(reinterpret_cast<const uint4*>(K + src + half)));
+        vlo = svlm_ptx::ld_in(reinterpret_cast<const uint4*>(V + src));
+        vhi = svlm_ptx::ld_in(reinterpret_cast<const uint4*>(V + src + half));
+    };
+    const int tid = threadIdx.x;
+    if (tid < items) load(tid);
+    const bool ok = append_few_body(cd, types, pos, n, [&](int slot, const int (&c)[3]) {
+        s_slot[tid] = slot;
+        for (int k = 0; k < 3; ++k) s_c[tid][k] = c[k];
+    });
+    if (!ok) return;
+    __syncthreads();
+    for (int i = tid; i < items; i += blockDim.x) {
+        if (i != tid) load(i);
+        const int token = token_of(i), g = i & ((1 << gshift) - 1);
+        const int c[3] = {s_c[token][0], s_c[token][1], s_c[token][2]};
+        float cs[8], sn[8];
+        first_rotation(cd, g, c, cs, sn);
+        rotate8(lo, hi, cs, sn);
+        const size_t dst = ((size_t)row_of(i) * cd.n_slots + s_slot[token]) * d + g * 8;
+        *reinterpret_cast<Bf16x8*>(cd.K + dst) = lo;
+        *reinterpret_cast<Bf16x8*>(cd.K + dst + half) = hi;
+        *reinterpret_cast<uint4*>(cd.V + dst) = vlo;
+        *reinterpret_cast<uint4*>(cd.V + dst + half) = vhi;
+    }
+}
+
+template <bool ROTATE>
 __global__ void __launch_bounds__(META_THREADS) evict_meta_kernel(SvlmCacheDev cd) {
     svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();
-    evict_meta_body(cd);
+    evict_meta_body<ROTATE>(cd);
 }
 
+template <bool ROTATE>
 __global__ void __launch_bounds__(META_THREADS) evict_meta_batch_kernel(SvlmCacheList list) {
     __shared__ SvlmCacheDev s_cd;
     svlm_load_desc(&s_cd, list.cd[blockIdx.x / cluster_nctarank()]);
     svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();
-    evict_meta_body(s_cd);
+    evict_meta_body<ROTATE>(s_cd);
 }
 
 int append_form_of(int n, int n_pages) {
@@ -824,10 +907,32 @@ cudaError_t svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmC
     return svlm_launch_chained(kernel, dim3(list.n), dim3(append_threads(form, n)), 0, 1, st, list, types, pos, n);
 }
 
-cudaError_t svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, cudaStream_t st) {
-    int c = evict_cluster(geom.n_slots);            // (the caches share the number of pages, not the exact capacity)
+// One launch for a whole append or eviction of a small cache.  The lines: what one block moves by itself against a second launch
+// on all SMs.  Append and eviction of a chunk in a row, replayed from a graph, us: 2.4 K elements of new keys written in the
+// same launch 14.6, in a second one 15.9, 32 K 25.2 and 17.4; 12.5 K elements of kept keys re-rotated in the same launch 15.2,
+// in a second one 15.9, 35 K 17.2 and 17.4, 155 K 32.9 and 17.7.  (By plain calls a launch less saves the host 2 us more.)
+constexpr long long APPEND_WRITE_ELEMENTS = 8192;      // of the appended keys
+constexpr long long EVICT_ROTATE_ELEMENTS = 16384;     // of the keys that the windows keep
+static_assert(EVICT_ROTATE_ELEMENTS / 64 <= META_THREADS, "a thread per retained token (heads have 64 dims at least)");
+bool svlm_append_in_one(const SvlmCacheDev& cd, int layer, int n) {
+    return n <= META_THREADS && (long long)n * (layer < 0 ? cd.layers : 1) * cd.kv_heads * cd.head_dim <= APPEND_WRITE_ELEMENTS;
+}
+bool svlm_evict_in_one(const SvlmCacheDev& cd) {
+    const long long kept = std::min((long long)cd.n_sink + cd.vision_window + cd.text_window, (long long)cd.n_slots);
+    return kept * cd.layers * cd.kv_heads * cd.head_dim <= EVICT_ROTATE_ELEMENTS;
+}
+
+cudaError_t svlm_launch_append_in_one(const SvlmCacheDev& cd, int layer, const void* K, const void* V, const unsigned char* types, const int* pos, int n, cudaStream_t st) {
+    const int layers = layer < 0 ? cd.layers : 1, items = n * layers * cd.kv_heads * (cd.head_dim / 16);
+    const int threads = std::min(META_THREADS, std::max(append_threads(APPEND_FEW, n), (items + 31) / 32 * 32));
+    return svlm_launch_chained(append_meta_write_kernel, dim3(1), dim3(threads), 0, 1, st, cd, types, pos, n, static_cast<const uint16_t*>(K),
+                               static_cast<const uint16_t*>(V), layers);
+}
+
+cudaError_t svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, bool rotate, cudaStream_t st) {
+    int c = rotate ? 1 : evict_cluster(geom.n_slots);            // (the caches share the number of pages, not the exact capacity)
     while (c > 1 && c * list.n > 96) c /= 2;        // 16 clusters of 8 do not find room at once (a CTA fills an SM)
-    return svlm_launch_chained(evict_meta_batch_kernel, dim3(c * list.n), dim3(META_THREADS), 0, c, st, list);
+    return svlm_launch_chained(rotate ? evict_meta_batch_kernel<true> : evict_meta_batch_kernel<false>, dim3(c * list.n), dim3(META_THREADS), 0, c, st, list);
 }
 
 cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n,
@@ -837,7 +942,7 @@ cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char*
     return svlm_launch_chained(kernel, dim3(1), dim3(append_threads(form, n)), 0, 1, st, cd, types, pos, n);
 }
 
-cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, cudaStream_t st) {
-    const int c = evict_cluster(cd.capacity);
-    return svlm_launch_chained(evict_meta_kernel, dim3(c), dim3(META_THREADS), 0, c, st, cd);
+cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, bool rotate, cudaStream_t st) {
+    const int c = rotate ? 1 : evict_cluster(cd.capacity);
+    return svlm_launch_chained(rotate ? evict_meta_kernel<true> : evict_meta_kernel<false>, dim3(c), dim3(META_THREADS), 0, c, st, cd);
 }

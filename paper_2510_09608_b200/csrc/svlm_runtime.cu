@@ -502,6 +502,11 @@ int svlm_cache_append(svlm_cache* c, int layer, const void* K, const void* V, co
         if (!token_type || !pos) return SVLM_ERR_ARG;
         if (n > c->dev.capacity) return SVLM_ERR_CAPACITY;
         c->configured_locked = true;
+        if (svlm_append_in_one(c->dev, layer, n)) {
+            SVLM_CUDA(svlm_launch_append_in_one(c->dev, layer, K, V, token_type, pos, n, c->stream));
+            note_append(c, n);
+            return SVLM_OK;
+        }
         SVLM_CUDA(svlm_launch_append_meta(c->dev, token_type, pos, n, c->stream));
         note_append(c, n);
     } else if (n != c->pending_n) {
@@ -567,9 +572,10 @@ int svlm_cache_evict(svlm_cache* c) {
     if (!c) return SVLM_ERR_ARG;
     DeviceGuard guard(c->device);
     c->last_decode_layer = -1;
-    SVLM_CUDA(svlm_launch_evict_meta(c->dev, c->stream));
+    const bool in_one = c->dev.contiguous && svlm_evict_in_one(c->dev);
+    SVLM_CUDA(svlm_launch_evict_meta(c->dev, in_one, c->stream));
     note_evict(c);
-    if (c->dev.contiguous) SVLM_CUDA(svlm_launch_evict_rotate(c->dev, c->stream));
+    if (c->dev.contiguous && !in_one) SVLM_CUDA(svlm_launch_evict_rotate(c->dev, c->stream));
     return SVLM_OK;
 }
 
@@ -579,14 +585,15 @@ int svlm_cache_evict_batched(svlm_cache* const* caches, int n_caches) {
     if (rc != SVLM_OK) return rc;
     svlm_cache* c0 = caches[0];
     DeviceGuard guard(c0->device);
-    bool rotate = false;
+    bool rotate = false, in_one = true;
     for (int i = 0; i < n_caches; ++i) {
+        in_one = in_one && svlm_evict_in_one(caches[i]->dev);
         caches[i]->last_decode_layer = -1;
         rotate = rotate || caches[i]->dev.contiguous;   // a cache with native positions never sets evict_moved
     }
-    SVLM_CUDA(svlm_launch_evict_meta_batch(list, c0->dev, c0->stream));
+    SVLM_CUDA(svlm_launch_evict_meta_batch(list, c0->dev, rotate && in_one, c0->stream));
     for (int i = 0; i < n_caches; ++i) note_evict(caches[i]);
-    if (rotate) SVLM_CUDA(svlm_launch_evict_rotate_batch(list, c0->dev, c0->stream));
+    if (rotate && !in_one) SVLM_CUDA(svlm_launch_evict_rotate_batch(list, c0->dev, c0->stream));
     return SVLM_OK;
 }
 

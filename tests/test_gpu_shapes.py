@@ -130,6 +130,30 @@ def test_append_sizes_and_large_evictions(sizes, sink_any):
     s.check_kv(0)
 
 
+# --- appends and evictions of small caches in one launch each, at the lines to the two-launch forms: as many new rows as one
+# --- block writes and one more, as many kept tokens as it re-rotates and one more, all layers at once, positions beyond 2^16
+@pytest.mark.parametrize("over", [0, 1])
+@pytest.mark.parametrize("d,hk,layers,sizes,capacity,base,contiguous", [
+    (64, 1, 1, (37, 128, 129, 1, 31), 256, 0, True), (128, 2, 1, (32, 33, 1, 3), 200, 0, True), (64, 1, 3, (42, 43, 33, 2), 100, 0, True),
+    (64, 2, 2, (1, 2, 32, 33), 100, 70000, False), (128, 1, 2, (7, 31, 32, 33), 70, 70000, True), (64, 1, 1, (40, 200), 2600, 0, True)])
+def test_small_caches_in_one_launch(d, hk, layers, sizes, capacity, base, contiguous, over):
+    from harness import SideBySide
+    keep = 16384 // (d * hk * layers) + over                  # tokens the windows keep: one block re-rotates them, or a launch of its own
+    wl = _wl(2, layers=layers, q_heads=hk, kv_heads=hk, head_dim=d, rope_mode=0, sections=(d // 2, 0, 0), n_sink=6, vision_window=keep - 26, text_window=20)
+    s = SideBySide(wl, capacity=max(capacity, keep + 4 + max(sizes)), contiguous=contiguous)
+    rng = np.random.default_rng(sum(sizes))
+    gid, pos = 0, base
+    for rep in range(3):
+        for n in sizes:
+            s._append(np.arange(gid, gid + n), rng.integers(0, 2, n).astype(np.uint8), (pos + np.arange(n)).astype(np.int32))
+            gid, pos = gid + n, pos + n + (gid % 3)
+            s.check_metadata()
+            s.evict()
+            s.check_metadata()
+            for layer in range(layers):
+                s.check_kv(layer)
+
+
 # --- decode: one to three units per warp, a second round, the step to the streaming kernel; one, two and three caches
 @pytest.mark.parametrize("d,hq,hk,vw,streams", [
     (128, 28, 4, 100, 1), (64, 5, 1, 40, 1), (128, 8, 8, 4700, 1), (128, 8, 8, 6300, 1), (64, 16, 8, 6300, 1),
