@@ -32,6 +32,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "svlm_append_one.cuh"
 #include "svlm_dev.h"
 #include "svlm_launch.h"
 #include "svlm_ptx.cuh"
@@ -139,6 +140,111 @@ __device__ __forceinline__ void st_tagged2(void* p, unsigned a, unsigned b, unsi
 }
 __device__ __forceinline__ void ld_tagged2(const void* p, unsigned long long& a, unsigned long long& b) {
     asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+
+// ---- a decode step that appends its token itself ------------------------------------------------------------------
+//
+// Where one launch attends in all of a cache's layers (caches of one layer), the token's bookkeeping needs no launch of its own in front: every CTA works out from the old metadata what the token changes, uses the
+// list of pages as it will be, and counts itself as through with the old metadata; the last one to do so writes the change
+// down at its end (nobody waits).  A launch and its chain of round trips less in front of each step: one layer of 4/1 heads of
+// 64 over 200 keys 8.9 -> 7.1 us, 16 streams of 4 heads of 128 over 9216 keys 56.4 -> 55.2.  A step that is followed by
+// another layer's keeps the launch of its own: that layer's kernel reads the metadata ahead, while this one runs.  So do all
+// layers in one call, whose inputs may be in host memory: there every CTA would fetch type and position over the bus
+// (a second of 28 layers end to end 5.12 -> 5.29 ms).
+struct DecNoAppend { static constexpr bool on = false; };
+struct DecAppend {
+    static constexpr bool on = true;
+    const unsigned char* types;      // [n_caches]; the positions are the queries'
+    SvlmCacheList list;
+};
+__device__ __forceinline__ SvlmOneRule dec_rule(const DecAppend& app, int ci) { return SvlmOneRule(*app.list.cd[ci]); }
+struct DecNoRule {};
+__device__ __forceinline__ DecNoRule dec_rule(const DecNoAppend&, int) { return {}; }
+struct DecOne {                      // in shared memory
+    SvlmOneToken token;
+    int page;                        // of the list's entry that grows, if none appears
+    int slot;                        // a sink's, or in a page that appears
+};
+// The list of active pages as it will be, into tile_pk (page | lo << 16 | hi << 24), by all THREADS of the block; returns
+// the number of its entries, the token's slot (-1: it does not fit) and the total shift.  Ends with a barrier; every
+// thread has then read what it needs of the old metadata.
+template <int THREADS, int MAX_TILES>
+__device__ __forceinline__ int list_with_token(const SvlmAttendBatch& b, const SvlmAttendView& vw, const DecAppend& app, const SvlmOneRule& rule,
+                                               const int* q_pos, int ci, DecOne& one, unsigned* tile_pk, int& new_slot, long long& shift) {
+    constexpr int N = (MAX_TILES + THREADS - 1) / THREADS;
+    const int n_pages = b.n_slots / SVLM_PAGE;
+    int4 tl[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if ((int)threadIdx.x + k * THREADS < n_pages) tl[k] = ld_l2(reinterpret_cast<const int4*>(vw.tiles + threadIdx.x + k * THREADS));
+    const SvlmCacheDev& cd = *app.list.cd[ci];
+    const SvlmCtrl* ct = vw.ctrl;
+    shift = ld_l2(&ct->shift_total);
+    if (threadIdx.x < 32) {          // one warp for all: its lanes' values are the same
+        SvlmCtrl c;
+        c.n_total = ld_l2(&ct->n_total);
+        c.cursor = ld_l2(&ct->cursor);
+        c.shift_total = shift;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) { c.n_type[k] = ld_l2(&ct->n_type[k]); c.ring_n[k] = ld_l2(&ct->ring_n[k]); c.ring_lo[k] = ld_l2(&ct->ring_lo[k]); }
+        c.sink_fill = ld_l2(&ct->sink_fill);
+        c.n_stored = ld_l2(&ct->n_stored);
+        c.free_top = ld_l2(&ct->free_top);
+        c.n_tiles = ld_l2(&ct->n_tiles);
+        const int pw = b.rope_mode == 0 ? 0 : 1;
+        const int* qp = q_pos + (size_t)ci * (2 * pw + 1);
+        const int p[3] = {ld_in(qp), ld_in(qp + pw), ld_in(qp + 2 * pw)};
+        const SvlmOneToken t = svlm_one_token(rule, c, ld_in(app.types + ci) ? 1 : 0, p);
+        if (threadIdx.x == 0) {
+            one.token = t;
+            one.page = -1;
+            one.slot = t.ok && (t.adds || t.is_sink) ? svlm_one_slot(cd, t) : 0;
+        }
+    }
+    __syncthreads();
+    const bool ok = one.token.ok, adds = one.token.adds;
+    const int at = one.token.at, n0 = one.token.n_tiles0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int i = threadIdx.x + k * THREADS;
+        if (i >= n0) continue;
+        const bool grows = ok && !adds && i == at;
+        if (grows) one.page = tl[k].x;
+        const int j = i + (ok && adds && i >= at);
+        if (j < MAX_TILES) tile_pk[j] = (unsigned)tl[k].x | ((unsigned)tl[k].y << 16) | ((unsigned)(tl[k].z + grows) << 24);
+    }
+    if (threadIdx.x == 0 && ok && adds && at < MAX_TILES) {
+        const int off = one.slot % SVLM_PAGE;
+        tile_pk[at] = (unsigned)(one.slot / SVLM_PAGE) | ((unsigned)off << 16) | ((unsigned)(off + 1) << 24);
+    }
+    __syncthreads();
+    new_slot = !ok ? -1 : (adds || one.token.is_sink ? one.slot : one.page * SVLM_PAGE + (int)(one.token.u % SVLM_PAGE));
+    return min(n0 + (ok && adds), MAX_TILES);
+}
+// By one thread, behind the barrier above: counts the CTA in; returns how many were there before (not to be looked at before
+// the thread has nothing better to do: the answer takes a round trip).
+__device__ __forceinline__ unsigned through_with_metadata(const SvlmAttendView& vw) {
+    unsigned prev;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(prev) : "l"(&vw.ctrl->append_seen) : "memory");
+    return prev;
+}
+// By that thread's warp, later: in the last CTA of the cache's `ctas` to be counted (before: of lane 0) the token's change is written down.
+__device__ __forceinline__ void write_token_down(const DecAppend& app, int ci, const DecOne& one, int slot, unsigned before, unsigned ctas) {
+    if (__shfl_sync(0xffffffffu, before, 0) + 1 != ctas) return;
+    const SvlmCacheDev& cd = *app.list.cd[ci];
+    if ((threadIdx.x & 31) == 0) cd.ctrl->append_seen = 0;      // ready for the next launch
+    const SvlmOneToken& t = one.token;
+    const int lane = threadIdx.x & 31;
+    if (t.ok && t.adds)                      // entries behind the new one move up by one, from the end
+        for (int hi = t.n_tiles0; hi > t.at; hi -= 32) {
+            const int i = hi - 1 - lane;
+            SvlmTile tile;
+            if (i >= t.at) tile = cd.tiles[i];
+            __syncwarp();
+            if (i >= t.at) cd.tiles[i + 1] = tile;
+            __syncwarp();
+        }
+    if (lane == 0) svlm_one_commit(cd, t, slot);
 }
 
 // ---- the part both kernels share: from the consumer warps' accumulators to the output -----------------------
@@ -482,6 +588,7 @@ struct DecShared {
     int abort_flag;
     int last;
     unsigned tile_pk[DEC_MAX_TILES];   // page | lo << 16 | hi << 24
+    DecOne one;                        // a step that appends its token itself
 };
 
 // Position of a 16-byte chunk inside a stage: 64-dim panels of [32 keys][128 B], chunks XOR-swizzled
@@ -490,11 +597,11 @@ __device__ __forceinline__ int sw_off(int key, int chunk) {
     return (chunk >> 3) * (SUB * 128) + key * 128 + (((chunk & 7) ^ (key & 7)) << 4);
 }
 
-template <int D>
+template <int D, typename Append>
 __global__ void __launch_bounds__(DEC_THREADS, 2)
 decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t* Q,
               const int* q_pos, int q_heads, uint16_t* __restrict__ out, int splits,
-              const uint16_t* Knew, const uint16_t* Vnew, int early_loads) {
+              const uint16_t* Knew, const uint16_t* Vnew, int early_loads, Append app) {
     constexpr int KB = D / 64;                       // 64-dim panels per row
     constexpr int PANEL_BYTES = SUB * 128;
     constexpr int STAGE_BYTES = 2 * KB * PANEL_BYTES;   // K panels then V panels
@@ -528,13 +635,23 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
     // otherwise after the grid-dependency wait.  A kernel that has to wait does so BEFORE it lets its
     // successor start: a successor with early loads then only ever runs behind a completed metadata
     // kernel (whatever that kernel's own trigger), not merely behind one that has been launched.
+    const auto rule = dec_rule(app, ci);      // (read ahead: nothing in the stream writes it)
     if (!early_loads) pdl_wait();
     pdl_launch_dependents();
-    const int n_tiles = min(ld_l2(&vw.ctrl->n_tiles), DEC_MAX_TILES);
     const unsigned wait_limit = ld_l2(&vw.ctrl->wait_limit);
-    for (int i = threadIdx.x; i < n_tiles; i += DEC_THREADS) {
-        const int4 tl = ld_l2(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
-        sh.tile_pk[i] = (unsigned)tl.x | ((unsigned)tl.y << 16) | ((unsigned)tl.z << 24);
+    int n_tiles, new_slot = -1;
+    long long shift;
+    unsigned before = 0;               // (of the producer's thread)
+    if constexpr (Append::on) {
+        n_tiles = list_with_token<DEC_THREADS, DEC_MAX_TILES>(b, vw, app, rule, q_pos, ci, sh.one, sh.tile_pk, new_slot, shift);
+        if (warp == DEC_CWARPS && lane == 0) before = through_with_metadata(vw);
+    } else {
+        n_tiles = min(ld_l2(&vw.ctrl->n_tiles), DEC_MAX_TILES);
+        for (int i = threadIdx.x; i < n_tiles; i += DEC_THREADS) {
+            const int4 tl = ld_l2(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
+            sh.tile_pk[i] = (unsigned)tl.x | ((unsigned)tl.y << 16) | ((unsigned)tl.z << 24);
+        }
+        shift = ld_l2(&vw.ctrl->shift_total);
     }
     if (early_loads && threadIdx.x < 3) {
         // Bring the call's own small inputs towards L2 while the previous kernel still runs (a hint:
@@ -546,14 +663,12 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
         for (int o = 0; o < bytes; o += 128)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p) + o));
     }
-    const long long shift = ld_l2(&vw.ctrl->shift_total);
     // the new token of a fused step: where it lives and whether it is still stored there
-    int new_slot = -1;
-    if (Knew && warp < DEC_CWARPS) {
+    if (!Append::on && Knew && warp < DEC_CWARPS) {
         const int s = ld_l2(vw.new_slot);
         if (ld_l2(&vw.ctrl->append_n) == 1 && ld_l2(vw.slot_gid + s) == ld_l2(&vw.ctrl->n_total) - 1) new_slot = s;
     }
-    __syncthreads();
+    if (!Append::on) __syncthreads();
 
     const int total_q = 4 * n_tiles;
     const int q0 = (int)((long long)split * total_q / splits), q1 = (int)((long long)(split + 1) * total_q / splits);
@@ -609,6 +724,10 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
                 ++it;
             }
         }
+        if constexpr (Append::on) {
+            __syncwarp();
+            write_token_down(app, ci, sh.one, new_slot, before, gridDim.x * gridDim.y * n_layers);
+        }
     } else {
         // ================= consumers =================
         const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
@@ -617,7 +736,7 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
             const int pair = threadIdx.x & (HALF - 1);
             const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
             float2 cs;
-            if (new_slot >= 0) {
+            if (!Append::on && new_slot >= 0) {
                 // fused step: the query is the appended token, its position is already in the metadata,
                 // so the rotation factors do not have to wait for the previous kernel
                 cs = svlm_rope_cs(tab, HALF, pair, ld_l2(vw.slot_c + (size_t)axis * b.n_slots + new_slot), b.theta[pair]);
@@ -826,6 +945,7 @@ struct LayShared {
     uint16_t q[8 * (128 + QROW_PAD)];  // rotated query rows
     uint16_t fresh[2 * 128];           // fused step: the new token's rotated key [D], then its value [D]
     unsigned tile_pk[DEC_MAX_TILES];   // page | lo << 16 | hi << 24
+    DecOne one;                        // a step that appends its token itself
 };
 
 // Position of a 16-byte chunk inside a unit's slot: 64-dim panels of [16 keys][128 B], chunks XOR-swizzled by
@@ -835,11 +955,11 @@ __device__ __forceinline__ int lay_off(int key, int chunk) {
 }
 
 // ANYWHERE: Q, Knew or Vnew does not begin at a word (a choice inside the kernel cost 4 % of a layer-step).
-template <int D, bool ANYWHERE>
+template <int D, bool ANYWHERE, typename Append>
 __global__ void __launch_bounds__(LAY_THREADS, 2)
 decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* q_pos, int q_heads,
                     uint16_t* __restrict__ out, int splits, const uint16_t* Knew,
-                    const uint16_t* Vnew, int early_loads TRACE_PARAM) {
+                    const uint16_t* Vnew, int early_loads, Append app TRACE_PARAM) {
     if (threadIdx.x == 0) STAMP(0);                  // kernel entry
     constexpr int CH = D / 8;                        // 16-byte chunks per row
     constexpr int ITEM_BYTES = UNIT * D * 2;         // K or V of one unit
@@ -865,12 +985,22 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* 
     // otherwise after the grid-dependency wait.  A kernel that has to wait does so BEFORE it lets its
     // successor start: a successor with early loads then only ever runs behind a completed metadata
     // kernel (whatever that kernel's own trigger), not merely behind one that has been launched.
+    const auto rule = dec_rule(app, ci);      // (read ahead: nothing in the stream writes it)
     if (!early_loads) pdl_wait();
     pdl_launch_dependents();
-    const int n_tiles = min(ld_l2(&vw.ctrl->n_tiles), DEC_MAX_TILES);
-    for (int i = threadIdx.x; i < n_tiles; i += LAY_THREADS) {
-        const int4 tl = ld_l2(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
-        sh.tile_pk[i] = (unsigned)tl.x | ((unsigned)tl.y << 16) | ((unsigned)tl.z << 24);
+    int n_tiles, new_slot = -1;
+    long long shift;
+    unsigned before = 0;                             // (of the last warp's first thread)
+    if constexpr (Append::on) {
+        n_tiles = list_with_token<LAY_THREADS, DEC_MAX_TILES>(b, vw, app, rule, q_pos, ci, sh.one, sh.tile_pk, new_slot, shift);
+        if (warp == DEC_CWARPS - 1 && lane == 0) before = through_with_metadata(vw);
+    } else {
+        n_tiles = min(ld_l2(&vw.ctrl->n_tiles), DEC_MAX_TILES);
+        for (int i = threadIdx.x; i < n_tiles; i += LAY_THREADS) {
+            const int4 tl = ld_l2(reinterpret_cast<const int4*>(vw.tiles + i));   // page, lo, hi, pad
+            sh.tile_pk[i] = (unsigned)tl.x | ((unsigned)tl.y << 16) | ((unsigned)tl.z << 24);
+        }
+        shift = ld_l2(&vw.ctrl->shift_total);
     }
     if (early_loads && warp == DEC_CWARPS - 1 && lane < 3) {
         // Bring the call's own small inputs towards L2 while the previous kernel still runs (a hint:
@@ -883,10 +1013,8 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* 
             asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p) + o));
     }
     if (threadIdx.x == 0) sh.wait_limit = (int)min(ld_l2(&vw.ctrl->wait_limit), 0x7fffffffu);
-    const long long shift = ld_l2(&vw.ctrl->shift_total);
     // the new token of a fused step: where it lives and whether it is still stored there
-    int new_slot = -1;
-    if (Knew) {
+    if (!Append::on && Knew) {
         const int s = ld_l2(vw.new_slot);
         if (ld_l2(&vw.ctrl->append_n) == 1 && ld_l2(vw.slot_gid + s) == ld_l2(&vw.ctrl->n_total) - 1) new_slot = s;
     }
@@ -989,6 +1117,50 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* 
             if (j < u.n) load_unit(Vh, u.row[j], sv[j]);
         cp_async_commit();
     };
+    // ---- query rows: rotate at q_pos - shift_total, round to bf16, park in shared memory -----------------------
+    // A thread takes two neighbouring pairs (i, i + D/2) of a head.  In a fused step the query is the appended token, its
+    // position is already in the metadata, so the factors do not have to wait for the previous kernel; otherwise the
+    // position comes with the call.  (Every warp loading the query straight into its fragments: 0.2 us later.)
+    constexpr int LPH = HALF / 2;                    // threads per head
+    constexpr int HSTEP = LAY_THREADS / LPH, HN = (8 + HSTEP - 1) / HSTEP;       // heads in one pass; passes
+    const int p2 = threadIdx.x % LPH;
+    const bool prep_new = new_slot >= 0 && threadIdx.x < LPH;
+    float2 f[2];
+    auto factors = [&] {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int pair = 2 * p2 + e;
+            const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
+            const long long c = !Append::on && new_slot >= 0 ? (long long)ld_l2(vw.slot_c + (size_t)axis * b.n_slots + new_slot)
+                                                             : (long long)ld_in(q_pos + (b.rope_mode == 0 ? ci : 3 * ci + axis)) - shift;
+            const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
+            f[e] = svlm_rope_cs_batched(tab, HALF, pair, (int)c);
+            if (__builtin_expect(c <= -65536 || c >= 65536, 0)) f[e] = svlm_rope_cs(tab, HALF, pair, c, b.theta[pair]);
+        }
+    };
+    unsigned ep = 0;                                 // the KV head's epoch (same round trip as the query)
+    unsigned lo[HN], hi[HN], klo = 0, khi = 0, vlo = 0, vhi = 0;
+    auto rows = [&] {                                // all loads first: one round trip
+        if (threadIdx.x == 0) ep = ld_l2(epoch);
+        auto two = [](const uint16_t* p) {           // two neighbouring elements
+            return ANYWHERE ? (unsigned)ld_in(p) | (unsigned)ld_in(p + 1) << 16 : ld_in(reinterpret_cast<const unsigned*>(p));
+        };
+#pragma unroll
+        for (int k = 0; k < HN; ++k) {
+            const int h = threadIdx.x / LPH + k * HSTEP;
+            const uint16_t* row = Q + (q_head0 + (h < G ? h : 0)) * D + 2 * p2;   // n_q = 1
+            lo[k] = two(row);
+            hi[k] = two(row + HALF);
+        }
+        // fused step: the new token's key and value rows come in with the query; the key is rotated with the query's
+        // factors (same token, same position) and both wait in shared memory for the warp whose unit holds the token's slot
+        if (prep_new) {
+            const size_t off = kv_head * D + 2 * p2;
+            klo = two(Knew + off); khi = two(Knew + off + HALF);
+            vlo = two(Vnew + off); vhi = two(Vnew + off + HALF);
+        }
+    };
+    if (Append::on) { rows(); factors(); }           // (the wait is behind us: together with the keys, not after them)
     if (n_rounds > 0) {
         get_units(0, u);
         front(early_loads == 2);
@@ -999,58 +1171,22 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* 
     }
     if (threadIdx.x == 0) STAMP(2);                  // the first round's keys are in registers
 
-    // ---- query rows: rotate at q_pos - shift_total, round to bf16, park in shared memory -----------------------
-    // A thread takes two neighbouring pairs (i, i + D/2) of a head.  In a fused step the query is the appended token, its
-    // position is already in the metadata, so the factors do not have to wait for the previous kernel; otherwise the
-    // position comes with the call.  (Every warp loading the query straight into its fragments: 0.2 us later.)
     unsigned qf[KSTEPS][2];
     const int new_row16 = new_slot & ~15;            // first slot of the unit that holds the new token (fused step)
     {
-        constexpr int LPH = HALF / 2;                // threads per head
-        constexpr int HSTEP = LAY_THREADS / LPH, HN = (8 + HSTEP - 1) / HSTEP;   // heads in one pass; passes
-        const int p2 = threadIdx.x % LPH;
-        if (new_slot < 0 && early_loads) pdl_wait();
-        float2 f[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int pair = 2 * p2 + e;
-            const int axis = b.rope_mode == 0 ? 0 : (pair < b.sec_t ? 0 : (pair < b.sec_th ? 1 : 2));
-            const long long c = new_slot >= 0 ? (long long)ld_l2(vw.slot_c + (size_t)axis * b.n_slots + new_slot)
-                                              : (long long)ld_in(q_pos + (b.rope_mode == 0 ? ci : 3 * ci + axis)) - shift;
-            const float2* tab = reinterpret_cast<const float2*>(b.rope_tab);
-            f[e] = svlm_rope_cs_batched(tab, HALF, pair, (int)c);
-            if (__builtin_expect(c <= -65536 || c >= 65536, 0)) f[e] = svlm_rope_cs(tab, HALF, pair, c, b.theta[pair]);
+        if (!Append::on) {
+            if (new_slot < 0 && early_loads) pdl_wait();
+            factors();
+            if (new_slot >= 0 && early_loads) pdl_wait();
         }
-        if (new_slot >= 0 && early_loads) pdl_wait();
         if (threadIdx.x == 0) STAMP(3);              // the previous kernel has completed
-        unsigned ep = 0;                             // the KV head's epoch (same round trip as the query)
-        if (threadIdx.x == 0) ep = ld_l2(epoch);
+        if (!Append::on) rows();
         auto rotate2 = [&](unsigned& lo, unsigned& hi) {
             const float x0 = __uint_as_float(lo << 16), x1 = __uint_as_float(lo & 0xffff0000u);
             const float y0 = __uint_as_float(hi << 16), y1 = __uint_as_float(hi & 0xffff0000u);
             lo = pack_bf16(x0 * f[0].x - y0 * f[0].y, x1 * f[1].x - y1 * f[1].y);
             hi = pack_bf16(y0 * f[0].x + x0 * f[0].y, y1 * f[1].x + x1 * f[1].y);
         };
-        auto two = [](const uint16_t* p) {           // two neighbouring elements
-            return ANYWHERE ? (unsigned)ld_in(p) | (unsigned)ld_in(p + 1) << 16 : ld_in(reinterpret_cast<const unsigned*>(p));
-        };
-        unsigned lo[HN], hi[HN];
-#pragma unroll
-        for (int k = 0; k < HN; ++k) {               // all loads first: one round trip
-            const int h = threadIdx.x / LPH + k * HSTEP;
-            const uint16_t* row = Q + (q_head0 + (h < G ? h : 0)) * D + 2 * p2;   // n_q = 1
-            lo[k] = two(row);
-            hi[k] = two(row + HALF);
-        }
-        // fused step: the new token's key and value rows come in with the query; the key is rotated with the query's
-        // factors (same token, same position) and both wait in shared memory for the warp whose unit holds the token's slot
-        const bool prep_new = new_slot >= 0 && threadIdx.x < LPH;
-        unsigned klo = 0, khi = 0, vlo = 0, vhi = 0;
-        if (prep_new) {
-            const size_t off = kv_head * D + 2 * p2;
-            klo = two(Knew + off); khi = two(Knew + off + HALF);
-            vlo = two(Vnew + off); vhi = two(Vnew + off + HALF);
-        }
 #pragma unroll
         for (int k = 0; k < HN; ++k) {
             const int h = threadIdx.x / LPH + k * HSTEP;
@@ -1227,6 +1363,9 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* 
     auto stamp7 = [](int) {};
 #endif
     cta_merge_and_record<D, true>(o, m, l, reinterpret_cast<float*>(ring), part, stamp7, &sh.tag);
+    if constexpr (Append::on) {
+        if (warp == DEC_CWARPS - 1) write_token_down(app, ci, sh.one, new_slot, before, gridDim.x * gridDim.y);
+    }
 
     // ---- the first splits of this KV head combine all the splits' records -----------------------------
     __syncthreads();                                  // the merge slabs in `ring` are read
@@ -1305,7 +1444,7 @@ int svlm_decode_splits(int n_pages, int kv_heads, int problems) {
 
 cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
                                int q_heads, void* out, int splits, const void* Knew, const void* Vnew, int early_loads,
-                               bool tagged, cudaStream_t st) {
+                               bool tagged, const SvlmCacheList* list, const unsigned char* types, cudaStream_t st) {
     const int problems = b.n_caches * n_layers;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(splits, b.kv_heads, problems);
@@ -1320,39 +1459,34 @@ cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layer
     uint16_t* Op = (uint16_t*)out;
     const uint16_t* Kn = (const uint16_t*)Knew;
     const uint16_t* Vn = (const uint16_t*)Vnew;
-    cudaError_t e;
-    if (tagged) {
 #ifdef SVLM_DECODE_TRACE
-        int trace_idx = -1;
-        if (g_decode_trace_next >= 0 && g_decode_trace_next < SVLM_TR_LAUNCHES && splits * b.kv_heads <= SVLM_TR_CTAS)
-            trace_idx = g_decode_trace_next++;
+    int trace_idx = -1;
+    if (tagged && g_decode_trace_next >= 0 && g_decode_trace_next < SVLM_TR_LAUNCHES && splits * b.kv_heads <= SVLM_TR_CTAS)
+        trace_idx = g_decode_trace_next++;
 #endif
-        auto go = [&](auto kernel, size_t smem, cudaError_t allowed) {
-            if (allowed != cudaSuccess) return allowed;
-            cfg.dynamicSmemBytes = smem;
-            return cudaLaunchKernelEx(&cfg, kernel, b, layer0, Qp, q_pos, q_heads, Op, splits, Kn, Vn, early_loads TRACE_ARG);
-        };
-        constexpr size_t smem128 = decode_layer_smem<128>(), smem64 = decode_layer_smem<64>();
-        const bool words = (((uintptr_t)Q | (uintptr_t)Knew | (uintptr_t)Vnew) & 3) == 0;
-        if (b.head_dim == 128)
-            e = words ? go(decode_layer_kernel<128, false>, smem128, svlm_allow_smem<decode_layer_kernel<128, false>>(smem128))
-                      : go(decode_layer_kernel<128, true>, smem128, svlm_allow_smem<decode_layer_kernel<128, true>>(smem128));
-        else
-            e = words ? go(decode_layer_kernel<64, false>, smem64, svlm_allow_smem<decode_layer_kernel<64, false>>(smem64))
-                      : go(decode_layer_kernel<64, true>, smem64, svlm_allow_smem<decode_layer_kernel<64, true>>(smem64));
-    } else if (b.head_dim == 128) {
-        e = svlm_allow_smem<decode_stream_kernel<128>>(decode_stream_smem<128>());
-        if (e != cudaSuccess) return e;
-        cfg.dynamicSmemBytes = decode_stream_smem<128>();
-        e = cudaLaunchKernelEx(&cfg, decode_stream_kernel<128>, b, layer0, n_layers, Qp, q_pos, q_heads, Op, splits, Kn, Vn,
-                               early_loads);
-    } else {
-        e = svlm_allow_smem<decode_stream_kernel<64>>(decode_stream_smem<64>());
-        if (e != cudaSuccess) return e;
-        cfg.dynamicSmemBytes = decode_stream_smem<64>();
-        e = cudaLaunchKernelEx(&cfg, decode_stream_kernel<64>, b, layer0, n_layers, Qp, q_pos, q_heads, Op, splits, Kn, Vn,
-                               early_loads);
-    }
+    auto layer = [&](auto kernel, size_t smem, cudaError_t allowed, const auto& app) {
+        if (allowed != cudaSuccess) return allowed;
+        cfg.dynamicSmemBytes = smem;
+        return cudaLaunchKernelEx(&cfg, kernel, b, layer0, Qp, q_pos, q_heads, Op, splits, Kn, Vn, early_loads, app TRACE_ARG);
+    };
+    auto stream = [&](auto kernel, size_t smem, cudaError_t allowed, const auto& app) {
+        if (allowed != cudaSuccess) return allowed;
+        cfg.dynamicSmemBytes = smem;
+        return cudaLaunchKernelEx(&cfg, kernel, b, layer0, n_layers, Qp, q_pos, q_heads, Op, splits, Kn, Vn, early_loads, app);
+    };
+    const bool words = (((uintptr_t)Q | (uintptr_t)Knew | (uintptr_t)Vnew) & 3) == 0;
+    auto go = [&](auto dim, const auto& app) {
+        constexpr int D = decltype(dim)::value;
+        using A = std::decay_t<decltype(app)>;
+        constexpr size_t lay = decode_layer_smem<D>(), str = decode_stream_smem<D>();
+        if (!tagged) return stream(decode_stream_kernel<D, A>, str, svlm_allow_smem<decode_stream_kernel<D, A>>(str), app);
+        return words ? layer(decode_layer_kernel<D, false, A>, lay, svlm_allow_smem<decode_layer_kernel<D, false, A>>(lay), app)
+                     : layer(decode_layer_kernel<D, true, A>, lay, svlm_allow_smem<decode_layer_kernel<D, true, A>>(lay), app);
+    };
+    auto with = [&](const auto& app) {
+        return b.head_dim == 128 ? go(std::integral_constant<int, 128>{}, app) : go(std::integral_constant<int, 64>{}, app);
+    };
+    const cudaError_t e = list ? with(DecAppend{types, *list}) : with(DecNoAppend{});
     svlm_count_launch();
     const cudaError_t last = cudaGetLastError();
     return e != cudaSuccess ? e : last;

@@ -33,6 +33,7 @@ struct SvlmCtrl {            // one per cache, device memory; only meta kernels 
     int status;              // sticky svlm_status
     int append_n;            // tokens staged by the latest metadata append (0 if it was dropped)
     int evict_moved;         // 1 if the latest evict shifted any retained token
+    unsigned append_seen;    // thread blocks of a decode step that appends by itself that are through with the old metadata; 0 between launches
     unsigned wait_limit;     // polls a bounded device-side wait makes before it gives up (set at creation)
 };
 

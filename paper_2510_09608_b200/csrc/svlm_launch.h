@@ -105,12 +105,14 @@ bool svlm_decode_supported(int n_pages);
 // layers attended here, so the kernel may read them before the previous kernel has finished.
 // early_loads == 2: moreover that previous kernel was itself a decode step of this cache (the per-layer kernel then
 // paces its read-ahead, one unit's worth per warp at a time).
+// list non-null: the caches have one layer, and the token's metadata is appended by this launch too (types [n_caches],
+// positions q_pos); null: svlm_launch_append_meta has run before, or nothing is appended.
 // tagged: the per-layer kernel (one layer of one or a few caches; its splits hand their partial results over in tagged
 // words in the views' areas of svlm_decode_tagged_bytes, sized for one cache's splits); otherwise the streaming kernel
 // with its arrival counters in the views' scratch.
 cudaError_t svlm_launch_decode(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
                                int q_heads, void* out, int splits, const void* Knew, const void* Vnew, int early_loads,
-                               bool tagged, cudaStream_t st);
+                               bool tagged, const SvlmCacheList* list, const unsigned char* types, cudaStream_t st);
 // Splits of the per-layer kernel for one layer of n_caches caches with `pages` pages or fewer, 0 where the streaming kernel
 // is the better one (either gives the same result).
 int svlm_decode_layer_splits(int n_pages, int pages, int layers, int kv_heads, int n_caches, int head_dim);

@@ -5,6 +5,7 @@
 
 #include <algorithm>
 
+#include "svlm_append_one.cuh"
 #include "svlm_dev.h"
 #include "svlm_launch.h"
 #include "svlm_ptx.cuh"
@@ -171,117 +172,23 @@ __device__ void rebuild_tiles(const SvlmCacheDev& cd, int sink_fill, const long 
 constexpr int ONE_THREADS = 128;
 constexpr int ONE_ENTRIES = 4;      // list entries per thread
 __device__ __forceinline__ void append_one_body(const SvlmCacheDev& cd, const unsigned char* types, const int* pos) {
-    __shared__ int s_state;       // 0: go on; 1: append dropped (capacity)
-    SvlmCtrl* ctrl = cd.ctrl;
     const int tid = threadIdx.x;
     SvlmTile old[ONE_ENTRIES];    // entries tid, tid + 128, ... of the present list (garbage beyond its end; never used then)
 #pragma unroll
     for (int k = 0; k < ONE_ENTRIES; ++k)
         if (tid + k * ONE_THREADS < cd.n_pages) old[k] = cd.tiles[tid + k * ONE_THREADS];
-    const int n_tiles0 = ctrl->n_tiles;
-    const long long n_total0 = ctrl->n_total;
-    const int ty = types[0] ? 1 : 0;
-    const long long ord = ctrl->n_type[ty];
-    const long long cursor0 = ctrl->cursor;
-    const long long shift = cd.contiguous ? ctrl->shift_total : 0;
-    const long long ring_n0[2] = {ctrl->ring_n[0], ctrl->ring_n[1]};
-    const long long ring_lo0[2] = {ctrl->ring_lo[0], ctrl->ring_lo[1]};
-    const int sink_fill0 = ctrl->sink_fill;
-    const int n_stored0 = ctrl->n_stored;
-    const int free_top0 = ctrl->free_top;
-    long long p[3];
-    if (cd.rope_mode == 0) { p[0] = p[1] = p[2] = pos[0]; }
-    else { p[0] = pos[0]; p[1] = pos[1]; p[2] = pos[2]; }
-
-    const long long gid = n_total0;
-    const bool is_sink = cd.sink_any ? (gid < cd.n_sink) : (ty == 0 && ord < cd.n_sink);
-    const long long u = ring_n0[ty];                       // the token's ring ordinal if it is not a sink
-    const bool new_page = !is_sink && (u % SVLM_PAGE) == 0;
-    // the list as it is: sink pages, text ring pages, vision ring pages
-    const int ns0 = (sink_fill0 + SVLM_PAGE - 1) / SVLM_PAGE;
-    int cnt0[2];
-    for (int t = 0; t < 2; ++t)
-        cnt0[t] = ring_n0[t] > ring_lo0[t] ? (int)((ring_n0[t] - 1) / SVLM_PAGE - ring_lo0[t] / SVLM_PAGE + 1) : 0;
-    // the entry the token lands in: position in the OLD list if it exists there, else where it is inserted
-    bool adds;              // a new entry appears
-    int at;                 // old index of the entry that grows, or new index of the entry that appears
-    if (is_sink) {
-        adds = (sink_fill0 % SVLM_PAGE) == 0;
-        at = adds ? ns0 : ns0 - 1;
-    } else {
-        const int cnt1 = (int)(u / SVLM_PAGE - ring_lo0[ty] / SVLM_PAGE + 1);
-        adds = cnt1 != cnt0[ty];
-        at = ns0 + (ty ? cnt0[0] : 0) + (adds ? cnt0[ty] : cnt0[ty] - 1);
-    }
-    if (tid == 0) {
-        const bool ok = (n_stored0 + 1 <= cd.capacity) && (!new_page || free_top0 >= 1) &&
-                        (!is_sink || sink_fill0 + 1 <= cd.n_sink_pages * SVLM_PAGE);
-        s_state = ok ? 0 : 1;
-        if (!ok) {
-            ctrl->append_n = 0;
-            if (ctrl->status == 0) ctrl->status = -2;   // SVLM_ERR_CAPACITY
-        }
-    }
-    __syncthreads();                                    // also: every old entry is in registers
-    if (s_state) return;
-
-    // entries behind an inserted one move up by one; the one that grows is rewritten by its owner
+    const SvlmCtrl ctrl = *cd.ctrl;
+    const int ty = types[0] ? 1 : 0, pw = cd.rope_mode == 0 ? 0 : 1;
+    const int p[3] = {pos[0], pos[pw], pos[2 * pw]};
+    const SvlmOneToken t = svlm_one_token(SvlmOneRule(cd), ctrl, ty, p);
+    __syncthreads();              // every old entry is in registers
+    if (t.ok && t.adds)           // entries behind the new one move up by one
 #pragma unroll
-    for (int k = 0; k < ONE_ENTRIES; ++k) {
-        const int i = tid + k * ONE_THREADS;
-        if (i >= n_tiles0) continue;
-        if (adds && i >= at) cd.tiles[i + 1] = old[k];
-        if (!adds && i == at) {
-            old[k].hi += 1;
-            old[k].max_gid = gid;
-            cd.tiles[i] = old[k];
+        for (int k = 0; k < ONE_ENTRIES; ++k) {
+            const int i = tid + k * ONE_THREADS;
+            if (i < t.n_tiles0 && i >= t.at) cd.tiles[i + 1] = old[k];
         }
-    }
-    if (tid == 0) {
-        int slot, page;
-        if (is_sink) {
-            slot = (int)(cd.sink_any ? gid : ord);
-            page = slot / SVLM_PAGE;
-        } else {
-            const int pt = (int)(u / SVLM_PAGE) & (cd.pt_size - 1);
-            if (new_page) {
-                page = cd.free_stack[free_top0 - 1];
-                cd.page_table[ty][pt] = page;
-                ctrl->free_top = free_top0 - 1;
-            } else {
-                page = cd.page_table[ty][pt];
-            }
-            slot = page * SVLM_PAGE + (int)(u % SVLM_PAGE);
-        }
-        if (adds) {
-            SvlmTile tl;
-            tl.page = page;
-            tl.lo = slot % SVLM_PAGE;
-            tl.hi = tl.lo + 1;
-            tl.pad = 0;
-            tl.min_gid = tl.max_gid = gid;
-            cd.tiles[at] = tl;
-            ctrl->n_tiles = n_tiles0 + 1;
-        }
-        const long long top = max(p[0], max(p[1], p[2])) + 1;
-        cd.slot_gid[slot] = gid;
-        cd.slot_type[slot] = (unsigned char)ty;
-        cd.slot_a[slot] = (int)max(0ll, top - cursor0);
-        cd.slot_delta[slot] = 0;
-        cd.new_slot[0] = slot;
-        for (int k = 0; k < 3; ++k) cd.slot_c[k * cd.n_slots + slot] = (int)(p[k] - shift);
-        ctrl->n_total = n_total0 + 1;
-        ctrl->n_type[ty] = ord + 1;
-        ctrl->cursor = max(cursor0, top);
-        if (is_sink) {
-            ctrl->sink_cnt[ty] += 1;
-            ctrl->sink_fill = sink_fill0 + 1;
-        } else {
-            ctrl->ring_n[ty] = u + 1;
-        }
-        ctrl->n_stored = n_stored0 + 1;
-        ctrl->append_n = 1;
-    }
+    if (tid == 0) svlm_one_commit(cd, t, t.ok ? svlm_one_slot(cd, t) : 0);
 }
 
 // ---------------------------------------------------------------------------------------------

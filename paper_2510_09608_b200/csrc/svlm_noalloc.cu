@@ -92,7 +92,7 @@ extern "C" int svlm_attend_decode_noalloc(svlm_cache* c, int layer, const void* 
         b.rope_tab = d.rope_tab;
         b.q_varlen = 0;
         v.ws = scratch;
-        if (svlm_launch_decode(b, layer, 1, Q, q_pos, q_heads, out, splits, nullptr, nullptr, 0, false, c->stream) != cudaSuccess)
+        if (svlm_launch_decode(b, layer, 1, Q, q_pos, q_heads, out, splits, nullptr, nullptr, 0, false, nullptr, nullptr, c->stream) != cudaSuccess)
             rc = SVLM_ERR_CUDA;
     }
     if (prev != c->device) cudaSetDevice(prev);

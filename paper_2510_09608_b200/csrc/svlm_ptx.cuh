@@ -103,6 +103,11 @@ SVLM_LOAD2(ld_l2, float2, "ld.global.cg.v2.f32", "=f")
 SVLM_LOAD4(ld_l2, float4, "ld.global.cg.v4.f32", "=f")
 SVLM_LOAD4(ld_l2, int4, "ld.global.cg.v4.s32", "=r")
 SVLM_LOAD4(ld_l2, uint4, "ld.global.cg.v4.u32", "=r")
+__device__ __forceinline__ unsigned char ld_in(const unsigned char* p) {
+    unsigned v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return (unsigned char)v;
+}
 #undef SVLM_LOAD
 #undef SVLM_LOAD2
 #undef SVLM_LOAD4

@@ -278,8 +278,10 @@ SvlmPrefillLoad expected_load(const svlm_cache* c) {
 }
 
 // call_layers: of a call that is launched layer by layer, all its layers (it takes the kernel that one launch of them would).
+// list, types: a decode step whose launch appends the token by itself (the host's counts have it already).
 int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void* Q, const int32_t* q_pos, int n_q,
-                  int q_heads, void* out, const void* Knew = nullptr, const void* Vnew = nullptr, int call_layers = 0) {
+                  int q_heads, void* out, const void* Knew = nullptr, const void* Vnew = nullptr, int call_layers = 0,
+                  const SvlmCacheList* list = nullptr, const uint8_t* types = nullptr) {
     svlm_cache* c0 = caches[0];
     if (!Q || !q_pos || !out || n_q < 1 || q_heads < 1) return SVLM_ERR_ARG;
     if (q_heads % c0->dev.kv_heads) return SVLM_ERR_ARG;
@@ -287,6 +289,7 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     const int group = q_heads / c0->dev.kv_heads;
     const bool split_kv = n_q == 1 && group <= 8 && svlm_decode_supported(c0->dev.n_pages);
     const bool chunk = n_q >= 2 && svlm_prefill_supported(c0->dev.n_pages, group);
+    if (list && !split_kv) return SVLM_ERR_ARG;      // (only the decode kernels append by themselves)
     if (split_kv && !decode_aligned(Q, Knew, Vnew, out, q_pos)) return SVLM_ERR_ARG;
     if (chunk && !(aligned(16, Q, out) && aligned(4, q_pos))) return SVLM_ERR_ARG;      // (the general kernel reads and writes element by element)
     SvlmAttendBatch b;
@@ -333,7 +336,7 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
         int splits = n_layers == 1 ? svlm_decode_layer_splits(c0->dev.n_pages, pages, c0->dev.layers, c0->dev.kv_heads, n_caches, c0->dev.head_dim) : 0;
         const bool tagged = splits > 0;
         if (!tagged) splits = svlm_decode_splits(c0->dev.n_pages, c0->dev.kv_heads, n_caches * n_layers);
-        SVLM_CUDA(svlm_launch_decode(b, layer0, n_layers, Q, q_pos, q_heads, out, splits, Knew, Vnew, early, tagged, c0->stream));
+        SVLM_CUDA(svlm_launch_decode(b, layer0, n_layers, Q, q_pos, q_heads, out, splits, Knew, Vnew, early, tagged, list, types, c0->stream));
         return SVLM_OK;
     }
     if (Knew) return SVLM_ERR_ARG;   // the fused step exists for the split-KV kernel only
@@ -347,6 +350,32 @@ int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void
     svlm_launch_attend_simple(b, layer0, n_layers, Q, q_pos, n_q, q_heads, out, c0->stream);
     SVLM_CUDA(cudaGetLastError());
     return SVLM_OK;
+}
+
+// A decode step of one or several caches, whose arguments have been checked.  For caches of one layer its launch appends the
+// token itself (see svlm_decode.cu); the host's counts then go back if it fails.
+int decode_step(const SvlmCacheList& list, svlm_cache* const* caches, int n_caches, int layer, const void* K, const void* V, const uint8_t* token_type,
+                const int32_t* pos, const void* Q, int q_heads, void* out) {
+    svlm_cache* c0 = caches[0];
+    if (layer > 0) return attend_common(caches, n_caches, layer, Q, pos, 1, q_heads, out, K, V);
+    struct Counts { long long appended, stored; int pending; bool settled; } before[SVLM_MAX_BATCH];
+    const bool itself = c0->dev.layers == 1;
+    if (!itself)
+        SVLM_CUDA(n_caches == 1 ? svlm_launch_append_meta(c0->dev, token_type, pos, 1, c0->stream)
+                                : svlm_launch_append_meta_batch(list, c0->dev, token_type, pos, 1, c0->stream));
+    for (int i = 0; i < n_caches; ++i) {
+        svlm_cache* c = caches[i];
+        before[i] = {c->appended, c->stored_est, c->pending_n, c->meta_settled};
+        note_append(c, 1);
+    }
+    if (!itself) return attend_common(caches, n_caches, layer, Q, pos, 1, q_heads, out, K, V);
+    const int rc = attend_common(caches, n_caches, layer, Q, pos, 1, q_heads, out, K, V, 0, &list, token_type);
+    if (rc != SVLM_OK)
+        for (int i = 0; i < n_caches; ++i) {
+            svlm_cache* c = caches[i];
+            c->appended = before[i].appended; c->stored_est = before[i].stored; c->pending_n = before[i].pending; c->meta_settled = before[i].settled;
+        }
+    return rc;
 }
 
 }  // namespace
@@ -614,13 +643,14 @@ int svlm_decode_step(svlm_cache* c, int layer, const void* K, const void* V, con
         if (!token_type) return SVLM_ERR_ARG;
         c->configured_locked = true;
         c->last_decode_layer = -1;
-        SVLM_CUDA(svlm_launch_append_meta(c->dev, token_type, pos, 1, c->stream));
-        note_append(c, 1);
     } else if (c->pending_n != 1) {
         return SVLM_ERR_ORDER;
     }
     svlm_cache* one[1] = {c};
-    return attend_common(one, 1, layer, Q, pos, 1, q_heads, out, K, V);
+    SvlmCacheList list;
+    list.n = 1;
+    list.cd[0] = c->dev_copy;
+    return decode_step(list, one, 1, layer, K, V, token_type, pos, Q, q_heads, out);
 }
 
 int svlm_decode_step_batched(svlm_cache* const* caches, int n_caches, int layer, const void* K, const void* V,
@@ -640,13 +670,11 @@ int svlm_decode_step_batched(svlm_cache* const* caches, int n_caches, int layer,
             c->configured_locked = true;
             c->last_decode_layer = -1;
         }
-        SVLM_CUDA(svlm_launch_append_meta_batch(list, c0->dev, token_type, pos, 1, c0->stream));
-        for (int i = 0; i < n_caches; ++i) note_append(caches[i], 1);
     } else {
         for (int i = 0; i < n_caches; ++i)
             if (caches[i]->pending_n != 1) return SVLM_ERR_ORDER;
     }
-    return attend_common(caches, n_caches, layer, Q, pos, 1, q_heads, out, K, V);
+    return decode_step(list, caches, n_caches, layer, K, V, token_type, pos, Q, q_heads, out);
 }
 
 int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int layer, const void* Q, const int32_t* q_pos,

@@ -309,6 +309,69 @@ def test_decode_inputs_at_any_element(d, hq, hk, kept, streams):
     assert torch.equal(run(1), want) and want.any()
 
 
+# --- decode steps whose launch appends the token itself (one cache or several of one layer; beside them all layers at once): tokens that
+# --- open pages of either ring and of the sinks, vision among text, evictions in between, both kernels, and a cache that is full
+@pytest.mark.parametrize("d,hq,hk,layers,streams,rope_1d,sink_any,fill", [
+    (64, 4, 1, 1, 1, True, False, 60), (128, 28, 4, 1, 1, False, False, 500), (128, 8, 4, 3, 1, False, True, 100), (64, 16, 8, 1, 4, True, True, 250),
+    (128, 14, 2, 1, 2, False, False, 130), (128, 28, 4, 1, 5, False, False, 300)])
+def test_decode_steps_that_append_by_themselves(d, hq, hk, layers, streams, rope_1d, sink_any, fill):
+    from harness import SideBySide, assert_close, bits_to_dev, dev_to_f64
+    from paper_2510_09608_b200 import binding
+    half = d // 2
+    wl = _wl(2, layers=layers, q_heads=hq, kv_heads=hk, head_dim=d, rope_mode=0 if rope_1d else 1,
+             sections=(half, 0, 0) if rope_1d else (half // 4, 3 * half // 8, 3 * half // 8), n_sink=130, vision_window=fill, text_window=140)
+    rng = np.random.default_rng(fill)
+    sides = [SideBySide(wl, stream=i, capacity=130 + fill + 140 + 160, sink_any=sink_any) for i in range(streams)]
+    at = [0] * streams                                           # next ordinal, and its native position
+    shaped = lambda p: np.asarray(p, np.int32) if rope_1d else np.repeat(np.asarray(p, np.int32)[:, None], 3, axis=1)     # noqa: E731
+    for i, s in enumerate(sides):
+        n = fill + 17 * i
+        s._append(np.arange(n), rng.integers(0, 2, n).astype(np.uint8), shaped(np.arange(n)))
+        at[i] = n
+    before = binding.launch_count()
+    steps = 290
+    for step in range(steps):
+        types = rng.integers(0, 2, streams).astype(np.uint8)
+        pos = np.stack([shaped([at[i]]) for i in range(streams)])          # [streams, 1(, 3)]
+        ty, ps = torch.from_numpy(types).cuda(), torch.from_numpy(pos).cuda()
+        gids = [np.arange(at[i], at[i] + 1) for i in range(streams)]
+        rows = lambda what: np.stack([np.stack([getattr(s.stream, what)(l, g) for s, g in zip(sides, gids)]) for l in range(layers)])  # noqa: E731  [layers, streams, 1, heads, d]
+        K, V, Q = (bits_to_dev(rows(w)) for w in "kvq")
+        if streams > 1:
+            out = binding.decode_step_batched([s.cache for s in sides], 0, K[0, :, 0].contiguous(), V[0, :, 0].contiguous(), ty, ps[:, 0].contiguous(), Q[0, :, 0].contiguous())[None, :, None]
+        elif layers > 1:
+            out = sides[0].cache.decode_step(-1, K[:, 0].contiguous(), V[:, 0].contiguous(), ty, ps[0], Q[:, 0].contiguous())[:, None]
+        else:
+            out = sides[0].cache.decode_step(0, K[0, 0], V[0, 0], ty, ps[0], Q[0, 0])[None, None]
+        for i, s in enumerate(sides):
+            s.ref.append(None, None, types[i:i + 1], pos[i])
+            at[i] += 1
+        if step % 41 == 0 or step == steps - 1:
+            for i, s in enumerate(sides):
+                s.check_metadata()
+                for l in {0, layers - 1}:
+                    s._give_values_to_ref(l)
+                    assert_close(s._stats(dev_to_f64(out)[l, i], s.ref.attend(l, s.stream.q(l, gids[i]), pos[i])))
+        if step % 97 == 96:
+            for s in sides:
+                s.evict()
+                s.check_metadata()
+    if streams == 1 and layers == 1:
+        assert binding.launch_count() - before <= steps + 2 * (steps // 97)     # one launch a step
+    for s in sides:
+        for l in {0, layers - 1}:
+            s.check_kv(l)
+    s = sides[0]                                                 # until it is full: the token is dropped, the status says so, nothing else moves
+    kept = len(s.cache.query()["gids"])
+    K, V, Q = (bits_to_dev(np.stack([getattr(s.stream, w)(l, np.arange(1)) for l in range(layers)])) for w in "kvq")
+    ty = torch.zeros(1, dtype=torch.uint8, device="cuda")
+    for _ in range(130 + fill + 140 + 160 - kept + 3):
+        s.cache.decode_step(-1, K, V, ty, torch.from_numpy(shaped([at[0]])).cuda(), Q)
+        at[0] += 1
+    assert s.cache.status() == binding.ERR_CAPACITY
+    assert len(s.cache.query()["gids"]) == 130 + fill + 140 + 160
+
+
 def test_decode_alternating_single_and_batched():
     """The same caches decode by themselves, in pairs and all together in turn: the per-layer kernel writes its tagged records
     with 37 splits, then 18, the streaming kernel its own scratch with 9, and none may take another's leftovers for its own."""
