@@ -47,6 +47,7 @@ __device__ int block_excl_sum(int v, int& carry, int* warp_buf) {
     return res;
 }
 
+template <int WARPS>
 __device__ long long block_excl_sum64(long long v, long long& carry, long long* warp_buf) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     long long inc = v;
@@ -58,17 +59,17 @@ __device__ long long block_excl_sum64(long long v, long long& carry, long long* 
     if (lane == 31) warp_buf[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        long long w = warp_buf[lane];
+        long long w = lane < WARPS ? warp_buf[lane] : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             long long t = __shfl_up_sync(0xffffffffu, w, o);
             if (lane >= o) w += t;
         }
-        warp_buf[lane] = w;
+        if (lane < WARPS) warp_buf[lane] = w;
     }
     __syncthreads();
     const long long before = (warp ? warp_buf[warp - 1] : 0);
-    const long long total = warp_buf[META_WARPS - 1];
+    const long long total = warp_buf[WARPS - 1];
     const long long res = carry + before + inc - v;
     __syncthreads();
     carry += total;
@@ -469,6 +470,7 @@ __device__ __forceinline__ int count_below(const long long* g, int n, long long 
     return lo;
 }
 
+constexpr int ROTATE_THREADS = 256;
 constexpr int EV_SMEM = 2048;   // evicted tokens of one call whose lists also fit in shared memory
 constexpr int KEPT_BATCH = 2;   // retained tokens a thread handles per round (loads of a round are issued together)
 constexpr int EV_CLUSTER = 8;   // most CTAs (one thread-block cluster) that share the retained tokens of one cache
@@ -507,15 +509,17 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // 7 now (append and eviction of a chunk in a row: 22.6 -> 17.4 us).
 //
 // ROTATE: a single CTA serves the cache (a retained token per thread at most) and re-rotates the moved keys as well, where
-// that is so little that a launch of its own costs more (svlm_evict_in_one).
-template <bool ROTATE>
+// that is so little that a launch of its own costs more (svlm_evict_in_one); of no more threads than that takes, since the
+// barriers cost by the warp (ROTATE_THREADS).
+template <bool ROTATE, int THREADS>
 __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
+    constexpr int PER_CTA = KEPT_BATCH * THREADS;           // retained tokens of a CTA and round
     const int crank = (int)cluster_ctarank(), n_ctas = (int)cluster_nctarank();
-    __shared__ long long wbuf64[2][META_WARPS];
+    __shared__ long long wbuf64[2][(THREADS / 32)];
     __shared__ long long s_gid[EV_SMEM];       // ordinals of the evicted tokens: text ring, then vision ring
     __shared__ long long s_pref[EV_SMEM + 2];  // exclusive prefix sums of their advances (n+1 entries per ring)
     __shared__ int s_moved;
-    __shared__ int2 moved_slots[ROTATE ? META_THREADS : 1]; // slot and shift of the retained tokens (slot -1: none, or not moved)
+    __shared__ int2 moved_slots[ROTATE ? THREADS : 1]; // slot and shift of the retained tokens (slot -1: none, or not moved)
     SvlmCtrl* ctrl = cd.ctrl;
     const int tid = threadIdx.x;
     if (tid == 0) s_moved = 0;
@@ -544,7 +548,7 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
     auto kept_slots = [&](long long base) {
 #pragma unroll
         for (int u = 0; u < KEPT_BATCH; ++u) {
-            const long long i = base + (long long)u * META_THREADS + tid;
+            const long long i = base + (long long)u * THREADS + tid;
             if (i >= n_kept) k_slot[u] = -1;
             else if (i < sink_fill) k_slot[u] = (int)i;
             else if (i < sink_fill + kept_ring[0]) k_slot[u] = ring_slot(cd, 0, lo1[0] + (i - sink_fill));
@@ -573,7 +577,7 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
             e_g[t] = e_slot[t] >= 0 ? cd.slot_gid[e_slot[t]] : 0;
         }
     };
-    const long long base0 = (long long)crank * EV_PER_CTA;
+    const long long base0 = (long long)crank * PER_CTA;
     const bool lists = crank == n_ctas - 1;       // this CTA writes the page list
     auto page_of = [&](int t, long long k) { return cd.page_table[t][(int)k & (cd.pt_size - 1)]; };
     evicted_slots(0);
@@ -583,13 +587,13 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
 
     // evicted tokens in ordinal (= stream) order, with exclusive prefix sums of a
     long long freed[2] = {0, 0};
-    for (int base = 0; base < max(n_ev[0], n_ev[1]); base += META_THREADS) {
+    for (int base = 0; base < max(n_ev[0], n_ev[1]); base += THREADS) {
         const int i = base + tid;
         if (base) { evicted_slots(base); evicted_data(); }
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             if (base >= n_ev[t]) continue;            // uniform over the block
-            const long long ex = block_excl_sum64(e_a[t], freed[t], wbuf64[t]);
+            const long long ex = block_excl_sum64<THREADS / 32>(e_a[t], freed[t], wbuf64[t]);
             if (e_slot[t] >= 0) {
                 if (in_smem) {
                     s_gid[(t ? n_ev[0] : 0) + i] = e_g[t];
@@ -612,7 +616,7 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
 
     int moved = 0;
     if (ROTATE) moved_slots[tid] = make_int2(-1, 0);
-    for (long long base = base0; base < n_kept; base += (long long)n_ctas * EV_PER_CTA) {
+    for (long long base = base0; base < n_kept; base += (long long)n_ctas * PER_CTA) {
         if (base != base0) { kept_slots(base); kept_data(); }
         int E[KEPT_BATCH];
 #pragma unroll
@@ -638,7 +642,7 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
     if (moved) s_moved = 1;
     const TileList tl(sink_fill, lo1, ring_n);
     if (lists)
-        for (int i = tid; i < tl.total; i += META_THREADS) {      // (the ordinals of retained tokens do not change here)
+        for (int i = tid; i < tl.total; i += THREADS) {      // (the ordinals of retained tokens do not change here)
             SvlmTile tile = tl.entry(i, page_of);
             tile.min_gid = cd.slot_gid[tile.page * SVLM_PAGE + tile.lo];
             tile.max_gid = cd.slot_gid[tile.page * SVLM_PAGE + tile.hi - 1];
@@ -651,15 +655,15 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
         cnt[t] = max(0ll, min(lo1[t] / SVLM_PAGE, ceil_page(ring_n[t])) - first[t]);
     }
     if (crank == 0)
-        for (long long i = tid; i < cnt[0] + cnt[1]; i += META_THREADS) {
+        for (long long i = tid; i < cnt[0] + cnt[1]; i += THREADS) {
             const int t = i < cnt[0] ? 0 : 1;
             cd.free_stack[free_top0 + i] = page_of(t, first[t] + (t ? i - cnt[0] : i));
         }
     __syncthreads();
     cluster_wait();      // every CTA has read them: now the evicted slots can be marked empty
     if (crank == 0) {
-        for (int base = 0; base < max(n_ev[0], n_ev[1]); base += META_THREADS) {
-            if (max(n_ev[0], n_ev[1]) > META_THREADS) evicted_slots(base);      // (else this thread's are still at hand)
+        for (int base = 0; base < max(n_ev[0], n_ev[1]); base += THREADS) {
+            if (max(n_ev[0], n_ev[1]) > THREADS) evicted_slots(base);      // (else this thread's are still at hand)
 #pragma unroll
             for (int t = 0; t < 2; ++t)
                 if (e_slot[t] >= 0) {
@@ -685,7 +689,7 @@ __device__ __forceinline__ void evict_meta_body(const SvlmCacheDev& cd) {
     if (ROTATE && s_moved) {                       // (moved_slots was complete at the barrier above)
         const int half = cd.head_dim / 2, gshift = cd.head_dim == 128 ? 3 : 2, rows = cd.layers * cd.kv_heads;
         const size_t stride = (size_t)cd.n_slots * cd.head_dim;
-        for (int i = tid; i < (int)n_kept << gshift; i += META_THREADS) {
+        for (int i = tid; i < (int)n_kept << gshift; i += THREADS) {
             const int2 mv = moved_slots[i >> gshift];
             if (mv.x < 0) continue;
             const int g = i & ((1 << gshift) - 1);
@@ -782,19 +786,19 @@ __global__ void __launch_bounds__(META_THREADS) append_meta_write_kernel(SvlmCac
 }
 
 template <bool ROTATE>
-__global__ void __launch_bounds__(META_THREADS) evict_meta_kernel(SvlmCacheDev cd) {
+__global__ void __launch_bounds__(ROTATE ? ROTATE_THREADS : META_THREADS) evict_meta_kernel(SvlmCacheDev cd) {
     svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();
-    evict_meta_body<ROTATE>(cd);
+    evict_meta_body<ROTATE, ROTATE ? ROTATE_THREADS : META_THREADS>(cd);
 }
 
 template <bool ROTATE>
-__global__ void __launch_bounds__(META_THREADS) evict_meta_batch_kernel(SvlmCacheList list) {
+__global__ void __launch_bounds__(ROTATE ? ROTATE_THREADS : META_THREADS) evict_meta_batch_kernel(SvlmCacheList list) {
     __shared__ SvlmCacheDev s_cd;
     svlm_load_desc(&s_cd, list.cd[blockIdx.x / cluster_nctarank()]);
     svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();
-    evict_meta_body<ROTATE>(s_cd);
+    evict_meta_body<ROTATE, ROTATE ? ROTATE_THREADS : META_THREADS>(s_cd);
 }
 
 int append_form_of(int n, int n_pages) {
@@ -816,11 +820,12 @@ cudaError_t svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmC
 
 // One launch for a whole append or eviction of a small cache.  The lines: what one block moves by itself against a second launch
 // on all SMs.  Append and eviction of a chunk in a row, replayed from a graph, us: 2.4 K elements of new keys written in the
-// same launch 14.6, in a second one 15.9, 32 K 25.2 and 17.4; 12.5 K elements of kept keys re-rotated in the same launch 15.2,
-// in a second one 15.9, 35 K 17.2 and 17.4, 155 K 32.9 and 17.7.  (By plain calls a launch less saves the host 2 us more.)
-constexpr long long APPEND_WRITE_ELEMENTS = 8192;      // of the appended keys
+// same launch 14.3, in a second one 15.3, 4 K 15.5 and 16.3, 8 K 17.4 and 16.6, 32 K 25.2 and 17.4; 8 K elements of kept keys
+// re-rotated in the same launch 15.2, in a second one 16.6, 17 K 17.5 and 17.3 (one head) or 14.9 and 15.8 (two of 128), 155 K
+// 32.9 and 17.7.  (By plain calls a launch less saves the host 2 us more.)
+constexpr long long APPEND_WRITE_ELEMENTS = 4096;      // of the appended keys
 constexpr long long EVICT_ROTATE_ELEMENTS = 16384;     // of the keys that the windows keep
-static_assert(EVICT_ROTATE_ELEMENTS / 64 <= META_THREADS, "a thread per retained token (heads have 64 dims at least)");
+static_assert(EVICT_ROTATE_ELEMENTS / 64 <= ROTATE_THREADS, "a thread per retained token (heads have 64 dims at least)");
 bool svlm_append_in_one(const SvlmCacheDev& cd, int layer, int n) {
     return n <= META_THREADS && (long long)n * (layer < 0 ? cd.layers : 1) * cd.kv_heads * cd.head_dim <= APPEND_WRITE_ELEMENTS;
 }
@@ -839,7 +844,7 @@ cudaError_t svlm_launch_append_in_one(const SvlmCacheDev& cd, int layer, const v
 cudaError_t svlm_launch_evict_meta_batch(const SvlmCacheList& list, const SvlmCacheDev& geom, bool rotate, cudaStream_t st) {
     int c = rotate ? 1 : evict_cluster(geom.n_slots);            // (the caches share the number of pages, not the exact capacity)
     while (c > 1 && c * list.n > 96) c /= 2;        // 16 clusters of 8 do not find room at once (a CTA fills an SM)
-    return svlm_launch_chained(rotate ? evict_meta_batch_kernel<true> : evict_meta_batch_kernel<false>, dim3(c * list.n), dim3(META_THREADS), 0, c, st, list);
+    return svlm_launch_chained(rotate ? evict_meta_batch_kernel<true> : evict_meta_batch_kernel<false>, dim3(c * list.n), dim3(rotate ? ROTATE_THREADS : META_THREADS), 0, c, st, list);
 }
 
 cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n,
@@ -851,5 +856,5 @@ cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char*
 
 cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, bool rotate, cudaStream_t st) {
     const int c = rotate ? 1 : evict_cluster(cd.capacity);
-    return svlm_launch_chained(rotate ? evict_meta_kernel<true> : evict_meta_kernel<false>, dim3(c), dim3(META_THREADS), 0, c, st, cd);
+    return svlm_launch_chained(rotate ? evict_meta_kernel<true> : evict_meta_kernel<false>, dim3(c), dim3(rotate ? ROTATE_THREADS : META_THREADS), 0, c, st, cd);
 }

@@ -134,8 +134,8 @@ def test_append_sizes_and_large_evictions(sizes, sink_any):
 # --- block writes and one more, as many kept tokens as it re-rotates and one more, all layers at once, positions beyond 2^16
 @pytest.mark.parametrize("over", [0, 1])
 @pytest.mark.parametrize("d,hk,layers,sizes,capacity,base,contiguous", [
-    (64, 1, 1, (37, 128, 129, 1, 31), 256, 0, True), (128, 2, 1, (32, 33, 1, 3), 200, 0, True), (64, 1, 3, (42, 43, 33, 2), 100, 0, True),
-    (64, 2, 2, (1, 2, 32, 33), 100, 70000, False), (128, 1, 2, (7, 31, 32, 33), 70, 70000, True), (64, 1, 1, (40, 200), 2600, 0, True)])
+    (64, 1, 1, (37, 64, 65, 1, 31), 256, 0, True), (128, 2, 1, (16, 17, 1, 3), 200, 0, True), (64, 1, 3, (21, 22, 33, 2), 100, 0, True),
+    (64, 2, 2, (1, 2, 16, 17), 100, 70000, False), (128, 1, 2, (7, 15, 16, 17), 70, 70000, True), (64, 1, 1, (40, 300), 2600, 0, True)])
 def test_small_caches_in_one_launch(d, hk, layers, sizes, capacity, base, contiguous, over):
     from harness import SideBySide
     keep = 16384 // (d * hk * layers) + over                  # tokens the windows keep: one block re-rotates them, or a launch of its own
