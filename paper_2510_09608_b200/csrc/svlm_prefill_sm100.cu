@@ -9,8 +9,8 @@
 // made from the numbers of rows and an estimate of the pages (svlm_prefill_plan.h): first whole units, round by round over
 // the grid (neighbouring CTAs then stream the same pages at the same time), then its share of the last one to two rounds'
 // units, dealt out evenly in pages, so that no SM idles in a last wave (120 of 148 SMs had work for one stream's chunk before, 960 CTAs were 6.5
-// waves for eight streams).  A unit that is cut between CTAs is merged by the last of them to finish it: the others
-// leave their un-normalised (O, m, l) in the cache's scratch, arrival counters say who is last, nobody waits.
+// waves for eight streams).  A unit that is cut between CTAs is merged by those that end in it, each a share of its columns,
+// through un-normalised pieces (O, m, l) in the cache's scratch; nothing depends on a wait (meet_pieces).
 //
 // Roles (384 threads, registers moved from warpgroup 2 to the softmax with setmaxnreg):
 //   warps 0-3, 4-7   softmax of tile A, B, one thread per row; also that tile's query rotation and output
