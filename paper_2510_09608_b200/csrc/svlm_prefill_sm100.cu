@@ -87,7 +87,7 @@ __device__ __forceinline__ void rescale_o(unsigned tO, int D, float corr) {
     for (int q = 0; q < D; q += 8) {
         float o[8];
         tmem_ld8(tO + q, o);
-        tmem_wait_ld();
+        tmem_wait_ld<8>(o);
 #pragma unroll
         for (int k = 0; k < 8; ++k) o[k] *= corr;
         tmem_st8(tO + q, o);
@@ -109,7 +109,7 @@ __device__ __forceinline__ void softmax_page(int g, unsigned tS, unsigned tO, in
     float s[128];
     tmem_ld32(tS, s);
     tmem_ld32(tS + 32, s + 32);
-    tmem_wait_ld();
+    tmem_wait_ld<64>(s);
     tmem_ld32(tS + 64, s + 64);
     tmem_ld32(tS + 96, s + 96);
     float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -121,7 +121,7 @@ __device__ __forceinline__ void softmax_page(int g, unsigned tS, unsigned tO, in
         }
 #pragma unroll
         for (int k = 64 * h; k < 64 * h + 64; k += 2) mx[(k >> 1) & 3] = max3(mx[(k >> 1) & 3], s[k], s[k + 1]);
-        if (h == 0) tmem_wait_ld();
+        if (h == 0) tmem_wait_ld<64>(s + 64);
     }
     const float mx_row = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]) * c;
     const bool grow = mx_row > m_ref + 8.f;
@@ -589,7 +589,8 @@ __device__ __forceinline__ void publish_columns(const PfPlan& plan, int tail, in
     for (int q = 0; q < D / 16; ++q) {
         if ((q >= q0 && q < q1) == others) continue;
         float o[16];
-        tmem_ld16_wait(tO + q * 16, o);
+        tmem_ld16(tO + q * 16, o);
+        tmem_wait_ld<16>(o);
 #pragma unroll
         for (int i = 0; i < 4; ++i) __stcg(po + (q * 4 + i) * 128, make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]));
     }
@@ -727,7 +728,8 @@ __device__ __forceinline__ void merge_shares(const PfPlan& plan, int tail, const
                     float* a = o2 + 16 * i;
                     if (mine && have_o) {
                         __syncwarp();
-                        tmem_ld16_wait(tO + (q + i) * 16, a);
+                        tmem_ld16(tO + (q + i) * 16, a);
+                        tmem_wait_ld<16>(a);
                     }
 #pragma unroll
                     for (int c = 0; c < 16; ++c) if (fa > 0.f) o1[16 * i + c] += a[c] * fa;
@@ -1024,7 +1026,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     float o[32];
                     if (have_o) {
                         tmem_ld32(tO + q4 * 32, o);
-                        tmem_wait_ld();
+                        tmem_wait_ld<32>(o);
                     }
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] = have_o ? o[i] * inv : 0.f;

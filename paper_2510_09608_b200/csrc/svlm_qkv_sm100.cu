@@ -216,7 +216,7 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             for (int c32 = ew >> 2; c32 < width / 32; c32 += 2) {
                 float v[32];
                 tmem_ld32(tacc + c32 * 32, v);
-                tmem_wait_ld();
+                tmem_wait_ld<32>(v);
 #pragma unroll
                 for (int k = 0; k < 32; ++k) tr[(c32 * 32 + k) * QK_EPI_ROW] = v[k];
             }

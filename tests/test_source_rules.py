@@ -22,3 +22,24 @@ def test_only_constants_take_the_read_only_path():
         assert used <= constants, (name, used - constants)
         restricted = set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", src))
         assert restricted <= {"tab", "W"}, (name, restricted)
+
+
+def test_waits_for_tensor_memory_name_what_was_loaded():
+    """tcgen05.ld fills its registers when the wait behind it is over.  Two volatile statements stay in order, but arithmetic on the
+    registers is no such statement: only the wait's naming them keeps it behind."""
+    loads = waits = 0
+    for name in sorted(os.listdir(CSRC)):
+        src = _source(name)
+        if name == "svlm_tc.cuh":
+            body = re.search(r"void tmem_wait_ld\(float\* v\) \{(.*?)\n\}", src, flags=re.S).group(1)
+            assert body.index("tcgen05.wait::ld") < body.index('"+f"(v[i])') and src.count("tcgen05.wait::ld") == 1
+            continue
+        assert "tcgen05.ld" not in src and "tcgen05.wait::ld" not in src, name
+        # between a wait and the one before it: the loads it waits for, and it names as many registers as they fill
+        for part in re.split(r"(?<=;)", src):
+            if m := re.search(r"\btmem_ld(\d+)\(", part):
+                loads += int(m.group(1))
+            if re.search(r"\btmem_wait_ld\b", part):
+                waits += int(re.search(r"tmem_wait_ld<(\d+)>\(\w", part).group(1))
+        assert loads == waits, (name, loads, waits)
+    assert loads > 0
