@@ -306,8 +306,9 @@ struct PfGroup {
     PfWork w;
     PfWalk walk;
     int more;                // segments follow
-    int known;               // the cache that the next three belong to (-1: none): a launch does not change its metadata
+    int known;               // the cache that the next five belong to (-1: none): a launch does not change its metadata
     int n_tiles;
+    unsigned wait_limit;
     long long n_total, shift;
     long long first[128];    // smallest ordinals of the first pages of its list
     unsigned merge_later;    // shares of the first segment's unit that this CTA has to merge at the end
@@ -937,7 +938,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 if (fresh) {
                     ask = pf_ask(b, rows);
                 } else {
-                    ask.n_tiles = gr.n_tiles; ask.n_total = gr.n_total; ask.shift = gr.shift; ask.wait_limit = gr.w.wait_limit;
+                    ask.n_tiles = gr.n_tiles; ask.n_total = gr.n_total; ask.shift = gr.shift; ask.wait_limit = gr.wait_limit;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) ask.first[k] = gr.first[lane + 32 * k];
                 }
@@ -950,7 +951,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 bar_sync(BAR_WG + g, 128);
                 if (m == 0) gr.walk = walk;
                 if (fresh && m < 32) {
-                    if (m == 0) { gr.known = rows.ci; gr.n_tiles = ask.n_tiles; gr.n_total = ask.n_total; gr.shift = ask.shift; }
+                    if (m == 0) { gr.known = rows.ci; gr.n_tiles = ask.n_tiles; gr.n_total = ask.n_total; gr.shift = ask.shift; gr.wait_limit = ask.wait_limit; }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) gr.first[m + 32 * k] = ask.first[k];
                 }

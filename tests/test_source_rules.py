@@ -43,3 +43,17 @@ def test_waits_for_tensor_memory_name_what_was_loaded():
                 waits += int(re.search(r"tmem_wait_ld<(\d+)>\(\w", part).group(1))
         assert loads == waits, (name, loads, waits)
     assert loads > 0
+
+
+def test_what_a_chunk_prefill_block_keeps_of_a_cache_is_written_behind_the_barrier():
+    """Between units all threads read what is known of the cache while thread 0 replaces the segment's own fields: the two sets are
+    disjoint, and the first one is written behind the barrier that follows the reads."""
+    src = _source("svlm_prefill_sm100.cu")
+    at = src.index("rows.ci != gr.known")
+    known = src[src.index("} else {", at):src.index("rot.load_pos", at)]
+    read = set(re.findall(r"= gr\.([\w.]+)", known))
+    barrier = src.index("bar_sync(BAR_WG + g, 128);", at)
+    assert len(read) == 5
+    written_before = set(re.findall(r"gr\.(\w+)(?:\[[^]]*\])? = ", src[at:barrier]))
+    written_behind = set(re.findall(r"gr\.(\w+)(?:\[[^]]*\])? = ", src[barrier:src.index("PfTileRotation<D>::rotate", barrier)]))
+    assert read <= written_behind and not {r.split(".")[0] for r in read} & written_before, (read, written_before, written_behind)
