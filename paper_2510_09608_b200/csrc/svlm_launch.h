@@ -149,7 +149,7 @@ SvlmPrefillSmall svlm_prefill_small_plan(const SvlmAttendBatch& b, int call_laye
 cudaError_t svlm_launch_prefill_small(const SvlmAttendBatch& b, int layer0, int n_layers, const void* Q, const int* q_pos,
                                       int n_q, int q_heads, SvlmPrefillSmall how, void* out, cudaStream_t st);
 size_t svlm_prefill_slot_bytes(int n_pages, int head_dim);
-constexpr size_t svlm_prefill_counter_bytes = 4096;
+constexpr size_t svlm_prefill_counter_bytes = 8192;
 cudaError_t svlm_launch_prefill(const SvlmAttendBatch& b, int layer0, int n_layers, int call_layers, const void* Q, const int* q_pos,
                                 int n_q, int q_heads, void* out, const SvlmPrefillLoad* held, void* counters, void* slots,
                                 cudaStream_t st);

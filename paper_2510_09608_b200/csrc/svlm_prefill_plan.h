@@ -26,10 +26,38 @@ struct PfPlan {
     int tail;                         // the units from here on are dealt out by x
     unsigned short x[PF_MAX_CTAS + 1];// where each CTA's share of them begins, in 1/128 units
     unsigned g_magic;                 // for dividing by the heads per KV head (pf_div)
-    unsigned* counters;               // filled in at the launch: [2 * PF_MAX_CTAS][2] arrivals per (tail unit, tile), zero between launches;
+    unsigned* counters;               // filled in at the launch: [2 * PF_MAX_CTAS][2][2] per (tail unit, tile) arrivals, zero between launches, and a turn;
     unsigned char* slots;             //   [2 * grid] partial results
 };
-static_assert(2 * PF_MAX_CTAS * 2 * sizeof(unsigned) <= svlm_prefill_counter_bytes, "counters");
+static_assert(2 * PF_MAX_CTAS * 2 * 2 * sizeof(unsigned) <= svlm_prefill_counter_bytes, "counters");
+
+// How a cut unit of the tail is divided: its pieces lie with the thread blocks [first, last], those with an empty share left out;
+// the ones that end in it (all of them but one that has other segments to come) share the merge, in blocks of 16 columns, the
+// first `sharers` of them.
+struct PfCut {
+    int first, last, pieces, sharers;
+    unsigned mine;                    // blocks of columns that are thread block cta's, a bit each
+};
+__host__ __device__ inline PfCut pf_cut(const PfPlan& plan, int tail, int cta, int blocks) {
+    const int u0 = tail * PF_FRAC, u1 = u0 + PF_FRAC;
+    PfCut c;
+    for (c.first = cta; plan.x[c.first] > u0; --c.first) {}
+    for (c.last = cta; plan.x[c.last + 1] < u1; ++c.last) {}
+    int ends = 0, me = blocks;
+    c.pieces = 0;
+    for (int k = c.first; k <= c.last; ++k) {
+        if (plan.x[k] == plan.x[k + 1]) continue;
+        ++c.pieces;
+        if (plan.x[k + 1] > u1) continue;
+        if (k == cta) me = ends;
+        ++ends;
+    }
+    c.sharers = ends < blocks ? ends : blocks;
+    c.mine = 0;
+    for (int q = 0; q < blocks; ++q)
+        if (q * c.sharers >= me * blocks && q * c.sharers < (me + 1) * blocks) c.mine |= 1u << q;
+    return c;
+}
 
 // The work split of one launch (see the top of svlm_prefill_sm100.cu): whole units in rounds over the grid while at least two rounds
 // are left, the rest cut so that every CTA ends at the same level.  Beginning a unit, or another piece of one, costs as

@@ -271,33 +271,6 @@ __device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfSeg&
     return w;
 }
 
-// How a cut unit of the tail is divided, from the launch's arguments alone: its pieces lie with the CTAs [first, last], those
-// with an empty share left out; the CTAs that end in it (all of them but one that has other segments to come) share the merge,
-// in blocks of 16 columns, the first `sharers` of them.
-struct PfCut {
-    int first, last, pieces, sharers;
-    int me;                  // this CTA's share, -1: none
-};
-template <int D>
-__device__ __forceinline__ PfCut pf_cut(const PfPlan& plan, int tail) {
-    const int u0 = tail * PF_FRAC, u1 = u0 + PF_FRAC, cta = blockIdx.x;
-    PfCut c;
-    for (c.first = cta; plan.x[c.first] > u0; --c.first) {}
-    for (c.last = cta; plan.x[c.last + 1] < u1; ++c.last) {}
-    int ends = 0;
-    c.pieces = 0;
-    c.me = -1;
-    for (int k = c.first; k <= c.last; ++k) {
-        if (plan.x[k] == plan.x[k + 1]) continue;
-        ++c.pieces;
-        if (plan.x[k + 1] > u1) continue;
-        if (k == cta) c.me = ends;
-        ++ends;
-    }
-    c.sharers = min(ends, D / 16);
-    if (c.me >= c.sharers) c.me = -1;
-    return c;
-}
 // The softmax warpgroups keep what they know about their segment in shared memory: the page loop needs nearly all of
 // their registers for the row of scores.
 struct PfGroup {
@@ -311,7 +284,7 @@ struct PfGroup {
     unsigned wait_limit;
     long long n_total, shift;
     long long first[128];    // smallest ordinals of the first pages of its list
-    unsigned merge_later;    // shares of the first segment's unit that this CTA has to merge at the end
+    unsigned merge_later;    // blocks of columns of the first segment's unit that this CTA has to merge at the end
 };
 
 struct PfShared {            // control part of shared memory, behind the tiles
@@ -319,8 +292,8 @@ struct PfShared {            // control part of shared memory, behind the tiles
     unsigned long long s_full[2], all_done[2];
     unsigned tmem_base;
     int abort_flag;
-    unsigned take[2];                      // per tile: shares of a cut unit that this CTA has to merge
-    int leave[2];                          // its own share is left to whoever comes last
+    unsigned take[2];                      // per tile: blocks of columns of a cut unit that this CTA has to merge
+    int leave[2];                          // its own ones are left to whoever comes last
     PfCut cut[2];                          // of the CTA's last segment, of its first one
     PfGroup group[2];
 };
@@ -578,17 +551,14 @@ struct PfSlot {
     __device__ __forceinline__ float2* ml(int g, int m) const { return reinterpret_cast<float2*>(base + (size_t)PF_ROWS * D * 4) + g * 128 + m; }
 };
 
+// Blocks of 16 columns of this CTA's piece of a cut unit into its slot (un-normalised, fp32).
 template <int D>
-__device__ __forceinline__ int share_begin(const PfCut& c, int s) { return pf_small_div(s * (D / 16), c.sharers); }   // in blocks of 16 columns
-
-// Columns of this CTA's piece of a cut unit into its slot (un-normalised, fp32): the blocks of 16 in [q0, q1), or all others.
-template <int D>
-__device__ __forceinline__ void publish_columns(const PfPlan& plan, int tail, int g, int m, unsigned tO, bool have_o, int q0, int q1, bool others) {
+__device__ __forceinline__ void publish_columns(const PfPlan& plan, int tail, int g, int m, unsigned tO, bool have_o, unsigned blocks) {
     if (!have_o) return;
     float4* po = PfSlot<D>(plan, tail, blockIdx.x).o(g, m);
 #pragma unroll 1
-    for (int q = 0; q < D / 16; ++q) {
-        if ((q >= q0 && q < q1) == others) continue;
+    for (; blocks; blocks &= blocks - 1) {
+        const int q = __ffs(blocks) - 1;
         float o[16];
         tmem_ld16(tO + q * 16, o);
         tmem_wait_ld<16>(o);
@@ -597,145 +567,149 @@ __device__ __forceinline__ void publish_columns(const PfPlan& plan, int tail, in
     }
 }
 
-// The meeting of a unit's pieces, per tile: a word that counts arrivals (bits 0-7) and sharers that are through with it
-// (8-15) and names the shares whose owners did not wait (16-23).  A sharer has put down what the others need of its piece,
+// The meeting of a unit's pieces, per tile.  One word counts arrivals (bits 0-7) and names the blocks of columns whose owners did
+// not wait (16-23); a second one moves on when everybody is there.  A sharer has put down what the others need of its piece,
 // counts itself in and waits for the rest, which the work split lets end at the same time: `polls` times at most.  If they
 // are not there by then (their thread blocks may not even be running: another launch may hold the SMs) it puts down its own
-// columns too, names its share and leaves; whoever comes last merges those shares.  So nothing depends on a wait, and
-// whoever brings the word to its end clears it for the next launch.  Returns the shares this CTA has to merge.
+// columns too, names them and leaves; whoever comes last merges them.  So nothing depends on a wait.  The last one clears the
+// first word for the next launch.  Returns the blocks this CTA has to merge.
 constexpr int PF_MEET_POLLS = 14;         // polls: the control block's limit >> this (64 by default, some 40 us)
 template <int D>
 __device__ __forceinline__ unsigned meet_pieces(PfShared& sh, const PfPlan& plan, int tail, const PfCut& cut, int g, int m, unsigned tO, float m_row, float l,
                                                 bool have_o, unsigned polls) {
-    unsigned* word = plan.counters + tail * 2 + g;
-    const int q0 = cut.me < 0 ? 0 : share_begin<D>(cut, cut.me), q1 = cut.me < 0 ? 0 : share_begin<D>(cut, cut.me + 1);
-    auto add = [&](unsigned v) {                          // returns the new value; the end of the meeting clears the word
-        unsigned prev;
-        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(prev) : "l"(word), "r"(v) : "memory");
-        prev += v;
-        if ((prev & 0xffff) == (unsigned)(cut.pieces | cut.sharers << 8)) *word = 0;
-        return prev;
-    };
-    const PfSlot<D> slot(plan, tail, blockIdx.x);
-    __stcg(slot.ml(g, m), make_float2(have_o ? m_row : -INFINITY, l));
-    publish_columns<D>(plan, tail, g, m, tO, have_o, q0, q1, true);
+    constexpr unsigned ALL = (1u << (D / 16)) - 1;
+    unsigned* word = plan.counters + (tail * 2 + g) * 2;
+    unsigned turn = 0;                                       // of the second word: it cannot move before this CTA has arrived
+    if (m == 0) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(turn) : "l"(word + 1) : "memory");
+    __stcg(PfSlot<D>(plan, tail, blockIdx.x).ml(g, m), make_float2(have_o ? m_row : -INFINITY, l));
+    publish_columns<D>(plan, tail, g, m, tO, have_o, ALL & ~cut.mine);
     bar_sync(BAR_WG + g, 128);
     if (m == 0) {
         __threadfence();
-        const unsigned seen = add(1);
-        bool all = (seen & 255) == (unsigned)cut.pieces;
-        unsigned take = all ? seen >> 16 : 0;
-        if (cut.me >= 0) {
+        unsigned before, take = 0;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(word) : "memory");
+        bool all = (before & 255) == (unsigned)cut.pieces - 1;
+        if (all) {
+            take = cut.mine | before >> 16;
+            *word = 0;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word + 1) : "memory");
+        } else if (cut.mine) {
             for (unsigned p = 0; !all && p < polls; ++p) {
                 unsigned now;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(word) : "memory");
-                all = (now & 255) == (unsigned)cut.pieces;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(word + 1) : "memory");
+                all = now != turn;
             }
-            if (all) { take |= 1u << cut.me; add(1u << 8); }
+            take = all ? cut.mine : 0;
         }
         sh.take[g] = take;
-        sh.leave[g] = cut.me >= 0 && !all;
+        sh.leave[g] = cut.mine && !all;
     }
     bar_sync(BAR_WG + g, 128);
     if (sh.leave[g]) {
-        publish_columns<D>(plan, tail, g, m, tO, have_o, q0, q1, false);
+        publish_columns<D>(plan, tail, g, m, tO, have_o, cut.mine);
         bar_sync(BAR_WG + g, 128);
         if (m == 0) {
             __threadfence();
-            const unsigned seen = add((1u << 8) + (0x10000u << cut.me));
-            sh.take[g] = (seen & 255) == (unsigned)cut.pieces ? 1u << cut.me : 0;      // (the last one came in between: it did not see the name)
+            unsigned before;
+            asm volatile("atom.or.acq_rel.gpu.global.b32 %0, [%1], %2;" : "=r"(before) : "l"(word), "r"(cut.mine << 16) : "memory");
+            const unsigned n = before & 255;
+            const bool late = n == 0 || n == (unsigned)cut.pieces;      // the last one came in between: it has not seen the names, and clears or has cleared the word
+            if (late) *word = 0;
+            sh.take[g] = late ? cut.mine : 0;
         }
         bar_sync(BAR_WG + g, 128);
     }
     return sh.take[g];
 }
 
-// Some shares of a cut unit's output from its pieces: those of a share's owner come last, from TMEM if the owner is this CTA
-// (own: its last segment), all others from the slots in their order.  So the same bits come out every time, whoever does it.
-// 64 columns of two other pieces are asked for at once, together with the pieces' (m, l): mostly that is all there is (one
-// round trip to L2, where two pieces' 32 columns at a time, after the (m, l), took four).
+// Some blocks of columns of a cut unit's output from its pieces, in the order of the pieces, whoever does it: the same bits
+// every time.  This CTA's own piece may still be in TMEM (own: its last segment).  64 columns of the first two pieces are asked
+// for at once, together with all pieces' (m, l), and the row's maximum and sum are taken once for all blocks.
 template <int D>
-__device__ __forceinline__ void merge_shares(const PfPlan& plan, int tail, const PfCut& cut, unsigned take, const PfRows& w, int g, int m, int G, int q_heads,
+__device__ __forceinline__ void merge_blocks(const PfPlan& plan, int tail, const PfCut& cut, unsigned take, const PfRows& w, int g, int m, int G, int q_heads,
                                              bool own, unsigned tO, float m_row, float l, bool have_o, uint16_t* __restrict__ out) {
-    const int last = cut.last;
-    int owner = blockIdx.x, left;
-    auto after = [&](int k) {                                // the next piece that is not the owner's, last + 1: none
-        for (++k; k <= last && (k == owner || plan.x[k] >= plan.x[k + 1]); ++k) {}
+    const int first = cut.first, last = cut.last, me = own ? (int)blockIdx.x : -1;
+    const float m_own = have_o ? m_row : -INFINITY;
+    auto after = [&](int k) {                                // the next piece, last + 1: none
+        for (++k; k <= last && plan.x[k] >= plan.x[k + 1]; ++k) {}
         return k;
     };
-    auto load = [&](int k, int q, int nb, float (&o)[64]) {  // nb blocks of 16 columns (of a piece without pages: left over from earlier, not used)
-        const float4* po = PfSlot<D>(plan, tail, k).o(g, m) + q * 4 * 128;
+    auto load = [&](int k, int q, int nb, float (&o)[64]) {  // nb blocks (of a piece without pages: left over from earlier, not used)
+        if (k == me) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if (j < 4 * nb) {
-                const float4 v = ld_l2(po + j * 128);
-                o[4 * j] = v.x; o[4 * j + 1] = v.y; o[4 * j + 2] = v.z; o[4 * j + 3] = v.w;
-            }
+            for (int i = 0; i < 4; ++i)
+                if (i < nb && have_o) {
+                    __syncwarp();
+                    tmem_ld16(tO + (q + i) * 16, o + 16 * i);
+                    tmem_wait_ld<16>(o + 16 * i);
+                }
+        } else {
+            const float4* po = PfSlot<D>(plan, tail, k).o(g, m) + q * 4 * 128;
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (j < 4 * nb) {
+                    const float4 v = ld_l2(po + j * 128);
+                    o[4 * j] = v.x; o[4 * j + 1] = v.y; o[4 * j + 2] = v.z; o[4 * j + 3] = v.w;
+                }
+        }
     };
-    auto ml_of = [&](int k) { return k > last ? make_float2(-INFINITY, 0.f) : ld_l2(PfSlot<D>(plan, tail, k).ml(g, m)); };
+    auto ml_of = [&](int k) { return k == me ? make_float2(m_own, l) : ld_l2(PfSlot<D>(plan, tail, k).ml(g, m)); };
     const int mg = w.m0 + g * 128 + m;
     uint16_t* dst = out_row(out, w, min(mg, w.m_total - 1), plan.g_magic, G, q_heads, D);
     const bool wide = !(reinterpret_cast<uintptr_t>(out) & 31);
+    const int k2 = after(first);                             // (the first CTA's share is not empty, and a cut unit has two pieces at least)
+    const float m1 = ml_of(first).x, m2 = ml_of(k2).x;
+    float M = -INFINITY, inv = -1.f;
 #pragma unroll 1
-    for (; take; take &= take - 1) {
-        const int s = __ffs(take) - 1, q1 = share_begin<D>(cut, s + 1);
-        const bool mine = own && s == cut.me;
-        owner = blockIdx.x;
-        if (!mine)                                           // the s-th of the unit's pieces: those of the CTAs that end in it come first
-            for (owner = cut.first - 1, left = s; left >= 0; --left)
-                for (++owner; plan.x[owner] >= plan.x[owner + 1]; ++owner) {}
-        const int k1 = after(cut.first - 1), k2 = after(k1);
-        const float2 mla = mine ? make_float2(have_o ? m_row : -INFINITY, l) : ml_of(owner), ml1 = ml_of(k1), ml2 = ml_of(k2);
-        float M = -INFINITY, inv = 0.f;
+    while (take) {
+        const int q = __ffs(take) - 1, nb = min(4, __ffs(~(take >> q)) - 1);
+        take &= ~(((1u << nb) - 1) << q);
+        float o1[64], o2[64];
+        load(first, q, nb, o1);
+        load(k2, q, nb, o2);
+        if (inv < 0.f) {                                     // first time: the row's maximum and sum over all pieces, four in flight
+            float L = 0.f;
 #pragma unroll 1
-        for (int q = share_begin<D>(cut, s); q < q1; q += 4) {
-            const int nb = min(4, q1 - q);
-            float o1[64], o2[64];
-            load(k1, q, nb, o1);                             // (a cut unit has two pieces at least)
-            if (k2 <= last) load(k2, q, nb, o2);
-            if (inv == 0.f) {                                // first time: the row's maximum and sum over all pieces
-                M = max3(mla.x, ml1.x, ml2.x);
-                float L = 0.f;
-                auto add = [&](const float2& ml) { if (ml.x > -INFINITY) L += ml.y * exp2f(ml.x - M); };
-                add(mla); add(ml1); add(ml2);
-                for (int k = after(k2); k <= last; k = after(k)) {
-                    const float2 ml = ml_of(k);
-                    const float Mn = fmaxf(M, ml.x);
-                    if (Mn > M) { L *= exp2f(M - Mn); M = Mn; }      // M = -inf gives 0
-                    add(ml);
+            for (int k0 = first; k0 <= last; k0 += 4) {
+                float2 ml[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int k = min(k0 + i, last);
+                    ml[i] = ml_of(k);
+                    if (k0 + i > last || plan.x[k] >= plan.x[k + 1]) ml[i].x = -INFINITY;
                 }
-                inv = L > 0.f ? 1.f / L : 1.f;               // nothing visible: all weights below are 0
-            }
-            auto weight = [&](float mk) { return mk > -INFINITY ? exp2f(mk - M) * inv : 0.f; };
-            const float fa = weight(mla.x), f1 = weight(ml1.x), f2 = weight(ml2.x);
+                const float Mn = fmaxf(fmaxf(M, fmaxf(ml[0].x, ml[1].x)), fmaxf(ml[2].x, ml[3].x));
+                if (Mn > -INFINITY) {
+                    L *= exp2f(M - Mn);                      // M = -inf gives 0
 #pragma unroll
-            for (int c = 0; c < 64; ++c) {
-                float x = 0.f;
-                if (f1 > 0.f) x += o1[c] * f1;
-                if (f2 > 0.f) x += o2[c] * f2;
-                o1[c] = x;
-            }
-#pragma unroll 1
-            for (int k = after(k2); k <= last; k = after(k)) {
-                const float f = weight(ml_of(k).x);
-                load(k, q, nb, o2);
-#pragma unroll
-                for (int c = 0; c < 64; ++c) if (f > 0.f) o1[c] += o2[c] * f;
-            }
-            if (!mine) load(owner, q, nb, o2);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (i < nb) {
-                    float* a = o2 + 16 * i;
-                    if (mine && have_o) {
-                        __syncwarp();
-                        tmem_ld16(tO + (q + i) * 16, a);
-                        tmem_wait_ld<16>(a);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) if (fa > 0.f) o1[16 * i + c] += a[c] * fa;
-                    if (mg < w.m_total) store_row16(dst + (q + i) * 16, o1 + 16 * i, wide);
+                    for (int i = 0; i < 4; ++i) if (ml[i].x > -INFINITY) L += ml[i].y * exp2f(ml[i].x - Mn);
+                    M = Mn;
                 }
+            }
+            inv = L > 0.f ? 1.f / L : 0.f;
+        }
+        auto weight = [&](float mk) { return exp2f(mk - M) * inv; };
+        const bool has1 = m1 > -INFINITY, has2 = m2 > -INFINITY;
+        const float f1 = weight(m1), f2 = weight(m2);
+#pragma unroll
+        for (int c = 0; c < 64; ++c) {
+            float x = has1 ? o1[c] * f1 : 0.f;
+            if (has2) x += o2[c] * f2;
+            o1[c] = x;
+        }
+#pragma unroll 1
+        for (int k = after(k2); k <= last; k = after(k)) {
+            const float mk = ml_of(k).x;
+            load(k, q, nb, o2);
+            if (mk > -INFINITY) {
+                const float f = weight(mk);
+#pragma unroll
+                for (int c = 0; c < 64; ++c) o1[c] += o2[c] * f;
+            }
+        }
+        if (mg < w.m_total) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) if (i < nb) store_row16(dst + (q + i) * 16, o1 + 16 * i, wide);
         }
     }
 }
@@ -773,7 +747,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
     }
     if (threadIdx.x == 32 || threadIdx.x == 64) {      // cut units: the last segment's, and the first one's where that is the end of one
         const int x0 = plan.x[blockIdx.x], x1 = plan.x[blockIdx.x + 1], which = threadIdx.x / 32 - 1;
-        if (x0 < x1) sh.cut[which] = pf_cut<D>(plan, (which ? x0 : x1 - 1) / PF_FRAC);
+        if (x0 < x1) sh.cut[which] = pf_cut(plan, (which ? x0 : x1 - 1) / PF_FRAC, blockIdx.x, D / 16);
     }
     // Set up while the predecessor ends (programmatic dependent launch); everything read from here on may be its work.
     // The wait comes before the trigger: a successor that starts early then finds all earlier work done.
@@ -1049,11 +1023,11 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         bar_sync(BAR_WG + g, 128);
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
-            const unsigned shares = pass == 0 ? take : gr.merge_later;
-            if (!shares) continue;
+            const unsigned blocks = pass == 0 ? take : gr.merge_later;
+            if (!blocks) continue;
             const int tail = (pass == 0 ? plan.x[blockIdx.x + 1] - 1 : (int)plan.x[blockIdx.x]) / PF_FRAC;
             const PfRows rows = pf_rows(b, plan, plan.tail + tail, n_q_arg, G, layer0, n_layers);
-            merge_shares<D>(plan, tail, sh.cut[pass], shares, rows, g, m, G, q_heads, pass == 0, tO, m_ref, l, have_o, out);
+            merge_blocks<D>(plan, tail, sh.cut[pass], blocks, rows, g, m, G, q_heads, pass == 0, tO, m_ref, l, have_o, out);
         }
     }
 

@@ -169,6 +169,25 @@ PLAN_PROGRAM = r"""
 
 static SvlmAttendBatch batch(int kv_heads) { SvlmAttendBatch b{}; b.n_caches = 1; b.kv_heads = kv_heads; return b; }
 
+// A cut unit's pieces are counted alike by all that hold one, and its columns are shared out once among those that end in it.
+static void check_cut_units(const PfPlan& plan, int grid, int nt, int blocks) {
+    for (int t = 0; t < nt; ++t) {
+        const int u0 = t * PF_FRAC, u1 = u0 + PF_FRAC;
+        int pieces = 0;
+        unsigned shared = 0;
+        for (int k = 0; k < grid; ++k) pieces += plan.x[k] < plan.x[k + 1] && plan.x[k] < u1 && plan.x[k + 1] > u0;
+        if (pieces < 2) continue;
+        for (int k = 0; k < grid; ++k) {
+            if (!(plan.x[k] < plan.x[k + 1] && plan.x[k] < u1 && plan.x[k + 1] > u0)) continue;
+            const PfCut c = pf_cut(plan, t, k, blocks);
+            assert(c.pieces == pieces && c.sharers >= 1 && plan.x[c.first] <= u0 && plan.x[c.first] < plan.x[c.first + 1] && plan.x[c.last + 1] >= u1);
+            assert(!(c.mine & shared) && (!c.mine || plan.x[k + 1] <= u1));
+            shared |= c.mine;
+        }
+        assert(shared == (1u << blocks) - 1);
+    }
+}
+
 int main() {
     PfPlanMemo& memo = pf_plan_memo();
     SvlmAttendBatch b = batch(4);
@@ -198,6 +217,7 @@ int main() {
                                 assert(p.plan.x[i] <= p.plan.x[i + 1]);
                                 if (!cut) assert(p.plan.x[i] % PF_FRAC == 0);
                             }
+                            for (int blocks : {4, 8}) check_cut_units(p.plan, p.grid, nt, blocks);
                             ++checked;
                         }
     std::printf("%lld\n", checked);
