@@ -33,7 +33,11 @@ static_assert(2 * PF_MAX_CTAS * 2 * 2 * sizeof(unsigned) <= svlm_prefill_counter
 
 // How a cut unit of the tail is divided: its pieces lie with the thread blocks [first, last], those with an empty share left out;
 // the ones that end in it (all of them but one that has other segments to come) share the merge, in blocks of 16 columns, the
-// first `sharers` of them.
+// first `sharers` of them; 0: whoever comes last merges all.  Sharing pays from two that end together and eight blocks on: a
+// thread block that shares puts its columns down before it knows whether it is the last, and the last one by itself has half
+// as much to read at head_dim 64.  Us per layer with its append, shared and by the last one alone: head_dim 64, 12/2 heads, 524 tokens
+// over 9200 keys 52.8, 50.5; 16/8 heads, 390 tokens over 1250 keys 35.8, 34.6; head_dim 128, 28/4 heads, 69 tokens over 9200 keys 47.0, 57 (the merge
+// before there were shares), 524 tokens 85.7, 91; one that ends in the unit, 1500 tokens 177.9, 177.0.
 struct PfCut {
     int first, last, pieces, sharers;
     unsigned mine;                    // blocks of columns that are thread block cta's, a bit each
@@ -52,7 +56,7 @@ __host__ __device__ inline PfCut pf_cut(const PfPlan& plan, int tail, int cta, i
         if (k == cta) me = ends;
         ++ends;
     }
-    c.sharers = ends < blocks ? ends : blocks;
+    c.sharers = blocks < 8 || ends < 2 ? 0 : ends < blocks ? ends : blocks;
     c.mine = 0;
     for (int q = 0; q < blocks; ++q)
         if (q * c.sharers >= me * blocks && q * c.sharers < (me + 1) * blocks) c.mine |= 1u << q;

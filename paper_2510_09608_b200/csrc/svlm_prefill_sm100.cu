@@ -9,7 +9,7 @@
 // made from the numbers of rows and an estimate of the pages (svlm_prefill_plan.h): first whole units, round by round over
 // the grid (neighbouring CTAs then stream the same pages at the same time), then its share of the last one to two rounds'
 // units, dealt out evenly in pages, so that no SM idles in a last wave (120 of 148 SMs had work for one stream's chunk before, 960 CTAs were 6.5
-// waves for eight streams).  A unit that is cut between CTAs is merged by those that end in it, each a share of its columns,
+// waves for eight streams).  A unit that is cut between CTAs is merged by those that end in it, each a share of its columns, or by the last of them,
 // through un-normalised pieces (O, m, l) in the cache's scratch; nothing depends on a wait (meet_pieces).
 //
 // Roles (384 threads, registers moved from warpgroup 2 to the softmax with setmaxnreg):
@@ -573,12 +573,26 @@ __device__ __forceinline__ void publish_columns(const PfPlan& plan, int tail, in
 // are not there by then (their thread blocks may not even be running: another launch may hold the SMs) it puts down its own
 // columns too, names them and leaves; whoever comes last merges them.  So nothing depends on a wait.  The last one clears the
 // first word for the next launch.  Returns the blocks this CTA has to merge.
+// Where nobody shares, the last one merges all, and keeps its piece in TMEM if the others are there already (last: the CTA's last
+// segment, whose piece may stay there).
 constexpr int PF_MEET_POLLS = 14;         // polls: the control block's limit >> this (64 by default, some 40 us)
 template <int D>
 __device__ __forceinline__ unsigned meet_pieces(PfShared& sh, const PfPlan& plan, int tail, const PfCut& cut, int g, int m, unsigned tO, float m_row, float l,
-                                                bool have_o, unsigned polls) {
+                                                bool have_o, bool last, unsigned polls) {
     constexpr unsigned ALL = (1u << (D / 16)) - 1;
     unsigned* word = plan.counters + (tail * 2 + g) * 2;
+    if (last && cut.sharers == 0) {
+        if (m == 0) {
+            unsigned now;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(word) : "memory");
+            sh.take[g] = (now & 255) == (unsigned)cut.pieces - 1 ? ALL : 0;
+        }
+        bar_sync(BAR_WG + g, 128);
+        if (sh.take[g]) {
+            if (m == 0) *word = 0;
+            return ALL;
+        }
+    }
     unsigned turn = 0;                                       // of the second word: it cannot move before this CTA has arrived
     if (m == 0) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(turn) : "l"(word + 1) : "memory");
     __stcg(PfSlot<D>(plan, tail, blockIdx.x).ml(g, m), make_float2(have_o ? m_row : -INFINITY, l));
@@ -590,7 +604,7 @@ __device__ __forceinline__ unsigned meet_pieces(PfShared& sh, const PfPlan& plan
         asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(word) : "memory");
         bool all = (before & 255) == (unsigned)cut.pieces - 1;
         if (all) {
-            take = cut.mine | before >> 16;
+            take = cut.sharers ? cut.mine | before >> 16 : ALL;
             *word = 0;
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word + 1) : "memory");
         } else if (cut.mine) {
@@ -1011,7 +1025,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     }
                 }
             } else if (gr.more) {                                      // the end of a unit that others have begun
-                const unsigned take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[1], g, m, tO, m_ref, l, have_o, 0);
+                const unsigned take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[1], g, m, tO, m_ref, l, have_o, false, 0);
                 if (m == 0) gr.merge_later = take;
             }
         }
@@ -1019,7 +1033,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         const bool have_o = ok && gr.w.n_proc > 0;
         unsigned take = 0;
         if (gr.seg.e - gr.seg.a < PF_FRAC)
-            take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[0], g, m, tO, m_ref, l, have_o, gr.w.wait_limit >> PF_MEET_POLLS);
+            take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[0], g, m, tO, m_ref, l, have_o, true, gr.w.wait_limit >> PF_MEET_POLLS);
         bar_sync(BAR_WG + g, 128);
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
