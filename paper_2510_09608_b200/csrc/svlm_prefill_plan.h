@@ -58,7 +58,7 @@ __host__ __device__ inline PfCut pf_cut(const PfPlan& plan, int tail, int cta, i
     }
     c.sharers = blocks < 8 || ends < 2 ? 0 : ends < blocks ? ends : blocks;
     c.mine = 0;
-    for (int q = 0; q < blocks; ++q)
+    for (int q = 0; q < blocks && me < c.sharers; ++q)
         if (q * c.sharers >= me * blocks && q * c.sharers < (me + 1) * blocks) c.mine |= 1u << q;
     return c;
 }
