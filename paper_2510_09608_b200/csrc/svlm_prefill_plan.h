@@ -13,7 +13,11 @@ constexpr int PF_MAX_CTAS = 160;
 // 56.6 us, 12 48.9, 8 44.8.
 constexpr int PF_MIN_PAGES = 4;
 constexpr int PF_MAX_PIECES = 9;
-constexpr int PF_PIECE = 8;           // what beginning a unit is reckoned as, in pages (one stream, 28 layers: 10: 2.52 ms, 8: 2.43, 5: 2.43; four layers of a long chunk 1.71, 1.72 with 5)
+// What beginning a unit is reckoned as, in pages.  The cuts also decide against which reference maximum a row's weights are
+// rounded to bf16 (a piece begins its own), so another number here changes outputs in their last places: it stays where it is
+// unless that is worth it.  With 8, 196 chunk shapes (69 to 4133 tokens, 1200 to 9200 keys, six head shapes, one to eight streams) take 0.3 % less on
+// average, between 4 % less (69 tokens, 28/4 heads) and 3 % more (12/2 heads of 64, 266 tokens).
+constexpr int PF_PIECE = 10;
 constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
 
 // The work split, made on the host: it needs the numbers of rows, and of the pages only an estimate (a unit's pages are

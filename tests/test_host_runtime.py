@@ -204,6 +204,7 @@ int main() {
     for (int n = 2; n < 400; n += 13) pf_plan(b, 1, n, 7, held, 148, true);
     // every page fraction of every unit is dealt out once, in order
     long long checked = 0;
+    unsigned cuts = 2166136261u;
     for (int kv_heads : {1, 4, 8})
         for (int G : {1, 4, 7})
             for (int n : {2, 37, 256, 531, 4133})
@@ -221,21 +222,23 @@ int main() {
                                 assert(p.plan.x[i] <= p.plan.x[i + 1]);
                                 if (!cut) assert(p.plan.x[i] % PF_FRAC == 0);
                             }
+                            for (int i = 0; i <= p.grid; ++i) cuts = (cuts ^ p.plan.x[i]) * 16777619u;
                             for (int blocks : {4, 8}) check_cut_units(p.plan, p.grid, nt, blocks);
                             ++checked;
                         }
-    std::printf("%lld\n", checked);
+    std::printf("%lld %u\n", checked, cuts);
 }
 """
 
 
 def test_chunk_prefill_work_split(tmp_path):
-    """The host's work split: remembered by sizes alone, and complete."""
+    """The host's work split: remembered by sizes alone, complete, and with the cuts where they have been: a row's weights are rounded
+    against the reference maximum of its piece, so outputs change in their last places with the cuts."""
     src, exe = tmp_path / "plan.cpp", tmp_path / "plan"
     src.write_text(PLAN_PROGRAM)
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-I/usr/local/cuda/include", "-I" + os.path.join(ROOT, "paper_2510_09608_b200", "csrc"),
                            "-o", str(exe), str(src)])
-    assert subprocess.check_output([str(exe)], text=True).strip() == str(3 * 3 * 5 * 4 * 2 * 2)
+    assert subprocess.check_output([str(exe)], text=True).strip() == f"{3 * 3 * 5 * 4 * 2 * 2} 3026906603"
 
 
 def test_a_cache_that_fits_without_the_scratch_for_cut_units(host):
