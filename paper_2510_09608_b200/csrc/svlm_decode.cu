@@ -144,13 +144,18 @@ __device__ __forceinline__ void ld_tagged2(const void* p, unsigned long long& a,
 
 // ---- a decode step that appends its token itself ------------------------------------------------------------------
 //
-// Where one launch attends in all of a cache's layers (caches of one layer), the token's bookkeeping needs no launch of its own in front: every CTA works out from the old metadata what the token changes, uses the
-// list of pages as it will be, and counts itself as through with the old metadata; the last one to do so writes the change
-// down at its end (nobody waits).  A launch and its chain of round trips less in front of each step: one layer of 4/1 heads of
-// 64 over 200 keys 8.9 -> 7.1 us, 16 streams of 4 heads of 128 over 9216 keys 56.4 -> 55.2.  A step that is followed by
-// another layer's keeps the launch of its own: that layer's kernel reads the metadata ahead, while this one runs.  So do all
-// layers in one call, whose inputs may be in host memory: there every CTA would fetch type and position over the bus
-// (a second of 28 layers end to end 5.12 -> 5.29 ms).
+// Where one launch attends in all of a cache's layers (caches of one layer), the token's bookkeeping needs no launch of
+// its own in front: every CTA works out from the old metadata what the token changes, uses the list of pages as it will
+// be, and counts itself as through with the old metadata; the last one to do so writes the change down at its end (nobody
+// waits).  A launch and its chain of round trips less in front of each step: one layer of 4/1 heads of 64 over 200 keys
+// 8.7 -> 7.7 us, 16 streams of 4 heads of 128 over 9216 keys 54.3 -> 52.3.  A step that is followed by another layer's keeps the
+// launch of its own: that layer's kernel reads the metadata ahead, while this one runs.  So do all layers in one call of a
+// deeper cache, whose inputs may be in host memory: there every CTA would fetch type and position over the bus (a second of
+// 28 layers end to end 5.12 -> 5.29 ms).
+// Its successor starts when this kernel is gone, not beside it: the next step's CTAs would take the places that become free
+// one by one, two on some SMs and none on others (by calls, 8 heads of 128: 9216 keys 15.0 us a step, this way 12.2, with the
+// launch of its own 13.7; 17,500 keys 21.3, 16.7, 18.1; replayed from a graph, where the next step is not there yet: 12.0
+// either way, the smallest step above 7.0 and 7.7).
 struct DecNoAppend { static constexpr bool on = false; };
 struct DecAppend {
     static constexpr bool on = true;
@@ -637,7 +642,7 @@ decode_stream_kernel(SvlmAttendBatch b, int layer0, int n_layers, const uint16_t
     // kernel (whatever that kernel's own trigger), not merely behind one that has been launched.
     const auto rule = dec_rule(app, ci);      // (read ahead: nothing in the stream writes it)
     if (!early_loads) pdl_wait();
-    pdl_launch_dependents();
+    if (!Append::on) pdl_launch_dependents();
     const unsigned wait_limit = ld_l2(&vw.ctrl->wait_limit);
     int n_tiles, new_slot = -1;
     long long shift;
@@ -987,7 +992,7 @@ decode_layer_kernel(SvlmAttendBatch b, int layer, const uint16_t* Q, const int* 
     // kernel (whatever that kernel's own trigger), not merely behind one that has been launched.
     const auto rule = dec_rule(app, ci);      // (read ahead: nothing in the stream writes it)
     if (!early_loads) pdl_wait();
-    pdl_launch_dependents();
+    if (!Append::on) pdl_launch_dependents();
     int n_tiles, new_slot = -1;
     long long shift;
     unsigned before = 0;                             // (of the last warp's first thread)

@@ -57,3 +57,10 @@ def test_what_a_chunk_prefill_block_keeps_of_a_cache_is_written_behind_the_barri
     written_before = set(re.findall(r"gr\.(\w+)(?:\[[^]]*\])? = ", src[at:barrier]))
     written_behind = set(re.findall(r"gr\.(\w+)(?:\[[^]]*\])? = ", src[barrier:src.index("PfTileRotation<D>::rotate", barrier)]))
     assert read <= written_behind and not {r.split(".")[0] for r in read} & written_before, (read, written_before, written_behind)
+
+
+def test_a_decode_step_that_appends_lets_nobody_start_beside_it():
+    """The next step's thread blocks would take the places that its own leave one by one, unevenly over the SMs."""
+    src = _source("svlm_decode.cu")
+    starts = [line.strip() for line in src.splitlines() if "pdl_launch_dependents" in line]
+    assert len(starts) == 2 and all(line.startswith("if (!Append::on)") for line in starts), starts
