@@ -66,8 +66,9 @@ inline int svlm_sm_count() {
 // metadata (svlm_meta.cu).  Where one of these fails, whatever was to follow it must not be launched: it would take the
 // metadata of the operation before for its own.
 cudaError_t svlm_launch_append_meta(const SvlmCacheDev& cd, const unsigned char* types, const int* pos, int n, cudaStream_t st);
-// rotate: the launch re-rotates the moved keys too (svlm_evict_in_one; otherwise svlm_launch_evict_rotate has to follow)
-bool svlm_evict_in_one(const SvlmCacheDev& cd);
+// rotate: the launch re-rotates the moved keys too (svlm_evict_in_one; otherwise svlm_launch_evict_rotate has to follow).
+// stored: what the cache is expected to hold (the route depends on it, the result does not)
+bool svlm_evict_in_one(const SvlmCacheDev& cd, long long stored);
 cudaError_t svlm_launch_evict_meta(const SvlmCacheDev& cd, bool rotate, cudaStream_t st);
 // an append's metadata and its keys and values (svlm_launch_kv_write's) in one launch, where svlm_append_in_one says so
 bool svlm_append_in_one(const SvlmCacheDev& cd, int layer, int n);

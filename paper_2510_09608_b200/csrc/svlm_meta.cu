@@ -825,13 +825,18 @@ cudaError_t svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmC
 // 32.9 and 17.7.  (By plain calls a launch less saves the host 2 us more.)
 constexpr long long APPEND_WRITE_ELEMENTS = 4096;      // of the appended keys
 constexpr long long EVICT_ROTATE_ELEMENTS = 16384;     // of the keys that the windows keep
+// An eviction in one launch also walks over the tokens that leave, with 256 threads where the other form has 1024.  Append and
+// eviction of n tokens over 190 kept, one head of 64, vision, text and both in turn, us in one launch and in two: 700 20.6,
+// 19.4, 22.7 and 22.2, 20.9, 22.8; 1024 20.7, 22.6, 22.7 and 22.6, 22.7, 23.9; 1536 26.8, 26.8, 28.2 and 26.8, 28.5, 27.1; 2048 28.8, 28.8,
+// 30.6 and 27.3, 28.8, 28.8; 3000 35.0, 35.5, 35.9 and 32.9, 33.0, 34.7.
+constexpr long long EVICT_ROTATE_LEAVING = 1024;
 static_assert(EVICT_ROTATE_ELEMENTS / 64 <= ROTATE_THREADS, "a thread per retained token (heads have 64 dims at least)");
 bool svlm_append_in_one(const SvlmCacheDev& cd, int layer, int n) {
     return n <= META_THREADS && (long long)n * (layer < 0 ? cd.layers : 1) * cd.kv_heads * cd.head_dim <= APPEND_WRITE_ELEMENTS;
 }
-bool svlm_evict_in_one(const SvlmCacheDev& cd) {
-    const long long kept = std::min((long long)cd.n_sink + cd.vision_window + cd.text_window, (long long)cd.n_slots);
-    return kept * cd.layers * cd.kv_heads * cd.head_dim <= EVICT_ROTATE_ELEMENTS;
+bool svlm_evict_in_one(const SvlmCacheDev& cd, long long stored) {
+    const long long windows = (long long)cd.n_sink + cd.vision_window + cd.text_window, kept = std::min(windows, (long long)cd.n_slots);
+    return stored - windows <= EVICT_ROTATE_LEAVING && kept * cd.layers * cd.kv_heads * cd.head_dim <= EVICT_ROTATE_ELEMENTS;
 }
 
 cudaError_t svlm_launch_append_in_one(const SvlmCacheDev& cd, int layer, const void* K, const void* V, const unsigned char* types, const int* pos, int n, cudaStream_t st) {

@@ -601,7 +601,7 @@ int svlm_cache_evict(svlm_cache* c) {
     if (!c) return SVLM_ERR_ARG;
     DeviceGuard guard(c->device);
     c->last_decode_layer = -1;
-    const bool in_one = c->dev.contiguous && svlm_evict_in_one(c->dev);
+    const bool in_one = c->dev.contiguous && svlm_evict_in_one(c->dev, c->stored_est);
     SVLM_CUDA(svlm_launch_evict_meta(c->dev, in_one, c->stream));
     note_evict(c);
     if (c->dev.contiguous && !in_one) SVLM_CUDA(svlm_launch_evict_rotate(c->dev, c->stream));
@@ -616,7 +616,7 @@ int svlm_cache_evict_batched(svlm_cache* const* caches, int n_caches) {
     DeviceGuard guard(c0->device);
     bool rotate = false, in_one = true;
     for (int i = 0; i < n_caches; ++i) {
-        in_one = in_one && svlm_evict_in_one(caches[i]->dev);
+        in_one = in_one && svlm_evict_in_one(caches[i]->dev, caches[i]->stored_est);
         caches[i]->last_decode_layer = -1;
         rotate = rotate || caches[i]->dev.contiguous;   // a cache with native positions never sets evict_moved
     }

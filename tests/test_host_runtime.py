@@ -281,3 +281,25 @@ for vw, tw, n, kernel in ((512, 64, 130, "prefill_small"), (1536, 128, 520, "14p
     ran()
     assert attend(c, n) == OK and kernel in ran()[-1], kernel
 """)
+
+
+def test_evictions_of_many_tokens_take_two_launches(host):
+    """One launch serves a small cache's eviction with few threads, which also walk over all tokens that leave: few of them only."""
+    host("""
+small = dict(layers=1, hk=1, d=64, sink=4, vw=120, tw=70, capacity=5000)
+def evicts(c, batch=None):
+    ran()
+    assert (lib.svlm_cache_evict_batched(arr(batch), len(batch)) if batch else lib.svlm_cache_evict(c)) == OK
+    return [l.split()[0] for l in ran()]
+one = lambda names: len(names) == 1 and "evict_meta" in names[0]
+two = lambda names: len(names) == 2 and "evict_meta" in names[0] and "evict_rotate" in names[1]
+c, d = new(**small), new(**small)
+for n, kernels in ((194, one), (1024, one), (30, one), (1025, two), (4608, two), (1024, one)):
+    assert append(c, n, layer=-1) == OK
+    assert kernels(evicts(c)), n
+for n, kernels in ((1024, one), (1025, two)):                # of a batch: by the cache that has most to lose
+    assert append(c, 40, layer=-1) == OK and append(d, n, layer=-1) == OK
+    if n == 1024:
+        assert append(d, 194, layer=-1) == OK                # (the windows were empty)
+    assert kernels(evicts(None, [c, d])), n
+""")
