@@ -830,12 +830,13 @@ int svlm_decode_step_host(svlm_cache* c, int layer, const void* K_host, const vo
         return SVLM_ERR_ARG;
     if (layer <= 0 && !token_type_host) return SVLM_ERR_ARG;
     DeviceGuard guard(c->device);
-    if (layer < 0) {
+    if (layer < 0 && c->dev.layers > 1) {
         // All layers of a generated token in one launch: the inputs are a few KB per layer, and when all of them sit
         // in pinned, mapped host memory the kernels read them where they are and write the output where it belongs,
         // which costs one bus round trip inside the kernel instead of five small copies in front of it and one
         // behind (7.4-7.8 -> 6.2 ms per chunk end to end on the config-3 step).  Not for a single layer: there all
-        // 37 CTAs of a KV head would fetch the same query over the bus (measured: 36 against 32 ms per chunk).
+        // 37 CTAs of a KV head would fetch the same query over the bus (measured: 36 against 32 ms per chunk; all layers of a
+        // one-layer cache, whose step also appends in every CTA: 4/1 heads of 64 over 200 keys 42 us, staged 23, 28/4 heads over 9200 47, 26).
         // Anything else goes through the staging buffer below.
         void* dK = mapped_alias(K_host);
         void* dV = dK ? mapped_alias(V_host) : nullptr;

@@ -13,7 +13,7 @@ std::map<const void*, std::string> g_names;
 std::string g_log, g_fail;
 cudaError_t g_last = cudaSuccess;
 size_t g_alloc_limit = ~(size_t)0;
-int g_capturing = 0;
+int g_capturing = 0, g_mapped = 0;
 cudaError_t done(cudaError_t e) { if (e != cudaSuccess) g_last = e; return e; }
 cudaError_t launch(const void* f, dim3 grid, dim3 block) {
     const std::string& name = g_names[f];
@@ -30,6 +30,7 @@ void fake_fail(const char* kernel) { g_fail = kernel; }          // launches of 
 const char* fake_log() { static std::string out; out = g_log; g_log.clear(); return out.c_str(); }   // launches since the last call
 void fake_alloc_limit(size_t bytes) { g_alloc_limit = bytes; }   // allocations above this size fail
 void fake_capturing(int on) { g_capturing = on; }                // the streams are being captured
+void fake_mapped(int on) { g_mapped = on; }                      // host memory is page-locked and mapped
 
 // ---- the runtime's calls that the library makes ----
 static dim3 g_grid, g_block;
@@ -74,7 +75,11 @@ cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cu
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = nullptr; return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void*) { std::memset(a, 0, sizeof *a); return cudaSuccess; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
+    std::memset(a, 0, sizeof *a);
+    if (g_mapped) { a->type = cudaMemoryTypeHost; a->devicePointer = const_cast<void*>(p); }
+    return cudaSuccess;
+}
 cudaError_t cudaGetSymbolAddress(void** p, const void* s) { *p = const_cast<void*>(s); return cudaSuccess; }
 cudaError_t cudaGetDriverEntryPoint(const char*, void** f, unsigned long long, cudaDriverEntryPointQueryResult* r) {
     *f = reinterpret_cast<void*>(encode_nothing);

@@ -207,23 +207,24 @@ def test_projection_shapes(layers, n, in_dim, out_dim):
 
 
 # --- one layer's token from host memory, page-locked or not: moved by kernels up to 64 KB, by copies above; the same bits as
-# --- from device memory
+# --- from device memory (two layers in turn; all layers of a cache that has one, where the step appends by itself)
+@pytest.mark.parametrize("layers", [2, 1])
 @pytest.mark.parametrize("d,hq,hk,pinned", [(64, 4, 1, True), (128, 28, 4, True), (128, 28, 4, False), (128, 96, 12, True), (128, 160, 20, False)])
-def test_host_decode_steps_of_one_layer(d, hq, hk, pinned):
+def test_host_decode_steps_of_one_layer(d, hq, hk, pinned, layers):
     from paper_2510_09608_b200 import binding
     rng = np.random.default_rng(hq)
     bits = lambda *shape: torch.from_numpy(rng.standard_normal(shape).astype(np.float32)).to(torch.bfloat16)      # noqa: E731
     keep = (lambda t: t.pin_memory()) if pinned else (lambda t: t)
-    dev, host = (binding.Cache(2, hk, d, 4, 150, 60, 512) for _ in range(2))
+    dev, host = (binding.Cache(layers, hk, d, 4, 150, 60, 512) for _ in range(2))
     for c in (dev, host):
         c.set_rope(binding.ROPE_1D, 1.0e4)
-    k, v = bits(2, 200, hk, d), bits(2, 200, hk, d)
+    k, v = bits(layers, 200, hk, d), bits(layers, 200, hk, d)
     ty, ps = torch.ones(200, dtype=torch.uint8), torch.arange(200, dtype=torch.int32)
     for c in (dev, host):
         c.append(-1, k.cuda(), v.cuda(), ty.cuda(), ps.cuda())
         c.evict()
     for step in range(3):
-        for l in range(2):
+        for l in (range(2) if layers == 2 else (-1,)):
             k, v, q = bits(1, hk, d), bits(1, hk, d), bits(1, hq, d)
             ty, ps = torch.zeros(1, dtype=torch.uint8), torch.tensor([200 + step], dtype=torch.int32)
             want = dev.decode_step(l, k.cuda(), v.cuda(), ty.cuda(), ps.cuda(), q.cuda())

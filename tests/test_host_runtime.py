@@ -303,3 +303,23 @@ for n, kernels in ((1024, one), (1025, two)):                # of a batch: by th
         assert append(d, 194, layer=-1) == OK                # (the windows were empty)
     assert kernels(evicts(None, [c, d])), n
 """)
+
+
+def test_which_host_buffers_the_kernels_read_in_place(host):
+    """All layers of a token from mapped host memory: the decode launch reads them where they are, one of each for all the thread
+    blocks that want them.  One layer goes through device memory, also when it is all that the cache has."""
+    host("""
+fake.fake_mapped(1)
+buf = (C.c_char * (1 << 16))()
+at = vp(C.addressof(buf) + 63 & ~63)
+def kernels(layers, layer):
+    c = new(layers=layers)
+    assert append(c, 40, layer=-1) == OK
+    ran()
+    assert lib.svlm_decode_step_host(c, layer, at, at, at, at, at, 28, at) == OK
+    return " ".join(l.split()[0] for l in ran())
+deep = kernels(3, -1)
+assert "host_in" not in deep and "append_meta" in deep and "decode" in deep
+for layers, layer in ((3, 0), (1, 0), (1, -1)):
+    assert "host_in" in kernels(layers, layer), (layers, layer)
+""")
