@@ -18,7 +18,7 @@
 #define SVLM_MAX_HALF 64   // head_dim/2 <= 64
 #define SVLM_MAX_BATCH 32
 
-struct SvlmCtrl {            // one per cache, device memory; only meta kernels write it
+struct SvlmCtrl {            // one per cache, device memory; written by the metadata kernels and by decode steps that append by themselves
     long long n_total;       // tokens ever appended = next stream ordinal (gid)
     long long n_type[2];     // per-type ordinals issued so far (TEXT, VISION)
     long long cursor;        // native position cursor (max native index + 1 seen so far)

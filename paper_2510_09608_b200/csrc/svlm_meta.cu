@@ -741,48 +741,44 @@ __global__ void __launch_bounds__(FORM == APPEND_ONE ? ONE_THREADS : META_THREAD
 }
 
 // Append of a few tokens with the write of their keys and values in one launch: the block that places the tokens also rotates
-// and stores their rows, a thread per (token, 8 pairs) and row of [layer][kv head].  The first rows are asked for before
-// the metadata, which they have nothing to do with.
-__global__ void __launch_bounds__(META_THREADS) append_meta_write_kernel(SvlmCacheDev cd, const unsigned char* types, const int* pos, int n, const uint16_t* K,
-                                                                         const uint16_t* V, int layers) {
-    __shared__ int s_slot[META_THREADS], s_c[META_THREADS][3];
+// and stores their rows, a thread per (token, 8 pairs) and row of [layer][kv head].  The rows are asked for before the
+// metadata, which they have nothing to do with.
+constexpr long long APPEND_WRITE_ELEMENTS = 4096;      // of the appended keys (svlm_append_in_one)
+constexpr int APPEND_WRITE_THREADS = APPEND_WRITE_ELEMENTS / 16, APPEND_WRITE_TOKENS = APPEND_WRITE_ELEMENTS / 64;   // (heads have 64 dims at least)
+__global__ void __launch_bounds__(APPEND_WRITE_THREADS) append_meta_write_kernel(SvlmCacheDev cd, const unsigned char* types, const int* pos, int n, const uint16_t* K,
+                                                                                 const uint16_t* V, int layers) {
+    __shared__ int s_slot[APPEND_WRITE_TOKENS], s_c[APPEND_WRITE_TOKENS][3];
     svlm_ptx::pdl_wait();
     svlm_ptx::pdl_launch_dependents();
     const int half = cd.head_dim / 2, gshift = cd.head_dim == 128 ? 3 : 2, d = cd.head_dim, rows = layers * cd.kv_heads;
-    const int items = (n * rows) << gshift;           // (small: APPEND_WRITE_ELEMENTS)
+    const int tid = threadIdx.x, token = (tid >> gshift) / rows, row = (tid >> gshift) % rows, g = tid & ((1 << gshift) - 1);
+    const bool writes = token < n;
     Bf16x8 lo, hi;
     uint4 vlo, vhi;
-    auto row_of = [&](int i) { return (i >> gshift) % rows; };                   // the same token's rows lie together in a layer
-    auto token_of = [&](int i) { return (i >> gshift) / rows; };
-    auto load = [&](int i) {
-        const int r = row_of(i), l = r / cd.kv_heads, h = r - l * cd.kv_heads;
-        const size_t src = (((size_t)l * n + token_of(i)) * cd.kv_heads + h) * d + (i & ((1 << gshift) - 1)) * 8;
+    if (writes) {
+        const int l = row / cd.kv_heads, h = row - l * cd.kv_heads;
+        const size_t src = (((size_t)l * n + token) * cd.kv_heads + h) * d + g * 8;
         lo = bf16x8(svlm_ptx::ld_in(reinterpret_cast<const uint4*>(K + src)));
         hi = bf16x8(svlm_ptx::ld_in(reinterpret_cast<const uint4*>(K + src + half)));
         vlo = svlm_ptx::ld_in(reinterpret_cast<const uint4*>(V + src));
         vhi = svlm_ptx::ld_in(reinterpret_cast<const uint4*>(V + src + half));
-    };
-    const int tid = threadIdx.x;
-    if (tid < items) load(tid);
+    }
     const bool ok = append_few_body(cd, types, pos, n, [&](int slot, const int (&c)[3]) {
         s_slot[tid] = slot;
         for (int k = 0; k < 3; ++k) s_c[tid][k] = c[k];
     });
     if (!ok) return;
     __syncthreads();
-    for (int i = tid; i < items; i += blockDim.x) {
-        if (i != tid) load(i);
-        const int token = token_of(i), g = i & ((1 << gshift) - 1);
-        const int c[3] = {s_c[token][0], s_c[token][1], s_c[token][2]};
-        float cs[8], sn[8];
-        first_rotation(cd, g, c, cs, sn);
-        rotate8(lo, hi, cs, sn);
-        const size_t dst = ((size_t)row_of(i) * cd.n_slots + s_slot[token]) * d + g * 8;
-        *reinterpret_cast<Bf16x8*>(cd.K + dst) = lo;
-        *reinterpret_cast<Bf16x8*>(cd.K + dst + half) = hi;
-        *reinterpret_cast<uint4*>(cd.V + dst) = vlo;
-        *reinterpret_cast<uint4*>(cd.V + dst + half) = vhi;
-    }
+    if (!writes) return;
+    const int c[3] = {s_c[token][0], s_c[token][1], s_c[token][2]};
+    float cs[8], sn[8];
+    first_rotation(cd, g, c, cs, sn);
+    rotate8(lo, hi, cs, sn);
+    const size_t dst = ((size_t)row * cd.n_slots + s_slot[token]) * d + g * 8;
+    *reinterpret_cast<Bf16x8*>(cd.K + dst) = lo;
+    *reinterpret_cast<Bf16x8*>(cd.K + dst + half) = hi;
+    *reinterpret_cast<uint4*>(cd.V + dst) = vlo;
+    *reinterpret_cast<uint4*>(cd.V + dst + half) = vhi;
 }
 
 template <bool ROTATE>
@@ -823,7 +819,6 @@ cudaError_t svlm_launch_append_meta_batch(const SvlmCacheList& list, const SvlmC
 // same launch 14.3, in a second one 15.3, 4 K 15.5 and 16.3, 8 K 17.4 and 16.6, 32 K 25.2 and 17.4; 8 K elements of kept keys
 // re-rotated in the same launch 15.2, in a second one 16.6, 17 K 17.5 and 17.3 (one head) or 14.9 and 15.8 (two of 128), 155 K
 // 32.9 and 17.7.  (By plain calls a launch less saves the host 2 us more.)
-constexpr long long APPEND_WRITE_ELEMENTS = 4096;      // of the appended keys
 constexpr long long EVICT_ROTATE_ELEMENTS = 16384;     // of the keys that the windows keep
 // An eviction in one launch also walks over the tokens that leave, with 256 threads where the other form has 1024.  Append and
 // eviction of n tokens over 190 kept, one head of 64, vision, text and both in turn, us in one launch and in two: 700 20.6,
@@ -832,7 +827,7 @@ constexpr long long EVICT_ROTATE_ELEMENTS = 16384;     // of the keys that the w
 constexpr long long EVICT_ROTATE_LEAVING = 1024;
 static_assert(EVICT_ROTATE_ELEMENTS / 64 <= ROTATE_THREADS, "a thread per retained token (heads have 64 dims at least)");
 bool svlm_append_in_one(const SvlmCacheDev& cd, int layer, int n) {
-    return n <= META_THREADS && (long long)n * (layer < 0 ? cd.layers : 1) * cd.kv_heads * cd.head_dim <= APPEND_WRITE_ELEMENTS;
+    return (long long)n * (layer < 0 ? cd.layers : 1) * cd.kv_heads * cd.head_dim <= APPEND_WRITE_ELEMENTS;
 }
 bool svlm_evict_in_one(const SvlmCacheDev& cd, long long stored) {
     const long long windows = (long long)cd.n_sink + cd.vision_window + cd.text_window, kept = std::min(windows, (long long)cd.n_slots);
@@ -841,7 +836,7 @@ bool svlm_evict_in_one(const SvlmCacheDev& cd, long long stored) {
 
 cudaError_t svlm_launch_append_in_one(const SvlmCacheDev& cd, int layer, const void* K, const void* V, const unsigned char* types, const int* pos, int n, cudaStream_t st) {
     const int layers = layer < 0 ? cd.layers : 1, items = n * layers * cd.kv_heads * (cd.head_dim / 16);
-    const int threads = std::min(META_THREADS, std::max(append_threads(APPEND_FEW, n), (items + 31) / 32 * 32));
+    const int threads = std::max(append_threads(APPEND_FEW, n), (items + 31) / 32 * 32);
     return svlm_launch_chained(append_meta_write_kernel, dim3(1), dim3(threads), 0, 1, st, cd, types, pos, n, static_cast<const uint16_t*>(K),
                                static_cast<const uint16_t*>(V), layers);
 }

@@ -108,6 +108,33 @@ def test_cut_units_without_waiting(d, hq, hk, frames, vw):
     assert_close(s._stats(dev_to_f64(out)[rows], want))
 
 
+def test_cut_units_of_two_streams_at_once():
+    """Two caches on two streams: pieces of one launch wait for others whose thread blocks the other launch keeps from running.
+    The same bits as one after the other."""
+    from paper_2510_09608_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    normal = lambda *shape: torch.randn(*shape, generator=gen, device="cuda", dtype=torch.bfloat16)      # noqa: E731
+    made = []
+    for hq, hk, n_q, kept in ((16, 2, 390, 8000), (28, 4, 133, 4500)):
+        c = binding.Cache(2, hk, 128, 64, kept, 100, kept + 300)
+        c.append(-1, normal(2, kept, hk, 128), normal(2, kept, hk, 128), torch.ones(kept, dtype=torch.uint8, device="cuda"),
+                 torch.arange(kept, dtype=torch.int32, device="cuda"))
+        q, pos = normal(2, n_q, hq, 128), torch.arange(kept - n_q, kept, dtype=torch.int32, device="cuda")
+        want = [c.attend(l, q[l], pos) for l in range(2)]
+        torch.cuda.synchronize()
+        c.set_stream(torch.cuda.Stream())
+        made.append((c, q, pos, want, [torch.empty_like(q) for _ in range(6)]))
+    torch.cuda.synchronize()
+    for rep in range(6):
+        for l in range(2):
+            for c, q, pos, _, outs in made:
+                c.attend(l, q[l], pos, outs[rep][l])
+    torch.cuda.synchronize()
+    for c, _, _, want, outs in made:
+        assert c.status() == binding.OK
+        assert all(torch.equal(out[l], want[l]) for out in outs for l in range(2))
+
+
 # --- append metadata: one token, up to 1024 (one per thread), more; sinks of either rule that end inside a chunk; evictions
 # --- of more tokens than fit the lists in shared memory
 @pytest.mark.parametrize("sink_any", [False, True])
@@ -152,6 +179,110 @@ def test_small_caches_in_one_launch(d, hk, layers, sizes, capacity, base, contig
             s.check_metadata()
             for layer in range(layers):
                 s.check_kv(layer)
+
+
+# --- one launch each, what the shapes above leave out: more tokens of one ring leaving than the block has threads, three position
+# --- axes that differ, positions beyond 2^16, an append that does not fit
+@pytest.mark.parametrize("d,hk,vision,leaving", [(64, 1, True, 300), (64, 1, False, 600), (128, 1, True, 257), (64, 2, False, 1000)])
+def test_small_caches_evict_more_than_they_keep(d, hk, vision, leaving):
+    from harness import SideBySide
+    wl = _wl(2, layers=1, q_heads=hk, kv_heads=hk, head_dim=d, rope_mode=0, sections=(d // 2, 0, 0), n_sink=4, vision_window=60, text_window=50)
+    s = SideBySide(wl, capacity=leaving + 400)
+    rng = np.random.default_rng(leaving)
+    gid = 0
+    for n, types in ((150, rng.integers(0, 2, 150)), (leaving, np.full(leaving, int(vision))), (40, rng.integers(0, 2, 40)), (leaving, np.full(leaving, int(vision)))):
+        s._append(np.arange(gid, gid + n), types.astype(np.uint8), (gid + np.arange(n)).astype(np.int32))
+        gid += n
+        s.evict()
+        s.check_metadata()
+        s.check_kv(0)
+
+
+@pytest.mark.parametrize("d,hk,layers,base", [(64, 1, 1, 0), (64, 2, 2, 0), (128, 1, 1, 70000)])
+def test_small_appends_of_three_axes_and_beyond_capacity(d, hk, layers, base):
+    from harness import SideBySide
+    from paper_2510_09608_b200 import binding
+    wl = _wl(2, layers=layers, q_heads=hk, kv_heads=hk, head_dim=d, rope_mode=1, sections=(d // 8, d // 16 * 3, d // 16 * 3), n_sink=6, vision_window=34, text_window=20)
+    s = SideBySide(wl, capacity=90)
+    rng = np.random.default_rng(d)
+    gid, top = 0, base
+    for n in (13, 16, 1, 11, 15, 16):
+        types = rng.integers(0, 2, n).astype(np.uint8)
+        pos = (top + rng.integers(0, 30, (n, 3))).astype(np.int32)          # three axes that differ, not in order
+        s._append(np.arange(gid, gid + n), types, pos)
+        gid, top = gid + n, top + 30
+        s.check_metadata()
+        s.evict()
+        s.check_metadata()
+        for layer in range(layers):
+            s.check_kv(layer)
+    kept = s.ref.count()
+    for n in (16, 16):                                                       # the second one does not fit
+        pos = np.repeat((top + np.arange(n, dtype=np.int32))[:, None], 3, axis=1)
+        if kept + n <= 90:
+            s._append(np.arange(gid, gid + n), np.ones(n, np.uint8), pos)
+            gid, top, kept = gid + n, top + n, kept + n
+    before = (s.cache.query(), [s.cache.read_kv(l, kept) for l in range(layers)])
+    k = torch.ones(layers, 90 - kept + 1, hk, d, dtype=torch.bfloat16, device="cuda")
+    n = k.shape[1]
+    assert n * layers * hk * d <= 4096                                       # one launch places and writes
+    s.cache.append(-1, k, k, torch.ones(n, dtype=torch.uint8, device="cuda"), torch.full((n, 3), top, dtype=torch.int32, device="cuda"))
+    after = (s.cache.query(), [s.cache.read_kv(l, kept) for l in range(layers)])
+    assert s.cache.status() == binding.ERR_CAPACITY
+    assert all(np.array_equal(before[0][key], after[0][key]) for key in ("gids", "pos", "types")) and before[0]["shift_total"] == after[0]["shift_total"]
+    assert all(np.array_equal(x, y) for a, b in zip(before[1], after[1]) for x, y in zip(a, b))
+
+
+def test_small_caches_evict_together():
+    """One launch for caches of different windows, one of them with native positions (its keys stay as they are), with more
+    leaving one of them than the block has threads."""
+    from harness import SideBySide
+    from paper_2510_09608_b200 import binding
+    windows, natives = [(40, 30), (90, 12), (7, 100)], [False, True, False]
+    sides = []
+    for i, ((vw, tw), native) in enumerate(zip(windows, natives)):
+        wl = _wl(2, layers=1, q_heads=1, kv_heads=1, head_dim=64, rope_mode=0, sections=(32, 0, 0), n_sink=5, vision_window=vw, text_window=tw)
+        sides.append(SideBySide(wl, stream=i, capacity=640, contiguous=not native))
+    rng = np.random.default_rng(3)
+    at = [0] * 3
+    for rep, sizes in enumerate([(60, 90, 20), (30, 400, 300), (10, 20, 500), (64, 1, 64)]):
+        for i, (s, n) in enumerate(zip(sides, sizes)):
+            types = np.ones(n, np.uint8) if n >= 400 else rng.integers(0, 2, n).astype(np.uint8)
+            s._append(np.arange(at[i], at[i] + n), types, (at[i] + np.arange(n)).astype(np.int32))
+            at[i] += n
+        launches = binding.launch_count()
+        binding.evict_batched([s.cache for s in sides])
+        assert binding.launch_count() == launches + 1
+        for s in sides:
+            s.rot.evict(s.ref)
+            s.check_metadata()
+            s.check_kv(0)
+
+
+def test_a_captured_small_eviction_replayed_with_more_to_evict():
+    """The route was chosen when the graph was captured; what leaves when it is replayed is more than fits the lists in shared memory."""
+    from harness import SideBySide
+    wl = _wl(2, layers=1, q_heads=1, kv_heads=1, head_dim=64, rope_mode=0, sections=(32, 0, 0), n_sink=5, vision_window=90, text_window=60)
+    s = SideBySide(wl, capacity=3600)
+    rng = np.random.default_rng(9)
+    s._append(np.arange(200), rng.integers(0, 2, 200).astype(np.uint8), np.arange(200, dtype=np.int32))
+    s.evict()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        s.cache.set_stream(torch.cuda.current_stream())
+        s.cache.evict()
+    s.cache.set_stream(torch.cuda.current_stream())
+    gid = 200
+    for n in (30, 3000, 40, 2500):
+        s._append(np.arange(gid, gid + n), rng.integers(0, 2, n).astype(np.uint8), (gid + np.arange(n)).astype(np.int32))
+        gid += n
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        s.rot.evict(s.ref)
+        s.check_metadata()
+        s.check_kv(0)
 
 
 # --- decode: one to three units per warp, a second round, the step to the streaming kernel; one, two and three caches

@@ -107,6 +107,48 @@ assert append(c, 40) == OK and steps() == OK and lib.svlm_cache_evict(c) == OK
 """)
 
 
+def test_a_failed_launch_of_a_call_that_is_one_launch_ends_it(host):
+    """Steps that append by themselves (one cache by either decode kernel, a batch), appends and evictions of small caches: the host's
+    counts are what they were, nothing else is launched, and the next call does what it would have done."""
+    host("""
+def fails(kernel, calls, caches, n):
+    fake.fake_fail(kernel)
+    for call in calls:
+        ran()
+        assert call() == CUDA and ran() == [] and fake.cudaGetLastError() == 0, kernel
+        fake.fake_fail(b"")
+        for c in caches:
+            assert attend(c, n + 1, hq=8) == ORDER and attend(c, n, hq=8) == OK      # n tokens so far
+        fake.fake_fail(kernel)
+    fake.fake_fail(b"")
+near = new(hk=8)                                          # one layer: the per-layer kernel, over more keys the streaming one
+far = new(hk=8, vw=26000, tw=100, capacity=26300)
+four = [new(hk=8) for _ in range(4)]
+for c in [near, far] + four:
+    assert append(c, 40) == OK
+for _ in range(20):
+    assert append(far, 1300) == OK
+batched = lambda cs: lib.svlm_decode_step_batched(arr(cs), len(cs), 0, vp(P), vp(P), vp(P), vp(P), vp(P), 8, vp(P))
+fails(b"decode_layer", [lambda: step(near, hq=8), lambda: step(near, hq=8, layer=-1), lambda: batched([near])], [near], 40)
+fails(b"decode_stream", [lambda: step(far, hq=8)], [far], 26040)
+fails(b"decode_stream", [lambda: batched(four)], four, 40)
+for call, name in ((lambda: step(near, hq=8), "decode_layer"), (lambda: step(far, hq=8), "decode_stream"), (lambda: batched(four), "decode_stream")):
+    ran()
+    assert call() == OK
+    got = ran()
+    assert len(got) == 1 and name in got[0], got
+assert attend(near, 42, hq=8) == ORDER and attend(near, 41, hq=8) == OK
+small = [new(hk=1, d=64, vw=120, tw=70, capacity=400) for _ in range(2)]
+for c in small:
+    ran()
+    assert append(c, 40) == OK
+    got = ran()
+    assert len(got) == 1 and "append_meta_write" in got[0], got
+fails(b"append_meta_write", [lambda: append(small[0], 40), lambda: append(small[0], 40, layer=-1)], small, 40)
+fails(b"evict_meta", [lambda: lib.svlm_cache_evict(small[0]), lambda: lib.svlm_cache_evict_batched(arr(small), 2)], small, 40)
+""")
+
+
 def test_a_captured_call_is_reckoned_with_full_windows(host):
     """A graph captured while the windows fill is replayed when they are full: the kernels are chosen for that, and so they are
     for plain calls of the same cache afterwards, whose appends the host may not have seen."""
