@@ -213,12 +213,12 @@ int svlm_attend_batched_varlen(svlm_cache* const* caches, int n_caches, int laye
  * the single-cache calls).  Same requirements on the caches as svlm_attend_batched; a cache may appear
  * only once.
  *
- * svlm_decode_step_batched = svlm_decode_step on every cache, one metadata launch (layer 0) and one
- * attention launch for all of them:
+ * svlm_decode_step_batched = svlm_decode_step on every cache, one attention launch for all of them, behind one metadata
+ * launch for layer 0 of caches with several layers:
  *   K, V        bf16 [n_caches][kv_heads][head_dim]      Q, out   bf16 [n_caches][q_heads][head_dim]
  *   token_type  uint8 [n_caches]      pos   int32 [n_caches] or [n_caches][3]
  * svlm_cache_evict_batched = svlm_cache_evict on every cache, one metadata launch and one re-rotation
- * launch for all of them.
+ * launch for all of them (small caches: one launch that does both).
  * Errors: as the single-cache calls; SVLM_ERR_ARG also for mismatched or repeated caches.
  */
 int svlm_decode_step_batched(svlm_cache* const* caches, int n_caches, int layer, const void* K, const void* V,
@@ -240,7 +240,7 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
 /*
  * svlm_decode_step with host buffers (layer -1: all layers of the token in one launch); returns with out_host
  * filled.  The step's inputs are a few KB: they are gathered in a page-locked buffer of the library and go up in
- * one copy.  For layer -1, when every buffer is itself page-locked and mapped (as pinned allocations are under
+ * one copy.  For layer -1 of a cache with several layers, when every buffer is itself page-locked and mapped (as pinned allocations are under
  * unified addressing) and 16-byte aligned, nothing is copied at all: the kernels read the inputs and write the
  * output where they are.
  */

@@ -27,6 +27,7 @@
 //                 now each issuer's waits run while the other one's MMAs execute
 //   3490 -> 2700  P handed over through named barriers instead of mbarriers (450 -> 50 cycles), in two halves, so that
 //                 the first half's P V runs under the second half's exponentials
+//   2700 -> 3200  all exponentials on the special-function unit (softmax_page), which costs less where power is the limit
 //   softmax of a page 2200 -> 1500 cycles: the whole row in registers (one pass over TMEM), packed fp32 pairs
 // Per-page bookkeeping that cost a masked page 2 us (descriptor loads, two barriers and a bisection through shared
 // memory) is now a few shuffles on values that arrive while the thread waits for S.
@@ -575,6 +576,12 @@ __device__ __forceinline__ void publish_columns(const PfPlan& plan, int tail, in
 // first word for the next launch.  Returns the blocks this CTA has to merge.
 // Where nobody shares, the last one merges all, and keeps its piece in TMEM if the others are there already (last: the CTA's last
 // segment, whose piece may stay there).
+// Why wait, and how long: us per layer with its append, 28/4 heads of 128 over 9200 keys, 64 polls, 32, 16, 8 and (attention
+// alone) none against 64: 69 tokens 48.6, 48.6, 53.9, 58.0 (46 and 38), 266 tokens 63.7, 63.9, 65.5, 67.1; over 43 shapes 1.059, 1.049,
+// 1.015 and 1.001 times the speed of the last one merging by itself.  A block that waits keeps its SM from other streams: two
+// equal streams' attention calls, nothing between them, run at 0.83-0.98 of that speed (0.91-0.96 with 8 polls), whole
+// chunks of two streams at 0.93-1.03, unequal streams at 1.00-1.09, beside matrix products 0.97-1.00.  Waiting only for pieces
+// that have been begun, or whose blocks started together, made no difference to any of these.
 constexpr int PF_MEET_POLLS = 14;         // polls: the control block's limit >> this (64 by default, some 40 us)
 template <int D>
 __device__ __forceinline__ unsigned meet_pieces(PfShared& sh, const PfPlan& plan, int tail, const PfCut& cut, int g, int m, unsigned tO, float m_row, float l,
