@@ -14,21 +14,29 @@
 //
 // Roles (384 threads, registers moved from warpgroup 2 to the softmax with setmaxnreg):
 //   warps 0-3, 4-7   softmax of tile A, B, one thread per row; also that tile's query rotation and output
-//   warp 8           TMA: K and V pages (128 slots, 128-byte swizzle) into one 4-stage ring, K(0) V(0) K(1) ...; it
+//   warp 8           TMA: K and V pages (128 slots, 128-byte swizzle) into one 4-stage ring, K(0) K(1) V(0) K(2) V(1) ...; it
 //                    runs ahead into the next unit while the current one ends
 //   warps 9, 10      issue tcgen05.mma for tile A, B: S = Q K^T into 128 TMEM columns, O += P V with P read from
-//                    TMEM (P is written over the first 64 columns of S: no shared-memory round trip)
-//   warp 11          nothing (setmaxnreg works on whole warpgroups)
-// What bounds the page loop is each tile's serial chain S -> softmax -> P V -> next S beside the tensor time of both
-// tiles (2048 cycles per page pair).  Measured on it (cycles per page pair, head_dim 128, clock read in an instrumented copy):
-//   3750 -> 3490  two issuers with the turn handed on through a named barrier: a wait on an mbarrier costs ~300 cycles
-//                 even when it is already complete (the shared-memory pipe is saturated by the operand reads), and the
-//                 tensor queue is only ~2 MMAs deep, so a single issuer idled the pipe for four such waits per pair;
-//                 now each issuer's waits run while the other one's MMAs execute
+//                    TMEM (no shared-memory round trip), and say to the softmax that P V is done
+//   warp 11          says to the softmax that S is there
+// TMEM: O of both tiles (256 columns at head_dim 128), P of both (64 each, bf16), and one buffer of 128 for S that the tiles take
+// in turns: S(A,0) S(B,0) S(A,1) S(B,1) ...  A tile's scores stay there only until they are in its softmax warps' registers, then
+// the other tile's come, so S(j+1) of a tile is there before its P V(j) has begun and the softmax warps go from page to page
+// without a wait.  (Before, P lay over its own S, and each tile was the serial chain S -> softmax -> P V -> next S.)
+// Measured on the page loop (cycles per page pair, head_dim 128, clock read in an instrumented copy; tensor time is 2048 of them, and
+// the special-function unit's 2048):
+//   3750 -> 3490  two issuers, each one's waits under the other one's MMAs
 //   3490 -> 2700  P handed over through named barriers instead of mbarriers (450 -> 50 cycles), in two halves, so that
 //                 the first half's P V runs under the second half's exponentials
 //   2700 -> 3200  all exponentials on the special-function unit (softmax_page), which costs less where power is the limit
-//   softmax of a page 2200 -> 1500 cycles: the whole row in registers (one pass over TMEM), packed fp32 pairs
+//   3240 -> 3850  one buffer for S, but waits of one lane and shuffles in warps 9-11: each such step of theirs takes 300 to 700 cycles beside
+//                 the softmax warps, whose exponentials, loads, shuffles and mbarrier operations go through the same queue
+//                 (softmax warps waiting on the mbarriers themselves: 3200, of which 300 each for two waits that were complete)
+//   3850 -> 2750  these waits as short loops of the whole warp (mbar_wait_short); -> 2600 by giving the columns away before the
+//                 maximum, and with one form of the softmax for all pages
+//   softmax of a page 2200 -> 1500 cycles for a warp by itself: the whole row in registers (one pass over TMEM), packed fp32 pairs
+// With P over its own S -> now (28/4 heads of 128): 531 tokens over 31,000 keys with append and eviction 241 -> 220 us, eight layers of a
+// second of video in a burst 690 -> 618; at the power limit all 28 layers 2471 -> 2312, four layers of 4133 tokens 1724 -> 1599.
 // Per-page bookkeeping that cost a masked page 2 us (descriptor loads, two barriers and a bisection through shared
 // memory) is now a few shuffles on values that arrive while the thread waits for S.
 // Every mbarrier wait is bounded: on expiry the CTA records SVLM_ERR_TIMEOUT in the caches' status words, keeps up its
@@ -73,10 +81,11 @@ __device__ __forceinline__ float ex2(float x) { float y; asm("ex2.approx.ftz.f32
 
 // ---- named barriers (the hardware's, not shared memory): ids ----------------------------------------------------
 constexpr int BAR_WG = 1;      // + tile: the softmax warpgroup alone (128)
-constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM and it is this tile's turn (128 softmax + 32 other issuer + 32 issuer)
+constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM (128 softmax + 32 issuer)
 constexpr int BAR_P2 = 5;      // + tile: second half of P (128 + 32)
-constexpr int BAR_TURN_B = 7;  // first S of tile B in a unit (32 + 32)
-constexpr int BAR_TURN_A = 8;  // first S of tile A in a unit after the first
+constexpr int BAR_READ = 7;    // + tile: its S is in registers, the columns are free (128 + 32 issuer of the S that comes there next)
+constexpr int BAR_S = 11;      // + tile: S is in TMEM (128 + 32 warp 11)
+constexpr int BAR_PV = 13;     // + tile: P V is done: its P may be overwritten, its accumulator touched (128 + 32 issuer)
 constexpr int BAR_Q = 9;       // + tile: the tile's query rows are in shared memory, its accumulator is free (128 + 32)
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
@@ -93,73 +102,6 @@ __device__ __forceinline__ void rescale_o(unsigned tO, int D, float corr) {
         for (int k = 0; k < 8; ++k) o[k] *= corr;
         tmem_st8(tO + q, o);
     }
-}
-
-// One page of one row: S (128 fp32 columns at tS, this thread's TMEM lane) -> P (bf16 pairs in the first 64
-// columns of the same buffer), with a lazily moving reference maximum (O is rescaled only when the maximum grows by
-// more than 2^8).  The whole row is loaded once; the first half's maximum is taken while the second half is on its
-// way.  P goes out in chunks of 32 keys; once the exponentials of the third chunk are done, the first two chunks are
-// certainly stored and are handed to the issuer (BAR_P1).  On MASKED pages the row sees the columns [vlo, vlo + vlen).
-// All exponentials on the special-function unit, although it then has as many cycles of work as the tensor pipe: a polynomial
-// on the FMA pipe for a quarter of them made a cold launch 5 % faster, but a chunk of many layers runs at the power limit,
-// where its instructions cost clock (28 layers 2580 -> 2535 us, four layers of a long chunk 1740 -> 1718, one layer 105.0).
-template <bool MASKED>
-__device__ __forceinline__ void softmax_page(int g, unsigned tS, unsigned tO, int D, unsigned vlo, unsigned vlen, float c,
-                                             float m_ref, bool have_o, float& rowsum, float& corr, float& m_new) {
-    auto visible = [&](int k) { return (unsigned)k - vlo < vlen; };
-    float s[128];
-    tmem_ld32(tS, s);
-    tmem_ld32(tS + 32, s + 32);
-    tmem_wait_ld<64>(s);
-    tmem_ld32(tS + 64, s + 64);
-    tmem_ld32(tS + 96, s + 96);
-    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (MASKED) {
-#pragma unroll
-            for (int k = 64 * h; k < 64 * h + 64; ++k) s[k] = visible(k) ? s[k] : -INFINITY;
-        }
-#pragma unroll
-        for (int k = 64 * h; k < 64 * h + 64; k += 2) mx[(k >> 1) & 3] = max3(mx[(k >> 1) & 3], s[k], s[k + 1]);
-        if (h == 0) tmem_wait_ld<64>(s + 64);
-    }
-    const float mx_row = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]) * c;
-    const bool grow = mx_row > m_ref + 8.f;
-    m_new = grow ? mx_row : m_ref;
-    const float m_use = m_new == -INFINITY ? 0.f : m_new;
-    corr = 1.f;
-    if (__any_sync(0xffffffffu, grow)) {
-        corr = grow ? exp2f(m_ref - m_use) : 1.f;   // m_ref = -inf gives 0
-        if (have_o) rescale_o(tO, D, corr);         // S of this page was issued after P V of the previous one: O is quiescent
-    }
-    const u64 c2 = pk64(c, c), nm2 = pk64(-m_use, -m_use);
-    u64 sum[2] = {0ull, 0ull};
-#pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-        unsigned pk[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int k = ch * 32 + 2 * i;
-            const u64 t = fma2(pk64(s[k], s[k + 1]), c2, nm2);
-            float e0, e1;
-            un64(t, e0, e1);
-            e0 = ex2(e0);
-            e1 = ex2(e1);
-            sum[i & 1] = add2(sum[i & 1], pk64(e0, e1));
-            pk[i] = pack2(e0, e1);
-        }
-        if (ch == 2) {
-            tmem_wait_st();
-            tc_fence_before();
-            bar_arrive(BAR_P1 + g, 192);
-        }
-        tmem_st16(tS + ch * 16, pk);
-    }
-    float a0, a1, b0, b1;
-    un64(sum[0], a0, a1);
-    un64(sum[1], b0, b1);
-    rowsum = (a0 + a1) + (b0 + b1);
 }
 
 // n / G with magic = ceil(2^32 / G), which is exact for n < 2^32 / G; magic = 0: the launch has other numbers.
@@ -290,9 +232,10 @@ struct PfGroup {
 
 struct PfShared {            // control part of shared memory, behind the tiles
     unsigned long long full[PF_RING], empty[PF_RING];
-    unsigned long long s_full[2], all_done[2];
+    unsigned long long s_full[2], pv_done[2];
     unsigned tmem_base;
     int abort_flag;
+    unsigned asked[2];                     // products S that the tile's issuer has come past
     unsigned take[2];                      // per tile: blocks of columns of a cut unit that this CTA has to merge
     int leave[2];                          // its own ones are left to whoever comes last
     PfCut cut[2];                          // of the CTA's last segment, of its first one
@@ -300,11 +243,110 @@ struct PfShared {            // control part of shared memory, behind the tiles
 };
 static_assert(sizeof(PfShared) <= 3072, "control block must fit behind the tiles");
 
+// The columns of tensor memory (see the top).  Taking turns with one buffer of scores also keeps the two tiles half a page apart:
+// with one each, which fit at head_dim 64, both do their exponentials at the same time, then neither (12/2 heads of 64, 4133
+// tokens over 9200 keys 161 -> 177 us).
+template <int D>
+struct PfColumns {
+    static constexpr unsigned S = 0;
+    __device__ __forceinline__ static unsigned P(int g) { return 128 + g * 64; }
+    __device__ __forceinline__ static unsigned O(int g) { return 256 + g * D; }
+};
+struct PfTmem { unsigned S, P, O; };      // of this thread's row
+
+// One page of one row: S (128 fp32 columns, this thread's TMEM lane) -> P (64 columns of bf16 pairs), with a lazily
+// moving reference maximum (O is rescaled only when the maximum grows by more than 2^8).  The whole row is loaded once
+// and its columns given away (BAR_READ); the first half's maximum is taken while the second half is on its way.  Before
+// P or O is touched, P V of the previous page has to be through (BAR_PV; it usually is, by then).  P goes out in chunks of 32 keys; once the exponentials of the third chunk are done, the first two chunks are
+// certainly stored and are handed to the issuer (BAR_P1).  Of the blocks of 32 columns in mixed, the row sees those in
+// [vlo, vlo + vlen): the blocks at the edge of what is visible, usually one or two (a second instance of this function for such
+// pages, every column compared, had 28/4 heads, 2600 tokens over 2500 keys at 108 us a layer, this way it is 88; and it cost the
+// other pages 2 %).
+// All exponentials on the special-function unit, although it then has as many cycles of work as the tensor pipe: a polynomial
+// on the FMA pipe for a quarter of them made a cold launch 5 % faster, but a chunk of many layers runs at the power limit,
+// where its instructions cost clock (28 layers 2580 -> 2535 us, four layers of a long chunk 1740 -> 1718, one layer 105.0).
+template <int D>
+__device__ __forceinline__ void softmax_page(int g, const PfTmem& t, unsigned mixed, unsigned vlo, unsigned vlen, bool have_o, float& m_ref, float& l) {
+    constexpr float c = D == 128 ? 0.12751743082459868f : 0.18033688011112042f;      // log2(e) / sqrt(D)
+    auto visible = [&](int k) { return (unsigned)k - vlo < vlen; };
+    float s[128];
+    tmem_ld32(t.S, s);
+    tmem_ld32(t.S + 32, s + 32);
+    tmem_ld32(t.S + 64, s + 64);
+    tmem_ld32(t.S + 96, s + 96);
+    tmem_wait_ld<128>(s);
+    tc_fence_before();
+    bar_arrive(BAR_READ + g, 160);
+    if (mixed) {
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch)
+            if ((mixed >> ch) & 1) {
+#pragma unroll
+                for (int k = 32 * ch; k < 32 * ch + 32; ++k) s[k] = visible(k) ? s[k] : -INFINITY;
+            }
+    }
+    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int k = 0; k < 128; k += 2) mx[(k >> 1) & 3] = max3(mx[(k >> 1) & 3], s[k], s[k + 1]);
+    const float mx_row = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]) * c;
+    const bool grow = mx_row > m_ref + 8.f;
+    const float m_new = grow ? mx_row : m_ref;
+    const float m_use = m_new == -INFINITY ? 0.f : m_new;
+    float corr = 1.f;
+    bool wait_pv = have_o;
+    if (__any_sync(0xffffffffu, grow)) {
+        corr = grow ? exp2f(m_ref - m_use) : 1.f;   // m_ref = -inf gives 0
+        if (have_o) {
+            bar_sync(BAR_PV + g, 160);
+            tc_fence_after();
+            rescale_o(t.O, D, corr);
+            wait_pv = false;
+        }
+    }
+    const u64 c2 = pk64(c, c), nm2 = pk64(-m_use, -m_use);
+    u64 sum[2] = {0ull, 0ull};
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) {
+        unsigned pk[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int k = ch * 32 + 2 * i;
+            const u64 x = fma2(pk64(s[k], s[k + 1]), c2, nm2);
+            float e0, e1;
+            un64(x, e0, e1);
+            e0 = ex2(e0);
+            e1 = ex2(e1);
+            sum[i & 1] = add2(sum[i & 1], pk64(e0, e1));
+            pk[i] = pack2(e0, e1);
+        }
+        if (ch == 0 && wait_pv) {
+            bar_sync(BAR_PV + g, 160);
+            tc_fence_after();
+        }
+        if (ch == 2) {
+            tmem_wait_st();
+            tc_fence_before();
+            bar_arrive(BAR_P1 + g, 160);
+        }
+        tmem_st16(t.P + ch * 16, pk);
+    }
+    float a0, a1, b0, b1;
+    un64(sum[0], a0, a1);
+    un64(sum[1], b0, b1);
+    l = l * corr + ((a0 + a1) + (b0 + b1));
+    m_ref = m_new;
+    tmem_wait_st();
+    tc_fence_before();
+    bar_arrive(BAR_P2 + g, 160);
+}
+
+
 // A warp's walk over the pages of a segment, 32 tiles of the cache's page list at a time, one per lane.
 struct PfPages {
     int base, seen;
-    unsigned left, info;     // pages of the window still to come; per lane: page | lo << 14 | (hi - 1) << 21 | masked << 28 | causal << 29
-    __device__ __forceinline__ void begin() { base = 0; seen = 0; left = 0; info = 0; }
+    unsigned left, info;     // pages of the window still to come; per lane: page | lo << 14 | (hi - 1) << 21 | masked << 28 | causal << 29 | no gaps << 30
+    int first, at;           // per lane: ordinal of slot lo, relative to the first query token; lane of the latest page
+    __device__ __forceinline__ void begin() { base = 0; seen = 0; left = 0; info = 0; first = 0; at = 0; }
     // r_lo: rows from this token on are served; a page all of them see in full needs no mask
     __device__ __forceinline__ unsigned next(const PfWork& w, int r_lo) {
         const int lane = threadIdx.x & 31;
@@ -317,7 +359,9 @@ struct PfPages {
                 const longlong2 g = ld_l2(reinterpret_cast<const longlong2*>(&tp->min_gid));
                 vis = g.x <= w.gid_hi;
                 const unsigned causal = g.y > w.gid_q0 + r_lo, ragged = a.y > 0 || a.z < SVLM_PAGE;
-                info = (unsigned)a.x | ((unsigned)a.y << 14) | ((unsigned)(a.z - 1) << 21) | ((causal | ragged) << 28) | (causal << 29);
+                info = (unsigned)a.x | ((unsigned)a.y << 14) | ((unsigned)(a.z - 1) << 21) | ((causal | ragged) << 28) | (causal << 29) |
+                       ((unsigned)(g.y - g.x == a.z - 1 - a.y) << 30);       // ordinals grow with the offset: then one after another
+                first = (int)max(g.x - w.gid_q0, -0x40000000ll);
             }
             const unsigned all = __ballot_sync(0xffffffffu, vis);
             const int rank = seen + __popc(all & ((1u << lane) - 1));
@@ -325,10 +369,11 @@ struct PfPages {
             seen += __popc(all);
             base += 32;
         }
-        const int at = left ? __ffs(left) - 1 : 0;
+        at = left ? __ffs(left) - 1 : 0;
         left &= left - 1;
         return __shfl_sync(0xffffffffu, info, at);
     }
+    __device__ __forceinline__ int first_here() const { return __shfl_sync(0xffffffffu, first, at); }
 };
 // Rotates one 128-row tile of queries at q_pos - shift_total, rounds to bf16 and stores it K-major swizzled.  Called by
 // the 128 threads of the tile's softmax warpgroup.  A work item is (row, 8 pairs): a 16-byte chunk of the row's low half
@@ -739,6 +784,7 @@ template <int D>
 __global__ void __launch_bounds__(PF_THREADS, 1)
 prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant__ PfPlan plan, int layer0, int n_layers,
                const uint16_t* Q, const int* q_pos, int n_q_arg, int q_heads, uint16_t* __restrict__ out) {
+    using Col = PfColumns<D>;
     constexpr int KB = D / 64;                 // 64-element (128-byte) blocks along d
     constexpr int TILE_BYTES = 128 * D * 2;    // one K or V page of one head, or one 128-row Q tile
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -758,7 +804,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
     // ---- set-up: barriers, TMEM ------------------------------------------------------
     if (threadIdx.x == 0) {
         for (int s = 0; s < PF_RING; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 2); }   // both issuers release a page
-        for (int s = 0; s < 2; ++s) { mbar_init(&sh.s_full[s], 1); mbar_init(&sh.all_done[s], 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&sh.s_full[s], 1); mbar_init(&sh.pv_done[s], 1); sh.asked[s] = 0; }
         sh.abort_flag = 0;
         mbar_init_fence();
     }
@@ -784,7 +830,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         walk.begin(plan);
         bool ok = true;
         if (warp == 8) {
-            // ================= TMA producer: K(0) V(0) K(1) V(1) ... through one ring, unit after unit =================
+            // ================= TMA producer: K(0) K(1) V(0) K(2) V(1) ... V(n-1) through one ring, unit after unit =================
             unsigned item = 0;
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
@@ -794,32 +840,38 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 const void* tmV = reinterpret_cast<const unsigned char*>(w.vw->tmaps) + 128;
                 PfPages pages;
                 pages.begin();
-                for (int j = 0; j < w.n_proc && ok; ++j) {
-                    const int y = (int)(rows.head_row0 + (size_t)(pages.next(w, 0) & 0x3FFF) * SVLM_PAGE);
+                int y = 0, y_before = 0;
+                for (int j = 0; j <= w.n_proc && ok; ++j) {
+                    if (j < w.n_proc) y = (int)(rows.head_row0 + (size_t)(pages.next(w, 0) & 0x3FFF) * SVLM_PAGE);
                     if (lane == 0) {
 #pragma unroll
                         for (int kv = 0; kv < 2; ++kv) {
-                            const unsigned st = (item + kv) % PF_RING;
-                            if (ok) ok = mbar_wait(&sh.empty[st], (((item + kv) / PF_RING) & 1) ^ 1, abort_flag, w.wait_limit);   // first pass: already free
+                            if (kv ? j == 0 : j == w.n_proc) continue;
+                            const unsigned st = item % PF_RING;
+                            if (ok) ok = mbar_wait(&sh.empty[st], ((item / PF_RING) & 1) ^ 1, abort_flag, w.wait_limit);   // first pass: already free
                             if (!ok) break;
                             mbar_expect_tx(&sh.full[st], TILE_BYTES);
 #pragma unroll
                             for (int kb = 0; kb < KB; ++kb)
-                                tma_load_2d(ring + st * TILE_BYTES + kb * (128 * 128), kv ? tmV : tmK, kb * 64, y, &sh.full[st]);
+                                tma_load_2d(ring + st * TILE_BYTES + kb * (128 * 128), kv ? tmV : tmK, kb * 64, kv ? y_before : y, &sh.full[st]);
+                            ++item;
                         }
                     }
                     ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-                    item += 2;
+                    y_before = y;
                 }
                 if (!ok) break;
             }
         } else if (warp < 11) {
             // ================= MMA issuer of tile g =================
-            // Per tile the order is S(0) | PV(j) S(j+1) | ...: the tensor pipe executes one thread's instructions in
-            // order, so S(j+1) overwrites the columns of P(j) only after PV(j) has read them.  The whole warp runs the
-            // loop (waits, descriptor arithmetic: warp-uniform values the compiler can keep in uniform registers); one
-            // elected lane executes the tcgen05 instructions.  The number of named-barrier operations depends on the
-            // work list only, never on whether a wait has run out.
+            // Per tile the order is S(0) | S(j+1) PV(j) | ...  The whole warp runs the loop (waits, descriptor arithmetic:
+            // warp-uniform values the compiler can keep in uniform registers); one elected lane executes the tcgen05
+            // instructions.  The number of named-barrier operations depends on the work list only, never on whether a wait
+            // has run out, and so does their order: nobody arrives at a barrier again before the others have been there.
+            //   BAR_READ of B's page j-1 -> S of A's page j -> BAR_S -> BAR_READ of A's page j -> S of B's page j -> ...
+            //   BAR_P2 of a page -> its BAR_PV -> the next page's BAR_P1
+            // Without a working wait everybody goes on along these lines, the issuers without issuing anything, and warp 11
+            // follows them by their count of products (asked).
             const int g = warp - 9;
             const unsigned tmem = __shfl_sync(0xffffffffu, sh.tmem_base, 0);
             const bool leader = elect_one();
@@ -827,15 +879,12 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             constexpr unsigned IDESC_O = make_idesc(128, D, 1);
             // descriptors: the 14-bit start-address field counts 16-byte units, so moving inside a tile is an
             // addition to the low word (all tile addresses stay below the field's range: shared memory is 228 KB)
+            const unsigned tmem_s = tmem + Col::S, tmem_p = tmem + Col::P(g), tmem_o = tmem + Col::O(g);
             const unsigned long long dq = smem_desc(smem_u32(sQ + g * TILE_BYTES), 16, 1024);   // Q, K: K-major
             const unsigned long long dk = smem_desc(smem_u32(ring), 16, 1024);
             const unsigned long long dv = smem_desc(smem_u32(ring), 128 * 128, 1024);           // V: MN-major
             unsigned wait_limit = 0;
-            auto wait_item = [&](unsigned n) {                      // one lane polls, all lanes get the answer
-                int r = 1;
-                if (lane == 0) r = mbar_wait(&sh.full[n % PF_RING], (n / PF_RING) & 1, abort_flag, wait_limit);
-                return __shfl_sync(0xffffffffu, r, 0) != 0;
-            };
+            auto wait_item = [&](int n) { if (ok) ok = __all_sync(0xffffffffu, mbar_wait_short(&sh.full[n % PF_RING], (n / PF_RING) & 1, abort_flag, wait_limit)); };
             auto issue_S = [&](unsigned n) {                        // S = Q K^T, K is ring item n
                 const unsigned st = n % PF_RING;
                 const unsigned long long b0 = dk + (unsigned)(st * TILE_BYTES >> 4);
@@ -843,7 +892,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks) {
                         const unsigned off = ((ks / 4) * (128 * 128) + (ks % 4) * 32) >> 4;
-                        tc_mma_ss(tmem + g * 128, dq + off, b0 + off, IDESC_S, ks > 0);
+                        tc_mma_ss(tmem_s, dq + off, b0 + off, IDESC_S, ks > 0);
                     }
                     tc_commit(&sh.s_full[g]);
                     tc_commit(&sh.empty[st]);
@@ -857,60 +906,79 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {                   // 16 keys per MMA: A = 8 TMEM columns of bf16 pairs
                         const int ks = half * 4 + k;
-                        tc_mma_ts(tmem + 256 + g * 128, tmem + g * 128 + ks * 8, b0 + (unsigned)(ks * 2048 >> 4), IDESC_O, accumulate || k > 0);
+                        tc_mma_ts(tmem_o, tmem_p + ks * 8, b0 + (unsigned)(ks * 2048 >> 4), IDESC_O, accumulate || k > 0);
                     }
-                    if (half) tc_commit(&sh.empty[st]);
+                    if (half) { tc_commit(&sh.pv_done[g]); tc_commit(&sh.empty[st]); }
                 }
                 __syncwarp();
             };
-            unsigned item = 0;
-            bool first_unit = true;
+            int item = 0;
+            unsigned steps = 0, pvs = 0;
+            auto step_S = [&](unsigned n) {
+                // the order is A B A B ...: tile A's k-th S waits for B's k-1st to be read, tile B's for A's k-th
+                if (g == 1 || steps > 0) bar_sync(BAR_READ + (g ^ 1), 160);
+                if (ok) { tc_fence_after(); issue_S(n); }
+                ++steps;
+                if (lane == 0) *(volatile unsigned*)&sh.asked[g] = steps;
+            };
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
                 const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
                 const PfWork w = pf_work(b, seg, rows, plan.g_magic, G, pf_ask(b, rows));
-                const bool more = walk.more(plan);
                 wait_limit = w.wait_limit;
                 const int n = w.n_proc;
-                if (ok && n > 0) ok = wait_item(item);
+                // ring items: K(0) K(1) V(0) K(2) V(1) ... K(n-1) V(n-2) V(n-1)
+                auto k_of = [&](int j) { return j == 0 ? item : item + 2 * j - 1; };
+                auto v_of = [&](int j) { return j + 1 < n ? item + 2 * j + 2 : item + 2 * j + 1; };
+                if (n > 0) wait_item(item);
                 bar_sync(BAR_Q + g, 160);
-                if (g == 0) { if (!first_unit) bar_sync(BAR_TURN_A, 64); }
-                else bar_sync(BAR_TURN_B, 64);
-                if (ok && n > 0) { tc_fence_after(); issue_S(item); }
-                if (g == 0) bar_arrive(BAR_TURN_B, 64);
-                else if (n > 0) bar_arrive(BAR_P1, 192);
-                else if (more) bar_arrive(BAR_TURN_A, 64);
+                if (n > 0) step_S(item);
                 for (int j = 0; j < n; ++j) {
-                    if (ok) ok = wait_item(item + 2 * j + 1);                           // V(j)
-                    if (ok && j + 1 < n) ok = wait_item(item + 2 * j + 2);              // K(j+1)
-                    bar_sync(BAR_P1 + g, 192);
-                    if (ok) { tc_fence_after(); issue_PV(item + 2 * j + 1, 0, j > 0); }
+                    if (j + 1 < n) wait_item(k_of(j + 1));
+                    wait_item(v_of(j));
+                    if (j + 1 < n) step_S(k_of(j + 1));
+                    bar_sync(BAR_P1 + g, 160);
+                    if (ok) { tc_fence_after(); issue_PV(v_of(j), 0, j > 0); }
                     bar_sync(BAR_P2 + g, 160);
                     if (ok) {
                         tc_fence_after();
-                        issue_PV(item + 2 * j + 1, 1, true);
-                        if (j + 1 < n) issue_S(item + 2 * j + 2);
+                        issue_PV(v_of(j), 1, true);
+                        ok = __all_sync(0xffffffffu, mbar_wait_short(&sh.pv_done[g], pvs & 1, abort_flag, wait_limit));
+                        tc_fence_after();
+                        tc_fence_before();
                     }
-                    if (g == 0) bar_arrive(BAR_P1 + 1, 192);
-                    else if (j + 1 < n) bar_arrive(BAR_P1, 192);
-                    else if (more) bar_arrive(BAR_TURN_A, 64);
+                    bar_arrive(BAR_PV + g, 160);
+                    ++pvs;
                 }
-                if (leader && ok) {
-                    if (n > 0) tc_commit(&sh.all_done[g]);
-                    else mbar_arrive(&sh.all_done[g]);              // nothing was issued: nothing to track
-                }
-                __syncwarp();
                 item += 2 * n;
-                first_unit = false;
+            }
+            if (g == 0 && steps > 0) bar_sync(BAR_READ + 1, 160);           // tile B's last one, behind which none comes
+        } else {
+            // ================= warp 11: says to the softmax that S is there =================
+            // (A wait on an mbarrier costs a softmax warp ~300 cycles even when it is complete, a named barrier 40.)
+            unsigned steps = 0;
+            while (walk.more(plan)) {
+                const PfSeg seg = walk.next(plan);
+                const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
+                const PfWork w = pf_work(b, seg, rows, plan.g_magic, G, pf_ask(b, rows));
+                for (int j = 0; j < w.n_proc; ++j, ++steps)
+#pragma unroll
+                    for (int g = 0; g < 2; ++g) {
+                        if (ok) ok = __all_sync(0xffffffffu, mbar_wait_short(&sh.s_full[g], steps & 1, abort_flag, w.wait_limit));
+                        // after a wait that has run out the barriers keep their order all the same: not before the issuer has come past the product
+                        for (unsigned p = 0; !ok && p < (1u << 20) && (int)(*(volatile unsigned*)&sh.asked[g] - steps) <= 0; ++p) __nanosleep(64);
+                        tc_fence_after();
+                        tc_fence_before();
+                        bar_arrive(BAR_S + g, 160);
+                    }
             }
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
         // ================= softmax warpgroups: one thread per row of tile g =================
         const int g = warp >> 2, m = threadIdx.x & 127;
-        const unsigned tS = sh.tmem_base + g * 128 + ((unsigned)((warp & 3) * 32) << 16), tO = tS + 256;
-        constexpr float c = D == 128 ? 0.12751743082459868f : 0.18033688011112042f;      // log2(e) / sqrt(D)
-        unsigned phases = 0;                  // parities of the barriers this group waits on: bit 0 S, bit 1 end of a unit
+        const unsigned lanes = sh.tmem_base + ((unsigned)((warp & 3) * 32) << 16), tO = lanes + Col::O(g);
+        const PfTmem tm = {lanes + Col::S, lanes + Col::P(g), tO};
         bool ok = true;
         PfGroup& gr = sh.group[g];
         unsigned char* sQg = sQ + g * TILE_BYTES;
@@ -958,7 +1026,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             const int n_proc = w.n_proc;
             // (arrive: the issuer takes it from here.  A thread that would not be held up by the tensor pipe afterwards
             // has to sync instead, or it could arrive again before the issuer has seen the first time.)
-            if (ok && n_proc > 0) bar_arrive(BAR_Q + g, 160);
+            if (n_proc > 0) bar_arrive(BAR_Q + g, 160);
             else bar_sync(BAR_Q + g, 160);
             const int mt = gr.rows.m0 + g * 128;
             const int r = min(pf_div(mt + m, plan.g_magic, G), gr.rows.n_q - 1), r_lo = min(pf_div(mt, plan.g_magic, G), gr.rows.n_q - 1);
@@ -969,11 +1037,13 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             for (int j = 0; j < n_proc; ++j) {
                 const unsigned pi = pages.next(w, r_lo);
                 const bool masked = (pi >> 28) & 1;
-                unsigned vlo = 0, vlen = SVLM_PAGE;
+                unsigned vlo = 0, vlen = SVLM_PAGE, mixed = 0;      // mixed: of which 32 columns some row of the warp does not see all
                 if (masked) {
                     const int lo = (pi >> 14) & 127, hi = ((pi >> 21) & 127) + 1;
                     int end = hi;
-                    if ((pi >> 29) & 1) {     // the new chunk's tokens: causal
+                    if ((pi >> 30) & (pi >> 29) & 1) {     // the new chunk's tokens: causal.  One after another in the page: nothing to look up
+                        end = min(hi, lo + max(0, r - pages.first_here() + 1));
+                    } else if ((pi >> 29) & 1) {
                         const long long* gp = w.vw->slot_gid + (size_t)(pi & 0x3FFF) * SVLM_PAGE + 4 * lane;
                         const longlong2 ga = ld_in(reinterpret_cast<const longlong2*>(gp)), gb = ld_in(reinterpret_cast<const longlong2*>(gp) + 1);
                         const long long gv[4] = {ga.x, ga.y, gb.x, gb.y};
@@ -988,29 +1058,16 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     }
                     vlo = lo;
                     vlen = max(end, lo) - lo;
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch) mixed |= (unsigned)!__all_sync(0xffffffffu, lo <= 32 * ch && end >= 32 * ch + 32) << ch;
                 }
-                if (ok) ok = mbar_wait(&sh.s_full[g], phases & 1, abort_flag, w.wait_limit);
-                phases ^= 1;
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) {                    // keep the issuer's barriers supplied, in step with it
-                    bar_sync(BAR_P1 + g, 192);
-                    bar_sync(BAR_P2 + g, 160);
-                    continue;
-                }
+                bar_sync(BAR_S + g, 160);
                 tc_fence_after();
-                float rowsum, corr, m_new;
-                if (masked) softmax_page<true>(g, tS, tO, D, vlo, vlen, c, m_ref, j > 0, rowsum, corr, m_new);
-                else softmax_page<false>(g, tS, tO, D, vlo, vlen, c, m_ref, j > 0, rowsum, corr, m_new);
-                tmem_wait_st();
-                tc_fence_before();
-                bar_arrive(BAR_P2 + g, 160);
-                l = l * corr + rowsum;
-                m_ref = m_new;
+                softmax_page<D>(g, tm, mixed, vlo, vlen, j > 0, m_ref, l);
             }
-            if (ok) ok = mbar_wait(&sh.all_done[g], phases >> 1, abort_flag, w.wait_limit);
-            phases ^= 2;
-            ok = __all_sync(0xffffffffu, ok);
+            if (n_proc > 0) bar_sync(BAR_PV + g, 160);
             tc_fence_after();
+            ok = !*abort_flag;                // (of a wait that has run out nothing is known here: the barriers go on in their order)
             const bool have_o = ok && n_proc > 0;
             if (gr.seg.e - gr.seg.a == PF_FRAC) {                      // all of the unit's pages
                 const float inv = l > 0.f ? 1.f / l : 0.f;

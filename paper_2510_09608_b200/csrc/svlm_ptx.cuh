@@ -37,6 +37,31 @@ __device__ __forceinline__ bool mbar_wait(void* bar, unsigned parity, volatile i
     *abort_flag = 1;
     return false;
 }
+// `n` polls at most; a loop of few instructions, since what a wait costs is less the barrier than the fetching of its code.
+__device__ __forceinline__ bool mbar_poll(unsigned bar, unsigned parity, unsigned n) {
+    unsigned ok;
+    asm volatile("{\n.reg .pred p, q;\n.reg .u32 n;\nmov.u32 n, %3;\nsetp.ne.u32 p, 0, 0;\n"
+                 "setp.eq.u32 q, n, 0;\n@q bra DONE;\n"
+                 "LOOP:\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n@p bra DONE;\n"
+                 "sub.u32 n, n, 1;\nsetp.ne.u32 q, n, 0;\n@q bra LOOP;\n"
+                 "DONE:\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(n) : "memory");
+    return ok != 0;
+}
+// mbar_wait for a whole warp (all lanes poll: no branch by lane, nothing to hand around afterwards).
+__device__ __forceinline__ bool mbar_wait_short(void* bar, unsigned parity, volatile int* abort_flag, unsigned limit) {
+    const unsigned b = smem_u32(bar);
+#pragma unroll 1
+    while (!mbar_poll(b, parity, min(limit, 64u))) {
+        limit -= min(limit, 64u);
+        if (limit == 0 || *abort_flag) {
+            *abort_flag = 1;
+            return false;
+        }
+        __nanosleep(64);
+    }
+    return true;
+}
 // 2D tiled TMA load into this CTA's shared memory; completion is counted in bytes on `bar`.
 __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int x, int y, void* bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"

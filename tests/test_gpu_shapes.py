@@ -80,6 +80,30 @@ def test_large_chunk_prefill_gives_up_and_recovers(d, hq, hk):
     assert_close(s._stats(out[rows], s.ref.attend(0, s.stream.q(0, gids), pos, rows=rows)))
 
 
+# --- waits that run out somewhere in the middle of a unit: some polls, but too few for most waits.  The thread blocks come to their
+# --- end whoever gave up first, and the caches serve again
+@pytest.mark.parametrize("d,hq,hk", [(128, 28, 4), (64, 12, 2)])
+def test_large_chunk_prefill_gives_up_in_the_middle(d, hq, hk):
+    from paper_2510_09608_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    normal = lambda *shape: torch.randn(*shape, generator=gen, device="cuda", dtype=torch.bfloat16)      # noqa: E731
+    kept, n_q = 3000, 1400                                 # (several units per thread block)
+    c = binding.Cache(1, hk, d, 64, kept, 100, kept + 300)
+    c.append(0, normal(kept, hk, d), normal(kept, hk, d), torch.ones(kept, dtype=torch.uint8, device="cuda"), torch.arange(kept, dtype=torch.int32, device="cuda"))
+    q, pos = normal(n_q, hq, d), torch.arange(kept - n_q, kept, dtype=torch.int32, device="cuda")
+    want = c.attend(0, q, pos).clone()
+    seen = 0
+    for limit in (1, 2, 3, 5, 8, 13, 21, 34, 70):
+        c.debug_set_wait_limit(limit)
+        c.attend(0, q, pos)
+        status = c.status()
+        assert status in (binding.OK, binding.ERR_TIMEOUT)
+        seen += status == binding.ERR_TIMEOUT
+        c.debug_set_wait_limit(1 << 20)
+        assert torch.equal(c.attend(0, q, pos), want)
+    assert seen
+
+
 # --- pieces of a cut unit that do not wait for one another: the poll limit leaves the other waits alone and the meeting none,
 # --- so that whoever comes last puts the others' shares together; the same bits as when each merges its own
 @pytest.mark.parametrize("d,hq,hk,frames,vw", [(128, 28, 4, 7, 2304), (128, 28, 4, 1, 6000), (64, 12, 2, 7, 2304), (64, 16, 8, 1, 9000)])
