@@ -29,7 +29,7 @@ struct PfPlan {
     int rounds;                       // whole units per CTA first: CTA i takes units i, grid + i, ...
     int tail;                         // the units from here on are dealt out by x
     unsigned short x[PF_MAX_CTAS + 1];// where each CTA's share of them begins, in 1/128 units
-    unsigned g_magic;                 // for dividing by the heads per KV head (pf_div)
+    unsigned g_magic, g_shift;        // n / G = n * g_magic >> g_shift for n < 2^31 (pf_div)
     unsigned* counters;               // filled in at the launch: [2 * PF_MAX_CTAS][2][2] per (tail unit, tile) arrivals, zero between launches, and a turn;
     unsigned char* slots;             //   [2 * grid] partial results
 };
@@ -72,7 +72,9 @@ __host__ __device__ inline PfCut pf_cut(const PfPlan& plan, int tail, int cta, i
 // much as PF_PIECE pages.  The numbers of pages are estimates; a wrong one costs balance only.  cut: there is
 // scratch for the pieces of cut units.
 inline void pf_make_plan(PfPlan& plan, const SvlmAttendBatch& b, int n_layers, int n_q, int G, const SvlmPrefillLoad* held, int max_ctas, bool cut, int& grid) {
-    plan.g_magic = G > 1 && (unsigned long long)n_q * G * G < 0x100000000ull - 256ull * G ? (unsigned)((0x100000000ull + G - 1) / G) : 0u;   // (tiles reach past the last row)
+    plan.g_shift = 31;                                     // 31 + ceil(log2 G): the reciprocal rounded up to 32 bits is off by less than 2^-31 of 1 / G
+    while ((1ll << (plan.g_shift - 31)) < G) ++plan.g_shift;
+    plan.g_magic = (unsigned)(((1ull << plan.g_shift) + G - 1) / G);
     plan.units = 0;
     long long all = 0;                                     // pages of the whole launch
     const int per_unit = n_layers * b.kv_heads;

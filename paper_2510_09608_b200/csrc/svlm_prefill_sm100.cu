@@ -80,6 +80,7 @@ __device__ __forceinline__ float max3(float a, float b, float c) { float r; asm(
 __device__ __forceinline__ float ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
 // ---- named barriers (the hardware's, not shared memory): ids ----------------------------------------------------
+constexpr int BAR_ALL = 0;     // the thread block, as __syncthreads
 constexpr int BAR_WG = 1;      // + tile: the softmax warpgroup alone (128)
 constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM (128 softmax + 32 issuer)
 constexpr int BAR_P2 = 5;      // + tile: second half of P (128 + 32)
@@ -104,11 +105,14 @@ __device__ __forceinline__ void rescale_o(unsigned tO, int D, float corr) {
     }
 }
 
-// n / G with magic = ceil(2^32 / G), which is exact for n < 2^32 / G; magic = 0: the launch has other numbers.
-__device__ __forceinline__ int pf_div(int n, unsigned magic, int G) { return magic ? (int)__umulhi((unsigned)n, magic) : (G == 1 ? n : n / G); }
-// a / b for small numbers without the long division (a once-executed division costs hundreds of cycles of instruction fetch)
+// Divisions without a branch: once-executed code runs at the pace of its fetching, and each jump over a slow path that is not taken
+// is a new fetch (some 500 cycles where nothing has been there before).
+// n / G for 0 <= n < 2^31 (the plan's reciprocal).
+__device__ __forceinline__ int pf_div(int n, const PfPlan& plan) { return (int)(((unsigned long long)(unsigned)n * plan.g_magic) >> plan.g_shift); }
+// a / b for 0 <= a, 0 < b and a quotient below 2^20: the float quotient is off by one at most.
 __device__ __forceinline__ int pf_small_div(int a, int b) {
-    return a < (1 << 18) ? (int)(((float)a + 0.5f) * __frcp_rn((float)b)) : a / b;
+    const int q = (int)((float)a * __frcp_rn((float)b)), r = a - q * b;
+    return q + (r >= b) - (r < 0);
 }
 
 // A piece of the work list.
@@ -195,14 +199,14 @@ __device__ __forceinline__ PfAsk pf_ask(const SvlmAttendBatch& b, const PfRows& 
     for (int k = 0; k < 4; ++k) q.first[k] = ld_l2(&vw.tiles[min(lane + 32 * k, n_pages - 1)].min_gid);
     return q;
 }
-__device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfSeg& s, const PfRows& r, unsigned g_magic, int G, const PfAsk& q) {
+__device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfPlan& plan, const PfSeg& s, const PfRows& r, const PfAsk& q) {
     PfWork w;
     w.vw = &b.view[r.ci];
     w.n_tiles = q.n_tiles;
     w.gid_q0 = q.n_total - r.n_q;
     w.shift = q.shift;
     w.wait_limit = q.wait_limit;
-    w.gid_hi = w.gid_q0 + min(r.n_q - 1, pf_div(r.m0 + PF_ROWS - 1, g_magic, G));
+    w.gid_hi = w.gid_q0 + min(r.n_q - 1, pf_div(r.m0 + PF_ROWS - 1, plan));
     const int lane = threadIdx.x & 31;
     int n_act = 0;
 #pragma unroll
@@ -391,7 +395,7 @@ struct PfTileRotation {
     // element e of a row lives in block e/64, 16-byte chunk (e%64)/8, XOR-swizzled by row&7
     __device__ __forceinline__ static int at(int row, int e) { return (e / 64) * (128 * 128) + row * 128 + ((((e % 64) / 8) ^ (row & 7)) << 4); }
 
-    __device__ __forceinline__ static void load(const PfRows& w, int g, int m, int G, unsigned g_magic, int q_heads, const uint16_t* Q, unsigned char* sQ) {
+    __device__ __forceinline__ static void load(const PfPlan& plan, const PfRows& w, int g, int m, int G, int q_heads, const uint16_t* Q, unsigned char* sQ) {
         const int c8 = m % CH;
         const uint16_t* base = Q + (w.q_row0 * q_heads + w.hk * G) * D + c8 * 8;
         const unsigned dst = smem_u32(sQ);
@@ -400,7 +404,7 @@ struct PfTileRotation {
             const int row = m / CH + u * STEP, mg = w.m0 + g * 128 + row;
             const bool live = mg < w.m_total;
             // row (token r, head h) lies at r * q_heads + h = r * (q_heads - G) + mg
-            const uint16_t* src = live ? base + (size_t)(unsigned)(pf_div(mg, g_magic, G) * (q_heads - G) + mg) * D : base;
+            const uint16_t* src = live ? base + (size_t)(unsigned)(pf_div(mg, plan) * (q_heads - G) + mg) * D : base;
             const int n = live ? 16 : 0;                              // the rest is filled with zeros
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + at(row, c8 * 8)), "l"(src), "r"(n) : "memory");
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + at(row, HALF + c8 * 8)), "l"(src + HALF), "r"(n) : "memory");
@@ -423,10 +427,10 @@ struct PfTileRotation {
     __device__ __forceinline__ static bool is_near(long long c) { return c > -65536 && c < 65536; }
 
     // the tile's tokens and whether their factors fit the area
-    __device__ __forceinline__ static bool staged(const PfRows& w, int g, unsigned g_magic, int G, int& t_lo, int& n_tok) {
+    __device__ __forceinline__ static bool staged(const PfPlan& plan, const PfRows& w, int g, int& t_lo, int& n_tok) {
         const int mt = w.m0 + g * 128;
-        t_lo = min(w.n_q - 1, pf_div(mt, g_magic, G));
-        n_tok = min(w.n_q - 1, pf_div(mt + 127, g_magic, G)) - t_lo + 1;
+        t_lo = min(w.n_q - 1, pf_div(mt, plan));
+        n_tok = min(w.n_q - 1, pf_div(mt + 127, plan)) - t_lo + 1;
         return n_tok * (HALF * 8) <= PF_CS_BYTES;
     }
     // factors: per token HALF cosines, then HALF sines.  Eight consecutive lanes read eight values each at a time; the
@@ -476,13 +480,13 @@ struct PfTileRotation {
         }
     }
 
-    __device__ __forceinline__ static void rotate(const SvlmAttendBatch& b, const PfRows& w, long long shift, const int* q_pos, int g, int m,
-                                                  unsigned g_magic, int G, int t_lo, bool from_stage, const float* s_cs, unsigned char* sQ) {
+    __device__ __forceinline__ static void rotate(const SvlmAttendBatch& b, const PfPlan& plan, const PfRows& w, long long shift, const int* q_pos, int g, int m,
+                                                  int t_lo, bool from_stage, const float* s_cs, unsigned char* sQ) {
         const int c8 = m % CH;
-#pragma unroll 2
+#pragma unroll 1
         for (int u = 0; u < CH; ++u) {
             const int row = m / CH + u * STEP;
-            const int tk = min(pf_div(w.m0 + g * 128 + row, g_magic, G), w.n_q - 1);
+            const int tk = min(pf_div(w.m0 + g * 128 + row, plan), w.n_q - 1);
             uint4* plo = reinterpret_cast<uint4*>(sQ + at(row, c8 * 8));
             uint4* phi = reinterpret_cast<uint4*>(sQ + at(row, HALF + c8 * 8));
             const uint4 lo4 = *plo, hi4 = *phi;
@@ -582,8 +586,8 @@ __device__ __forceinline__ void store_row16(uint16_t* dst, const float* o, bool 
     }
 }
 
-__device__ __forceinline__ uint16_t* out_row(uint16_t* out, const PfRows& w, int mg, unsigned g_magic, int G, int q_heads, int D) {
-    const int r = pf_div(mg, g_magic, G);      // row (token r, head h) lies at r * q_heads + h = r * (q_heads - G) + mg
+__device__ __forceinline__ uint16_t* out_row(uint16_t* out, const PfPlan& plan, const PfRows& w, int mg, int G, int q_heads, int D) {
+    const int r = pf_div(mg, plan);      // row (token r, head h) lies at r * q_heads + h = r * (q_heads - G) + mg
     return out + (w.q_row0 * q_heads + w.hk * G + (size_t)(unsigned)(r * (q_heads - G) + mg)) * D;
 }
 
@@ -721,7 +725,7 @@ __device__ __forceinline__ void merge_blocks(const PfPlan& plan, int tail, const
     };
     auto ml_of = [&](int k) { return k == me ? make_float2(m_own, l) : ld_l2(PfSlot<D>(plan, tail, k).ml(g, m)); };
     const int mg = w.m0 + g * 128 + m;
-    uint16_t* dst = out_row(out, w, min(mg, w.m_total - 1), plan.g_magic, G, q_heads, D);
+    uint16_t* dst = out_row(out, plan, w, min(mg, w.m_total - 1), G, q_heads, D);
     const bool wide = !(reinterpret_cast<uintptr_t>(out) & 31);
     const int k2 = after(first);                             // (the first CTA's share is not empty, and a cut unit has two pieces at least)
     const float m1 = ml_of(first).x, m2 = ml_of(k2).x;
@@ -816,13 +820,19 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         const int x0 = plan.x[blockIdx.x], x1 = plan.x[blockIdx.x + 1], which = threadIdx.x / 32 - 1;
         if (x0 < x1) sh.cut[which] = pf_cut(plan, (which ? x0 : x1 - 1) / PF_FRAC, blockIdx.x, D / 16);
     }
-    // Set up while the predecessor ends (programmatic dependent launch); everything read from here on may be its work.
+    // Set up while the predecessor ends (programmatic dependent launch): the roles also work out where their first segment lies,
+    // which hangs on the launch's arguments only.  Everything read from here on may be the predecessor's work.
     // The wait comes before the trigger: a successor that starts early then finds all earlier work done.
-    pdl_wait();
-    pdl_launch_dependents();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
+    bool entered = false;
+    auto enter = [&] {
+        if (entered) return;
+        entered = true;
+        pdl_wait();
+        pdl_launch_dependents();
+        tc_fence_before();
+        bar_sync(BAR_ALL, PF_THREADS);
+        tc_fence_after();
+    };
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
@@ -835,7 +845,8 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
                 const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
-                const PfWork w = pf_work(b, seg, rows, plan.g_magic, G, pf_ask(b, rows));
+                enter();
+                const PfWork w = pf_work(b, plan, seg, rows, pf_ask(b, rows));
                 const void* tmK = w.vw->tmaps;
                 const void* tmV = reinterpret_cast<const unsigned char*>(w.vw->tmaps) + 128;
                 PfPages pages;
@@ -873,13 +884,12 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             // Without a working wait everybody goes on along these lines, the issuers without issuing anything, and warp 11
             // follows them by their count of products (asked).
             const int g = warp - 9;
-            const unsigned tmem = __shfl_sync(0xffffffffu, sh.tmem_base, 0);
             const bool leader = elect_one();
             constexpr unsigned IDESC_S = make_idesc(128, 128, 0);
             constexpr unsigned IDESC_O = make_idesc(128, D, 1);
             // descriptors: the 14-bit start-address field counts 16-byte units, so moving inside a tile is an
             // addition to the low word (all tile addresses stay below the field's range: shared memory is 228 KB)
-            const unsigned tmem_s = tmem + Col::S, tmem_p = tmem + Col::P(g), tmem_o = tmem + Col::O(g);
+            unsigned tmem_s = 0, tmem_p = 0, tmem_o = 0;
             const unsigned long long dq = smem_desc(smem_u32(sQ + g * TILE_BYTES), 16, 1024);   // Q, K: K-major
             const unsigned long long dk = smem_desc(smem_u32(ring), 16, 1024);
             const unsigned long long dv = smem_desc(smem_u32(ring), 128 * 128, 1024);           // V: MN-major
@@ -924,7 +934,12 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
                 const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
-                const PfWork w = pf_work(b, seg, rows, plan.g_magic, G, pf_ask(b, rows));
+                enter();
+                const PfWork w = pf_work(b, plan, seg, rows, pf_ask(b, rows));
+                const unsigned tmem = __shfl_sync(0xffffffffu, sh.tmem_base, 0);
+                tmem_s = tmem + Col::S;
+                tmem_p = tmem + Col::P(g);
+                tmem_o = tmem + Col::O(g);
                 wait_limit = w.wait_limit;
                 const int n = w.n_proc;
                 // ring items: K(0) K(1) V(0) K(2) V(1) ... K(n-1) V(n-2) V(n-1)
@@ -960,7 +975,8 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
                 const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
-                const PfWork w = pf_work(b, seg, rows, plan.g_magic, G, pf_ask(b, rows));
+                enter();
+                const PfWork w = pf_work(b, plan, seg, rows, pf_ask(b, rows));
                 for (int j = 0; j < w.n_proc; ++j, ++steps)
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
@@ -977,8 +993,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
         // ================= softmax warpgroups: one thread per row of tile g =================
         const int g = warp >> 2, m = threadIdx.x & 127;
-        const unsigned lanes = sh.tmem_base + ((unsigned)((warp & 3) * 32) << 16), tO = lanes + Col::O(g);
-        const PfTmem tm = {lanes + Col::S, lanes + Col::P(g), tO};
+        PfTmem tm = {};
         bool ok = true;
         PfGroup& gr = sh.group[g];
         unsigned char* sQg = sQ + g * TILE_BYTES;
@@ -995,7 +1010,10 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 // in the order in which the answers are needed: the memory system takes them one after another
                 PfTileRotation<D> rot;
                 int t_lo, n_tok;
-                const bool staged = PfTileRotation<D>::staged(rows, g, plan.g_magic, G, t_lo, n_tok);
+                const bool staged = PfTileRotation<D>::staged(plan, rows, g, t_lo, n_tok);
+                enter();
+                const unsigned lanes = sh.tmem_base + ((unsigned)((warp & 3) * 32) << 16);
+                tm = {lanes + Col::S, lanes + Col::P(g), lanes + Col::O(g)};
                 const bool fresh = rows.ci != gr.known;
                 PfAsk ask;
                 if (fresh) {
@@ -1006,8 +1024,8 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     for (int k = 0; k < 4; ++k) ask.first[k] = gr.first[lane + 32 * k];
                 }
                 if (staged) rot.load_pos(b, rows, q_pos, m, t_lo, n_tok, m / PfTileRotation<D>::HALF);
-                PfTileRotation<D>::load(rows, g, m, G, plan.g_magic, q_heads, Q, sQg);
-                const PfWork nw = pf_work(b, seg, rows, plan.g_magic, G, ask);
+                PfTileRotation<D>::load(plan, rows, g, m, G, q_heads, Q, sQg);
+                const PfWork nw = pf_work(b, plan, seg, rows, ask);
                 if (m == 0) { gr.seg = seg; gr.rows = rows; gr.w = nw; gr.more = walk.more(plan); }
                 if (staged) rot.stage(b, rows, nw.shift, q_pos, m, t_lo, n_tok, cs_g);
                 asm volatile("cp.async.wait_all;" ::: "memory");
@@ -1018,7 +1036,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
 #pragma unroll
                     for (int k = 0; k < 4; ++k) gr.first[m + 32 * k] = ask.first[k];
                 }
-                PfTileRotation<D>::rotate(b, rows, nw.shift, q_pos, g, m, plan.g_magic, G, t_lo, staged, cs_g, sQg);
+                PfTileRotation<D>::rotate(b, plan, rows, nw.shift, q_pos, g, m, t_lo, staged, cs_g, sQg);
             }
             fence_proxy_async();              // the tile feeds the tensor core
             tc_fence_before();                // (the previous unit's accumulator has been read)
@@ -1029,7 +1047,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             if (n_proc > 0) bar_arrive(BAR_Q + g, 160);
             else bar_sync(BAR_Q + g, 160);
             const int mt = gr.rows.m0 + g * 128;
-            const int r = min(pf_div(mt + m, plan.g_magic, G), gr.rows.n_q - 1), r_lo = min(pf_div(mt, plan.g_magic, G), gr.rows.n_q - 1);
+            const int r = min(pf_div(mt + m, plan), gr.rows.n_q - 1), r_lo = min(pf_div(mt, plan), gr.rows.n_q - 1);
             m_ref = -INFINITY;
             l = 0.f;
             PfPages pages;
@@ -1072,13 +1090,13 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             if (gr.seg.e - gr.seg.a == PF_FRAC) {                      // all of the unit's pages
                 const float inv = l > 0.f ? 1.f / l : 0.f;
                 const int mg = mt + m;
-                uint16_t* dst = out_row(out, gr.rows, min(mg, gr.rows.m_total - 1), plan.g_magic, G, q_heads, D);
+                uint16_t* dst = out_row(out, plan, gr.rows, min(mg, gr.rows.m_total - 1), G, q_heads, D);
                 const bool wide = !(reinterpret_cast<uintptr_t>(out) & 31);
 #pragma unroll 1
                 for (int q4 = 0; q4 < D / 32; ++q4) {
                     float o[32];
                     if (have_o) {
-                        tmem_ld32(tO + q4 * 32, o);
+                        tmem_ld32(tm.O + q4 * 32, o);
                         tmem_wait_ld<32>(o);
                     }
 #pragma unroll
@@ -1089,7 +1107,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     }
                 }
             } else if (gr.more) {                                      // the end of a unit that others have begun
-                const unsigned take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[1], g, m, tO, m_ref, l, have_o, false, 0);
+                const unsigned take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[1], g, m, tm.O, m_ref, l, have_o, false, 0);
                 if (m == 0) gr.merge_later = take;
             }
         }
@@ -1097,7 +1115,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         const bool have_o = ok && gr.w.n_proc > 0;
         unsigned take = 0;
         if (gr.seg.e - gr.seg.a < PF_FRAC)
-            take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[0], g, m, tO, m_ref, l, have_o, true, gr.w.wait_limit >> PF_MEET_POLLS);
+            take = meet_pieces<D>(sh, plan, gr.seg.tail, sh.cut[0], g, m, tm.O, m_ref, l, have_o, true, gr.w.wait_limit >> PF_MEET_POLLS);
         bar_sync(BAR_WG + g, 128);
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
@@ -1105,9 +1123,11 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             if (!blocks) continue;
             const int tail = (pass == 0 ? plan.x[blockIdx.x + 1] - 1 : (int)plan.x[blockIdx.x]) / PF_FRAC;
             const PfRows rows = pf_rows(b, plan, plan.tail + tail, n_q_arg, G, layer0, n_layers);
-            merge_blocks<D>(plan, tail, sh.cut[pass], blocks, rows, g, m, G, q_heads, pass == 0, tO, m_ref, l, have_o, out);
+            merge_blocks<D>(plan, tail, sh.cut[pass], blocks, rows, g, m, G, q_heads, pass == 0, tm.O, m_ref, l, have_o, out);
         }
     }
+
+    enter();                                   // (a thread block without work)
 
     // ---- teardown ------------------------------------------------------------------------------
     tc_fence_before();
