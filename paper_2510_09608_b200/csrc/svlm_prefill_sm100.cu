@@ -18,7 +18,7 @@
 //                    runs ahead into the next unit while the current one ends
 //   warps 9, 10      issue tcgen05.mma for tile A, B: S = Q K^T into 128 TMEM columns, O += P V with P read from
 //                    TMEM (no shared-memory round trip), and say to the softmax that P V is done
-//   warp 11          says to the softmax that S is there
+//   warp 11          fetches the cache's metadata, once; then it says to the softmax that S is there
 // TMEM: O of both tiles (256 columns at head_dim 128), P of both (64 each, bf16), and one buffer of 128 for S that the tiles take
 // in turns: S(A,0) S(B,0) S(A,1) S(B,1) ...  A tile's scores stay there only until they are in its softmax warps' registers, then
 // the other tile's come, so S(j+1) of a tile is there before its P V(j) has begun and the softmax warps go from page to page
@@ -85,9 +85,10 @@ constexpr int BAR_WG = 1;      // + tile: the softmax warpgroup alone (128)
 constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM (128 softmax + 32 issuer)
 constexpr int BAR_P2 = 5;      // + tile: second half of P (128 + 32)
 constexpr int BAR_READ = 7;    // + tile: its S is in registers, the columns are free (128 + 32 issuer of the S that comes there next)
-constexpr int BAR_S = 11;      // + tile: S is in TMEM (128 + 32 warp 11)
+constexpr int BAR_S = 11;      // + tile: S is in TMEM; the first time, the metadata is there (128 + 32 warp 11)
 constexpr int BAR_PV = 13;     // + tile: P V is done: its P may be overwritten, its accumulator touched (128 + 32 issuer)
 constexpr int BAR_Q = 9;       // + tile: the tile's query rows are in shared memory, its accumulator is free (128 + 32)
+constexpr int BAR_META = 15;   // the metadata is there (warps 8 to 11)
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
@@ -172,46 +173,77 @@ __device__ __forceinline__ PfRows pf_rows(const SvlmAttendBatch& b, const PfPlan
     return r;
 }
 
-// What the cache's metadata adds: the segment's pages.
+// An entry of a cache's page list, ordinals relative to the first query token (those of long ago: some large negative number).
+struct __align__(16) PfEntry {
+    unsigned info;                 // page | lo << 14 | (hi - 1) << 21 | partly filled << 28 | ordinals one after another << 30
+    int first, last, pad;
+};
+__device__ __forceinline__ PfEntry pf_entry(const int4& a, const longlong2& g, long long gid_q0) {
+    PfEntry e;
+    e.info = (unsigned)a.x | ((unsigned)a.y << 14) | ((unsigned)(a.z - 1) << 21) | ((unsigned)(a.y > 0 || a.z < SVLM_PAGE) << 28) |
+             ((unsigned)(g.y - g.x == a.z - 1 - a.y) << 30);      // (ordinals grow with the offset)
+    e.first = (int)max(g.x - gid_q0, -0x40000000ll);
+    e.last = (int)max(g.y - gid_q0, -0x40000000ll);
+    e.pad = 0;
+    return e;
+}
+__device__ __forceinline__ PfEntry pf_load_entry(const SvlmAttendView& vw, int j, long long gid_q0) {
+    const SvlmTile* tp = vw.tiles + j;
+    const int4 a = ld_l2(reinterpret_cast<const int4*>(tp));
+    return pf_entry(a, ld_l2(reinterpret_cast<const longlong2*>(&tp->min_gid)), gid_q0);
+}
+
+// What the cache's metadata says: fetched once per thread block, by warp 11, for the cache of the first segment.  All thread blocks
+// begin at the same time, and with twelve warps of each reading the same few lines of L2 they waited for one another: 3900 cycles until
+// the first page was known, 3300 now, and 11,700 until its S was there, 10,300 now (28/4 heads of 128, 524 tokens, many layers).
+// Segments of other caches come at different times; there each warp looks by itself.
+constexpr int PF_LIST = 128;
+struct PfMeta {
+    int ci, n_tiles;
+    unsigned wait_limit;
+    long long n_total, shift;
+    PfEntry list[PF_LIST];         // the first entries of its page list
+};
+
+// What the metadata adds to a segment: its pages.
 struct PfWork {
     const SvlmAttendView* vw;
+    const PfEntry* list;           // the first PF_LIST entries, null: to be looked up
     int n_tiles, p0, n_proc;       // entries of the page list; of the pages that some row of the unit may see, [p0, p0 + n_proc)
-    long long gid_hi, gid_q0;      // ordinals of the unit's last row's token and of the first query token
+    int rel_hi;                    // of the unit's last row's token
+    long long gid_q0;              // ordinal of the first query token
     long long shift;
     unsigned wait_limit;
 };
-// In two steps, so that a caller can have more in flight: the loads (the first pages' ordinals without waiting for their
-// count, so that everything takes one round trip), then what they say.
-struct PfAsk {
-    long long first[4], n_total, shift;
-    int n_tiles;
-    unsigned wait_limit;
-};
-__device__ __forceinline__ PfAsk pf_ask(const SvlmAttendBatch& b, const PfRows& r) {
-    PfAsk q;
-    const SvlmAttendView& vw = b.view[r.ci];
-    const int lane = threadIdx.x & 31, n_pages = b.n_slots / SVLM_PAGE;
-    q.n_tiles = ld_l2(&vw.ctrl->n_tiles);
-    q.n_total = ld_l2(&vw.ctrl->n_total);
-    q.shift = ld_l2(&vw.ctrl->shift_total);
-    q.wait_limit = ld_l2(&vw.ctrl->wait_limit);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) q.first[k] = ld_l2(&vw.tiles[min(lane + 32 * k, n_pages - 1)].min_gid);
-    return q;
-}
-__device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfPlan& plan, const PfSeg& s, const PfRows& r, const PfAsk& q) {
+__device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfPlan& plan, const PfMeta& meta, const PfSeg& s, const PfRows& r) {
     PfWork w;
     w.vw = &b.view[r.ci];
-    w.n_tiles = q.n_tiles;
-    w.gid_q0 = q.n_total - r.n_q;
-    w.shift = q.shift;
-    w.wait_limit = q.wait_limit;
-    w.gid_hi = w.gid_q0 + min(r.n_q - 1, pf_div(r.m0 + PF_ROWS - 1, plan));
+    w.rel_hi = min(r.n_q - 1, pf_div(r.m0 + PF_ROWS - 1, plan));
     const int lane = threadIdx.x & 31;
-    int n_act = 0;
+    int n_act = 0, j = lane;
+    if (r.ci == meta.ci) {
+        w.list = meta.list;
+        w.n_tiles = meta.n_tiles;
+        w.gid_q0 = meta.n_total - r.n_q;
+        w.shift = meta.shift;
+        w.wait_limit = meta.wait_limit;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) n_act += lane + 32 * k < w.n_tiles && q.first[k] <= w.gid_hi;
-    for (int j = lane + 128; j < w.n_tiles; j += 32) n_act += ld_l2(&w.vw->tiles[j].min_gid) <= w.gid_hi;
+        for (; j < PF_LIST; j += 32) n_act += j < w.n_tiles && meta.list[j].first <= w.rel_hi;
+    } else {
+        const SvlmCtrl* ctrl = w.vw->ctrl;
+        w.list = nullptr;
+        w.n_tiles = ld_l2(&ctrl->n_tiles);
+        const long long n_total = ld_l2(&ctrl->n_total);
+        w.shift = ld_l2(&ctrl->shift_total);
+        w.wait_limit = ld_l2(&ctrl->wait_limit);
+        long long first[4];        // without waiting for their number, so that everything takes one round trip
+#pragma unroll
+        for (int k = 0; k < 4; ++k) first[k] = ld_l2(&w.vw->tiles[min(lane + 32 * k, b.n_slots / SVLM_PAGE - 1)].min_gid);
+        w.gid_q0 = n_total - r.n_q;
+#pragma unroll
+        for (int k = 0; k < 4; ++k, j += 32) n_act += j < w.n_tiles && first[k] - w.gid_q0 <= w.rel_hi;
+    }
+    for (; j < w.n_tiles; j += 32) n_act += ld_l2(&w.vw->tiles[j].min_gid) - w.gid_q0 <= w.rel_hi;
     n_act = __reduce_add_sync(0xffffffffu, n_act);
     w.p0 = s.a * n_act / PF_FRAC;
     w.n_proc = s.e * n_act / PF_FRAC - w.p0;
@@ -226,11 +258,6 @@ struct PfGroup {
     PfWork w;
     PfWalk walk;
     int more;                // segments follow
-    int known;               // the cache that the next five belong to (-1: none): a launch does not change its metadata
-    int n_tiles;
-    unsigned wait_limit;
-    long long n_total, shift;
-    long long first[128];    // smallest ordinals of the first pages of its list
     unsigned merge_later;    // blocks of columns of the first segment's unit that this CTA has to merge at the end
 };
 
@@ -244,6 +271,8 @@ struct PfShared {            // control part of shared memory, behind the tiles
     int leave[2];                          // its own ones are left to whoever comes last
     PfCut cut[2];                          // of the CTA's last segment, of its first one
     PfGroup group[2];
+    int past[9][2];                        // per warp: PfPages
+    PfMeta meta;
 };
 static_assert(sizeof(PfShared) <= 3072, "control block must fit behind the tiles");
 
@@ -345,33 +374,35 @@ __device__ __forceinline__ void softmax_page(int g, const PfTmem& t, unsigned mi
 }
 
 
-// A warp's walk over the pages of a segment, 32 tiles of the cache's page list at a time, one per lane.
+// A warp's walk over the pages of a segment, 32 entries of the cache's page list at a time, one per lane.
 struct PfPages {
-    int base, seen;
-    unsigned left, info;     // pages of the window still to come; per lane: page | lo << 14 | (hi - 1) << 21 | masked << 28 | causal << 29 | no gaps << 30
-    int first, at;           // per lane: ordinal of slot lo, relative to the first query token; lane of the latest page
-    __device__ __forceinline__ void begin() { base = 0; seen = 0; left = 0; info = 0; first = 0; at = 0; }
+    int* past;               // in shared memory, since seldom wanted: entries looked at, pages seen among them
+    unsigned left, info;     // pages of the window still to come; per lane: the entry's info, needs a mask << 28, causal << 29
+    int first, at;           // per lane: ordinal of the page's first token, relative to the first query token; lane of the latest page
+    __device__ __forceinline__ void begin(PfShared& sh) {
+        past = sh.past[threadIdx.x >> 5];
+        past[0] = 0;
+        past[1] = 0;
+        left = 0; info = 0; first = 0; at = 0;
+    }
     // r_lo: rows from this token on are served; a page all of them see in full needs no mask
     __device__ __forceinline__ unsigned next(const PfWork& w, int r_lo) {
-        const int lane = threadIdx.x & 31;
-        while (left == 0 && base < w.n_tiles) {
-            const int j = base + lane;
-            bool vis = false;
-            if (j < w.n_tiles) {
-                const SvlmTile* tp = w.vw->tiles + j;
-                const int4 a = ld_l2(reinterpret_cast<const int4*>(tp));
-                const longlong2 g = ld_l2(reinterpret_cast<const longlong2*>(&tp->min_gid));
-                vis = g.x <= w.gid_hi;
-                const unsigned causal = g.y > w.gid_q0 + r_lo, ragged = a.y > 0 || a.z < SVLM_PAGE;
-                info = (unsigned)a.x | ((unsigned)a.y << 14) | ((unsigned)(a.z - 1) << 21) | ((causal | ragged) << 28) | (causal << 29) |
-                       ((unsigned)(g.y - g.x == a.z - 1 - a.y) << 30);       // ordinals grow with the offset: then one after another
-                first = (int)max(g.x - w.gid_q0, -0x40000000ll);
-            }
+        while (left == 0) {
+            const int base = past[0], seen = past[1];
+            if (base >= w.n_tiles) break;
+            const int lane = threadIdx.x & 31, j = min(base + lane, w.n_tiles - 1);
+            const PfEntry e = w.list && base < PF_LIST ? w.list[j] : pf_load_entry(*w.vw, j, w.gid_q0);
+            const bool vis = base + lane < w.n_tiles && e.first <= w.rel_hi;
+            const unsigned causal = e.last > r_lo;
+            info = e.info | (causal << 28) | (causal << 29);
+            first = e.first;
             const unsigned all = __ballot_sync(0xffffffffu, vis);
             const int rank = seen + __popc(all & ((1u << lane) - 1));
             left = __ballot_sync(0xffffffffu, vis && rank >= w.p0 && rank < w.p0 + w.n_proc);
-            seen += __popc(all);
-            base += 32;
+            __syncwarp();
+            past[0] = base + 32;
+            past[1] = seen + __popc(all);
+            __syncwarp();
         }
         at = left ? __ffs(left) - 1 : 0;
         left &= left - 1;
@@ -398,16 +429,16 @@ struct PfTileRotation {
     __device__ __forceinline__ static void load(const PfPlan& plan, const PfRows& w, int g, int m, int G, int q_heads, const uint16_t* Q, unsigned char* sQ) {
         const int c8 = m % CH;
         const uint16_t* base = Q + (w.q_row0 * q_heads + w.hk * G) * D + c8 * 8;
-        const unsigned dst = smem_u32(sQ);
+        const unsigned lo = smem_u32(sQ) + at(m / CH, c8 * 8), hi = smem_u32(sQ) + at(m / CH, HALF + c8 * 8);      // (STEP is a multiple of 8: the swizzle stays)
 #pragma unroll 2
         for (int u = 0; u < CH; ++u) {
-            const int row = m / CH + u * STEP, mg = w.m0 + g * 128 + row;
+            const int mg = w.m0 + g * 128 + m / CH + u * STEP;
             const bool live = mg < w.m_total;
             // row (token r, head h) lies at r * q_heads + h = r * (q_heads - G) + mg
             const uint16_t* src = live ? base + (size_t)(unsigned)(pf_div(mg, plan) * (q_heads - G) + mg) * D : base;
             const int n = live ? 16 : 0;                              // the rest is filled with zeros
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + at(row, c8 * 8)), "l"(src), "r"(n) : "memory");
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + at(row, HALF + c8 * 8)), "l"(src + HALF), "r"(n) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(lo + u * STEP * 128), "l"(src), "r"(n) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(hi + u * STEP * 128), "l"(src + HALF), "r"(n) : "memory");
         }
     }
     __device__ __forceinline__ static int axis_of(const SvlmAttendBatch& b, int pair) {
@@ -451,13 +482,13 @@ struct PfTileRotation {
 #pragma unroll 1
         for (int tk0 = m / HALF; tk0 < n_tok; tk0 += TPT * UN) {
             Near v[UN];
-            if (tk0 >= TPT) load_pos(b, w, q_pos, m, t_lo, n_tok, tk0);      // (the first batch is here already)
 #pragma unroll
-            for (int u = 0; u < UN; ++u) {
+            for (int u = 0; u < UN; ++u) {                                   // (the first batch of positions is here already)
                 const long long cl = (long long)c[u] - shift;
                 far |= !is_near(cl);
                 v[u] = near_load(tab, pair, (int)cl);
             }
+            load_pos(b, w, q_pos, m, t_lo, n_tok, tk0 + TPT * UN);           // beside the look-ups (of the last batch: its end once more)
 #pragma unroll
             for (int u = 0; u < UN; ++u) {
                 const int tk = tk0 + u * TPT;
@@ -845,12 +876,15 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
                 const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
-                enter();
-                const PfWork w = pf_work(b, plan, seg, rows, pf_ask(b, rows));
+                if (!entered) {
+                    enter();
+                    bar_sync(BAR_META, 128);
+                }
+                const PfWork w = pf_work(b, plan, sh.meta, seg, rows);
                 const void* tmK = w.vw->tmaps;
                 const void* tmV = reinterpret_cast<const unsigned char*>(w.vw->tmaps) + 128;
                 PfPages pages;
-                pages.begin();
+                pages.begin(sh);
                 int y = 0, y_before = 0;
                 for (int j = 0; j <= w.n_proc && ok; ++j) {
                     if (j < w.n_proc) y = (int)(rows.head_row0 + (size_t)(pages.next(w, 0) & 0x3FFF) * SVLM_PAGE);
@@ -934,8 +968,11 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
                 const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
-                enter();
-                const PfWork w = pf_work(b, plan, seg, rows, pf_ask(b, rows));
+                if (!entered) {
+                    enter();
+                    bar_sync(BAR_META, 128);
+                }
+                const PfWork w = pf_work(b, plan, sh.meta, seg, rows);
                 const unsigned tmem = __shfl_sync(0xffffffffu, sh.tmem_base, 0);
                 tmem_s = tmem + Col::S;
                 tmem_p = tmem + Col::P(g);
@@ -972,11 +1009,35 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             // ================= warp 11: says to the softmax that S is there =================
             // (A wait on an mbarrier costs a softmax warp ~300 cycles even when it is complete, a named barrier 40.)
             unsigned steps = 0;
+            auto fetch_meta = [&](const PfRows& r) {
+                const SvlmAttendView& vw = b.view[r.ci];
+                int4 a[PF_LIST / 32];
+                longlong2 g[PF_LIST / 32];
+#pragma unroll
+                for (int k = 0; k < PF_LIST / 32; ++k) {             // (pages that are not there: left over from earlier, not used)
+                    const SvlmTile* tp = vw.tiles + min(lane + 32 * k, b.n_slots / SVLM_PAGE - 1);
+                    a[k] = ld_l2(reinterpret_cast<const int4*>(tp));
+                    g[k] = ld_l2(reinterpret_cast<const longlong2*>(&tp->min_gid));
+                }
+                const int n_tiles = ld_l2(&vw.ctrl->n_tiles);
+                const long long n_total = ld_l2(&vw.ctrl->n_total), shift = ld_l2(&vw.ctrl->shift_total);
+                const unsigned wait_limit = ld_l2(&vw.ctrl->wait_limit);
+#pragma unroll
+                for (int k = 0; k < PF_LIST / 32; ++k) sh.meta.list[lane + 32 * k] = pf_entry(a[k], g[k], n_total - r.n_q);
+                if (lane == 0) { sh.meta.ci = r.ci; sh.meta.n_tiles = n_tiles; sh.meta.wait_limit = wait_limit; sh.meta.n_total = n_total; sh.meta.shift = shift; }
+                __syncwarp();
+            };
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
                 const PfRows rows = pf_rows(b, plan, seg.unit, n_q_arg, G, layer0, n_layers);
-                enter();
-                const PfWork w = pf_work(b, plan, seg, rows, pf_ask(b, rows));
+                if (!entered) {
+                    enter();
+                    fetch_meta(rows);
+                    bar_sync(BAR_META, 128);
+                    bar_arrive(BAR_S, 160);
+                    bar_arrive(BAR_S + 1, 160);
+                }
+                const PfWork w = pf_work(b, plan, sh.meta, seg, rows);
                 for (int j = 0; j < w.n_proc; ++j, ++steps)
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
@@ -999,7 +1060,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
         unsigned char* sQg = sQ + g * TILE_BYTES;
         float* cs_g = reinterpret_cast<float*>(s_cs + g * PF_CS_BYTES);
         float m_ref = -INFINITY, l = 0.f;
-        if (m == 0) { gr.walk.begin(plan); gr.merge_later = 0; gr.known = -1; gr.more = gr.walk.more(plan); gr.seg.a = 0; gr.seg.e = PF_FRAC; }
+        if (m == 0) { gr.walk.begin(plan); gr.merge_later = 0; gr.more = gr.walk.more(plan); gr.seg.a = 0; gr.seg.e = PF_FRAC; }
         bar_sync(BAR_WG + g, 128);
         while (gr.more) {
             bar_sync(BAR_WG + g, 128);        // everybody is through with the previous segment's fields
@@ -1011,31 +1072,19 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 PfTileRotation<D> rot;
                 int t_lo, n_tok;
                 const bool staged = PfTileRotation<D>::staged(plan, rows, g, t_lo, n_tok);
+                const bool start = !entered;
                 enter();
                 const unsigned lanes = sh.tmem_base + ((unsigned)((warp & 3) * 32) << 16);
                 tm = {lanes + Col::S, lanes + Col::P(g), lanes + Col::O(g)};
-                const bool fresh = rows.ci != gr.known;
-                PfAsk ask;
-                if (fresh) {
-                    ask = pf_ask(b, rows);
-                } else {
-                    ask.n_tiles = gr.n_tiles; ask.n_total = gr.n_total; ask.shift = gr.shift; ask.wait_limit = gr.wait_limit;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) ask.first[k] = gr.first[lane + 32 * k];
-                }
                 if (staged) rot.load_pos(b, rows, q_pos, m, t_lo, n_tok, m / PfTileRotation<D>::HALF);
                 PfTileRotation<D>::load(plan, rows, g, m, G, q_heads, Q, sQg);
-                const PfWork nw = pf_work(b, plan, seg, rows, ask);
+                if (start) bar_sync(BAR_S + g, 160);
+                const PfWork nw = pf_work(b, plan, sh.meta, seg, rows);
                 if (m == 0) { gr.seg = seg; gr.rows = rows; gr.w = nw; gr.more = walk.more(plan); }
                 if (staged) rot.stage(b, rows, nw.shift, q_pos, m, t_lo, n_tok, cs_g);
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 bar_sync(BAR_WG + g, 128);
                 if (m == 0) gr.walk = walk;
-                if (fresh && m < 32) {
-                    if (m == 0) { gr.known = rows.ci; gr.n_tiles = ask.n_tiles; gr.n_total = ask.n_total; gr.shift = ask.shift; gr.wait_limit = ask.wait_limit; }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) gr.first[m + 32 * k] = ask.first[k];
-                }
                 PfTileRotation<D>::rotate(b, plan, rows, nw.shift, q_pos, g, m, t_lo, staged, cs_g, sQg);
             }
             fence_proxy_async();              // the tile feeds the tensor core
@@ -1047,11 +1096,11 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             if (n_proc > 0) bar_arrive(BAR_Q + g, 160);
             else bar_sync(BAR_Q + g, 160);
             const int mt = gr.rows.m0 + g * 128;
-            const int r = min(pf_div(mt + m, plan), gr.rows.n_q - 1), r_lo = min(pf_div(mt, plan), gr.rows.n_q - 1);
             m_ref = -INFINITY;
             l = 0.f;
+            const int r = min(pf_div(mt + m, plan), gr.rows.n_q - 1), r_lo = min(pf_div(mt, plan), gr.rows.n_q - 1);
             PfPages pages;
-            pages.begin();
+            pages.begin(sh);
             for (int j = 0; j < n_proc; ++j) {
                 const unsigned pi = pages.next(w, r_lo);
                 const bool masked = (pi >> 28) & 1;
