@@ -197,7 +197,7 @@ __device__ __forceinline__ PfEntry pf_load_entry(const SvlmAttendView& vw, int j
 // begin at the same time, and with twelve warps of each reading the same few lines of L2 they waited for one another: 3900 cycles until
 // the first page was known, 3300 now, and 11,700 until its S was there, 10,300 now (28/4 heads of 128, 524 tokens, many layers).
 // Segments of other caches come at different times; there each warp looks by itself.
-constexpr int PF_LIST = 128;
+constexpr int PF_LIST = 96;
 struct PfMeta {
     int ci, n_tiles;
     unsigned wait_limit;
@@ -215,35 +215,52 @@ struct PfWork {
     long long shift;
     unsigned wait_limit;
 };
-__device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfPlan& plan, const PfMeta& meta, const PfSeg& s, const PfRows& r) {
+// What is known of a cache.
+struct PfAsk {
+    int first[PF_LIST / 32];       // of the first pages, relative to the first query token
+    int n_tiles;
+    long long n_total, shift;
+    unsigned wait_limit;
+};
+// From its control block and its page list (the ordinals without waiting for their count, so that everything takes one round trip).
+__device__ __forceinline__ PfAsk pf_ask(const SvlmAttendBatch& b, const PfRows& r) {
+    PfAsk q;
+    const SvlmAttendView& vw = b.view[r.ci];
+    q.n_tiles = ld_l2(&vw.ctrl->n_tiles);
+    q.n_total = ld_l2(&vw.ctrl->n_total);
+    q.shift = ld_l2(&vw.ctrl->shift_total);
+    q.wait_limit = ld_l2(&vw.ctrl->wait_limit);
+    long long first[PF_LIST / 32];
+#pragma unroll
+    for (int k = 0; k < PF_LIST / 32; ++k) first[k] = ld_l2(&vw.tiles[min((int)(threadIdx.x & 31) + 32 * k, b.n_slots / SVLM_PAGE - 1)].min_gid);
+#pragma unroll
+    for (int k = 0; k < PF_LIST / 32; ++k) q.first[k] = (int)max(first[k] - (q.n_total - r.n_q), -0x40000000ll);
+    return q;
+}
+__device__ __forceinline__ PfAsk pf_known(const PfMeta& meta) {
+    PfAsk q;
+    q.n_tiles = meta.n_tiles;
+    q.n_total = meta.n_total;
+    q.shift = meta.shift;
+    q.wait_limit = meta.wait_limit;
+#pragma unroll
+    for (int k = 0; k < PF_LIST / 32; ++k) q.first[k] = meta.list[(threadIdx.x & 31) + 32 * k].first;
+    return q;
+}
+__device__ __forceinline__ PfWork pf_work(const SvlmAttendBatch& b, const PfPlan& plan, const PfMeta& meta, const PfSeg& s, const PfRows& r, const PfAsk& q) {
     PfWork w;
     w.vw = &b.view[r.ci];
+    w.list = r.ci == meta.ci ? meta.list : nullptr;
+    w.n_tiles = q.n_tiles;
+    w.gid_q0 = q.n_total - r.n_q;
+    w.shift = q.shift;
+    w.wait_limit = q.wait_limit;
     w.rel_hi = min(r.n_q - 1, pf_div(r.m0 + PF_ROWS - 1, plan));
     const int lane = threadIdx.x & 31;
-    int n_act = 0, j = lane;
-    if (r.ci == meta.ci) {
-        w.list = meta.list;
-        w.n_tiles = meta.n_tiles;
-        w.gid_q0 = meta.n_total - r.n_q;
-        w.shift = meta.shift;
-        w.wait_limit = meta.wait_limit;
+    int n_act = 0;
 #pragma unroll
-        for (; j < PF_LIST; j += 32) n_act += j < w.n_tiles && meta.list[j].first <= w.rel_hi;
-    } else {
-        const SvlmCtrl* ctrl = w.vw->ctrl;
-        w.list = nullptr;
-        w.n_tiles = ld_l2(&ctrl->n_tiles);
-        const long long n_total = ld_l2(&ctrl->n_total);
-        w.shift = ld_l2(&ctrl->shift_total);
-        w.wait_limit = ld_l2(&ctrl->wait_limit);
-        long long first[4];        // without waiting for their number, so that everything takes one round trip
-#pragma unroll
-        for (int k = 0; k < 4; ++k) first[k] = ld_l2(&w.vw->tiles[min(lane + 32 * k, b.n_slots / SVLM_PAGE - 1)].min_gid);
-        w.gid_q0 = n_total - r.n_q;
-#pragma unroll
-        for (int k = 0; k < 4; ++k, j += 32) n_act += j < w.n_tiles && first[k] - w.gid_q0 <= w.rel_hi;
-    }
-    for (; j < w.n_tiles; j += 32) n_act += ld_l2(&w.vw->tiles[j].min_gid) - w.gid_q0 <= w.rel_hi;
+    for (int k = 0; k < PF_LIST / 32; ++k) n_act += lane + 32 * k < w.n_tiles && q.first[k] <= w.rel_hi;
+    for (int j = lane + PF_LIST; j < w.n_tiles; j += 32) n_act += ld_l2(&w.vw->tiles[j].min_gid) - w.gid_q0 <= w.rel_hi;
     n_act = __reduce_add_sync(0xffffffffu, n_act);
     w.p0 = s.a * n_act / PF_FRAC;
     w.n_proc = s.e * n_act / PF_FRAC - w.p0;
@@ -258,6 +275,11 @@ struct PfGroup {
     PfWork w;
     PfWalk walk;
     int more;                // segments follow
+    int known;               // the cache that the next five belong to (-1: none): a launch does not change its metadata
+    int n_tiles;
+    unsigned wait_limit;
+    long long n_total, shift;
+    int first[PF_LIST];      // smallest ordinals of the first pages of its list, relative to the first query token
     unsigned merge_later;    // blocks of columns of the first segment's unit that this CTA has to merge at the end
 };
 
@@ -880,7 +902,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     enter();
                     bar_sync(BAR_META, 128);
                 }
-                const PfWork w = pf_work(b, plan, sh.meta, seg, rows);
+                const PfWork w = pf_work(b, plan, sh.meta, seg, rows, rows.ci == sh.meta.ci ? pf_known(sh.meta) : pf_ask(b, rows));
                 const void* tmK = w.vw->tmaps;
                 const void* tmV = reinterpret_cast<const unsigned char*>(w.vw->tmaps) + 128;
                 PfPages pages;
@@ -972,7 +994,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     enter();
                     bar_sync(BAR_META, 128);
                 }
-                const PfWork w = pf_work(b, plan, sh.meta, seg, rows);
+                const PfWork w = pf_work(b, plan, sh.meta, seg, rows, rows.ci == sh.meta.ci ? pf_known(sh.meta) : pf_ask(b, rows));
                 const unsigned tmem = __shfl_sync(0xffffffffu, sh.tmem_base, 0);
                 tmem_s = tmem + Col::S;
                 tmem_p = tmem + Col::P(g);
@@ -1023,7 +1045,15 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 const long long n_total = ld_l2(&vw.ctrl->n_total), shift = ld_l2(&vw.ctrl->shift_total);
                 const unsigned wait_limit = ld_l2(&vw.ctrl->wait_limit);
 #pragma unroll
-                for (int k = 0; k < PF_LIST / 32; ++k) sh.meta.list[lane + 32 * k] = pf_entry(a[k], g[k], n_total - r.n_q);
+                for (int k = 0; k < PF_LIST / 32; ++k) {
+                    const PfEntry e = pf_entry(a[k], g[k], n_total - r.n_q);
+                    sh.meta.list[lane + 32 * k] = e;
+                    sh.group[0].first[lane + 32 * k] = sh.group[1].first[lane + 32 * k] = e.first;
+                }
+                if (lane < 2) {
+                    PfGroup& gr = sh.group[lane];
+                    gr.known = r.ci; gr.n_tiles = n_tiles; gr.n_total = n_total; gr.shift = shift; gr.wait_limit = wait_limit;
+                }
                 if (lane == 0) { sh.meta.ci = r.ci; sh.meta.n_tiles = n_tiles; sh.meta.wait_limit = wait_limit; sh.meta.n_total = n_total; sh.meta.shift = shift; }
                 __syncwarp();
             };
@@ -1037,7 +1067,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     bar_arrive(BAR_S, 160);
                     bar_arrive(BAR_S + 1, 160);
                 }
-                const PfWork w = pf_work(b, plan, sh.meta, seg, rows);
+                const PfWork w = pf_work(b, plan, sh.meta, seg, rows, rows.ci == sh.meta.ci ? pf_known(sh.meta) : pf_ask(b, rows));
                 for (int j = 0; j < w.n_proc; ++j, ++steps)
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
@@ -1076,15 +1106,32 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 enter();
                 const unsigned lanes = sh.tmem_base + ((unsigned)((warp & 3) * 32) << 16);
                 tm = {lanes + Col::S, lanes + Col::P(g), lanes + Col::O(g)};
-                if (staged) rot.load_pos(b, rows, q_pos, m, t_lo, n_tok, m / PfTileRotation<D>::HALF);
                 PfTileRotation<D>::load(plan, rows, g, m, G, q_heads, Q, sQg);
-                if (start) bar_sync(BAR_S + g, 160);
-                const PfWork nw = pf_work(b, plan, sh.meta, seg, rows);
+                if (start) {                  // warp 11 has put down what is known of the first segment's cache
+                    if (staged) rot.load_pos(b, rows, q_pos, m, t_lo, n_tok, m / PfTileRotation<D>::HALF);
+                    bar_sync(BAR_S + g, 160);
+                }
+                const bool fresh = rows.ci != gr.known;
+                PfAsk ask;
+                if (fresh) {
+                    ask = pf_ask(b, rows);
+                } else {
+                    ask.n_tiles = gr.n_tiles; ask.n_total = gr.n_total; ask.shift = gr.shift; ask.wait_limit = gr.wait_limit;
+#pragma unroll
+                    for (int k = 0; k < PF_LIST / 32; ++k) ask.first[k] = gr.first[lane + 32 * k];
+                }
+                if (!start && staged) rot.load_pos(b, rows, q_pos, m, t_lo, n_tok, m / PfTileRotation<D>::HALF);
+                const PfWork nw = pf_work(b, plan, sh.meta, seg, rows, ask);
                 if (m == 0) { gr.seg = seg; gr.rows = rows; gr.w = nw; gr.more = walk.more(plan); }
                 if (staged) rot.stage(b, rows, nw.shift, q_pos, m, t_lo, n_tok, cs_g);
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 bar_sync(BAR_WG + g, 128);
                 if (m == 0) gr.walk = walk;
+                if (fresh && m < 32) {
+                    if (m == 0) { gr.known = rows.ci; gr.n_tiles = ask.n_tiles; gr.n_total = ask.n_total; gr.shift = ask.shift; gr.wait_limit = ask.wait_limit; }
+#pragma unroll
+                    for (int k = 0; k < PF_LIST / 32; ++k) gr.first[m + 32 * k] = ask.first[k];
+                }
                 PfTileRotation<D>::rotate(b, plan, rows, nw.shift, q_pos, g, m, t_lo, staged, cs_g, sQg);
             }
             fence_proxy_async();              // the tile feeds the tensor core
