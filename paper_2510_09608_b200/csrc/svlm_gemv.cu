@@ -28,7 +28,8 @@ __device__ __forceinline__ void mma_bf16_16816(float* c, unsigned a0, unsigned a
 // vectors come from the predecessor.  Sized to fit beside a decode step's CTA: a decoder's chain of projections and decode
 // steps otherwise leaves HBM idle while a decode step combines its partial results.  Chain of 3584 -> 4608, decode step,
 // 3584 -> 3584 (77.6 MB): 28.9 us per layer with two blocks per SM that fetched one row per warp ahead, 24.5 with slots
-// only (each refill is a round trip to L2 of over 1 us), 23.3 with both.
+// only (each refill is a round trip to L2 of over 1 us), 23.3 with both.  The weights are marked as read once (l2_read_once):
+// two tokens of that chain through 28 layers 1331 -> 1306 us.
 constexpr int GV_THREADS = 256;
 constexpr int GT_WARPS = 8;
 constexpr int GT_SLOTS = GT_WARPS;      // one per warp
@@ -46,9 +47,15 @@ struct __align__(16) GtShared {
 };
 static_assert(sizeof(GtShared) % 16 == 0 && (GT_SLOTS * 8 * GT_ROW) % 128 == 0 && GT_ROW % 16 == 0 && GT_PAD % 8 == 0, "16-byte accesses");
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, void* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(svlm_ptx::smem_u32(dst)), "l"(src), "r"(bytes), "r"(svlm_ptx::smem_u32(bar)) : "memory");
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, void* bar, unsigned long long policy) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                 ::"r"(svlm_ptx::smem_u32(dst)), "l"(src), "r"(bytes), "r"(svlm_ptx::smem_u32(bar)), "l"(policy) : "memory");
+}
+// (the read-only path: weights are written by no kernel)
+__device__ __forceinline__ uint4 ld_weights(const uint4* p, unsigned long long policy) {
+    uint4 v;
+    asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
+    return v;
 }
 
 // parts: stages per group of eight rows; ks: elements of K per stage (a multiple of 64; the last part may be shorter)
@@ -71,6 +78,7 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
     }
     __syncthreads();
     pdl_launch_dependents();
+    const unsigned long long once = l2_read_once();
     // stage s: rows from r0 + (s / parts) * 8, elements from (s % parts) * ks.  A warp's stages are warp, warp + GT_WARPS, ...:
     // those at even places come through its slot, those at odd places through registers.
     auto fetch = [&](int s) {
@@ -79,7 +87,7 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         void* bar = &sh.full[warp];
         if (lane == 0) mbar_expect_tx(bar, rows * len);
         __syncwarp();
-        if (lane < rows) bulk_load(ring + (warp * 8 + lane) * GT_ROW, W + (size_t)(row + lane) * in_dim + k0, len, bar);
+        if (lane < rows) bulk_load(ring + (warp * 8 + lane) * GT_ROW, W + (size_t)(row + lane) * in_dim + k0, len, bar, once);
     };
     uint4 wr[GT_KB];
     auto load_regs = [&](int s) {
@@ -87,7 +95,7 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         const int row = min(r0 + s / parts * 8 + g, r1 - 1), k0 = s % parts * ks, kbs = min(ks, in_dim - k0) / 32;
         const uint4* p = reinterpret_cast<const uint4*>(W + (size_t)row * in_dim + k0) + kq;
 #pragma unroll
-        for (int kb = 0; kb < GT_KB; ++kb) wr[kb] = kb < kbs ? __ldg(p + 4 * kb) : make_uint4(0, 0, 0, 0);
+        for (int kb = 0; kb < GT_KB; ++kb) wr[kb] = kb < kbs ? ld_weights(p + 4 * kb, once) : make_uint4(0, 0, 0, 0);
     };
     fetch(warp);
     load_regs(warp + GT_WARPS);
@@ -96,7 +104,7 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         const char* p = reinterpret_cast<const char*>(W + (size_t)row * in_dim);
         const size_t bytes = (size_t)(r1 - row) * in_dim * 2;               // a multiple of 128
         for (size_t o = (size_t)threadIdx.x * 2048; o < bytes; o += GT_WARPS * 32 * 2048)
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p + o), "r"((unsigned)min((size_t)2048, bytes - o)) : "memory");
+            asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(p + o), "r"((unsigned)min((size_t)2048, bytes - o)), "l"(once) : "memory");
     }
     const unsigned wait_limit = ld_l2(&ctrl->wait_limit);                  // written at creation only, never by a kernel
     pdl_wait();

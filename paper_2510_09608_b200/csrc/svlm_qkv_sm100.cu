@@ -62,6 +62,13 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, in
     asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(bar) : "memory");
 }
+// The same with an L2 policy.  The weights are marked as read once (l2_read_once): their 59 MB per layer of the 7B shape used to push
+// everything else out of L2, the kernels' code included, whose first page then took the chunk prefill 7100 cycles, not 3400.
+// Chunk with projections, 28 layers: 3040 -> 2899 us.
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, int x, int y, unsigned bar, unsigned long long policy) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
+                 ::"r"(smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(bar), "l"(policy) : "memory");
+}
 // D (both CTAs' tensor memory) (+)= A B, operands in both CTAs' shared memory at the same addresses
 __device__ __forceinline__ void tc_mma_ss_pair(unsigned d_tmem, unsigned long long a_desc, unsigned long long b_desc, unsigned idesc,
                                                unsigned accumulate) {
@@ -80,7 +87,7 @@ __device__ __forceinline__ void tc_commit_pair(void* bar) {
 // Grid: (2 * pairs of heads, token tiles of `width`), clusters of two.
 __global__ void __launch_bounds__(QK_THREADS, 1)
 qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ SvlmCacheDev cd,
-                  int layer, int n, int hidden, int q_heads, int kv_heads_used, int width, uint16_t* __restrict__ Q_out) {
+                  int layer, int n, int hidden, int q_heads, int kv_heads_used, int width, int w_once, uint16_t* __restrict__ Q_out) {
     constexpr int D = 128, HALF = 64;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* ring = smem_raw;                                      // [stage][W tile | half of the X tile]
@@ -124,6 +131,7 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         // and phases are counted, not divided out, and addresses advance with them)
         if (lane == 0) {
             const int first = warp ? 1 : 0, y = i0 + (int)rank * (width / 2);
+            const unsigned long long once = w_once ? l2_read_once() : l2_read_again();
             unsigned bar = map_to_rank(&sh.full[first], 0);
             int st = first;
             unsigned phase = 1;                                  // first pass: already free
@@ -131,7 +139,7 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             for (int kb = first, x = first * QK_BK; kb < n_kb; kb += 2, x += 2 * QK_BK) {
                 if (!mbar_wait(&sh.empty[st], phase, abort_flag, wait_limit)) break;
                 if (rank == 0) mbar_expect_tx(&sh.full[st], 2 * stage_bytes);
-                tma_load_2d_pair(dst, &tmW, x, head * D, bar);   // rows past the end read as zeros
+                tma_load_2d_pair(dst, &tmW, x, head * D, bar, once);   // rows past the end read as zeros
                 tma_load_2d_pair(dst + QK_W_TILE, &tmX, x, y, bar);
                 dst += 2 * stage_bytes;
                 bar += 16;
@@ -318,6 +326,9 @@ cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmC
     if (e != cudaSuccess) return e;
     const int kv = with_append ? cd.kv_heads : 0;
     const dim3 grid((q_heads + 2 * kv + 1) / 2 * 2, (n + width - 1) / width);
+    // all tiles at once: whoever shares rows of W reads them at the same time, and nobody later (4133 tokens, where later tiles read them
+    // again: 2103 us with an ordinary policy, 2149 as read once)
+    const int w_once = (int)(grid.x * grid.y) <= svlm_sm_count();
     return svlm_launch_chained(qkv_append_kernel, grid, dim3(QK_THREADS), qkv_smem(), 2, st, *static_cast<const CUtensorMap*>(tmX),
-                               *static_cast<const CUtensorMap*>(tmW), cd, layer, n, hidden, q_heads, kv, width, static_cast<uint16_t*>(Q_out));
+                               *static_cast<const CUtensorMap*>(tmW), cd, layer, n, hidden, q_heads, kv, width, w_once, static_cast<uint16_t*>(Q_out));
 }
