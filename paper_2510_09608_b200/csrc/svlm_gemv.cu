@@ -94,8 +94,14 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         if (s >= n_stages) return;
         const int row = min(r0 + s / parts * 8 + g, r1 - 1), k0 = s % parts * ks, kbs = min(ks, in_dim - k0) / 32;
         const uint4* p = reinterpret_cast<const uint4*>(W + (size_t)row * in_dim + k0) + kq;
+        if (kbs == GT_KB) {
 #pragma unroll
-        for (int kb = 0; kb < GT_KB; ++kb) wr[kb] = kb < kbs ? ld_weights(p + 4 * kb, once) : make_uint4(0, 0, 0, 0);
+            for (int kb = 0; kb < GT_KB; ++kb) wr[kb] = ld_weights(p + 4 * kb, once);
+        } else {
+#pragma unroll
+            for (int kb = 0; kb < GT_KB; ++kb)
+                if (kb < kbs) wr[kb] = ld_weights(p + 4 * kb, once);
+        }
     };
     fetch(warp);
     load_regs(warp + GT_WARPS);
@@ -112,7 +118,7 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
     for (int i = threadIdx.x; i < n * row16; i += GT_WARPS * 32)
         *reinterpret_cast<uint4*>(sx + (size_t)(i / row16) * GT_PAD + (size_t)i * 8) = ld_l2(reinterpret_cast<const uint4*>(X) + i);
     __syncthreads();
-    const bool live = g < n;
+    const bool live = g < n;                                                // (the other rows of the MMA hold the last token once more: nobody reads their sums)
     const uint16_t* xrow = sx + (size_t)min(g, n - 1) * (in_dim + GT_PAD) + kq * 8;
     auto put = [&](int s, const float (&c)[4][4]) {
         if (live)
@@ -122,15 +128,21 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
     for (int s = warp; s < n_stages; s += 2 * GT_WARPS) {
         const int s1 = s + GT_WARPS;
         if (s1 < n_stages) {
-            const int k0 = s1 % parts * ks, last = min(ks, in_dim - k0) / 32 - 1;
+            const int k0 = s1 % parts * ks, kbs = min(ks, in_dim - k0) / 32;
             const uint16_t* xs = xrow + k0;
             float c[4][4] = {};                                             // four independent chains
-#pragma unroll
-            for (int kb = 0; kb < GT_KB; ++kb) {
-                uint4 a = *reinterpret_cast<const uint4*>(xs + min(kb, last) * 32);
-                if (!live || kb > last) a = make_uint4(0, 0, 0, 0);
+            auto block = [&](int kb) {
+                const uint4 a = *reinterpret_cast<const uint4*>(xs + kb * 32);
                 mma_bf16_16816(c[2 * (kb & 1)], a.x, 0u, a.y, 0u, wr[kb].x, wr[kb].y);
                 mma_bf16_16816(c[2 * (kb & 1) + 1], a.z, 0u, a.w, 0u, wr[kb].z, wr[kb].w);
+            };
+            if (kbs == GT_KB) {
+#pragma unroll
+                for (int kb = 0; kb < GT_KB; ++kb) block(kb);
+            } else {
+#pragma unroll
+                for (int kb = 0; kb < GT_KB; ++kb)
+                    if (kb < kbs) block(kb);
             }
             load_regs(s1 + 2 * GT_WARPS);
             put(s1, c);
@@ -142,16 +154,18 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         const unsigned char* wrow = ring + (warp * 8 + g) * GT_ROW + kq * 16;
         const uint16_t* xs = xrow + k0;
         float c[4][4] = {};
-#pragma unroll 2
-        for (int kb = 0; kb < kbs; kb += 2) {
+        auto block = [&](int kb, int u) {
+            const uint4 w = *reinterpret_cast<const uint4*>(wrow + kb * 64);
+            const uint4 a = *reinterpret_cast<const uint4*>(xs + kb * 32);
+            mma_bf16_16816(c[2 * u], a.x, 0u, a.y, 0u, w.x, w.y);
+            mma_bf16_16816(c[2 * u + 1], a.z, 0u, a.w, 0u, w.z, w.w);
+        };
+        if (kbs == GT_KB) {
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const uint4 w = *reinterpret_cast<const uint4*>(wrow + (kb + u) * 64);
-                uint4 a = *reinterpret_cast<const uint4*>(xs + (kb + u) * 32);
-                if (!live) a = make_uint4(0, 0, 0, 0);
-                mma_bf16_16816(c[2 * u], a.x, 0u, a.y, 0u, w.x, w.y);
-                mma_bf16_16816(c[2 * u + 1], a.z, 0u, a.w, 0u, w.z, w.w);
-            }
+            for (int kb = 0; kb < GT_KB; ++kb) block(kb, kb & 1);
+        } else {
+#pragma unroll 1
+            for (int kb = 0; kb < kbs; kb += 2) { block(kb, 0); block(kb + 1, 1); }
         }
         __syncwarp();
         fence_proxy_async();                                                // the slot's reads before the copy that refills it
