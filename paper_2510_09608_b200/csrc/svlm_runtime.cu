@@ -792,6 +792,10 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
             if (rc != SVLM_OK) break;
             SVLM_CUDA(cudaEventRecord(c->ev_done[l], c->stream));
             SVLM_CUDA(cudaStreamWaitEvent(c->copy_out, c->ev_done[l], 0));
+            // A layer's output starts down with the next layer but one's queries on their way up, not in the middle of a copy: the two
+            // directions keep their speed only side by side (28 layers of 524 queries, attended in less time than their copy
+            // takes: 2870 us as soon as the output is there, this way 2600).
+            if (l + 1 < nl) SVLM_CUDA(cudaStreamWaitEvent(c->copy_out, c->ev_in[l + 1], 0));
             SVLM_CUDA(cudaMemcpyAsync(static_cast<char*>(out_host) + l * layer_bytes, s + q_bytes + l * layer_bytes, layer_bytes,
                                       cudaMemcpyDeviceToHost, c->copy_out));
         }
