@@ -36,6 +36,44 @@ def test_chunk_prefill_work_split(d, hq, hk, frames, vw, base, contiguous):
     assert_close(s.attend(0, rows=rows))
 
 
+# --- page lists longer than what a thread block keeps of one (96 entries), and the pages of other caches than its first one's:
+# --- chunks of several units per thread block in one launch over caches of different lengths
+@pytest.mark.parametrize("d,hq,hk", [(64, 7, 1), (128, 6, 2)])
+def test_chunk_prefill_of_many_pages(d, hq, hk):
+    from harness import SideBySide, assert_close
+    wl = _wl(2, layers=1, q_heads=hq, kv_heads=hk, head_dim=d, sections=(d // 8, d // 16 * 3, d // 16 * 3), n_sink=40, vision_window=13000, text_window=70,
+             frames=15, grid_h=8, grid_w=9, text_max=21)
+    s = SideBySide(wl)
+    for _ in range(13):
+        s.append_chunk()
+        s.evict()
+    assert_close(s.attend(0, rows=list(range(0, len(s.last[0]), 61))))
+
+
+def test_chunk_prefill_of_several_caches_at_once():
+    from paper_2510_09608_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    normal = lambda *shape: torch.randn(*shape, generator=gen, device="cuda", dtype=torch.bfloat16)      # noqa: E731
+    hq, hk, d = 28, 4, 128
+    caches, q, pos, want, n_q = [], [], [], [], [1500, 37, 2100, 900]
+    for n, kept in zip(n_q, (3000, 14000, 2500, 6000)):
+        c = binding.Cache(1, hk, d, 64, 14000, 100, 14300)
+        c.append(0, normal(kept, hk, d), normal(kept, hk, d), torch.ones(kept, dtype=torch.uint8, device="cuda"), torch.arange(kept, dtype=torch.int32, device="cuda"))
+        caches.append(c)
+        q.append(normal(n, hq, d))
+        pos.append(torch.arange(kept - n, kept, dtype=torch.int32, device="cuda"))
+        want.append(c.attend(0, q[-1], pos[-1]).clone())
+    out = torch.empty(sum(n_q), hq, d, dtype=torch.bfloat16, device="cuda")
+    binding.attend_batched_varlen(caches, 0, torch.cat(q), torch.cat(pos), n_q, out)
+    at = 0
+    for n, w in zip(n_q, want):
+        # the cuts lie elsewhere, so weights are rounded to bf16 against other reference maxima: 2^-9 of a weight each, and outputs (below 1 in
+        # size here) to bf16 once more
+        assert (out[at:at + n].float() - w.float()).abs().max() < 2e-2
+        at += n
+    assert all(c.status() == binding.OK for c in caches)
+
+
 # --- chunks of few rows: rows at the edges of a 16-row tile, one to eight thread blocks over the keys, two tiles per block,
 # --- partly filled pages, positions beyond 2^16
 @pytest.mark.parametrize("d,hq,hk,frames,gh,gw,vw,base,contiguous", [
