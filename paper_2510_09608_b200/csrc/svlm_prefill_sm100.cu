@@ -85,7 +85,7 @@ constexpr int BAR_WG = 1;      // + tile: the softmax warpgroup alone (128)
 constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM (128 softmax + 32 issuer)
 constexpr int BAR_P2 = 5;      // + tile: second half of P (128 + 32)
 constexpr int BAR_READ = 7;    // + tile: its S is in registers, the columns are free (128 + 32 issuer of the S that comes there next)
-constexpr int BAR_S = 11;      // + tile: S is in TMEM; the first time, the metadata is there (128 + 32 warp 11)
+constexpr int BAR_S = 11;      // + tile: S is in TMEM (128 + 32 warp 11 + 32 issuer); the first time, the metadata is there (128 + 32 warp 11)
 constexpr int BAR_PV = 13;     // + tile: P V is done: its P may be overwritten, its accumulator touched (128 + 32 issuer)
 constexpr int BAR_Q = 9;       // + tile: the tile's query rows are in shared memory, its accumulator is free (128 + 32)
 constexpr int BAR_META = 15;   // the metadata is there (warps 8 to 11)
@@ -275,7 +275,7 @@ struct PfGroup {
     PfWork w;
     PfWalk walk;
     int more;                // segments follow
-    int known;               // the cache that the next five belong to (-1: none): a launch does not change its metadata
+    int known;               // the cache that the next five belong to (warp 11 sets the first one): a launch does not change its metadata
     int n_tiles;
     unsigned wait_limit;
     long long n_total, shift;
@@ -288,7 +288,6 @@ struct PfShared {            // control part of shared memory, behind the tiles
     unsigned long long s_full[2], pv_done[2];
     unsigned tmem_base;
     int abort_flag;
-    unsigned asked[2];                     // products S that the tile's issuer has come past
     unsigned take[2];                      // per tile: blocks of columns of a cut unit that this CTA has to merge
     int leave[2];                          // its own ones are left to whoever comes last
     PfCut cut[2];                          // of the CTA's last segment, of its first one
@@ -861,7 +860,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
     // ---- set-up: barriers, TMEM ------------------------------------------------------
     if (threadIdx.x == 0) {
         for (int s = 0; s < PF_RING; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 2); }   // both issuers release a page
-        for (int s = 0; s < 2; ++s) { mbar_init(&sh.s_full[s], 1); mbar_init(&sh.pv_done[s], 1); sh.asked[s] = 0; }
+        for (int s = 0; s < 2; ++s) { mbar_init(&sh.s_full[s], 1); mbar_init(&sh.pv_done[s], 1); }
         sh.abort_flag = 0;
         mbar_init_fence();
     }
@@ -937,8 +936,8 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             // has run out, and so does their order: nobody arrives at a barrier again before the others have been there.
             //   BAR_READ of B's page j-1 -> S of A's page j -> BAR_S -> BAR_READ of A's page j -> S of B's page j -> ...
             //   BAR_P2 of a page -> its BAR_PV -> the next page's BAR_P1
-            // Without a working wait everybody goes on along these lines, the issuers without issuing anything, and warp 11
-            // follows them by their count of products (asked).
+            // Without a working wait everybody goes on along these lines, the issuers without issuing anything: BAR_S holds the softmax
+            // until the issuer has come past the product, whether it asked for it or not, and warp 11 until the softmax is there.
             const int g = warp - 9;
             const bool leader = elect_one();
             constexpr unsigned IDESC_S = make_idesc(128, 128, 0);
@@ -985,7 +984,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 if (g == 1 || steps > 0) bar_sync(BAR_READ + (g ^ 1), 160);
                 if (ok) { tc_fence_after(); issue_S(n); }
                 ++steps;
-                if (lane == 0) *(volatile unsigned*)&sh.asked[g] = steps;
+                bar_arrive(BAR_S + g, 192);
             };
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
@@ -1064,19 +1063,19 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     enter();
                     fetch_meta(rows);
                     bar_sync(BAR_META, 128);
-                    bar_arrive(BAR_S, 160);
-                    bar_arrive(BAR_S + 1, 160);
+                    bar_sync(BAR_S, 160);
+                    bar_sync(BAR_S + 1, 160);
                 }
                 const PfWork w = pf_work(b, plan, sh.meta, seg, rows, rows.ci == sh.meta.ci ? pf_known(sh.meta) : pf_ask(b, rows));
                 for (int j = 0; j < w.n_proc; ++j, ++steps)
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
                         if (ok) ok = __all_sync(0xffffffffu, mbar_wait_short(&sh.s_full[g], steps & 1, abort_flag, w.wait_limit));
-                        // after a wait that has run out the barriers keep their order all the same: not before the issuer has come past the product
-                        for (unsigned p = 0; !ok && p < (1u << 20) && (int)(*(volatile unsigned*)&sh.asked[g] - steps) <= 0; ++p) __nanosleep(64);
                         tc_fence_after();
                         tc_fence_before();
-                        bar_arrive(BAR_S + g, 160);
+                        // (sync: after a wait that has run out nothing else would keep it from being here again before the softmax has been.  It
+                        // holds nobody up: the other tile's next product begins when this one is in registers)
+                        bar_sync(BAR_S + g, 192);
                     }
             }
         }
@@ -1175,7 +1174,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
 #pragma unroll
                     for (int ch = 0; ch < 4; ++ch) mixed |= (unsigned)!__all_sync(0xffffffffu, lo <= 32 * ch && end >= 32 * ch + 32) << ch;
                 }
-                bar_sync(BAR_S + g, 160);
+                bar_sync(BAR_S + g, 192);
                 tc_fence_after();
                 softmax_page<D>(g, tm, mixed, vlo, vlen, j > 0, m_ref, l);
             }
