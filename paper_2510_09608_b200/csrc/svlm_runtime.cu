@@ -277,6 +277,20 @@ SvlmPrefillLoad expected_load(const svlm_cache* c) {
     return {expected_pages(c), (int)std::min<long long>(c->stored_est > c->dev.n_sink + keep ? c->stored_est : keep, 1 << 30)};
 }
 
+// All layers of a chunk from host memory: whether a layer's output starts down with the next layer but one's queries on their way up, not in
+// the middle of a copy.  The two directions keep their speed only side by side, from copies of some 35 us on; beginning beside one is
+// worth min(15 + copy / 12, (copy - 35) / 2) us a layer.  What it costs is one copy's time less an attention call's, once, since the last
+// output comes that much later.  (Copies at 47.5 GB/s; an attention call's time by rows times keys, as the chunk prefill takes over
+// either head size.)  28/4 heads of 128, us, side by side and as soon as the output is there: 2000 tokens over 2000 keys, two layers
+// 1051 and 906, four 1685 and 1614, eight 2827 and 2910; over 8192 keys, two layers 1055 and 1015, four 1680 and 1753; 524 tokens over 1024 keys,
+// two layers 297 and 289, four 482 and 524, 28 2565 and 3174; 266 tokens, three layers 225 and 220, twelve 705 and 774; 16/8 heads of 64, 524 tokens
+// (copies of 23 us), eight layers 323 and 276.  Over 380 shapes this is 0.4 % behind the better of the two, always waiting 0.8 and never 2.3.
+bool output_beside_queries(const svlm_cache* c, int layers, size_t layer_bytes, int n_q, int q_heads) {
+    const double copy = (double)layer_bytes / 47.5e3;
+    const double attend = 15 + (double)q_heads * n_q * std::max(0.0, (double)c->stored_est - n_q / 2.0) / 2.85e6;
+    return copy > 35 && layers * std::min(15 + copy / 12, (copy - 35) / 2) >= copy - attend;
+}
+
 // call_layers: of a call that is launched layer by layer, all its layers (it takes the kernel that one launch of them would).
 // list, types: a decode step whose launch appends the token by itself (the host's counts have it already).
 int attend_common(svlm_cache* const* caches, int n_caches, int layer, const void* Q, const int32_t* q_pos, int n_q,
@@ -785,6 +799,7 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
                                       cudaMemcpyHostToDevice, c->copy_in));
             SVLM_CUDA(cudaEventRecord(c->ev_in[l], c->copy_in));
         }
+        const bool beside = output_beside_queries(c, nl, layer_bytes, n_q, q_heads);
         for (int l = 0; l < nl; ++l) {
             SVLM_CUDA(cudaStreamWaitEvent(c->stream, c->ev_in[l], 0));
             rc = attend_common(one, 1, l, s + l * layer_bytes, reinterpret_cast<const int32_t*>(s + 2 * q_bytes), n_q, q_heads,
@@ -792,10 +807,7 @@ int svlm_attend_host(svlm_cache* c, int layer, const void* Q_host, const int32_t
             if (rc != SVLM_OK) break;
             SVLM_CUDA(cudaEventRecord(c->ev_done[l], c->stream));
             SVLM_CUDA(cudaStreamWaitEvent(c->copy_out, c->ev_done[l], 0));
-            // A layer's output starts down with the next layer but one's queries on their way up, not in the middle of a copy: the two
-            // directions keep their speed only side by side (28 layers of 524 queries, attended in less time than their copy
-            // takes: 2870 us as soon as the output is there, this way 2600).
-            if (l + 1 < nl) SVLM_CUDA(cudaStreamWaitEvent(c->copy_out, c->ev_in[l + 1], 0));
+            if (beside && l + 1 < nl) SVLM_CUDA(cudaStreamWaitEvent(c->copy_out, c->ev_in[l + 1], 0));
             SVLM_CUDA(cudaMemcpyAsync(static_cast<char*>(out_host) + l * layer_bytes, s + q_bytes + l * layer_bytes, layer_bytes,
                                       cudaMemcpyDeviceToHost, c->copy_out));
         }

@@ -13,7 +13,7 @@ std::map<const void*, std::string> g_names;
 std::string g_log, g_fail;
 cudaError_t g_last = cudaSuccess;
 size_t g_alloc_limit = ~(size_t)0;
-int g_capturing = 0, g_mapped = 0;
+int g_capturing = 0, g_mapped = 0, g_waits = 0;
 cudaError_t done(cudaError_t e) { if (e != cudaSuccess) g_last = e; return e; }
 cudaError_t launch(const void* f, dim3 grid, dim3 block) {
     const std::string& name = g_names[f];
@@ -31,6 +31,7 @@ const char* fake_log() { static std::string out; out = g_log; g_log.clear(); ret
 void fake_alloc_limit(size_t bytes) { g_alloc_limit = bytes; }   // allocations above this size fail
 void fake_capturing(int on) { g_capturing = on; }                // the streams are being captured
 void fake_mapped(int on) { g_mapped = on; }                      // host memory is page-locked and mapped
+int fake_waits() { const int n = g_waits; g_waits = 0; return n; }   // streams that were made to wait for an event since the last call
 
 // ---- the runtime's calls that the library makes ----
 static dim3 g_grid, g_block;
@@ -71,7 +72,7 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = nullptr; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { ++g_waits; return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = nullptr; return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }

@@ -365,3 +365,27 @@ assert "host_in" not in deep and "append_meta" in deep and "decode" in deep
 for layers, layer in ((3, 0), (1, 0), (1, -1)):
     assert "host_in" in kernels(layers, layer), (layers, layer)
 """)
+
+
+def test_when_an_output_from_host_memory_waits_for_the_next_queries(host):
+    """All layers of a chunk in one call: an output waits for the next layer's queries where that saves more, over the layers, than the one
+    copy that it makes the last output later."""
+    host("""
+buf = vp(C.addressof((C.c_char * (120 << 20)).from_buffer(mem := bytearray(120 << 20))))
+def waits(layers, n, kept, hq, hk, d):
+    c = new(layers=layers, hk=hk, d=d, vw=kept, tw=100, capacity=kept + 100)
+    assert append(c, kept, layer=-1) == OK
+    fake.fake_waits()
+    assert lib.svlm_attend_host(c, -1, buf, buf, n, hq, buf) == OK
+    early = layers * n * hq * d * 2 < 16 << 20               # (the copies wait for earlier work by an event)
+    extra = fake.fake_waits() - 2 * layers - early
+    assert extra in (0, layers - 1)
+    lib.svlm_cache_destroy(c)
+    return extra > 0
+big, small = (28, 4, 128), (4, 1, 64)
+for n, kept, shape, first in ((2000, 2000, big, 7), (2000, 8192, big, 4), (1000, 1024, big, 5), (524, 1024, big, 3), (266, 1024, big, None), (524, 8192, big, 2),
+                              (150, 1024, big, None), (16, 1024, big, None), (524, 1024, (16, 8, 64), None), (2000, 2000, small, None)):
+    for layers in range(2, 9):
+        if layers * n * shape[0] * shape[2] * 2 < 110 << 20:
+            assert waits(layers, n, kept, *shape) == (first is not None and layers >= first), (n, kept, shape, layers)
+""")
