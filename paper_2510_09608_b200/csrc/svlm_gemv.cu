@@ -59,6 +59,13 @@ __device__ __forceinline__ uint4 ld_weights(const uint4* p, unsigned long long p
 }
 
 // parts: stages per group of eight rows; ks: elements of K per stage (a multiple of 64; the last part may be shorter)
+// FORM: which of the stages are GT_KS long.  Each has its own kernel, since a launch of 2 to 8 us notices the fetching of code that it does
+// not run (one token, weights from HBM, us, one kernel for all: 3584 x 512 2.87, this way 2.49; 2048 x 6144 5.98, 5.33):
+//   GT_WHOLE  all (in_dim a multiple of GT_KS): nothing to choose or to look at
+//   GT_MIXED  all but the last: a uniform branch.  4544 x 4096 10.5 with selects, 9.8 this way
+//   GT_SHORT  none: selects.  1344 x 4096 3.63 with branches, 3.1 this way; 3136 x 4096 7.9, 7.3
+enum GtForm { GT_WHOLE, GT_MIXED, GT_SHORT };
+template <int FORM>
 __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16_t* X, const uint16_t* __restrict__ W,
                                                                  uint16_t* __restrict__ Y, int n, int in_dim, int out_dim, int parts,
                                                                  int ks, SvlmCtrl* ctrl) {
@@ -94,7 +101,10 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         if (s >= n_stages) return;
         const int row = min(r0 + s / parts * 8 + g, r1 - 1), k0 = s % parts * ks, kbs = min(ks, in_dim - k0) / 32;
         const uint4* p = reinterpret_cast<const uint4*>(W + (size_t)row * in_dim + k0) + kq;
-        if (kbs == GT_KB) {
+        if (FORM == GT_SHORT) {
+#pragma unroll
+            for (int kb = 0; kb < GT_KB; ++kb) wr[kb] = kb < kbs ? __ldg(p + 4 * kb) : make_uint4(0, 0, 0, 0);
+        } else if (FORM == GT_WHOLE || kbs == GT_KB) {
 #pragma unroll
             for (int kb = 0; kb < GT_KB; ++kb) wr[kb] = ld_weights(p + 4 * kb, once);
         } else {
@@ -136,7 +146,16 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
                 mma_bf16_16816(c[2 * (kb & 1)], a.x, 0u, a.y, 0u, wr[kb].x, wr[kb].y);
                 mma_bf16_16816(c[2 * (kb & 1) + 1], a.z, 0u, a.w, 0u, wr[kb].z, wr[kb].w);
             };
-            if (kbs == GT_KB) {
+            if (FORM == GT_SHORT) {                                         // (written out: with the selects in `block` 1344 x 4096 takes 3.7 us)
+                const int last = kbs - 1;
+#pragma unroll
+                for (int kb = 0; kb < GT_KB; ++kb) {
+                    uint4 a = *reinterpret_cast<const uint4*>(xs + min(kb, last) * 32);
+                    if (!live || kb > last) a = make_uint4(0, 0, 0, 0);
+                    mma_bf16_16816(c[2 * (kb & 1)], a.x, 0u, a.y, 0u, wr[kb].x, wr[kb].y);
+                    mma_bf16_16816(c[2 * (kb & 1) + 1], a.z, 0u, a.w, 0u, wr[kb].z, wr[kb].w);
+                }
+            } else if (FORM == GT_WHOLE || kbs == GT_KB) {
 #pragma unroll
                 for (int kb = 0; kb < GT_KB; ++kb) block(kb);
             } else {
@@ -156,11 +175,15 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
         float c[4][4] = {};
         auto block = [&](int kb, int u) {
             const uint4 w = *reinterpret_cast<const uint4*>(wrow + kb * 64);
-            const uint4 a = *reinterpret_cast<const uint4*>(xs + kb * 32);
+            uint4 a = *reinterpret_cast<const uint4*>(xs + kb * 32);
+            if (FORM == GT_SHORT && !live) a = make_uint4(0, 0, 0, 0);
             mma_bf16_16816(c[2 * u], a.x, 0u, a.y, 0u, w.x, w.y);
             mma_bf16_16816(c[2 * u + 1], a.z, 0u, a.w, 0u, w.z, w.w);
         };
-        if (kbs == GT_KB) {
+        if (FORM == GT_SHORT) {
+#pragma unroll 2
+            for (int kb = 0; kb < kbs; kb += 2) { block(kb, 0); block(kb + 1, 1); }
+        } else if (FORM == GT_WHOLE || kbs == GT_KB) {
 #pragma unroll
             for (int kb = 0; kb < GT_KB; ++kb) block(kb, kb & 1);
         } else {
@@ -193,24 +216,29 @@ __global__ void __launch_bounds__(GT_WARPS * 32, 2) gemv_few_kernel(const uint16
     }
 }
 
+// Elements of K per stage: as few stages as go, about equally long, all but the last a multiple of 64.
+int few_stage(int in_dim) {
+    const int parts = (in_dim + GT_KS - 1) / GT_KS;
+    return ((in_dim + parts - 1) / parts + 63) / 64 * 64;
+}
+
+template <int FORM>
 cudaError_t launch_few(const uint16_t* X, const uint16_t* W, uint16_t* Y, int n, int in_dim, int out_dim, SvlmCtrl* ctrl, cudaStream_t st) {
     const size_t fixed = (size_t)GT_SLOTS * 8 * GT_ROW + sizeof(GtShared);
     // (the limit of the longest token rows this kernel takes, so that a later call finds it raised)
-    const cudaError_t e = svlm_allow_smem<gemv_few_kernel>(fixed + GT_MAX_X);
+    const cudaError_t e = svlm_allow_smem<gemv_few_kernel<FORM>>(fixed + GT_MAX_X);
     if (e != cudaSuccess) return e;
-    const int parts = (in_dim + GT_KS - 1) / GT_KS;
-    const int ks = ((in_dim + parts - 1) / parts + 63) / 64 * 64;
+    const int parts = (in_dim + GT_KS - 1) / GT_KS, ks = few_stage(in_dim);
     const int most_rows = GT_MAX_STAGES / parts * 8;
     const int blocks = std::max(std::min((out_dim + 7) / 8, svlm_sm_count()), (out_dim + most_rows - 1) / most_rows);
-    return svlm_launch_chained(gemv_few_kernel, dim3(blocks), dim3(GT_WARPS * 32), fixed + (size_t)n * (in_dim + GT_PAD) * 2, 1, st, X, W, Y, n,
+    return svlm_launch_chained(gemv_few_kernel<FORM>, dim3(blocks), dim3(GT_WARPS * 32), fixed + (size_t)n * (in_dim + GT_PAD) * 2, 1, st, X, W, Y, n,
                                in_dim, out_dim, parts, ks, ctrl);
 }
 
 // What the kernel above takes: the token rows fit beside the ring, a group's stages fit the partial sums, and the last
 // stage of a group is not empty (in_dim is a multiple of 64).
 bool few_supported(int n, int in_dim) {
-    const int parts = (in_dim + GT_KS - 1) / GT_KS;
-    const int ks = ((in_dim + parts - 1) / parts + 63) / 64 * 64;
+    const int parts = (in_dim + GT_KS - 1) / GT_KS, ks = few_stage(in_dim);
     return n <= 4 && in_dim % 64 == 0 && parts <= GT_MAX_STAGES && (parts - 1) * ks < in_dim && (size_t)n * (in_dim + GT_PAD) * 2 <= GT_MAX_X;
 }
 
@@ -293,6 +321,9 @@ cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int i
     // 5.1 / 5.6, 3584 x 4608 5.6 / 6.6-7.4.  Not with fewer rows of W (3584 x 2048 4.8 / 4.3, x 512 3.9 / 3.2), longer ones
     // (4096 x 1536 5.6 / 4.2, 8192 x 1024 8.0 / 4.8) or such as lie a multiple of 4 KB apart (2048 x 6144 7.0 / 5.4).
     const bool in_batches = in_dim <= 1792 || (in_dim <= 3584 && in_dim % 2048 && out_dim / 8 >= 2 * svlm_sm_count());
-    if (few_supported(n, in_dim) && !(from_l2 && in_batches)) return launch_few(x, w, y, n, in_dim, out_dim, ctrl, st);
+    if (few_supported(n, in_dim) && !(from_l2 && in_batches)) {
+        const auto launch = in_dim % GT_KS == 0 ? launch_few<GT_WHOLE> : few_stage(in_dim) == GT_KS ? launch_few<GT_MIXED> : launch_few<GT_SHORT>;
+        return launch(x, w, y, n, in_dim, out_dim, ctrl, st);
+    }
     return svlm_launch_chained(gemv_mma_kernel, dim3((out_dim + 7) / 8), dim3(GV_THREADS), 0, 1, st, x, w, y, n, in_dim, out_dim);
 }

@@ -399,6 +399,13 @@ def test_projection_shapes(layers, n, in_dim, out_dim):
     assert c.status() == binding.OK
 
 
+# --- rows in whole stages, with a shorter last one, all shorter; one to four stages per warp, one to four tokens
+@pytest.mark.parametrize("n", [1, 2, 3, 4])
+@pytest.mark.parametrize("in_dim,out_dim", [(512, 9088), (2048, 6144), (3584, 2048), (2880, 4096), (4544, 1152), (1344, 4096), (896, 8448), (1280, 640)])
+def test_projection_stages(n, in_dim, out_dim):
+    test_projection_shapes(512, n, in_dim, out_dim)
+
+
 # --- one layer's token from host memory, page-locked or not: moved by kernels up to 64 KB, by copies above; the same bits as
 # --- from device memory (two layers in turn; all layers of a cache that has one, where the step appends by itself)
 @pytest.mark.parametrize("layers", [2, 1])

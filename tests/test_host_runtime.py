@@ -204,6 +204,16 @@ assert "gemv_{kernel}" in "".join(ran())
 """)
 
 
+@pytest.mark.parametrize("in_dim,form", [(512, 0), (3584, 0), (8192, 0), (2304, 1), (4160, 1), (5440, 1), (64, 2), (576, 2), (1280, 2), (1344, 2), (2688, 2)])
+def test_projection_form_of_a_few_tokens(host, in_dim, form):
+    """Rows in stages that are all of one length, all but the last, or all shorter: a kernel each."""
+    host(f"""
+c = new(layers=800, hk=1, d=64, vw=64, tw=16, capacity=128)
+assert lib.svlm_out_proj(c, vp(P), vp(P), {in_dim}, 4096, 1, vp(P)) == OK
+assert "gemv_few_kernelILi{form}E" in "".join(ran())
+""")
+
+
 PLAN_PROGRAM = r"""
 #include <cassert>
 #include <cstdio>
