@@ -326,9 +326,14 @@ cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmC
     if (e != cudaSuccess) return e;
     const int kv = with_append ? cd.kv_heads : 0;
     const dim3 grid((q_heads + 2 * kv + 1) / 2 * 2, (n + width - 1) / width);
-    // all tiles at once: whoever shares rows of W reads them at the same time, and nobody later (4133 tokens, where later tiles read them
-    // again: 2103 us with an ordinary policy, 2149 as read once)
-    const int w_once = (int)(grid.x * grid.y) <= svlm_sm_count();
+    // Read once: all tiles at a time, so that whoever shares rows of W reads them together and nobody later (4133 tokens, where later tiles
+    // read them again: 2103 us with an ordinary policy, 2149 as read once); and not where all layers' weights, on both sides of the
+    // attention and taken to be of this one's size, stay in L2 from pass to pass and a short chunk leaves them there.  Chunk with both
+    // projections, us a layer, ordinary policy and read once: hidden 1024, four layers, 20 tokens 30.05 and 30.48, 133 tokens 35.07 and 35.21, 524
+    // 58.18 and 57.78; hidden 2048, three layers (57 MB), 20 tokens 35.95 and 36.40, 524 57.1 and 56.1, four layers, 133 tokens 43.65 and 43.17;
+    // hidden 3584, one layer (59 MB), 20 tokens 56.6 and 57.4, 133 74.8 and 75.9, 200 78.9 and 75.7, 524 84.1 and 78.8, two layers, 20 tokens 53.6 and 51.4.
+    const size_t all = (size_t)cd.layers * 2 * grid.x * 128 * hidden * 2;
+    const int w_once = (int)(grid.x * grid.y) <= svlm_sm_count() && (n >= 160 || all >= (size_t)64 << 20);
     return svlm_launch_chained(qkv_append_kernel, grid, dim3(QK_THREADS), qkv_smem(), 2, st, *static_cast<const CUtensorMap*>(tmX),
                                *static_cast<const CUtensorMap*>(tmW), cd, layer, n, hidden, q_heads, kv, width, w_once, static_cast<uint16_t*>(Q_out));
 }

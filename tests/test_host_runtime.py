@@ -399,3 +399,18 @@ for n, kept, shape, first in ((2000, 2000, big, 7), (2000, 8192, big, 4), (1000,
         if layers * n * shape[0] * shape[2] * 2 < 110 << 20:
             assert waits(layers, n, kept, *shape) == (first is not None and layers >= first), (n, kept, shape, layers)
 """)
+
+
+def test_which_weights_of_a_chunk_are_read_once(host):
+    """Weights that stay in L2 from pass to pass keep their place there, unless the chunk is long; where tiles read them again, always."""
+    host("""
+fake.fake_watch(b"qkv_append", 9)
+def once(layers, hidden, out, n):
+    c = new(layers=layers, capacity=1500)
+    assert lib.svlm_out_proj(c, vp(P), vp(P), hidden, out, n, vp(P)) == OK and "qkv_append" in "".join(ran())
+    lib.svlm_cache_destroy(c)
+    return fake.fake_seen()
+for layers, hidden, out, n, want in ((4, 1024, 3072, 20, 0), (4, 1024, 3072, 159, 0), (4, 1024, 3072, 160, 1), (3, 2048, 2560, 133, 0), (4, 2048, 2560, 20, 1),
+                                     (1, 3584, 4608, 133, 0), (1, 3584, 4608, 524, 1), (2, 3584, 3584, 20, 1), (28, 3584, 3584, 531, 1), (28, 3584, 4608, 4133, 0)):
+    assert once(layers, hidden, out, n) == want, (layers, hidden, out, n)
+""")
