@@ -28,8 +28,9 @@ __device__ __forceinline__ void mma_bf16_16816(float* c, unsigned a0, unsigned a
 // vectors come from the predecessor.  Sized to fit beside a decode step's CTA: a decoder's chain of projections and decode
 // steps otherwise leaves HBM idle while a decode step combines its partial results.  Chain of 3584 -> 4608, decode step,
 // 3584 -> 3584 (77.6 MB): 28.9 us per layer with two blocks per SM that fetched one row per warp ahead, 24.5 with slots
-// only (each refill is a round trip to L2 of over 1 us), 23.3 with both.  The weights are marked as read once (l2_read_once):
-// two tokens of that chain through 28 layers 1331 -> 1306 us.
+// only (each refill is a round trip to L2 of over 1 us), 23.3 with both, 22.7 without selects where stages are whole (FORM below) and with
+// the weights marked as read once (l2_read_once): two tokens of that chain through 28 layers, both policies on the present code, 1297 -> 1274 us;
+// one layer's weights, which stay in L2, take the same time with either (2048 x 6144 4.77 us, 4096 x 4096 6.36).
 constexpr int GV_THREADS = 256;
 constexpr int GT_WARPS = 8;
 constexpr int GT_SLOTS = GT_WARPS;      // one per warp
@@ -317,9 +318,11 @@ cudaError_t svlm_launch_gemv(const void* X, const void* W, void* Y, int n, int i
     uint16_t* y = static_cast<uint16_t*>(Y);
     // Weights that stay in L2 from token to token: fetching ahead buys nothing, and more, smaller blocks are faster while a warp
     // of theirs has all its weights in flight at once (rows of up to 1792), or in two batches and there are two blocks per SM:
-    // us, one or four tokens, this kernel against the other: 1024 x 1536 2.5 / 2.5-2.9, 2560 x 4096 4.9 / 5.4, 3584 x 2560
-    // 5.1 / 5.6, 3584 x 4608 5.6 / 6.6-7.4.  Not with fewer rows of W (3584 x 2048 4.8 / 4.3, x 512 3.9 / 3.2), longer ones
-    // (4096 x 1536 5.6 / 4.2, 8192 x 1024 8.0 / 4.8) or such as lie a multiple of 4 KB apart (2048 x 6144 7.0 / 5.4).
+    // us, one and four tokens, this kernel against the other: 1024 x 1536 2.28 and 2.46 / 2.13 and 2.36, 1344 x 4096 2.57 and 2.60 / 2.94
+    // and 3.54, 1792 x 2048 2.56 and 2.62 / 2.47 and 2.99, 2560 x 4096 4.65 and 4.61 / 4.61 and 4.81, 3584 x 2560 4.77 and 5.03 / 4.56 and
+    // 5.25, 3584 x 4608 5.33 and 5.47 / 5.92 and 6.66.  Not with fewer rows of W (3584 x 2048 4.47 and 4.66 / 3.44 and 4.05, x 512 3.72 and
+    // 3.81 / 2.53 and 3.23), longer ones (4096 x 1536 6.16 and 6.39 / 3.54 and 3.71, 8192 x 1024 7.95 and 8.24 / 3.80 and 4.48) or such as lie a multiple of
+    // 4 KB apart (2048 x 6144 6.50 and 6.69 / 4.66 and 4.74).
     const bool in_batches = in_dim <= 1792 || (in_dim <= 3584 && in_dim % 2048 && out_dim / 8 >= 2 * svlm_sm_count());
     if (few_supported(n, in_dim) && !(from_l2 && in_batches)) {
         const auto launch = in_dim % GT_KS == 0 ? launch_few<GT_WHOLE> : few_stage(in_dim) == GT_KS ? launch_few<GT_MIXED> : launch_few<GT_SHORT>;

@@ -76,7 +76,6 @@ __global__ void __launch_bounds__(256) kv_write_kernel(SvlmCacheDev cd, int laye
         svlm_ptx::pdl_launch_dependents();
         load_rows(row0);
     }
-
     if (append_n != n || slot < 0) return;   // the metadata append was dropped (capacity) or does not match
     for (int r = row0; r < row1; r += UNROLL) {
         if (r != row0) load_rows(r);

@@ -15,8 +15,9 @@ constexpr int PF_MIN_PAGES = 4;
 constexpr int PF_MAX_PIECES = 9;
 // What beginning a unit is reckoned as, in pages.  The cuts also decide against which reference maximum a row's weights are
 // rounded to bf16 (a piece begins its own), so another number here changes outputs in their last places: it stays where it is
-// unless that is worth it.  With 8, 196 chunk shapes (69 to 4133 tokens, 1200 to 9200 keys, six head shapes, one to eight streams) take 0.3 % less on
-// average, between 4 % less (69 tokens, 28/4 heads) and 3 % more (12/2 heads of 64, 266 tokens).
+// unless that is worth it.  With 7, 270 chunk shapes (37 to 4133 tokens, 350 to 9200 keys, six head shapes, one to eight streams) take 0.3 % less on
+// average, between 6 % less (16/2 heads, 133 tokens over 4800 keys 37.5 -> 35.3 us a layer) and 6 % more (199 tokens 34.4 -> 36.5); with 5 0.1 % less,
+// between 5 % less and 10 % more.
 constexpr int PF_PIECE = 10;
 constexpr int PF_SNAP = 3;            // a cut closer than this many pages to a unit's end moves there: a piece costs ~3 pages of set-up
 

@@ -40,7 +40,8 @@
 // Per-page bookkeeping that cost a masked page 2 us (descriptor loads, two barriers and a bisection through shared
 // memory) is now a few shuffles on values that arrive while the thread waits for S.
 // Every mbarrier wait is bounded: on expiry the CTA records SVLM_ERR_TIMEOUT in the caches' status words, keeps up its
-// named-barrier arrivals (their number depends on the work list only), drains its copies, frees its TMEM and returns.
+// named-barrier arrivals (their number depends on the work list only, their order on one another only), drains its copies, frees its TMEM
+// and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
