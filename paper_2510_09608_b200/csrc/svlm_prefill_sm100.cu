@@ -86,10 +86,11 @@ constexpr int BAR_WG = 1;      // + tile: the softmax warpgroup alone (128)
 constexpr int BAR_P1 = 3;      // + tile: first half of P is in TMEM (128 softmax + 32 issuer)
 constexpr int BAR_P2 = 5;      // + tile: second half of P (128 + 32)
 constexpr int BAR_READ = 7;    // + tile: its S is in registers, the columns are free (128 + 32 issuer of the S that comes there next)
-constexpr int BAR_S = 11;      // + tile: S is in TMEM (128 + 32 warp 11 + 32 issuer); the first time, the metadata is there (128 + 32 warp 11)
+constexpr int BAR_S = 11;      // + tile: S is in TMEM; the first time, the metadata is there (128 + 32 warp 11)
 constexpr int BAR_PV = 13;     // + tile: P V is done: its P may be overwritten, its accumulator touched (128 + 32 issuer)
 constexpr int BAR_Q = 9;       // + tile: the tile's query rows are in shared memory, its accumulator is free (128 + 32)
-constexpr int BAR_META = 15;   // the metadata is there (warps 8 to 11)
+constexpr int BAR_META = 15;   // the metadata is there (warps 8 to 11), once; from then on
+constexpr int BAR_ASKED = 15;  // an issuer has come past its product S, the tiles in turn (32 issuer + 32 warp 11)
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
@@ -937,8 +938,9 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
             // has run out, and so does their order: nobody arrives at a barrier again before the others have been there.
             //   BAR_READ of B's page j-1 -> S of A's page j -> BAR_S -> BAR_READ of A's page j -> S of B's page j -> ...
             //   BAR_P2 of a page -> its BAR_PV -> the next page's BAR_P1
-            // Without a working wait everybody goes on along these lines, the issuers without issuing anything: BAR_S holds the softmax
-            // until the issuer has come past the product, whether it asked for it or not, and warp 11 until the softmax is there.
+            //   S of a page -> BAR_ASKED -> its BAR_S
+            // Without a working wait everybody goes on along these lines, the issuers without issuing anything.  An issuer is past a product
+            // only when the softmax has been at the earlier one's BAR_S, so BAR_ASKED keeps warp 11 from being there twice.
             const int g = warp - 9;
             const bool leader = elect_one();
             constexpr unsigned IDESC_S = make_idesc(128, 128, 0);
@@ -985,7 +987,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                 if (g == 1 || steps > 0) bar_sync(BAR_READ + (g ^ 1), 160);
                 if (ok) { tc_fence_after(); issue_S(n); }
                 ++steps;
-                bar_arrive(BAR_S + g, 192);
+                bar_arrive(BAR_ASKED, 64);
             };
             while (walk.more(plan)) {
                 const PfSeg seg = walk.next(plan);
@@ -1064,19 +1066,18 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
                     enter();
                     fetch_meta(rows);
                     bar_sync(BAR_META, 128);
-                    bar_sync(BAR_S, 160);
-                    bar_sync(BAR_S + 1, 160);
+                    bar_arrive(BAR_S, 160);
+                    bar_arrive(BAR_S + 1, 160);
                 }
                 const PfWork w = pf_work(b, plan, sh.meta, seg, rows, rows.ci == sh.meta.ci ? pf_known(sh.meta) : pf_ask(b, rows));
                 for (int j = 0; j < w.n_proc; ++j, ++steps)
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
                         if (ok) ok = __all_sync(0xffffffffu, mbar_wait_short(&sh.s_full[g], steps & 1, abort_flag, w.wait_limit));
+                        bar_sync(BAR_ASKED, 64);              // (nothing to wait for behind a wait that was met)
                         tc_fence_after();
                         tc_fence_before();
-                        // (sync: after a wait that has run out nothing else would keep it from being here again before the softmax has been.  It
-                        // holds nobody up: the other tile's next product begins when this one is in registers)
-                        bar_sync(BAR_S + g, 192);
+                        bar_arrive(BAR_S + g, 160);
                     }
             }
         }
@@ -1175,7 +1176,7 @@ prefill_kernel(const __grid_constant__ SvlmAttendBatch b, const __grid_constant_
 #pragma unroll
                     for (int ch = 0; ch < 4; ++ch) mixed |= (unsigned)!__all_sync(0xffffffffu, lo <= 32 * ch && end >= 32 * ch + 32) << ch;
                 }
-                bar_sync(BAR_S + g, 192);
+                bar_sync(BAR_S + g, 160);
                 tc_fence_after();
                 softmax_page<D>(g, tm, mixed, vlo, vlen, j > 0, m_ref, l);
             }

@@ -12,9 +12,9 @@ import pytest
 SOURCE = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_09608_b200", "csrc", "svlm_prefill_sm100.cu")
 
 # what the model below goes through, role by role and in the order of the source: operation, barrier, tile (g: its own, o: the other one), threads
-ISSUER = ["sync READ o 160", "arrive S g 192", "sync META - 128", "sync Q g 160", "sync P1 g 160", "sync P2 g 160", "arrive PV g 160", "sync READ 1 160"]
-RELAY = ["sync META - 128", "sync S 0 160", "sync S 1 160", "sync S g 192"]
-SOFTMAX = ["sync S g 160", "arrive Q g 160", "sync Q g 160", "sync S g 192", "sync PV g 160"]
+ISSUER = ["sync READ o 160", "arrive ASKED - 64", "sync META - 128", "sync Q g 160", "sync P1 g 160", "sync P2 g 160", "arrive PV g 160", "sync READ 1 160"]
+RELAY = ["sync META - 128", "arrive S 0 160", "arrive S 1 160", "sync ASKED - 64", "arrive S g 160"]
+SOFTMAX = ["sync S g 160", "arrive Q g 160", "sync Q g 160", "sync S g 160", "sync PV g 160"]
 PAGE = ["arrive READ g 160", "sync PV g 160", "sync PV g 160", "arrive P1 g 160", "arrive P2 g 160"]
 
 
@@ -25,7 +25,7 @@ def test_the_model_is_of_the_source():
     def ops(begin, end):
         part = src[src.index(begin):]
         found = re.findall(r"bar_(sync|arrive)\(BAR_(\w+)(?: \+ ([^,]+))?, (\d+)\)", part[:part.index(end)])
-        return [f"{op} {name} {'-' if name == 'META' else tile[at]} {n}" for op, name, at, n in found if name != "WG"]
+        return [f"{op} {name} {'-' if name in ('META', 'ASKED') else tile[at]} {n}" for op, name, at, n in found if name != "WG"]
     assert ops("= MMA issuer of tile g", "= warp 11") == ISSUER
     assert ops("= warp 11", "= softmax warpgroups") == RELAY
     assert ops("= softmax warpgroups", "if (sh.abort_flag)") == SOFTMAX
@@ -49,7 +49,7 @@ def _run(seed, segs, p_out):
     """segs: pages of the thread block's units; p_out: how likely a wait runs out at a look."""
     rnd = random.Random(seed)
     bars = {(b, g): _Barrier() for b in ("READ", "S", "Q", "P1", "P2", "PV") for g in (0, 1)}
-    bars["META"] = _Barrier()
+    bars["META"] = bars["ASKED"] = _Barrier()        # one of the hardware's
     queue, done, gave_up = [], set(), [False]        # products asked for, one issuer's in order; those that are through
     loaded, stored = {}, {}                          # pages whose S all four warps have taken, whose P they have put down
 
@@ -83,7 +83,7 @@ def _run(seed, segs, p_out):
                 assert gave_up[0] or before[2] < 0 or loaded.get(before) == 4, "scores overwritten"
                 queue.append(("S", g, steps))
             steps += 1
-            bars["S", g].arrive(me, 192)
+            bars["ASKED"].arrive(me, 64)
         for n in segs:
             if n and ok:
                 ok = yield from wait(None)
@@ -110,13 +110,14 @@ def _run(seed, segs, p_out):
         ok, steps = True, 0
         yield from sync("META", "relay", 128)
         for g in (0, 1):
-            yield from sync(("S", g), "relay", 160)
+            bars["S", g].arrive("relay", 160)
         for n in segs:
             for _ in range(n):
                 for g in (0, 1):
                     if ok:
                         ok = yield from wait(("S", g, steps))
-                    yield from sync(("S", g), "relay", 192)
+                    yield from sync("ASKED", "relay", 64)
+                    bars["S", g].arrive("relay", 160)
                 steps += 1
 
     def softmax(g, w):
@@ -128,7 +129,7 @@ def _run(seed, segs, p_out):
             else:
                 yield from sync(("Q", g), me, 160)
             for j in range(n):
-                yield from sync(("S", g), me, 192)
+                yield from sync(("S", g), me, 160)
                 assert gave_up[0] or ("S", g, page) in done, "scores not there"
                 loaded["S", g, page] = loaded.get(("S", g, page), 0) + 1
                 bars["READ", g].arrive(me, 160)
