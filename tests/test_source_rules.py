@@ -12,16 +12,8 @@ def _source(name):
 def test_only_constants_take_the_read_only_path():
     """Kernels start while the one before them still runs (programmatic dependent launch), so what an earlier kernel of the
     stream may write (inputs, positions, metadata) is loaded by svlm_ptx::ld_in and ld_l2, which stay behind the wait and are
-    coherent.  The read-only path (__ldg, const __restrict__, ld.global.nc) is for the rotation table and the projections' weights."""
+    coherent.  The read-only path (__ldg, const __restrict__) is for the rotation table and the projections' weights."""
     constants = {"tab", "p", "wp"}      # p, wp: rows of W (svlm_gemv.cu)
-    # the one inline load of that path, and what it is given
-    inline = [(name, src) for name in sorted(os.listdir(CSRC)) for src in [_source(name)] if re.search(r"ld\.global(\.\w+)*\.nc", src)]
-    assert [name for name, _ in inline] == ["svlm_gemv.cu"]
-    src = inline[0][1]
-    body = re.search(r"uint4 ld_weights\(const uint4\* p, .*?\n\}", src, flags=re.S).group(0)
-    assert len(re.findall(r"ld\.global(?:\.\w+)*\.nc", src)) == len(re.findall(r"ld\.global(?:\.\w+)*\.nc", body)) == 1
-    calls = re.findall(r"ld_weights\((?!const uint4\*)\s*(\w+)", src)
-    assert calls and set(calls) == {"p"} and len(re.findall(r"const uint4\* p = reinterpret_cast<const uint4\*>\(W \+", src)) == 1
     for name in sorted(os.listdir(CSRC)):
         src = _source(name)
         if "pdl_wait" not in src and name != "svlm_rope.cuh":
@@ -30,6 +22,17 @@ def test_only_constants_take_the_read_only_path():
         assert used <= constants, (name, used - constants)
         restricted = set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", src))
         assert restricted <= {"tab", "W"}, (name, restricted)
+
+
+def test_only_weights_take_the_inline_read_only_load():
+    """The same for ld.global.nc in inline assembly: one function has it, and what it is given are rows of W."""
+    inline = [(name, src) for name in sorted(os.listdir(CSRC)) for src in [_source(name)] if re.search(r"ld\.global(\.\w+)*\.nc", src)]
+    assert [name for name, _ in inline] == ["svlm_gemv.cu"]
+    src = inline[0][1]
+    body = re.search(r"uint4 ld_weights\(const uint4\* p, .*?\n\}", src, flags=re.S).group(0)
+    assert len(re.findall(r"ld\.global(?:\.\w+)*\.nc", src)) == len(re.findall(r"ld\.global(?:\.\w+)*\.nc", body)) == 1
+    calls = re.findall(r"ld_weights\((?!const uint4\*)\s*(\w+)", src)
+    assert calls and set(calls) == {"p"} and len(re.findall(r"const uint4\* p = reinterpret_cast<const uint4\*>\(W \+", src)) == 1
 
 
 def test_waits_for_tensor_memory_name_what_was_loaded():
