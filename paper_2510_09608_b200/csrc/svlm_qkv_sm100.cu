@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "svlm_dev.h"
 #include "svlm_launch.h"
@@ -65,6 +66,7 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, in
 // The same with an L2 policy.  The weights are marked as read once (l2_read_once): their 59 MB per layer of the 7B shape used to push
 // everything else out of L2, the kernels' code included, whose first page then took the chunk prefill 7100 cycles, not 3400.
 // 531 tokens with their projections, 28 layers, in a loop at the power limit, both policies on the present code: 3429 -> 3329 us.
+// (Projections behind one another with nothing between them only pay for it: 524 tokens 19.95 -> 20.15 us with the append.)
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, int x, int y, unsigned bar, unsigned long long policy) {
     asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
                  ::"r"(smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(bar), "l"(policy) : "memory");
@@ -84,10 +86,12 @@ __device__ __forceinline__ void tc_commit_pair(void* bar) {
 
 // kv_heads_used = cd.kv_heads for the projection with append; 0 turns the kernel into the plain projection
 // Y = X W^T (the output projection after attention): every 128-column block is then a "query head" and goes to Q_out.
-// Grid: (2 * pairs of heads, token tiles of `width`), clusters of two.
+// Grid: (2 * pairs of heads, token tiles of `width`), clusters of two.  W_ONCE: the weights are marked as read once; an instance each, since
+// an ordinary policy as an operand of the load is not free either (4096 tokens 106.7 us, without 106.2).
+template <bool W_ONCE>
 __global__ void __launch_bounds__(QK_THREADS, 1)
 qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ SvlmCacheDev cd,
-                  int layer, int n, int hidden, int q_heads, int kv_heads_used, int width, int w_once, uint16_t* __restrict__ Q_out) {
+                  int layer, int n, int hidden, int q_heads, int kv_heads_used, int width, uint16_t* __restrict__ Q_out) {
     constexpr int D = 128, HALF = 64;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* ring = smem_raw;                                      // [stage][W tile | half of the X tile]
@@ -131,7 +135,7 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         // and phases are counted, not divided out, and addresses advance with them)
         if (lane == 0) {
             const int first = warp ? 1 : 0, y = i0 + (int)rank * (width / 2);
-            const unsigned long long once = w_once ? l2_read_once() : l2_read_again();
+            const unsigned long long once = W_ONCE ? l2_read_once() : 0;
             unsigned bar = map_to_rank(&sh.full[first], 0);
             int st = first;
             unsigned phase = 1;                                  // first pass: already free
@@ -139,7 +143,8 @@ qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             for (int kb = first, x = first * QK_BK; kb < n_kb; kb += 2, x += 2 * QK_BK) {
                 if (!mbar_wait(&sh.empty[st], phase, abort_flag, wait_limit)) break;
                 if (rank == 0) mbar_expect_tx(&sh.full[st], 2 * stage_bytes);
-                tma_load_2d_pair(dst, &tmW, x, head * D, bar, once);   // rows past the end read as zeros
+                if (W_ONCE) tma_load_2d_pair(dst, &tmW, x, head * D, bar, once);   // rows past the end read as zeros
+                else tma_load_2d_pair(dst, &tmW, x, head * D, bar);
                 tma_load_2d_pair(dst + QK_W_TILE, &tmX, x, y, bar);
                 dst += 2 * stage_bytes;
                 bar += 16;
@@ -322,8 +327,6 @@ int svlm_proj_tile(int n, int hidden, int blocks128) {
 
 cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmCacheDev& cd, int layer, int n, int hidden,
                                    int q_heads, bool with_append, int width, void* Q_out, cudaStream_t st) {
-    cudaError_t e = svlm_allow_smem<qkv_append_kernel>(qkv_smem());
-    if (e != cudaSuccess) return e;
     const int kv = with_append ? cd.kv_heads : 0;
     const dim3 grid((q_heads + 2 * kv + 1) / 2 * 2, (n + width - 1) / width);
     // Read once: all tiles at a time, so that whoever shares rows of W reads them together and nobody later (4133 tokens, where later tiles
@@ -333,7 +336,13 @@ cudaError_t svlm_launch_qkv_append(const void* tmX, const void* tmW, const SvlmC
     // 58.18 and 57.78; hidden 2048, three layers (57 MB), 20 tokens 35.95 and 36.40, 524 57.1 and 56.1, four layers, 133 tokens 43.65 and 43.17;
     // hidden 3584, one layer (59 MB), 20 tokens 56.6 and 57.4, 133 74.8 and 75.9, 200 78.9 and 75.7, 524 84.1 and 78.8, two layers, 20 tokens 53.6 and 51.4.
     const size_t all = (size_t)cd.layers * 2 * grid.x * 128 * hidden * 2;
-    const int w_once = (int)(grid.x * grid.y) <= svlm_sm_count() && (n >= 160 || all >= (size_t)64 << 20);
-    return svlm_launch_chained(qkv_append_kernel, grid, dim3(QK_THREADS), qkv_smem(), 2, st, *static_cast<const CUtensorMap*>(tmX),
-                               *static_cast<const CUtensorMap*>(tmW), cd, layer, n, hidden, q_heads, kv, width, w_once, static_cast<uint16_t*>(Q_out));
+    const bool w_once = (int)(grid.x * grid.y) <= svlm_sm_count() && (n >= 160 || all >= (size_t)64 << 20);
+    const auto launch = [&](auto once) {
+        constexpr auto kernel = qkv_append_kernel<decltype(once)::value>;
+        const cudaError_t e = svlm_allow_smem<kernel>(qkv_smem());
+        if (e != cudaSuccess) return e;
+        return svlm_launch_chained(kernel, grid, dim3(QK_THREADS), qkv_smem(), 2, st, *static_cast<const CUtensorMap*>(tmX),
+                                   *static_cast<const CUtensorMap*>(tmW), cd, layer, n, hidden, q_heads, kv, width, static_cast<uint16_t*>(Q_out));
+    };
+    return w_once ? launch(std::true_type{}) : launch(std::false_type{});
 }

@@ -13,8 +13,7 @@ std::map<const void*, std::string> g_names;
 std::string g_log, g_fail;
 cudaError_t g_last = cudaSuccess;
 size_t g_alloc_limit = ~(size_t)0;
-int g_capturing = 0, g_mapped = 0, g_waits = 0, g_arg = 0, g_seen = 0;
-std::string g_watch;
+int g_capturing = 0, g_mapped = 0, g_waits = 0;
 cudaError_t done(cudaError_t e) { if (e != cudaSuccess) g_last = e; return e; }
 cudaError_t launch(const void* f, dim3 grid, dim3 block) {
     const std::string& name = g_names[f];
@@ -34,9 +33,6 @@ void fake_capturing(int on) { g_capturing = on; }                // the streams 
 void fake_mapped(int on) { g_mapped = on; }                      // host memory is page-locked and mapped
 int fake_waits() { const int n = g_waits; g_waits = 0; return n; }   // streams that were made to wait for an event since the last call
 
-void fake_watch(const char* kernel, int arg) { g_watch = kernel; g_arg = arg; }   // the value of an int argument, of its latest launch:
-int fake_seen() { return g_seen; }
-
 // ---- the runtime's calls that the library makes ----
 static dim3 g_grid, g_block;
 unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t, void*) { g_grid = grid; g_block = block; return 0; }
@@ -50,10 +46,7 @@ void __cudaUnregisterFatBinary(void**) {}
 void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, void*, void*, void*, void*, int*) { g_names[host] = name; }
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3 block, void**, size_t, cudaStream_t) { return launch(f, grid, block); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
-    if (!g_watch.empty() && g_names[f].find(g_watch) != std::string::npos) g_seen = *static_cast<int*>(args[g_arg]);
-    return launch(f, c->gridDim, c->blockDim);
-}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->gridDim, c->blockDim); }
 cudaError_t cudaMalloc(void** p, size_t n) {
     *p = n > g_alloc_limit ? nullptr : std::calloc(1, n);      // (zeros that cost nothing until they are touched)
     return done(*p ? cudaSuccess : cudaErrorMemoryAllocation);
