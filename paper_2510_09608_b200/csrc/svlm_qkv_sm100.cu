@@ -87,7 +87,7 @@ __device__ __forceinline__ void tc_commit_pair(void* bar) {
 // kv_heads_used = cd.kv_heads for the projection with append; 0 turns the kernel into the plain projection
 // Y = X W^T (the output projection after attention): every 128-column block is then a "query head" and goes to Q_out.
 // Grid: (2 * pairs of heads, token tiles of `width`), clusters of two.  W_ONCE: the weights are marked as read once; an instance each, since
-// an ordinary policy as an operand of the load is not free either (4096 tokens 106.7 us, without 106.2).
+// an ordinary policy as an operand of the load is not free either (4096 tokens 106.6 us with the append, without 106.3).
 template <bool W_ONCE>
 __global__ void __launch_bounds__(QK_THREADS, 1)
 qkv_append_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ SvlmCacheDev cd,
